@@ -29,8 +29,8 @@
  *  - Supported: head_dim 64 or 128; dtype fp32 or bf16; n_q_heads % n_kv_heads == 0,
  *    g <= 8; window * g <= 1024; pool_kernel odd, 1..15; at most 65535 units per call;
  *    every device pointer 16-byte aligned.  The tensor-core kernels (tcgen05 score passes and residual,
- *    TMA-fed decode) serve bf16 with head_dim 128; fp32 and head_dim 64 run on CUDA-core kernels of the
- *    same interface, written for parity rather than speed.
+ *    TMA-fed decode) serve bf16; fp32, and head_dim 64 with one map per layer, run on CUDA-core kernels of
+ *    the same interface, written for parity rather than speed.
  */
 #ifndef VECTOR_H_
 #define VECTOR_H_
@@ -163,7 +163,7 @@ VECTOR_API size_t vector_workspace_bytes(const vector_shape* shape, const vector
 VECTOR_API vector_status vector_score(const vector_shape* shape, const void* Q_obs, const void* K, int64_t N,
                            float* scores, float* raw_out, void* ws, size_t ws_bytes, void* stream);
 
-/* Build constant of the tensor-core score passes (bf16, head_dim 128): the share of the softmax
+/* Build constant of the tensor-core score passes (bf16): the share of the softmax
  * exponentials that is evaluated by a polynomial on the FMA pipe instead of the special-function
  * unit (the unit that bounds the passes).  For reading the pipe counters of vector_score. */
 VECTOR_API float vector_score_exp2_fma_share(void);

