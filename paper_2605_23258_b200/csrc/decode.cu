@@ -5,6 +5,7 @@
 // both pools once, accumulating p-weighted values and p-weighted keys, and the
 // d x d map is applied once per query head in the merge step.
 //
+// bf16 runs the kernels of decode_bf16.cuh and decode_pertile_tc.cuh; below, for fp32:
 //   split  grid (n_splits, U): online softmax over a slice of the logical key
 //          range [0, n_ret + n_apx); emits (m, l, acc_v[d], acc_k[d]) per head
 //   merge  grid (U): combines the splits, applies W to acc_k, normalises
@@ -18,30 +19,17 @@
 
 namespace vec {
 
-template <typename T, int EPL> struct RowLoad;
-template <> struct RowLoad<float, 4> {
+template <int EPL> struct RowLoad;
+template <> struct RowLoad<4> {
     static __device__ __forceinline__ void load(const float* p, int lane, float (&o)[4]) {
         float4 v = reinterpret_cast<const float4*>(p)[lane];
         o[0] = v.x; o[1] = v.y; o[2] = v.z; o[3] = v.w;
     }
 };
-template <> struct RowLoad<float, 2> {
+template <> struct RowLoad<2> {
     static __device__ __forceinline__ void load(const float* p, int lane, float (&o)[2]) {
         float2 v = reinterpret_cast<const float2*>(p)[lane];
         o[0] = v.x; o[1] = v.y;
-    }
-};
-template <> struct RowLoad<__nv_bfloat16, 4> {
-    static __device__ __forceinline__ void load(const __nv_bfloat16* p, int lane, float (&o)[4]) {
-        uint2 v = reinterpret_cast<const uint2*>(p)[lane];
-        o[0] = __uint_as_float(v.x << 16); o[1] = __uint_as_float(v.x & 0xffff0000u);
-        o[2] = __uint_as_float(v.y << 16); o[3] = __uint_as_float(v.y & 0xffff0000u);
-    }
-};
-template <> struct RowLoad<__nv_bfloat16, 2> {
-    static __device__ __forceinline__ void load(const __nv_bfloat16* p, int lane, float (&o)[2]) {
-        uint32_t v = reinterpret_cast<const uint32_t*>(p)[lane];
-        o[0] = __uint_as_float(v << 16); o[1] = __uint_as_float(v & 0xffff0000u);
     }
 };
 
@@ -51,10 +39,10 @@ template <int D> struct Rec { static constexpr int floats = 2 + 2 * D; };
 // With ROPE the approximated value is W applied to the key turned back by its original position
 // (apx_pos): the logit still uses the stored key, only the p-weighted key sum takes the turned one.
 // A lane holds EPL consecutive channels; the partner channel c +- D/2 sits in lane ^ 16.
-template <typename T, int D, int G, bool ROPE>
+template <int D, int G, bool ROPE>
 __global__ void __launch_bounds__(128)
-decode_split_generic(const T* __restrict__ q, const T* __restrict__ ret_k, const T* __restrict__ ret_v,
-                     const T* __restrict__ apx_k, const int32_t* __restrict__ apx_pos, int64_t cap_ret,
+decode_split_generic(const float* __restrict__ q, const float* __restrict__ ret_k, const float* __restrict__ ret_v,
+                     const float* __restrict__ apx_k, const int32_t* __restrict__ apx_pos, int64_t cap_ret,
                      int64_t cap_apx, int n_ret, int n_apx, int g, float scale, float theta,
                      float* __restrict__ partial) {
     constexpr int EPL = D / 32;
@@ -76,18 +64,18 @@ decode_split_generic(const T* __restrict__ q, const T* __restrict__ ret_k, const
 #pragma unroll
         for (int e = 0; e < EPL; ++e) { av[a][e] = 0.f; ak[a][e] = 0.f; qr[a][e] = 0.f; }
         if (a < g) {
-            RowLoad<T, EPL>::load(q + ((size_t)u * g + a) * D, lane, qr[a]);
+            RowLoad<EPL>::load(q + ((size_t)u * g + a) * D, lane, qr[a]);
 #pragma unroll
             for (int e = 0; e < EPL; ++e) qr[a][e] *= scale;
         }
     }
     for (int i = lo + wid; i < hi; i += 4) {
         const bool retained = i < n_ret;
-        const T* kp = retained ? ret_k + ((size_t)u * cap_ret + i) * D
+        const float* kp = retained ? ret_k + ((size_t)u * cap_ret + i) * D
                                : apx_k + ((size_t)u * cap_apx + (i - n_ret)) * D;
         float kx[EPL], vx[EPL];
-        RowLoad<T, EPL>::load(kp, lane, kx);
-        if (retained) RowLoad<T, EPL>::load(ret_v + ((size_t)u * cap_ret + i) * D, lane, vx);
+        RowLoad<EPL>::load(kp, lane, kx);
+        if (retained) RowLoad<EPL>::load(ret_v + ((size_t)u * cap_ret + i) * D, lane, vx);
         float kt[EPL];                       // what an approximated token contributes: the key, or the key turned back
 #pragma unroll
         for (int e = 0; e < EPL; ++e) kt[e] = kx[e];
@@ -151,14 +139,14 @@ decode_split_generic(const T* __restrict__ q, const T* __restrict__ ret_k, const
 }
 
 // grid (U), D threads.
-template <typename T, typename TO, int D>
+template <typename TO, int D>
 __global__ void __launch_bounds__(D)
-decode_merge_generic(const float* __restrict__ partial, const T* __restrict__ W, int LH, int g, int n_splits,
+decode_merge_generic(const float* __restrict__ partial, const float* __restrict__ W, int LH, int g, int n_splits,
                      TO* __restrict__ out) {
     constexpr int REC = Rec<D>::floats;
     __shared__ float aks[D];
     const int u = blockIdx.x, c = threadIdx.x;
-    const T* Wu = W + (size_t)(u % LH) * D * D;
+    const float* Wu = W + (size_t)(u % LH) * D * D;
     for (int a = 0; a < g; ++a) {
         const float* rec = partial + ((size_t)u * n_splits * g + a) * REC;
         const size_t stride = (size_t)g * REC;
@@ -177,26 +165,26 @@ decode_merge_generic(const float* __restrict__ partial, const T* __restrict__ W,
         __syncthreads();
         float proj = 0.f;
 #pragma unroll 8
-        for (int c2 = 0; c2 < D; ++c2) proj = fmaf(to_f32(Wu[(size_t)c * D + c2]), aks[c2], proj);
+        for (int c2 = 0; c2 < D; ++c2) proj = fmaf(Wu[(size_t)c * D + c2], aks[c2], proj);
         store_out(out + ((size_t)u * g + a) * D + c, (accv + proj) / L);
     }
 }
 
-template <typename T, int D, int G>
+template <int D, int G>
 static vector_status launch_decode(const Dims& dm, const void* q, const vector_cache* ch, const void* W, void* out,
                                    int out_dtype, float* partial, cudaStream_t st) {
     const int n_splits = decode_num_splits(dm.U, ch->n_ret + ch->n_apx);
     dim3 grid(n_splits, dm.U);
-    auto kern = dm.rope ? decode_split_generic<T, D, G, true> : decode_split_generic<T, D, G, false>;
-    kern<<<grid, 128, 0, st>>>((const T*)q, (const T*)ch->ret_k, (const T*)ch->ret_v, (const T*)ch->apx_k,
+    auto kern = dm.rope ? decode_split_generic<D, G, true> : decode_split_generic<D, G, false>;
+    kern<<<grid, 128, 0, st>>>((const float*)q, (const float*)ch->ret_k, (const float*)ch->ret_v, (const float*)ch->apx_k,
                                ch->apx_pos, ch->cap_ret, ch->cap_apx, (int)ch->n_ret, (int)ch->n_apx, dm.g,
                                dm.scale, dm.theta, partial);
     VEC_LAUNCH_CHECK();
     if (out_dtype == VECTOR_F32)
-        decode_merge_generic<T, float, D><<<dm.U, D, 0, st>>>(partial, (const T*)W, dm.LH, dm.g, n_splits,
+        decode_merge_generic<float, D><<<dm.U, D, 0, st>>>(partial, (const float*)W, dm.LH, dm.g, n_splits,
                                                              (float*)out);
     else
-        decode_merge_generic<T, __nv_bfloat16, D><<<dm.U, D, 0, st>>>(partial, (const T*)W, dm.LH, dm.g, n_splits,
+        decode_merge_generic<__nv_bfloat16, D><<<dm.U, D, 0, st>>>(partial, (const float*)W, dm.LH, dm.g, n_splits,
                                                                      (__nv_bfloat16*)out);
     VEC_LAUNCH_CHECK();
     return VECTOR_OK;
@@ -217,18 +205,21 @@ int* kernel_fault_address() {
     return addr[dev];
 }
 
-// bf16, head_dim 128: persistent TMA + tensor-core streaming kernel and the record merge.
-static vector_status launch_decode_bf16_d128(const Dims& dm, const void* q, const vector_cache* ch, const void* W,
-                                             void* out, int out_dtype, int mode, float* partial, cudaStream_t st) {
+// bf16: persistent TMA + tensor-core streaming kernel and the record merge.
+template <int D>
+static vector_status launch_decode_bf16(const Dims& dm, const void* q, const vector_cache* ch, const void* W,
+                                        void* out, int out_dtype, int mode, float* partial, cudaStream_t st) {
     using T = __nv_bfloat16;
+    using Plain = dbf::Cfg<D, false>;
+    using Rope = dbf::Cfg<D, true>;
     static PerDeviceOnce once;
     if (once.first()) {
-        cudaError_t e = cudaFuncSetAttribute(dbf::decode_stream_bf16_d128<false>,
-                                             cudaFuncAttributeMaxDynamicSharedMemorySize, dbf::SMEM_BYTES);
+        cudaError_t e = cudaFuncSetAttribute(dbf::decode_stream_bf16<D, false>,
+                                             cudaFuncAttributeMaxDynamicSharedMemorySize, Plain::SMEM_BYTES);
         if (e == cudaSuccess)
-            e = cudaFuncSetAttribute(dbf::decode_stream_bf16_d128<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                     dbf::SMEM_BYTES);
-        if (e == cudaSuccess)
+            e = cudaFuncSetAttribute(dbf::decode_stream_bf16<D, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                     Rope::SMEM_BYTES);
+        if (D == 128 && e == cudaSuccess)
             e = cudaFuncSetAttribute(dpt::decode_stream_pertile_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, dpt::SMEM_BYTES);
         if (e != cudaSuccess) { once.undo(); VEC_CUDA_CHECK(e); }
     }
@@ -237,24 +228,24 @@ static vector_status launch_decode_bf16_d128(const Dims& dm, const void* q, cons
     const dbf::Plan pl = dbf::make_plan(dm.U, ch->n_ret, ch->n_apx, sm_count());
     if (pl.s_max > decode_stream_slots(dm.U)) return VECTOR_ERR_WORKSPACE;
     dbf::Maps maps;
-    const uint64_t row_b = 256;
+    const uint64_t row_b = 2 * D;
     bool ok = true;
     if (ch->n_ret > 0) {
-        ok = ok && tma::encode_bf16_3d(&maps.ret_k, ch->ret_k, 128, (uint64_t)ch->n_ret, (uint64_t)dm.U, row_b,
+        ok = ok && tma::encode_bf16_3d(&maps.ret_k, ch->ret_k, D, (uint64_t)ch->n_ret, (uint64_t)dm.U, row_b,
                                        (uint64_t)ch->cap_ret * row_b, 64, 64);
-        ok = ok && tma::encode_bf16_3d(&maps.ret_v, ch->ret_v, 128, (uint64_t)ch->n_ret, (uint64_t)dm.U, row_b,
+        ok = ok && tma::encode_bf16_3d(&maps.ret_v, ch->ret_v, D, (uint64_t)ch->n_ret, (uint64_t)dm.U, row_b,
                                        (uint64_t)ch->cap_ret * row_b, 64, 64);
     }
     if (ch->n_apx > 0)
-        ok = ok && tma::encode_bf16_3d(&maps.apx_k, ch->apx_k, 128, (uint64_t)ch->n_apx, (uint64_t)dm.U, row_b,
+        ok = ok && tma::encode_bf16_3d(&maps.apx_k, ch->apx_k, D, (uint64_t)ch->n_apx, (uint64_t)dm.U, row_b,
                                        (uint64_t)ch->cap_apx * row_b, 64, 64);
     if (!ok) return VECTOR_ERR_CUDA;
     if (ch->n_ret == 0) { maps.ret_k = maps.apx_k; maps.ret_v = maps.apx_k; }   // never dereferenced: no such tiles
     if (ch->n_apx == 0) maps.apx_k = maps.ret_k;
     const float c2 = dm.scale * 1.4426950408889634f;
     RopePhases ph = {};
-    if (dm.rope) rope_phases(dm.theta, 128, &ph);
-    if (mode == 1) {
+    if (dm.rope) rope_phases(dm.theta, D, &ph);
+    if (D == 128 && mode == 1) {
         // reconstruction tile by tile on the tensor cores: its own streaming kernel, two consumer warps
         dpt::Maps pm;
         pm.ret_k = maps.ret_k; pm.ret_v = maps.ret_v; pm.apx_k = maps.apx_k;
@@ -265,34 +256,34 @@ static vector_status launch_decode_bf16_d128(const Dims& dm, const void* q, cons
         dpt::decode_stream_pertile_tc<<<pl.B, dpt::THREADS, dpt::SMEM_BYTES, st>>>(
             (const T*)q, pm, pl, (int)ch->n_ret, (int)ch->n_apx, dm.g, dm.LH, c2, partial, fault);
     } else if (dm.rope)
-        dbf::decode_stream_bf16_d128<true><<<pl.B, dbf::ROPE_THREADS, dbf::SMEM_BYTES, st>>>(
+        dbf::decode_stream_bf16<D, true><<<pl.B, Rope::THREADS, Rope::SMEM_BYTES, st>>>(
             (const T*)q, maps, pl, (int)ch->n_ret, (int)ch->n_apx, dm.g, dm.LH, c2, partial, fault, ch->apx_pos,
             (long long)ch->cap_apx, ph);
     else
-        dbf::decode_stream_bf16_d128<false><<<pl.B, dbf::THREADS, dbf::SMEM_BYTES, st>>>(
+        dbf::decode_stream_bf16<D, false><<<pl.B, Plain::THREADS, Plain::SMEM_BYTES, st>>>(
             (const T*)q, maps, pl, (int)ch->n_ret, (int)ch->n_apx, dm.g, dm.LH, c2, partial, fault, nullptr, 0, ph);
     VEC_LAUNCH_CHECK();
     // programmatic dependent launch: the merge blocks start while the streaming kernel drains
     const float* rec = partial;
     const int apply_w = mode == 1 ? 0 : 1;
-    const int cw = mode == 1 ? dpt::CONSUMERS : dbf::CONSUMER_WARPS;      // records a block leaves per unit
+    const int cw = mode == 1 ? dpt::CONSUMERS : dm.rope ? Rope::CONSUMER_WARPS : Plain::CONSUMER_WARPS;   // records a block leaves per unit
     const T* Wp = (const T*)W;
-    // blocks of 128 g threads; up to four heads leave the merge 128 registers a thread
+    // blocks of D g threads; up to 512 threads leave the merge 40 registers a thread with three blocks resident
 #define VEC_MERGE(TO, MAXT)                                                                                                  \
-    VEC_CUDA_CHECK(launch_maybe_dependent(true, dbf::decode_merge_bf16_d128<TO, MAXT>, dim3(dm.U), dim3(128 * dm.g), 0, st, rec, \
+    VEC_CUDA_CHECK(launch_maybe_dependent(true, dbf::decode_merge_bf16<TO, D, MAXT>, dim3(dm.U), dim3(D * dm.g), 0, st, rec, \
                                           Wp, dm.LH, dm.g, pl, apply_w, cw, (TO*)out))
-    if (out_dtype == VECTOR_F32) { if (dm.g <= 4) VEC_MERGE(float, 512); else VEC_MERGE(float, 1024); }
-    else { if (dm.g <= 4) VEC_MERGE(T, 512); else VEC_MERGE(T, 1024); }
+    if (out_dtype == VECTOR_F32) { if (D * dm.g <= 512) VEC_MERGE(float, 512); else VEC_MERGE(float, 1024); }
+    else { if (D * dm.g <= 512) VEC_MERGE(T, 512); else VEC_MERGE(T, 1024); }
 #undef VEC_MERGE
     return VECTOR_OK;
 }
 
-template <typename T, int D>
+template <int D>
 static vector_status launch_decode_g(const Dims& dm, const void* q, const vector_cache* ch, const void* W,
                                      void* out, int out_dtype, float* partial, cudaStream_t st) {
-    if (dm.g <= 2) return launch_decode<T, D, 2>(dm, q, ch, W, out, out_dtype, partial, st);
-    if (dm.g <= 4) return launch_decode<T, D, 4>(dm, q, ch, W, out, out_dtype, partial, st);
-    return launch_decode<T, D, 8>(dm, q, ch, W, out, out_dtype, partial, st);
+    if (dm.g <= 2) return launch_decode<D, 2>(dm, q, ch, W, out, out_dtype, partial, st);
+    if (dm.g <= 4) return launch_decode<D, 4>(dm, q, ch, W, out, out_dtype, partial, st);
+    return launch_decode<D, 8>(dm, q, ch, W, out, out_dtype, partial, st);
 }
 
 }  // namespace vec
@@ -321,10 +312,10 @@ extern "C" vector_status vector_decode_attn(const vector_shape* shape, const voi
     cudaStream_t st = (cudaStream_t)stream;
     float* partial = (float*)ws;
     if (dm.dtype == VECTOR_F32)
-        return dm.d == 64 ? launch_decode_g<float, 64>(dm, q, cache, W, out, out_dtype, partial, st)
-                          : launch_decode_g<float, 128>(dm, q, cache, W, out, out_dtype, partial, st);
-    if (dm.d == 64) return launch_decode_g<__nv_bfloat16, 64>(dm, q, cache, W, out, out_dtype, partial, st);
-    return launch_decode_bf16_d128(dm, q, cache, W, out, out_dtype, mode, partial, st);
+        return dm.d == 64 ? launch_decode_g<64>(dm, q, cache, W, out, out_dtype, partial, st)
+                          : launch_decode_g<128>(dm, q, cache, W, out, out_dtype, partial, st);
+    if (dm.d == 64) return launch_decode_bf16<64>(dm, q, cache, W, out, out_dtype, mode, partial, st);
+    return launch_decode_bf16<128>(dm, q, cache, W, out, out_dtype, mode, partial, st);
 }
 
 // ---------------------------------------------------------------------------

@@ -1,19 +1,19 @@
-// Decode attention over the mixed cache for bf16, head_dim 128 (HBM-bound).
+// Decode attention over the mixed cache for bf16, head_dim 64 or 128 (HBM-bound).
 //
-// Every K/V row is read once.  Each unit's rows are cut into 32 KB tiles -- a
-// retained tile = 64 keys + their 64 values, a key-only tile = 128 keys -- and
-// the global tile sequence is dealt out in equal contiguous ranges to one
+// Every K/V row is read once.  Each unit's rows are cut into tiles of 128 rows (32 KB
+// at head_dim 128, 16 KB at 64) -- a retained tile = 64 keys + their 64 values, a
+// key-only tile = 128 keys -- and the global tile sequence is dealt out in equal contiguous ranges to one
 // persistent block per SM: the load is balanced by bytes and there is no wave tail.
 //
 // Inside a block one producer thread streams the tiles with TMA
 // (cp.async.bulk.tensor, 128-byte swizzle, zero fill past the end of a pool)
-// into six 32 KB slots guarded by full/empty mbarriers.  Tiles go round-robin
-// to three consumer warps, each with two slots of its own (tile i: warp i % 3,
-// slot i % 6), so a warp sees every phase of the barriers it waits on -- with a
+// into slots that fill 192 KB, guarded by full/empty mbarriers.  Tiles go round-robin
+// to the consumer warps, each with slots of its own (head_dim 128: three warps with two
+// 32 KB slots each, tile i to warp i % 3 and slot i % 6), so a warp sees every phase of the barriers it waits on -- with a
 // parity wait, a waiter that skipped a phase could take an old completion for
 // the one it wants, since TMA copies land out of order.  A warp works through a
 // whole tile on its own, 64 keys at a time, and never synchronises with the others:
-//   S = Q K^T      64 m16n8k16 bf16 MMAs (eight independent accumulators), the g
+//   S = Q K^T      head_dim / 2 m16n8k16 bf16 MMAs (eight independent accumulators), the g
 //                  query heads padded to the MMA rows
 //   online softmax in fp32 registers, one rescale per 64 keys (exp2, scale folded in)
 //   O += P V  (retained tile)  or  A += P K  (key-only tile: the p-weighted key
@@ -21,7 +21,7 @@
 //             MMA rows 0-7 and bf16 lo in rows 8-15, one MMA for both parts
 // RoPE decoupling (ROPE): the value of a key-only token is W applied to the key turned back by its
 // original position.  The logits use the stored keys; before the P K product the warp rotates its 64
-// keys in shared memory, channel c with c + 64 by the angle -pos * theta^(-2c/128).  The angle is
+// keys in shared memory, channel c with c + D/2 by the angle -pos * theta^(-2c/D).  The angle is
 // taken exactly modulo one turn in 64-bit fixed point (pos * phase[c] wraps by itself), its sine and
 // cosine by the fast units.
 // A warp keeps one running state (m, l, O or A) per unit and writes it as its
@@ -40,21 +40,28 @@ namespace vec {
 namespace dbf {
 
 constexpr int KEYS = 64;                     // keys per softmax step (and per TMA box)
-constexpr int SLOTS = 6;                     // a multiple of CONSUMER_WARPS: a slot always serves the same warp
-constexpr int SLOT_BYTES = 32768;            // retained: K 16 KB | V 16 KB; key-only: keys 0-63 | keys 64-127
-constexpr int HALF_BYTES = 16384;            // 64 rows of 256 B as two swizzled 64 x 128 B boxes
 constexpr int BOX_BYTES = 8192;              // 64 rows x 128 bytes
-constexpr int CONSUMER_WARPS = 3;
-constexpr int THREADS = 32 * (CONSUMER_WARPS + 1);
 // With RoPE decoupling the block carries helper warps that turn a tile's keys back for the warp
 // that owns the tile: a team is that warp plus four helpers (warps 4 + 4 team .. 7 + 4 team), one
 // per warp scheduler (scheduler = warp index modulo 4), since the sine / cosine unit is per scheduler.
 constexpr int ROPE_HELPERS = 4;
-constexpr int ROPE_THREADS = 32 * (CONSUMER_WARPS + 1 + ROPE_HELPERS * CONSUMER_WARPS);
 constexpr int ROPE_TEAM_THREADS = 32 * (1 + ROPE_HELPERS);
-static_assert(CONSUMER_WARPS + 1 == 4 && ROPE_HELPERS == 4, "register hand-over is per warpgroup: owners + producer, then helpers");
-constexpr int REC = 4 + 2 * 128;             // m, l, value-scale, pad, acc_v[128], acc_k[128]
-constexpr int SMEM_BYTES = SLOTS * SLOT_BYTES + 1024;   // + alignment slack; barriers live in static smem
+template <int D, bool ROPE> struct Cfg {
+    static constexpr int HALF_BYTES = 64 * 2 * D;                    // 64 rows as D / 64 swizzled boxes
+    static constexpr int SLOT_BYTES = 2 * HALF_BYTES;                // retained: K | V; key-only: keys 0-63 | keys 64-127
+    // With 64-channel heads a softmax step brings in half the bytes for the same softmax arithmetic: a fourth consumer
+    // warp (one to a warp scheduler) makes up for it.  The RoPE block keeps three (its helper warps fill it).
+    // Measured: 512 units, 1639 retained + 3276 key-only rows, 431 MB: 87 us with the appended row = 4.9 TB/s (856 us on
+    // CUDA cores).
+    static constexpr int CONSUMER_WARPS = D == 128 || ROPE ? 3 : 4;
+    static constexpr int SLOTS = D == 128 ? 6 : 12;                  // a multiple of CONSUMER_WARPS: a slot always serves the same warp
+    static constexpr int THREADS = 32 * (CONSUMER_WARPS + 1 + (ROPE ? ROPE_HELPERS * CONSUMER_WARPS : 0));
+    static constexpr int SMEM_BYTES = SLOTS * SLOT_BYTES + 1024;     // + alignment slack; barriers live in static smem
+    static constexpr int REC = 4 + 2 * D;                            // m, l, value-scale, pad, acc_v[D], acc_k[D]
+    static_assert(SLOTS % CONSUMER_WARPS == 0, "a slot must always be consumed by the same warp");
+    static_assert(!ROPE || (CONSUMER_WARPS + 1 == 4 && ROPE_HELPERS == 4), "register hand-over is per warpgroup: owners + producer, then helpers");
+};
+constexpr int REC = Cfg<128, false>::REC;
 
 // How the tile sequence is dealt to blocks; the same arithmetic runs on host and device.
 struct Plan {
@@ -125,33 +132,36 @@ __device__ __forceinline__ uint32_t pack_bf16(float lo, float hi) {
     return *reinterpret_cast<uint32_t*>(&v);
 }
 
-// RoPE decoupling: rows 16 member .. 16 member + 15 of the 64 keys at kbase (two swizzled boxes:
-// channels 0-63 | 64-127) are turned back by their positions, in place, and left there as fp16 (a
+// RoPE decoupling: rows 16 member .. 16 member + 15 of the 64 keys at kbase (swizzled boxes of 64
+// channels) are turned back by their positions, in place, and left there as fp16 (a
 // turned key is not a bf16 number; eleven bits keep the key sum within the tolerance of the output,
 // eight do not; |k| beyond 65504 saturates).  Channel c pairs with
-// c + 64; the angle is position * theta^(-2c/128), taken as the 32-bit product of the position and
+// c + D/2; the angle is position * theta^(-2c/D), taken as the 32-bit product of the position and
 // the per-channel phase (turns per position as a fraction of 2^32), which is the angle modulo one turn.  pos16: lane l
 // holds the position of row 16 member + (l & 15).
+template <int D>
 __device__ __forceinline__ void derotate_rows(uint32_t kbase, int nrows, int member, uint32_t pos16,
                                               const uint32_t* phase_s, int lane) {
-    const int qc = lane & 7;                                        // 16-byte chunk: channel pairs 8 qc .. 8 qc + 7
+    constexpr int LPR = D / 16, RPP = 32 / LPR;                     // lanes a row, rows the warp takes at a time
+    const int qc = lane & (LPR - 1);                                // 16-byte chunk: channel pairs 8 qc .. 8 qc + 7
     uint32_t phase[8];                                              // this lane's eight channel pairs
 #pragma unroll
     for (int c = 0; c < 8; ++c) phase[c] = phase_s[qc * 8 + c];
 #pragma unroll 1
-    for (int j = 0; j < 4; j += 2) {
+    for (int j = 0; j < 16 / RPP; j += 2) {
         // two rows per round, the loads of both ahead of the stores
-        uint32_t off[2], pos[2], xs[2][4], ys[2][4];
+        uint32_t off[2], yoff[2], pos[2], xs[2][4], ys[2][4];
         bool live[2];
 #pragma unroll
         for (int u = 0; u < 2; ++u) {
-            const int rl = 4 * (j + u) + (lane >> 3), r = 16 * member + rl;
+            const int rl = RPP * (j + u) + lane / LPR, r = 16 * member + rl;
             pos[u] = __shfl_sync(0xffffffffu, pos16, rl);
             live[u] = r < nrows;
             off[u] = (uint32_t)r * 128u + (uint32_t)((qc ^ (r & 7)) << 4);
+            yoff[u] = D == 128 ? off[u] + BOX_BYTES : (uint32_t)r * 128u + (uint32_t)(((qc + LPR) ^ (r & 7)) << 4);   // the partner channels
             if (live[u]) {
                 asm volatile("ld.shared.v4.u32 {%0,%1,%2,%3}, [%4];\n" : "=r"(xs[u][0]), "=r"(xs[u][1]), "=r"(xs[u][2]), "=r"(xs[u][3]) : "r"(kbase + off[u]));
-                asm volatile("ld.shared.v4.u32 {%0,%1,%2,%3}, [%4];\n" : "=r"(ys[u][0]), "=r"(ys[u][1]), "=r"(ys[u][2]), "=r"(ys[u][3]) : "r"(kbase + BOX_BYTES + off[u]));
+                asm volatile("ld.shared.v4.u32 {%0,%1,%2,%3}, [%4];\n" : "=r"(ys[u][0]), "=r"(ys[u][1]), "=r"(ys[u][2]), "=r"(ys[u][3]) : "r"(kbase + yoff[u]));
             } else {
 #pragma unroll
                 for (int e = 0; e < 4; ++e) { xs[u][e] = 0u; ys[u][e] = 0u; }
@@ -181,7 +191,7 @@ __device__ __forceinline__ void derotate_rows(uint32_t kbase, int nrows, int mem
         for (int u = 0; u < 2; ++u) {
             if (live[u]) {
                 asm volatile("st.shared.v4.u32 [%0], {%1,%2,%3,%4};\n" ::"r"(kbase + off[u]), "r"(xs[u][0]), "r"(xs[u][1]), "r"(xs[u][2]), "r"(xs[u][3]) : "memory");
-                asm volatile("st.shared.v4.u32 [%0], {%1,%2,%3,%4};\n" ::"r"(kbase + BOX_BYTES + off[u]), "r"(ys[u][0]), "r"(ys[u][1]), "r"(ys[u][2]), "r"(ys[u][3]) : "memory");
+                asm volatile("st.shared.v4.u32 [%0], {%1,%2,%3,%4};\n" ::"r"(kbase + yoff[u]), "r"(ys[u][0]), "r"(ys[u][1]), "r"(ys[u][2]), "r"(ys[u][3]) : "memory");
             }
         }
     }
@@ -193,20 +203,20 @@ __device__ __forceinline__ void team_sync(int team) {
     asm volatile("bar.sync %0, %1;\n" ::"r"(2 + team), "n"(ROPE_TEAM_THREADS) : "memory");
 }
 
-static_assert(SLOTS % CONSUMER_WARPS == 0, "a slot must always be consumed by the same warp");
-
 struct Maps {
-    CUtensorMap ret_k, ret_v, apx_k;     // rank 3: (128 dims, pool rows, U units), box 64 x 64 x 1, 128B swizzle
+    CUtensorMap ret_k, ret_v, apx_k;     // rank 3: (D dims, pool rows, U units), box 64 x 64 x 1, 128B swizzle
 };
 
-// grid (plan.B), THREADS threads, SMEM_BYTES dynamic shared memory.
+// grid (plan.B), Cfg::THREADS threads, Cfg::SMEM_BYTES dynamic shared memory.
 // partial: [U][s_max][CONSUMER_WARPS][g][REC]; slot of (unit u, block b) = b - block_of_tile(first tile of u).
-template <bool ROPE>
-__global__ void __launch_bounds__(ROPE ? ROPE_THREADS : THREADS, 1)
-decode_stream_bf16_d128(const __nv_bfloat16* __restrict__ q, const __grid_constant__ Maps maps, Plan pl, int n_ret,
+template <int D, bool ROPE>
+__global__ void __launch_bounds__(Cfg<D, ROPE>::THREADS, 1)
+decode_stream_bf16(const __nv_bfloat16* __restrict__ q, const __grid_constant__ Maps maps, Plan pl, int n_ret,
                         int n_apx, int g, int LH, float scale_log2e, float* __restrict__ partial,
                         int* __restrict__ fault, const int32_t* __restrict__ apx_pos, long long cap_apx,
                         const __grid_constant__ RopePhases rope) {
+    constexpr int HALF_BYTES = Cfg<D, ROPE>::HALF_BYTES, SLOT_BYTES = Cfg<D, ROPE>::SLOT_BYTES, SLOTS = Cfg<D, ROPE>::SLOTS;
+    constexpr int CONSUMER_WARPS = Cfg<D, ROPE>::CONSUMER_WARPS, REC = Cfg<D, ROPE>::REC, BOXES = D / 64;
     extern __shared__ unsigned char smem_raw[];
     __shared__ uint32_t phase_s[ROPE ? 64 : 1];          // the phases rounded to 32 bits
     if (ROPE && threadIdx.x < 64) phase_s[threadIdx.x] = (uint32_t)((rope.phase[threadIdx.x] + 0x80000000ull) >> 32);
@@ -258,10 +268,10 @@ decode_stream_bf16_d128(const __nv_bfloat16* __restrict__ q, const __grid_consta
                 if (!team_ok[team]) continue;
                 const uint32_t base = tma::smem_u32(smem + (i % SLOTS) * SLOT_BYTES);
                 team_sync(team);                                   // the owner has its scores of half 0
-                derotate_rows(base, n0, member, p0, phase_s, lane);
+                derotate_rows<D>(base, n0, member, p0, phase_s, lane);
                 team_sync(team);                                   // ... and of half 1, if there is one
                 if (n1 > 0) {
-                    derotate_rows(base + HALF_BYTES, n1, member, p1, phase_s, lane);
+                    derotate_rows<D>(base + HALF_BYTES, n1, member, p1, phase_s, lane);
                     team_sync(team);
                 }
             }
@@ -283,16 +293,18 @@ decode_stream_bf16_d128(const __nv_bfloat16* __restrict__ q, const __grid_consta
                 tma::mbar_expect_tx(&full_bar[s], SLOT_BYTES);
                 if (t < pl.n_rt) {
                     const int row0 = t * KEYS;
-                    tma::load_3d_hint(st, &maps.ret_k, 0, row0, u, &full_bar[s], pol);
-                    tma::load_3d_hint(st + BOX_BYTES, &maps.ret_k, 64, row0, u, &full_bar[s], pol);
-                    tma::load_3d_hint(st + HALF_BYTES, &maps.ret_v, 0, row0, u, &full_bar[s], pol);
-                    tma::load_3d_hint(st + HALF_BYTES + BOX_BYTES, &maps.ret_v, 64, row0, u, &full_bar[s], pol);
+#pragma unroll
+                    for (int x = 0; x < BOXES; ++x) {
+                        tma::load_3d_hint(st + x * BOX_BYTES, &maps.ret_k, 64 * x, row0, u, &full_bar[s], pol);
+                        tma::load_3d_hint(st + HALF_BYTES + x * BOX_BYTES, &maps.ret_v, 64 * x, row0, u, &full_bar[s], pol);
+                    }
                 } else {
                     const int row0 = (t - pl.n_rt) * 2 * KEYS;
-                    tma::load_3d_hint(st, &maps.apx_k, 0, row0, u, &full_bar[s], pol);
-                    tma::load_3d_hint(st + BOX_BYTES, &maps.apx_k, 64, row0, u, &full_bar[s], pol);
-                    tma::load_3d_hint(st + HALF_BYTES, &maps.apx_k, 0, row0 + KEYS, u, &full_bar[s], pol);
-                    tma::load_3d_hint(st + HALF_BYTES + BOX_BYTES, &maps.apx_k, 64, row0 + KEYS, u, &full_bar[s], pol);
+#pragma unroll
+                    for (int x = 0; x < BOXES; ++x) {
+                        tma::load_3d_hint(st + x * BOX_BYTES, &maps.apx_k, 64 * x, row0, u, &full_bar[s], pol);
+                        tma::load_3d_hint(st + HALF_BYTES + x * BOX_BYTES, &maps.apx_k, 64 * x, row0 + KEYS, u, &full_bar[s], pol);
+                    }
                 }
                 if (++t == pl.n_tiles) { t = 0; ++u; }
             }
@@ -308,8 +320,8 @@ decode_stream_bf16_d128(const __nv_bfloat16* __restrict__ q, const __grid_consta
     const uint32_t pv_row = (uint32_t)(r8 + (mat & 1) * 8) * 128u;       // PV: matrices = (chunk lo|hi) x (keys 0-7|8-15)
     const uint32_t pv_x = (uint32_t)(((mat >> 1) ^ r8) << 4);
 
-    uint32_t qa[8][2];
-    float acc[16][4];                  // [dim tile][c0,c1: P_hi rows | c2,c3: P_lo rows]
+    uint32_t qa[D / 16][2];
+    float acc[D / 8][4];                  // [dim tile][c0,c1: P_hi rows | c2,c3: P_lo rows]
     float m = -INFINITY, l = 0.f, stash_scale = 1.f;
     bool stashed = false;
 
@@ -319,21 +331,21 @@ decode_stream_bf16_d128(const __nv_bfloat16* __restrict__ q, const __grid_consta
         return partial + ((((size_t)unit * pl.s_max + slot) * CONSUMER_WARPS + wq) * g + gid) * REC;
     };
     auto load_q = [&](int unit) {
-        const uint32_t* qrow = reinterpret_cast<const uint32_t*>(q + ((size_t)unit * g + min(gid, g - 1)) * 128);
+        const uint32_t* qrow = reinterpret_cast<const uint32_t*>(q + ((size_t)unit * g + min(gid, g - 1)) * D);
 #pragma unroll
-        for (int ks = 0; ks < 8; ++ks) {
+        for (int ks = 0; ks < D / 16; ++ks) {
             qa[ks][0] = gid < g ? qrow[ks * 8 + tig] : 0u;
             qa[ks][1] = gid < g ? qrow[ks * 8 + 4 + tig] : 0u;
         }
     };
     auto store_acc = [&](float* dst) {       // dims n*8 + 2 tig + {0,1} of head row gid
 #pragma unroll
-        for (int n = 0; n < 16; ++n)
+        for (int n = 0; n < D / 8; ++n)
             *reinterpret_cast<float2*>(dst + n * 8 + 2 * tig) = make_float2(acc[n][0] + acc[n][2], acc[n][1] + acc[n][3]);
     };
     auto zero_acc = [&]() {
 #pragma unroll
-        for (int n = 0; n < 16; ++n) { acc[n][0] = acc[n][1] = acc[n][2] = acc[n][3] = 0.f; }
+        for (int n = 0; n < D / 8; ++n) { acc[n][0] = acc[n][1] = acc[n][2] = acc[n][3] = 0.f; }
     };
     // Writes this warp's record of `unit` (an all-zero one with m = -inf if it met none of its tiles).
     auto flush = [&](int unit) {
@@ -343,26 +355,26 @@ decode_stream_bf16_d128(const __nv_bfloat16* __restrict__ q, const __grid_consta
         if (gid < g) {
             float* rec = record_of(unit);
             if (tig == 0) *reinterpret_cast<float4*>(rec) = make_float4(m * 0.69314718055994531f, lt, stashed ? stash_scale : 1.f, 0.f);
-            if (stashed) store_acc(rec + 4 + 128);      // value part was written at the pool switch
+            if (stashed) store_acc(rec + 4 + D);      // value part was written at the pool switch
             else {
                 store_acc(rec + 4);
 #pragma unroll
-                for (int n = 0; n < 16; ++n) *reinterpret_cast<float2*>(rec + 4 + 128 + n * 8 + 2 * tig) = make_float2(0.f, 0.f);
+                for (int n = 0; n < D / 8; ++n) *reinterpret_cast<float2*>(rec + 4 + D + n * 8 + 2 * tig) = make_float2(0.f, 0.f);
             }
         }
         zero_acc();
         m = -INFINITY; l = 0.f; stash_scale = 1.f; stashed = false;
     };
-    // One softmax step over the 64 keys at kbase (two swizzled boxes), in two parts.  The first
+    // One softmax step over the 64 keys at kbase (D / 64 swizzled boxes), in two parts.  The first
     // leaves the step's weights p in sc (this thread: head gid, keys 8 n + 2 tig, + 1), brings m, l
     // and the accumulators to the new running maximum and returns the factor it applied to them.
     auto scores64 = [&](uint32_t kbase, int nrows, bool retained, int unit, float (&sc)[8][2]) -> float {
-        // ---- S = Q K^T: eight 8-key column tiles, each its own accumulator chain over the 8 k-steps
+        // ---- S = Q K^T: eight 8-key column tiles, each its own accumulator chain over the D / 16 k-steps
         float zz[2];
 #pragma unroll
         for (int n = 0; n < 8; ++n) { sc[n][0] = 0.f; sc[n][1] = 0.f; }
 #pragma unroll
-        for (int ks = 0; ks < 8; ++ks) {
+        for (int ks = 0; ks < D / 16; ++ks) {
 #pragma unroll
             for (int j = 0; j < 4; ++j) {          // 16 keys per ldmatrix
                 uint32_t b0, b1, b2, b3;
@@ -404,14 +416,14 @@ decode_stream_bf16_d128(const __nv_bfloat16* __restrict__ q, const __grid_consta
         if (__any_sync(0xffffffffu, alpha != 1.f)) {
             {
 #pragma unroll
-                for (int n = 0; n < 16; ++n) { acc[n][0] *= alpha; acc[n][1] *= alpha; acc[n][2] *= alpha; acc[n][3] *= alpha; }
+                for (int n = 0; n < D / 8; ++n) { acc[n][0] *= alpha; acc[n][1] *= alpha; acc[n][2] *= alpha; acc[n][3] *= alpha; }
             }
         }
         return alpha;
     };
     // The second part adds p x (the 64 rows at vbase: values, or the keys themselves for a key-only tile).
     auto accumulate64 = [&](uint32_t vbase, bool retained, float (&sc)[8][2]) {
-        // ---- accumulate P x (V rows | K rows): four k-steps of 16 keys x 16 column tiles of 8 dims
+        // ---- accumulate P x (V rows | K rows): four k-steps of 16 keys x D / 8 column tiles of 8 dims
 #pragma unroll
         for (int kk = 0; kk < 4; ++kk) {
             // P as bf16 hi (MMA rows 0-7) + lo (rows 8-15)
@@ -421,7 +433,7 @@ decode_stream_bf16_d128(const __nv_bfloat16* __restrict__ q, const __grid_consta
                 const uint32_t a0 = pack_f16(p00, p01), a2 = pack_f16(p10, p11);
                 const uint32_t a1 = pack_f16(p00 - f16_lo(a0), p01 - f16_hi(a0)), a3 = pack_f16(p10 - f16_lo(a2), p11 - f16_hi(a2));
 #pragma unroll
-                for (int np = 0; np < 8; ++np) {
+                for (int np = 0; np < D / 16; ++np) {
                     uint32_t b0, b1, b2, b3;
                     ldsm_x4_t(vbase + (np >> 2) * BOX_BYTES + kk * 16 * 128 + pv_row + ((((2 * np) & 7) << 4) ^ pv_x), b0, b1, b2, b3);
                     mma_16_f16(acc[2 * np], a0, a1, a2, a3, b0, b1);
@@ -436,7 +448,7 @@ decode_stream_bf16_d128(const __nv_bfloat16* __restrict__ q, const __grid_consta
             const uint32_t a1 = pack_bf16(p00 - __bfloat162float(h00), p01 - __bfloat162float(h01));
             const uint32_t a3 = pack_bf16(p10 - __bfloat162float(h10), p11 - __bfloat162float(h11));
 #pragma unroll
-            for (int np = 0; np < 8; ++np) {
+            for (int np = 0; np < D / 16; ++np) {
                 uint32_t b0, b1, b2, b3;
                 ldsm_x4_t(vbase + (np >> 2) * BOX_BYTES + kk * 16 * 128 + pv_row + ((((2 * np) & 7) << 4) ^ pv_x), b0, b1, b2, b3);
                 mma_16(acc[2 * np], a0, a1, a2, a3, b0, b1);
@@ -509,44 +521,45 @@ decode_stream_bf16_d128(const __nv_bfloat16* __restrict__ q, const __grid_consta
     }
 }
 
-// Merge for head_dim 128: grid (U), 128 g threads -- thread (a, c) owns output dim c of head a.
+// Merge: grid (U), D g threads -- thread (a, c) owns output dim c of head a.
 // Combines the records of a unit, applies the unit's map to the p-weighted key sum and normalises:
 //   o = (sum_j f_j s_j acc_v_j + W sum_j f_j acc_k_j) / sum_j f_j l_j,   f_j = exp(m_j - max m).
 // Every load of a phase is independent of the others, so a phase costs one memory latency.
-// The product W (sum f acc_k) runs on warp-level MMAs, M = 128 output channels (warp w takes rows 16 w ..),
-// N = the unit's g query heads (padded to 8), K = 128: the A fragments are read straight from the map in
+// The product W (sum f acc_k) runs on warp-level MMAs, M = D output channels (warp w takes rows 16 w ..),
+// N = the unit's g query heads (padded to 8), K = D: the A fragments are read straight from the map in
 // global memory, 16 bytes a load -- thread (row r, quarter t) of a warp holds columns 8 (t + 4 jj) .. + 7 of
 // rows r and r + 8, and the k slots of MMA step 2 jj + h stand for columns 8 (t + 4 jj) + 4 h .. + 3, which the
 // B fragments follow; the key sum enters as bf16 hi + lo (sixteen mantissa bits), the map's elements are bf16
 // as stored.
-template <typename TO, int MAXT>
+template <typename TO, int D, int MAXT>
 __global__ void __launch_bounds__(MAXT, MAXT == 512 ? 3 : 1)
-decode_merge_bf16_d128(const float* __restrict__ partial, const __nv_bfloat16* __restrict__ W, int LH, int g,
+decode_merge_bf16(const float* __restrict__ partial, const __nv_bfloat16* __restrict__ W, int LH, int g,
                        Plan pl, int apply_w, int cw, TO* __restrict__ out) {
-    __shared__ __align__(16) __nv_bfloat16 akh[8][128], akl[8][128];      // key sums per head, hi and lo halves
-    __shared__ float pw[8][128];               // W times the key sum
+    constexpr int REC = 4 + 2 * D, PIECES = D / 8;                  // 16-byte pieces of a row of W
+    __shared__ __align__(16) __nv_bfloat16 akh[8][D], akl[8][D];          // key sums per head, hi and lo halves
+    __shared__ float pw[8][D];                 // W times the key sum
     __shared__ float fv[8][48], fk[8][48];     // per head, per record: factor for the value part / the key part
     __shared__ float Ls[8];
-    const int u = blockIdx.x, tid = threadIdx.x, a = tid >> 7, c = tid & 127, lane = tid & 31;
+    const int u = blockIdx.x, tid = threadIdx.x, a = tid / D, c = tid % D, lane = tid & 31;
     const int wid = tid >> 5, nwarps = blockDim.x >> 5, row = lane >> 2, quarter = lane & 3;
     // A fragments of 16 rows of W (the maps of a layer stay in L2: every sequence of the batch reads them)
-    const uint4* Wu = reinterpret_cast<const uint4*>(W + (size_t)(u % LH) * 128 * 128);       // 16 pieces per 256-byte row
-    uint4 A[8];
+    const uint4* Wu = reinterpret_cast<const uint4*>(W + (size_t)(u % LH) * D * D);
+    uint4 A[D / 16];
     auto load_rows = [&](int mt) {
 #pragma unroll
-        for (int jj = 0; jj < 4; ++jj) {
-            A[2 * jj + 0] = Wu[(16 * mt + row) * 16 + quarter + 4 * jj];
-            A[2 * jj + 1] = Wu[(16 * mt + row + 8) * 16 + quarter + 4 * jj];
+        for (int jj = 0; jj < D / 32; ++jj) {
+            A[2 * jj + 0] = Wu[(16 * mt + row) * PIECES + quarter + 4 * jj];
+            A[2 * jj + 1] = Wu[(16 * mt + row + 8) * PIECES + quarter + 4 * jj];
         }
     };
-    for (int i = tid; i < (8 - g) * 128; i += blockDim.x) {       // columns of B beyond the unit's heads
-        akh[g + i / 128][i % 128] = __float2bfloat16_rn(0.f);
-        akl[g + i / 128][i % 128] = __float2bfloat16_rn(0.f);
+    for (int i = tid; i < (8 - g) * D; i += blockDim.x) {         // columns of B beyond the unit's heads
+        akh[g + i / D][i % D] = __float2bfloat16_rn(0.f);
+        akl[g + i / D][i % D] = __float2bfloat16_rn(0.f);
     }
     // everything above reads only W, which the streaming kernel does not write; its records from here on
     asm volatile("griddepcontrol.wait;\n" ::: "memory");
     const int first = block_of_tile((long long)u * pl.n_tiles, pl);
-    const int n_rec = (block_of_tile((long long)(u + 1) * pl.n_tiles - 1, pl) - first + 1) * cw;   // <= 36; cw records per block
+    const int n_rec = (block_of_tile((long long)(u + 1) * pl.n_tiles - 1, pl) - first + 1) * cw;   // <= 48; cw records per block
     const float* base = partial + (size_t)u * pl.s_max * cw * g * REC;
     // The first six records' sums are requested before the headers are looked at, so that the two loads
     // share one memory latency (a unit lies in one or two blocks of the streaming kernel, three records
@@ -558,7 +571,7 @@ decode_merge_bf16_d128(const float* __restrict__ partial, const __nv_bfloat16* _
         const int j = min(k, n_rec - 1);
         const float* r = base + ((size_t)j * g + a) * REC + 4;
         rv[k] = r[c];
-        rk[k] = r[128 + c];
+        rk[k] = r[D + c];
     }
     if (c < 32) {
         // first warp of head a: headers of records lane and lane + 32
@@ -593,7 +606,7 @@ decode_merge_bf16_d128(const float* __restrict__ partial, const __nv_bfloat16* _
                 const int j = min(j0 + k, n_rec - 1);
                 const float* r = base + ((size_t)j * g + a) * REC + 4;
                 rv[k] = r[c];
-                rk[k] = r[128 + c];
+                rk[k] = r[D + c];
             }
         }
 #pragma unroll
@@ -605,7 +618,7 @@ decode_merge_bf16_d128(const float* __restrict__ partial, const __nv_bfloat16* _
         }
     }
     if (!apply_w) {           // per-tile form: the second part of a record is already sum p (W k)
-        store_out(out + ((size_t)u * g + a) * 128 + c, (av + ak) / Ls[a]);
+        store_out(out + ((size_t)u * g + a) * D + c, (av + ak) / Ls[a]);
         return;
     }
     {
@@ -614,11 +627,11 @@ decode_merge_bf16_d128(const float* __restrict__ partial, const __nv_bfloat16* _
         akl[a][c] = __float2bfloat16_rn(ak - __bfloat162float(hi));
     }
     __syncthreads();
-    for (int mt = wid; mt < 8; mt += nwarps) {
+    for (int mt = wid; mt < D / 16; mt += nwarps) {
         load_rows(mt);
         float d[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll
-        for (int jj = 0; jj < 4; ++jj) {
+        for (int jj = 0; jj < D / 32; ++jj) {
             const uint4 r0 = A[2 * jj], r1 = A[2 * jj + 1];
             const int col = 8 * (quarter + 4 * jj);
             const uint4 bh = *reinterpret_cast<const uint4*>(&akh[row][col]);      // B column = head `row`
@@ -633,7 +646,7 @@ decode_merge_bf16_d128(const float* __restrict__ partial, const __nv_bfloat16* _
         if (2 * quarter + 1 < g) { pw[2 * quarter + 1][16 * mt + row] = d[1]; pw[2 * quarter + 1][16 * mt + row + 8] = d[3]; }
     }
     __syncthreads();
-    store_out(out + ((size_t)u * g + a) * 128 + c, (av + pw[a][c]) / Ls[a]);
+    store_out(out + ((size_t)u * g + a) * D + c, (av + pw[a][c]) / Ls[a]);
 }
 
 }  // namespace dbf
