@@ -31,7 +31,7 @@ namespace vec {
 namespace rlt {
 
 using rtc::BOX_BYTES;
-using rtc::OPERAND_BYTES;
+constexpr int OPERAND_BYTES = rtc::RCfg<128, false>::OPERAND_BYTES;
 using rtc::TILE;
 
 constexpr int STAGES = 3;

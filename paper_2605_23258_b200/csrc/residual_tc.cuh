@@ -1,19 +1,20 @@
-// Reconstruction residual of Step 2 on the tensor cores (bf16, head_dim 128):
+// Reconstruction residual of Step 2 on the tensor cores (bf16, head_dim D = 64 or 128):
 //   eps[p] = || v_i - W k~_i ||^2,  i = idx[p],  k~ = the key, or under RoPE decoupling the key
-//   turned back by its position (the token index itself), channel c pairing with c + 64.
+//   turned back by its position (the token index itself), channel c pairing with c + D/2.
 // The gather of the listed K and V rows is what costs (64 flop per byte: HBM-bound), so the
 // kernel is built around keeping row loads in flight.  Per 128-row tile the accumulator in tensor
-// memory is D = K_tile W^T (one chain of 8 tcgen05.mma); the epilogue subtracts the value row,
+// memory is K_tile W^T (one chain of D / 16 tcgen05.mma); the epilogue subtracts the value row,
 // which it reads from the tile's copy in shared memory, squares and adds along its TMEM lane.
 //
 // Persistent blocks (one per SM) own equal contiguous ranges of the global tile sequence.
-//   warps 0-7   loaders: cp.async gathers of K and V rows into the stages, written directly in the
-//               128-byte-swizzled layout the MMA reads; row indices are fetched one tile ahead.
+//   loaders     (8 warps) cp.async gathers of K and V rows into the stages, written directly
+//               in the 128-byte-swizzled layout the MMA reads; row indices are fetched one tile ahead.
 //               Each thread gathers, for its rows, the 16-byte chunk qc of both key halves
-//               (channels 8 qc.. and 64 + 8 qc..) and the same two chunks of V.
-//   warp  8     MMA issuer, TMEM owner; also TMA-loads the unit's W when the range enters a new unit
-//   warps 9-12  epilogue: thread = row
-// Without RoPE: three stages of K | V (64 KB each), tiles published two behind the one being issued.
+//               (channels 8 qc.. and D/2 + 8 qc..) and the same two chunks of V.
+//   one warp    MMA issuer, TMEM owner; also TMA-loads the unit's W when the range enters a new unit
+//   4 warps     epilogue: thread = row
+// Without RoPE: stages of K | V (three of 64 KB at D = 128, five of 32 KB at D = 64), tiles published
+// all stages but one behind the one being issued: 128 KB of row loads stay in flight.
 // With RoPE: the turned key is no longer a bf16 number, so it goes to the tensor cores as a bf16
 // pair hi + lo (two chains over the same W), which keeps it to 2^-17 relative; two stages of
 // K hi | K lo | V (96 KB each).  A loader thread turns its own eight channel pairs of each of its
@@ -32,7 +33,6 @@ namespace rtc {
 
 constexpr int BOX_BYTES = 16384;                           // 128 rows x 128 bytes
 constexpr int TILE = 128;
-constexpr int OPERAND_BYTES = 2 * BOX_BYTES;               // 128 rows x 256 B as two swizzled halves
 constexpr int EPI_WARPS = 4;
 
 struct Params {
@@ -53,30 +53,35 @@ __device__ __forceinline__ uint32_t pack2_bf16(float lo, float hi) {
 }
 __device__ __forceinline__ long long range_begin(int b, long long n_tiles, int B) { return (long long)b * n_tiles / B; }
 
-constexpr int R_LOADER_WARPS = 8;
-constexpr int R_THREADS = 32 * (R_LOADER_WARPS + 1 + EPI_WARPS);
-template <bool ROPE> struct RCfg {
-    static constexpr int STAGES = ROPE ? 2 : 3;
+template <int D, bool ROPE> struct RCfg {
+    static constexpr int OPERAND_BYTES = (D / 64) * BOX_BYTES;     // 128 rows of D bf16 as D / 64 swizzled boxes
+    static constexpr int W_BYTES = 2 * D * D;
+    static constexpr int STAGES = ROPE ? 2 : D == 128 ? 3 : 5;
     static constexpr int STAGE_BYTES = (ROPE ? 3 : 2) * OPERAND_BYTES;
     static constexpr int V_OFFSET = (ROPE ? 2 : 1) * OPERAND_BYTES;
-    static constexpr int SMEM_BYTES = STAGES * STAGE_BYTES + OPERAND_BYTES + 1024;     // + W
-    static constexpr int TMEM_COLS = ROPE ? 256 : 512;          // one 128-column accumulator per stage
+    static constexpr int SMEM_BYTES = STAGES * STAGE_BYTES + W_BYTES + 1024;
+    static constexpr int TMEM_COLS = STAGES * D <= 128 ? 128 : STAGES * D <= 256 ? 256 : 512;   // one D-column accumulator per stage
+    static constexpr int LOADER_WARPS = 8;
+    static constexpr int THREADS = 32 * (LOADER_WARPS + 1 + EPI_WARPS);
 };
 struct RSync {
-    uint64_t full[3], done[3], empty[3];
+    uint64_t full[5], done[5], empty[5];
     uint64_t w_full, w_empty;
     uint32_t tmem_base;
 };
 
-// grid: min(multiprocessors, n_tiles) blocks, R_THREADS threads, RCfg<ROPE>::SMEM_BYTES dynamic shared memory.
-template <bool ROPE>
-__global__ void __launch_bounds__(R_THREADS, 1)
+// grid: min(multiprocessors, n_tiles) blocks, RCfg::THREADS threads, RCfg::SMEM_BYTES dynamic shared memory.
+template <int D, bool ROPE>
+__global__ void __launch_bounds__(RCfg<D, ROPE>::THREADS, 1)
 residual_tc(const __nv_bfloat16* __restrict__ K, const __nv_bfloat16* __restrict__ V,
                  const __grid_constant__ CUtensorMap mapW, const int32_t* __restrict__ idx, const Params P,
                  const __grid_constant__ RopePhases rope, float* __restrict__ eps, int* __restrict__ fault) {
     extern __shared__ unsigned char smem_raw[];
     __shared__ RSync sy;
-    constexpr int STAGES = RCfg<ROPE>::STAGES, R_STAGE_BYTES = RCfg<ROPE>::STAGE_BYTES, TMEM_COLS = RCfg<ROPE>::TMEM_COLS;
+    using C = RCfg<D, ROPE>;
+    constexpr int STAGES = C::STAGES, R_STAGE_BYTES = C::STAGE_BYTES, TMEM_COLS = C::TMEM_COLS, R_LOADER_WARPS = C::LOADER_WARPS;
+    constexpr int OPERAND_BYTES = C::OPERAND_BYTES;
+    constexpr int LPR = D / 16, RPP = 32 * R_LOADER_WARPS / LPR, PASSES = TILE / RPP;    // loader threads a row, rows a pass, passes
     __shared__ unsigned long long phase_s[64];
     unsigned char* smem = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
     unsigned char* stage0 = smem;
@@ -112,30 +117,33 @@ residual_tc(const __nv_bfloat16* __restrict__ K, const __nv_bfloat16* __restrict
 
     if (warp < R_LOADER_WARPS) {
         // ------------------------------------------------------------------ loaders
-        const int qc = tid & 7, rsub = tid >> 3;                    // chunk of each half, row inside a pass of 32 rows
-        const uint32_t dst_thread = (uint32_t)rsub * 128u + (uint32_t)((qc ^ (rsub & 7)) << 4);   // + half * BOX + pass * 4096
+        const int qc = tid & (LPR - 1), rsub = tid / LPR;           // chunk of each half, row inside a pass
+        const uint32_t dst_thread = (uint32_t)rsub * 128u + (uint32_t)((qc ^ (rsub & 7)) << 4);   // + pass * PASS_BYTES
+        // the same chunk of the other half: in the second box, or LPR chunks further in the row
+        const uint32_t other = D == 128 ? (uint32_t)BOX_BYTES : (uint32_t)(((qc + LPR) ^ (rsub & 7)) << 4) - (uint32_t)((qc ^ (rsub & 7)) << 4);
+        constexpr uint32_t PASS_BYTES = RPP * 128;
         uint2 fr[8];                                                 // phases of this thread's eight channel pairs
 #pragma unroll
         for (int e = 0; e < 8; ++e) fr[e] = reinterpret_cast<const uint2*>(phase_s)[qc * 8 + e];
-        int32_t prev[4], cur[4], nxt[4];
-        auto fetch_idx = [&](int i, int32_t (&out)[4]) {
+        int32_t prev[PASSES], cur[PASSES], nxt[PASSES];
+        auto fetch_idx = [&](int i, int32_t (&out)[PASSES]) {
             const long long gt = gt_lo + i;
             const int u = (int)(gt / P.tpu), t = (int)(gt - (long long)u * P.tpu);
 #pragma unroll
-            for (int p = 0; p < 4; ++p) {
-                const int row = t * TILE + p * 32 + rsub;
+            for (int p = 0; p < PASSES; ++p) {
+                const int row = t * TILE + p * RPP + rsub;
                 const int32_t v = row < P.n_idx ? idx[(size_t)u * P.n_idx + row] : -1;
                 out[p] = (unsigned long long)v < (unsigned long long)P.N ? v : -1;   // an index outside the unit reads as a row of zeros
             }
         };
         // Turns this thread's pairs of the tile in stage s (rows listed in pos) and publishes the tile.
-        auto turn_back = [&](int s, const int32_t (&pos)[4]) {
+        auto turn_back = [&](int s, const int32_t (&pos)[PASSES]) {
             const uint32_t hi0 = tma::smem_u32(stage0 + s * R_STAGE_BYTES) + dst_thread, lo0 = hi0 + OPERAND_BYTES;
 #pragma unroll
-            for (int p = 0; p < 4; ++p) {
+            for (int p = 0; p < PASSES; ++p) {
                 uint32_t xs[4], ys[4], xl[4], yl[4];
-                asm volatile("ld.shared.v4.u32 {%0,%1,%2,%3}, [%4];\n" : "=r"(xs[0]), "=r"(xs[1]), "=r"(xs[2]), "=r"(xs[3]) : "r"(hi0 + p * 4096));
-                asm volatile("ld.shared.v4.u32 {%0,%1,%2,%3}, [%4];\n" : "=r"(ys[0]), "=r"(ys[1]), "=r"(ys[2]), "=r"(ys[3]) : "r"(hi0 + BOX_BYTES + p * 4096));
+                asm volatile("ld.shared.v4.u32 {%0,%1,%2,%3}, [%4];\n" : "=r"(xs[0]), "=r"(xs[1]), "=r"(xs[2]), "=r"(xs[3]) : "r"(hi0 + p * PASS_BYTES));
+                asm volatile("ld.shared.v4.u32 {%0,%1,%2,%3}, [%4];\n" : "=r"(ys[0]), "=r"(ys[1]), "=r"(ys[2]), "=r"(ys[3]) : "r"(hi0 + other + p * PASS_BYTES));
                 const uint32_t tok = pos[p] >= 0 ? (uint32_t)pos[p] : 0u;      // rows past the list are zeros
 #pragma unroll
                 for (int e = 0; e < 4; ++e) {
@@ -157,10 +165,10 @@ residual_tc(const __nv_bfloat16* __restrict__ K, const __nv_bfloat16* __restrict
                     xl[e] = pack2_bf16(xo[0] - __uint_as_float(xs[e] << 16), xo[1] - __uint_as_float(xs[e] & 0xffff0000u));
                     yl[e] = pack2_bf16(yo[0] - __uint_as_float(ys[e] << 16), yo[1] - __uint_as_float(ys[e] & 0xffff0000u));
                 }
-                asm volatile("st.shared.v4.u32 [%0], {%1,%2,%3,%4};\n" ::"r"(hi0 + p * 4096), "r"(xs[0]), "r"(xs[1]), "r"(xs[2]), "r"(xs[3]) : "memory");
-                asm volatile("st.shared.v4.u32 [%0], {%1,%2,%3,%4};\n" ::"r"(hi0 + BOX_BYTES + p * 4096), "r"(ys[0]), "r"(ys[1]), "r"(ys[2]), "r"(ys[3]) : "memory");
-                asm volatile("st.shared.v4.u32 [%0], {%1,%2,%3,%4};\n" ::"r"(lo0 + p * 4096), "r"(xl[0]), "r"(xl[1]), "r"(xl[2]), "r"(xl[3]) : "memory");
-                asm volatile("st.shared.v4.u32 [%0], {%1,%2,%3,%4};\n" ::"r"(lo0 + BOX_BYTES + p * 4096), "r"(yl[0]), "r"(yl[1]), "r"(yl[2]), "r"(yl[3]) : "memory");
+                asm volatile("st.shared.v4.u32 [%0], {%1,%2,%3,%4};\n" ::"r"(hi0 + p * PASS_BYTES), "r"(xs[0]), "r"(xs[1]), "r"(xs[2]), "r"(xs[3]) : "memory");
+                asm volatile("st.shared.v4.u32 [%0], {%1,%2,%3,%4};\n" ::"r"(hi0 + other + p * PASS_BYTES), "r"(ys[0]), "r"(ys[1]), "r"(ys[2]), "r"(ys[3]) : "memory");
+                asm volatile("st.shared.v4.u32 [%0], {%1,%2,%3,%4};\n" ::"r"(lo0 + p * PASS_BYTES), "r"(xl[0]), "r"(xl[1]), "r"(xl[2]), "r"(xl[3]) : "memory");
+                asm volatile("st.shared.v4.u32 [%0], {%1,%2,%3,%4};\n" ::"r"(lo0 + other + p * PASS_BYTES), "r"(yl[0]), "r"(yl[1]), "r"(yl[2]), "r"(yl[3]) : "memory");
             }
             fence_async_proxy();
             tma::mbar_arrive(&sy.full[s]);
@@ -169,25 +177,25 @@ residual_tc(const __nv_bfloat16* __restrict__ K, const __nv_bfloat16* __restrict
         asm volatile("griddepcontrol.wait;\n" ::: "memory");      // idx is complete and visible from here on
         if (n_my > 0) fetch_idx(0, cur);
 #pragma unroll
-        for (int p = 0; p < 4; ++p) prev[p] = -1;
+        for (int p = 0; p < PASSES; ++p) prev[p] = -1;
         for (int i = 0; i < n_my && ok; ++i) {
             const int s = i % STAGES, round = i / STAGES;
             if (i + 1 < n_my) fetch_idx(i + 1, nxt);
             if (round > 0 && !tma::mbar_wait(&sy.empty[s], (round - 1) & 1, fault, 46)) { ok = false; break; }
             const int u = (int)((gt_lo + i) / P.tpu);
             const uint32_t kdst = tma::smem_u32(stage0 + s * R_STAGE_BYTES) + dst_thread;
-            const uint32_t vdst = kdst + RCfg<ROPE>::V_OFFSET;
-            const __nv_bfloat16* Ku = K + (size_t)u * P.N * 128 + qc * 8;
-            const __nv_bfloat16* Vu = V + (size_t)u * P.N * 128 + qc * 8;
+            const uint32_t vdst = kdst + C::V_OFFSET;
+            const __nv_bfloat16* Ku = K + (size_t)u * P.N * D + qc * 8;
+            const __nv_bfloat16* Vu = V + (size_t)u * P.N * D + qc * 8;
 #pragma unroll
-            for (int p = 0; p < 4; ++p) {
+            for (int p = 0; p < PASSES; ++p) {
                 const bool valid = cur[p] >= 0;
-                const size_t ro = valid ? (size_t)cur[p] * 128 : 0;
+                const size_t ro = valid ? (size_t)cur[p] * D : 0;
                 const uint32_t nb = valid ? 16u : 0u;                  // zero fill past the end of the list
-                cp_async16(kdst + p * 4096, Ku + ro, nb);
-                cp_async16(kdst + BOX_BYTES + p * 4096, Ku + ro + 64, nb);
-                cp_async16(vdst + p * 4096, Vu + ro, nb);
-                cp_async16(vdst + BOX_BYTES + p * 4096, Vu + ro + 64, nb);
+                cp_async16(kdst + p * PASS_BYTES, Ku + ro, nb);
+                cp_async16(kdst + other + p * PASS_BYTES, Ku + ro + D / 2, nb);
+                cp_async16(vdst + p * PASS_BYTES, Vu + ro, nb);
+                cp_async16(vdst + other + p * PASS_BYTES, Vu + ro + D / 2, nb);
             }
             cp_async_commit();
             if (ROPE) {
@@ -195,21 +203,24 @@ residual_tc(const __nv_bfloat16* __restrict__ K, const __nv_bfloat16* __restrict
                     cp_async_wait<1>();
                     turn_back((i - 1) % STAGES, prev);
                 }
-            } else if (i >= 2) {                         // ... of the tile before the previous one
-                cp_async_wait<2>();
+            } else if (i >= STAGES - 1) {                // ... of the tile STAGES - 1 before this one
+                cp_async_wait<STAGES - 1>();
                 fence_async_proxy();
-                tma::mbar_arrive(&sy.full[(i - 2) % STAGES]);
+                tma::mbar_arrive(&sy.full[(i - (STAGES - 1)) % STAGES]);
             }
 #pragma unroll
-            for (int p = 0; p < 4; ++p) { prev[p] = cur[p]; cur[p] = nxt[p]; }
+            for (int p = 0; p < PASSES; ++p) { prev[p] = cur[p]; cur[p] = nxt[p]; }
         }
         if (ROPE) {
             cp_async_wait<0>();
             if (ok && n_my > 0) turn_back((n_my - 1) % STAGES, prev);
         } else if (ok) {
-            if (n_my > 1) { cp_async_wait<1>(); fence_async_proxy(); tma::mbar_arrive(&sy.full[(n_my - 2) % STAGES]); }
-            cp_async_wait<0>();
-            if (n_my > 0) { fence_async_proxy(); tma::mbar_arrive(&sy.full[(n_my - 1) % STAGES]); }
+            auto publish = [&](int behind) {             // tile n_my - 1 - behind, if there is one
+                if (n_my > behind) { fence_async_proxy(); tma::mbar_arrive(&sy.full[(n_my - 1 - behind) % STAGES]); }
+            };
+            if constexpr (STAGES == 5) { cp_async_wait<3>(); publish(3); cp_async_wait<2>(); publish(2); }
+            cp_async_wait<1>(); publish(1);
+            cp_async_wait<0>(); publish(0);
         } else {
             cp_async_wait<0>();
         }
@@ -218,7 +229,7 @@ residual_tc(const __nv_bfloat16* __restrict__ K, const __nv_bfloat16* __restrict
         if (lane == 0) {
             tma::prefetch_map(&mapW);
             const uint32_t w_addr = tma::smem_u32(Ws);
-            const uint32_t idesc = tc::instr_desc(128, 128);
+            const uint32_t idesc = tc::instr_desc(128, D);
             int cur_u = -1;
             uint32_t n_units = 0;
             for (int i = 0; i < n_my; ++i) {
@@ -227,9 +238,9 @@ residual_tc(const __nv_bfloat16* __restrict__ K, const __nv_bfloat16* __restrict
                 const int u = (int)(gt / P.tpu);
                 if (u != cur_u) {
                     if (n_units > 0 && !tma::mbar_wait(&sy.w_empty, (n_units - 1) & 1, fault, 47)) break;
-                    tma::mbar_expect_tx(&sy.w_full, OPERAND_BYTES);
-                    tma::load_3d(Ws, &mapW, 0, 0, u % P.LH, &sy.w_full);
-                    tma::load_3d(Ws + BOX_BYTES, &mapW, 64, 0, u % P.LH, &sy.w_full);
+                    tma::mbar_expect_tx(&sy.w_full, C::W_BYTES);
+#pragma unroll
+                    for (int x = 0; x < D / 64; ++x) tma::load_3d(Ws + x * BOX_BYTES, &mapW, 64 * x, 0, u % P.LH, &sy.w_full);
                     if (!tma::mbar_wait(&sy.w_full, n_units & 1, fault, 48)) break;
                     cur_u = u;
                     ++n_units;
@@ -240,15 +251,15 @@ residual_tc(const __nv_bfloat16* __restrict__ K, const __nv_bfloat16* __restrict
                 if (!tma::mbar_wait(&sy.full[s], round & 1, fault, 49)) break;
                 tc::fence_after_sync();
                 const uint32_t hi_addr = tma::smem_u32(stage0 + s * R_STAGE_BYTES), lo_addr = hi_addr + OPERAND_BYTES;
-                const uint32_t d = sy.tmem_base + s * 128;
+                const uint32_t d = sy.tmem_base + s * D;
 #pragma unroll
-                for (int ks = 0; ks < 8; ++ks) {
+                for (int ks = 0; ks < D / 16; ++ks) {
                     const uint32_t o = (ks >> 2) * BOX_BYTES + (ks & 3) * 32;
                     tc::mma_bf16(d, tc::smem_desc(hi_addr + o), tc::smem_desc(w_addr + o), idesc, ks > 0);
                 }
                 if (ROPE) {
 #pragma unroll
-                    for (int ks = 0; ks < 8; ++ks) {
+                    for (int ks = 0; ks < D / 16; ++ks) {
                         const uint32_t o = (ks >> 2) * BOX_BYTES + (ks & 3) * 32;
                         tc::mma_bf16(d, tc::smem_desc(lo_addr + o), tc::smem_desc(w_addr + o), idesc, 1u);
                     }
@@ -273,13 +284,13 @@ residual_tc(const __nv_bfloat16* __restrict__ K, const __nv_bfloat16* __restrict
             tc::fence_after_sync();
             const long long gt = gt_lo + i;
             const int u = (int)(gt / P.tpu), t = (int)(gt - (long long)u * P.tpu);
-            const uint32_t v_addr = tma::smem_u32(stage0 + s * R_STAGE_BYTES) + RCfg<ROPE>::V_OFFSET + v_thread;
+            const uint32_t v_addr = tma::smem_u32(stage0 + s * R_STAGE_BYTES) + C::V_OFFSET + v_thread;
             uint32_t ra[32], rb[32];
-            const uint32_t taddr = lane_addr + s * 128;
+            const uint32_t taddr = lane_addr + s * D;
             tc::tmem_ld32(taddr, ra);
             float e0 = 0.f, e1 = 0.f, e2 = 0.f, e3 = 0.f;
 #pragma unroll
-            for (int ch = 0; ch < 4; ++ch) {
+            for (int ch = 0; ch < D / 32; ++ch) {
                 uint32_t (&cur)[32] = (ch & 1) ? rb : ra;
                 uint32_t (&nxt)[32] = (ch & 1) ? ra : rb;
                 uint32_t vv[16];                           // columns 32 ch .. 32 ch + 31 of the value row
@@ -291,7 +302,7 @@ residual_tc(const __nv_bfloat16* __restrict__ K, const __nv_bfloat16* __restrict
                                  : "r"(v_addr + (c16 >> 3) * BOX_BYTES + (((c16 & 7) ^ (r & 7)) << 4)));
                 }
                 tc::tmem_ld_wait(cur);
-                if (ch < 3) tc::tmem_ld32(taddr + (ch + 1) * 32, nxt);
+                if (ch + 1 < D / 32) tc::tmem_ld32(taddr + (ch + 1) * 32, nxt);
 #pragma unroll
                 for (int j = 0; j < 32; j += 4) {
                     const float a = __uint_as_float(cur[j]) - __uint_as_float(vv[j >> 1] << 16);

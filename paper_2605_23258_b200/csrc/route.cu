@@ -100,13 +100,13 @@ truncate_kernel(const float* __restrict__ eps, const int32_t* __restrict__ pool_
     truncate_general<NW>(e, n_pool, n_apx, emit, S, L, sel_dyn);
 }
 
-// Step 2 on CUDA cores.  grid (ceil(n_idx / 64), U), 256 threads; W^T staged in
+// Step 2 on CUDA cores (fp32).  grid (ceil(n_idx / 64), U), 256 threads; W^T staged in
 // dynamic shared memory as fp32 (D * (D+1) floats) plus one key row per warp.
 // With ROPE the regressor sees the key turned back by its position (the token index): channel c
 // pairs with c + D/2, angle -pos * theta^(-2c/D).
-template <typename T, int D, bool ROPE>
+template <int D, bool ROPE>
 __global__ void __launch_bounds__(256)
-residual_generic(const T* __restrict__ K, const T* __restrict__ V, const T* __restrict__ W, int64_t N,
+residual_generic(const float* __restrict__ K, const float* __restrict__ V, const float* __restrict__ W, int64_t N,
                  int LH, const int32_t* __restrict__ idx, int n_idx, float theta, float* __restrict__ eps) {
     extern __shared__ float smem[];
     __shared__ double inv_freq[D / 2];
@@ -114,10 +114,10 @@ residual_generic(const T* __restrict__ K, const T* __restrict__ V, const T* __re
     float* ks = smem + D * (D + 1);         // [8][D]
     if (ROPE) rope_fill_inv_freq(inv_freq, D, theta);
     const int u = blockIdx.y, lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    const T* Wu = W + (size_t)(u % LH) * D * D;
+    const float* Wu = W + (size_t)(u % LH) * D * D;
     for (int e = threadIdx.x; e < D * D; e += 256) {
         int co = e / D, ci = e % D;
-        Wt[ci * (D + 1) + co] = to_f32(Wu[e]);
+        Wt[ci * (D + 1) + co] = Wu[e];
     }
     __syncthreads();
     const int p_begin = blockIdx.x * 64;
@@ -129,11 +129,11 @@ residual_generic(const T* __restrict__ K, const T* __restrict__ V, const T* __re
             if (lane == 0) eps[(size_t)u * n_idx + p] = 0.f;
             continue;
         }
-        const T* kr = K + ((size_t)u * N + tok) * D;
-        const T* vr = V + ((size_t)u * N + tok) * D;
+        const float* kr = K + ((size_t)u * N + tok) * D;
+        const float* vr = V + ((size_t)u * N + tok) * D;
         __syncwarp();
 #pragma unroll
-        for (int c = lane; c < D; c += 32) kw[c] = to_f32(kr[c]);
+        for (int c = lane; c < D; c += 32) kw[c] = kr[c];
         __syncwarp();
         if (ROPE) {
 #pragma unroll
@@ -153,7 +153,7 @@ residual_generic(const T* __restrict__ K, const T* __restrict__ V, const T* __re
             float pred = 0.f;
 #pragma unroll 8
             for (int ci = 0; ci < D; ++ci) pred = fmaf(Wt[ci * (D + 1) + co], kw[ci], pred);
-            float r = to_f32(vr[co]) - pred;
+            float r = vr[co] - pred;
             e = fmaf(r, r, e);
         }
         e = warp_sum(e);
@@ -161,36 +161,37 @@ residual_generic(const T* __restrict__ K, const T* __restrict__ V, const T* __re
     }
 }
 
-template <typename T, int D>
+template <int D>
 static vector_status launch_residual(const Dims& dm, const void* K, const void* V, const void* W, int64_t N,
                                      const int32_t* idx, int64_t n_idx, float* eps, cudaStream_t st) {
     if (n_idx == 0) return VECTOR_OK;
     size_t smem = (size_t)(D * (D + 1) + 8 * D) * sizeof(float);
-    auto kern = dm.rope ? residual_generic<T, D, true> : residual_generic<T, D, false>;
+    auto kern = dm.rope ? residual_generic<D, true> : residual_generic<D, false>;
     VEC_CUDA_CHECK(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     dim3 grid((unsigned)((n_idx + 63) / 64), dm.U);
-    kern<<<grid, 256, smem, st>>>((const T*)K, (const T*)V, (const T*)W, N, dm.LH, idx, (int)n_idx, dm.theta, eps);
+    kern<<<grid, 256, smem, st>>>((const float*)K, (const float*)V, (const float*)W, N, dm.LH, idx, (int)n_idx, dm.theta, eps);
     VEC_LAUNCH_CHECK();
     return VECTOR_OK;
 }
 
-// bf16, head_dim 128: gather + tcgen05 residual kernel.
+// bf16: gather + tcgen05 residual kernel.
+template <int D>
 static vector_status launch_residual_tc(const Dims& dm, const void* K, const void* V, const void* W, int64_t N,
                                         const int32_t* idx, int64_t n_idx, float* eps, cudaStream_t st, bool dependent) {
     if (n_idx == 0) return VECTOR_OK;
+    using Plain = rtc::RCfg<D, false>;
+    using Rope = rtc::RCfg<D, true>;
     static PerDeviceOnce once;
     if (once.first()) {
-        cudaError_t e = cudaFuncSetAttribute(rtc::residual_tc<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             rtc::RCfg<false>::SMEM_BYTES);
+        cudaError_t e = cudaFuncSetAttribute(rtc::residual_tc<D, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, Plain::SMEM_BYTES);
         if (e == cudaSuccess)
-            e = cudaFuncSetAttribute(rtc::residual_tc<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                     rtc::RCfg<true>::SMEM_BYTES);
+            e = cudaFuncSetAttribute(rtc::residual_tc<D, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, Rope::SMEM_BYTES);
         if (e != cudaSuccess) { once.undo(); VEC_CUDA_CHECK(e); }
     }
     int* fault = kernel_fault_address();
     if (!fault) return VECTOR_ERR_CUDA;
     CUtensorMap mapW;
-    if (!tma::encode_bf16_3d(&mapW, W, 128, 128, (uint64_t)dm.LH, 256, 128 * 256, 64, 128)) return VECTOR_ERR_CUDA;
+    if (!tma::encode_bf16_3d(&mapW, W, D, D, (uint64_t)dm.LH, 2 * D, D * 2 * D, 64, D)) return VECTOR_ERR_CUDA;
     rtc::Params P;
     P.U = dm.U; P.LH = dm.LH; P.n_idx = (int)n_idx; P.N = N;
     P.tpu = (int)((n_idx + rtc::TILE - 1) / rtc::TILE);
@@ -198,28 +199,27 @@ static vector_status launch_residual_tc(const Dims& dm, const void* K, const voi
     const int sms = sm_count();
     const int blocks = (int)(P.n_tiles < sms ? P.n_tiles : sms);
     RopePhases ph = {};
-    if (dm.rope) rope_phases(dm.theta, 128, &ph);
+    if (dm.rope) rope_phases(dm.theta, D, &ph);
     // dependent: blocks may take SMs while the kernel that writes idx drains; the loaders wait for it
     const __nv_bfloat16* Kp = (const __nv_bfloat16*)K;
     const __nv_bfloat16* Vp = (const __nv_bfloat16*)V;
     if (dm.rope)
-        VEC_CUDA_CHECK(launch_maybe_dependent(dependent, rtc::residual_tc<true>, dim3(blocks), dim3(rtc::R_THREADS),
-                                              rtc::RCfg<true>::SMEM_BYTES, st, Kp, Vp, mapW, idx, P, ph, eps, fault));
+        VEC_CUDA_CHECK(launch_maybe_dependent(dependent, rtc::residual_tc<D, true>, dim3(blocks), dim3(Rope::THREADS),
+                                              Rope::SMEM_BYTES, st, Kp, Vp, mapW, idx, P, ph, eps, fault));
     else
-        VEC_CUDA_CHECK(launch_maybe_dependent(dependent, rtc::residual_tc<false>, dim3(blocks), dim3(rtc::R_THREADS),
-                                              rtc::RCfg<false>::SMEM_BYTES, st, Kp, Vp, mapW, idx, P, ph, eps, fault));
+        VEC_CUDA_CHECK(launch_maybe_dependent(dependent, rtc::residual_tc<D, false>, dim3(blocks), dim3(Plain::THREADS),
+                                              Plain::SMEM_BYTES, st, Kp, Vp, mapW, idx, P, ph, eps, fault));
     return VECTOR_OK;
 }
 
 static vector_status residual_dispatch(const Dims& dm, const void* K, const void* V, const void* W, int64_t N,
                                        const int32_t* idx, int64_t n_idx, float* eps, cudaStream_t st,
                                        bool dependent = false) {
-    if (dm.dtype == VECTOR_BF16 && dm.d == 128) return launch_residual_tc(dm, K, V, W, N, idx, n_idx, eps, st, dependent);
-    if (dm.dtype == VECTOR_F32)
-        return dm.d == 64 ? launch_residual<float, 64>(dm, K, V, W, N, idx, n_idx, eps, st)
-                          : launch_residual<float, 128>(dm, K, V, W, N, idx, n_idx, eps, st);
-    return dm.d == 64 ? launch_residual<__nv_bfloat16, 64>(dm, K, V, W, N, idx, n_idx, eps, st)
-                      : launch_residual<__nv_bfloat16, 128>(dm, K, V, W, N, idx, n_idx, eps, st);
+    if (dm.dtype == VECTOR_BF16)
+        return dm.d == 64 ? launch_residual_tc<64>(dm, K, V, W, N, idx, n_idx, eps, st, dependent)
+                          : launch_residual_tc<128>(dm, K, V, W, N, idx, n_idx, eps, st, dependent);
+    return dm.d == 64 ? launch_residual<64>(dm, K, V, W, N, idx, n_idx, eps, st)
+                      : launch_residual<128>(dm, K, V, W, N, idx, n_idx, eps, st);
 }
 
 // One-time opt-in to the dynamic shared memory of the selection kernels.
