@@ -91,6 +91,7 @@ __device__ __forceinline__ void producer_role(const CUtensorMap* mapQ, const CUt
     uint32_t kcount = 0, icount = 0;
     for (int it = blockIdx.x; it < P.n_items; it += gridDim.x, ++icount) {
         const Item im = decode_item(it, P);
+        if (icount == 1) asm volatile("griddepcontrol.wait;\n" ::: "memory");
         if (icount > 0 && !tma::mbar_wait(&sy.q_empty, (icount - 1) & 1, fault, 11)) return;
         tma::mbar_expect_tx(&sy.q_full, Cfg<D>::Q_BYTES);
 #pragma unroll
@@ -101,6 +102,7 @@ __device__ __forceinline__ void producer_role(const CUtensorMap* mapQ, const CUt
                              &sy.q_full);
         for (int t = im.t0; t < im.t1; ++t, ++kcount) {
             const uint32_t s = kcount % STAGES, round = kcount / STAGES;
+            if (kcount == STAGES) asm volatile("griddepcontrol.wait;\n" ::: "memory");     // as in the MMA role
             if (round > 0 && !tma::mbar_wait(&sy.k_empty[s], (round - 1) & 1, fault, 12)) return;
             tma::mbar_expect_tx(&sy.k_full[s], K_STAGE_BYTES);
 #pragma unroll
@@ -108,6 +110,9 @@ __device__ __forceinline__ void producer_role(const CUtensorMap* mapQ, const CUt
                 tma::load_3d(Ks + s * K_STAGE_BYTES + kh * BOX_BYTES, mapK, kh * 64, t * KT, im.u, &sy.k_full[s]);
         }
     }
+    // The next kernel's blocks may be scheduled from here on, when the last copies are under way: earlier they would
+    // sit beside this block for its whole run.
+    asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory");
 }
 
 template <int PASS, int D>
@@ -116,6 +121,8 @@ __device__ __forceinline__ void mma_role(const Params& P, Sync& sy, unsigned cha
     const uint32_t q_addr = tma::smem_u32(Qs), k_addr = tma::smem_u32(Ks);
     const uint32_t tmem = sy.tmem_base;
     uint32_t kcount = 0, icount = 0;
+    // the softmax warps of the second pass start once the first has drained: do not spend bounded polls on its run time
+    asm volatile("griddepcontrol.wait;\n" ::: "memory");
     for (int it = blockIdx.x; it < P.n_items; it += gridDim.x, ++icount) {
         const Item im = decode_item(it, P);
         if (!tma::mbar_wait(&sy.q_full, icount & 1, fault, 21)) return;
@@ -417,31 +424,59 @@ score_pass1_tc(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__
     block_teardown(sy);
 }
 
-// lse2[u][row] = log2 sum over all visible keys of exp2(logit2), from the chunk partials.  grid (U).
-__global__ void score_lse2_combine(const float2* __restrict__ partial, int R, int n_chunks, float* __restrict__ lse2) {
-    const int u = blockIdx.x;
-    for (int row = threadIdx.x; row < R; row += blockDim.x) {
-        float M = -INFINITY;
-        for (int c = 0; c < n_chunks; ++c) M = fmaxf(M, partial[((size_t)u * n_chunks + c) * R + row].x);
-        float L = 0.f;
-        for (int c = 0; c < n_chunks; ++c) {
-            const float2 p = partial[((size_t)u * n_chunks + c) * R + row];
-            if (p.x > -INFINITY) L += p.y * exp2f(p.x - M);
+// ---- pass 2 -----------------------------------------------------------------
+// log2 of a row's sum of exp2(logit2) from its 2 n_chunks (reference, sum) partials, `stride` apart: the even lane of a
+// pair takes the even tiles' partials, the odd lane the odd tiles', eight loads in flight each.
+__device__ __forceinline__ float row_lse2(const float2* __restrict__ p, int stride, int n_chunks) {
+    const size_t step = 2 * (size_t)stride;
+    p += (size_t)(threadIdx.x & 1) * stride;
+    float M = -INFINITY, L = 0.f;
+    for (int c0 = 0; c0 < n_chunks; c0 += 8) {
+        float2 v[8];
+        float m = M;
+#pragma unroll
+        for (int k = 0; k < 8; ++k) {
+            v[k] = c0 + k < n_chunks ? p[(size_t)(c0 + k) * step] : make_float2(-INFINITY, 0.f);
+            m = fmaxf(m, v[k].x);
         }
-        lse2[(size_t)u * R + row] = M + log2f(L);
+        if (m == -INFINITY) continue;                    // no visible key so far
+        L *= exp2f(M - m);
+#pragma unroll
+        for (int k = 0; k < 8; ++k) L += v[k].y * exp2f(v[k].x - m);
+        M = m;
     }
+    const unsigned pair = 3u << (threadIdx.x & 30);
+    const float M2 = __shfl_xor_sync(pair, M, 1), L2 = __shfl_xor_sync(pair, L, 1);
+    const float m = fmaxf(M, M2);                        // finite: every row sees at least one key
+    return m + log2f(L * exp2f(M - m) + L2 * exp2f(M2 - m));
 }
 
-// ---- pass 2 -----------------------------------------------------------------
+// lse2[u][row] = log2 sum over all visible keys of exp2(logit2).  grid (ceil(R / 128), U), 256 threads.
+__global__ void __launch_bounds__(256)
+score_lse2_rows(const float2* __restrict__ partial, int R, int n_chunks, float* __restrict__ lse2) {
+    asm volatile("griddepcontrol.wait;\n" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory");
+    const int u = blockIdx.y, row = blockIdx.x * 128 + (threadIdx.x >> 1);
+    if (row >= R) return;
+    const float l = row_lse2(partial + (size_t)u * 2 * n_chunks * R + row, R, n_chunks);
+    if ((threadIdx.x & 1) == 0) lse2[(size_t)u * R + row] = l;
+}
+
 // raw_part[(u * 2 RG + 2 rg + h) * N + key] = sum over rows [rg*256 + h*128, +128) of the softmax
 // probability of `key`; the parts are added up by the pooling kernel.  grid: one block per SM.
-template <int D>
+// INLINE_LSE, for blocks with few items: the rows' normalisers are formed from the chunk partials at the start of each
+// item, two threads a row, which saves a launch (one layer, 8 heads, 256 rows, 8192 keys: 26.5 us against 36.0 with a
+// kernel of its own, one block a unit).  With many items the stall at each item's start adds up, and score_lse2_rows
+// leaves them in lse2 beforehand.
+template <int D, bool INLINE_LSE>
 __global__ void __launch_bounds__(THREADS, 1)
 score_pass2_tc(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__ CUtensorMap mapK, const Params P,
-               const float* __restrict__ lse2, float* __restrict__ raw_part, int* __restrict__ fault) {
+               const float2* __restrict__ partial, const float* __restrict__ lse2, float* __restrict__ raw_part,
+               int* __restrict__ fault) {
     extern __shared__ unsigned char smem_raw[];
     __shared__ Sync sy;
-    __shared__ __align__(16) float neg_lse[SOFTMAX_WARPS][128];
+    // -lse2 of the item's rows: INLINE_LSE, 256 rows, two items in turn; else a copy of its 128 rows for every warp
+    __shared__ __align__(16) float neg_lse[INLINE_LSE ? 4 : SOFTMAX_WARPS][128];
     unsigned char* smem = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
     unsigned char* Qs = smem;
     unsigned char* Ks = smem + Cfg<D>::Q_BYTES;
@@ -457,20 +492,33 @@ score_pass2_tc(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__
         const uint32_t lane_addr = sy.tmem_base + ((uint32_t)(quarter * 32) << 16);
         const int key_in_tile = quarter * 32 + lane;
         const long long vis0 = P.N - P.w;
-        float* nl_w = neg_lse[warp];                   // this warp's copy of -lse2 of its 128 rows
-        uint32_t tcount = 0;
-        bool ok = true;
-        for (int it = blockIdx.x; it < P.n_items && ok; it += gridDim.x) {
+        uint32_t tcount = 0, icount = 0;
+        bool ok = true;                                // false once a wait gave up: touch nothing more (INLINE_LSE: but meet the barriers)
+        asm volatile("griddepcontrol.wait;\n" ::: "memory");      // the partials are complete and visible from here on
+        for (int it = blockIdx.x; it < P.n_items && (INLINE_LSE || ok); it += gridDim.x, ++icount) {
             const Item im = decode_item(it, P);
             const bool wg_active = im.rg * RG_ROWS + wg * 128 < P.R;
             const int row_base = im.rg * RG_ROWS + wg * 128;
-            __syncwarp();
+            float* nl_w;
+            if constexpr (INLINE_LSE) {
+                float* nl_item = neg_lse[2 * (icount & 1)];
+                const int r = threadIdx.x >> 1, row = im.rg * RG_ROWS + r;
+                const float lse = row < P.R ? row_lse2(partial + (size_t)im.u * 2 * P.n_chunks * P.R + row, P.R, P.n_chunks) : INFINITY;
+                if ((threadIdx.x & 1) == 0) nl_item[r] = -lse;           // -inf: padding rows add 0
+                // one barrier an item: whoever writes this half again, two items on, has seen every warp past this item
+                asm volatile("bar.sync 1, %0;\n" ::"n"(32 * SOFTMAX_WARPS) : "memory");
+                if (!ok) continue;
+                nl_w = nl_item + wg * 128;
+            } else {
+                nl_w = neg_lse[warp];
+                __syncwarp();
 #pragma unroll
-            for (int k = 0; k < 4; ++k) {
-                const int row = row_base + k * 32 + lane;
-                nl_w[k * 32 + lane] = row < P.R ? -lse2[(size_t)im.u * P.R + row] : -INFINITY;   // -inf: padding rows add 0
+                for (int k = 0; k < 4; ++k) {
+                    const int row = row_base + k * 32 + lane;
+                    nl_w[k * 32 + lane] = row < P.R ? -lse2[(size_t)im.u * P.R + row] : -INFINITY;   // -inf: padding rows add 0
+                }
+                __syncwarp();
             }
-            __syncwarp();
             float* out = raw_part + ((size_t)im.u * 2 * P.RG + 2 * im.rg + wg) * P.N;
             for (int t = im.t0; t < im.t1; ++t, ++tcount) {
                 if ((int)(tcount & 1) != grp) continue;
@@ -503,6 +551,7 @@ __global__ void __launch_bounds__(256)
 score_pool_parts(const float* __restrict__ raw_part, int parts, long long N, int w, int r, float* __restrict__ raw_out,
                  float* __restrict__ score) {
     __shared__ float rs[POOL_TILE + 16];
+    asm volatile("griddepcontrol.wait;\n" ::: "memory");        // the second pass's sums
     const int u = blockIdx.y;
     const long long i0 = (long long)blockIdx.x * POOL_TILE;
     const float* base = raw_part + (size_t)u * parts * N;
@@ -536,6 +585,7 @@ __global__ void __launch_bounds__(256)
 score_pool_parts_v4(const float* __restrict__ raw_part, int parts, long long N, int w, int r, float* __restrict__ raw_out,
                     float* __restrict__ score) {
     __shared__ __align__(16) float rs[POOL_TILE + 16];          // keys i0 - 8 .. i0 + POOL_TILE + 8
+    asm volatile("griddepcontrol.wait;\n" ::: "memory");        // the second pass's sums
     const int u = blockIdx.y;
     const long long i0 = (long long)blockIdx.x * POOL_TILE;
     const float* base = raw_part + (size_t)u * parts * N;
