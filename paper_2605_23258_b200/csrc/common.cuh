@@ -70,22 +70,29 @@ __device__ __forceinline__ void rope_fill_inv_freq(double* inv_freq, int d, floa
 // Kernel launch that may carry the programmatic-dependent attribute: with `dependent` the kernel may
 // be scheduled while the kernel before it in the stream drains (once every block of that one has
 // executed griddepcontrol.launch_dependents, or exited); it must execute griddepcontrol.wait before
-// it touches that kernel's output.
+// it touches anything that kernel, or one before it, reads or writes.  cluster > 1: thread block clusters of that size.
 template <typename... KArgs, typename... Args>
-inline cudaError_t launch_maybe_dependent(bool dependent, void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem,
+inline cudaError_t launch_maybe_dependent(bool dependent, int cluster, void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem,
                                           cudaStream_t st, Args... args) {
-    cudaLaunchAttribute attr;
-    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr.val.programmaticStreamSerializationAllowed = dependent ? 1 : 0;
+    cudaLaunchAttribute attr[2];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = dependent ? 1 : 0;
+    attr[1].id = cudaLaunchAttributeClusterDimension;
+    attr[1].val.clusterDim.x = cluster; attr[1].val.clusterDim.y = 1; attr[1].val.clusterDim.z = 1;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = grid;
     cfg.blockDim = block;
     cfg.dynamicSmemBytes = smem;
     cfg.stream = st;
-    cfg.attrs = &attr;
-    cfg.numAttrs = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = cluster > 1 ? 2 : 1;
     count_launch();
     return cudaLaunchKernelEx(&cfg, kernel, static_cast<KArgs>(args)...);
+}
+template <typename... KArgs, typename... Args>
+inline cudaError_t launch_maybe_dependent(bool dependent, void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem,
+                                          cudaStream_t st, Args... args) {
+    return launch_maybe_dependent(dependent, 1, kernel, grid, block, smem, st, args...);
 }
 
 }  // namespace vec

@@ -205,6 +205,46 @@ int* kernel_fault_address() {
     return addr[dev];
 }
 
+// Blocks per unit of the one-launch (cluster) form, 0 = stream and merge.  A cluster lies within one GPC and every
+// block fills its multiprocessor, so the largest size is taken at which all U clusters are resident at once.  That may
+// use fewer multiprocessors than the streaming form (48 units would need clusters of three that fit), whose second
+// kernel and records in global memory cost as much as about six tiles of a block (three with RoPE at 128 channels, whose
+// tiles take longest): the form with the fewer tiles a block, that cost included, runs.  Measured, four query heads, us
+// per step in a graph, stream against cluster: 128 channels, 8 units of 2457 rows 12.6 / 8.9, of 20000 rows 25.6 / 21.9;
+// 48 units of 1200 rows 15.8 / 13.2, of 2457 rows 18.7 / 18.1, with RoPE 26.4 / 31.2 for the last; 64 channels with
+// RoPE, 16 units of 5000 rows 19.4 / 13.2.
+template <int D, bool ROPE>
+static int decode_cluster_size(const dbf::Plan& pl, int U) {
+    using C = dbf::Cfg<D, ROPE>;
+    constexpr int MAXC = dbf::MAX_CLUSTER, EXTRA_TILES = ROPE && D == 128 ? 3 : 6;
+    static int resident[PerDeviceOnce::kMax][MAXC + 1] = {};      // clusters of each size the device holds at once
+    static std::mutex mu;
+    int dev = -1;
+    if (2 * U > sm_count() || cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= PerDeviceOnce::kMax) return 0;
+    std::lock_guard<std::mutex> lock(mu);
+    int* r = resident[dev];
+    if (r[0] == 0) {
+        auto kern = dbf::decode_stream_bf16<D, ROPE, true>;
+        bool ok = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, C::CLUSTER_SMEM_BYTES) == cudaSuccess &&
+                  cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess;
+        for (int c = 2; ok && c <= MAXC; ++c) {
+            cudaLaunchAttribute attr;
+            attr.id = cudaLaunchAttributeClusterDimension;
+            attr.val.clusterDim.x = c; attr.val.clusterDim.y = 1; attr.val.clusterDim.z = 1;
+            cudaLaunchConfig_t cfg = {};
+            cfg.gridDim = dim3(c); cfg.blockDim = dim3(C::THREADS); cfg.dynamicSmemBytes = C::CLUSTER_SMEM_BYTES;
+            cfg.attrs = &attr; cfg.numAttrs = 1;
+            int n = 0;
+            if (cudaOccupancyMaxActiveClusters(&n, kern, &cfg) == cudaSuccess) r[c] = n;
+        }
+        (void)cudaGetLastError();                                  // a size the device refuses counts as none resident
+        r[0] = 1;
+    }
+    for (int c = pl.n_tiles < MAXC ? pl.n_tiles : MAXC; c >= 2; --c)
+        if (r[c] >= U) return (pl.n_tiles + c - 1) / c <= (int)((pl.T + pl.B - 1) / pl.B) + EXTRA_TILES ? c : 0;
+    return 0;
+}
+
 // bf16: persistent TMA + tensor-core streaming kernel and the record merge.
 template <int D>
 static vector_status launch_decode_bf16(const Dims& dm, const void* q, const vector_cache* ch, const void* W,
@@ -214,10 +254,10 @@ static vector_status launch_decode_bf16(const Dims& dm, const void* q, const vec
     using Rope = dbf::Cfg<D, true>;
     static PerDeviceOnce once;
     if (once.first()) {
-        cudaError_t e = cudaFuncSetAttribute(dbf::decode_stream_bf16<D, false>,
+        cudaError_t e = cudaFuncSetAttribute(dbf::decode_stream_bf16<D, false, false>,
                                              cudaFuncAttributeMaxDynamicSharedMemorySize, Plain::SMEM_BYTES);
         if (e == cudaSuccess)
-            e = cudaFuncSetAttribute(dbf::decode_stream_bf16<D, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+            e = cudaFuncSetAttribute(dbf::decode_stream_bf16<D, true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                      Rope::SMEM_BYTES);
         if (D == 128 && e == cudaSuccess)
             e = cudaFuncSetAttribute(dpt::decode_stream_pertile_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, dpt::SMEM_BYTES);
@@ -255,14 +295,20 @@ static vector_status launch_decode_bf16(const Dims& dm, const void* q, const vec
             return VECTOR_ERR_CUDA;
         dpt::decode_stream_pertile_tc<<<pl.B, dpt::THREADS, dpt::SMEM_BYTES, st>>>(
             (const T*)q, pm, pl, (int)ch->n_ret, (int)ch->n_apx, dm.g, dm.LH, c2, partial, fault);
-    } else if (dm.rope)
-        dbf::decode_stream_bf16<D, true><<<pl.B, Rope::THREADS, Rope::SMEM_BYTES, st>>>(
-            (const T*)q, maps, pl, (int)ch->n_ret, (int)ch->n_apx, dm.g, dm.LH, c2, partial, fault, ch->apx_pos,
-            (long long)ch->cap_apx, ph);
-    else
-        dbf::decode_stream_bf16<D, false><<<pl.B, Plain::THREADS, Plain::SMEM_BYTES, st>>>(
-            (const T*)q, maps, pl, (int)ch->n_ret, (int)ch->n_apx, dm.g, dm.LH, c2, partial, fault, nullptr, 0, ph);
-    VEC_LAUNCH_CHECK();
+        VEC_LAUNCH_CHECK();
+    } else {
+        const T* qp = (const T*)q;
+        const T* Wq = (const T*)W;
+        const int n_ret = (int)ch->n_ret, n_apx = (int)ch->n_apx, out_f32 = out_dtype == VECTOR_F32;
+        const int csize = dm.rope ? decode_cluster_size<D, true>(pl, dm.U) : decode_cluster_size<D, false>(pl, dm.U);
+        auto kern = dm.rope ? (csize ? dbf::decode_stream_bf16<D, true, true> : dbf::decode_stream_bf16<D, true, false>)
+                            : (csize ? dbf::decode_stream_bf16<D, false, true> : dbf::decode_stream_bf16<D, false, false>);
+        const int threads = dm.rope ? Rope::THREADS : Plain::THREADS;
+        const size_t smem = csize ? (dm.rope ? Rope::CLUSTER_SMEM_BYTES : Plain::CLUSTER_SMEM_BYTES) : (dm.rope ? Rope::SMEM_BYTES : Plain::SMEM_BYTES);
+        VEC_CUDA_CHECK(launch_maybe_dependent(true, csize ? csize : 1, kern, dim3(csize ? csize * dm.U : pl.B), dim3(threads), smem, st, qp, maps, pl,
+                                              n_ret, n_apx, dm.g, dm.LH, c2, partial, fault, ch->apx_pos, (long long)ch->cap_apx, ph, Wq, out, out_f32));
+        if (csize) return VECTOR_OK;
+    }
     // programmatic dependent launch: the merge blocks start while the streaming kernel drains
     const float* rec = partial;
     const int apply_w = mode == 1 ? 0 : 1;

@@ -28,9 +28,15 @@
 // partial record when it leaves the unit; a warp that met no tile of a unit the
 // block touches writes an empty record.  The merge kernel combines a unit's
 // records, applies W and normalises.
+//
+// Few units (CLUSTER): one launch does it all.  A thread block cluster owns a unit, each of its
+// blocks an equal share of the unit's tiles; the warps' records stay in shared memory, a block
+// combines its own, and after a cluster barrier block r merges the query heads r, r + C, ... out of
+// the other blocks' shared memory and applies W.  No records in global memory, no second kernel.
 #ifndef VECTOR_DECODE_BF16_CUH_
 #define VECTOR_DECODE_BF16_CUH_
 
+#include "cluster.cuh"
 #include "common.cuh"
 #include "internal.h"
 #include "tcgen05.cuh"
@@ -58,6 +64,8 @@ template <int D, bool ROPE> struct Cfg {
     static constexpr int THREADS = 32 * (CONSUMER_WARPS + 1 + (ROPE ? ROPE_HELPERS * CONSUMER_WARPS : 0));
     static constexpr int SMEM_BYTES = SLOTS * SLOT_BYTES + 1024;     // + alignment slack; barriers live in static smem
     static constexpr int REC = 4 + 2 * D;                            // m, l, value-scale, pad, acc_v[D], acc_k[D]
+    static constexpr int CLUSTER_SMEM_BYTES = SMEM_BYTES + CONSUMER_WARPS * 8 * REC * 4;      // + the warps' records
+    static_assert(CLUSTER_SMEM_BYTES + 1024 <= 227 * 1024, "shared memory of a block, barriers included");
     static_assert(SLOTS % CONSUMER_WARPS == 0, "a slot must always be consumed by the same warp");
     static_assert(!ROPE || (CONSUMER_WARPS + 1 == 4 && ROPE_HELPERS == 4), "register hand-over is per warpgroup: owners + producer, then helpers");
 };
@@ -207,14 +215,157 @@ struct Maps {
     CUtensorMap ret_k, ret_v, apx_k;     // rank 3: (D dims, pool rows, U units), box 64 x 64 x 1, 128B swizzle
 };
 
-// grid (plan.B), Cfg::THREADS threads, Cfg::SMEM_BYTES dynamic shared memory.
-// partial: [U][s_max][CONSUMER_WARPS][g][REC]; slot of (unit u, block b) = b - block_of_tile(first tile of u).
+// Rows 16 mt .. + 15 of W times the key sums of n heads: pw[head][row].  One warp, M = 16 output channels, N = the heads
+// (padded to 8), K = D: the A fragments are read straight from the map in global memory, 16 bytes a load -- thread
+// (row r, quarter t) of a warp holds columns 8 (t + 4 jj) .. + 7 of rows r and r + 8, and the k slots of MMA step
+// 2 jj + h stand for columns 8 (t + 4 jj) + 4 h .. + 3, which the B fragments follow; the key sum enters as bf16
+// hi + lo (sixteen mantissa bits), the map's elements are bf16 as stored.
+template <int D>
+__device__ __forceinline__ void map_rows(const __nv_bfloat16* __restrict__ W, int mt, int n, const __nv_bfloat16 (&akh)[8][D],
+                                         const __nv_bfloat16 (&akl)[8][D], float (&pw)[8][D], int lane) {
+    constexpr int PIECES = D / 8;                                    // 16-byte pieces of a row of W
+    const int row = lane >> 2, quarter = lane & 3;
+    const uint4* Wu = reinterpret_cast<const uint4*>(W);
+    uint4 A[D / 16];
+#pragma unroll
+    for (int jj = 0; jj < D / 32; ++jj) {
+        A[2 * jj + 0] = Wu[(16 * mt + row) * PIECES + quarter + 4 * jj];
+        A[2 * jj + 1] = Wu[(16 * mt + row + 8) * PIECES + quarter + 4 * jj];
+    }
+    float d[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+    for (int jj = 0; jj < D / 32; ++jj) {
+        const uint4 r0 = A[2 * jj], r1 = A[2 * jj + 1];
+        const int col = 8 * (quarter + 4 * jj);
+        const uint4 bh = *reinterpret_cast<const uint4*>(&akh[row][col]);      // B column = head `row`
+        const uint4 bl = *reinterpret_cast<const uint4*>(&akl[row][col]);
+        mma_16(d, r0.x, r1.x, r0.y, r1.y, bh.x, bh.y);
+        mma_16(d, r0.x, r1.x, r0.y, r1.y, bl.x, bl.y);
+        mma_16(d, r0.z, r1.z, r0.w, r1.w, bh.z, bh.w);
+        mma_16(d, r0.z, r1.z, r0.w, r1.w, bl.z, bl.w);
+    }
+    // d[0], d[1]: row `row`, heads 2 quarter and 2 quarter + 1; d[2], d[3]: row `row` + 8
+    if (2 * quarter < n) { pw[2 * quarter][16 * mt + row] = d[0]; pw[2 * quarter][16 * mt + row + 8] = d[2]; }
+    if (2 * quarter + 1 < n) { pw[2 * quarter + 1][16 * mt + row] = d[1]; pw[2 * quarter + 1][16 * mt + row + 8] = d[3]; }
+}
+
+// The last part of the CLUSTER form: combines the records of a unit, which its cluster's blocks hold in shared
+// memory, applies W and writes out.  Every warp of every block of the cluster calls it, converged; the warps come from
+// different roles, so the block-wide barrier is the numbered one below.  recs: this block's [CONSUMER_WARPS][g][REC];
+// room: for a MergeShared (the slots, which nobody reads any more).
+template <int NT> __device__ __forceinline__ void merge_sync() { asm volatile("bar.sync 1, %0;\n" ::"n"(NT) : "memory"); }
+
+constexpr int MAX_CLUSTER = 16;
+template <int D> struct MergeShared {
+    __align__(16) float comb[8 * (4 + 2 * D)];                        // this block's sums per head, read by the whole cluster
+    __align__(16) __nv_bfloat16 akh[8][D], akl[8][D];                 // key sums of the heads this block merges, hi and lo
+    float avs[8][D], pw[8][D];                                        // their value sums; W times the key sums
+    float fac[8][MAX_CLUSTER], Ls[8];                                 // factor of every block's sums; sum of the weights
+};
 template <int D, bool ROPE>
+__device__ __forceinline__ void cluster_merge(const float* recs, unsigned char* room, const __nv_bfloat16* __restrict__ Wu, int g,
+                                              void* __restrict__ out_u, bool out_f32) {
+    using C = Cfg<D, ROPE>;
+    constexpr int REC = C::REC, CW = C::CONSUMER_WARPS, NT = C::THREADS, V4 = 2 * D / 4;
+    MergeShared<D>& S = *reinterpret_cast<MergeShared<D>*>(room);
+    auto& comb = S.comb; auto& fac = S.fac; auto& Ls = S.Ls; auto& akh = S.akh; auto& akl = S.akl; auto& avs = S.avs; auto& pw = S.pw;
+    const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+    const int nblk = (int)cl::nctas(), rank = (int)cl::rank();
+    merge_sync<NT>();                                                 // the warps' records are written
+    for (int e = tid; e < g * V4; e += NT) {
+        const int a = e / V4, c4 = e - a * V4;
+        float m[CW], M = -INFINITY, L = 0.f;
+        float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+        for (int w = 0; w < CW; ++w) { m[w] = recs[(w * g + a) * REC]; M = fmaxf(M, m[w]); }
+#pragma unroll
+        for (int w = 0; w < CW; ++w) {
+            if (m[w] == -INFINITY) continue;                          // a warp without tiles: its sums are not written
+            const float* r = recs + (w * g + a) * REC;
+            float f = __expf(m[w] - M);
+            L = fmaf(f, r[1], L);
+            if (c4 < D / 4) f *= r[2];                                // the values were parked at another reference
+            const float4 x = *reinterpret_cast<const float4*>(r + 4 + 4 * c4);
+            acc.x = fmaf(f, x.x, acc.x); acc.y = fmaf(f, x.y, acc.y); acc.z = fmaf(f, x.z, acc.z); acc.w = fmaf(f, x.w, acc.w);
+        }
+        if (c4 == 0) { comb[a * REC] = M; comb[a * REC + 1] = L; }
+        *reinterpret_cast<float4*>(comb + a * REC + 4 + 4 * c4) = acc;
+    }
+    for (int e = tid; e < 8 * D; e += NT) { akh[e / D][e % D] = __float2bfloat16_rn(0.f); akl[e / D][e % D] = __float2bfloat16_rn(0.f); }
+    __syncwarp();
+    cl::arrive_release();
+    cl::wait_acquire();                                               // every block's sums are ready
+    const int mine = rank < g ? (g - rank + nblk - 1) / nblk : 0;     // heads rank, rank + nblk, ...
+    const uint32_t comb_addr = tma::smem_u32(comb);
+    for (int k = wid; k < mine; k += NT / 32) {                       // a warp a head: the blocks' headers
+        const int a = rank + k * nblk;
+        float m = -INFINITY, l = 0.f;
+        if (lane < nblk) {
+            const uint32_t at = cl::map_to(comb_addr + (uint32_t)(a * REC) * 4u, (uint32_t)lane);
+            m = cl::ld_f32(at);
+            l = cl::ld_f32(at + 4);
+        }
+        const float M = warp_max(m);
+        const float f = m > -INFINITY ? __expf(m - M) : 0.f;
+        const float L = warp_sum(f * l);
+        if (lane < nblk) fac[k][lane] = f;
+        if (lane == 0) Ls[k] = L;
+    }
+    merge_sync<NT>();
+    for (int e = tid; e < mine * V4; e += NT) {
+        const int k = e / V4, c4 = e - k * V4, a = rank + k * nblk;
+        float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
+        for (int j0 = 0; j0 < nblk; j0 += 8) {                        // eight remote loads in flight
+            float4 x[8];
+#pragma unroll
+            for (int j = 0; j < 8; ++j) x[j] = cl::ld_f32x4(cl::map_to(comb_addr + (uint32_t)(a * REC + 4 + 4 * c4) * 4u, (uint32_t)min(j0 + j, nblk - 1)));
+#pragma unroll
+            for (int j = 0; j < 8; ++j) {
+                const float f = j0 + j < nblk ? fac[k][j0 + j] : 0.f;
+                acc.x = fmaf(f, x[j].x, acc.x); acc.y = fmaf(f, x[j].y, acc.y); acc.z = fmaf(f, x[j].z, acc.z); acc.w = fmaf(f, x[j].w, acc.w);
+            }
+        }
+        const float v[4] = {acc.x, acc.y, acc.z, acc.w};
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            const int c = 4 * c4 + i;
+            if (c < D) avs[k][c] = v[i];
+            else {
+                const __nv_bfloat16 hi = __float2bfloat16_rn(v[i]);
+                akh[k][c - D] = hi;
+                akl[k][c - D] = __float2bfloat16_rn(v[i] - __bfloat162float(hi));
+            }
+        }
+    }
+    __syncwarp();
+    cl::arrive_release();                                             // this block reads no other block's memory from here on
+    merge_sync<NT>();
+    if (mine > 0) {
+        for (int mt = wid; mt < D / 16; mt += NT / 32) map_rows<D>(Wu, mt, mine, akh, akl, pw, lane);
+        merge_sync<NT>();
+        for (int e = tid; e < mine * D; e += NT) {
+            const int k = e / D, c = e - k * D;
+            const float o = (avs[k][c] + pw[k][c]) / Ls[k];
+            const size_t at = (size_t)(rank + k * nblk) * D + c;
+            if (out_f32) reinterpret_cast<float*>(out_u)[at] = o;
+            else reinterpret_cast<__nv_bfloat16*>(out_u)[at] = __float2bfloat16_rn(o);
+        }
+    }
+    __syncwarp();
+    cl::wait_acquire();                                               // nobody reads this block's memory any more
+}
+
+// grid (plan.B), or (U x cluster size) in clusters, Cfg::THREADS threads, Cfg::SMEM_BYTES (CLUSTER_SMEM_BYTES) of
+// dynamic shared memory.
+// partial: [U][s_max][CONSUMER_WARPS][g][REC]; slot of (unit u, block b) = b - block_of_tile(first tile of u).
+// CLUSTER writes out itself and does not use partial.
+template <int D, bool ROPE, bool CLUSTER>
 __global__ void __launch_bounds__(Cfg<D, ROPE>::THREADS, 1)
 decode_stream_bf16(const __nv_bfloat16* __restrict__ q, const __grid_constant__ Maps maps, Plan pl, int n_ret,
                         int n_apx, int g, int LH, float scale_log2e, float* __restrict__ partial,
                         int* __restrict__ fault, const int32_t* __restrict__ apx_pos, long long cap_apx,
-                        const __grid_constant__ RopePhases rope) {
+                        const __grid_constant__ RopePhases rope, const __nv_bfloat16* __restrict__ W, void* __restrict__ out,
+                        int out_f32) {
     constexpr int HALF_BYTES = Cfg<D, ROPE>::HALF_BYTES, SLOT_BYTES = Cfg<D, ROPE>::SLOT_BYTES, SLOTS = Cfg<D, ROPE>::SLOTS;
     constexpr int CONSUMER_WARPS = Cfg<D, ROPE>::CONSUMER_WARPS, REC = Cfg<D, ROPE>::REC, BOXES = D / 64;
     extern __shared__ unsigned char smem_raw[];
@@ -227,22 +378,42 @@ decode_stream_bf16(const __nv_bfloat16* __restrict__ q, const __grid_constant__ 
     unsigned char* smem = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
     const int b = blockIdx.x;
     const int tid = threadIdx.x, lane = tid & 31, wq = tid >> 5;
-    const long long gt_lo = tile_begin(b, pl), gt_hi = tile_begin(b + 1, pl);
-    if (gt_lo >= gt_hi) return;
+    long long gt_lo, gt_hi;                              // never empty: no more blocks than tiles in either form
+    if (CLUSTER) {
+        const int C = (int)cl::nctas(), r = (int)cl::rank(), u = b / C;
+        gt_lo = (long long)u * pl.n_tiles + (long long)r * pl.n_tiles / C;
+        gt_hi = (long long)u * pl.n_tiles + (long long)(r + 1) * pl.n_tiles / C;
+    } else {
+        gt_lo = tile_begin(b, pl);
+        gt_hi = tile_begin(b + 1, pl);
+    }
     const int n_my = (int)(gt_hi - gt_lo);
     const int u0 = (int)(gt_lo / pl.n_tiles), t0 = (int)(gt_lo - (long long)u0 * pl.n_tiles);
     const int u_last = (int)((gt_hi - 1) / pl.n_tiles);
+    float* const recs = reinterpret_cast<float*>(smem + SLOTS * SLOT_BYTES);      // CLUSTER: the warps' records
 
-    // The merge kernel is launched as a programmatic dependent of this one: its blocks may be
-    // scheduled (and fetch W) as soon as SMs free up; it reads the records only after its own
-    // griddepcontrol.wait, which returns once this whole grid has finished and flushed.
-    asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory");
     if (tid == 0) {
 #pragma unroll
         for (int s = 0; s < SLOTS; ++s) { tma::mbar_init(&full_bar[s], 1); tma::mbar_init(&empty_bar[s], 1); }
         tma::mbar_fence_init();
     }
+    // Launched as a programmatic dependent itself: everything above touches only this block's own state.  The merge
+    // kernel is one of this kernel: its blocks may be scheduled as soon as SMs free up -- what was before this kernel
+    // has finished then -- and read the records only after their own wait.
+    asm volatile("griddepcontrol.wait;\n" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory");
     __syncthreads();
+    const __nv_bfloat16* const Wu = W + (size_t)(u0 % LH) * D * D;
+    if (CLUSTER) {                                                    // the map's way into L2, for the blocks that will apply it
+        const char* Wb = reinterpret_cast<const char*>(Wu);
+        for (int e = tid; e < 2 * D * D / 128; e += Cfg<D, ROPE>::THREADS) asm volatile("prefetch.global.L2 [%0];\n" ::"l"(Wb + 128 * e));
+        __syncwarp();
+    }
+    auto merge_unit = [&]() {                                         // CLUSTER: each role's last act
+        if (CLUSTER)
+            cluster_merge<D, ROPE>(recs, smem, Wu, g,
+                                   reinterpret_cast<char*>(out) + (size_t)u0 * g * D * (out_f32 ? 4 : 2), out_f32 != 0);
+    };
 
     if (ROPE && wq > CONSUMER_WARPS) {
         // ------------------------------------------------------------------ helpers (RoPE only)
@@ -276,6 +447,7 @@ decode_stream_bf16(const __nv_bfloat16* __restrict__ q, const __grid_constant__ 
                 }
             }
         }
+        merge_unit();
         return;
     }
 
@@ -309,7 +481,10 @@ decode_stream_bf16(const __nv_bfloat16* __restrict__ q, const __grid_constant__ 
                 if (++t == pl.n_tiles) { t = 0; ++u; }
             }
         }
-        return;      // the consumers wait on every tile's full barrier, so no copy outlives the block
+        // the consumers wait on every tile's full barrier, so no copy outlives the block
+        __syncwarp();
+        merge_unit();
+        return;
     }
     // ---------------------------------------------------------------------- consumers
     const int gid = lane >> 2, tig = lane & 3;
@@ -326,6 +501,7 @@ decode_stream_bf16(const __nv_bfloat16* __restrict__ q, const __grid_constant__ 
     bool stashed = false;
 
     auto record_of = [&](int unit) -> float* {
+        if (CLUSTER) return recs + (wq * g + gid) * REC;
         int slot = b - block_of_tile((long long)unit * pl.n_tiles, pl);
         if (slot < 0 || slot >= pl.s_max) { atomicCAS(fault, 0, 5); slot = 0; }     // cannot happen; never write out of bounds
         return partial + ((((size_t)unit * pl.s_max + slot) * CONSUMER_WARPS + wq) * g + gid) * REC;
@@ -356,7 +532,7 @@ decode_stream_bf16(const __nv_bfloat16* __restrict__ q, const __grid_constant__ 
             float* rec = record_of(unit);
             if (tig == 0) *reinterpret_cast<float4*>(rec) = make_float4(m * 0.69314718055994531f, lt, stashed ? stash_scale : 1.f, 0.f);
             if (stashed) store_acc(rec + 4 + D);      // value part was written at the pool switch
-            else {
+            else if (!CLUSTER || m > -INFINITY) {     // (the cluster's merge looks no further than an empty record's header)
                 store_acc(rec + 4);
 #pragma unroll
                 for (int n = 0; n < D / 8; ++n) *reinterpret_cast<float2*>(rec + 4 + D + n * 8 + 2 * tig) = make_float2(0.f, 0.f);
@@ -519,44 +695,32 @@ decode_stream_bf16(const __nv_bfloat16* __restrict__ q, const __grid_constant__ 
         }
         flush(u);
     }
+    __syncwarp();
+    merge_unit();
 }
 
 // Merge: grid (U), D g threads -- thread (a, c) owns output dim c of head a.
 // Combines the records of a unit, applies the unit's map to the p-weighted key sum and normalises:
 //   o = (sum_j f_j s_j acc_v_j + W sum_j f_j acc_k_j) / sum_j f_j l_j,   f_j = exp(m_j - max m).
 // Every load of a phase is independent of the others, so a phase costs one memory latency.
-// The product W (sum f acc_k) runs on warp-level MMAs, M = D output channels (warp w takes rows 16 w ..),
-// N = the unit's g query heads (padded to 8), K = D: the A fragments are read straight from the map in
-// global memory, 16 bytes a load -- thread (row r, quarter t) of a warp holds columns 8 (t + 4 jj) .. + 7 of
-// rows r and r + 8, and the k slots of MMA step 2 jj + h stand for columns 8 (t + 4 jj) + 4 h .. + 3, which the
-// B fragments follow; the key sum enters as bf16 hi + lo (sixteen mantissa bits), the map's elements are bf16
-// as stored.
+// The product W (sum f acc_k) runs on warp-level MMAs (map_rows).
 template <typename TO, int D, int MAXT>
 __global__ void __launch_bounds__(MAXT, MAXT == 512 ? 3 : 1)
 decode_merge_bf16(const float* __restrict__ partial, const __nv_bfloat16* __restrict__ W, int LH, int g,
                        Plan pl, int apply_w, int cw, TO* __restrict__ out) {
-    constexpr int REC = 4 + 2 * D, PIECES = D / 8;                  // 16-byte pieces of a row of W
+    constexpr int REC = 4 + 2 * D;
     __shared__ __align__(16) __nv_bfloat16 akh[8][D], akl[8][D];          // key sums per head, hi and lo halves
     __shared__ float pw[8][D];                 // W times the key sum
     __shared__ float fv[8][48], fk[8][48];     // per head, per record: factor for the value part / the key part
     __shared__ float Ls[8];
     const int u = blockIdx.x, tid = threadIdx.x, a = tid / D, c = tid % D, lane = tid & 31;
-    const int wid = tid >> 5, nwarps = blockDim.x >> 5, row = lane >> 2, quarter = lane & 3;
-    // A fragments of 16 rows of W (the maps of a layer stay in L2: every sequence of the batch reads them)
-    const uint4* Wu = reinterpret_cast<const uint4*>(W + (size_t)(u % LH) * D * D);
-    uint4 A[D / 16];
-    auto load_rows = [&](int mt) {
-#pragma unroll
-        for (int jj = 0; jj < D / 32; ++jj) {
-            A[2 * jj + 0] = Wu[(16 * mt + row) * PIECES + quarter + 4 * jj];
-            A[2 * jj + 1] = Wu[(16 * mt + row + 8) * PIECES + quarter + 4 * jj];
-        }
-    };
+    const int wid = tid >> 5, nwarps = blockDim.x >> 5;
+    const __nv_bfloat16* Wu = W + (size_t)(u % LH) * D * D;       // the maps of a layer stay in L2: every sequence of the batch reads them
     for (int i = tid; i < (8 - g) * D; i += blockDim.x) {         // columns of B beyond the unit's heads
         akh[g + i / D][i % D] = __float2bfloat16_rn(0.f);
         akl[g + i / D][i % D] = __float2bfloat16_rn(0.f);
     }
-    // everything above reads only W, which the streaming kernel does not write; its records from here on
+    // the streaming kernel's records from here on
     asm volatile("griddepcontrol.wait;\n" ::: "memory");
     const int first = block_of_tile((long long)u * pl.n_tiles, pl);
     const int n_rec = (block_of_tile((long long)(u + 1) * pl.n_tiles - 1, pl) - first + 1) * cw;   // <= 48; cw records per block
@@ -627,24 +791,7 @@ decode_merge_bf16(const float* __restrict__ partial, const __nv_bfloat16* __rest
         akl[a][c] = __float2bfloat16_rn(ak - __bfloat162float(hi));
     }
     __syncthreads();
-    for (int mt = wid; mt < D / 16; mt += nwarps) {
-        load_rows(mt);
-        float d[4] = {0.f, 0.f, 0.f, 0.f};
-#pragma unroll
-        for (int jj = 0; jj < D / 32; ++jj) {
-            const uint4 r0 = A[2 * jj], r1 = A[2 * jj + 1];
-            const int col = 8 * (quarter + 4 * jj);
-            const uint4 bh = *reinterpret_cast<const uint4*>(&akh[row][col]);      // B column = head `row`
-            const uint4 bl = *reinterpret_cast<const uint4*>(&akl[row][col]);
-            mma_16(d, r0.x, r1.x, r0.y, r1.y, bh.x, bh.y);
-            mma_16(d, r0.x, r1.x, r0.y, r1.y, bl.x, bl.y);
-            mma_16(d, r0.z, r1.z, r0.w, r1.w, bh.z, bh.w);
-            mma_16(d, r0.z, r1.z, r0.w, r1.w, bl.z, bl.w);
-        }
-        // d[0], d[1]: row `row`, heads 2 quarter and 2 quarter + 1; d[2], d[3]: row `row` + 8
-        if (2 * quarter < g) { pw[2 * quarter][16 * mt + row] = d[0]; pw[2 * quarter][16 * mt + row + 8] = d[2]; }
-        if (2 * quarter + 1 < g) { pw[2 * quarter + 1][16 * mt + row] = d[1]; pw[2 * quarter + 1][16 * mt + row + 8] = d[3]; }
-    }
+    for (int mt = wid; mt < D / 16; mt += nwarps) map_rows<D>(Wu, mt, g, akh, akl, pw, lane);
     __syncthreads();
     store_out(out + ((size_t)u * g + a) * D + c, (av + pw[a][c]) / Ls[a]);
 }
