@@ -45,7 +45,8 @@ template <int D> struct Cfg {
     static constexpr int Q_BYTES = HALVES * 2 * BOX_BYTES;          // [k half][256 rows][128 B]
     static constexpr int K_STAGE_BYTES = HALVES * BOX_BYTES;        // [k half][128 keys][128 B]
     static constexpr int STAGES = 8 / HALVES;
-    static constexpr int SMEM_BYTES = Q_BYTES + STAGES * K_STAGE_BYTES + 1024;
+    static constexpr int NQ = D == 64 ? 2 : 1;                      // row groups held: the next item's is fetched ahead where it fits
+    static constexpr int SMEM_BYTES = NQ * Q_BYTES + STAGES * K_STAGE_BYTES + 1024;
 };
 constexpr int SOFTMAX_WARPS = 16;
 constexpr int THREADS = 32 * (SOFTMAX_WARPS + 2);
@@ -73,7 +74,7 @@ __device__ __forceinline__ Item decode_item(int it, const Params& P) {
 
 // Barriers and the TMEM base of one block.
 struct Sync {
-    uint64_t q_full, q_empty;
+    uint64_t q_full[2], q_empty[2];
     uint64_t k_full[8], k_empty[8];
     uint64_t acc_full[4], acc_empty[4];
     uint32_t tmem_base;
@@ -85,29 +86,38 @@ struct Sync {
 template <int D>
 __device__ __forceinline__ void producer_role(const CUtensorMap* mapQ, const CUtensorMap* mapK, const Params& P,
                                               Sync& sy, unsigned char* Qs, unsigned char* Ks, int* fault) {
-    constexpr int HALVES = Cfg<D>::HALVES, STAGES = Cfg<D>::STAGES, K_STAGE_BYTES = Cfg<D>::K_STAGE_BYTES;
+    constexpr int HALVES = Cfg<D>::HALVES, STAGES = Cfg<D>::STAGES, K_STAGE_BYTES = Cfg<D>::K_STAGE_BYTES, NQ = Cfg<D>::NQ;
     tma::prefetch_map(mapQ);
     tma::prefetch_map(mapK);
     uint32_t kcount = 0, icount = 0;
-    for (int it = blockIdx.x; it < P.n_items; it += gridDim.x, ++icount) {
-        const Item im = decode_item(it, P);
-        if (icount == 1) asm volatile("griddepcontrol.wait;\n" ::: "memory");
-        if (icount > 0 && !tma::mbar_wait(&sy.q_empty, (icount - 1) & 1, fault, 11)) return;
-        tma::mbar_expect_tx(&sy.q_full, Cfg<D>::Q_BYTES);
+    auto load_q = [&](const Item& im) -> bool {
+        const uint32_t b = icount % NQ, use = icount / NQ;
+        if (use > 0 && !tma::mbar_wait(&sy.q_empty[b], (use - 1) & 1, fault, 11)) return false;
+        tma::mbar_expect_tx(&sy.q_full[b], Cfg<D>::Q_BYTES);
 #pragma unroll
         for (int kh = 0; kh < HALVES; ++kh)
 #pragma unroll
             for (int rb = 0; rb < 2; ++rb)
-                tma::load_3d(Qs + kh * 2 * BOX_BYTES + rb * BOX_BYTES, mapQ, kh * 64, im.rg * RG_ROWS + rb * 128, im.u,
-                             &sy.q_full);
+                tma::load_3d(Qs + b * Cfg<D>::Q_BYTES + (kh * 2 + rb) * BOX_BYTES, mapQ, kh * 64, im.rg * RG_ROWS + rb * 128, im.u,
+                             &sy.q_full[b]);
+        return true;
+    };
+    for (int it = blockIdx.x; it < P.n_items; it += gridDim.x, ++icount) {
+        const Item im = decode_item(it, P);
+        if (icount == NQ) asm volatile("griddepcontrol.wait;\n" ::: "memory");      // as in the MMA role
+        // With one row group held, its successor has to wait for the item's last product: the next keys go first
+        // (they waited behind it: 4 to 5 thousand cycles an item, of 22 thousand at 15 tiles of 64 channels).
+        const int q_at = min(im.t0 + STAGES, im.t1) - 1;
+        if (NQ > 1 && !load_q(im)) return;
         for (int t = im.t0; t < im.t1; ++t, ++kcount) {
             const uint32_t s = kcount % STAGES, round = kcount / STAGES;
-            if (kcount == STAGES) asm volatile("griddepcontrol.wait;\n" ::: "memory");     // as in the MMA role
+            if (kcount == STAGES) asm volatile("griddepcontrol.wait;\n" ::: "memory");
             if (round > 0 && !tma::mbar_wait(&sy.k_empty[s], (round - 1) & 1, fault, 12)) return;
             tma::mbar_expect_tx(&sy.k_full[s], K_STAGE_BYTES);
 #pragma unroll
             for (int kh = 0; kh < HALVES; ++kh)
                 tma::load_3d(Ks + s * K_STAGE_BYTES + kh * BOX_BYTES, mapK, kh * 64, t * KT, im.u, &sy.k_full[s]);
+            if (NQ == 1 && t == q_at && !load_q(im)) return;
         }
     }
     // The next kernel's blocks may be scheduled from here on, when the last copies are under way: earlier they would
@@ -117,15 +127,16 @@ __device__ __forceinline__ void producer_role(const CUtensorMap* mapQ, const CUt
 
 template <int PASS, int D>
 __device__ __forceinline__ void mma_role(const Params& P, Sync& sy, unsigned char* Qs, unsigned char* Ks, int* fault) {
-    constexpr int STAGES = Cfg<D>::STAGES, K_STAGE_BYTES = Cfg<D>::K_STAGE_BYTES, K_STEPS = D / 16;
-    const uint32_t q_addr = tma::smem_u32(Qs), k_addr = tma::smem_u32(Ks);
+    constexpr int STAGES = Cfg<D>::STAGES, K_STAGE_BYTES = Cfg<D>::K_STAGE_BYTES, K_STEPS = D / 16, NQ = Cfg<D>::NQ;
+    const uint32_t k_addr = tma::smem_u32(Ks);
     const uint32_t tmem = sy.tmem_base;
     uint32_t kcount = 0, icount = 0;
     // the softmax warps of the second pass start once the first has drained: do not spend bounded polls on its run time
     asm volatile("griddepcontrol.wait;\n" ::: "memory");
     for (int it = blockIdx.x; it < P.n_items; it += gridDim.x, ++icount) {
         const Item im = decode_item(it, P);
-        if (!tma::mbar_wait(&sy.q_full, icount & 1, fault, 21)) return;
+        const uint32_t qb = icount % NQ, q_addr = tma::smem_u32(Qs) + qb * Cfg<D>::Q_BYTES;
+        if (!tma::mbar_wait(&sy.q_full[qb], (icount / NQ) & 1, fault, 21)) return;
         fence_after_sync();
         for (int t = im.t0; t < im.t1; ++t, ++kcount) {
             const uint32_t s = kcount % STAGES, round = kcount / STAGES;
@@ -160,14 +171,14 @@ __device__ __forceinline__ void mma_role(const Params& P, Sync& sy, unsigned cha
             }
             mma_commit(&sy.k_empty[s]);       // the stage is free once these MMAs have read it
         }
-        mma_commit(&sy.q_empty);
+        mma_commit(&sy.q_empty[qb]);
     }
 }
 
 __device__ __forceinline__ void block_setup(Sync& sy, int empty_count) {
     if (threadIdx.x == 0) {
-        tma::mbar_init(&sy.q_full, 1);
-        tma::mbar_init(&sy.q_empty, 1);
+#pragma unroll
+        for (int b = 0; b < 2; ++b) { tma::mbar_init(&sy.q_full[b], 1); tma::mbar_init(&sy.q_empty[b], 1); }
 #pragma unroll
         for (int s = 0; s < 8; ++s) { tma::mbar_init(&sy.k_full[s], 1); tma::mbar_init(&sy.k_empty[s], 1); }
 #pragma unroll
@@ -192,16 +203,17 @@ __device__ __forceinline__ void block_teardown(Sync& sy) {
     }
 }
 
-// sum_i exp2(v[i] * c + n[i]) over 32 accumulator columns; n is either one value for all columns
-// (pass 1: minus the row's reference) or a table in shared memory (pass 2: minus the rows' lse).
-// Written in three stages (all FMAs, all exponentials, a tree of adds) so that the 32 MUFU
+// sum_i exp2(v[i] * c + n[i]) over 32 (pass 1) or 16 (pass 2) accumulator columns; n is either one value for all
+// columns (pass 1: minus the row's reference) or a table in shared memory (pass 2: minus the rows' lse).
+// Written in three stages (all FMAs, all exponentials, a tree of adds) so that the MUFU
 // operations issue back to back and nothing waits on the result of the one just before it.
-__device__ __forceinline__ void sum_tree32(const float (&e)[32], uint64_t& acc) {
-    uint64_t p[16];
+template <int C>
+__device__ __forceinline__ void sum_tree(const float (&e)[C], uint64_t& acc) {
+    uint64_t p[C / 2];
 #pragma unroll
-    for (int i = 0; i < 16; ++i) p[i] = pack2(e[2 * i], e[2 * i + 1]);
+    for (int i = 0; i < C / 2; ++i) p[i] = pack2(e[2 * i], e[2 * i + 1]);
 #pragma unroll
-    for (int w = 8; w >= 1; w >>= 1)
+    for (int w = C / 4; w >= 1; w >>= 1)
 #pragma unroll
         for (int i = 0; i < w; ++i) p[i] = add2(p[i], p[i + w]);
     acc = add2(acc, p[0]);
@@ -210,17 +222,20 @@ __device__ __forceinline__ void sum_tree32(const float (&e)[32], uint64_t& acc) 
 // 16 exponentials are evaluated on the FMA pipe instead: 2^x = 2^n p(f) with n = round(x),
 // f = x - n in [-1/2, 1/2] and p the degree-4 minimax polynomial of 2^f (relative error 2.7e-6);
 // n is added to the exponent field.  x is clamped to [-126, 128]: results below 2^-126 do not
-// matter to a sum whose largest term is of order one, and at the upper end the exponent field must
+// matter to a sum whose largest term is of order one, and at the upper end (UPPER: the first pass, whose
+// reference lags; in the second no logit exceeds its row's normaliser by more than rounding) the exponent field must
 // not wrap -- 2^128 comes out as about 3.4e38 (or a NaN), which the overflow test of the first pass
 // (sum above 2^64, or not finite) catches, whereas a wrapped exponent would pass as a tiny term.
 #ifndef VECTOR_SCORE_POLY16
 #define VECTOR_SCORE_POLY16 4
 #endif
 constexpr int POLY16 = VECTOR_SCORE_POLY16;
+template <bool UPPER>
 __device__ __forceinline__ void exp2_poly_pair(float x0, float x1, float& e0, float& e1) {
     const float magic = 12582912.f;                    // 1.5 * 2^23: adding it leaves round(x) in the low mantissa bits
-    x0 = fminf(fmaxf(x0, -126.f), 128.f);
-    x1 = fminf(fmaxf(x1, -126.f), 128.f);
+    x0 = fmaxf(x0, -126.f);
+    x1 = fmaxf(x1, -126.f);
+    if (UPPER) { x0 = fminf(x0, 128.f); x1 = fminf(x1, 128.f); }
     const uint64_t x2 = pack2(x0, x1);
     const uint64_t t2 = add2(x2, pack2(magic, magic));
     const uint64_t n2 = add2(t2, pack2(-magic, -magic));
@@ -236,11 +251,12 @@ __device__ __forceinline__ void exp2_poly_pair(float x0, float x1, float& e0, fl
     e0 = __uint_as_float(__float_as_uint(p0) + (__float_as_uint(t0) << 23));
     e1 = __uint_as_float(__float_as_uint(p1) + (__float_as_uint(t1) << 23));
 }
-// e[i] = 2^x[i] for 32 exponents: the first POLY16 of every 16 by polynomial, the rest by MUFU.
-__device__ __forceinline__ void exp2_32(const float (&x)[32], float (&e)[32]) {
+// e[i] = 2^x[i] for C exponents: the first POLY16 of every 16 by polynomial, the rest by MUFU.
+template <bool UPPER, int C>
+__device__ __forceinline__ void exp2_all(const float (&x)[C], float (&e)[C]) {
 #pragma unroll
-    for (int i = 0; i < 32; i += 2) {
-        if ((i & 15) < POLY16) exp2_poly_pair(x[i], x[i + 1], e[i], e[i + 1]);
+    for (int i = 0; i < C; i += 2) {
+        if ((i & 15) < POLY16) exp2_poly_pair<UPPER>(x[i], x[i + 1], e[i], e[i + 1]);
         else { e[i] = ex2(x[i]); e[i + 1] = ex2(x[i + 1]); }
     }
 }
@@ -249,24 +265,23 @@ __device__ __forceinline__ float exp2_sum32(const uint32_t (&v)[32], float c, fl
     float x[32], e[32];
 #pragma unroll
     for (int i = 0; i < 32; i += 2) unpack2(fma2(pack2(v[i], v[i + 1]), c2, n2), x[i], x[i + 1]);
-    exp2_32(x, e);
+    exp2_all<true>(x, e);
     uint64_t acc = pack2(0.f, 0.f);
-    sum_tree32(e, acc);
+    sum_tree(e, acc);
     float s0, s1;
     unpack2(acc, s0, s1);
     return s0 + s1;
 }
-__device__ __forceinline__ void exp2_acc32(const uint32_t (&v)[32], float c, const float4* __restrict__ n, uint64_t& acc) {
+__device__ __forceinline__ void exp2_acc16(const uint32_t (&v)[16], float c, const float4 (&n)[4], uint64_t& acc) {
     const uint64_t c2 = pack2(c, c);
-    float x[32], e[32];
+    float x[16], e[16];
 #pragma unroll
-    for (int i = 0; i < 8; ++i) {
-        const float4 n4 = n[i];
-        unpack2(fma2(pack2(v[4 * i], v[4 * i + 1]), c2, pack2(n4.x, n4.y)), x[4 * i], x[4 * i + 1]);
-        unpack2(fma2(pack2(v[4 * i + 2], v[4 * i + 3]), c2, pack2(n4.z, n4.w)), x[4 * i + 2], x[4 * i + 3]);
+    for (int i = 0; i < 4; ++i) {
+        unpack2(fma2(pack2(v[4 * i], v[4 * i + 1]), c2, pack2(n[i].x, n[i].y)), x[4 * i], x[4 * i + 1]);
+        unpack2(fma2(pack2(v[4 * i + 2], v[4 * i + 3]), c2, pack2(n[i].z, n[i].w)), x[4 * i + 2], x[4 * i + 3]);
     }
-    exp2_32(x, e);
-    sum_tree32(e, acc);
+    exp2_all<false>(x, e);
+    sum_tree(e, acc);
 }
 __device__ __forceinline__ float max32(const uint32_t (&v)[32]) {
     float a = max3(__uint_as_float(v[0]), __uint_as_float(v[1]), __uint_as_float(v[2]));
@@ -335,32 +350,37 @@ __device__ __forceinline__ void softmax_tile_pass1(uint32_t taddr, float c, long
 // One accumulator tile of pass 2 for this thread's key: sum over 128 rows of exp2(logit2 - lse2[row]).
 // Masked tiles: row j of the window (j0 = window index of the tile's first row, advancing cyclically
 // with period w) sees this key only if key - (N - w) <= j.
+// 16 columns at a time: the rows' lse, 16 registers, are then on their way before the accumulator's load is waited for.
 template <bool MASKED>
 __device__ __forceinline__ float softmax_tile_pass2(uint32_t taddr, float c, const float* nl_w, long long key_rel,
                                                     int j0, int w, uint64_t& empty_bar, int lane) {
-    uint32_t ra[32], rb[32];
-    tmem_ld32(taddr, ra);
+    uint32_t ra[16], rb[16];
+    tmem_ld16(taddr, ra);
     uint64_t acc = pack2(0.f, 0.f);
     float sm = 0.f;
     int j = j0;
 #pragma unroll
-    for (int ch = 0; ch < 4; ++ch) {
-        uint32_t (&cur)[32] = (ch & 1) ? rb : ra;
-        uint32_t (&nxt)[32] = (ch & 1) ? ra : rb;
-        tmem_ld_wait(cur);
-        if (ch < 3) {
-            tmem_ld32(taddr + (ch + 1) * 32, nxt);
+    for (int ch = 0; ch < 8; ++ch) {
+        uint32_t (&cur)[16] = (ch & 1) ? rb : ra;
+        uint32_t (&nxt)[16] = (ch & 1) ? ra : rb;
+        float4 n[4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) n[i] = reinterpret_cast<const float4*>(nl_w + ch * 16)[i];
+        tmem_ld_wait16(cur);
+        if (ch < 7) {
+            tmem_ld16(taddr + (ch + 1) * 16, nxt);
         } else {
             fence_before_sync();
             __syncwarp();
             if (lane == 0) tma::mbar_arrive(&empty_bar);
         }
         if (!MASKED) {
-            exp2_acc32(cur, c, reinterpret_cast<const float4*>(nl_w + ch * 32), acc);
+            exp2_acc16(cur, c, n, acc);
         } else {
 #pragma unroll
-            for (int i = 0; i < 32; ++i) {
-                const float p = ex2(fmaf(__uint_as_float(cur[i]), c, nl_w[ch * 32 + i]));
+            for (int i = 0; i < 16; ++i) {
+                const float nl = (i & 3) == 0 ? n[i >> 2].x : (i & 3) == 1 ? n[i >> 2].y : (i & 3) == 2 ? n[i >> 2].z : n[i >> 2].w;
+                const float p = ex2(fmaf(__uint_as_float(cur[i]), c, nl));
                 if (key_rel <= j) sm += p;
                 if (++j == w) j = 0;
             }
@@ -382,7 +402,7 @@ score_pass1_tc(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__
     __shared__ Sync sy;
     unsigned char* smem = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
     unsigned char* Qs = smem;
-    unsigned char* Ks = smem + Cfg<D>::Q_BYTES;
+    unsigned char* Ks = smem + Cfg<D>::NQ * Cfg<D>::Q_BYTES;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     block_setup(sy, 4);
 
@@ -479,7 +499,7 @@ score_pass2_tc(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__
     __shared__ __align__(16) float neg_lse[INLINE_LSE ? 4 : SOFTMAX_WARPS][128];
     unsigned char* smem = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
     unsigned char* Qs = smem;
-    unsigned char* Ks = smem + Cfg<D>::Q_BYTES;
+    unsigned char* Ks = smem + Cfg<D>::NQ * Cfg<D>::Q_BYTES;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     block_setup(sy, 8);
 
