@@ -90,7 +90,8 @@ typedef struct {
  * and a key-only pool, rows in ascending original position.  All device memory,
  * caller-owned.  cap_* are row capacities per unit; n_* the rows in use (equal
  * for all units).  A decoded token is appended by writing its K/V row at
- * ret_*[u][n_ret] and bumping n_ret (<= cap_ret): no library call is needed.
+ * ret_*[u][n_ret] and bumping n_ret (<= cap_ret): vector_append writes the rows,
+ * or the caller does.
  */
 typedef struct {
     void*    ret_k;     /* [U][cap_ret][d]                                          */
@@ -230,6 +231,14 @@ VECTOR_API vector_status vector_compact(const vector_shape* shape, const vector_
                              const void* K, const void* V,
                              const int32_t* ret_idx, const int32_t* apx_idx,
                              const vector_cache* cache, void* stream);
+
+/*
+ * Appends a generated token in full: k_new, v_new (device [U][d] of shape->dtype) become row cache->n_ret of ret_k and
+ * ret_v, and pos its entry of ret_pos, for every unit.  The caller bumps n_ret afterwards.  VECTOR_ERR_SHAPE if the
+ * retained pool is full.
+ */
+VECTOR_API vector_status vector_append(const vector_shape* shape, const vector_cache* cache, const void* k_new,
+                                       const void* v_new, int32_t pos, void* stream);
 
 /*
  * Generation-time attention over the mixed cache (Step 3: values of approximated

@@ -10,7 +10,7 @@ from .binding import (  # noqa: F401
     load_library, library_path,
     vector_status_string, vector_plan_budget, vector_calibrate, vector_workspace_bytes,
     vector_score, vector_score_keydiff, vector_pool_select, vector_residual, vector_truncate, vector_route,
-    vector_compact, vector_diagnostics, DIAG_FIELDS, vector_decode_attn, alloc_cache, alloc_workspace,
+    vector_compact, vector_append, vector_diagnostics, DIAG_FIELDS, vector_decode_attn, alloc_cache, alloc_workspace,
     vector_layer_workspace_bytes, vector_layer_scores, vector_residual_layer, vector_route_layer, vector_compact_layer,
     vector_decode_attn_layer,
     vector_r2_global, vector_r2_global_workspace_bytes, R2_FIELDS, vector_sync_check,

@@ -11,6 +11,7 @@ from __future__ import annotations
 
 import ctypes
 import os
+import struct
 from dataclasses import dataclass
 
 import torch
@@ -50,6 +51,13 @@ class _Cache(ctypes.Structure):
                 ("n_ret", ctypes.c_int64), ("n_apx", ctypes.c_int64)]
 
 
+# The same structs as packed bytes, which the calls below pass by pointer (the library reads them during the call): a third
+# of the cost of filling a ctypes.Structure, and a decode step of one layer is short enough to see it.
+_pack_shape = struct.Struct("8ifif").pack
+_pack_budget = struct.Struct("7q").pack
+_pack_cache = struct.Struct("5P4q").pack
+
+
 @dataclass
 class Shape:
     batch: int
@@ -80,6 +88,10 @@ class Shape:
         return _Shape(self.batch, self.n_layers, self.n_q_heads, self.n_kv_heads, self.head_dim, self.dtype,
                       self.window, self.pool_kernel, self.sm_scale, self.rope_enabled, self.rope_theta)
 
+    def _p(self) -> bytes:
+        return _pack_shape(self.batch, self.n_layers, self.n_q_heads, self.n_kv_heads, self.head_dim, self.dtype,
+                           self.window, self.pool_kernel, self.sm_scale, self.rope_enabled, self.rope_theta)
+
 
 @dataclass
 class Budget:
@@ -95,6 +107,10 @@ class Budget:
         return _Budget(self.n_tokens, self.n_budget_pairs, self.n_a, self.n_pool, self.n_apx, self.n_ret,
                        self.n_evict)
 
+    def _p(self) -> bytes:
+        return _pack_budget(self.n_tokens, self.n_budget_pairs, self.n_a, self.n_pool, self.n_apx, self.n_ret,
+                            self.n_evict)
+
 
 @dataclass
 class Cache:
@@ -107,10 +123,10 @@ class Cache:
     n_ret: int
     n_apx: int
 
-    def _c(self) -> _Cache:
-        return _Cache(self.ret_k.data_ptr(), self.ret_v.data_ptr(), self.apx_k.data_ptr(),
-                      self.ret_pos.data_ptr(), self.apx_pos.data_ptr(),
-                      self.ret_k.shape[1], self.apx_k.shape[1], self.n_ret, self.n_apx)
+    def _p(self) -> bytes:
+        return _pack_cache(self.ret_k.data_ptr(), self.ret_v.data_ptr(), self.apx_k.data_ptr(),
+                           self.ret_pos.data_ptr(), self.apx_pos.data_ptr(),
+                           self.ret_k.shape[1], self.apx_k.shape[1], self.n_ret, self.n_apx)
 
 
 def library_path() -> str:
@@ -127,12 +143,12 @@ def load_library() -> ctypes.CDLL:
                           "(nvcc, sm_100a). There is no fallback path.")
     lib = ctypes.CDLL(_LIB_PATH)
     P, I32, I64, SZ = ctypes.c_void_p, ctypes.c_int32, ctypes.c_int64, ctypes.c_size_t
-    SP, BP, CP = ctypes.POINTER(_Shape), ctypes.POINTER(_Budget), ctypes.POINTER(_Cache)
+    SP = BP = CP = P              # structs: packed bytes, or ctypes.byref of a Structure
     lib.vector_status_string.restype = ctypes.c_char_p
     lib.vector_status_string.argtypes = [ctypes.c_int]
     lib.vector_last_cuda_error.restype = ctypes.c_int
     lib.vector_last_cuda_error.argtypes = []
-    lib.vector_plan_budget.argtypes = [I64, I64, I64, I32, BP]
+    lib.vector_plan_budget.argtypes = [I64, I64, I64, I32, ctypes.POINTER(_Budget)]
     lib.vector_calibrate.argtypes = [P, P, I64, I32, I32, I32, ctypes.c_double, P, P]
     lib.vector_workspace_bytes.restype = SZ
     lib.vector_workspace_bytes.argtypes = [SP, BP]
@@ -144,6 +160,8 @@ def load_library() -> ctypes.CDLL:
     lib.vector_truncate.argtypes = [SP, BP, P, P, P, P, P, P, SZ, P]
     lib.vector_route.argtypes = [SP, BP, P, P, P, P, P, P, P, P, P, P, SZ, P]
     lib.vector_compact.argtypes = [SP, BP, P, P, P, P, CP, P]
+    lib.vector_append.argtypes = [SP, CP, P, P, I32, P]
+    lib.vector_append.restype = ctypes.c_int
     lib.vector_diagnostics.argtypes = [SP, BP, P, P, P, P, P, P, P]
     lib.vector_diagnostics.restype = ctypes.c_int
     lib.vector_decode_attn.argtypes = [SP, P, CP, P, P, I32, I32, P, SZ, P]
@@ -192,8 +210,8 @@ def _dev(t: torch.Tensor | None, dtype=None, name="tensor"):
 
 
 def _stream(stream) -> int:
-    if stream is None:
-        return torch.cuda.current_stream().cuda_stream
+    if stream is None:          # the handle itself: building a torch.cuda.Stream for it takes 3 us
+        return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device())
     return stream.cuda_stream if hasattr(stream, "cuda_stream") else int(stream)
 
 
@@ -256,7 +274,7 @@ def vector_calibrate(K: torch.Tensor, V: torch.Tensor, lam: float, want_r2: bool
 
 
 def vector_workspace_bytes(shape: Shape, budget: Budget) -> int:
-    return int(load_library().vector_workspace_bytes(ctypes.byref(shape._c()), ctypes.byref(budget._c())))
+    return int(load_library().vector_workspace_bytes(shape._p(), budget._p()))
 
 
 def alloc_workspace(shape: Shape, budget: Budget, device="cuda") -> torch.Tensor:
@@ -278,7 +296,7 @@ def alloc_cache(shape: Shape, budget: Budget, extra_rows: int = 0, device="cuda"
 
 def vector_score(shape: Shape, Q_obs, K, N: int, scores, raw_out=None, ws=None, stream=None):
     wp, wn = _ws(ws)
-    rc = load_library().vector_score(ctypes.byref(shape._c()), _dev(Q_obs, shape.torch_dtype, "Q_obs"),
+    rc = load_library().vector_score(shape._p(), _dev(Q_obs, shape.torch_dtype, "Q_obs"),
                                      _dev(K, shape.torch_dtype, "K"), N, _dev(scores, torch.float32, "scores"),
                                      _dev(raw_out, torch.float32, "raw_out"), wp, wn, _stream(stream))
     _check(rc, "vector_score")
@@ -286,21 +304,21 @@ def vector_score(shape: Shape, Q_obs, K, N: int, scores, raw_out=None, ws=None, 
 
 def vector_score_keydiff(shape: Shape, K, N: int, scores, ws=None, stream=None):
     wp, wn = _ws(ws)
-    rc = load_library().vector_score_keydiff(ctypes.byref(shape._c()), _dev(K, shape.torch_dtype, "K"), N,
+    rc = load_library().vector_score_keydiff(shape._p(), _dev(K, shape.torch_dtype, "K"), N,
                                              _dev(scores, torch.float32, "scores"), wp, wn, _stream(stream))
     _check(rc, "vector_score_keydiff")
 
 
 def vector_pool_select(shape: Shape, budget: Budget, scores, pool_idx, ws=None, stream=None):
     wp, wn = _ws(ws)
-    rc = load_library().vector_pool_select(ctypes.byref(shape._c()), ctypes.byref(budget._c()),
+    rc = load_library().vector_pool_select(shape._p(), budget._p(),
                                            _dev(scores, torch.float32, "scores"),
                                            _dev(pool_idx, torch.int32, "pool_idx"), wp, wn, _stream(stream))
     _check(rc, "vector_pool_select")
 
 
 def vector_residual(shape: Shape, K, V, W, N: int, idx, n_idx: int, eps, stream=None):
-    rc = load_library().vector_residual(ctypes.byref(shape._c()), _dev(K, shape.torch_dtype, "K"),
+    rc = load_library().vector_residual(shape._p(), _dev(K, shape.torch_dtype, "K"),
                                         _dev(V, shape.torch_dtype, "V"), _dev(W, shape.torch_dtype, "W"), N,
                                         _dev(idx, torch.int32, "idx"), n_idx, _dev(eps, torch.float32, "eps"),
                                         _stream(stream))
@@ -309,7 +327,7 @@ def vector_residual(shape: Shape, K, V, W, N: int, idx, n_idx: int, eps, stream=
 
 def vector_truncate(shape: Shape, budget: Budget, eps, pool_idx, tier, ret_idx, apx_idx, ws=None, stream=None):
     wp, wn = _ws(ws)
-    rc = load_library().vector_truncate(ctypes.byref(shape._c()), ctypes.byref(budget._c()),
+    rc = load_library().vector_truncate(shape._p(), budget._p(),
                                         _dev(eps, torch.float32, "eps"), _dev(pool_idx, torch.int32, "pool_idx"),
                                         _dev(tier, torch.uint8, "tier"), _dev(ret_idx, torch.int32, "ret_idx"),
                                         _dev(apx_idx, torch.int32, "apx_idx"), wp, wn, _stream(stream))
@@ -319,7 +337,7 @@ def vector_truncate(shape: Shape, budget: Budget, eps, pool_idx, tier, ret_idx, 
 def vector_route(shape: Shape, budget: Budget, scores, K, V, W, tier, ret_idx, apx_idx, eps_out=None,
                  pool_idx_out=None, ws=None, stream=None):
     wp, wn = _ws(ws)
-    rc = load_library().vector_route(ctypes.byref(shape._c()), ctypes.byref(budget._c()),
+    rc = load_library().vector_route(shape._p(), budget._p(),
                                      _dev(scores, torch.float32, "scores"), _dev(K, shape.torch_dtype, "K"),
                                      _dev(V, shape.torch_dtype, "V"), _dev(W, shape.torch_dtype, "W"),
                                      _dev(tier, torch.uint8, "tier"), _dev(ret_idx, torch.int32, "ret_idx"),
@@ -333,7 +351,7 @@ DIAG_FIELDS = ("E", "r2_approx", "mu_a", "sum_evicted_w", "sum_approximated_w", 
 
 def vector_diagnostics(shape: Shape, budget: Budget, importance, tier, pool_idx, eps, V, out, stream=None):
     """out [U][8] fp32: the DIAG_FIELDS of every unit."""
-    rc = load_library().vector_diagnostics(ctypes.byref(shape._c()), ctypes.byref(budget._c()),
+    rc = load_library().vector_diagnostics(shape._p(), budget._p(),
                                            _dev(importance, torch.float32, "importance"), _dev(tier, torch.uint8, "tier"),
                                            _dev(pool_idx, torch.int32, "pool_idx"), _dev(eps, torch.float32, "eps"),
                                            _dev(V, shape.torch_dtype, "V"), _dev(out, torch.float32, "out"), _stream(stream))
@@ -344,13 +362,13 @@ R2_FIELDS = ("r2", "ss_res", "ss_tot", "n")
 
 
 def vector_r2_global_workspace_bytes(shape: Shape, N: int) -> int:
-    return int(load_library().vector_r2_global_workspace_bytes(ctypes.byref(shape._c()), N))
+    return int(load_library().vector_r2_global_workspace_bytes(shape._p(), N))
 
 
 def vector_r2_global(shape: Shape, K, V, W, N: int, out, ws, stream=None):
     """out [U][4] fp32: the R2_FIELDS of every unit over all N tokens."""
     wp, wn = _ws(ws)
-    rc = load_library().vector_r2_global(ctypes.byref(shape._c()), _dev(K, shape.torch_dtype, "K"),
+    rc = load_library().vector_r2_global(shape._p(), _dev(K, shape.torch_dtype, "K"),
                                          _dev(V, shape.torch_dtype, "V"), _dev(W, shape.torch_dtype, "W"),
                                          N, _dev(out, torch.float32, "out"), wp, wn, _stream(stream))
     _check(rc, "vector_r2_global")
@@ -362,39 +380,47 @@ def vector_sync_check(stream=None):
 
 
 def vector_compact(shape: Shape, budget: Budget, K, V, ret_idx, apx_idx, cache: Cache, stream=None):
-    c = cache._c()
-    rc = load_library().vector_compact(ctypes.byref(shape._c()), ctypes.byref(budget._c()),
+    c = cache._p()
+    rc = load_library().vector_compact(shape._p(), budget._p(),
                                        _dev(K, shape.torch_dtype, "K"), _dev(V, shape.torch_dtype, "V"),
                                        _dev(ret_idx, torch.int32, "ret_idx"), _dev(apx_idx, torch.int32, "apx_idx"),
-                                       ctypes.byref(c), _stream(stream))
+                                       c, _stream(stream))
     _check(rc, "vector_compact")
+
+
+def vector_append(shape: Shape, cache: Cache, k_new, v_new, pos: int, stream=None):
+    """k_new, v_new [U][d] become row cache.n_ret of the retained pool; the caller bumps cache.n_ret."""
+    c = cache._p()
+    rc = load_library().vector_append(shape._p(), c, _dev(k_new, shape.torch_dtype, "k_new"),
+                                      _dev(v_new, shape.torch_dtype, "v_new"), pos, _stream(stream))
+    _check(rc, "vector_append")
 
 
 def vector_decode_attn(shape: Shape, q, cache: Cache, W, out, mode: int = 0, ws=None, stream=None):
     wp, wn = _ws(ws)
-    c = cache._c()
+    c = cache._p()
     if out.dtype not in (torch.float32, torch.bfloat16):
         raise ValueError("out must be fp32 or bf16")
     out_dt = VECTOR_BF16 if out.dtype == torch.bfloat16 else VECTOR_F32
-    rc = load_library().vector_decode_attn(ctypes.byref(shape._c()), _dev(q, shape.torch_dtype, "q"),
-                                           ctypes.byref(c), _dev(W, shape.torch_dtype, "W"), _dev(out, None, "out"),
+    rc = load_library().vector_decode_attn(shape._p(), _dev(q, shape.torch_dtype, "q"),
+                                           c, _dev(W, shape.torch_dtype, "W"), _dev(out, None, "out"),
                                            out_dt, mode, wp, wn, _stream(stream))
     _check(rc, "vector_decode_attn")
 
 
 # ---- one map per layer: scores, tiers and index lists per (sequence, layer); pools per head
 def vector_layer_workspace_bytes(shape: Shape, budget: Budget) -> int:
-    return int(load_library().vector_layer_workspace_bytes(ctypes.byref(shape._c()), ctypes.byref(budget._c())))
+    return int(load_library().vector_layer_workspace_bytes(shape._p(), budget._p()))
 
 
 def vector_layer_scores(shape: Shape, scores, N: int, layer_scores, stream=None):
-    rc = load_library().vector_layer_scores(ctypes.byref(shape._c()), _dev(scores, torch.float32, "scores"), N,
+    rc = load_library().vector_layer_scores(shape._p(), _dev(scores, torch.float32, "scores"), N,
                                             _dev(layer_scores, torch.float32, "layer_scores"), _stream(stream))
     _check(rc, "vector_layer_scores")
 
 
 def vector_residual_layer(shape: Shape, K, V, W_layer, N: int, idx, n_idx: int, eps, stream=None):
-    rc = load_library().vector_residual_layer(ctypes.byref(shape._c()), _dev(K, shape.torch_dtype, "K"),
+    rc = load_library().vector_residual_layer(shape._p(), _dev(K, shape.torch_dtype, "K"),
                                               _dev(V, shape.torch_dtype, "V"), _dev(W_layer, shape.torch_dtype, "W_layer"),
                                               N, _dev(idx, torch.int32, "idx"), n_idx, _dev(eps, torch.float32, "eps"),
                                               _stream(stream))
@@ -404,7 +430,7 @@ def vector_residual_layer(shape: Shape, K, V, W_layer, N: int, idx, n_idx: int, 
 def vector_route_layer(shape: Shape, budget: Budget, layer_scores, K, V, W_layer, tier, ret_idx, apx_idx,
                        eps_out=None, pool_idx_out=None, ws=None, stream=None):
     wp, wn = _ws(ws)
-    rc = load_library().vector_route_layer(ctypes.byref(shape._c()), ctypes.byref(budget._c()),
+    rc = load_library().vector_route_layer(shape._p(), budget._p(),
                                            _dev(layer_scores, torch.float32, "layer_scores"),
                                            _dev(K, shape.torch_dtype, "K"), _dev(V, shape.torch_dtype, "V"),
                                            _dev(W_layer, shape.torch_dtype, "W_layer"), _dev(tier, torch.uint8, "tier"),
@@ -415,22 +441,22 @@ def vector_route_layer(shape: Shape, budget: Budget, layer_scores, K, V, W_layer
 
 
 def vector_compact_layer(shape: Shape, budget: Budget, K, V, ret_idx, apx_idx, cache: Cache, stream=None):
-    c = cache._c()
-    rc = load_library().vector_compact_layer(ctypes.byref(shape._c()), ctypes.byref(budget._c()),
+    c = cache._p()
+    rc = load_library().vector_compact_layer(shape._p(), budget._p(),
                                              _dev(K, shape.torch_dtype, "K"), _dev(V, shape.torch_dtype, "V"),
                                              _dev(ret_idx, torch.int32, "ret_idx"), _dev(apx_idx, torch.int32, "apx_idx"),
-                                             ctypes.byref(c), _stream(stream))
+                                             c, _stream(stream))
     _check(rc, "vector_compact_layer")
 
 
 def vector_decode_attn_layer(shape: Shape, q, cache: Cache, W_layer, out, ws=None, stream=None):
     wp, wn = _ws(ws)
-    c = cache._c()
+    c = cache._p()
     if out.dtype not in (torch.float32, torch.bfloat16):
         raise ValueError("out must be fp32 or bf16")
     out_dt = VECTOR_BF16 if out.dtype == torch.bfloat16 else VECTOR_F32
-    rc = load_library().vector_decode_attn_layer(ctypes.byref(shape._c()), _dev(q, shape.torch_dtype, "q"),
-                                                 ctypes.byref(c), _dev(W_layer, shape.torch_dtype, "W_layer"),
+    rc = load_library().vector_decode_attn_layer(shape._p(), _dev(q, shape.torch_dtype, "q"),
+                                                 c, _dev(W_layer, shape.torch_dtype, "W_layer"),
                                                  _dev(out, None, "out"), out_dt, wp, wn, _stream(stream))
     _check(rc, "vector_decode_attn_layer")
 
@@ -440,7 +466,7 @@ VECTOR_STATIC_SCRATCH_BYTES = 16 << 20
 
 def vector_decode_scratch_bytes(shape: Shape) -> int:
     """Bytes of split-KV scratch a decode call of this shape needs (0 for an unsupported shape)."""
-    return int(load_library().vector_decode_scratch_bytes(ctypes.byref(shape._c())))
+    return int(load_library().vector_decode_scratch_bytes(shape._p()))
 
 
 def vector_decode_attn_static(shape: Shape, q, cache: Cache, W, out, mode: int = 0, stream=None):
@@ -452,11 +478,11 @@ def vector_decode_attn_static(shape: Shape, q, cache: Cache, W, out, mode: int =
     that need more raise VectorError (workspace).  Calls on one device share that array,
     so calls that overlap on the GPU race; make the first call per device at start-up.
     """
-    c = cache._c()
+    c = cache._p()
     if out.dtype not in (torch.float32, torch.bfloat16):
         raise ValueError("out must be fp32 or bf16")
     out_dt = VECTOR_BF16 if out.dtype == torch.bfloat16 else VECTOR_F32
-    rc = load_library().vector_decode_attn_static(ctypes.byref(shape._c()), _dev(q, shape.torch_dtype, "q"),
-                                                  ctypes.byref(c), _dev(W, shape.torch_dtype, "W"),
+    rc = load_library().vector_decode_attn_static(shape._p(), _dev(q, shape.torch_dtype, "q"),
+                                                  c, _dev(W, shape.torch_dtype, "W"),
                                                   _dev(out, None, "out"), out_dt, mode, _stream(stream))
     _check(rc, "vector_decode_attn_static")

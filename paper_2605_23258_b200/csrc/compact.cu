@@ -62,9 +62,35 @@ compact_kernel(const uint4* __restrict__ K, const uint4* __restrict__ V, int64_t
     }
 }
 
+// One generated token's K and V rows into the retained pool: row n_ret of every unit.  A thread moves one 16-byte piece.
+// What an append costs is its launch (three tensor assignments took 21 us of host time for 8 units of 128 channels), so
+// the kernel is a programmatic dependent of what precedes it and lets its own dependent (the decode step) start early.
+__global__ void __launch_bounds__(256)
+append_kernel(const uint4* __restrict__ k_new, const uint4* __restrict__ v_new, int lp, long long n, int64_t row, int64_t cap_ret,
+              int32_t pos, uint4* __restrict__ ret_k, uint4* __restrict__ ret_v, int32_t* __restrict__ ret_pos) {
+    asm volatile("griddepcontrol.wait;\n" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory");
+    const long long i = (long long)blockIdx.x * 256 + threadIdx.x;        // (unit, key or value, piece)
+    if (i >= n) return;
+    const int piece = (int)(i & ((1 << lp) - 1)), is_v = (int)(i >> lp) & 1;
+    const long long u = i >> (lp + 1);
+    const size_t dst = (((size_t)u * cap_ret + row) << lp) + piece;
+    if (is_v) ret_v[dst] = v_new[(u << lp) + piece];
+    else ret_k[dst] = k_new[(u << lp) + piece];
+    if (piece == 0 && !is_v) ret_pos[(size_t)u * cap_ret + row] = pos;
+}
+
 }  // namespace vec
 
 using namespace vec;
+
+// log2 of the 16-byte pieces of a row: 8, 16 or 32 for the supported shapes.
+static int log2_pieces(const Dims& dm) {
+    const int pieces = dm.d * dm.esize / 16;
+    int lp = 0;
+    while ((1 << lp) < pieces) ++lp;
+    return lp;
+}
 
 static vector_status compact_launch(const vector_shape* shape, const vector_budget* budget, const void* K,
                                     const void* V, const int32_t* ret_idx, const int32_t* apx_idx,
@@ -79,11 +105,9 @@ static vector_status compact_launch(const vector_shape* shape, const vector_budg
         return VECTOR_ERR_SHAPE;
     if (budget->n_ret > 0 && (!ret_idx || !cache->ret_k || !cache->ret_v || !cache->ret_pos)) return VECTOR_ERR_NULL;
     if (budget->n_apx > 0 && (!apx_idx || !cache->apx_k || !cache->apx_pos)) return VECTOR_ERR_NULL;
-    const int pieces = dm.d * dm.esize / 16;
     const int64_t rows = 2 * budget->n_ret + budget->n_apx;
     if (rows == 0) return VECTOR_OK;
-    int lp = 0;
-    while ((1 << lp) < pieces) ++lp;                  // pieces is 8, 16 or 32 for the supported shapes
+    const int lp = log2_pieces(dm);
     const int rows_per_block = COMPACT_PASSES * (COMPACT_THREADS >> lp);
     const int64_t chunks = (rows + rows_per_block - 1) / rows_per_block;
     const int64_t blocks = (int64_t)dm.U * chunks;
@@ -106,4 +130,19 @@ extern "C" vector_status vector_compact_layer(const vector_shape* shape, const v
                                               const void* V, const int32_t* ret_idx, const int32_t* apx_idx,
                                               const vector_cache* cache, void* stream) {
     return compact_launch(shape, budget, K, V, ret_idx, apx_idx, cache, stream, true);
+}
+
+extern "C" vector_status vector_append(const vector_shape* shape, const vector_cache* cache, const void* k_new,
+                                       const void* v_new, int32_t pos, void* stream) {
+    Dims dm;
+    vector_status rc = check_shape(shape, &dm);
+    if (rc != VECTOR_OK) return rc;
+    if (!cache || !k_new || !v_new || !cache->ret_k || !cache->ret_v || !cache->ret_pos) return VECTOR_ERR_NULL;
+    if (cache->n_ret < 0 || cache->n_ret >= cache->cap_ret) return VECTOR_ERR_SHAPE;
+    const int lp = log2_pieces(dm);
+    const long long n = (long long)dm.U << (lp + 1);
+    VEC_CUDA_CHECK(launch_maybe_dependent(true, append_kernel, dim3((unsigned)((n + 255) / 256)), dim3(256), 0, (cudaStream_t)stream,
+                                          (const uint4*)k_new, (const uint4*)v_new, lp, n, cache->n_ret, cache->cap_ret, pos,
+                                          (uint4*)cache->ret_k, (uint4*)cache->ret_v, cache->ret_pos));
+    return VECTOR_OK;
 }

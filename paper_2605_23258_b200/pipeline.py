@@ -68,9 +68,16 @@ class Compressor:
         c = self.cache
         if c.n_ret >= c.ret_k.shape[1]:
             raise ValueError("retained pool is full")
-        c.ret_k[:, c.n_ret] = k_new
-        c.ret_v[:, c.n_ret] = v_new
-        c.ret_pos[:, c.n_ret] = pos
+        rk = c.ret_k
+        U, _, d = rk.shape
+        if (type(pos) is int and -2**31 <= pos < 2**31 and k_new.shape == (U, d) and v_new.shape == (U, d)
+                and k_new.dtype == v_new.dtype == rk.dtype and k_new.is_contiguous() and v_new.is_contiguous()
+                and k_new.get_device() == v_new.get_device() == rk.get_device()):
+            B.vector_append(self.shape, c, k_new, v_new, pos)
+        else:                                   # anything that assigns to the rows: other types, broadcast or strided inputs
+            c.ret_k[:, c.n_ret] = k_new
+            c.ret_v[:, c.n_ret] = v_new
+            c.ret_pos[:, c.n_ret] = pos
         c.n_ret += 1
 
     def decode(self, q, W, out, mode: int = 0):
