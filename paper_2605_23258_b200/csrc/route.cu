@@ -56,10 +56,12 @@ __device__ __noinline__ void truncate_general(const float* __restrict__ e, int n
     sel::select_emit<true, NW, false>(e, n_pool, n_apx, n_apx > 0, S, L, dyn, emit);
 }
 
-// Step 1.  grid (U), 32 NW threads, L.bytes() of dynamic shared memory.
+// Step 1.  grid (U), 32 NW threads, L.bytes() of dynamic shared memory.  zero (nullable): [U][n_pool] floats set to zero,
+// for a residual kernel that adds its results up.
 template <int NW>
 __global__ void VEC_SEL_BOUNDS(NW)
-pool_select_kernel(const float* __restrict__ scores, int64_t N, int n_pool, int32_t* __restrict__ pool_idx, const Layout L) {
+pool_select_kernel(const float* __restrict__ scores, int64_t N, int n_pool, int32_t* __restrict__ pool_idx, float* __restrict__ zero,
+                   const Layout L) {
     __shared__ sel::Scratch S;
     extern __shared__ __align__(16) uint32_t sel_dyn[];
     // inside vector_route the residual kernel is launched as a programmatic dependent: its blocks may
@@ -69,6 +71,8 @@ pool_select_kernel(const float* __restrict__ scores, int64_t N, int n_pool, int3
     const float* s = scores + (size_t)u * N;
     int32_t* out = pool_idx + (size_t)u * n_pool;
     if (n_pool <= 0) return;
+    if (zero)
+        for (int i = threadIdx.x; i < n_pool; i += 32 * NW) zero[(size_t)u * n_pool + i] = 0.f;
     if (L.keyed && sel::select_lean<false, NW, true>(s, n, n_pool, S, L, sel_dyn, PoolOut{out})) return;
     pool_select_general<NW>(s, n, n_pool, out, S, L, sel_dyn);
 }
@@ -252,15 +256,15 @@ static SelPlan plan_selection(int64_t n, int U) {
 }
 
 static vector_status launch_pool_select(const Dims& dm, const vector_budget* budget, const float* scores, int32_t* pool,
-                                        cudaStream_t st) {
+                                        cudaStream_t st, float* zero = nullptr) {
     vector_status rc = select_kernels_setup();
     if (rc != VECTOR_OK) return rc;
     const int64_t n = budget->n_tokens;
     const SelPlan p = plan_selection(n, dm.U);
     const Layout L = p.L;
-    if (p.nw == 8) pool_select_kernel<8><<<dm.U, 256, L.bytes(), st>>>(scores, n, (int)budget->n_pool, pool, L);
-    else if (p.nw == 16) pool_select_kernel<16><<<dm.U, 512, L.bytes(), st>>>(scores, n, (int)budget->n_pool, pool, L);
-    else pool_select_kernel<32><<<dm.U, 1024, L.bytes(), st>>>(scores, n, (int)budget->n_pool, pool, L);
+    if (p.nw == 8) pool_select_kernel<8><<<dm.U, 256, L.bytes(), st>>>(scores, n, (int)budget->n_pool, pool, zero, L);
+    else if (p.nw == 16) pool_select_kernel<16><<<dm.U, 512, L.bytes(), st>>>(scores, n, (int)budget->n_pool, pool, zero, L);
+    else pool_select_kernel<32><<<dm.U, 1024, L.bytes(), st>>>(scores, n, (int)budget->n_pool, pool, zero, L);
     VEC_LAUNCH_CHECK();
     return VECTOR_OK;
 }
@@ -332,7 +336,7 @@ residual_layer_generic(const T* __restrict__ K, const T* __restrict__ V, const T
 
 static vector_status residual_layer_dispatch(const Dims& dm, int Hkv, int L, const void* K, const void* V, const void* W,
                                              int64_t N, const int32_t* idx, int64_t n_idx, float* eps, cudaStream_t st,
-                                             bool dependent) {
+                                             bool dependent, bool eps_zeroed) {
     if (n_idx == 0) return VECTOR_OK;
     const int UL = dm.U / Hkv;
     if (dm.dtype == VECTOR_BF16 && dm.d == 128) {
@@ -350,9 +354,13 @@ static vector_status residual_layer_dispatch(const Dims& dm, int Hkv, int L, con
         rlt::Params P;
         P.UL = UL; P.L = L; P.Hkv = Hkv; P.n_idx = (int)n_idx; P.N = N;
         P.tpu = (int)((n_idx + rlt::TILE - 1) / rlt::TILE);
-        P.n_tiles = (long long)UL * P.tpu;
+        P.pairs = (Hkv + 1) / 2;
+        const long long tiles = (long long)UL * P.tpu;
+        P.n_items = tiles * P.pairs;
         const int sms = sm_count();
-        const int blocks = (int)(P.n_tiles < sms ? P.n_tiles : sms);
+        // a block gets at least a tile, or exactly half of one where that leaves no more blocks than multiprocessors
+        const int blocks = (int)(tiles >= sms ? sms : 2 * tiles <= sms && P.pairs > 1 ? 2 * tiles : tiles);
+        if (!eps_zeroed) VEC_CUDA_CHECK(cudaMemsetAsync(eps, 0, (size_t)UL * (size_t)n_idx * sizeof(float), st));
         VEC_CUDA_CHECK(launch_maybe_dependent(dependent, rlt::residual_layer_tc, dim3(blocks), dim3(rlt::THREADS), rlt::SMEM_BYTES,
                                               st, (const __nv_bfloat16*)K, (const __nv_bfloat16*)V, mapW, idx, P, eps, fault));
         return VECTOR_OK;
@@ -457,7 +465,7 @@ extern "C" vector_status vector_residual_layer(const vector_shape* shape, const 
     if (N <= 0 || N > (int64_t(1) << 30) || n_idx < 0 || n_idx > N) return VECTOR_ERR_SHAPE;
     if (dm.rope) return VECTOR_ERR_UNSUPPORTED;
     return residual_layer_dispatch(dm, shape->n_kv_heads, shape->n_layers, K, V, W_layer, N, idx, n_idx, eps,
-                                   (cudaStream_t)stream, false);
+                                   (cudaStream_t)stream, false, false);
 }
 
 extern "C" vector_status vector_route_layer(const vector_shape* shape, const vector_budget* budget, const float* layer_scores,
@@ -482,8 +490,8 @@ extern "C" vector_status vector_route_layer(const vector_shape* shape, const vec
     p += align256((size_t)dl.U * (size_t)budget->n_pool * sizeof(int32_t));
     float* eps = eps_out ? eps_out : (float*)p;
     cudaStream_t st = (cudaStream_t)stream;
-    if ((rc = launch_pool_select(dl, budget, layer_scores, pool, st)) != VECTOR_OK) return rc;
-    rc = residual_layer_dispatch(dm, Hkv, shape->n_layers, K, V, W_layer, budget->n_tokens, pool, budget->n_pool, eps, st, true);
+    if ((rc = launch_pool_select(dl, budget, layer_scores, pool, st, eps)) != VECTOR_OK) return rc;      // zeroes eps as well
+    rc = residual_layer_dispatch(dm, Hkv, shape->n_layers, K, V, W_layer, budget->n_tokens, pool, budget->n_pool, eps, st, true, true);
     if (rc != VECTOR_OK) return rc;
     return launch_truncate(dl, budget, eps, pool, tier, ret_idx, apx_idx, st, true);
 }

@@ -1,0 +1,39 @@
+"""Residuals with one map per layer on the tensor-core kernel: odd numbers of heads, list ends around a tile, so few tiles that
+each is cut in two, and so many that blocks' ranges end inside tiles.  Bound: fp32 accumulation of exact products over
+Hkv d inputs in any order, |eps - want| <= 2 sqrt(want) |delta| + |delta|^2 + 2^-20 want, delta_c = (D + 2) 2^-23
+(|v_c| + sum |W||k|)."""
+import numpy as np
+import pytest
+import torch
+
+import paper_2605_23258_b200 as vec
+
+pytestmark = pytest.mark.gpu
+DEV = "cuda"
+
+
+@pytest.mark.parametrize("layers,Hkv,n_idx", [(1, 1, 1), (2, 3, 129), (1, 8, 128), (3, 2, 300), (30, 8, 700), (75, 3, 257), (151, 1, 100)])
+def test_residual_layer(oracle, layers, Hkv, n_idx):
+    N, d = 800, 128
+    D = Hkv * d
+    gen = torch.Generator(device=DEV).manual_seed(layers * 10 + Hkv)
+    K = (torch.randn(layers * Hkv, N, d, generator=gen, device=DEV) * 2).to(torch.bfloat16)
+    W = (torch.randn(layers, D, D, generator=gen, device=DEV) / np.sqrt(D)).to(torch.bfloat16)
+    V = torch.randn(layers * Hkv, N, d, generator=gen, device=DEV).to(torch.bfloat16)
+    idx = torch.stack([torch.randperm(N, generator=gen, device=DEV)[:n_idx].sort().values for _ in range(layers)]).to(torch.int32)
+    sh = vec.Shape(1, layers, 2 * Hkv, Hkv, d, vec.VECTOR_BF16, 16)
+    eps = [torch.full((layers, n_idx), float("nan"), device=DEV) for _ in range(2)]
+    for e in eps:
+        vec.vector_residual_layer(sh, K, V, W, N, idx, n_idx, e)
+    torch.cuda.synchronize()
+    assert vec.vector_device_fault() == 0
+    assert torch.equal(eps[0], eps[1])
+    for l in range(0, layers, max(1, layers // 5)):
+        rows = idx[l].long()
+        k = torch.cat([K[l * Hkv + h][rows] for h in range(Hkv)], 1).double().cpu().numpy()
+        v = torch.cat([V[l * Hkv + h][rows] for h in range(Hkv)], 1).double().cpu().numpy()
+        w = W[l].double().cpu().numpy()
+        want = oracle.residual_layer(K[l * Hkv:(l + 1) * Hkv].cpu(), V[l * Hkv:(l + 1) * Hkv].cpu(), W[l].cpu(), idx[l].cpu().numpy())
+        dn = np.sqrt((((D + 2) * 2.0 ** -23 * (np.abs(v) + np.abs(k) @ np.abs(w).T)) ** 2).sum(1))
+        err = np.abs(eps[0][l].double().cpu().numpy() - want)
+        assert np.all(err <= 2 * np.sqrt(want) * dn + dn ** 2 + 2.0 ** -20 * want), (l, float(err.max()))
