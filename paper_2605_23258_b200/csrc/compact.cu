@@ -21,6 +21,8 @@ compact_kernel(const uint4* __restrict__ K, const uint4* __restrict__ V, int64_t
                uint4* __restrict__ ret_k, uint4* __restrict__ ret_v, uint4* __restrict__ apx_k,
                int32_t* __restrict__ ret_pos, int32_t* __restrict__ apx_pos, int64_t cap_ret, int64_t cap_apx,
                int chunks, int idx_div) {
+    asm volatile("griddepcontrol.wait;\n" ::: "memory");        // launched as a programmatic dependent: nothing is touched before
+    asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory");
     const int rows = 2 * n_ret + n_apx, pieces = 1 << lp;
     const int u = blockIdx.x / chunks, chunk = blockIdx.x - u * chunks;
     const int ui = u / idx_div;                      // owner of the index lists: the unit, or its (sequence, layer)
@@ -112,11 +114,10 @@ static vector_status compact_launch(const vector_shape* shape, const vector_budg
     const int64_t chunks = (rows + rows_per_block - 1) / rows_per_block;
     const int64_t blocks = (int64_t)dm.U * chunks;
     if (blocks > 0x7fffffffLL) return VECTOR_ERR_SHAPE;
-    compact_kernel<<<(unsigned)blocks, COMPACT_THREADS, 0, (cudaStream_t)stream>>>(
+    VEC_CUDA_CHECK(launch_maybe_dependent(true, compact_kernel, dim3((unsigned)blocks), dim3(COMPACT_THREADS), 0, (cudaStream_t)stream,
         (const uint4*)K, (const uint4*)V, budget->n_tokens, lp, ret_idx, apx_idx, (int)budget->n_ret,
         (int)budget->n_apx, (uint4*)cache->ret_k, (uint4*)cache->ret_v, (uint4*)cache->apx_k, cache->ret_pos,
-        cache->apx_pos, cache->cap_ret, cache->cap_apx, (int)chunks, per_layer ? shape->n_kv_heads : 1);
-    VEC_LAUNCH_CHECK();
+        cache->apx_pos, cache->cap_ret, cache->cap_apx, (int)chunks, per_layer ? shape->n_kv_heads : 1));
     return VECTOR_OK;
 }
 

@@ -5,13 +5,13 @@
 // both pools once, accumulating p-weighted values and p-weighted keys, and the
 // d x d map is applied once per query head in the merge step.
 //
-// bf16 runs the kernels of decode_bf16.cuh and decode_pertile_tc.cuh; below, for fp32:
-//   split  grid (n_splits, U): online softmax over a slice of the logical key
-//          range [0, n_ret + n_apx); emits (m, l, acc_v[d], acc_k[d]) per head
-//   merge  grid (U): combines the splits, applies W to acc_k, normalises
+// bf16 runs the kernels of decode_bf16.cuh and decode_pertile_tc.cuh; below, for fp32, one
+// launch: a thread block cluster per unit, its blocks a slice each of the logical key range
+// [0, n_ret + n_apx); the blocks' sums are merged over distributed shared memory.
 #include <cmath>
 #include <mutex>
 
+#include "cluster.cuh"
 #include "common.cuh"
 #include "decode_bf16.cuh"
 #include "decode_pertile_tc.cuh"
@@ -33,28 +33,36 @@ template <> struct RowLoad<2> {
     }
 };
 
-// Partial record per (unit, split, head): [m, l, acc_v[D], acc_k[D]]
-template <int D> struct Rec { static constexpr int floats = 2 + 2 * D; };
+// Record of a warp or a block, per head: m, l, pad, acc_v[D], acc_k[D].
+template <int D> struct Rec { static constexpr int floats = 4 + 2 * D; };
+constexpr int F32_WARPS = 8, F32_ROWS = 4, F32_MAX_CLUSTER = 16;
 
+// A warp takes four rows at a time, a row across its lanes: the loads and the dot products' reductions of the four are
+// independent, where one row at a time left a chain of load, five shuffles and two exponentials per row and head (2 units of
+// 2 heads and 384 rows: 43 us, and 12 us for a merge kernel of two blocks).
 // With ROPE the approximated value is W applied to the key turned back by its original position
 // (apx_pos): the logit still uses the stored key, only the p-weighted key sum takes the turned one.
 // A lane holds EPL consecutive channels; the partner channel c +- D/2 sits in lane ^ 16.
+// grid (U x cluster size), 256 threads, F32_WARPS * g records of dynamic shared memory.
 template <int D, int G, bool ROPE>
-__global__ void __launch_bounds__(128)
-decode_split_generic(const float* __restrict__ q, const float* __restrict__ ret_k, const float* __restrict__ ret_v,
-                     const float* __restrict__ apx_k, const int32_t* __restrict__ apx_pos, int64_t cap_ret,
-                     int64_t cap_apx, int n_ret, int n_apx, int g, float scale, float theta,
-                     float* __restrict__ partial) {
-    constexpr int EPL = D / 32;
-    constexpr int REC = Rec<D>::floats;
-    __shared__ float sm[4][G][REC];
-    __shared__ double inv_freq[D / 2];
+__global__ void __launch_bounds__(32 * F32_WARPS)
+decode_f32(const float* __restrict__ q, const float* __restrict__ ret_k, const float* __restrict__ ret_v,
+           const float* __restrict__ apx_k, const int32_t* __restrict__ apx_pos, int64_t cap_ret, int64_t cap_apx, int n_ret,
+           int n_apx, int g, int LH, float scale, float theta, const float* __restrict__ W, void* __restrict__ out, int out_bf16) {
+    constexpr int EPL = D / 32, REC = Rec<D>::floats, NT = 32 * F32_WARPS;
+    extern __shared__ __align__(16) float recs[];               // [F32_WARPS][g][REC]
+    __shared__ __align__(16) float comb[G][REC];                // this block's sums, read by the whole cluster
+    __shared__ __align__(16) float aks[G][D];                   // merged key sums of this block's heads, and their value sums
+    __shared__ float avs[G][D], fac[G][F32_MAX_CLUSTER], Ls[G];
+    __shared__ double inv_freq[ROPE ? D / 2 : 1];
     if (ROPE) { rope_fill_inv_freq(inv_freq, D, theta); __syncthreads(); }
-    const int u = blockIdx.y, split = blockIdx.x, n_splits = gridDim.x;
+    // a programmatic dependent of what precedes it; nothing of its inputs is touched before this
+    asm volatile("griddepcontrol.wait;\n" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory");
+    const int C = (int)cl::nctas(), rank = (int)cl::rank(), u = blockIdx.x / C;
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     const int total = n_ret + n_apx;
-    const int per = (total + n_splits - 1) / n_splits;
-    const int lo = split * per, hi = min(total, lo + per);
+    const int lo = (int)((long long)rank * total / C), hi = (int)((long long)(rank + 1) * total / C);
 
     float qr[G][EPL], av[G][EPL], ak[G][EPL], m[G], l[G];
 #pragma unroll
@@ -69,44 +77,66 @@ decode_split_generic(const float* __restrict__ q, const float* __restrict__ ret_
             for (int e = 0; e < EPL; ++e) qr[a][e] *= scale;
         }
     }
-    for (int i = lo + wid; i < hi; i += 4) {
-        const bool retained = i < n_ret;
-        const float* kp = retained ? ret_k + ((size_t)u * cap_ret + i) * D
-                               : apx_k + ((size_t)u * cap_apx + (i - n_ret)) * D;
-        float kx[EPL], vx[EPL];
-        RowLoad<EPL>::load(kp, lane, kx);
-        if (retained) RowLoad<EPL>::load(ret_v + ((size_t)u * cap_ret + i) * D, lane, vx);
-        float kt[EPL];                       // what an approximated token contributes: the key, or the key turned back
+    for (int i0 = lo + wid; i0 < hi; i0 += F32_ROWS * F32_WARPS) {
+        float kx[F32_ROWS][EPL], vx[F32_ROWS][EPL], kt[F32_ROWS][EPL];        // kt: what an approximated token contributes
 #pragma unroll
-        for (int e = 0; e < EPL; ++e) kt[e] = kx[e];
-        if (ROPE && !retained) {
-            const double pos = (double)apx_pos[(size_t)u * cap_apx + (i - n_ret)];
+        for (int r = 0; r < F32_ROWS; ++r) {
+            const int i = i0 + r * F32_WARPS;
 #pragma unroll
-            for (int e = 0; e < EPL; ++e) {
-                float cs, sn;
-                rope_cos_sin(pos, inv_freq[(lane * EPL + e) % (D / 2)], cs, sn);
-                const float other = __shfl_xor_sync(0xffffffffu, kx[e], 16);
-                kt[e] = lane < 16 ? fmaf(kx[e], cs, other * sn) : fmaf(kx[e], cs, -other * sn);
+            for (int e = 0; e < EPL; ++e) { kx[r][e] = 0.f; vx[r][e] = 0.f; }
+            if (i < hi) {
+                RowLoad<EPL>::load(i < n_ret ? ret_k + ((size_t)u * cap_ret + i) * D : apx_k + ((size_t)u * cap_apx + (i - n_ret)) * D, lane, kx[r]);
+                if (i < n_ret) RowLoad<EPL>::load(ret_v + ((size_t)u * cap_ret + i) * D, lane, vx[r]);
+            }
+        }
+#pragma unroll
+        for (int r = 0; r < F32_ROWS; ++r) {
+            const int i = i0 + r * F32_WARPS;
+            const bool apx = i < hi && i >= n_ret;
+#pragma unroll
+            for (int e = 0; e < EPL; ++e) kt[r][e] = apx ? kx[r][e] : 0.f;
+            if (ROPE && apx) {
+                const double pos = (double)apx_pos[(size_t)u * cap_apx + (i - n_ret)];
+#pragma unroll
+                for (int e = 0; e < EPL; ++e) {
+                    float cs, sn;
+                    rope_cos_sin(pos, inv_freq[(lane * EPL + e) % (D / 2)], cs, sn);
+                    const float other = __shfl_xor_sync(0xffffffffu, kx[r][e], 16);
+                    kt[r][e] = lane < 16 ? fmaf(kx[r][e], cs, other * sn) : fmaf(kx[r][e], cs, -other * sn);
+                }
             }
         }
 #pragma unroll
         for (int a = 0; a < G; ++a) {
             if (a < g) {
-                float s = 0.f;
+                float s[F32_ROWS];
 #pragma unroll
-                for (int e = 0; e < EPL; ++e) s = fmaf(qr[a][e], kx[e], s);
-                s = warp_sum(s);
-                float mn = fmaxf(m[a], s);
-                float corr = __expf(m[a] - mn);     // first row: exp(-inf) = 0
-                float p = __expf(s - mn);
+                for (int r = 0; r < F32_ROWS; ++r) {
+                    s[r] = 0.f;
+#pragma unroll
+                    for (int e = 0; e < EPL; ++e) s[r] = fmaf(qr[a][e], kx[r][e], s[r]);
+                }
+#pragma unroll
+                for (int o = 16; o > 0; o >>= 1)
+#pragma unroll
+                    for (int r = 0; r < F32_ROWS; ++r) s[r] += __shfl_xor_sync(0xffffffffu, s[r], o);
+                float mn = m[a];
+#pragma unroll
+                for (int r = 0; r < F32_ROWS; ++r) {
+                    if (i0 + r * F32_WARPS >= hi) s[r] = -INFINITY;
+                    mn = fmaxf(mn, s[r]);                       // finite: row i0 is valid
+                }
+                const float corr = __expf(m[a] - mn);           // first rows: exp(-inf) = 0
                 m[a] = mn;
-                l[a] = l[a] * corr + p;
+                l[a] *= corr;
 #pragma unroll
-                for (int e = 0; e < EPL; ++e) {
-                    av[a][e] *= corr;
-                    ak[a][e] *= corr;
-                    if (retained) av[a][e] = fmaf(p, vx[e], av[a][e]);
-                    else          ak[a][e] = fmaf(p, kt[e], ak[a][e]);
+                for (int e = 0; e < EPL; ++e) { av[a][e] *= corr; ak[a][e] *= corr; }
+#pragma unroll
+                for (int r = 0; r < F32_ROWS; ++r) {
+                    const float p = __expf(s[r] - mn);
+                    l[a] += p;
+#pragma unroll
+                    for (int e = 0; e < EPL; ++e) { av[a][e] = fmaf(p, vx[r][e], av[a][e]); ak[a][e] = fmaf(p, kt[r][e], ak[a][e]); }
                 }
             }
         }
@@ -114,79 +144,112 @@ decode_split_generic(const float* __restrict__ q, const float* __restrict__ ret_
 #pragma unroll
     for (int a = 0; a < G; ++a) {
         if (a < g) {
-            if (lane == 0) { sm[wid][a][0] = m[a]; sm[wid][a][1] = l[a]; }
+            float* r = recs + (wid * g + a) * REC;
+            if (lane == 0) { r[0] = m[a]; r[1] = l[a]; }
 #pragma unroll
-            for (int e = 0; e < EPL; ++e) {
-                sm[wid][a][2 + lane * EPL + e] = av[a][e];
-                sm[wid][a][2 + D + lane * EPL + e] = ak[a][e];
-            }
+            for (int e = 0; e < EPL; ++e) { r[4 + lane * EPL + e] = av[a][e]; r[4 + D + lane * EPL + e] = ak[a][e]; }
         }
     }
     __syncthreads();
-    float* out = partial + ((size_t)u * n_splits + split) * g * REC;
-    for (int a = 0; a < g; ++a) {
-        float M = fmaxf(fmaxf(sm[0][a][0], sm[1][a][0]), fmaxf(sm[2][a][0], sm[3][a][0]));
-        float f[4];
+    for (int e = threadIdx.x; e < g * 2 * D; e += NT) {         // the block's sums
+        const int a = e / (2 * D), c = e % (2 * D);
+        float M = -INFINITY, L = 0.f, v = 0.f;
 #pragma unroll
-        for (int wv = 0; wv < 4; ++wv) f[wv] = sm[wv][a][0] > -INFINITY ? __expf(sm[wv][a][0] - M) : 0.f;
-        for (int c = threadIdx.x; c < REC; c += 128) {
-            float v;
-            if (c == 0) v = M;
-            else v = f[0] * sm[0][a][c] + f[1] * sm[1][a][c] + f[2] * sm[2][a][c] + f[3] * sm[3][a][c];
-            out[a * REC + c] = v;
+        for (int w = 0; w < F32_WARPS; ++w) M = fmaxf(M, recs[(w * g + a) * REC]);
+#pragma unroll
+        for (int w = 0; w < F32_WARPS; ++w) {
+            const float* r = recs + (w * g + a) * REC;
+            const float f = r[0] > -INFINITY ? __expf(r[0] - M) : 0.f;
+            L = fmaf(f, r[1], L);
+            v = fmaf(f, r[4 + c], v);
         }
+        if (c == 0) { comb[a][0] = M; comb[a][1] = L; }
+        comb[a][4 + c] = v;
     }
-}
-
-// grid (U), D threads.
-template <typename TO, int D>
-__global__ void __launch_bounds__(D)
-decode_merge_generic(const float* __restrict__ partial, const float* __restrict__ W, int LH, int g, int n_splits,
-                     TO* __restrict__ out) {
-    constexpr int REC = Rec<D>::floats;
-    __shared__ float aks[D];
-    const int u = blockIdx.x, c = threadIdx.x;
+    // the map, a row across a warp's lanes, requested before the cluster's barrier
+    constexpr int ROWS = D / F32_WARPS;
     const float* Wu = W + (size_t)(u % LH) * D * D;
-    for (int a = 0; a < g; ++a) {
-        const float* rec = partial + ((size_t)u * n_splits * g + a) * REC;
-        const size_t stride = (size_t)g * REC;
-        float M = -INFINITY;
-        for (int s = 0; s < n_splits; ++s) M = fmaxf(M, rec[s * stride]);
-        float L = 0.f, accv = 0.f, acck = 0.f;
-        for (int s = 0; s < n_splits; ++s) {
-            const float* r = rec + s * stride;
-            float f = r[0] > -INFINITY ? __expf(r[0] - M) : 0.f;
-            L += f * r[1];
-            accv += f * r[2 + c];
-            acck += f * r[2 + D + c];
+    float wr[ROWS][EPL];
+#pragma unroll
+    for (int r = 0; r < ROWS; ++r) RowLoad<EPL>::load(Wu + (size_t)(r * F32_WARPS + wid) * D, lane, wr[r]);
+    cl::arrive_release();
+    cl::wait_acquire();                                         // every block's sums are ready
+    const int mine = rank < g ? (g - rank + C - 1) / C : 0;     // this block merges heads rank, rank + C, ...
+    for (int k = wid; k < mine; k += F32_WARPS) {
+        const int a = rank + k * C;
+        float mj = -INFINITY, lj = 0.f;
+        if (lane < C) {
+            const uint32_t at = cl::map_to(tma::smem_u32(&comb[a][0]), (uint32_t)lane);
+            mj = cl::ld_f32(at);
+            lj = cl::ld_f32(at + 4);
         }
-        __syncthreads();
-        aks[c] = acck;
-        __syncthreads();
-        float proj = 0.f;
-#pragma unroll 8
-        for (int c2 = 0; c2 < D; ++c2) proj = fmaf(Wu[(size_t)c * D + c2], aks[c2], proj);
-        store_out(out + ((size_t)u * g + a) * D + c, (accv + proj) / L);
+        const float M = warp_max(mj);
+        const float f = mj > -INFINITY ? __expf(mj - M) : 0.f;
+        const float L = warp_sum(f * lj);
+        if (lane < C) fac[k][lane] = f;
+        if (lane == 0) Ls[k] = L;
     }
+    __syncthreads();
+    for (int e = threadIdx.x; e < mine * 2 * D; e += NT) {
+        const int k = e / (2 * D), c = e % (2 * D);
+        const uint32_t at = tma::smem_u32(&comb[rank + k * C][4 + c]);
+        float v = 0.f;
+        for (int j0 = 0; j0 < C; j0 += 8) {                     // eight remote loads in flight
+            float x[8];
+#pragma unroll
+            for (int j = 0; j < 8; ++j) x[j] = cl::ld_f32(cl::map_to(at, (uint32_t)min(j0 + j, C - 1)));
+#pragma unroll
+            for (int j = 0; j < 8; ++j) v = fmaf(j0 + j < C ? fac[k][j0 + j] : 0.f, x[j], v);
+        }
+        if (c < D) avs[k][c] = v;
+        else aks[k][c - D] = v;
+    }
+    cl::arrive_release();                                       // this block reads no other block's memory from here on
+    __syncthreads();
+    for (int k = 0; k < mine; ++k) {
+        float a[EPL];
+        RowLoad<EPL>::load(aks[k], lane, a);
+#pragma unroll
+        for (int r = 0; r < ROWS; ++r) {
+            float x = 0.f;
+#pragma unroll
+            for (int e = 0; e < EPL; ++e) x = fmaf(wr[r][e], a[e], x);
+            x = warp_sum(x);
+            const int c = r * F32_WARPS + wid;
+            const size_t at = ((size_t)u * g + rank + k * C) * D + c;
+            const float o = (avs[k][c] + x) / Ls[k];
+            if (lane == 0) {
+                if (out_bf16) reinterpret_cast<__nv_bfloat16*>(out)[at] = __float2bfloat16_rn(o);
+                else reinterpret_cast<float*>(out)[at] = o;
+            }
+        }
+    }
+    __syncwarp();
+    cl::wait_acquire();                                         // nobody reads this block's memory any more
 }
 
-template <int D, int G>
-static vector_status launch_decode(const Dims& dm, const void* q, const vector_cache* ch, const void* W, void* out,
-                                   int out_dtype, float* partial, cudaStream_t st) {
-    const int n_splits = decode_num_splits(dm.U, ch->n_ret + ch->n_apx);
-    dim3 grid(n_splits, dm.U);
-    auto kern = dm.rope ? decode_split_generic<D, G, true> : decode_split_generic<D, G, false>;
-    kern<<<grid, 128, 0, st>>>((const float*)q, (const float*)ch->ret_k, (const float*)ch->ret_v, (const float*)ch->apx_k,
-                               ch->apx_pos, ch->cap_ret, ch->cap_apx, (int)ch->n_ret, (int)ch->n_apx, dm.g,
-                               dm.scale, dm.theta, partial);
-    VEC_LAUNCH_CHECK();
-    if (out_dtype == VECTOR_F32)
-        decode_merge_generic<float, D><<<dm.U, D, 0, st>>>(partial, (const float*)W, dm.LH, dm.g, n_splits,
-                                                             (float*)out);
-    else
-        decode_merge_generic<__nv_bfloat16, D><<<dm.U, D, 0, st>>>(partial, (const float*)W, dm.LH, dm.g, n_splits,
-                                                                     (__nv_bfloat16*)out);
-    VEC_LAUNCH_CHECK();
+template <int D, int G, bool ROPE>
+static vector_status launch_decode_f32(const Dims& dm, const void* q, const vector_cache* ch, const void* W, void* out,
+                                       int out_dtype, cudaStream_t st) {
+    auto kern = decode_f32<D, G, ROPE>;
+    static PerDeviceOnce once;
+    if (once.first()) {
+        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, F32_WARPS * G * Rec<D>::floats * 4);
+        if (e == cudaSuccess) e = cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+        if (e != cudaSuccess) { once.undo(); VEC_CUDA_CHECK(e); }
+    }
+    // blocks a unit: one pass over the rows of a block's warps at the least, four blocks a multiprocessor at the most
+    const int64_t rows = ch->n_ret + ch->n_apx;
+    int64_t c = (rows + F32_ROWS * F32_WARPS - 1) / (F32_ROWS * F32_WARPS);
+    const int64_t fill = (4 * (int64_t)sm_count() + dm.U - 1) / dm.U;
+    if (c > fill) c = fill;
+    if (c > F32_MAX_CLUSTER) c = F32_MAX_CLUSTER;
+    if (c > 8 && c < F32_MAX_CLUSTER) c = 8;                    // beyond the portable size only the largest
+    VEC_CUDA_CHECK(launch_maybe_dependent(true, (int)c, kern, dim3((unsigned)(c * dm.U)), dim3(32 * F32_WARPS),
+                                          (size_t)F32_WARPS * dm.g * Rec<D>::floats * 4, st, (const float*)q, (const float*)ch->ret_k,
+                                          (const float*)ch->ret_v, (const float*)ch->apx_k, ch->apx_pos, ch->cap_ret, ch->cap_apx,
+                                          (int)ch->n_ret, (int)ch->n_apx, dm.g, dm.LH, dm.scale, dm.theta, (const float*)W, out,
+                                          out_dtype == VECTOR_BF16 ? 1 : 0));
     return VECTOR_OK;
 }
 
@@ -324,12 +387,12 @@ static vector_status launch_decode_bf16(const Dims& dm, const void* q, const vec
     return VECTOR_OK;
 }
 
-template <int D>
-static vector_status launch_decode_g(const Dims& dm, const void* q, const vector_cache* ch, const void* W,
-                                     void* out, int out_dtype, float* partial, cudaStream_t st) {
-    if (dm.g <= 2) return launch_decode<D, 2>(dm, q, ch, W, out, out_dtype, partial, st);
-    if (dm.g <= 4) return launch_decode<D, 4>(dm, q, ch, W, out, out_dtype, partial, st);
-    return launch_decode<D, 8>(dm, q, ch, W, out, out_dtype, partial, st);
+template <int D, bool ROPE>
+static vector_status launch_decode_g(const Dims& dm, const void* q, const vector_cache* ch, const void* W, void* out, int out_dtype,
+                                     cudaStream_t st) {
+    if (dm.g <= 2) return launch_decode_f32<D, 2, ROPE>(dm, q, ch, W, out, out_dtype, st);
+    if (dm.g <= 4) return launch_decode_f32<D, 4, ROPE>(dm, q, ch, W, out, out_dtype, st);
+    return launch_decode_f32<D, 8, ROPE>(dm, q, ch, W, out, out_dtype, st);
 }
 
 }  // namespace vec
@@ -358,8 +421,10 @@ extern "C" vector_status vector_decode_attn(const vector_shape* shape, const voi
     cudaStream_t st = (cudaStream_t)stream;
     float* partial = (float*)ws;
     if (dm.dtype == VECTOR_F32)
-        return dm.d == 64 ? launch_decode_g<64>(dm, q, cache, W, out, out_dtype, partial, st)
-                          : launch_decode_g<128>(dm, q, cache, W, out, out_dtype, partial, st);
+        return dm.d == 64 ? (dm.rope ? launch_decode_g<64, true>(dm, q, cache, W, out, out_dtype, st)
+                                     : launch_decode_g<64, false>(dm, q, cache, W, out, out_dtype, st))
+                          : (dm.rope ? launch_decode_g<128, true>(dm, q, cache, W, out, out_dtype, st)
+                                     : launch_decode_g<128, false>(dm, q, cache, W, out, out_dtype, st));
     if (dm.d == 64) return launch_decode_bf16<64>(dm, q, cache, W, out, out_dtype, mode, partial, st);
     return launch_decode_bf16<128>(dm, q, cache, W, out, out_dtype, mode, partial, st);
 }

@@ -101,7 +101,7 @@ vector_status check_budget(const vector_budget* b, int window) {
 }
 
 int score_num_chunks(int U, int R, int64_t N) {
-    int64_t tiles = (N + 127) / 128;
+    int64_t tiles = (N + 63) / 64;
     int64_t row_tiles = (R + 63) / 64;
     int64_t want = (8 * sm_count() + (int64_t)U * row_tiles - 1) / ((int64_t)U * row_tiles);
     if (want < 1) want = 1;
@@ -156,29 +156,14 @@ size_t select_ws_bytes(const Dims& D, const vector_budget& b) {
            align256((size_t)D.U * (size_t)b.n_pool * sizeof(float));
 }
 
-int decode_num_splits(int U, int64_t rows) {
-    int64_t want = (4 * sm_count() + U - 1) / U;
-    int64_t max_by_rows = (rows + 255) / 256;   // at least 256 rows per split
-    if (want > max_by_rows) want = max_by_rows;
-    if (want > 64) want = 64;
-    if (want < 1) want = 1;
-    return (int)want;
-}
-
 int decode_stream_slots(int U) {
     int s = (2 * sm_count() + U - 1) / U + 1;
     return s < 12 ? s : 12;
 }
 
 size_t decode_ws_bytes(const Dims& D) {
-    // the split count never exceeds what decode_num_splits returns for an unbounded row count,
-    // nor the record slots per unit of the persistent kernel
-    int s = decode_num_splits(D.U, int64_t(1) << 40);
-    // split kernel: per (unit, split, head) m, l, acc_v[d], acc_k[d]
-    size_t a = (size_t)D.U * s * D.g * (2 + 2 * (size_t)D.d) * sizeof(float);
     // persistent kernel: per (unit, slot, consumer warp, head) a 4-float header, acc_v[128], acc_k[128]
-    size_t b = (size_t)D.U * decode_stream_slots(D.U) * 4 * D.g * (4 + 256) * sizeof(float);
-    return align256(a > b ? a : b);
+    return align256((size_t)D.U * decode_stream_slots(D.U) * 4 * D.g * (4 + 256) * sizeof(float));
 }
 
 }  // namespace vec

@@ -67,8 +67,6 @@ struct PerDeviceOnce {
     void undo();           // the set-up failed: try again on the next call
 };
 size_t select_ws_bytes(const Dims& D, const vector_budget& b);
-// Number of key splits of one unit in decode attention for `rows` logical keys.
-int decode_num_splits(int U, int64_t rows);
 // Record slots per unit that the persistent bf16 decode kernel may use (two blocks per SM).
 int decode_stream_slots(int U);
 size_t decode_ws_bytes(const Dims& D);

@@ -64,8 +64,10 @@ pool_select_kernel(const float* __restrict__ scores, int64_t N, int n_pool, int3
                    const Layout L) {
     __shared__ sel::Scratch S;
     extern __shared__ __align__(16) uint32_t sel_dyn[];
-    // inside vector_route the residual kernel is launched as a programmatic dependent: its blocks may
-    // take SMs as this grid's blocks leave them; it reads the index lists only after its own wait
+    // A programmatic dependent of what precedes it: nothing is touched before the wait.  Inside vector_route the residual
+    // kernel is one of this kernel: its blocks may take SMs as this grid's blocks leave them -- what was before this kernel
+    // has finished then -- and it reads the index lists only after its own wait.
+    asm volatile("griddepcontrol.wait;\n" ::: "memory");
     asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory");
     const int u = blockIdx.x, n = (int)N;
     const float* s = scores + (size_t)u * N;
@@ -104,78 +106,123 @@ truncate_kernel(const float* __restrict__ eps, const int32_t* __restrict__ pool_
     truncate_general<NW>(e, n_pool, n_apx, emit, S, L, sel_dyn);
 }
 
-// Step 2 on CUDA cores (fp32).  grid (ceil(n_idx / 64), U), 256 threads; W^T staged in
-// dynamic shared memory as fp32 (D * (D+1) floats) plus one key row per warp.
+// Step 2 on CUDA cores (fp32).  A warp takes RW listed rows at once, a lane the output channels lane, lane + 32, ...: an
+// element of W^T read from shared memory serves the RW rows, and their loads are under way while W is staged (one row after
+// the other, each from its load to its sum: 30 us for 2 units of 384 rows).  RW = 4 where that leaves a block for
+// every multiprocessor, else 2.  grid (ceil(n_idx / (8 RW)), U), 256 threads; dynamic shared memory: W^T as D * (D+1)
+// floats plus RW key rows per warp.
 // With ROPE the regressor sees the key turned back by its position (the token index): channel c
 // pairs with c + D/2, angle -pos * theta^(-2c/D).
-template <int D, bool ROPE>
+template <int D, bool ROPE, int RW>
 __global__ void __launch_bounds__(256)
 residual_generic(const float* __restrict__ K, const float* __restrict__ V, const float* __restrict__ W, int64_t N,
                  int LH, const int32_t* __restrict__ idx, int n_idx, float theta, float* __restrict__ eps) {
-    extern __shared__ float smem[];
-    __shared__ double inv_freq[D / 2];
-    float* Wt = smem;                       // Wt[c_in * (D+1) + c_out]
-    float* ks = smem + D * (D + 1);         // [8][D]
+    constexpr int CPL = D / 32;             // channels per lane
+    extern __shared__ __align__(16) float smem[];
+    __shared__ double inv_freq[ROPE ? D / 2 : 1];
+    float* ks = smem;                       // [8][RW][D]
+    float* Wt = smem + 8 * RW * D;          // Wt[c_in * (D+1) + c_out]
     if (ROPE) rope_fill_inv_freq(inv_freq, D, theta);
+    asm volatile("griddepcontrol.wait;\n" ::: "memory");              // idx is complete and visible from here on
+    asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory");
     const int u = blockIdx.y, lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    const int p0 = (blockIdx.x * 8 + wid) * RW;
+    int64_t tok[RW];
+    float kr[RW][CPL], vr[RW][CPL];
+#pragma unroll
+    for (int r = 0; r < RW; ++r) tok[r] = p0 + r < n_idx ? idx[(size_t)u * n_idx + p0 + r] : -1;
+#pragma unroll
+    for (int r = 0; r < RW; ++r) {
+        const bool in = (uint64_t)tok[r] < (uint64_t)N;          // an index outside the unit reads as a row of zeros
+#pragma unroll
+        for (int m = 0; m < CPL; ++m) {
+            kr[r][m] = in ? K[((size_t)u * N + tok[r]) * D + lane + 32 * m] : 0.f;
+            vr[r][m] = in ? V[((size_t)u * N + tok[r]) * D + lane + 32 * m] : 0.f;
+        }
+    }
     const float* Wu = W + (size_t)(u % LH) * D * D;
+#pragma unroll 16
     for (int e = threadIdx.x; e < D * D; e += 256) {
-        int co = e / D, ci = e % D;
+        const int co = e / D, ci = e % D;
         Wt[ci * (D + 1) + co] = Wu[e];
     }
-    __syncthreads();
-    const int p_begin = blockIdx.x * 64;
-    const int p_end = min(n_idx, p_begin + 64);
-    float* kw = ks + wid * D;
-    for (int p = p_begin + wid; p < p_end; p += 8) {
-        const int64_t tok = idx[(size_t)u * n_idx + p];
-        if ((uint64_t)tok >= (uint64_t)N) {          // an index outside the unit reads as a row of zeros
-            if (lane == 0) eps[(size_t)u * n_idx + p] = 0.f;
-            continue;
-        }
-        const float* kr = K + ((size_t)u * N + tok) * D;
-        const float* vr = V + ((size_t)u * N + tok) * D;
-        __syncwarp();
+    float* kw = ks + wid * RW * D;
 #pragma unroll
-        for (int c = lane; c < D; c += 32) kw[c] = kr[c];
-        __syncwarp();
-        if (ROPE) {
+    for (int r = 0; r < RW; ++r)
+#pragma unroll
+        for (int m = 0; m < CPL; ++m) kw[r * D + lane + 32 * m] = kr[r][m];
+    __syncthreads();
+    if (ROPE) {
+#pragma unroll
+        for (int r = 0; r < RW; ++r)
 #pragma unroll
             for (int c = lane; c < D / 2; c += 32) {
                 float cs, sn;
-                rope_cos_sin((double)tok, inv_freq[c], cs, sn);
-                const float x = kw[c], y = kw[c + D / 2];
-                kw[c] = fmaf(x, cs, y * sn);
-                kw[c + D / 2] = fmaf(y, cs, -x * sn);
+                rope_cos_sin((double)tok[r], inv_freq[c], cs, sn);
+                const float x = kw[r * D + c], y = kw[r * D + c + D / 2];
+                kw[r * D + c] = fmaf(x, cs, y * sn);
+                kw[r * D + c + D / 2] = fmaf(y, cs, -x * sn);
             }
-            __syncwarp();
+        __syncwarp();
+    }
+    float pred[RW][CPL];
+#pragma unroll
+    for (int r = 0; r < RW; ++r)
+#pragma unroll
+        for (int m = 0; m < CPL; ++m) pred[r][m] = 0.f;
+#pragma unroll 4
+    for (int ci = 0; ci < D; ci += 4) {
+        float4 k[RW];
+#pragma unroll
+        for (int r = 0; r < RW; ++r) k[r] = *reinterpret_cast<const float4*>(kw + r * D + ci);
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+#pragma unroll
+            for (int m = 0; m < CPL; ++m) {
+                const float w = Wt[(ci + q) * (D + 1) + lane + 32 * m];
+#pragma unroll
+                for (int r = 0; r < RW; ++r) pred[r][m] = fmaf(w, q == 0 ? k[r].x : q == 1 ? k[r].y : q == 2 ? k[r].z : k[r].w, pred[r][m]);
+            }
         }
+    }
+#pragma unroll
+    for (int r = 0; r < RW; ++r) {
         float e = 0.f;
 #pragma unroll
-        for (int m = 0; m < D / 32; ++m) {
-            int co = lane + 32 * m;
-            float pred = 0.f;
-#pragma unroll 8
-            for (int ci = 0; ci < D; ++ci) pred = fmaf(Wt[ci * (D + 1) + co], kw[ci], pred);
-            float r = vr[co] - pred;
-            e = fmaf(r, r, e);
+        for (int m = 0; m < CPL; ++m) {
+            const float x = vr[r][m] - pred[r][m];
+            e = fmaf(x, x, e);
         }
         e = warp_sum(e);
-        if (lane == 0) eps[(size_t)u * n_idx + p] = e;
+        if (lane == 0 && p0 + r < n_idx) eps[(size_t)u * n_idx + p0 + r] = e;
     }
+}
+
+template <int D, bool ROPE, int RW>
+static vector_status launch_residual_rows(const Dims& dm, const void* K, const void* V, const void* W, int64_t N, const int32_t* idx,
+                                          int64_t n_idx, float* eps, cudaStream_t st) {
+    constexpr int SMEM = (D * (D + 1) + 8 * RW * D) * (int)sizeof(float);
+    auto kern = residual_generic<D, ROPE, RW>;
+    static PerDeviceOnce once;
+    if (once.first()) {
+        const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM);
+        if (e != cudaSuccess) { once.undo(); VEC_CUDA_CHECK(e); }
+    }
+    VEC_CUDA_CHECK(launch_maybe_dependent(true, kern, dim3((unsigned)((n_idx + 8 * RW - 1) / (8 * RW)), dm.U), dim3(256), SMEM, st,
+                                          (const float*)K, (const float*)V, (const float*)W, N, dm.LH, idx, (int)n_idx, dm.theta, eps));
+    return VECTOR_OK;
 }
 
 template <int D>
 static vector_status launch_residual(const Dims& dm, const void* K, const void* V, const void* W, int64_t N,
                                      const int32_t* idx, int64_t n_idx, float* eps, cudaStream_t st) {
     if (n_idx == 0) return VECTOR_OK;
-    size_t smem = (size_t)(D * (D + 1) + 8 * D) * sizeof(float);
-    auto kern = dm.rope ? residual_generic<D, true> : residual_generic<D, false>;
-    VEC_CUDA_CHECK(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    dim3 grid((unsigned)((n_idx + 63) / 64), dm.U);
-    kern<<<grid, 256, smem, st>>>((const float*)K, (const float*)V, (const float*)W, N, dm.LH, idx, (int)n_idx, dm.theta, eps);
-    VEC_LAUNCH_CHECK();
-    return VECTOR_OK;
+    const bool many = (n_idx + 31) / 32 * dm.U >= sm_count();
+    if (dm.rope)
+        return many ? launch_residual_rows<D, true, 4>(dm, K, V, W, N, idx, n_idx, eps, st)
+                    : launch_residual_rows<D, true, 2>(dm, K, V, W, N, idx, n_idx, eps, st);
+    return many ? launch_residual_rows<D, false, 4>(dm, K, V, W, N, idx, n_idx, eps, st)
+                : launch_residual_rows<D, false, 2>(dm, K, V, W, N, idx, n_idx, eps, st);
 }
 
 // bf16: gather + tcgen05 residual kernel.
@@ -262,10 +309,13 @@ static vector_status launch_pool_select(const Dims& dm, const vector_budget* bud
     const int64_t n = budget->n_tokens;
     const SelPlan p = plan_selection(n, dm.U);
     const Layout L = p.L;
-    if (p.nw == 8) pool_select_kernel<8><<<dm.U, 256, L.bytes(), st>>>(scores, n, (int)budget->n_pool, pool, zero, L);
-    else if (p.nw == 16) pool_select_kernel<16><<<dm.U, 512, L.bytes(), st>>>(scores, n, (int)budget->n_pool, pool, zero, L);
-    else pool_select_kernel<32><<<dm.U, 1024, L.bytes(), st>>>(scores, n, (int)budget->n_pool, pool, zero, L);
-    VEC_LAUNCH_CHECK();
+#define VEC_POOL(NW)                                                                                                     \
+    VEC_CUDA_CHECK(launch_maybe_dependent(true, pool_select_kernel<NW>, dim3(dm.U), dim3(32 * NW), L.bytes(), st, scores, n, \
+                                          (int)budget->n_pool, pool, zero, L))
+    if (p.nw == 8) VEC_POOL(8);
+    else if (p.nw == 16) VEC_POOL(16);
+    else VEC_POOL(32);
+#undef VEC_POOL
     return VECTOR_OK;
 }
 
