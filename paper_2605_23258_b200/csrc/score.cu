@@ -15,57 +15,73 @@
 namespace vec {
 
 constexpr int ST = 64;    // tile edge (rows and keys) of the CUDA-core score kernels (fp32)
-constexpr int SK = 32;    // head-dim slice staged per step
 
-// acc[i][j] += sum_c Q[row0 + ty + 16 i][c] * K[key0 + tx + 16 j][c]
+// The CUDA-core passes hold a whole 64 x D tile of each operand in shared memory (rows D + 1 apart) and request the next
+// tile of the one that changes before they work on this one: with 32-channel slices loaded between barriers a pass was a
+// chain of load latencies (13 + 11 us for 2 units of 64 rows and 1024 keys).
+template <int D> struct TileRegs { float4 v[ST * D / 1024]; };
 template <int D>
-__device__ __forceinline__ void tile_qk(const float* __restrict__ Qu, const float* __restrict__ Ku, int R,
-                                        int64_t N, int row0, int64_t key0, float (*Qs)[SK + 1],
-                                        float (*Ks)[SK + 1], float acc[4][4]) {
-    const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
+__device__ __forceinline__ void tile_request(const float* __restrict__ src, int64_t row0, int64_t n_rows, TileRegs<D>& t) {
+#pragma unroll
+    for (int e = 0; e < ST * D / 1024; ++e) {
+        const int idx = threadIdx.x + 256 * e, r = idx / (D / 4), c4 = idx % (D / 4);
+        t.v[e] = row0 + r < n_rows ? reinterpret_cast<const float4*>(src + (row0 + r) * D)[c4] : make_float4(0.f, 0.f, 0.f, 0.f);
+    }
+}
+template <int D>
+__device__ __forceinline__ void tile_store(const TileRegs<D>& t, float* dst) {
+#pragma unroll
+    for (int e = 0; e < ST * D / 1024; ++e) {
+        const int idx = threadIdx.x + 256 * e, r = idx / (D / 4), c = idx % (D / 4) * 4;
+        float* p = dst + r * (D + 1) + c;
+        p[0] = t.v[e].x; p[1] = t.v[e].y; p[2] = t.v[e].z; p[3] = t.v[e].w;
+    }
+}
+// acc[i][j] = sum_c Qs[ty + 16 i][c] * Ks[tx + 16 j][c]
+template <int D>
+__device__ __forceinline__ void tile_qk(const float* Qs, const float* Ks, float acc[4][4]) {
+    const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
 #pragma unroll
     for (int i = 0; i < 4; ++i)
 #pragma unroll
         for (int j = 0; j < 4; ++j) acc[i][j] = 0.f;
-    for (int dc = 0; dc < D; dc += SK) {
-        __syncthreads();
+#pragma unroll 16
+    for (int kk = 0; kk < D; ++kk) {
+        float a[4], b[4];
 #pragma unroll
-        for (int e = 0; e < (ST * SK) / 256; ++e) {
-            int idx = tid + 256 * e, r = idx / SK, c = idx % SK;
-            int row = row0 + r;
-            int64_t key = key0 + r;
-            Qs[r][c] = row < R ? Qu[(size_t)row * D + dc + c] : 0.f;
-            Ks[r][c] = key < N ? Ku[(size_t)key * D + dc + c] : 0.f;
-        }
-        __syncthreads();
+        for (int i = 0; i < 4; ++i) a[i] = Qs[(ty + 16 * i) * (D + 1) + kk];
 #pragma unroll
-        for (int kk = 0; kk < SK; ++kk) {
-            float a[4], b[4];
+        for (int j = 0; j < 4; ++j) b[j] = Ks[(tx + 16 * j) * (D + 1) + kk];
 #pragma unroll
-            for (int i = 0; i < 4; ++i) a[i] = Qs[ty + 16 * i][kk];
+        for (int i = 0; i < 4; ++i)
 #pragma unroll
-            for (int j = 0; j < 4; ++j) b[j] = Ks[tx + 16 * j][kk];
-#pragma unroll
-            for (int i = 0; i < 4; ++i)
-#pragma unroll
-                for (int j = 0; j < 4; ++j) acc[i][j] = fmaf(a[i], b[j], acc[i][j]);
-        }
+            for (int j = 0; j < 4; ++j) acc[i][j] = fmaf(a[i], b[j], acc[i][j]);
     }
 }
+template <int D> constexpr int tile_smem() { return 2 * ST * (D + 1) * (int)sizeof(float); }
 
-// grid (n_chunks, row_tiles, U), 256 threads
+// grid (n_chunks, row_tiles, U), 256 threads, tile_smem of dynamic shared memory
 template <int D>
 __global__ void __launch_bounds__(256)
 score_pass1_generic(const float* __restrict__ Q, const float* __restrict__ K, int64_t N, int R, int w,
                     float scale, int64_t chunk_len, float2* __restrict__ partial) {
-    __shared__ float Qs[ST][SK + 1];
-    __shared__ float Ks[ST][SK + 1];
+    extern __shared__ float tiles[];
+    float *Qs = tiles, *Ks = tiles + ST * (D + 1);
+    asm volatile("griddepcontrol.wait;\n" ::: "memory");        // launched as a programmatic dependent: nothing is touched before
+    asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory");
     const int u = blockIdx.z, row0 = blockIdx.y * ST, chunk = blockIdx.x, n_chunks = gridDim.x;
     const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
     const float* Qu = Q + (size_t)u * R * D;
     const float* Ku = K + (size_t)u * N * D;
     const int64_t k_begin = (int64_t)chunk * chunk_len;
     const int64_t k_end = min(N, k_begin + chunk_len);
+    TileRegs<D> next;
+    tile_request<D>(Ku, k_begin, k_end, next);
+    {
+        TileRegs<D> q;
+        tile_request<D>(Qu, row0, R, q);
+        tile_store<D>(q, Qs);
+    }
     float m[4], l[4];
     int64_t last_visible[4];   // row j of the window sits at position N - w + j
 #pragma unroll
@@ -76,8 +92,12 @@ score_pass1_generic(const float* __restrict__ Q, const float* __restrict__ K, in
         last_visible[i] = row < R ? N - w + (row % w) : -1;
     }
     for (int64_t key0 = k_begin; key0 < k_end; key0 += ST) {
+        __syncthreads();                                  // the tile before this one has been read
+        tile_store<D>(next, Ks);
+        __syncthreads();
+        if (key0 + ST < k_end) tile_request<D>(Ku, key0 + ST, k_end, next);
         float acc[4][4];
-        tile_qk<D>(Qu, Ku, R, N, row0, key0, Qs, Ks, acc);
+        tile_qk<D>(Qs, Ks, acc);
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
             float s[4], mx = m[i];
@@ -110,45 +130,86 @@ score_pass1_generic(const float* __restrict__ Q, const float* __restrict__ K, in
     }
 }
 
-// grid (U), block 256: lse[u][row] from the chunk partials
-__global__ void score_lse_combine(const float2* __restrict__ partial, int R, int n_chunks,
-                                  float* __restrict__ lse) {
-    const int u = blockIdx.x;
-    for (int row = threadIdx.x; row < R; row += blockDim.x) {
-        float M = -INFINITY;
-        for (int c = 0; c < n_chunks; ++c) M = fmaxf(M, partial[((size_t)u * n_chunks + c) * R + row].x);
-        float L = 0.f;
-        for (int c = 0; c < n_chunks; ++c) {
-            float2 p = partial[((size_t)u * n_chunks + c) * R + row];
-            if (p.x > -INFINITY) L += p.y * expf(p.x - M);
+// lse of a row from its chunk partials, `stride` apart, four lanes (of one aligned group) together.
+__device__ __forceinline__ float row_lse(const float2* __restrict__ p, int stride, int n_chunks) {
+    const int part = threadIdx.x & 3;
+    float M = -INFINITY, L = 0.f;
+    for (int c0 = part; c0 < n_chunks; c0 += 16) {
+        float2 v[4];
+        float m = M;
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            v[k] = c0 + 4 * k < n_chunks ? p[(size_t)(c0 + 4 * k) * stride] : make_float2(-INFINITY, 0.f);
+            m = fmaxf(m, v[k].x);
         }
-        lse[(size_t)u * R + row] = M + logf(L);
+        if (m == -INFINITY) continue;
+        L *= expf(M - m);
+#pragma unroll
+        for (int k = 0; k < 4; ++k) L += v[k].y * expf(v[k].x - m);
+        M = m;
     }
+#pragma unroll
+    for (int o = 1; o < 4; o <<= 1) {
+        const float M2 = __shfl_xor_sync(0xffffffffu, M, o), L2 = __shfl_xor_sync(0xffffffffu, L, o);
+        const float m = fmaxf(M, M2);
+        L = m > -INFINITY ? L * expf(M - m) + L2 * expf(M2 - m) : 0.f;
+        M = m;
+    }
+    return M + logf(L);
+}
+// lse[u][row].  grid (ceil(R / 64), U), 256 threads
+__global__ void __launch_bounds__(256)
+score_lse_rows(const float2* __restrict__ partial, int R, int n_chunks, float* __restrict__ lse) {
+    asm volatile("griddepcontrol.wait;\n" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory");
+    const int row = blockIdx.x * 64 + (threadIdx.x >> 2);
+    const float v = row_lse(partial + (size_t)blockIdx.y * n_chunks * R + min(row, R - 1), R, n_chunks);
+    if (row < R && (threadIdx.x & 3) == 0) lse[(size_t)blockIdx.y * R + row] = v;
 }
 
-// grid (key_tiles, U), 256 threads
-template <int D>
+// grid (key_tiles, U), 256 threads, tile_smem of dynamic shared memory.  INLINE_LSE: a block forms the normalisers of its
+// rows itself from the chunk partials (a launch less; every key tile repeats it).
+template <int D, bool INLINE_LSE>
 __global__ void __launch_bounds__(256)
 score_pass2_generic(const float* __restrict__ Q, const float* __restrict__ K, int64_t N, int R, int w,
-                    float scale, const float* __restrict__ lse, float* __restrict__ raw) {
-    __shared__ float Qs[ST][SK + 1];
-    __shared__ float Ks[ST][SK + 1];
+                    float scale, const float2* __restrict__ partial, int n_chunks, const float* __restrict__ lse, float* __restrict__ raw) {
+    extern __shared__ float tiles[];
+    float *Qs = tiles, *Ks = tiles + ST * (D + 1);
     __shared__ float red[16][ST];
+    __shared__ float lse_s[ST];
+    asm volatile("griddepcontrol.wait;\n" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory");
     const int u = blockIdx.y;
     const int64_t key0 = (int64_t)blockIdx.x * ST;
     const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
     const float* Qu = Q + (size_t)u * R * D;
-    const float* Ku = K + (size_t)u * N * D;
-    const float* lse_u = lse + (size_t)u * R;
+    TileRegs<D> next;
+    {
+        TileRegs<D> k;
+        tile_request<D>(K + (size_t)u * N * D, key0, N, k);
+        tile_request<D>(Qu, 0, R, next);
+        tile_store<D>(k, Ks);
+    }
     float col[4] = {0.f, 0.f, 0.f, 0.f};
     for (int row0 = 0; row0 < R; row0 += ST) {
+        __syncthreads();                                  // the rows before these have been read
+        tile_store<D>(next, Qs);
+        if (INLINE_LSE) {
+            const int row = row0 + (tid >> 2);
+            const float v = row_lse(partial + (size_t)u * n_chunks * R + min(row, R - 1), R, n_chunks);
+            if ((tid & 3) == 0) lse_s[tid >> 2] = v;
+        } else if (tid < ST && row0 + tid < R) {
+            lse_s[tid] = lse[(size_t)u * R + row0 + tid];
+        }
+        __syncthreads();
+        if (row0 + ST < R) tile_request<D>(Qu, row0 + ST, R, next);
         float acc[4][4];
-        tile_qk<D>(Qu, Ku, R, N, row0, key0, Qs, Ks, acc);
+        tile_qk<D>(Qs, Ks, acc);
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
             int row = row0 + ty + 16 * i;
             if (row < R) {
-                float ls = lse_u[row];
+                float ls = lse_s[ty + 16 * i];
                 int64_t last_visible = N - w + (row % w);
 #pragma unroll
                 for (int j = 0; j < 4; ++j) {
@@ -173,6 +234,8 @@ score_pass2_generic(const float* __restrict__ Q, const float* __restrict__ K, in
 // score[i] = max_{|j-i| <= r, 0 <= j < N-w} raw[j] for i < N-w ; +inf for the window tokens
 __global__ void score_pool_kernel(const float* __restrict__ raw, int64_t N, int w, int r, int64_t total,
                                   float* __restrict__ score) {
+    asm volatile("griddepcontrol.wait;\n" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory");
     int64_t gi = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (gi >= total) return;
     int64_t u = gi / N, i = gi - u * N;
@@ -187,25 +250,34 @@ __global__ void score_pool_kernel(const float* __restrict__ raw, int64_t N, int 
 }
 
 template <int D>
-static vector_status launch_score(const Dims& dm, const void* Q, const void* K, int64_t N, float* scores,
+static vector_status launch_score(const Dims& dm, const float* Q, const float* K, int64_t N, float* scores,
                                   float* raw, float2* partial, float* lse, cudaStream_t st) {
-    const int n_chunks = score_num_chunks(dm.U, dm.R, N);
+    constexpr int SMEM = tile_smem<D>();
+    static PerDeviceOnce once;
+    if (once.first()) {
+        cudaError_t e = cudaFuncSetAttribute(score_pass1_generic<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM);
+        if (e == cudaSuccess) e = cudaFuncSetAttribute(score_pass2_generic<D, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM);
+        if (e == cudaSuccess) e = cudaFuncSetAttribute(score_pass2_generic<D, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM);
+        if (e != cudaSuccess) { once.undo(); VEC_CUDA_CHECK(e); }
+    }
+    int n_chunks = score_num_chunks(dm.U, dm.R, N);
     int64_t chunk_len = (N + n_chunks - 1) / n_chunks;
-    chunk_len = (chunk_len + 127) / 128 * 128;
+    chunk_len = (chunk_len + ST - 1) / ST * ST;
+    n_chunks = (int)((N + chunk_len - 1) / chunk_len);            // none empty
     const int row_tiles = (dm.R + ST - 1) / ST;
-    dim3 g1(n_chunks, row_tiles, dm.U);
-    score_pass1_generic<D><<<g1, 256, 0, st>>>((const float*)Q, (const float*)K, N, dm.R, dm.w, dm.scale,
-                                                  chunk_len, partial);
-    VEC_LAUNCH_CHECK();
-    score_lse_combine<<<dm.U, 256, 0, st>>>(partial, dm.R, n_chunks, lse);
-    VEC_LAUNCH_CHECK();
-    dim3 g2((unsigned)((N + ST - 1) / ST), dm.U);
-    score_pass2_generic<D><<<g2, 256, 0, st>>>((const float*)Q, (const float*)K, N, dm.R, dm.w, dm.scale, lse, raw);
-    VEC_LAUNCH_CHECK();
+    VEC_CUDA_CHECK(launch_maybe_dependent(true, score_pass1_generic<D>, dim3(n_chunks, row_tiles, dm.U), dim3(256), SMEM, st, Q, K, N,
+                                          dm.R, dm.w, dm.scale, chunk_len, partial));
+    // the partials of a row tile: no more than the rows' own elements
+    const bool inline_lse = n_chunks <= 32;
+    if (!inline_lse)
+        VEC_CUDA_CHECK(launch_maybe_dependent(true, score_lse_rows, dim3((dm.R + 63) / 64, dm.U), dim3(256), 0, st, partial, dm.R,
+                                              n_chunks, lse));
+    VEC_CUDA_CHECK(launch_maybe_dependent(true, inline_lse ? score_pass2_generic<D, true> : score_pass2_generic<D, false>,
+                                          dim3((unsigned)((N + ST - 1) / ST), dm.U), dim3(256), SMEM, st, Q, K, N, dm.R, dm.w, dm.scale,
+                                          partial, n_chunks, lse, raw));
     int64_t total = (int64_t)dm.U * N;
-    score_pool_kernel<<<(unsigned)((total + 255) / 256), 256, 0, st>>>(raw, N, dm.w, dm.pool_kernel / 2,
-                                                                       total, scores);
-    VEC_LAUNCH_CHECK();
+    VEC_CUDA_CHECK(launch_maybe_dependent(true, score_pool_kernel, dim3((unsigned)((total + 255) / 256)), dim3(256), 0, st, raw, N, dm.w,
+                                          dm.pool_kernel / 2, total, scores));
     return VECTOR_OK;
 }
 
@@ -284,6 +356,7 @@ extern "C" vector_status vector_score(const vector_shape* shape, const void* Q_o
     p += align256((size_t)dm.U * dm.R * sizeof(float));
     float* raw = need_raw ? (float*)p : raw_out;
     cudaStream_t st = (cudaStream_t)stream;
-    return dm.d == 64 ? launch_score<64>(dm, Q_obs, K, N, scores, raw, partial, lse, st)
-                      : launch_score<128>(dm, Q_obs, K, N, scores, raw, partial, lse, st);
+    const float *q = (const float*)Q_obs, *k = (const float*)K;
+    return dm.d == 64 ? launch_score<64>(dm, q, k, N, scores, raw, partial, lse, st)
+                      : launch_score<128>(dm, q, k, N, scores, raw, partial, lse, st);
 }
