@@ -241,19 +241,24 @@ static vector_status launch_layer_mma(const Dims& dm, int L, const void* q, cons
     }
     const int UL = dm.U / dlm::HKV;
     const int64_t tiles = (ch->n_ret + dlm::RT - 1) / dlm::RT + (ch->n_apx + dlm::AT - 1) / dlm::AT;
-    int64_t n_splits = (2 * (int64_t)sm_count() + UL - 1) / UL;       // two rounds of blocks
-    if (n_splits > tiles) n_splits = tiles;
-    if (n_splits > 32) n_splits = 32;
-    if (n_splits < 1) n_splits = 1;
-    dlm::decode_layer_mma<<<dim3((unsigned)n_splits, UL), dlm::THREADS, dlm::SMEM_BYTES, st>>>(
+    // Splits: a multiprocessor holds one block, so the time goes with whole rounds of blocks over the splits' number (32
+    // layers: 9 splits are two rounds, 10 were three: 218 us against 150); a split also costs its records (about 3 % of a
+    // round each).
+    int64_t n_splits = 1;
+    double best = 1e30;
+    for (int64_t n = 1; n <= 32 && n <= tiles; ++n) {
+        const double t = (double)((n * UL + sm_count() - 1) / sm_count()) / (double)n * (1.0 + 0.03 * n / ((n * UL + sm_count() - 1) / sm_count()));
+        if (t < best - 1e-9) { best = t; n_splits = n; }
+    }
+    VEC_CUDA_CHECK(launch_maybe_dependent(true, dlm::decode_layer_mma, dim3((unsigned)n_splits, UL), dim3(dlm::THREADS), dlm::SMEM_BYTES, st,
         (const T*)q, (const T*)ch->ret_k, (const T*)ch->ret_v, (const T*)ch->apx_k, (long long)ch->cap_ret, (long long)ch->cap_apx,
-        (int)ch->n_ret, (int)ch->n_apx, dm.g, dm.scale * 1.4426950408889634f, partial);
-    VEC_LAUNCH_CHECK();
+        (int)ch->n_ret, (int)ch->n_apx, dm.g, dm.scale * 1.4426950408889634f, partial));
     if (out_dtype == VECTOR_F32)
-        dlm::decode_layer_merge_mma<float><<<dm.U, 256, 0, st>>>(partial, (const T*)W, L, dm.g, (int)n_splits, (float*)out);
+        VEC_CUDA_CHECK(launch_maybe_dependent(true, dlm::decode_layer_merge_mma<float>, dim3(dm.U), dim3(dlm::MERGE_THREADS), 0, st, partial,
+                                              (const T*)W, L, dm.g, (int)n_splits, (float*)out));
     else
-        dlm::decode_layer_merge_mma<T><<<dm.U, 256, 0, st>>>(partial, (const T*)W, L, dm.g, (int)n_splits, (T*)out);
-    VEC_LAUNCH_CHECK();
+        VEC_CUDA_CHECK(launch_maybe_dependent(true, dlm::decode_layer_merge_mma<T>, dim3(dm.U), dim3(dlm::MERGE_THREADS), 0, st, partial,
+                                              (const T*)W, L, dm.g, (int)n_splits, (T*)out));
     return VECTOR_OK;
 }
 

@@ -30,6 +30,8 @@ constexpr int RT = 16, AT = 32;                            // tokens per retaine
 constexpr int STAGE_BYTES = 65536, HEAD_RET = RT * 256, HEAD_APX = AT * 256;
 constexpr int PS_ROW = 80;                                 // bytes per row of P: 32 tokens + padding (conflict-free ldmatrix)
 constexpr int STAGES = 2;
+constexpr int RET_COST = 1, APX_COST = 2;                  // relative time of a tile (measured: 1:1 246, 1:2 239, 2:5 248, 1:4 258 us
+                                                           // a step of 32 layers and 7200 rows; 82, 58, 62 and 74 for one layer)
 constexpr int SMEM_BYTES = STAGES * STAGE_BYTES + 2 * MQ * PS_ROW + MQ * 4 + 128;
 constexpr int REC = 2 + 128 + HKV * 128;
 
@@ -38,6 +40,8 @@ __global__ void __launch_bounds__(THREADS, 1)
 decode_layer_mma(const __nv_bfloat16* __restrict__ q, const __nv_bfloat16* __restrict__ ret_k,
                  const __nv_bfloat16* __restrict__ ret_v, const __nv_bfloat16* __restrict__ apx_k, long long cap_ret,
                  long long cap_apx, int n_ret, int n_apx, int g, float scale_log2e, float* __restrict__ partial) {
+    asm volatile("griddepcontrol.wait;\n" ::: "memory");        // launched as a programmatic dependent: nothing is touched before
+    asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory");
     extern __shared__ __align__(128) unsigned char lsm[];
     unsigned char* stage0 = lsm;
     unsigned char* ps_hi = lsm + STAGES * STAGE_BYTES;
@@ -46,9 +50,14 @@ decode_layer_mma(const __nv_bfloat16* __restrict__ q, const __nv_bfloat16* __res
     const int split = blockIdx.x, n_splits = gridDim.x, ul = blockIdx.y;
     const int tid = threadIdx.x, lane = tid & 31, h = tid >> 5;
     const int gid = lane >> 2, tig = lane & 3, mat = lane >> 3, r8 = lane & 7;
-    const int n_rt = (n_ret + RT - 1) / RT, n_at = (n_apx + AT - 1) / AT, n_tiles = n_rt + n_at;
-    const int per = (n_tiles + n_splits - 1) / n_splits;
-    const int t_lo = min(n_tiles, split * per), t_hi = min(n_tiles, t_lo + per);
+    const int n_rt = (n_ret + RT - 1) / RT, n_at = (n_apx + AT - 1) / AT;
+    // A key-only tile takes 192 MMAs a warp, a retained one 64 (both bring in 64 KB): the slices are equal in time, not in tiles.
+    const long long weight = (long long)RET_COST * n_rt + (long long)APX_COST * n_at;
+    auto tile_at = [&](long long x) -> int {          // first tile that begins at or after x
+        return x <= (long long)RET_COST * n_rt ? (int)((x + RET_COST - 1) / RET_COST)
+                                               : n_rt + (int)((x - (long long)RET_COST * n_rt + APX_COST - 1) / APX_COST);
+    };
+    const int t_lo = tile_at(weight * split / n_splits), t_hi = tile_at(weight * (split + 1) / n_splits);
     const size_t u = (size_t)ul * HKV + h;
 
     for (int i = tid; i < 2 * MQ * PS_ROW / 4 + MQ; i += THREADS) reinterpret_cast<uint32_t*>(ps_hi)[i] = 0u;   // P and the factors
@@ -253,22 +262,29 @@ decode_layer_mma(const __nv_bfloat16* __restrict__ q, const __nv_bfloat16* __res
 // Merge for the same shapes: combines the splits' records of a unit, applies row block h of the layer's map
 // to the merged key sums of all heads and normalises,
 //   o_a = (sum_s f_s acc_v_s + W[h rows] sum_s f_s acc_k_s) / sum_s f_s l_s,   f_s = exp(m_s - max m).
-// grid (U), 256 threads.  The product runs on warp-level MMAs: M = the head's 128 output channels (warp w:
-// rows 16 w ..), N = the unit's g query heads (padded to 8), K = 8 x 128; A fragments straight from the map
-// (16-byte loads: thread (row r, quarter t) holds columns 8 (t + 4 jj) .. + 7 of rows r and r + 8 of a
+// grid (U), 512 threads.  The product runs on warp-level MMAs: M = the head's 128 output channels (warps w and w + 8:
+// rows 16 w .., each half of the input heads), N = the unit's g query heads (padded to 8), K = 8 x 128; A fragments straight
+// from the map (16-byte loads: thread (row r, quarter t) holds columns 8 (t + 4 jj) .. + 7 of rows r and r + 8 of a
 // 128-column block, the k slots of an MMA step follow that order in both operands), the key sums as bf16
-// hi + lo in shared memory.
+// hi + lo in shared memory.  What it costs is memory latency (42 MB of records and 64 MB of map from L2 over 256 blocks):
+// hence eight-byte loads with eight splits of two elements in flight, and 16 warps on the map's rows.
+constexpr int MERGE_THREADS = 512;
 template <typename TO>
-__global__ void __launch_bounds__(256)
+__global__ void __launch_bounds__(MERGE_THREADS)
 decode_layer_merge_mma(const float* __restrict__ partial, const __nv_bfloat16* __restrict__ W, int L, int g, int n_splits,
                        TO* __restrict__ out) {
     constexpr int KD = HKV * 128;
     __shared__ __align__(16) __nv_bfloat16 akh[8][KD], akl[8][KD];          // 32 KB
-    __shared__ float accv[8][128], pw[8][128], fs[8][32], Ls[8];
+    __shared__ float accv[8][128], pw[2][8][128], fs[8][32], Ls[8];
     const int u = blockIdx.x, tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
     const int h = u % HKV, layer = (u / HKV) % L;
     const int row = lane >> 2, quarter = lane & 3;
     const float* rec0 = partial + (size_t)u * n_splits * g * REC;
+    for (int i = tid; i < (8 - g) * KD; i += MERGE_THREADS) {            // columns of B beyond the unit's heads
+        akh[g + i / KD][i % KD] = __float2bfloat16_rn(0.f);
+        akl[g + i / KD][i % KD] = __float2bfloat16_rn(0.f);
+    }
+    asm volatile("griddepcontrol.wait;\n" ::: "memory");                 // the split kernel's records
     // factors of the splits: warp a < g takes head a
     if (wid < g) {
         const float mj = lane < n_splits ? rec0[((size_t)lane * g + wid) * REC] : -INFINITY;
@@ -279,40 +295,40 @@ decode_layer_merge_mma(const float* __restrict__ partial, const __nv_bfloat16* _
         const float Lsum = warp_sum(f * lj);
         if (lane == 0) Ls[wid] = Lsum;
     }
-    for (int i = tid; i < (8 - g) * KD; i += 256) {            // columns of B beyond the unit's heads
-        akh[g + i / KD][i % KD] = __float2bfloat16_rn(0.f);
-        akl[g + i / KD][i % KD] = __float2bfloat16_rn(0.f);
-    }
     __syncthreads();
-    // merged sums: element e of a record's 128 + 1024 values, coalesced over the threads; eight splits' loads
-    // in flight at a time
-    for (int a = 0; a < g; ++a) {
-        for (int e = tid; e < 128 + KD; e += 256) {
-            const float* src = rec0 + (size_t)a * REC + 2 + e;
-            float v = 0.f;
-            for (int s0 = 0; s0 < n_splits; s0 += 8) {
-                float x[8];
+    // merged sums: a thread has two neighbouring elements of a record's 128 + 1024 values
+    constexpr int PAIRS = (128 + KD) / 2;
+    for (int i = tid; i < g * PAIRS; i += MERGE_THREADS) {
+        const int a = i / PAIRS, e = (i - a * PAIRS) * 2;
+        const float* src = rec0 + (size_t)a * REC + 2 + e;
+        float v0 = 0.f, v1 = 0.f;
+        for (int s0 = 0; s0 < n_splits; s0 += 8) {
+            float2 x[8];
 #pragma unroll
-                for (int k = 0; k < 8; ++k) x[k] = src[(size_t)min(s0 + k, n_splits - 1) * g * REC];      // always a valid record
+            for (int k = 0; k < 8; ++k) x[k] = *reinterpret_cast<const float2*>(src + (size_t)min(s0 + k, n_splits - 1) * g * REC);   // always a valid record
 #pragma unroll
-                for (int k = 0; k < 8; ++k) v = fmaf(s0 + k < n_splits ? fs[a][s0 + k] : 0.f, x[k], v);
+            for (int k = 0; k < 8; ++k) {
+                const float f = s0 + k < n_splits ? fs[a][s0 + k] : 0.f;
+                v0 = fmaf(f, x[k].x, v0);
+                v1 = fmaf(f, x[k].y, v1);
             }
-            if (e < 128) accv[a][e] = v;
-            else {
-                const __nv_bfloat16 hi = __float2bfloat16_rn(v);
-                akh[a][e - 128] = hi;
-                akl[a][e - 128] = __float2bfloat16_rn(v - __bfloat162float(hi));
-            }
+        }
+        if (e < 128) { accv[a][e] = v0; accv[a][e + 1] = v1; }
+        else {
+            const uint32_t hi = dbf::pack_bf16(v0, v1);
+            *reinterpret_cast<uint32_t*>(&akh[a][e - 128]) = hi;
+            *reinterpret_cast<uint32_t*>(&akl[a][e - 128]) = dbf::pack_bf16(v0 - __uint_as_float(hi << 16), v1 - __uint_as_float(hi & 0xffff0000u));
         }
     }
     __syncthreads();
-    // rows 16 wid .. of the head's block of the map times the key sums
+    // rows 16 (wid % 8) .. of the head's block of the map times the key sums of four input heads
     {
-        const uint4* Wr0 = reinterpret_cast<const uint4*>(W + ((size_t)layer * KD + (size_t)h * 128 + 16 * wid + row) * KD);
+        const int half = wid >> 3, r0 = 16 * (wid & 7) + row;
+        const uint4* Wr0 = reinterpret_cast<const uint4*>(W + ((size_t)layer * KD + (size_t)h * 128 + r0) * KD);
         const uint4* Wr1 = Wr0 + 8 * (KD / 8);                 // row + 8
         float d[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll 2
-        for (int kc = 0; kc < HKV; ++kc) {                     // 128 columns a time: 16 pieces of 16 bytes per row
+        for (int kc = half * (HKV / 2); kc < (half + 1) * (HKV / 2); ++kc) {                     // 128 columns a time: 16 pieces of 16 bytes per row
             uint4 A[8];
 #pragma unroll
             for (int jj = 0; jj < 4; ++jj) {
@@ -321,24 +337,24 @@ decode_layer_merge_mma(const float* __restrict__ partial, const __nv_bfloat16* _
             }
 #pragma unroll
             for (int jj = 0; jj < 4; ++jj) {
-                const uint4 r0 = A[2 * jj], r1 = A[2 * jj + 1];
+                const uint4 a0 = A[2 * jj], a1 = A[2 * jj + 1];
                 const int col = kc * 128 + 8 * (quarter + 4 * jj);
                 const uint4 bh = *reinterpret_cast<const uint4*>(&akh[row][col]);      // B column = head `row`
                 const uint4 bl = *reinterpret_cast<const uint4*>(&akl[row][col]);
-                dbf::mma_16(d, r0.x, r1.x, r0.y, r1.y, bh.x, bh.y);
-                dbf::mma_16(d, r0.x, r1.x, r0.y, r1.y, bl.x, bl.y);
-                dbf::mma_16(d, r0.z, r1.z, r0.w, r1.w, bh.z, bh.w);
-                dbf::mma_16(d, r0.z, r1.z, r0.w, r1.w, bl.z, bl.w);
+                dbf::mma_16(d, a0.x, a1.x, a0.y, a1.y, bh.x, bh.y);
+                dbf::mma_16(d, a0.x, a1.x, a0.y, a1.y, bl.x, bl.y);
+                dbf::mma_16(d, a0.z, a1.z, a0.w, a1.w, bh.z, bh.w);
+                dbf::mma_16(d, a0.z, a1.z, a0.w, a1.w, bl.z, bl.w);
             }
         }
         // d[0], d[1]: row `row`, heads 2 quarter and 2 quarter + 1; d[2], d[3]: row `row` + 8
-        if (2 * quarter < g) { pw[2 * quarter][16 * wid + row] = d[0]; pw[2 * quarter][16 * wid + row + 8] = d[2]; }
-        if (2 * quarter + 1 < g) { pw[2 * quarter + 1][16 * wid + row] = d[1]; pw[2 * quarter + 1][16 * wid + row + 8] = d[3]; }
+        if (2 * quarter < g) { pw[half][2 * quarter][r0] = d[0]; pw[half][2 * quarter][r0 + 8] = d[2]; }
+        if (2 * quarter + 1 < g) { pw[half][2 * quarter + 1][r0] = d[1]; pw[half][2 * quarter + 1][r0 + 8] = d[3]; }
     }
     __syncthreads();
-    for (int i = tid; i < g * 128; i += 256) {
+    for (int i = tid; i < g * 128; i += MERGE_THREADS) {
         const int a = i >> 7, c = i & 127;
-        store_out(out + ((size_t)u * g + a) * 128 + c, (accv[a][c] + pw[a][c]) / Ls[a]);
+        store_out(out + ((size_t)u * g + a) * 128 + c, (accv[a][c] + (pw[0][a][c] + pw[1][a][c])) / Ls[a]);
     }
 }
 
