@@ -241,13 +241,13 @@ static vector_status launch_layer_mma(const Dims& dm, int L, const void* q, cons
     }
     const int UL = dm.U / dlm::HKV;
     const int64_t tiles = (ch->n_ret + dlm::RT - 1) / dlm::RT + (ch->n_apx + dlm::AT - 1) / dlm::AT;
-    // Splits: a multiprocessor holds one block, so the time goes with whole rounds of blocks over the splits' number (32
-    // layers: 9 splits are two rounds, 10 were three: 218 us against 150); a split also costs its records (about 3 % of a
-    // round each).
+    // Splits: a multiprocessor holds one block, so the time goes with whole rounds of blocks over the splits' number; a block
+    // costs about eight tiles besides: its first loads, its records (32 layers of 7200 rows: 215 us a step, 238 with none counted).
+    const double cost = dlm::RET_COST * (double)((ch->n_ret + dlm::RT - 1) / dlm::RT) + dlm::APX_COST * (double)((ch->n_apx + dlm::AT - 1) / dlm::AT);
     int64_t n_splits = 1;
-    double best = 1e30;
+    double best = 1e300;
     for (int64_t n = 1; n <= 32 && n <= tiles; ++n) {
-        const double t = (double)((n * UL + sm_count() - 1) / sm_count()) / (double)n * (1.0 + 0.03 * n / ((n * UL + sm_count() - 1) / sm_count()));
+        const double t = (double)((n * UL + sm_count() - 1) / sm_count()) * (cost / (double)n + 8.0);
         if (t < best - 1e-9) { best = t; n_splits = n; }
     }
     VEC_CUDA_CHECK(launch_maybe_dependent(true, dlm::decode_layer_mma, dim3((unsigned)n_splits, UL), dim3(dlm::THREADS), dlm::SMEM_BYTES, st,
