@@ -17,9 +17,10 @@
 // all stages but one behind the one being issued: 128 KB of row loads stay in flight.
 // With RoPE: the turned key is no longer a bf16 number, so it goes to the tensor cores as a bf16
 // pair hi + lo (two chains over the same W), which keeps it to 2^-17 relative; two stages of
-// K hi | K lo | V (96 KB each).  A loader thread turns its own eight channel pairs of each of its
-// rows back once its own copies of the previous tile have landed (no cross-thread hand-over),
-// writes hi in place and lo into the second operand tile.
+// K hi | K lo | V (96 KB each).  A loader thread takes its chunks of the keys straight into registers,
+// a pass of the next tile requested as soon as that pass of this tile has been read, turns its eight channel
+// pairs of each of its rows back and writes hi and lo; the values follow with cp.async and a barrier of
+// their own.  With the keys landing in the stage, a tile's loads waited for the epilogue of the tile before last.
 #ifndef VECTOR_RESIDUAL_TC_CUH_
 #define VECTOR_RESIDUAL_TC_CUH_
 
@@ -45,6 +46,11 @@ __device__ __forceinline__ void cp_async16(uint32_t dst, const void* src, uint32
 }
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
 template <int N> __device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group %0;\n" ::"n"(N) : "memory"); }
+__device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;\n" ::: "memory"); }
+// One arrival on `bar` when all cp.async of this thread so far have completed.
+__device__ __forceinline__ void cp_async_arrive(uint64_t* bar) {
+    asm volatile("cp.async.mbarrier.arrive.noinc.shared::cta.b64 [%0];\n" ::"r"(tma::smem_u32(bar)) : "memory");
+}
 __device__ __forceinline__ void fence_async_proxy() { asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory"); }
 
 __device__ __forceinline__ uint32_t pack2_bf16(float lo, float hi) {
@@ -78,6 +84,7 @@ template <int D, bool ROPE> struct RCfg {
 };
 struct RSync {
     uint64_t full[5], done[5], empty[5];
+    uint64_t v_full[2];              // RoPE: the stage's values have landed
     uint64_t w_full, w_empty;
     uint32_t tmem_base;
 };
@@ -114,6 +121,7 @@ residual_tc(const __nv_bfloat16* __restrict__ K, const __nv_bfloat16* __restrict
             tma::mbar_init(&sy.full[s], 32 * R_LOADER_WARPS);
             tma::mbar_init(&sy.done[s], 1);
             tma::mbar_init(&sy.empty[s], EPI_WARPS);
+            if (ROPE) tma::mbar_init(&sy.v_full[s], 32 * R_LOADER_WARPS);
         }
         tma::mbar_init(&sy.w_full, 1);
         tma::mbar_init(&sy.w_empty, 1);
@@ -137,25 +145,40 @@ residual_tc(const __nv_bfloat16* __restrict__ K, const __nv_bfloat16* __restrict
         uint2 fr[8];                                                 // phases of this thread's eight channel pairs
 #pragma unroll
         for (int e = 0; e < 8; ++e) fr[e] = reinterpret_cast<const uint2*>(phase_s)[qc * 8 + e];
-        int32_t prev[PASSES], cur[PASSES], nxt[PASSES];
+        int32_t cur[PASSES], nxt[PASSES];
         Cursor at = cursor_at(gt_lo, P.tpu), ahead = at;             // the tile at hand; the tile whose rows are fetched next
         auto fetch_idx = [&](int32_t (&out)[PASSES]) {
 #pragma unroll
             for (int p = 0; p < PASSES; ++p) {
                 const int row = ahead.t * TILE + p * RPP + rsub;
-                const int32_t v = row < P.n_idx ? idx[(size_t)ahead.u * P.n_idx + row] : -1;
-                out[p] = (unsigned long long)v < (unsigned long long)P.N ? v : -1;   // an index outside the unit reads as a row of zeros
+                out[p] = row < P.n_idx ? idx[(size_t)ahead.u * P.n_idx + row] : -1;
             }
             ahead.next(P.tpu);
         };
-        // Turns this thread's pairs of the tile in stage s (rows listed in pos) and publishes the tile.
-        auto turn_back = [&](int s, const int32_t (&pos)[PASSES]) {
+        // An index outside the unit reads as a row of zeros.  Checked when the rows come up, not when they are fetched: the
+        // check would wait for the fetch (2 900 of 7 000 cycles a tile with RoPE).
+        auto check_idx = [&](int32_t (&rows)[PASSES]) {
+#pragma unroll
+            for (int p = 0; p < PASSES; ++p) rows[p] = (unsigned long long)rows[p] < (unsigned long long)P.N ? rows[p] : -1;
+        };
+        // RoPE: this thread's key chunks of a tile: per pass, eight channels of the first half and their partners.
+        uint4 kx[PASSES], ky[PASSES];
+        auto request = [&](const __nv_bfloat16* Ku, int p, int32_t row) {
+            kx[p] = ky[p] = make_uint4(0u, 0u, 0u, 0u);                  // zero past the end of the list
+            if (row >= 0) {
+                const __nv_bfloat16* kr = Ku + (size_t)row * D;
+                kx[p] = __ldg(reinterpret_cast<const uint4*>(kr));
+                ky[p] = __ldg(reinterpret_cast<const uint4*>(kr + D / 2));
+            }
+        };
+        // Turns the pairs of tile i (rows listed in pos), writes them to stage s and publishes it; a pass's registers take
+        // the next tile's keys (rows listed in next_rows) as soon as they have been read.
+        auto turn_back = [&](int i, int s, const int32_t (&pos)[PASSES], const int32_t (&next_rows)[PASSES], const __nv_bfloat16* K_next) {
             const uint32_t hi0 = tma::smem_u32(stage0 + s * R_STAGE_BYTES) + dst_thread, lo0 = hi0 + OPERAND_BYTES;
 #pragma unroll
             for (int p = 0; p < PASSES; ++p) {
-                uint32_t xs[4], ys[4], xl[4], yl[4];
-                asm volatile("ld.shared.v4.u32 {%0,%1,%2,%3}, [%4];\n" : "=r"(xs[0]), "=r"(xs[1]), "=r"(xs[2]), "=r"(xs[3]) : "r"(hi0 + p * PASS_BYTES));
-                asm volatile("ld.shared.v4.u32 {%0,%1,%2,%3}, [%4];\n" : "=r"(ys[0]), "=r"(ys[1]), "=r"(ys[2]), "=r"(ys[3]) : "r"(hi0 + other + p * PASS_BYTES));
+                uint32_t xs[4] = {kx[p].x, kx[p].y, kx[p].z, kx[p].w}, ys[4] = {ky[p].x, ky[p].y, ky[p].z, ky[p].w}, xl[4], yl[4];
+                if (i + 1 < n_my) request(K_next, p, next_rows[p]);
                 const uint32_t tok = pos[p] >= 0 ? (uint32_t)pos[p] : 0u;      // rows past the list are zeros
 #pragma unroll
                 for (int e = 0; e < 4; ++e) {
@@ -188,53 +211,75 @@ residual_tc(const __nv_bfloat16* __restrict__ K, const __nv_bfloat16* __restrict
         bool ok = true;
         asm volatile("griddepcontrol.wait;\n" ::: "memory");      // idx is complete and visible from here on
         if (n_my > 0) fetch_idx(cur);
+        if constexpr (ROPE) {
+            if (n_my > 0) {
+                check_idx(cur);
 #pragma unroll
-        for (int p = 0; p < PASSES; ++p) prev[p] = -1;
-        for (int i = 0; i < n_my && ok; ++i) {
-            const int s = i % STAGES, round = i / STAGES;
-            if (i + 1 < n_my) fetch_idx(nxt);
-            if (round > 0 && !tma::mbar_wait(&sy.empty[s], (round - 1) & 1, fault, 46)) { ok = false; break; }
-            const uint32_t kdst = tma::smem_u32(stage0 + s * R_STAGE_BYTES) + dst_thread;
-            const uint32_t vdst = kdst + C::V_OFFSET;
-            const __nv_bfloat16* Ku = K + (size_t)at.u * P.N * D + qc * 8;
-            const __nv_bfloat16* Vu = V + (size_t)at.u * P.N * D + qc * 8;
-            at.next(P.tpu);
-#pragma unroll
-            for (int p = 0; p < PASSES; ++p) {
-                const bool valid = cur[p] >= 0;
-                const size_t ro = valid ? (size_t)cur[p] * D : 0;
-                const uint32_t nb = valid ? 16u : 0u;                  // zero fill past the end of the list
-                cp_async16(kdst + p * PASS_BYTES, Ku + ro, nb);
-                cp_async16(kdst + other + p * PASS_BYTES, Ku + ro + D / 2, nb);
-                cp_async16(vdst + p * PASS_BYTES, Vu + ro, nb);
-                cp_async16(vdst + other + p * PASS_BYTES, Vu + ro + D / 2, nb);
+                for (int p = 0; p < PASSES; ++p) request(K + (size_t)at.u * P.N * D + qc * 8, p, cur[p]);
             }
-            cp_async_commit();
-            if (ROPE) {
-                if (i > 0) {                             // this thread's copies of the previous tile have landed
-                    cp_async_wait<1>();
-                    turn_back((i - 1) % STAGES, prev);
+            if (n_my > 1) fetch_idx(nxt);
+            for (int i = 0; i < n_my && ok; ++i) {
+                const int s = i % STAGES, round = i / STAGES;
+                int32_t after[PASSES];
+                if (i + 2 < n_my) fetch_idx(after);
+                if (i + 1 < n_my) check_idx(nxt);
+                if (round > 0 && !tma::mbar_wait(&sy.empty[s], (round - 1) & 1, fault, 46)) { ok = false; break; }
+                const uint32_t vdst = tma::smem_u32(stage0 + s * R_STAGE_BYTES) + C::V_OFFSET + dst_thread;
+                const __nv_bfloat16* Vu = V + (size_t)at.u * P.N * D + qc * 8;
+#pragma unroll
+                for (int p = 0; p < PASSES; ++p) {
+                    const size_t ro = cur[p] >= 0 ? (size_t)cur[p] * D : 0;
+                    const uint32_t nb = cur[p] >= 0 ? 16u : 0u;
+                    cp_async16(vdst + p * PASS_BYTES, Vu + ro, nb);
+                    cp_async16(vdst + other + p * PASS_BYTES, Vu + ro + D / 2, nb);
                 }
-            } else if (i >= STAGES - 1) {                // ... of the tile STAGES - 1 before this one
-                cp_async_wait<STAGES - 1>();
-                fence_async_proxy();
-                tma::mbar_arrive(&sy.full[(i - (STAGES - 1)) % STAGES]);
-            }
+                cp_async_arrive(&sy.v_full[s]);          // arrives once this thread's copies have landed
+                at.next(P.tpu);
+                turn_back(i, s, cur, nxt, K + (size_t)at.u * P.N * D + qc * 8);
 #pragma unroll
-            for (int p = 0; p < PASSES; ++p) { prev[p] = cur[p]; cur[p] = nxt[p]; }
-        }
-        if (ROPE) {
-            cp_async_wait<0>();
-            if (ok && n_my > 0) turn_back((n_my - 1) % STAGES, prev);
-        } else if (ok) {
-            auto publish = [&](int behind) {             // tile n_my - 1 - behind, if there is one
-                if (n_my > behind) { fence_async_proxy(); tma::mbar_arrive(&sy.full[(n_my - 1 - behind) % STAGES]); }
-            };
-            if constexpr (STAGES == 5) { cp_async_wait<3>(); publish(3); cp_async_wait<2>(); publish(2); }
-            cp_async_wait<1>(); publish(1);
-            cp_async_wait<0>(); publish(0);
+                for (int p = 0; p < PASSES; ++p) { cur[p] = nxt[p]; nxt[p] = after[p]; }
+            }
+            cp_async_wait_all();
         } else {
-            cp_async_wait<0>();
+            for (int i = 0; i < n_my && ok; ++i) {
+                const int s = i % STAGES, round = i / STAGES;
+                if (i + 1 < n_my) fetch_idx(nxt);
+                check_idx(cur);
+                if (round > 0 && !tma::mbar_wait(&sy.empty[s], (round - 1) & 1, fault, 46)) { ok = false; break; }
+                const uint32_t kdst = tma::smem_u32(stage0 + s * R_STAGE_BYTES) + dst_thread;
+                const uint32_t vdst = kdst + C::V_OFFSET;
+                const __nv_bfloat16* Ku = K + (size_t)at.u * P.N * D + qc * 8;
+                const __nv_bfloat16* Vu = V + (size_t)at.u * P.N * D + qc * 8;
+                at.next(P.tpu);
+#pragma unroll
+                for (int p = 0; p < PASSES; ++p) {
+                    const bool valid = cur[p] >= 0;
+                    const size_t ro = valid ? (size_t)cur[p] * D : 0;
+                    const uint32_t nb = valid ? 16u : 0u;                  // zero fill past the end of the list
+                    cp_async16(kdst + p * PASS_BYTES, Ku + ro, nb);
+                    cp_async16(kdst + other + p * PASS_BYTES, Ku + ro + D / 2, nb);
+                    cp_async16(vdst + p * PASS_BYTES, Vu + ro, nb);
+                    cp_async16(vdst + other + p * PASS_BYTES, Vu + ro + D / 2, nb);
+                }
+                cp_async_commit();
+                if (i >= STAGES - 1) {                   // this thread's copies of the tile STAGES - 1 before this one have landed
+                    cp_async_wait<STAGES - 1>();
+                    fence_async_proxy();
+                    tma::mbar_arrive(&sy.full[(i - (STAGES - 1)) % STAGES]);
+                }
+#pragma unroll
+                for (int p = 0; p < PASSES; ++p) cur[p] = nxt[p];
+            }
+            if (ok) {
+                auto publish = [&](int behind) {             // tile n_my - 1 - behind, if there is one
+                    if (n_my > behind) { fence_async_proxy(); tma::mbar_arrive(&sy.full[(n_my - 1 - behind) % STAGES]); }
+                };
+                if constexpr (STAGES == 5) { cp_async_wait<3>(); publish(3); cp_async_wait<2>(); publish(2); }
+                cp_async_wait<1>(); publish(1);
+                cp_async_wait<0>(); publish(0);
+            } else {
+                cp_async_wait<0>();
+            }
         }
     } else if (warp == R_LOADER_WARPS) {
         // ------------------------------------------------------------------ W loads and MMA issue
@@ -292,7 +337,7 @@ residual_tc(const __nv_bfloat16* __restrict__ K, const __nv_bfloat16* __restrict
         for (int i = 0; i < n_my; ++i, at.next(P.tpu)) {
             const int s = i % STAGES, round = i / STAGES;
             // the value rows were written by the loaders: observe their barrier, then the MMA's
-            if (!tma::mbar_wait_warp(&sy.full[s], round & 1, fault, 50)) break;
+            if (!tma::mbar_wait_warp(ROPE ? &sy.v_full[s] : &sy.full[s], round & 1, fault, 50)) break;
             if (!tma::mbar_wait_warp(&sy.done[s], round & 1, fault, 51)) break;
             tc::fence_after_sync();
             const int u = at.u, t = at.t;
