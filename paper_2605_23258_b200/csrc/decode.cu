@@ -15,6 +15,7 @@
 #include "common.cuh"
 #include "decode_bf16.cuh"
 #include "decode_pertile_tc.cuh"
+#include "decode_rope.cuh"
 #include "internal.h"
 
 namespace vec {
@@ -271,15 +272,16 @@ int* kernel_fault_address() {
 // Blocks per unit of the one-launch (cluster) form, 0 = stream and merge.  A cluster lies within one GPC and every
 // block fills its multiprocessor, so the largest size is taken at which all U clusters are resident at once.  That may
 // use fewer multiprocessors than the streaming form (48 units would need clusters of three that fit), whose second
-// kernel and records in global memory cost as much as about six tiles of a block (three with RoPE at 128 channels, whose
-// tiles take longest): the form with the fewer tiles a block, that cost included, runs.  Measured, four query heads, us
-// per step in a graph, stream against cluster: 128 channels, 8 units of 2457 rows 12.6 / 8.9, of 20000 rows 25.6 / 21.9;
-// 48 units of 1200 rows 15.8 / 13.2, of 2457 rows 18.7 / 18.1, with RoPE 26.4 / 31.2 for the last; 64 channels with
-// RoPE, 16 units of 5000 rows 19.4 / 13.2.
+// kernel and records in global memory cost as much as some tiles of a block: twice as many of 64 channels, which are half
+// the size, and fewer with RoPE, whose tiles take longer.  The form with the fewer tiles a block, that cost included, runs.
+// Measured, four query heads, us per step in a graph, cluster against stream: 128 channels, 8 units of 2457 rows 9.2 / 12.4,
+// of 19660 rows 21.9 / 25.2; 48 units of 1200 rows 13.4 / 15.7, 2457 rows 18.3 / 18.7, 4800 rows 27.9 / 25.7, with RoPE 15.2 /
+// 18.0, 23.2 / 22.6, 38.6 / 33.5; 64 channels, 48 units of 4800 rows 16.1 / 18.8, with RoPE of 2457 rows 17.4 / 18.3, 4800 rows
+// 28.0 / 25.8.
 template <int D, bool ROPE>
 static int decode_cluster_size(const dbf::Plan& pl, int U) {
     using C = dbf::Cfg<D, ROPE>;
-    constexpr int MAXC = dbf::MAX_CLUSTER, EXTRA_TILES = ROPE && D == 128 ? 3 : 6;
+    constexpr int MAXC = dbf::MAX_CLUSTER, EXTRA_TILES = (ROPE ? 6 : 9) * 128 / D;
     static int resident[PerDeviceOnce::kMax][MAXC + 1] = {};      // clusters of each size the device holds at once
     static std::mutex mu;
     int dev = -1;
@@ -287,7 +289,7 @@ static int decode_cluster_size(const dbf::Plan& pl, int U) {
     std::lock_guard<std::mutex> lock(mu);
     int* r = resident[dev];
     if (r[0] == 0) {
-        auto kern = dbf::decode_stream_bf16<D, ROPE, true>;
+        auto kern = [] { if constexpr (ROPE) return dbf::decode_stream_rope<D, true>; else return dbf::decode_stream_bf16<D, true>; }();
         bool ok = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, C::CLUSTER_SMEM_BYTES) == cudaSuccess &&
                   cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess;
         for (int c = 2; ok && c <= MAXC; ++c) {
@@ -317,10 +319,10 @@ static vector_status launch_decode_bf16(const Dims& dm, const void* q, const vec
     using Rope = dbf::Cfg<D, true>;
     static PerDeviceOnce once;
     if (once.first()) {
-        cudaError_t e = cudaFuncSetAttribute(dbf::decode_stream_bf16<D, false, false>,
+        cudaError_t e = cudaFuncSetAttribute(dbf::decode_stream_bf16<D, false>,
                                              cudaFuncAttributeMaxDynamicSharedMemorySize, Plain::SMEM_BYTES);
         if (e == cudaSuccess)
-            e = cudaFuncSetAttribute(dbf::decode_stream_bf16<D, true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+            e = cudaFuncSetAttribute(dbf::decode_stream_rope<D, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                      Rope::SMEM_BYTES);
         if (D == 128 && e == cudaSuccess)
             e = cudaFuncSetAttribute(dpt::decode_stream_pertile_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, dpt::SMEM_BYTES);
@@ -364,12 +366,18 @@ static vector_status launch_decode_bf16(const Dims& dm, const void* q, const vec
         const T* Wq = (const T*)W;
         const int n_ret = (int)ch->n_ret, n_apx = (int)ch->n_apx, out_f32 = out_dtype == VECTOR_F32;
         const int csize = dm.rope ? decode_cluster_size<D, true>(pl, dm.U) : decode_cluster_size<D, false>(pl, dm.U);
-        auto kern = dm.rope ? (csize ? dbf::decode_stream_bf16<D, true, true> : dbf::decode_stream_bf16<D, true, false>)
-                            : (csize ? dbf::decode_stream_bf16<D, false, true> : dbf::decode_stream_bf16<D, false, false>);
-        const int threads = dm.rope ? Rope::THREADS : Plain::THREADS;
-        const size_t smem = csize ? (dm.rope ? Rope::CLUSTER_SMEM_BYTES : Plain::CLUSTER_SMEM_BYTES) : (dm.rope ? Rope::SMEM_BYTES : Plain::SMEM_BYTES);
-        VEC_CUDA_CHECK(launch_maybe_dependent(true, csize ? csize : 1, kern, dim3(csize ? csize * dm.U : pl.B), dim3(threads), smem, st, qp, maps, pl,
-                                              n_ret, n_apx, dm.g, dm.LH, c2, partial, fault, ch->apx_pos, (long long)ch->cap_apx, ph, Wq, out, out_f32));
+        const dim3 grid(csize ? csize * dm.U : pl.B);
+        const int cl = csize ? csize : 1;
+        if (dm.rope) {
+            auto kern = csize ? dbf::decode_stream_rope<D, true> : dbf::decode_stream_rope<D, false>;
+            VEC_CUDA_CHECK(launch_maybe_dependent(true, cl, kern, grid, dim3(Rope::THREADS), csize ? Rope::CLUSTER_SMEM_BYTES : Rope::SMEM_BYTES,
+                                                  st, qp, maps, pl, n_ret, n_apx, dm.g, dm.LH, c2, partial, fault, ch->apx_pos,
+                                                  (long long)ch->cap_apx, ph, Wq, out, out_f32));
+        } else {
+            auto kern = csize ? dbf::decode_stream_bf16<D, true> : dbf::decode_stream_bf16<D, false>;
+            VEC_CUDA_CHECK(launch_maybe_dependent(true, cl, kern, grid, dim3(Plain::THREADS), csize ? Plain::CLUSTER_SMEM_BYTES : Plain::SMEM_BYTES,
+                                                  st, qp, maps, pl, n_ret, n_apx, dm.g, dm.LH, c2, partial, fault, Wq, out, out_f32));
+        }
         if (csize) return VECTOR_OK;
     }
     // programmatic dependent launch: the merge blocks start while the streaming kernel drains

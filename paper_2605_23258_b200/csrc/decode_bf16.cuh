@@ -19,11 +19,6 @@
 //   O += P V  (retained tile)  or  A += P K  (key-only tile: the p-weighted key
 //             sum that the merge step multiplies by W); P enters as bf16 hi in
 //             MMA rows 0-7 and bf16 lo in rows 8-15, one MMA for both parts
-// RoPE decoupling (ROPE): the value of a key-only token is W applied to the key turned back by its
-// original position.  The logits use the stored keys; before the P K product the warp rotates its 64
-// keys in shared memory, channel c with c + D/2 by the angle -pos * theta^(-2c/D).  The angle is
-// taken exactly modulo one turn in 64-bit fixed point (pos * phase[c] wraps by itself), its sine and
-// cosine by the fast units.
 // A warp keeps one running state (m, l, O or A) per unit and writes it as its
 // partial record when it leaves the unit; a warp that met no tile of a unit the
 // block touches writes an empty record.  The merge kernel combines a unit's
@@ -33,6 +28,7 @@
 // blocks an equal share of the unit's tiles; the warps' records stay in shared memory, a block
 // combines its own, and after a cluster barrier block r merges the query heads r, r + C, ... out of
 // the other blocks' shared memory and applies W.  No records in global memory, no second kernel.
+// RoPE decoupling has a streaming kernel of its own (decode_rope.cuh) with the same tiles and records.
 #ifndef VECTOR_DECODE_BF16_CUH_
 #define VECTOR_DECODE_BF16_CUH_
 
@@ -47,27 +43,28 @@ namespace dbf {
 
 constexpr int KEYS = 64;                     // keys per softmax step (and per TMA box)
 constexpr int BOX_BYTES = 8192;              // 64 rows x 128 bytes
-// With RoPE decoupling the block carries helper warps that turn a tile's keys back for the warp
-// that owns the tile: a team is that warp plus four helpers (warps 4 + 4 team .. 7 + 4 team), one
-// per warp scheduler (scheduler = warp index modulo 4), since the sine / cosine unit is per scheduler.
-constexpr int ROPE_HELPERS = 4;
-constexpr int ROPE_TEAM_THREADS = 32 * (1 + ROPE_HELPERS);
+// With RoPE decoupling a team of warps works on a tile (decode_rope.cuh) and leaves one record.
+constexpr int ROPE_TEAMS = 3;
 template <int D, bool ROPE> struct Cfg {
     static constexpr int HALF_BYTES = 64 * 2 * D;                    // 64 rows as D / 64 swizzled boxes
     static constexpr int SLOT_BYTES = 2 * HALF_BYTES;                // retained: K | V; key-only: keys 0-63 | keys 64-127
     // With 64-channel heads a softmax step brings in half the bytes for the same softmax arithmetic: a fourth consumer
-    // warp (one to a warp scheduler) makes up for it.  The RoPE block keeps three (its helper warps fill it).
-    // Measured: 512 units, 1639 retained + 3276 key-only rows, 431 MB: 87 us with the appended row = 4.9 TB/s (856 us on
+    // warp (one to a warp scheduler) makes up for it.
+    // Measured: 512 units, 1639 retained + 3276 key-only rows, 431 MB: 82 us with the appended row = 5.3 TB/s (856 us on
     // CUDA cores).
-    static constexpr int CONSUMER_WARPS = D == 128 || ROPE ? 3 : 4;
+    static constexpr int CONSUMER_WARPS = ROPE ? ROPE_TEAMS : D == 128 ? 3 : 4;      // whose records a block leaves
     static constexpr int SLOTS = D == 128 ? 6 : 12;                  // a multiple of CONSUMER_WARPS: a slot always serves the same warp
-    static constexpr int THREADS = 32 * (CONSUMER_WARPS + 1 + (ROPE ? ROPE_HELPERS * CONSUMER_WARPS : 0));
-    static constexpr int SMEM_BYTES = SLOTS * SLOT_BYTES + 1024;     // + alignment slack; barriers live in static smem
+    static constexpr int THREADS = ROPE ? 512 : 32 * (CONSUMER_WARPS + 1);
+    static constexpr int STEP_BYTES = 2048 + 4 * KEYS + 32;          // RoPE: a step's weights, positions and factors
+    static constexpr int P_BYTES = ROPE ? ROPE_TEAMS * 2 * STEP_BYTES : 0;
+    static constexpr int SMEM_BYTES = SLOTS * SLOT_BYTES + P_BYTES + 1024;     // + alignment slack; barriers live in static smem
     static constexpr int REC = 4 + 2 * D;                            // m, l, value-scale, pad, acc_v[D], acc_k[D]
-    static constexpr int CLUSTER_SMEM_BYTES = SMEM_BYTES + CONSUMER_WARPS * 8 * REC * 4;      // + the warps' records
+    // CLUSTER: the warps' headers and value sums behind the slots, [CONSUMER_WARPS][g][4 + D]; a warp's key sums, [g][D], take
+    // the last of its own slots once it has worked through its tiles
+    static constexpr int CREC = 4 + D;
+    static constexpr int CLUSTER_SMEM_BYTES = SMEM_BYTES + CONSUMER_WARPS * 8 * CREC * 4;
     static_assert(CLUSTER_SMEM_BYTES + 1024 <= 227 * 1024, "shared memory of a block, barriers included");
     static_assert(SLOTS % CONSUMER_WARPS == 0, "a slot must always be consumed by the same warp");
-    static_assert(!ROPE || (CONSUMER_WARPS + 1 == 4 && ROPE_HELPERS == 4), "register hand-over is per warpgroup: owners + producer, then helpers");
 };
 constexpr int REC = Cfg<128, false>::REC;
 
@@ -140,80 +137,138 @@ __device__ __forceinline__ uint32_t pack_bf16(float lo, float hi) {
     return *reinterpret_cast<uint32_t*>(&v);
 }
 
-// RoPE decoupling: rows 16 member .. 16 member + 15 of the 64 keys at kbase (swizzled boxes of 64
-// channels) are turned back by their positions, in place, and left there as fp16 (a
-// turned key is not a bf16 number; eleven bits keep the key sum within the tolerance of the output,
-// eight do not; |k| beyond 65504 saturates).  Channel c pairs with
-// c + D/2; the angle is position * theta^(-2c/D), taken as the 32-bit product of the position and
-// the per-channel phase (turns per position as a fraction of 2^32), which is the angle modulo one turn.  pos16: lane l
-// holds the position of row 16 member + (l & 15).
-template <int D>
-__device__ __forceinline__ void derotate_rows(uint32_t kbase, int nrows, int member, uint32_t pos16,
-                                              const uint32_t* phase_s, int lane) {
-    constexpr int LPR = D / 16, RPP = 32 / LPR;                     // lanes a row, rows the warp takes at a time
-    const int qc = lane & (LPR - 1);                                // 16-byte chunk: channel pairs 8 qc .. 8 qc + 7
-    uint32_t phase[8];                                              // this lane's eight channel pairs
-#pragma unroll
-    for (int c = 0; c < 8; ++c) phase[c] = phase_s[qc * 8 + c];
-#pragma unroll 1
-    for (int j = 0; j < 16 / RPP; j += 2) {
-        // two rows per round, the loads of both ahead of the stores
-        uint32_t off[2], yoff[2], pos[2], xs[2][4], ys[2][4];
-        bool live[2];
-#pragma unroll
-        for (int u = 0; u < 2; ++u) {
-            const int rl = RPP * (j + u) + lane / LPR, r = 16 * member + rl;
-            pos[u] = __shfl_sync(0xffffffffu, pos16, rl);
-            live[u] = r < nrows;
-            off[u] = (uint32_t)r * 128u + (uint32_t)((qc ^ (r & 7)) << 4);
-            yoff[u] = D == 128 ? off[u] + BOX_BYTES : (uint32_t)r * 128u + (uint32_t)(((qc + LPR) ^ (r & 7)) << 4);   // the partner channels
-            if (live[u]) {
-                asm volatile("ld.shared.v4.u32 {%0,%1,%2,%3}, [%4];\n" : "=r"(xs[u][0]), "=r"(xs[u][1]), "=r"(xs[u][2]), "=r"(xs[u][3]) : "r"(kbase + off[u]));
-                asm volatile("ld.shared.v4.u32 {%0,%1,%2,%3}, [%4];\n" : "=r"(ys[u][0]), "=r"(ys[u][1]), "=r"(ys[u][2]), "=r"(ys[u][3]) : "r"(kbase + yoff[u]));
-            } else {
-#pragma unroll
-                for (int e = 0; e < 4; ++e) { xs[u][e] = 0u; ys[u][e] = 0u; }
-            }
-        }
-#pragma unroll
-        for (int u = 0; u < 2; ++u) {
-#pragma unroll
-            for (int e = 0; e < 4; ++e) {
-                float x[2], y[2], cs[2], sn[2], xo[2], yo[2];
-#pragma unroll
-                for (int h = 0; h < 2; ++h) {
-                    x[h] = __uint_as_float(h ? (xs[u][e] & 0xffff0000u) : (xs[u][e] << 16));
-                    y[h] = __uint_as_float(h ? (ys[u][e] & 0xffff0000u) : (ys[u][e] << 16));
-                    rope_phase32_cos_sin(pos[u], phase[2 * e + h], cs[h], sn[h]);
-                }
-                // both pairs of the word at once on the packed FMA path
-                const uint64_t x2 = tc::pack2(x[0], x[1]), y2 = tc::pack2(y[0], y[1]);
-                const uint64_t c2 = tc::pack2(cs[0], cs[1]), s2 = tc::pack2(sn[0], sn[1]);
-                tc::unpack2(tc::fma2(x2, c2, tc::mul2(y2, s2)), xo[0], xo[1]);
-                tc::unpack2(tc::fma2(y2, c2, tc::mul2(x2, tc::pack2(-sn[0], -sn[1]))), yo[0], yo[1]);
-                xs[u][e] = pack_f16(xo[0], xo[1]);
-                ys[u][e] = pack_f16(yo[0], yo[1]);
-            }
-        }
-#pragma unroll
-        for (int u = 0; u < 2; ++u) {
-            if (live[u]) {
-                asm volatile("st.shared.v4.u32 [%0], {%1,%2,%3,%4};\n" ::"r"(kbase + off[u]), "r"(xs[u][0]), "r"(xs[u][1]), "r"(xs[u][2]), "r"(xs[u][3]) : "memory");
-                asm volatile("st.shared.v4.u32 [%0], {%1,%2,%3,%4};\n" ::"r"(kbase + yoff[u]), "r"(ys[u][0]), "r"(ys[u][1]), "r"(ys[u][2]), "r"(ys[u][3]) : "memory");
-            }
-        }
-    }
-    // the slot is refilled by a bulk copy once released: order these stores ahead of it
-    asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
-}
-// All threads of team `team` (its owner warp and the helpers).
-__device__ __forceinline__ void team_sync(int team) {
-    asm volatile("bar.sync %0, %1;\n" ::"r"(2 + team), "n"(ROPE_TEAM_THREADS) : "memory");
-}
-
 struct Maps {
     CUtensorMap ret_k, ret_v, apx_k;     // rank 3: (D dims, pool rows, U units), box 64 x 64 x 1, 128B swizzle
 };
+
+// This block's share of the tile sequence: never empty, there are no more blocks than tiles in either form.
+template <bool CLUSTER>
+__device__ __forceinline__ void block_range(const Plan& pl, long long& lo, long long& hi) {
+    const int b = blockIdx.x;
+    if (CLUSTER) {
+        const int C = (int)cl::nctas(), r = (int)cl::rank(), u = b / C;
+        lo = (long long)u * pl.n_tiles + (long long)r * pl.n_tiles / C;
+        hi = (long long)u * pl.n_tiles + (long long)(r + 1) * pl.n_tiles / C;
+    } else {
+        lo = tile_begin(b, pl);
+        hi = tile_begin(b + 1, pl);
+    }
+}
+// The producer thread: the block's tiles in order, each into the next slot.
+template <int D, bool ROPE>
+__device__ __forceinline__ void produce(const Maps& maps, const Plan& pl, long long gt_lo, int n_my, unsigned char* smem,
+                                        uint64_t* full_bar, uint64_t* empty_bar, int* fault) {
+    using C = Cfg<D, ROPE>;
+    constexpr int BOXES = D / 64;
+    tma::prefetch_map(&maps.ret_k); tma::prefetch_map(&maps.ret_v); tma::prefetch_map(&maps.apx_k);
+    const uint64_t pol = tma::policy_evict_first();      // the cache is read once per step
+    int u = (int)(gt_lo / pl.n_tiles), t = (int)(gt_lo - (long long)u * pl.n_tiles);
+    for (int i = 0; i < n_my; ++i) {
+        const int s = i % C::SLOTS, round = i / C::SLOTS;
+        if (round > 0 && !tma::mbar_wait(&empty_bar[s], (round - 1) & 1, fault, 1)) break;
+        unsigned char* st = smem + s * C::SLOT_BYTES;
+        tma::mbar_expect_tx(&full_bar[s], C::SLOT_BYTES);
+        if (t < pl.n_rt) {
+            const int row0 = t * KEYS;
+#pragma unroll
+            for (int x = 0; x < BOXES; ++x) {
+                tma::load_3d_hint(st + x * BOX_BYTES, &maps.ret_k, 64 * x, row0, u, &full_bar[s], pol);
+                tma::load_3d_hint(st + C::HALF_BYTES + x * BOX_BYTES, &maps.ret_v, 64 * x, row0, u, &full_bar[s], pol);
+            }
+        } else {
+            const int row0 = (t - pl.n_rt) * 2 * KEYS;
+#pragma unroll
+            for (int x = 0; x < BOXES; ++x) {
+                tma::load_3d_hint(st + x * BOX_BYTES, &maps.apx_k, 64 * x, row0, u, &full_bar[s], pol);
+                tma::load_3d_hint(st + C::HALF_BYTES + x * BOX_BYTES, &maps.apx_k, 64 * x, row0 + KEYS, u, &full_bar[s], pol);
+            }
+        }
+        if (++t == pl.n_tiles) { t = 0; ++u; }
+    }
+}
+// The g query heads of a unit as A fragments, rows g .. 7 zero.
+template <int D>
+__device__ __forceinline__ void load_queries(const __nv_bfloat16* __restrict__ q, int unit, int g, int lane, uint32_t (&qa)[D / 16][2]) {
+    const int gid = lane >> 2, tig = lane & 3;
+    const uint32_t* qrow = reinterpret_cast<const uint32_t*>(q + ((size_t)unit * g + min(gid, g - 1)) * D);
+#pragma unroll
+    for (int ks = 0; ks < D / 16; ++ks) {
+        qa[ks][0] = gid < g ? qrow[ks * 8 + tig] : 0u;
+        qa[ks][1] = gid < g ? qrow[ks * 8 + 4 + tig] : 0u;
+    }
+}
+// The weights of a softmax step over the 64 keys at kbase (D / 64 swizzled boxes), of which nrows >= 1 are valid: sc (this
+// thread: head gid, keys 8 n + 2 tig, + 1) against the new running maximum m; l follows.  Returns the factor that what
+// was summed up before has to take.
+template <int D>
+__device__ __forceinline__ float score_step(uint32_t kbase, int nrows, float scale_log2e, const uint32_t (&qa)[D / 16][2], int lane,
+                                            float& m, float& l, float (&sc)[8][2]) {
+    // per-lane ldmatrix geometry (swizzle: 16-byte chunk index XOR (row & 7), rows are 128 bytes): matrices =
+    // (keys 0-7|8-15) x (chunk lo|hi)
+    const int tig = lane & 3, mat = lane >> 3, r8 = lane & 7;
+    const uint32_t qk_row = (uint32_t)(r8 + (mat >> 1) * 8) * 128u, qk_x = (uint32_t)(((mat & 1) ^ r8) << 4);
+    // ---- S = Q K^T: eight 8-key column tiles, each its own accumulator chain over the D / 16 k-steps
+    float zz[2];
+#pragma unroll
+    for (int n = 0; n < 8; ++n) { sc[n][0] = 0.f; sc[n][1] = 0.f; }
+#pragma unroll
+    for (int ks = 0; ks < D / 16; ++ks) {
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {          // 16 keys per ldmatrix
+            uint32_t b0, b1, b2, b3;
+            // k-step ks covers 16-byte chunks 2ks, 2ks+1 of the row: box ks/4, chunk (2ks)%8 (+1)
+            ldsm_x4(kbase + (ks >> 2) * BOX_BYTES + j * 16 * 128 + qk_row + ((((2 * ks) & 7) << 4) ^ qk_x), b0, b1, b2, b3);
+            mma_lo8(sc[2 * j][0], sc[2 * j][1], zz[0], zz[1], qa[ks][0], qa[ks][1], b0, b1);
+            mma_lo8(sc[2 * j + 1][0], sc[2 * j + 1][1], zz[0], zz[1], qa[ks][0], qa[ks][1], b2, b3);
+        }
+    }
+    // ---- online softmax over these 64 keys (row = head gid, shared by the 4 threads of a quad)
+    float mx = -INFINITY;
+#pragma unroll
+    for (int n = 0; n < 8; ++n) {
+        const int kc = n * 8 + 2 * tig;
+        sc[n][0] = kc < nrows ? sc[n][0] * scale_log2e : -INFINITY;
+        sc[n][1] = kc + 1 < nrows ? sc[n][1] * scale_log2e : -INFINITY;
+        mx = fmaxf(mx, fmaxf(sc[n][0], sc[n][1]));
+    }
+    mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 1));
+    mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 2));
+    const float m_new = fmaxf(m, mx);      // finite: key 0 of the step is valid for every row
+    const float alpha = exp2f(m - m_new);  // 0 on the first step
+    float ls = 0.f;
+#pragma unroll
+    for (int n = 0; n < 8; ++n) {
+        sc[n][0] = exp2f(sc[n][0] - m_new);
+        sc[n][1] = exp2f(sc[n][1] - m_new);
+        ls += sc[n][0] + sc[n][1];
+    }
+    l = l * alpha + ls;
+    m = m_new;
+    return alpha;
+}
+// The weights of keys 16 kk .. + 15 as an A fragment: hi in MMA rows 0-7, lo in rows 8-15.
+__device__ __forceinline__ void weights_bf16(const float (&sc)[8][2], int kk, uint32_t (&a)[4]) {
+    const float p00 = sc[2 * kk][0], p01 = sc[2 * kk][1], p10 = sc[2 * kk + 1][0], p11 = sc[2 * kk + 1][1];
+    const __nv_bfloat16 h00 = __float2bfloat16_rn(p00), h01 = __float2bfloat16_rn(p01);
+    const __nv_bfloat16 h10 = __float2bfloat16_rn(p10), h11 = __float2bfloat16_rn(p11);
+    a[0] = pack_bf16(__bfloat162float(h00), __bfloat162float(h01));
+    a[1] = pack_bf16(p00 - __bfloat162float(h00), p01 - __bfloat162float(h01));
+    a[2] = pack_bf16(__bfloat162float(h10), __bfloat162float(h11));
+    a[3] = pack_bf16(p10 - __bfloat162float(h10), p11 - __bfloat162float(h11));
+}
+// acc += P x over rows 16 kk .. + 15 of the 64 rows at vbase: D / 8 column tiles of 8 dims.
+template <int D>
+__device__ __forceinline__ void accumulate_step(uint32_t vbase, int kk, const uint32_t (&a)[4], float (&acc)[D / 8][4], int lane) {
+    const int mat = lane >> 3, r8 = lane & 7;             // matrices = (chunk lo|hi) x (rows 0-7|8-15)
+    const uint32_t pv_row = (uint32_t)(r8 + (mat & 1) * 8) * 128u, pv_x = (uint32_t)(((mat >> 1) ^ r8) << 4);
+#pragma unroll
+    for (int np = 0; np < D / 16; ++np) {
+        uint32_t b0, b1, b2, b3;
+        ldsm_x4_t(vbase + (np >> 2) * BOX_BYTES + kk * 16 * 128 + pv_row + ((((2 * np) & 7) << 4) ^ pv_x), b0, b1, b2, b3);
+        mma_16(acc[2 * np], a[0], a[1], a[2], a[3], b0, b1);
+        mma_16(acc[2 * np + 1], a[0], a[1], a[2], a[3], b2, b3);
+    }
+}
 
 // Rows 16 mt .. + 15 of W times the key sums of n heads: pw[head][row].  One warp, M = 16 output channels, N = the heads
 // (padded to 8), K = D: the A fragments are read straight from the map in global memory, 16 bytes a load -- thread
@@ -251,8 +306,9 @@ __device__ __forceinline__ void map_rows(const __nv_bfloat16* __restrict__ W, in
 
 // The last part of the CLUSTER form: combines the records of a unit, which its cluster's blocks hold in shared
 // memory, applies W and writes out.  Every warp of every block of the cluster calls it, converged; the warps come from
-// different roles, so the block-wide barrier is the numbered one below.  recs: this block's [CONSUMER_WARPS][g][REC];
-// room: for a MergeShared (the slots, which nobody reads any more).
+// different roles, so the block-wide barrier is the numbered one below.  recs: this block's [CONSUMER_WARPS][g][CREC] (header:
+// m, l, value-scale, whether there are key sums); room: the slots, which nobody reads any more -- a MergeShared at their
+// start, the warps' key sums in their last CONSUMER_WARPS.
 template <int NT> __device__ __forceinline__ void merge_sync() { asm volatile("bar.sync 1, %0;\n" ::"n"(NT) : "memory"); }
 
 constexpr int MAX_CLUSTER = 16;
@@ -266,7 +322,8 @@ template <int D, bool ROPE>
 __device__ __forceinline__ void cluster_merge(const float* recs, unsigned char* room, const __nv_bfloat16* __restrict__ Wu, int g,
                                               void* __restrict__ out_u, bool out_f32) {
     using C = Cfg<D, ROPE>;
-    constexpr int REC = C::REC, CW = C::CONSUMER_WARPS, NT = C::THREADS, V4 = 2 * D / 4;
+    constexpr int REC = C::REC, CREC = C::CREC, CW = C::CONSUMER_WARPS, NT = C::THREADS, V4 = 2 * D / 4;
+    static_assert(sizeof(MergeShared<D>) <= (C::SLOTS - CW) * C::SLOT_BYTES, "the key sums lie behind it");
     MergeShared<D>& S = *reinterpret_cast<MergeShared<D>*>(room);
     auto& comb = S.comb; auto& fac = S.fac; auto& Ls = S.Ls; auto& akh = S.akh; auto& akl = S.akl; auto& avs = S.avs; auto& pw = S.pw;
     const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
@@ -277,15 +334,18 @@ __device__ __forceinline__ void cluster_merge(const float* recs, unsigned char* 
         float m[CW], M = -INFINITY, L = 0.f;
         float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
-        for (int w = 0; w < CW; ++w) { m[w] = recs[(w * g + a) * REC]; M = fmaxf(M, m[w]); }
+        for (int w = 0; w < CW; ++w) { m[w] = recs[(w * g + a) * CREC]; M = fmaxf(M, m[w]); }
 #pragma unroll
         for (int w = 0; w < CW; ++w) {
             if (m[w] == -INFINITY) continue;                          // a warp without tiles: its sums are not written
-            const float* r = recs + (w * g + a) * REC;
+            const float* r = recs + (w * g + a) * CREC;
             float f = __expf(m[w] - M);
             L = fmaf(f, r[1], L);
+            const float* src = r + 4 + 4 * c4;
             if (c4 < D / 4) f *= r[2];                                // the values were parked at another reference
-            const float4 x = *reinterpret_cast<const float4*>(r + 4 + 4 * c4);
+            else if (r[3] == 0.f) continue;                           // no key-only tile
+            else src = reinterpret_cast<const float*>(room + (C::SLOTS - CW + w) * C::SLOT_BYTES) + a * D + 4 * (c4 - D / 4);
+            const float4 x = *reinterpret_cast<const float4*>(src);
             acc.x = fmaf(f, x.x, acc.x); acc.y = fmaf(f, x.y, acc.y); acc.z = fmaf(f, x.z, acc.z); acc.w = fmaf(f, x.w, acc.w);
         }
         if (c4 == 0) { comb[a * REC] = M; comb[a * REC + 1] = L; }
@@ -359,36 +419,25 @@ __device__ __forceinline__ void cluster_merge(const float* recs, unsigned char* 
 // dynamic shared memory.
 // partial: [U][s_max][CONSUMER_WARPS][g][REC]; slot of (unit u, block b) = b - block_of_tile(first tile of u).
 // CLUSTER writes out itself and does not use partial.
-template <int D, bool ROPE, bool CLUSTER>
-__global__ void __launch_bounds__(Cfg<D, ROPE>::THREADS, 1)
+template <int D, bool CLUSTER>
+__global__ void __launch_bounds__(Cfg<D, false>::THREADS, 1)
 decode_stream_bf16(const __nv_bfloat16* __restrict__ q, const __grid_constant__ Maps maps, Plan pl, int n_ret,
                         int n_apx, int g, int LH, float scale_log2e, float* __restrict__ partial,
-                        int* __restrict__ fault, const int32_t* __restrict__ apx_pos, long long cap_apx,
-                        const __grid_constant__ RopePhases rope, const __nv_bfloat16* __restrict__ W, void* __restrict__ out,
-                        int out_f32) {
-    constexpr int HALF_BYTES = Cfg<D, ROPE>::HALF_BYTES, SLOT_BYTES = Cfg<D, ROPE>::SLOT_BYTES, SLOTS = Cfg<D, ROPE>::SLOTS;
-    constexpr int CONSUMER_WARPS = Cfg<D, ROPE>::CONSUMER_WARPS, REC = Cfg<D, ROPE>::REC, BOXES = D / 64;
+                        int* __restrict__ fault, const __nv_bfloat16* __restrict__ W, void* __restrict__ out, int out_f32) {
+    using C = Cfg<D, false>;
+    constexpr int HALF_BYTES = C::HALF_BYTES, SLOT_BYTES = C::SLOT_BYTES, SLOTS = C::SLOTS;
+    constexpr int CONSUMER_WARPS = C::CONSUMER_WARPS, REC = C::REC, CREC = C::CREC;
     extern __shared__ unsigned char smem_raw[];
-    __shared__ uint32_t phase_s[ROPE ? 64 : 1];          // the phases rounded to 32 bits
-    if (ROPE && threadIdx.x < 64) phase_s[threadIdx.x] = (uint32_t)((rope.phase[threadIdx.x] + 0x80000000ull) >> 32);
-    __shared__ volatile int team_ok[CONSUMER_WARPS];     // RoPE: the owner's go / no-go for the tile at hand
     __shared__ __align__(8) uint64_t full_bar[SLOTS];
     __shared__ __align__(8) uint64_t empty_bar[SLOTS];
     // 128B-swizzled TMA boxes want 1024-byte aligned destinations
     unsigned char* smem = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
     const int b = blockIdx.x;
     const int tid = threadIdx.x, lane = tid & 31, wq = tid >> 5;
-    long long gt_lo, gt_hi;                              // never empty: no more blocks than tiles in either form
-    if (CLUSTER) {
-        const int C = (int)cl::nctas(), r = (int)cl::rank(), u = b / C;
-        gt_lo = (long long)u * pl.n_tiles + (long long)r * pl.n_tiles / C;
-        gt_hi = (long long)u * pl.n_tiles + (long long)(r + 1) * pl.n_tiles / C;
-    } else {
-        gt_lo = tile_begin(b, pl);
-        gt_hi = tile_begin(b + 1, pl);
-    }
+    long long gt_lo, gt_hi;
+    block_range<CLUSTER>(pl, gt_lo, gt_hi);
     const int n_my = (int)(gt_hi - gt_lo);
-    const int u0 = (int)(gt_lo / pl.n_tiles), t0 = (int)(gt_lo - (long long)u0 * pl.n_tiles);
+    const int u0 = (int)(gt_lo / pl.n_tiles);
     const int u_last = (int)((gt_hi - 1) / pl.n_tiles);
     float* const recs = reinterpret_cast<float*>(smem + SLOTS * SLOT_BYTES);      // CLUSTER: the warps' records
 
@@ -406,81 +455,18 @@ decode_stream_bf16(const __nv_bfloat16* __restrict__ q, const __grid_constant__ 
     const __nv_bfloat16* const Wu = W + (size_t)(u0 % LH) * D * D;
     if (CLUSTER) {                                                    // the map's way into L2, for the blocks that will apply it
         const char* Wb = reinterpret_cast<const char*>(Wu);
-        for (int e = tid; e < 2 * D * D / 128; e += Cfg<D, ROPE>::THREADS) asm volatile("prefetch.global.L2 [%0];\n" ::"l"(Wb + 128 * e));
+        for (int e = tid; e < 2 * D * D / 128; e += C::THREADS) asm volatile("prefetch.global.L2 [%0];\n" ::"l"(Wb + 128 * e));
         __syncwarp();
     }
     auto merge_unit = [&]() {                                         // CLUSTER: each role's last act
         if (CLUSTER)
-            cluster_merge<D, ROPE>(recs, smem, Wu, g,
+            cluster_merge<D, false>(recs, smem, Wu, g,
                                    reinterpret_cast<char*>(out) + (size_t)u0 * g * D * (out_f32 ? 4 : 2), out_f32 != 0);
     };
 
-    if (ROPE && wq > CONSUMER_WARPS) {
-        // ------------------------------------------------------------------ helpers (RoPE only)
-        // A helper walks its owner's key-only tiles and turns back its quarter of each 64 keys
-        // between the owner's two team barriers.  It waits on nothing but those barriers, which the
-        // owner reaches for every key-only tile whether or not its own (bounded) waits succeeded.
-        // The block is compiled for 128 registers a thread (512 threads): the three helper
-        // warpgroups hand registers over to the first one (the three owners and the producer).
-        asm volatile("setmaxnreg.dec.sync.aligned.u32 96;\n");
-        const int team = (wq - CONSUMER_WARPS - 1) / ROPE_HELPERS, member = (wq - CONSUMER_WARPS - 1) % ROPE_HELPERS;
-        int i = team;
-        for (int u = u0; u <= u_last; ++u) {
-            const long long unit_end = (long long)(u + 1) * pl.n_tiles - gt_lo;
-            for (; i < n_my && i < unit_end; i += CONSUMER_WARPS) {
-                const int t = (int)(gt_lo + i - (long long)u * pl.n_tiles);
-                if (t < pl.n_rt) continue;
-                const int r0 = (t - pl.n_rt) * 2 * KEYS;
-                const int32_t* pr = apx_pos + (size_t)u * cap_apx + r0 + 16 * member + (lane & 15);
-                const int n0 = min(KEYS, n_apx - r0), n1 = min(KEYS, n_apx - r0 - KEYS);      // n1 <= 0: no second half
-                const uint32_t p0 = 16 * member + (lane & 15) < n0 ? (uint32_t)__ldg(pr) : 0u;
-                const uint32_t p1 = 16 * member + (lane & 15) < n1 ? (uint32_t)__ldg(pr + KEYS) : 0u;
-                team_sync(team);                                   // the owner has published its verdict
-                if (!team_ok[team]) continue;
-                const uint32_t base = tma::smem_u32(smem + (i % SLOTS) * SLOT_BYTES);
-                team_sync(team);                                   // the owner has its scores of half 0
-                derotate_rows<D>(base, n0, member, p0, phase_s, lane);
-                team_sync(team);                                   // ... and of half 1, if there is one
-                if (n1 > 0) {
-                    derotate_rows<D>(base + HALF_BYTES, n1, member, p1, phase_s, lane);
-                    team_sync(team);
-                }
-            }
-        }
-        merge_unit();
-        return;
-    }
-
-    if (ROPE) asm volatile("setmaxnreg.inc.sync.aligned.u32 216;\n");
     if (wq == CONSUMER_WARPS) {
         // ------------------------------------------------------------------ producer
-        if (lane == 0) {
-            tma::prefetch_map(&maps.ret_k); tma::prefetch_map(&maps.ret_v); tma::prefetch_map(&maps.apx_k);
-            const uint64_t pol = tma::policy_evict_first();      // the cache is read once per step
-            int u = u0, t = t0;
-            for (int i = 0; i < n_my; ++i) {
-                const int s = i % SLOTS, round = i / SLOTS;
-                if (round > 0 && !tma::mbar_wait(&empty_bar[s], (round - 1) & 1, fault, 1)) break;
-                unsigned char* st = smem + s * SLOT_BYTES;
-                tma::mbar_expect_tx(&full_bar[s], SLOT_BYTES);
-                if (t < pl.n_rt) {
-                    const int row0 = t * KEYS;
-#pragma unroll
-                    for (int x = 0; x < BOXES; ++x) {
-                        tma::load_3d_hint(st + x * BOX_BYTES, &maps.ret_k, 64 * x, row0, u, &full_bar[s], pol);
-                        tma::load_3d_hint(st + HALF_BYTES + x * BOX_BYTES, &maps.ret_v, 64 * x, row0, u, &full_bar[s], pol);
-                    }
-                } else {
-                    const int row0 = (t - pl.n_rt) * 2 * KEYS;
-#pragma unroll
-                    for (int x = 0; x < BOXES; ++x) {
-                        tma::load_3d_hint(st + x * BOX_BYTES, &maps.apx_k, 64 * x, row0, u, &full_bar[s], pol);
-                        tma::load_3d_hint(st + HALF_BYTES + x * BOX_BYTES, &maps.apx_k, 64 * x, row0 + KEYS, u, &full_bar[s], pol);
-                    }
-                }
-                if (++t == pl.n_tiles) { t = 0; ++u; }
-            }
-        }
+        if (lane == 0) produce<D, false>(maps, pl, gt_lo, n_my, smem, full_bar, empty_bar, fault);
         // the consumers wait on every tile's full barrier, so no copy outlives the block
         __syncwarp();
         merge_unit();
@@ -488,31 +474,16 @@ decode_stream_bf16(const __nv_bfloat16* __restrict__ q, const __grid_constant__ 
     }
     // ---------------------------------------------------------------------- consumers
     const int gid = lane >> 2, tig = lane & 3;
-    // per-lane ldmatrix geometry (swizzle: 16-byte chunk index XOR (row & 7), rows are 128 bytes)
-    const int mat = lane >> 3, r8 = lane & 7;
-    const uint32_t qk_row = (uint32_t)(r8 + (mat >> 1) * 8) * 128u;      // QK: matrices = (keys 0-7|8-15) x (chunk lo|hi)
-    const uint32_t qk_x = (uint32_t)(((mat & 1) ^ r8) << 4);
-    const uint32_t pv_row = (uint32_t)(r8 + (mat & 1) * 8) * 128u;       // PV: matrices = (chunk lo|hi) x (keys 0-7|8-15)
-    const uint32_t pv_x = (uint32_t)(((mat >> 1) ^ r8) << 4);
-
     uint32_t qa[D / 16][2];
     float acc[D / 8][4];                  // [dim tile][c0,c1: P_hi rows | c2,c3: P_lo rows]
     float m = -INFINITY, l = 0.f, stash_scale = 1.f;
     bool stashed = false;
 
     auto record_of = [&](int unit) -> float* {
-        if (CLUSTER) return recs + (wq * g + gid) * REC;
+        if (CLUSTER) return recs + (wq * g + gid) * CREC;
         int slot = b - block_of_tile((long long)unit * pl.n_tiles, pl);
         if (slot < 0 || slot >= pl.s_max) { atomicCAS(fault, 0, 5); slot = 0; }     // cannot happen; never write out of bounds
         return partial + ((((size_t)unit * pl.s_max + slot) * CONSUMER_WARPS + wq) * g + gid) * REC;
-    };
-    auto load_q = [&](int unit) {
-        const uint32_t* qrow = reinterpret_cast<const uint32_t*>(q + ((size_t)unit * g + min(gid, g - 1)) * D);
-#pragma unroll
-        for (int ks = 0; ks < D / 16; ++ks) {
-            qa[ks][0] = gid < g ? qrow[ks * 8 + tig] : 0u;
-            qa[ks][1] = gid < g ? qrow[ks * 8 + 4 + tig] : 0u;
-        }
     };
     auto store_acc = [&](float* dst) {       // dims n*8 + 2 tig + {0,1} of head row gid
 #pragma unroll
@@ -530,132 +501,50 @@ decode_stream_bf16(const __nv_bfloat16* __restrict__ q, const __grid_constant__ 
         lt += __shfl_xor_sync(0xffffffffu, lt, 2);
         if (gid < g) {
             float* rec = record_of(unit);
-            if (tig == 0) *reinterpret_cast<float4*>(rec) = make_float4(m * 0.69314718055994531f, lt, stashed ? stash_scale : 1.f, 0.f);
-            if (stashed) store_acc(rec + 4 + D);      // value part was written at the pool switch
-            else if (!CLUSTER || m > -INFINITY) {     // (the cluster's merge looks no further than an empty record's header)
+            if (tig == 0) *reinterpret_cast<float4*>(rec) = make_float4(m * 0.69314718055994531f, lt, stashed ? stash_scale : 1.f, stashed ? 1.f : 0.f);
+            if (stashed) {                            // value part was written at the pool switch
+                store_acc(CLUSTER ? reinterpret_cast<float*>(smem + (SLOTS - CONSUMER_WARPS + wq) * SLOT_BYTES) + gid * D : rec + 4 + D);
+            } else if (!CLUSTER) {
                 store_acc(rec + 4);
 #pragma unroll
                 for (int n = 0; n < D / 8; ++n) *reinterpret_cast<float2*>(rec + 4 + D + n * 8 + 2 * tig) = make_float2(0.f, 0.f);
+            } else if (m > -INFINITY) {               // (the cluster's merge looks no further than the header says)
+                store_acc(rec + 4);
             }
         }
         zero_acc();
         m = -INFINITY; l = 0.f; stash_scale = 1.f; stashed = false;
     };
-    // One softmax step over the 64 keys at kbase (D / 64 swizzled boxes), in two parts.  The first
-    // leaves the step's weights p in sc (this thread: head gid, keys 8 n + 2 tig, + 1), brings m, l
-    // and the accumulators to the new running maximum and returns the factor it applied to them.
-    auto scores64 = [&](uint32_t kbase, int nrows, bool retained, int unit, float (&sc)[8][2]) -> float {
-        // ---- S = Q K^T: eight 8-key column tiles, each its own accumulator chain over the D / 16 k-steps
-        float zz[2];
-#pragma unroll
-        for (int n = 0; n < 8; ++n) { sc[n][0] = 0.f; sc[n][1] = 0.f; }
-#pragma unroll
-        for (int ks = 0; ks < D / 16; ++ks) {
-#pragma unroll
-            for (int j = 0; j < 4; ++j) {          // 16 keys per ldmatrix
-                uint32_t b0, b1, b2, b3;
-                // k-step ks covers 16-byte chunks 2ks, 2ks+1 of the 256-byte row: box ks/4, chunk (2ks)%8 (+1)
-                ldsm_x4(kbase + (ks >> 2) * BOX_BYTES + j * 16 * 128 + qk_row + ((((2 * ks) & 7) << 4) ^ qk_x), b0, b1, b2, b3);
-                mma_lo8(sc[2 * j][0], sc[2 * j][1], zz[0], zz[1], qa[ks][0], qa[ks][1], b0, b1);
-                mma_lo8(sc[2 * j + 1][0], sc[2 * j + 1][1], zz[0], zz[1], qa[ks][0], qa[ks][1], b2, b3);
-            }
-        }
-        // ---- online softmax over these 64 keys (row = head gid, shared by the 4 threads of a quad)
-        float mx = -INFINITY;
-#pragma unroll
-        for (int n = 0; n < 8; ++n) {
-            const int kc = n * 8 + 2 * tig;
-            sc[n][0] = kc < nrows ? sc[n][0] * scale_log2e : -INFINITY;
-            sc[n][1] = kc + 1 < nrows ? sc[n][1] * scale_log2e : -INFINITY;
-            mx = fmaxf(mx, fmaxf(sc[n][0], sc[n][1]));
-        }
-        mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 1));
-        mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 2));
+    // One softmax step over the 64 keys at kbase, in two parts.  The first leaves the step's weights p in sc (this thread:
+    // head gid, keys 8 n + 2 tig, + 1) and brings m, l and the accumulators to the new running maximum.
+    auto scores64 = [&](uint32_t kbase, int nrows, bool retained, int unit, float (&sc)[8][2]) {
+        const float alpha = score_step<D>(kbase, nrows, scale_log2e, qa, lane, m, l, sc);
         if (!retained && !stashed) {           // first key-only keys of this unit for this warp: park sum p v
             if (gid < g) store_acc(record_of(unit) + 4);
             zero_acc();
             stashed = true;
             stash_scale = 1.f;
         }
-        const float m_new = fmaxf(m, mx);      // finite: key 0 of the step is valid for every row
-        const float alpha = exp2f(m - m_new);  // 0 on the first step
-        float ls = 0.f;
-#pragma unroll
-        for (int n = 0; n < 8; ++n) {
-            sc[n][0] = exp2f(sc[n][0] - m_new);
-            sc[n][1] = exp2f(sc[n][1] - m_new);
-            ls += sc[n][0] + sc[n][1];
-        }
-        l = l * alpha + ls;
-        m = m_new;
         stash_scale *= alpha;
         if (__any_sync(0xffffffffu, alpha != 1.f)) {
-            {
 #pragma unroll
-                for (int n = 0; n < D / 8; ++n) { acc[n][0] *= alpha; acc[n][1] *= alpha; acc[n][2] *= alpha; acc[n][3] *= alpha; }
-            }
+            for (int n = 0; n < D / 8; ++n) { acc[n][0] *= alpha; acc[n][1] *= alpha; acc[n][2] *= alpha; acc[n][3] *= alpha; }
         }
-        return alpha;
     };
     // The second part adds p x (the 64 rows at vbase: values, or the keys themselves for a key-only tile).
-    auto accumulate64 = [&](uint32_t vbase, bool retained, float (&sc)[8][2]) {
-        // ---- accumulate P x (V rows | K rows): four k-steps of 16 keys x D / 8 column tiles of 8 dims
+    auto accumulate64 = [&](uint32_t vbase, float (&sc)[8][2]) {
 #pragma unroll
         for (int kk = 0; kk < 4; ++kk) {
-            // P as bf16 hi (MMA rows 0-7) + lo (rows 8-15)
-            const float p00 = sc[2 * kk][0], p01 = sc[2 * kk][1], p10 = sc[2 * kk + 1][0], p11 = sc[2 * kk + 1][1];
-            if (ROPE && !retained) {
-                // the turned keys are fp16: so are the weights, again as hi + lo
-                const uint32_t a0 = pack_f16(p00, p01), a2 = pack_f16(p10, p11);
-                const uint32_t a1 = pack_f16(p00 - f16_lo(a0), p01 - f16_hi(a0)), a3 = pack_f16(p10 - f16_lo(a2), p11 - f16_hi(a2));
-#pragma unroll
-                for (int np = 0; np < D / 16; ++np) {
-                    uint32_t b0, b1, b2, b3;
-                    ldsm_x4_t(vbase + (np >> 2) * BOX_BYTES + kk * 16 * 128 + pv_row + ((((2 * np) & 7) << 4) ^ pv_x), b0, b1, b2, b3);
-                    mma_16_f16(acc[2 * np], a0, a1, a2, a3, b0, b1);
-                    mma_16_f16(acc[2 * np + 1], a0, a1, a2, a3, b2, b3);
-                }
-                continue;
-            }
-            const __nv_bfloat16 h00 = __float2bfloat16_rn(p00), h01 = __float2bfloat16_rn(p01);
-            const __nv_bfloat16 h10 = __float2bfloat16_rn(p10), h11 = __float2bfloat16_rn(p11);
-            const uint32_t a0 = pack_bf16(__bfloat162float(h00), __bfloat162float(h01));
-            const uint32_t a2 = pack_bf16(__bfloat162float(h10), __bfloat162float(h11));
-            const uint32_t a1 = pack_bf16(p00 - __bfloat162float(h00), p01 - __bfloat162float(h01));
-            const uint32_t a3 = pack_bf16(p10 - __bfloat162float(h10), p11 - __bfloat162float(h11));
-#pragma unroll
-            for (int np = 0; np < D / 16; ++np) {
-                uint32_t b0, b1, b2, b3;
-                ldsm_x4_t(vbase + (np >> 2) * BOX_BYTES + kk * 16 * 128 + pv_row + ((((2 * np) & 7) << 4) ^ pv_x), b0, b1, b2, b3);
-                mma_16(acc[2 * np], a0, a1, a2, a3, b0, b1);
-                mma_16(acc[2 * np + 1], a0, a1, a2, a3, b2, b3);
-            }
+            uint32_t a[4];
+            weights_bf16(sc, kk, a);
+            accumulate_step<D>(vbase, kk, a, acc, lane);
         }
     };
 
     auto step64 = [&](uint32_t kbase, uint32_t vbase, int nrows, bool retained, int unit) {
         float sc[8][2];
         scores64(kbase, nrows, retained, unit, sc);
-        accumulate64(vbase, retained, sc);
-    };
-    // A key-only tile under RoPE decoupling.  The scores come from the keys as stored, the key sum
-    // wants them without the rotation: the helpers turn each half back between the two uses, and
-    // the owner forms the second half's scores (then the first half's sum) in the meantime.
-    auto rope_tile = [&](uint32_t base, int n0, int n1, int unit) {
-        float sc0[8][2], sc1[8][2];
-        scores64(base, n0, false, unit, sc0);
-        team_sync(wq);                         // every lane is past its last read of half 0 as stored
-        if (n1 > 0) {
-            const float alpha = scores64(base + HALF_BYTES, n1, false, unit, sc1);
-#pragma unroll
-            for (int n = 0; n < 8; ++n) { sc0[n][0] *= alpha; sc0[n][1] *= alpha; }     // the sums moved to the new maximum
-        }
-        team_sync(wq);                         // half 0 is turned back (and half 1 is free to be)
-        accumulate64(base, false, sc0);
-        if (n1 > 0) {
-            team_sync(wq);                     // half 1 is turned back
-            accumulate64(base + HALF_BYTES, false, sc1);
-        }
+        accumulate64(vbase, sc);
     };
 
     zero_acc();
@@ -669,12 +558,8 @@ decode_stream_bf16(const __nv_bfloat16* __restrict__ q, const __grid_constant__ 
             const int s = i % SLOTS, round = i / SLOTS;
             const int t = (int)(gt_lo + i - (long long)u * pl.n_tiles);
             if (ok) {
-                if (!loaded) { load_q(u); loaded = true; }
+                if (!loaded) { load_queries<D>(q, u, g, lane, qa); loaded = true; }
                 ok = tma::mbar_wait_warp(&full_bar[s], round & 1, fault, 2);
-            }
-            if (ROPE && t >= pl.n_rt) {        // tell the helpers whether this key-only tile is worked on
-                if (lane == 0) team_ok[wq] = ok ? 1 : 0;
-                team_sync(wq);
             }
             if (!ok) continue;
             const uint32_t base = tma::smem_u32(smem + s * SLOT_BYTES);
@@ -682,13 +567,9 @@ decode_stream_bf16(const __nv_bfloat16* __restrict__ q, const __grid_constant__ 
                 step64(base, base + HALF_BYTES, min(KEYS, n_ret - t * KEYS), true, u);
             } else {
                 const int r0 = (t - pl.n_rt) * 2 * KEYS;
-                if (ROPE) {
-                    rope_tile(base, min(KEYS, n_apx - r0), min(KEYS, n_apx - r0 - KEYS), u);
-                } else {
-                    step64(base, base, min(KEYS, n_apx - r0), false, u);
-                    if (n_apx - r0 > KEYS)
-                        step64(base + HALF_BYTES, base + HALF_BYTES, min(KEYS, n_apx - r0 - KEYS), false, u);
-                }
+                step64(base, base, min(KEYS, n_apx - r0), false, u);
+                if (n_apx - r0 > KEYS)
+                    step64(base + HALF_BYTES, base + HALF_BYTES, min(KEYS, n_apx - r0 - KEYS), false, u);
             }
             __syncwarp();
             if (lane == 0) tma::mbar_arrive(&empty_bar[s]);
