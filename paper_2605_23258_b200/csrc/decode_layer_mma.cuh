@@ -4,19 +4,23 @@
 // in which a block owns a slice of the tokens of one (sequence, layer) and ALL its heads, so that every
 // approximated key is read once for the key sums of all query heads of the layer.
 //
-// Split kernel: 8 warps, warp w = KV head w.  The slice is walked in tiles that fill one 64 KB stage (two
-// stages, cp.async, the next tile in flight while this one is worked on; a third stage would leave the
-// first-level cache, where the spilled registers live, a few KB): 16 retained tokens (keys and
-// values of the 8 heads) or 32 approximated tokens (keys of the 8 heads).  Per tile
-//   phase 1  warp h: logits of its g query heads against head h's keys (M = the heads padded to 16 rows),
-//            online softmax; for an approximated tile the probabilities go to shared memory as bf16
-//            hi + lo, P[32 query heads][32 tokens], with the rescaling factor of each query head;
+// Split kernel: 8 warps, warp w = KV head w.  The slice is walked in tiles that fill one 64 KB stage (three
+// stages, cp.async): 16 retained tokens (keys and values of the 8 heads) or 32 approximated tokens (keys of the 8
+// heads).  Per tile
+//   phase 1  warp h: logits of its g query heads against head h's keys (the keys fill the 16 rows of the MMAs, the heads
+//            their eight columns), online softmax; for an approximated tile the probabilities go to shared memory as
+//            bf16 hi + lo, P[32 query heads][32 tokens], with the rescaling factor of each query head;
 //   phase 2  warp h': its accumulator acc_k[32 query heads][128] (key sums over head h') is rescaled and
-//            takes P K_h' (both halves of P); for a retained tile warp h adds P V_h for its own heads.
+//            takes P K_h' (both halves of P); for a retained tile warp h adds V_h^T P for its own heads.
+// Phase 1 is a chain of dependent MMAs, shuffles and exponentials, phase 2 a run of independent MMAs: with two warps to a
+// scheduler neither hides the other's latency unless they are the same warp's instructions.  So phase 1 of tile t + 1 is
+// laid between the MMAs of phase 2 of tile t, one barrier a tile; the third stage is the tile in flight meanwhile.
 // Records have the layout of the CUDA-core split kernel: per (unit, split, head) m, l, acc_v[128],
 // acc_k[8][128].
 #ifndef VECTOR_DECODE_LAYER_MMA_CUH_
 #define VECTOR_DECODE_LAYER_MMA_CUH_
+
+#include <type_traits>
 
 #include "common.cuh"
 #include "decode_bf16.cuh"
@@ -29,10 +33,11 @@ constexpr int HKV = 8, THREADS = 32 * HKV, MQ = 32;        // query heads per la
 constexpr int RT = 16, AT = 32;                            // tokens per retained / approximated tile
 constexpr int STAGE_BYTES = 65536, HEAD_RET = RT * 256, HEAD_APX = AT * 256;
 constexpr int PS_ROW = 80;                                 // bytes per row of P: 32 tokens + padding (conflict-free ldmatrix)
-constexpr int STAGES = 2;
+constexpr int STAGES = 3;
 constexpr int RET_COST = 1, APX_COST = 2;                  // relative time of a tile (measured: 1:1 246, 1:2 239, 2:5 248, 1:4 258 us
                                                            // a step of 32 layers and 7200 rows; 82, 58, 62 and 74 for one layer)
-constexpr int SMEM_BYTES = STAGES * STAGE_BYTES + 2 * MQ * PS_ROW + MQ * 4 + 128;
+constexpr int P_BYTES = 2 * MQ * PS_ROW + MQ * 4;          // P hi, P lo, factors: one set for each of two tiles
+constexpr int SMEM_BYTES = STAGES * STAGE_BYTES + 2 * P_BYTES + 128;
 constexpr int REC = 2 + 128 + HKV * 128;
 
 // grid (n_splits, U / 8), THREADS threads, SMEM_BYTES dynamic shared memory.
@@ -44,9 +49,8 @@ decode_layer_mma(const __nv_bfloat16* __restrict__ q, const __nv_bfloat16* __res
     asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory");
     extern __shared__ __align__(128) unsigned char lsm[];
     unsigned char* stage0 = lsm;
-    unsigned char* ps_hi = lsm + STAGES * STAGE_BYTES;
-    unsigned char* ps_lo = ps_hi + MQ * PS_ROW;
-    float* alpha_s = reinterpret_cast<float*>(ps_lo + MQ * PS_ROW);
+    unsigned char* const ps = lsm + STAGES * STAGE_BYTES;
+    const uint32_t dump = tma::smem_u32(ps + 2 * P_BYTES);      // where the rows of absent heads go
     const int split = blockIdx.x, n_splits = gridDim.x, ul = blockIdx.y;
     const int tid = threadIdx.x, lane = tid & 31, h = tid >> 5;
     const int gid = lane >> 2, tig = lane & 3, mat = lane >> 3, r8 = lane & 7;
@@ -60,8 +64,8 @@ decode_layer_mma(const __nv_bfloat16* __restrict__ q, const __nv_bfloat16* __res
     const int t_lo = tile_at(weight * split / n_splits), t_hi = tile_at(weight * (split + 1) / n_splits);
     const size_t u = (size_t)ul * HKV + h;
 
-    for (int i = tid; i < 2 * MQ * PS_ROW / 4 + MQ; i += THREADS) reinterpret_cast<uint32_t*>(ps_hi)[i] = 0u;   // P and the factors
-    // the g query rows of this head as A fragments (rows g .. 15 zero)
+    for (int i = tid; i < 2 * P_BYTES / 4; i += THREADS) reinterpret_cast<uint32_t*>(ps)[i] = 0u;
+    // the g query rows of this head as B fragments (columns g .. 7 zero)
     uint32_t qa[8][2];
     {
         const uint32_t* qrow = reinterpret_cast<const uint32_t*>(q + (u * g + min(gid, g - 1)) * 128);
@@ -71,14 +75,14 @@ decode_layer_mma(const __nv_bfloat16* __restrict__ q, const __nv_bfloat16* __res
             qa[ks][1] = gid < g ? qrow[ks * 8 + 4 + tig] : 0u;
         }
     }
-    float acc_k[2][16][4], acc_v[16][2];
+    float acc_k[2][16][4], acc_v[8][4];            // acc_v[n]: dims 16 n + gid (, + 8) of heads 2 tig, + 1
 #pragma unroll
     for (int n = 0; n < 16; ++n) {
-        acc_v[n][0] = acc_v[n][1] = 0.f;
+        if (n < 8) acc_v[n][0] = acc_v[n][1] = acc_v[n][2] = acc_v[n][3] = 0.f;
 #pragma unroll
         for (int mt = 0; mt < 2; ++mt) acc_k[mt][n][0] = acc_k[mt][n][1] = acc_k[mt][n][2] = acc_k[mt][n][3] = 0.f;
     }
-    float m = -INFINITY, l = 0.f;
+    float m[2] = {-INFINITY, -INFINITY}, l[2] = {0.f, 0.f};       // of heads 2 tig, + 1; l: this lane's tokens only
 
     // 4096 16-byte pieces per tile, 16 per thread; rows past the pool's end are filled with zeros.  A thread's
     // pieces share the 16-byte column (tid & 15) and the token row (tid >> 4, + 16 for every other piece of an
@@ -116,132 +120,186 @@ decode_layer_mma(const __nv_bfloat16* __restrict__ q, const __nv_bfloat16* __res
         rtc::cp_async_commit();
     };
 
-    prefetch(t_lo);
-    for (int t = t_lo; t < t_hi; ++t) {
-        unsigned char* st = stage0 + ((t - t_lo) % STAGES) * STAGE_BYTES;
-        rtc::cp_async_wait<0>();
-        __syncthreads();                       // the tile has landed; everyone is done with the stage of tile t - 1, P and the factors
-        prefetch(t + 1);                       // into the stage of tile t - 1
-        const bool retained = t < n_rt;
-        const int ntok = retained ? min(RT, n_ret - t * RT) : min(AT, n_apx - (t - n_rt) * AT);
-        const uint32_t kbase = tma::smem_u32(st) + h * (retained ? HEAD_RET : HEAD_APX);
-        // ---- phase 1: logits of this head's query rows, 16 tokens per ldmatrix
-        float sc[4][2], zz[2];
+    // State of a tile between its two phases: the factors of heads 2 tig, + 1 and, retained, P as B fragments.
+    float alpha[2] = {1.f, 1.f}, sc[2][4];
+    uint32_t bp[2][2];
+    const uint32_t k_row = (uint32_t)((r8 + (mat & 1) * 8) * 256);        // ldmatrix: (rows 0-7 | 8-15) x (16-byte chunk lo | hi)
+    const int k_ch = mat >> 1;
+    auto stage_of = [&](int t) { return tma::smem_u32(stage0 + ((t - t_lo) % STAGES) * STAGE_BYTES); };
+    // logits, k step `item / J` of the 16 tokens `item % J`, J = 1 (retained) or 2
+    auto logit_item = [&](uint32_t kbase, int item, int J) {
+        const int ks = item / J, j = item % J;
+        uint32_t a0, a1, a2, a3;
+        dbf::ldsm_x4(kbase + j * 16 * 256 + k_row + (((2 * ks + k_ch) ^ r8) << 4), a0, a1, a2, a3);
+        dbf::mma_16(sc[j], a0, a1, a2, a3, qa[ks][0], qa[ks][1]);
+    };
+    // softmax of a tile's logits; leaves P and the factors where phase 2 takes them
+    auto softmax = [&](auto ret, int t, float (&al)[2], uint32_t (&b)[2][2]) {
+        constexpr bool RET = decltype(ret)::value;
+        constexpr int J = RET ? 1 : 2;
+        const int ntok = RET ? min(RT, n_ret - t * RT) : min(AT, n_apx - (t - n_rt) * AT);
+        float mx[2] = {-INFINITY, -INFINITY};
 #pragma unroll
-        for (int n = 0; n < 4; ++n) sc[n][0] = sc[n][1] = 0.f;
+        for (int j = 0; j < J; ++j)
 #pragma unroll
-        for (int ks = 0; ks < 8; ++ks) {
+            for (int e = 0; e < 4; ++e) {
+                sc[j][e] = 16 * j + 8 * (e >> 1) + gid < ntok ? sc[j][e] * scale_log2e : -INFINITY;
+                mx[e & 1] = fmaxf(mx[e & 1], sc[j][e]);
+            }
 #pragma unroll
-            for (int j = 0; j < 2; ++j) {
-                if (j == 0 || !retained) {
-                    uint32_t b0, b1, b2, b3;
-                    dbf::ldsm_x4(kbase + (j * 16 + r8 + (mat >> 1) * 8) * 256 + (((2 * ks + (mat & 1)) ^ r8) << 4), b0, b1, b2, b3);
-                    dbf::mma_lo8(sc[2 * j][0], sc[2 * j][1], zz[0], zz[1], qa[ks][0], qa[ks][1], b0, b1);
-                    dbf::mma_lo8(sc[2 * j + 1][0], sc[2 * j + 1][1], zz[0], zz[1], qa[ks][0], qa[ks][1], b2, b3);
+        for (int o = 4; o < 32; o <<= 1)
+#pragma unroll
+            for (int e = 0; e < 2; ++e) mx[e] = fmaxf(mx[e], __shfl_xor_sync(0xffffffffu, mx[e], o));
+#pragma unroll
+        for (int e = 0; e < 2; ++e) {
+            const float m_new = fmaxf(m[e], mx[e]);        // finite: a tile holds at least one token
+            al[e] = exp2f(m[e] - m_new);
+            m[e] = m_new;
+            l[e] *= al[e];
+        }
+        unsigned char* const pb = ps + (t & 1) * P_BYTES;
+#pragma unroll
+        for (int j = 0; j < J; ++j) {
+            uint32_t hi[2], lo[2];                         // tokens gid and gid + 8 of the 16
+#pragma unroll
+            for (int e = 0; e < 2; ++e) {
+                const float p0 = exp2f(sc[j][2 * e] - m[0]), p1 = exp2f(sc[j][2 * e + 1] - m[1]);
+                l[0] += p0;
+                l[1] += p1;
+                hi[e] = dbf::pack_bf16(p0, p1);
+                lo[e] = dbf::pack_bf16(p0 - __uint_as_float(hi[e] << 16), p1 - __uint_as_float(hi[e] & 0xffff0000u));
+            }
+            if (RET) {
+#pragma unroll
+                for (int e = 0; e < 2; ++e) {
+                    asm volatile("movmatrix.sync.aligned.m8n8.trans.b16 %0, %1;\n" : "=r"(b[0][e]) : "r"(hi[e]));
+                    asm volatile("movmatrix.sync.aligned.m8n8.trans.b16 %0, %1;\n" : "=r"(b[1][e]) : "r"(lo[e]));
                 }
+            } else {
+                // matrices (hi | lo) x (tokens 0-7 | 8-15), transposed on the way: a row a head
+                const uint32_t at = r8 < g ? tma::smem_u32(pb) + (mat >> 1) * MQ * PS_ROW + (h * g + r8) * PS_ROW + j * 32 + (mat & 1) * 16 : dump + r8 * 16;
+                asm volatile("stmatrix.sync.aligned.m8n8.x4.trans.shared.b16 [%0], {%1,%2,%3,%4};\n" ::"r"(at), "r"(hi[0]), "r"(hi[1]), "r"(lo[0]), "r"(lo[1]) : "memory");
             }
         }
-        float mx = -INFINITY;
 #pragma unroll
-        for (int n = 0; n < 4; ++n) {
-            const int kc = n * 8 + 2 * tig;
-            sc[n][0] = kc < ntok ? sc[n][0] * scale_log2e : -INFINITY;
-            sc[n][1] = kc + 1 < ntok ? sc[n][1] * scale_log2e : -INFINITY;
-            mx = fmaxf(mx, fmaxf(sc[n][0], sc[n][1]));
-        }
-        mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 1));
-        mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 2));
-        const float m_new = fmaxf(m, mx);              // finite: a tile holds at least one token
-        const float alpha = exp2f(m - m_new);
-        float ls = 0.f;
-#pragma unroll
-        for (int n = 0; n < 4; ++n) {
-            sc[n][0] = exp2f(sc[n][0] - m_new);
-            sc[n][1] = exp2f(sc[n][1] - m_new);
-            ls += sc[n][0] + sc[n][1];
-        }
-        l = l * alpha + ls;
-        m = m_new;
-        if (gid < g) {
-            if (tig == 0) alpha_s[h * g + gid] = alpha;
-            if (!retained) {
-#pragma unroll
-                for (int n = 0; n < 4; ++n) {
-                    const uint32_t hi = dbf::pack_bf16(sc[n][0], sc[n][1]);
-                    const uint32_t lo = dbf::pack_bf16(sc[n][0] - __uint_as_float(hi << 16), sc[n][1] - __uint_as_float(hi & 0xffff0000u));
-                    *reinterpret_cast<uint32_t*>(ps_hi + (h * g + gid) * PS_ROW + (n * 8 + 2 * tig) * 2) = hi;
-                    *reinterpret_cast<uint32_t*>(ps_lo + (h * g + gid) * PS_ROW + (n * 8 + 2 * tig) * 2) = lo;
-                }
-            }
-        }
-        const int changed = __syncthreads_or(gid < g && alpha != 1.f);
-        // ---- phase 2: rescale, then the tile's contribution
+        for (int e = 0; e < 2; ++e)
+            if (lane < 4 && 2 * lane + e < g) reinterpret_cast<float*>(pb + 2 * MQ * PS_ROW)[h * g + 2 * lane + e] = al[e];
+    };
+    // Phase 2 of tile t with phase 1 of tile t + 1 between its MMAs.  next: 0 none, 1 retained, 2 approximated.
+    auto interval = [&](auto ret, auto next, int t, int changed) {
+        constexpr bool RET = decltype(ret)::value;
+        constexpr int NEXT = decltype(next)::value, J = NEXT == 1 ? 1 : 2, ITEMS = NEXT == 0 ? 0 : 8 * J;
+        const uint32_t st = stage_of(t), kn = stage_of(t + 1) + h * (NEXT == 1 ? HEAD_RET : HEAD_APX);
         if (changed) {
+            const float* f = reinterpret_cast<const float*>(ps + (t & 1) * P_BYTES + 2 * MQ * PS_ROW);
 #pragma unroll
             for (int mt = 0; mt < 2; ++mt) {
-                const float f0 = alpha_s[16 * mt + gid], f1 = alpha_s[16 * mt + 8 + gid];
+                const float f0 = f[16 * mt + gid], f1 = f[16 * mt + 8 + gid];
 #pragma unroll
                 for (int n = 0; n < 16; ++n) { acc_k[mt][n][0] *= f0; acc_k[mt][n][1] *= f0; acc_k[mt][n][2] *= f1; acc_k[mt][n][3] *= f1; }
             }
 #pragma unroll
-            for (int n = 0; n < 16; ++n) { acc_v[n][0] *= alpha; acc_v[n][1] *= alpha; }
+            for (int n = 0; n < 8; ++n) { acc_v[n][0] *= alpha[0]; acc_v[n][1] *= alpha[1]; acc_v[n][2] *= alpha[0]; acc_v[n][3] *= alpha[1]; }
         }
-        if (retained) {
-            // sum p v for this head's own query rows: P from the registers, hi then lo
-            const uint32_t vbase = tma::smem_u32(st) + 32768 + h * HEAD_RET;
-            const uint32_t a0 = dbf::pack_bf16(sc[0][0], sc[0][1]), a2 = dbf::pack_bf16(sc[1][0], sc[1][1]);
-            const uint32_t l0 = dbf::pack_bf16(sc[0][0] - __uint_as_float(a0 << 16), sc[0][1] - __uint_as_float(a0 & 0xffff0000u));
-            const uint32_t l2 = dbf::pack_bf16(sc[1][0] - __uint_as_float(a2 << 16), sc[1][1] - __uint_as_float(a2 & 0xffff0000u));
-            // the hi and the lo product of an accumulator are kept a whole sweep apart: back to back the second
-            // would wait for the first
 #pragma unroll
-            for (int part = 0; part < 2; ++part) {
-                const uint32_t x0 = part ? l0 : a0, x2 = part ? l2 : a2;
+        for (int j = 0; j < 2; ++j) sc[j][0] = sc[j][1] = sc[j][2] = sc[j][3] = 0.f;
+        float al[2] = {1.f, 1.f};
+        uint32_t b[2][2] = {};
+        if (RET) {
+            // sum p v for this head's own query rows; the hi and the lo product of an accumulator are kept apart: back to
+            // back the second would wait for the first
+            const uint32_t vbase = st + 32768 + h * HEAD_RET;
 #pragma unroll
-                for (int np = 0; np < 8; ++np) {
-                    uint32_t b0, b1, b2, b3;
-                    dbf::ldsm_x4_t(vbase + (r8 + (mat & 1) * 8) * 256 + (((2 * np + (mat >> 1)) ^ r8) << 4), b0, b1, b2, b3);
-                    dbf::mma_lo8(acc_v[2 * np][0], acc_v[2 * np][1], zz[0], zz[1], x0, x2, b0, b1);
-                    dbf::mma_lo8(acc_v[2 * np + 1][0], acc_v[2 * np + 1][1], zz[0], zz[1], x0, x2, b2, b3);
-                }
+            for (int q4 = 0; q4 < 2; ++q4) {
+                uint32_t a[4][4];
+#pragma unroll
+                for (int n = 0; n < 4; ++n)
+                    dbf::ldsm_x4_t(vbase + k_row + (((2 * (4 * q4 + n) + k_ch) ^ r8) << 4), a[n][0], a[n][2], a[n][1], a[n][3]);
+#pragma unroll
+                for (int part = 0; part < 2; ++part)
+#pragma unroll
+                    for (int n = 0; n < 4; ++n) {
+                        dbf::mma_16(acc_v[4 * q4 + n], a[n][0], a[n][1], a[n][2], a[n][3], bp[part][0], bp[part][1]);
+                        const int it = 8 * q4 + 4 * part + n;                  // of 16
+                        if (it < ITEMS) logit_item(kn, it, J);
+                    }
             }
+            if constexpr (NEXT != 0) softmax(std::bool_constant<NEXT == 1>{}, t + 1, al, b);
         } else {
             // key sums over head h (= this warp) for all query heads of the layer: P[32 x 32] K_h[32 x 128]
-            const uint32_t pa = (uint32_t)(((lane & 7) + ((lane >> 3) & 1) * 8) * PS_ROW + (lane >> 4) * 16);
-            const uint32_t ph = tma::smem_u32(ps_hi) + pa, pl = tma::smem_u32(ps_lo) + pa;
+            const uint32_t kbase = st + h * HEAD_APX;
+            const uint32_t ph = tma::smem_u32(ps + (t & 1) * P_BYTES) + (uint32_t)((r8 + (mat & 1) * 8) * PS_ROW + (mat >> 1) * 16);
 #pragma unroll
             for (int kk = 0; kk < 2; ++kk) {
-                uint32_t ah[2][4], al[2][4];
-#pragma unroll
-                for (int mt = 0; mt < 2; ++mt) {
-                    dbf::ldsm_x4(ph + mt * 16 * PS_ROW + kk * 32, ah[mt][0], ah[mt][1], ah[mt][2], ah[mt][3]);
-                    dbf::ldsm_x4(pl + mt * 16 * PS_ROW + kk * 32, al[mt][0], al[mt][1], al[mt][2], al[mt][3]);
-                }
 #pragma unroll
                 for (int part = 0; part < 2; ++part) {             // hi sweep, then lo sweep (see above)
+                    uint32_t a[2][4];
+#pragma unroll
+                    for (int mt = 0; mt < 2; ++mt)
+                        dbf::ldsm_x4(ph + part * MQ * PS_ROW + mt * 16 * PS_ROW + kk * 32, a[mt][0], a[mt][1], a[mt][2], a[mt][3]);
 #pragma unroll
                     for (int np = 0; np < 8; ++np) {
                         uint32_t b0, b1, b2, b3;
-                        dbf::ldsm_x4_t(kbase + (kk * 16 + r8 + (mat & 1) * 8) * 256 + (((2 * np + (mat >> 1)) ^ r8) << 4), b0, b1, b2, b3);
+                        dbf::ldsm_x4_t(kbase + kk * 16 * 256 + k_row + (((2 * np + k_ch) ^ r8) << 4), b0, b1, b2, b3);
 #pragma unroll
                         for (int mt = 0; mt < 2; ++mt) {
-                            const uint32_t* a = part ? al[mt] : ah[mt];
-                            dbf::mma_16(acc_k[mt][2 * np], a[0], a[1], a[2], a[3], b0, b1);
-                            dbf::mma_16(acc_k[mt][2 * np + 1], a[0], a[1], a[2], a[3], b2, b3);
+                            dbf::mma_16(acc_k[mt][2 * np], a[mt][0], a[mt][1], a[mt][2], a[mt][3], b0, b1);
+                            dbf::mma_16(acc_k[mt][2 * np + 1], a[mt][0], a[mt][1], a[mt][2], a[mt][3], b2, b3);
                         }
+                        const int it = 16 * kk + 8 * part + np;                // of 32
+                        if (it < ITEMS) logit_item(kn, it, J);
                     }
                 }
+                if constexpr (NEXT != 0) if (kk == 0) softmax(std::bool_constant<NEXT == 1>{}, t + 1, al, b);
             }
         }
+#pragma unroll
+        for (int e = 0; e < 2; ++e) { alpha[e] = al[e]; bp[0][e] = b[0][e]; bp[1][e] = b[1][e]; }
+    };
+    using Ret = std::true_type;
+    using Apx = std::false_type;
+    using None = std::integral_constant<int, 0>;
+    using NextRet = std::integral_constant<int, 1>;
+    using NextApx = std::integral_constant<int, 2>;
+
+    prefetch(t_lo);
+    prefetch(t_lo + 1);
+    if (t_lo < t_hi) {
+        rtc::cp_async_wait<1>();
+        __syncthreads();                       // the first tile has landed
+#pragma unroll
+        for (int j = 0; j < 2; ++j) sc[j][0] = sc[j][1] = sc[j][2] = sc[j][3] = 0.f;
+        if (t_lo < n_rt) {
+#pragma unroll
+            for (int it = 0; it < 8; ++it) logit_item(stage_of(t_lo) + h * HEAD_RET, it, 1);
+            softmax(Ret{}, t_lo, alpha, bp);
+        } else {
+#pragma unroll
+            for (int it = 0; it < 16; ++it) logit_item(stage_of(t_lo) + h * HEAD_APX, it, 2);
+            softmax(Apx{}, t_lo, alpha, bp);
+        }
+    }
+    for (int t = t_lo; t < t_hi; ++t) {
+        rtc::cp_async_wait<0>();
+        // tile t + 1 has landed, P and the factors of tile t are written; everyone is done with tile t - 1, whose stage tile t + 2 takes
+        const int changed = __syncthreads_or((2 * tig < g && alpha[0] != 1.f) || (2 * tig + 1 < g && alpha[1] != 1.f));
+        prefetch(t + 2);
+        if (t + 1 == t_hi) { if (t < n_rt) interval(Ret{}, None{}, t, changed); else interval(Apx{}, None{}, t, changed); }
+        else if (t + 1 < n_rt) interval(Ret{}, NextRet{}, t, changed);
+        else if (t < n_rt) interval(Ret{}, NextApx{}, t, changed);
+        else interval(Apx{}, NextApx{}, t, changed);
     }
     // ---- records.  Warp h: m, l and sum p v of its own query rows; every warp: its head's key sums for all rows
-    l += __shfl_xor_sync(0xffffffffu, l, 1);
-    l += __shfl_xor_sync(0xffffffffu, l, 2);
-    if (gid < g) {
-        float* rec = partial + ((u * n_splits + split) * g + gid) * REC;
-        if (tig == 0) { rec[0] = m * 0.69314718055994531f; rec[1] = l; }
 #pragma unroll
-        for (int n = 0; n < 16; ++n) *reinterpret_cast<float2*>(rec + 2 + n * 8 + 2 * tig) = make_float2(acc_v[n][0], acc_v[n][1]);
+    for (int e = 0; e < 2; ++e) {
+#pragma unroll
+        for (int o = 4; o < 32; o <<= 1) l[e] += __shfl_xor_sync(0xffffffffu, l[e], o);
+        if (2 * tig + e < g) {
+            float* rec = partial + ((u * n_splits + split) * g + 2 * tig + e) * REC;
+            if (gid == 0) { rec[0] = m[e] * 0.69314718055994531f; rec[1] = l[e]; }
+#pragma unroll
+            for (int n = 0; n < 8; ++n) { rec[2 + 16 * n + gid] = acc_v[n][e]; rec[2 + 16 * n + 8 + gid] = acc_v[n][2 + e]; }
+        }
     }
     const int n_q = HKV * g;
 #pragma unroll
