@@ -242,7 +242,8 @@ static vector_status launch_layer_mma(const Dims& dm, int L, const void* q, cons
     const int UL = dm.U / dlm::HKV;
     const int64_t tiles = (ch->n_ret + dlm::RT - 1) / dlm::RT + (ch->n_apx + dlm::AT - 1) / dlm::AT;
     // Splits: a multiprocessor holds one block, so the time goes with whole rounds of blocks over the splits' number; a block
-    // costs about eight tiles besides: its first loads, its records (32 layers of 7200 rows: 215 us a step, 238 with none counted).
+    // costs about eight retained tiles besides: its first loads, its records (four to fourteen counted make no difference from 2000 to
+    // 100000 tokens; with none counted, 32 layers of 7200 rows took a tenth longer).
     const double cost = dlm::RET_COST * (double)((ch->n_ret + dlm::RT - 1) / dlm::RT) + dlm::APX_COST * (double)((ch->n_apx + dlm::AT - 1) / dlm::AT);
     int64_t n_splits = 1;
     double best = 1e300;
@@ -250,9 +251,21 @@ static vector_status launch_layer_mma(const Dims& dm, int L, const void* q, cons
         const double t = (double)((n * UL + sm_count() - 1) / sm_count()) * (cost / (double)n + 8.0);
         if (t < best - 1e-9) { best = t; n_splits = n; }
     }
+    int* fault = kernel_fault_address();
+    if (!fault) return VECTOR_ERR_CUDA;
+    dbf::Maps maps;
+    bool ok = true;
+    if (ch->n_ret > 0) {
+        ok = ok && tma::encode_bf16_3d(&maps.ret_k, ch->ret_k, 128, (uint64_t)ch->n_ret, (uint64_t)dm.U, 256, (uint64_t)ch->cap_ret * 256, 64, dlm::RT, dlm::HKV);
+        ok = ok && tma::encode_bf16_3d(&maps.ret_v, ch->ret_v, 128, (uint64_t)ch->n_ret, (uint64_t)dm.U, 256, (uint64_t)ch->cap_ret * 256, 64, dlm::RT, dlm::HKV);
+    }
+    if (ch->n_apx > 0)
+        ok = ok && tma::encode_bf16_3d(&maps.apx_k, ch->apx_k, 128, (uint64_t)ch->n_apx, (uint64_t)dm.U, 256, (uint64_t)ch->cap_apx * 256, 64, dlm::AT, dlm::HKV);
+    if (!ok) return VECTOR_ERR_CUDA;
+    if (ch->n_ret == 0) { maps.ret_k = maps.apx_k; maps.ret_v = maps.apx_k; }   // never dereferenced: no such tiles
+    if (ch->n_apx == 0) maps.apx_k = maps.ret_k;
     VEC_CUDA_CHECK(launch_maybe_dependent(true, dlm::decode_layer_mma, dim3((unsigned)n_splits, UL), dim3(dlm::THREADS), dlm::SMEM_BYTES, st,
-        (const T*)q, (const T*)ch->ret_k, (const T*)ch->ret_v, (const T*)ch->apx_k, (long long)ch->cap_ret, (long long)ch->cap_apx,
-        (int)ch->n_ret, (int)ch->n_apx, dm.g, dm.scale * 1.4426950408889634f, partial));
+        (const T*)q, maps, (int)ch->n_ret, (int)ch->n_apx, dm.g, dm.scale * 1.4426950408889634f, partial, fault));
     if (out_dtype == VECTOR_F32)
         VEC_CUDA_CHECK(launch_maybe_dependent(true, dlm::decode_layer_merge_mma<float>, dim3(dm.U), dim3(dlm::MERGE_THREADS), 0, st, partial,
                                               (const T*)W, L, dm.g, (int)n_splits, (float*)out));

@@ -5,7 +5,7 @@
 // approximated key is read once for the key sums of all query heads of the layer.
 //
 // Split kernel: 8 warps, warp w = KV head w.  The slice is walked in tiles that fill one 64 KB stage (three
-// stages, cp.async): 16 retained tokens (keys and values of the 8 heads) or 32 approximated tokens (keys of the 8
+// stages, TMA): 16 retained tokens (keys and values of the 8 heads) or 32 approximated tokens (keys of the 8
 // heads).  Per tile
 //   phase 1  warp h: logits of its g query heads against head h's keys (the keys fill the 16 rows of the MMAs, the heads
 //            their eight columns), online softmax; for an approximated tile the probabilities go to shared memory as
@@ -15,6 +15,9 @@
 // Phase 1 is a chain of dependent MMAs, shuffles and exponentials, phase 2 a run of independent MMAs: with two warps to a
 // scheduler neither hides the other's latency unless they are the same warp's instructions.  So phase 1 of tile t + 1 is
 // laid between the MMAs of phase 2 of tile t, one barrier a tile; the third stage is the tile in flight meanwhile.
+// What bounds it: the warps' own instructions -- tensor pipe 41 % busy, HBM 0.74 of a copy's rate in the streaming
+// kernel -- with eight warps, whose accumulators leave no room for more.  Measured, 32 layers of 7200 rows, 630 MB, in a
+// graph: 144 us; 173 with tiles copied in 16-byte pieces by all threads, 210 with the two phases one after the other.
 // Records have the layout of the CUDA-core split kernel: per (unit, split, head) m, l, acc_v[128],
 // acc_k[8][128].
 #ifndef VECTOR_DECODE_LAYER_MMA_CUH_
@@ -24,32 +27,43 @@
 
 #include "common.cuh"
 #include "decode_bf16.cuh"
-#include "residual_tc.cuh"
 
 namespace vec {
 namespace dlm {
 
 constexpr int HKV = 8, THREADS = 32 * HKV, MQ = 32;        // query heads per layer the accumulators hold
 constexpr int RT = 16, AT = 32;                            // tokens per retained / approximated tile
-constexpr int STAGE_BYTES = 65536, HEAD_RET = RT * 256, HEAD_APX = AT * 256;
+// A stage: boxes of 64 channels x the tile's tokens x the 8 heads (128-byte rows, 128-byte swizzle); retained: keys, channels
+// 0-63 and 64-127, then values; approximated: keys.
+constexpr int STAGE_BYTES = 65536, HEAD_RET = RT * 128, HEAD_APX = AT * 128, BOX_RET = HKV * HEAD_RET, BOX_APX = HKV * HEAD_APX;
 constexpr int PS_ROW = 80;                                 // bytes per row of P: 32 tokens + padding (conflict-free ldmatrix)
 constexpr int STAGES = 3;
-constexpr int RET_COST = 1, APX_COST = 2;                  // relative time of a tile (measured: 1:1 246, 1:2 239, 2:5 248, 1:4 258 us
-                                                           // a step of 32 layers and 7200 rows; 82, 58, 62 and 74 for one layer)
+constexpr int RET_COST = 1, APX_COST = 2;                  // relative time of a tile (measured in a graph: 1:1 176, 2:3 154, 1:2 144, 4:9 150,
+                                                           // 2:5 157 us a step of 32 layers and 7200 rows; 48, 44, 43, 43, 43 for one layer)
 constexpr int P_BYTES = 2 * MQ * PS_ROW + MQ * 4;          // P hi, P lo, factors: one set for each of two tiles
-constexpr int SMEM_BYTES = STAGES * STAGE_BYTES + 2 * P_BYTES + 128;
+constexpr int SMEM_BYTES = STAGES * STAGE_BYTES + 2 * P_BYTES + 128 + 1024;       // + alignment slack
 constexpr int REC = 2 + 128 + HKV * 128;
+
+// The weights' reference follows the running maximum only when that has moved by more than SLACK (in powers of two): any
+// reference serves, weights up to 2^SLACK cost no precision, and with 32 heads to a tile one of them moves in most tiles, which
+// made every warp rescale 160 accumulators (32 layers of 7200 rows: 147 -> 143 us in a graph).
+constexpr float SLACK = 8.f;
+// (tc::ex2 gives zero for results below 2^-126: next to a weight of at least 2^-SLACK they do not change an fp32 sum.)
 
 // grid (n_splits, U / 8), THREADS threads, SMEM_BYTES dynamic shared memory.
 __global__ void __launch_bounds__(THREADS, 1)
-decode_layer_mma(const __nv_bfloat16* __restrict__ q, const __nv_bfloat16* __restrict__ ret_k,
-                 const __nv_bfloat16* __restrict__ ret_v, const __nv_bfloat16* __restrict__ apx_k, long long cap_ret,
-                 long long cap_apx, int n_ret, int n_apx, int g, float scale_log2e, float* __restrict__ partial) {
-    asm volatile("griddepcontrol.wait;\n" ::: "memory");        // launched as a programmatic dependent: nothing is touched before
+decode_layer_mma(const __nv_bfloat16* __restrict__ q, const __grid_constant__ dbf::Maps maps, int n_ret, int n_apx, int g,
+                 float scale_log2e, float* __restrict__ partial, int* __restrict__ fault) {
+    __shared__ __align__(8) uint64_t full_bar[STAGES];
+    if (threadIdx.x == 0) {
+        for (int s = 0; s < STAGES; ++s) tma::mbar_init(&full_bar[s], 1);
+        tma::mbar_fence_init();
+    }
+    asm volatile("griddepcontrol.wait;\n" ::: "memory");        // launched as a programmatic dependent: nothing of its inputs is touched before
     asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory");
-    extern __shared__ __align__(128) unsigned char lsm[];
-    unsigned char* stage0 = lsm;
-    unsigned char* const ps = lsm + STAGES * STAGE_BYTES;
+    extern __shared__ unsigned char lsm[];
+    unsigned char* const stage0 = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(lsm) + 1023) & ~uintptr_t(1023));
+    unsigned char* const ps = stage0 + STAGES * STAGE_BYTES;
     const uint32_t dump = tma::smem_u32(ps + 2 * P_BYTES);      // where the rows of absent heads go
     const int split = blockIdx.x, n_splits = gridDim.x, ul = blockIdx.y;
     const int tid = threadIdx.x, lane = tid & 31, h = tid >> 5;
@@ -84,53 +98,43 @@ decode_layer_mma(const __nv_bfloat16* __restrict__ q, const __nv_bfloat16* __res
     }
     float m[2] = {-INFINITY, -INFINITY}, l[2] = {0.f, 0.f};       // of heads 2 tig, + 1; l: this lane's tokens only
 
-    // 4096 16-byte pieces per tile, 16 per thread; rows past the pool's end are filled with zeros.  A thread's
-    // pieces share the 16-byte column (tid & 15) and the token row (tid >> 4, + 16 for every other piece of an
-    // approximated tile); they differ in the head (and, retained, in keys or values): fixed strides from one address.
-    const int p_tok = tid >> 4, p_ch = tid & 15;
-    const uint32_t p_dst = (uint32_t)(p_tok * 256 + ((p_ch ^ (p_tok & 7)) << 4));
-    const size_t ret_head = (size_t)cap_ret * 128, apx_head = (size_t)cap_apx * 128;      // elements from one head's pool to the next
-    auto load_tile = [&](int t, unsigned char* st) {
-        const uint32_t dst = tma::smem_u32(st) + p_dst;
-        if (t < n_rt) {
-            const int tok = t * RT + p_tok;
-            const bool in = tok < n_ret;
-            const size_t off = ((size_t)ul * HKV * cap_ret + (in ? tok : 0)) * 128 + p_ch * 8;
-            const __nv_bfloat16* ks = ret_k + off;
-            const __nv_bfloat16* vs = ret_v + off;
+    bool ok = true;                            // false once a wait gave up: walk on and touch nothing
+    // One thread requests a tile; rows past the pool's end are filled with zeros.
+    const uint64_t pol = tma::policy_evict_first();                 // the cache is read once per step
+    auto prefetch = [&](int t) {
+        if (tid == 0 && t < t_hi && ok) {
+            unsigned char* st = stage0 + ((t - t_lo) % STAGES) * STAGE_BYTES;
+            uint64_t* bar = &full_bar[(t - t_lo) % STAGES];
+            tma::mbar_expect_tx(bar, STAGE_BYTES);
 #pragma unroll
-            for (int hh = 0; hh < HKV; ++hh) {
-                rtc::cp_async16(dst + hh * HEAD_RET, ks + hh * ret_head, in ? 16u : 0u);
-                rtc::cp_async16(dst + 32768 + hh * HEAD_RET, vs + hh * ret_head, in ? 16u : 0u);
-            }
-        } else {
-            const int tok = (t - n_rt) * AT + p_tok;
-            const bool in0 = tok < n_apx, in1 = tok + 16 < n_apx;
-            const __nv_bfloat16* k0 = apx_k + ((size_t)ul * HKV * cap_apx + (in0 ? tok : 0)) * 128 + p_ch * 8;
-            const __nv_bfloat16* k1 = apx_k + ((size_t)ul * HKV * cap_apx + (in1 ? tok + 16 : 0)) * 128 + p_ch * 8;
-#pragma unroll
-            for (int hh = 0; hh < HKV; ++hh) {
-                rtc::cp_async16(dst + hh * HEAD_APX, k0 + hh * apx_head, in0 ? 16u : 0u);
-                rtc::cp_async16(dst + hh * HEAD_APX + 16 * 256, k1 + hh * apx_head, in1 ? 16u : 0u);
+            for (int x = 0; x < 2; ++x) {
+                if (t < n_rt) {
+                    tma::load_3d_hint(st + x * BOX_RET, &maps.ret_k, 64 * x, t * RT, ul * HKV, bar, pol);
+                    tma::load_3d_hint(st + 32768 + x * BOX_RET, &maps.ret_v, 64 * x, t * RT, ul * HKV, bar, pol);
+                } else {
+                    tma::load_3d_hint(st + x * BOX_APX, &maps.apx_k, 64 * x, (t - n_rt) * AT, ul * HKV, bar, pol);
+                }
             }
         }
+        __syncwarp();
     };
-    auto prefetch = [&](int t) {
-        if (t < t_hi) load_tile(t, stage0 + ((t - t_lo) % STAGES) * STAGE_BYTES);
-        rtc::cp_async_commit();
+    auto landed = [&](int t) {
+        if (ok && t < t_hi) ok = tma::mbar_wait_warp(&full_bar[(t - t_lo) % STAGES], ((t - t_lo) / STAGES) & 1, fault, 2);
     };
 
     // State of a tile between its two phases: the factors of heads 2 tig, + 1 and, retained, P as B fragments.
     float alpha[2] = {1.f, 1.f}, sc[2][4];
     uint32_t bp[2][2];
-    const uint32_t k_row = (uint32_t)((r8 + (mat & 1) * 8) * 256);        // ldmatrix: (rows 0-7 | 8-15) x (16-byte chunk lo | hi)
-    const int k_ch = mat >> 1;
+    // ldmatrix of 16 rows, (rows 0-7 | 8-15) x (16-byte chunk 2 c | 2 c + 1): a lane's address for c is this one with bits 5 and 6
+    // XORed by c % 4 (the swizzle), in box c / 4
+    const uint32_t frag = (uint32_t)((r8 + (mat & 1) * 8) * 128 + (((mat >> 1) ^ r8) << 4));
+    auto chunk = [](uint32_t base, int c, uint32_t box) { return (base ^ (uint32_t)((c & 3) << 5)) + (c >> 2) * box; };
     auto stage_of = [&](int t) { return tma::smem_u32(stage0 + ((t - t_lo) % STAGES) * STAGE_BYTES); };
     // logits, k step `item / J` of the 16 tokens `item % J`, J = 1 (retained) or 2
     auto logit_item = [&](uint32_t kbase, int item, int J) {
         const int ks = item / J, j = item % J;
         uint32_t a0, a1, a2, a3;
-        dbf::ldsm_x4(kbase + j * 16 * 256 + k_row + (((2 * ks + k_ch) ^ r8) << 4), a0, a1, a2, a3);
+        dbf::ldsm_x4(chunk(kbase, ks, J == 1 ? BOX_RET : BOX_APX) + j * 16 * 128, a0, a1, a2, a3);
         dbf::mma_16(sc[j], a0, a1, a2, a3, qa[ks][0], qa[ks][1]);
     };
     // softmax of a tile's logits; leaves P and the factors where phase 2 takes them
@@ -143,7 +147,8 @@ decode_layer_mma(const __nv_bfloat16* __restrict__ q, const __nv_bfloat16* __res
         for (int j = 0; j < J; ++j)
 #pragma unroll
             for (int e = 0; e < 4; ++e) {
-                sc[j][e] = 16 * j + 8 * (e >> 1) + gid < ntok ? sc[j][e] * scale_log2e : -INFINITY;
+                sc[j][e] *= scale_log2e;
+                if (ntok < 16 * J && 16 * j + 8 * (e >> 1) + gid >= ntok) sc[j][e] = -INFINITY;
                 mx[e & 1] = fmaxf(mx[e & 1], sc[j][e]);
             }
 #pragma unroll
@@ -152,8 +157,8 @@ decode_layer_mma(const __nv_bfloat16* __restrict__ q, const __nv_bfloat16* __res
             for (int e = 0; e < 2; ++e) mx[e] = fmaxf(mx[e], __shfl_xor_sync(0xffffffffu, mx[e], o));
 #pragma unroll
         for (int e = 0; e < 2; ++e) {
-            const float m_new = fmaxf(m[e], mx[e]);        // finite: a tile holds at least one token
-            al[e] = exp2f(m[e] - m_new);
+            const float m_new = mx[e] > m[e] + SLACK ? mx[e] : m[e];          // finite: a tile holds at least one token
+            al[e] = tc::ex2(m[e] - m_new);
             m[e] = m_new;
             l[e] *= al[e];
         }
@@ -163,7 +168,7 @@ decode_layer_mma(const __nv_bfloat16* __restrict__ q, const __nv_bfloat16* __res
             uint32_t hi[2], lo[2];                         // tokens gid and gid + 8 of the 16
 #pragma unroll
             for (int e = 0; e < 2; ++e) {
-                const float p0 = exp2f(sc[j][2 * e] - m[0]), p1 = exp2f(sc[j][2 * e + 1] - m[1]);
+                const float p0 = tc::ex2(sc[j][2 * e] - m[0]), p1 = tc::ex2(sc[j][2 * e + 1] - m[1]);
                 l[0] += p0;
                 l[1] += p1;
                 hi[e] = dbf::pack_bf16(p0, p1);
@@ -189,7 +194,7 @@ decode_layer_mma(const __nv_bfloat16* __restrict__ q, const __nv_bfloat16* __res
     auto interval = [&](auto ret, auto next, int t, int changed) {
         constexpr bool RET = decltype(ret)::value;
         constexpr int NEXT = decltype(next)::value, J = NEXT == 1 ? 1 : 2, ITEMS = NEXT == 0 ? 0 : 8 * J;
-        const uint32_t st = stage_of(t), kn = stage_of(t + 1) + h * (NEXT == 1 ? HEAD_RET : HEAD_APX);
+        const uint32_t st = stage_of(t) + frag, kn = stage_of(t + 1) + frag + h * (NEXT == 1 ? HEAD_RET : HEAD_APX);
         if (changed) {
             const float* f = reinterpret_cast<const float*>(ps + (t & 1) * P_BYTES + 2 * MQ * PS_ROW);
 #pragma unroll
@@ -214,7 +219,7 @@ decode_layer_mma(const __nv_bfloat16* __restrict__ q, const __nv_bfloat16* __res
                 uint32_t a[4][4];
 #pragma unroll
                 for (int n = 0; n < 4; ++n)
-                    dbf::ldsm_x4_t(vbase + k_row + (((2 * (4 * q4 + n) + k_ch) ^ r8) << 4), a[n][0], a[n][2], a[n][1], a[n][3]);
+                    dbf::ldsm_x4_t(chunk(vbase, 4 * q4 + n, BOX_RET), a[n][0], a[n][2], a[n][1], a[n][3]);
 #pragma unroll
                 for (int part = 0; part < 2; ++part)
 #pragma unroll
@@ -240,7 +245,7 @@ decode_layer_mma(const __nv_bfloat16* __restrict__ q, const __nv_bfloat16* __res
 #pragma unroll
                     for (int np = 0; np < 8; ++np) {
                         uint32_t b0, b1, b2, b3;
-                        dbf::ldsm_x4_t(kbase + kk * 16 * 256 + k_row + (((2 * np + k_ch) ^ r8) << 4), b0, b1, b2, b3);
+                        dbf::ldsm_x4_t(chunk(kbase, np, BOX_APX) + kk * 16 * 128, b0, b1, b2, b3);
 #pragma unroll
                         for (int mt = 0; mt < 2; ++mt) {
                             dbf::mma_16(acc_k[mt][2 * np], a[mt][0], a[mt][1], a[mt][2], a[mt][3], b0, b1);
@@ -262,28 +267,29 @@ decode_layer_mma(const __nv_bfloat16* __restrict__ q, const __nv_bfloat16* __res
     using NextRet = std::integral_constant<int, 1>;
     using NextApx = std::integral_constant<int, 2>;
 
+    __syncthreads();                           // the barriers, P and the factors are initialised
     prefetch(t_lo);
     prefetch(t_lo + 1);
-    if (t_lo < t_hi) {
-        rtc::cp_async_wait<1>();
-        __syncthreads();                       // the first tile has landed
+    landed(t_lo);
+    if (t_lo < t_hi && ok) {
 #pragma unroll
         for (int j = 0; j < 2; ++j) sc[j][0] = sc[j][1] = sc[j][2] = sc[j][3] = 0.f;
         if (t_lo < n_rt) {
 #pragma unroll
-            for (int it = 0; it < 8; ++it) logit_item(stage_of(t_lo) + h * HEAD_RET, it, 1);
+            for (int it = 0; it < 8; ++it) logit_item(stage_of(t_lo) + frag + h * HEAD_RET, it, 1);
             softmax(Ret{}, t_lo, alpha, bp);
         } else {
 #pragma unroll
-            for (int it = 0; it < 16; ++it) logit_item(stage_of(t_lo) + h * HEAD_APX, it, 2);
+            for (int it = 0; it < 16; ++it) logit_item(stage_of(t_lo) + frag + h * HEAD_APX, it, 2);
             softmax(Apx{}, t_lo, alpha, bp);
         }
     }
     for (int t = t_lo; t < t_hi; ++t) {
-        rtc::cp_async_wait<0>();
-        // tile t + 1 has landed, P and the factors of tile t are written; everyone is done with tile t - 1, whose stage tile t + 2 takes
+        // P and the factors of tile t are written; everyone is done with tile t - 1, whose stage tile t + 2 takes
         const int changed = __syncthreads_or((2 * tig < g && alpha[0] != 1.f) || (2 * tig + 1 < g && alpha[1] != 1.f));
         prefetch(t + 2);
+        landed(t + 1);
+        if (!ok) continue;
         if (t + 1 == t_hi) { if (t < n_rt) interval(Ret{}, None{}, t, changed); else interval(Apx{}, None{}, t, changed); }
         else if (t + 1 < n_rt) interval(Ret{}, NextRet{}, t, changed);
         else if (t < n_rt) interval(Ret{}, NextApx{}, t, changed);

@@ -105,12 +105,12 @@ inline EncodeFn encoder() {
 // Rows at or beyond `rows` read as zero.  Returns false if the driver rejects the description.
 inline bool encode_bf16_3d(CUtensorMap* out, const void* base, uint64_t inner, uint64_t rows, uint64_t slabs,
                            uint64_t row_stride_bytes, uint64_t slab_stride_bytes, uint32_t box_inner,
-                           uint32_t box_rows) {
+                           uint32_t box_rows, uint32_t box_slabs = 1) {
     EncodeFn fn = encoder();
     if (!fn) return false;
     cuuint64_t dims[3] = {inner, rows, slabs};
     cuuint64_t strides[2] = {row_stride_bytes, slab_stride_bytes};
-    cuuint32_t box[3] = {box_inner, box_rows, 1};
+    cuuint32_t box[3] = {box_inner, box_rows, box_slabs};
     cuuint32_t estr[3] = {1, 1, 1};
     return fn(out, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(base), dims, strides, box, estr,
               CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
