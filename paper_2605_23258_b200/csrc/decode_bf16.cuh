@@ -43,8 +43,11 @@ namespace dbf {
 
 constexpr int KEYS = 64;                     // keys per softmax step (and per TMA box)
 constexpr int BOX_BYTES = 8192;              // 64 rows x 128 bytes
-// With RoPE decoupling a team of warps works on a tile (decode_rope.cuh) and leaves one record.
-constexpr int ROPE_TEAMS = 3;
+// The softmax's reference follows the running maximum only when that has moved by more than SLACK (in powers of two): any
+// reference serves, weights up to 2^SLACK cost no precision, and the accumulators are rescaled a few times instead of in every
+// other step (a step of 512 units of 4915 rows, 64 channels: 73.9 -> 72.3 us, with RoPE 131.4 -> 125.8; 128 channels 132.1 ->
+// 131.4 and 170.2 -> 166.8).  tc::ex2 gives zero below 2^-126: next to a weight of at least 2^-SLACK that changes no fp32 sum.
+constexpr float SLACK = 8.f;
 template <int D, bool ROPE> struct Cfg {
     static constexpr int HALF_BYTES = 64 * 2 * D;                    // 64 rows as D / 64 swizzled boxes
     static constexpr int SLOT_BYTES = 2 * HALF_BYTES;                // retained: K | V; key-only: keys 0-63 | keys 64-127
@@ -52,11 +55,13 @@ template <int D, bool ROPE> struct Cfg {
     // warp (one to a warp scheduler) makes up for it.
     // Measured: 512 units, 1639 retained + 3276 key-only rows, 431 MB: 82 us with the appended row = 5.3 TB/s (856 us on
     // CUDA cores).
-    static constexpr int CONSUMER_WARPS = ROPE ? ROPE_TEAMS : D == 128 ? 3 : 4;      // whose records a block leaves
+    // With RoPE decoupling a consumer is a team (decode_rope.cuh): a score warp and some sum warps.
+    // Four teams at 64 channels, of two sum warps with as many channel pairs each as the four have at 128.
+    static constexpr int CONSUMER_WARPS = D == 128 ? 3 : 4, SUM_WARPS = ROPE ? D / 32 : 0;
     static constexpr int SLOTS = D == 128 ? 6 : 12;                  // a multiple of CONSUMER_WARPS: a slot always serves the same warp
-    static constexpr int THREADS = ROPE ? 512 : 32 * (CONSUMER_WARPS + 1);
+    static constexpr int THREADS = 32 * (CONSUMER_WARPS * (1 + SUM_WARPS) + 1);
     static constexpr int STEP_BYTES = 2048 + 4 * KEYS + 32;          // RoPE: a step's weights, positions and factors
-    static constexpr int P_BYTES = ROPE ? ROPE_TEAMS * 2 * STEP_BYTES : 0;
+    static constexpr int P_BYTES = ROPE ? CONSUMER_WARPS * 2 * STEP_BYTES : 0;
     static constexpr int SMEM_BYTES = SLOTS * SLOT_BYTES + P_BYTES + 1024;     // + alignment slack; barriers live in static smem
     static constexpr int REC = 4 + 2 * D;                            // m, l, value-scale, pad, acc_v[D], acc_k[D]
     // CLUSTER: the warps' headers and value sums behind the slots, [CONSUMER_WARPS][g][4 + D]; a warp's key sums, [g][D], take
@@ -233,13 +238,13 @@ __device__ __forceinline__ float score_step(uint32_t kbase, int nrows, float sca
     }
     mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 1));
     mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 2));
-    const float m_new = fmaxf(m, mx);      // finite: key 0 of the step is valid for every row
-    const float alpha = exp2f(m - m_new);  // 0 on the first step
+    const float m_new = mx > m + SLACK ? mx : m;      // finite: key 0 of the step is valid for every row
+    const float alpha = tc::ex2(m - m_new);           // 0 on the first step
     float ls = 0.f;
 #pragma unroll
     for (int n = 0; n < 8; ++n) {
-        sc[n][0] = exp2f(sc[n][0] - m_new);
-        sc[n][1] = exp2f(sc[n][1] - m_new);
+        sc[n][0] = tc::ex2(sc[n][0] - m_new);
+        sc[n][1] = tc::ex2(sc[n][1] - m_new);
         ls += sc[n][0] + sc[n][1];
     }
     l = l * alpha + ls;

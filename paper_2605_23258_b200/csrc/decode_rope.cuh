@@ -4,11 +4,11 @@
 // A key-only token's logit takes the key as stored, its contribution to the key sum the key turned back by the token's
 // position.  Turning a key back costs a sine, a cosine and about ten instructions per channel pair, several times the rest
 // of the tile, so that warps that own whole tiles (decode_bf16.cuh) would be bound by their own instruction chains.  A
-// block therefore has three teams, tile i to team i % 3, of five warps each:
+// block therefore has teams, tile i to team i % TEAMS: three of five warps, or, at 64 channels, four of three:
 //   score warp   S = Q K^T and the online softmax, 64 keys a step; it leaves the weights as MMA A fragments (hi and
 //                lo halves; bf16 for values, fp16 for turned keys), the factor the older sums take, and the keys' positions
 //                in one of the team's two step buffers
-//   4 sum warps  each owns a quarter of the channel pairs (c, c + D/2).  It takes the rows as MMA B fragments straight from
+//   sum warps    each owns 16 of the channel pairs (c, c + D/2).  It takes the rows as MMA B fragments straight from
 //                the slot -- both channels of a pair lie in the same thread's fragments -- turns them in registers (fp16,
 //                eleven bits: a turned key is not a bf16 number and eight bits would not keep the key sum within the
 //                tolerance of the output; |k| beyond 65504 saturates) and multiplies: nothing is written back
@@ -16,6 +16,8 @@
 // cycles per 64 keys, 2300 of them busy) and the sum warps (2500 busy) waiting for one another.  Measured, 128 units of 3000
 // retained + 6000 key-only rows, 393 MB, with the appended row and the merge: 86 us; 104 us with warps that owned whole tiles
 // and twelve helpers that turned keys back in shared memory (a fence and three block barriers per 64 keys).
+// 64 channels, 512 units of 1639 + 3276 rows, in a graph: 112 us; 126 with three teams of five warps, whose score warps
+// took most of the time (72 without rotation).
 // The angle is position * theta^(-2c/D), taken as the 32-bit product of the position and the
 // channel's phase (turns per position as a fraction of 2^32), which is the angle modulo one turn.
 #ifndef VECTOR_DECODE_ROPE_CUH_
@@ -26,7 +28,6 @@
 namespace vec {
 namespace dbf {
 
-constexpr int SUM_WARPS = 4;
 constexpr uint32_t STEP_POS = 2048, STEP_ALPHA = STEP_POS + 4 * KEYS;     // a step buffer: weights [16 keys][hi | lo of 8 keys][head][8 keys], positions, factors
 
 // x and y, the two channels of eight pairs (two keys to a register), turned back by pos[] * phase and left as fp16.
@@ -77,8 +78,8 @@ __device__ __forceinline__ void score_step_keys(uint32_t kbase, int nrows, float
         for (int e = 0; e < 2; ++e) mx[e] = fmaxf(mx[e], __shfl_xor_sync(0xffffffffu, mx[e], o));
 #pragma unroll
     for (int e = 0; e < 2; ++e) {
-        const float m_new = fmaxf(m[e], mx[e]);        // finite: key 0 of the step is valid for every head
-        alpha[e] = exp2f(m[e] - m_new);                // 0 on the first step
+        const float m_new = mx[e] > m[e] + SLACK ? mx[e] : m[e];       // finite: key 0 of the step is valid for every head
+        alpha[e] = tc::ex2(m[e] - m_new);                              // 0 on the first step
         m[e] = m_new;
         l[e] *= alpha[e];
     }
@@ -86,13 +87,13 @@ __device__ __forceinline__ void score_step_keys(uint32_t kbase, int nrows, float
     for (int j = 0; j < 4; ++j)
 #pragma unroll
         for (int e = 0; e < 4; ++e) {
-            sc[j][e] = exp2f(sc[j][e] - m[e & 1]);
+            sc[j][e] = tc::ex2(sc[j][e] - m[e & 1]);
             l[e & 1] += sc[j][e];
         }
 }
 
-// grid, shared memory, partial, CLUSTER: as for decode_stream_bf16.  Warps 0-2 score, warp 3 is the producer, warps 4 + 4 w ..
-// 7 + 4 w are the sum warps of team w.
+// grid, shared memory, partial, CLUSTER: as for decode_stream_bf16.  Warps 0 .. TEAMS - 1 score, the next one is the producer, then
+// come the sum warps, team by team.
 template <int D, bool CLUSTER>
 __global__ void __launch_bounds__(Cfg<D, true>::THREADS, 1)
 decode_stream_rope(const __nv_bfloat16* __restrict__ q, const __grid_constant__ Maps maps, Plan pl, int n_ret, int n_apx, int g,
@@ -100,8 +101,8 @@ decode_stream_rope(const __nv_bfloat16* __restrict__ q, const __grid_constant__ 
                    const int32_t* __restrict__ apx_pos, long long cap_apx, const __grid_constant__ RopePhases rope,
                    const __nv_bfloat16* __restrict__ W, void* __restrict__ out, int out_f32) {
     using C = Cfg<D, true>;
-    constexpr int HALF_BYTES = C::HALF_BYTES, SLOT_BYTES = C::SLOT_BYTES, SLOTS = C::SLOTS, TEAMS = C::CONSUMER_WARPS;
-    constexpr int REC = C::REC, CREC = C::CREC, PAIRS = D / 64;               // column tiles of 8 channel pairs of a sum warp
+    constexpr int HALF_BYTES = C::HALF_BYTES, SLOT_BYTES = C::SLOT_BYTES, SLOTS = C::SLOTS, TEAMS = C::CONSUMER_WARPS, SUM_WARPS = C::SUM_WARPS;
+    constexpr int REC = C::REC, CREC = C::CREC, PAIRS = 2;                    // column tiles of 8 channel pairs of a sum warp
     extern __shared__ unsigned char smem_raw[];
     __shared__ __align__(8) uint64_t full_bar[SLOTS], empty_bar[SLOTS];
     __shared__ __align__(8) uint64_t step_full[TEAMS][2], step_empty[TEAMS][2];
@@ -260,11 +261,9 @@ decode_stream_rope(const __nv_bfloat16* __restrict__ q, const __grid_constant__ 
                 *reinterpret_cast<float2*>(dst + x * (D / 2) + 8 * (PAIRS * part + p) + 2 * tig) =
                     make_float2(acc[x][p][0] + acc[x][p][2], acc[x][p][1] + acc[x][p][3]);
     };
-    // Where a lane's rows of its column tiles lie within 16 rows at a multiple of 16 (ldmatrix.trans, swizzled).  128 channels:
-    // matrices (tile | tile + 1) x (rows 0-7 | 8-15), the partner channels one box further; 64 channels: the partner
-    // tiles take the place of tile + 1.
-    const uint32_t frag = (uint32_t)(r8 + (mat & 1) * 8) * 128u +
-                          (uint32_t)(((D == 128 ? 2 * part + (mat >> 1) : part + 4 * (mat >> 1)) ^ r8) << 4);
+    // Where a lane's rows of its column tiles lie within 16 rows at a multiple of 16 (ldmatrix.trans, swizzled): matrices
+    // (tile | tile + 1) x (rows 0-7 | 8-15), the partner channels one box further, or half a row at 64 channels.
+    const uint32_t frag = (uint32_t)(r8 + (mat & 1) * 8) * 128u + (uint32_t)(((2 * part + (mat >> 1)) ^ r8) << 4);
     zero_acc();
     for (int u = u0; u <= u_last; ++u) {
         const long long unit_end = (long long)(u + 1) * pl.n_tiles - gt_lo;
@@ -299,12 +298,8 @@ decode_stream_rope(const __nv_bfloat16* __restrict__ q, const __grid_constant__ 
                     uint32_t a[4], rx[PAIRS][2], ry[PAIRS][2];            // B fragments: low and high channels, rows 0-7 | 8-15
                     ldsm_x4(st + kk * 512 + lane * 16, a[0], a[1], a[2], a[3]);
                     const uint32_t at = base + kk * 16 * 128;
-                    if constexpr (D == 128) {
-                        ldsm_x4_t(at, rx[0][0], rx[0][1], rx[1][0], rx[1][1]);
-                        ldsm_x4_t(at + BOX_BYTES, ry[0][0], ry[0][1], ry[1][0], ry[1][1]);
-                    } else {
-                        ldsm_x4_t(at, rx[0][0], rx[0][1], ry[0][0], ry[0][1]);
-                    }
+                    ldsm_x4_t(at, rx[0][0], rx[0][1], rx[1][0], rx[1][1]);
+                    ldsm_x4_t(D == 128 ? at + BOX_BYTES : at ^ 64u, ry[0][0], ry[0][1], ry[1][0], ry[1][1]);
                     if (retained) {
 #pragma unroll
                         for (int p = 0; p < PAIRS; ++p) {
