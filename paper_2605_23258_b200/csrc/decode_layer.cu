@@ -236,21 +236,13 @@ static vector_status launch_layer_mma(const Dims& dm, int L, const void* q, cons
     using T = __nv_bfloat16;
     static PerDeviceOnce once;
     if (once.first()) {
-        const cudaError_t e = cudaFuncSetAttribute(dlm::decode_layer_mma, cudaFuncAttributeMaxDynamicSharedMemorySize, dlm::SMEM_BYTES);
+        cudaError_t e = cudaFuncSetAttribute(dlm::decode_layer_mma, cudaFuncAttributeMaxDynamicSharedMemorySize, dlm::SMEM_BYTES);
+        if (e == cudaSuccess) e = cudaFuncSetAttribute(dlm::decode_layer_merge_mma<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, dlm::MERGE_PAD);
+        if (e == cudaSuccess) e = cudaFuncSetAttribute(dlm::decode_layer_merge_mma<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, dlm::MERGE_PAD);
         if (e != cudaSuccess) { once.undo(); VEC_CUDA_CHECK(e); }
     }
     const int UL = dm.U / dlm::HKV;
-    const int64_t tiles = (ch->n_ret + dlm::RT - 1) / dlm::RT + (ch->n_apx + dlm::AT - 1) / dlm::AT;
-    // Splits: a multiprocessor holds one block, so the time goes with whole rounds of blocks over the splits' number; a block
-    // costs about eight retained tiles besides: its first loads, its records (four to fourteen counted make no difference from 2000 to
-    // 100000 tokens; with none counted, 32 layers of 7200 rows took a tenth longer).
-    const double cost = dlm::RET_COST * (double)((ch->n_ret + dlm::RT - 1) / dlm::RT) + dlm::APX_COST * (double)((ch->n_apx + dlm::AT - 1) / dlm::AT);
-    int64_t n_splits = 1;
-    double best = 1e300;
-    for (int64_t n = 1; n <= 32 && n <= tiles; ++n) {
-        const double t = (double)((n * UL + sm_count() - 1) / sm_count()) * (cost / (double)n + 8.0);
-        if (t < best - 1e-9) { best = t; n_splits = n; }
-    }
+    const dlm::Plan pl = dlm::make_plan(UL, ch->n_ret, ch->n_apx, sm_count());
     int* fault = kernel_fault_address();
     if (!fault) return VECTOR_ERR_CUDA;
     dbf::Maps maps;
@@ -264,14 +256,18 @@ static vector_status launch_layer_mma(const Dims& dm, int L, const void* q, cons
     if (!ok) return VECTOR_ERR_CUDA;
     if (ch->n_ret == 0) { maps.ret_k = maps.apx_k; maps.ret_v = maps.apx_k; }   // never dereferenced: no such tiles
     if (ch->n_apx == 0) maps.apx_k = maps.ret_k;
-    VEC_CUDA_CHECK(launch_maybe_dependent(true, dlm::decode_layer_mma, dim3((unsigned)n_splits, UL), dim3(dlm::THREADS), dlm::SMEM_BYTES, st,
-        (const T*)q, maps, (int)ch->n_ret, (int)ch->n_apx, dm.g, dm.scale * 1.4426950408889634f, partial, fault));
+    VEC_CUDA_CHECK(launch_maybe_dependent(true, dlm::decode_layer_mma, dim3((unsigned)pl.B), dim3(dlm::THREADS), dlm::SMEM_BYTES, st,
+        (const T*)q, maps, pl, (int)ch->n_ret, (int)ch->n_apx, dm.g, dm.scale * 1.4426950408889634f, partial, fault));
+    // The merge's blocks start while the streaming kernel's last ones run, three to each multiprocessor that is free by then:
+    // shared memory that nobody uses keeps them to one or two when that is enough for all of them.  Measured so and with three to
+    // a multiprocessor, us a step in a graph: 32 pairs of 600 rows 38 / 43, of 7200 rows 133 / 140; 16 of 4900 rows 62 / 76.
+    const size_t pad = dm.U <= sm_count() ? dlm::MERGE_PAD : dm.U <= 2 * sm_count() ? dlm::MERGE_PAD / 2 : 0;
     if (out_dtype == VECTOR_F32)
-        VEC_CUDA_CHECK(launch_maybe_dependent(true, dlm::decode_layer_merge_mma<float>, dim3(dm.U), dim3(dlm::MERGE_THREADS), 0, st, partial,
-                                              (const T*)W, L, dm.g, (int)n_splits, (float*)out));
+        VEC_CUDA_CHECK(launch_maybe_dependent(true, dlm::decode_layer_merge_mma<float>, dim3(dm.U), dim3(dlm::MERGE_THREADS), pad, st, partial,
+                                              (const T*)W, L, dm.g, pl, (float*)out));
     else
-        VEC_CUDA_CHECK(launch_maybe_dependent(true, dlm::decode_layer_merge_mma<T>, dim3(dm.U), dim3(dlm::MERGE_THREADS), 0, st, partial,
-                                              (const T*)W, L, dm.g, (int)n_splits, (T*)out));
+        VEC_CUDA_CHECK(launch_maybe_dependent(true, dlm::decode_layer_merge_mma<T>, dim3(dm.U), dim3(dlm::MERGE_THREADS), pad, st, partial,
+                                              (const T*)W, L, dm.g, pl, (T*)out));
     return VECTOR_OK;
 }
 

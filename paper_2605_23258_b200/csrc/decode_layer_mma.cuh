@@ -15,9 +15,11 @@
 // Phase 1 is a chain of dependent MMAs, shuffles and exponentials, phase 2 a run of independent MMAs: with two warps to a
 // scheduler neither hides the other's latency unless they are the same warp's instructions.  So phase 1 of tile t + 1 is
 // laid between the MMAs of phase 2 of tile t, one barrier a tile; the third stage is the tile in flight meanwhile.
+// The tiles of all (sequence, layer) pairs form one row, dealt in equal contiguous pieces to persistent blocks (Plan).
 // What bounds it: the warps' own instructions -- tensor pipe 41 % busy, HBM 0.74 of a copy's rate in the streaming
-// kernel -- with eight warps, whose accumulators leave no room for more.  Measured, 32 layers of 7200 rows, 630 MB, in a
-// graph: 144 us; 173 with tiles copied in 16-byte pieces by all threads, 210 with the two phases one after the other.
+// kernel -- with eight warps, whose accumulators leave no room for more.  Measured, 32 pairs of 7200 rows, 630 MB, in a
+// graph: 130 us; 143 with whole splits of a pair in two rounds of blocks, 173 with tiles copied in 16-byte pieces by all
+// threads, 210 with the two phases one after the other.
 // Records have the layout of the CUDA-core split kernel: per (unit, split, head) m, l, acc_v[128],
 // acc_k[8][128].
 #ifndef VECTOR_DECODE_LAYER_MMA_CUH_
@@ -50,9 +52,44 @@ constexpr int REC = 2 + 128 + HKV * 128;
 constexpr float SLACK = 8.f;
 // (tc::ex2 gives zero for results below 2^-126: next to a weight of at least 2^-SLACK they do not change an fp32 sum.)
 
-// grid (n_splits, U / 8), THREADS threads, SMEM_BYTES dynamic shared memory.
+// How the work is dealt: the (sequence, layer) pairs' tiles in one row, weighted by their cost, cut into B equal pieces, one
+// persistent block each.  A pair's records: one of every block that reaches into it.  The same arithmetic runs on host and device.
+struct Plan {
+    int n_rt, n_at, UL;        // retained / key-only tiles of a pair, pairs
+    int weight, B, s_max;      // cost of a pair, blocks, record slots of a pair
+};
+constexpr int MAX_RECORDS = 32;
+__host__ __device__ inline Plan make_plan(int UL, long long n_ret, long long n_apx, int max_blocks) {
+    Plan p;
+    p.UL = UL;
+    p.n_rt = (int)((n_ret + RT - 1) / RT);
+    p.n_at = (int)((n_apx + AT - 1) / AT);
+    p.weight = RET_COST * p.n_rt + APX_COST * p.n_at;
+    const long long total = (long long)UL * p.weight;
+    const auto limit = [](long long x, long long most) { return x < most ? x : most; };
+    long long b = limit(max_blocks, total / 4);                // two key-only tiles a block at the least
+    b = b < 1 ? 1 : b;
+    // The same number of blocks for every pair leaves some multiprocessors idle, but no block with the ends of two pairs; a
+    // record costs a block about eight retained tiles (its first loads, 147 KB written, and read again by the merge).  Measured in
+    // a graph, all multiprocessors against whole blocks a pair, us: 32 pairs of 600 rows 48 / 43, of 7200 rows 140 / 146; 16
+    // pairs of 4900 rows 80 / 76 (the merge three blocks to a multiprocessor in all of them).
+    if (b >= UL) {
+        const long long whole = b / UL * UL;
+        const long long reach = b == whole ? 1 : 2;            // pairs a block reaches into
+        if (total / whole + 8 <= total / b + 8 * reach) b = whole;
+    }
+    if (b > (long long)UL * (MAX_RECORDS - 2)) b = (long long)UL * limit(b / UL, MAX_RECORDS);
+    p.B = (int)b;
+    p.s_max = b % UL == 0 ? (int)(b / UL) : (int)(b / UL) + 2;      // a pair's share of the blocks begins and ends inside one
+    return p;
+}
+__host__ __device__ inline long long cost_begin(int b, const Plan& p) { return (long long)b * p.weight * p.UL / p.B; }
+__host__ __device__ inline int block_of_cost(long long x, const Plan& p) { return (int)(((x + 1) * p.B - 1) / ((long long)p.weight * p.UL)); }
+
+// grid (plan.B), THREADS threads, SMEM_BYTES dynamic shared memory.  partial: [U][s_max][g][REC]; slot of (pair, block b) =
+// b - block_of_cost(first cost of the pair).
 __global__ void __launch_bounds__(THREADS, 1)
-decode_layer_mma(const __nv_bfloat16* __restrict__ q, const __grid_constant__ dbf::Maps maps, int n_ret, int n_apx, int g,
+decode_layer_mma(const __nv_bfloat16* __restrict__ q, const __grid_constant__ dbf::Maps maps, Plan pl, int n_ret, int n_apx, int g,
                  float scale_log2e, float* __restrict__ partial, int* __restrict__ fault) {
     __shared__ __align__(8) uint64_t full_bar[STAGES];
     if (threadIdx.x == 0) {
@@ -65,61 +102,61 @@ decode_layer_mma(const __nv_bfloat16* __restrict__ q, const __grid_constant__ db
     unsigned char* const stage0 = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(lsm) + 1023) & ~uintptr_t(1023));
     unsigned char* const ps = stage0 + STAGES * STAGE_BYTES;
     const uint32_t dump = tma::smem_u32(ps + 2 * P_BYTES);      // where the rows of absent heads go
-    const int split = blockIdx.x, n_splits = gridDim.x, ul = blockIdx.y;
     const int tid = threadIdx.x, lane = tid & 31, h = tid >> 5;
     const int gid = lane >> 2, tig = lane & 3, mat = lane >> 3, r8 = lane & 7;
-    const int n_rt = (n_ret + RT - 1) / RT, n_at = (n_apx + AT - 1) / AT;
-    // A key-only tile takes 192 MMAs a warp, a retained one 64 (both bring in 64 KB): the slices are equal in time, not in tiles.
-    const long long weight = (long long)RET_COST * n_rt + (long long)APX_COST * n_at;
-    auto tile_at = [&](long long x) -> int {          // first tile that begins at or after x
-        return x <= (long long)RET_COST * n_rt ? (int)((x + RET_COST - 1) / RET_COST)
-                                               : n_rt + (int)((x - (long long)RET_COST * n_rt + APX_COST - 1) / APX_COST);
+    const int b = blockIdx.x, n_rt = pl.n_rt, n_tiles = pl.n_rt + pl.n_at;
+    // A key-only tile takes 144 MMAs a warp, a retained one 24 (both bring in 64 KB): the pieces are equal in time, not in tiles.
+    auto tile_at = [&](int x) -> int {                // first tile of a pair that begins at or after x
+        return x <= RET_COST * n_rt ? (x + RET_COST - 1) / RET_COST : n_rt + (x - RET_COST * n_rt + APX_COST - 1) / APX_COST;
     };
-    const int t_lo = tile_at(weight * split / n_splits), t_hi = tile_at(weight * (split + 1) / n_splits);
-    const size_t u = (size_t)ul * HKV + h;
+    const long long c_lo = cost_begin(b, pl), c_hi = cost_begin(b + 1, pl);           // never empty
+    const int u_first = (int)(c_lo / pl.weight), u_last = (int)((c_hi - 1) / pl.weight);
+    const int first_lo = tile_at((int)(c_lo - (long long)u_first * pl.weight)), last_hi = tile_at((int)(c_hi - (long long)u_last * pl.weight));
 
     for (int i = tid; i < 2 * P_BYTES / 4; i += THREADS) reinterpret_cast<uint32_t*>(ps)[i] = 0u;
-    // the g query rows of this head as B fragments (columns g .. 7 zero)
-    uint32_t qa[8][2];
-    {
-        const uint32_t* qrow = reinterpret_cast<const uint32_t*>(q + (u * g + min(gid, g - 1)) * 128);
-#pragma unroll
-        for (int ks = 0; ks < 8; ++ks) {
-            qa[ks][0] = gid < g ? qrow[ks * 8 + tig] : 0u;
-            qa[ks][1] = gid < g ? qrow[ks * 8 + 4 + tig] : 0u;
-        }
-    }
+    uint32_t qa[8][2];                             // the g query rows of this head as B fragments (columns g .. 7 zero)
     float acc_k[2][16][4], acc_v[8][4];            // acc_v[n]: dims 16 n + gid (, + 8) of heads 2 tig, + 1
+    auto zero_acc = [&]() {
 #pragma unroll
-    for (int n = 0; n < 16; ++n) {
-        if (n < 8) acc_v[n][0] = acc_v[n][1] = acc_v[n][2] = acc_v[n][3] = 0.f;
+        for (int n = 0; n < 16; ++n) {
+            if (n < 8) acc_v[n][0] = acc_v[n][1] = acc_v[n][2] = acc_v[n][3] = 0.f;
 #pragma unroll
-        for (int mt = 0; mt < 2; ++mt) acc_k[mt][n][0] = acc_k[mt][n][1] = acc_k[mt][n][2] = acc_k[mt][n][3] = 0.f;
-    }
+            for (int mt = 0; mt < 2; ++mt) acc_k[mt][n][0] = acc_k[mt][n][1] = acc_k[mt][n][2] = acc_k[mt][n][3] = 0.f;
+        }
+    };
+    zero_acc();
     float m[2] = {-INFINITY, -INFINITY}, l[2] = {0.f, 0.f};       // of heads 2 tig, + 1; l: this lane's tokens only
 
     bool ok = true;                            // false once a wait gave up: walk on and touch nothing
-    // One thread requests a tile; rows past the pool's end are filled with zeros.
+    // One thread requests tile t of pair u, or as many tiles into the following pairs as t lies past its end, into stage sg;
+    // rows past the pool's end are filled with zeros.
     const uint64_t pol = tma::policy_evict_first();                 // the cache is read once per step
-    auto prefetch = [&](int t) {
-        if (tid == 0 && t < t_hi && ok) {
-            unsigned char* st = stage0 + ((t - t_lo) % STAGES) * STAGE_BYTES;
-            uint64_t* bar = &full_bar[(t - t_lo) % STAGES];
-            tma::mbar_expect_tx(bar, STAGE_BYTES);
+    auto request = [&](int u, int t, int sg) {
+        if (tid == 0 && ok) {
+            while (u <= u_last && t >= (u == u_last ? last_hi : n_tiles)) {
+                t -= u == u_last ? last_hi : n_tiles;
+                ++u;
+            }
+            if (u <= u_last) {
+                unsigned char* st = stage0 + sg * STAGE_BYTES;
+                tma::mbar_expect_tx(&full_bar[sg], STAGE_BYTES);
 #pragma unroll
-            for (int x = 0; x < 2; ++x) {
-                if (t < n_rt) {
-                    tma::load_3d_hint(st + x * BOX_RET, &maps.ret_k, 64 * x, t * RT, ul * HKV, bar, pol);
-                    tma::load_3d_hint(st + 32768 + x * BOX_RET, &maps.ret_v, 64 * x, t * RT, ul * HKV, bar, pol);
-                } else {
-                    tma::load_3d_hint(st + x * BOX_APX, &maps.apx_k, 64 * x, (t - n_rt) * AT, ul * HKV, bar, pol);
+                for (int x = 0; x < 2; ++x) {
+                    if (t < n_rt) {
+                        tma::load_3d_hint(st + x * BOX_RET, &maps.ret_k, 64 * x, t * RT, u * HKV, &full_bar[sg], pol);
+                        tma::load_3d_hint(st + 32768 + x * BOX_RET, &maps.ret_v, 64 * x, t * RT, u * HKV, &full_bar[sg], pol);
+                    } else {
+                        tma::load_3d_hint(st + x * BOX_APX, &maps.apx_k, 64 * x, (t - n_rt) * AT, u * HKV, &full_bar[sg], pol);
+                    }
                 }
             }
         }
         __syncwarp();
     };
+    // Tile t of the pair at hand is tile t + off of the block's piece.
+    int off = 0;
     auto landed = [&](int t) {
-        if (ok && t < t_hi) ok = tma::mbar_wait_warp(&full_bar[(t - t_lo) % STAGES], ((t - t_lo) / STAGES) & 1, fault, 2);
+        if (ok) ok = tma::mbar_wait_warp(&full_bar[(t + off) % STAGES], ((t + off) / STAGES) & 1, fault, 2);
     };
 
     // State of a tile between its two phases: the factors of heads 2 tig, + 1 and, retained, P as B fragments.
@@ -129,7 +166,7 @@ decode_layer_mma(const __nv_bfloat16* __restrict__ q, const __grid_constant__ db
     // XORed by c % 4 (the swizzle), in box c / 4
     const uint32_t frag = (uint32_t)((r8 + (mat & 1) * 8) * 128 + (((mat >> 1) ^ r8) << 4));
     auto chunk = [](uint32_t base, int c, uint32_t box) { return (base ^ (uint32_t)((c & 3) << 5)) + (c >> 2) * box; };
-    auto stage_of = [&](int t) { return tma::smem_u32(stage0 + ((t - t_lo) % STAGES) * STAGE_BYTES); };
+    auto stage_of = [&](int t) { return tma::smem_u32(stage0 + ((t + off) % STAGES) * STAGE_BYTES); };
     // logits, k step `item / J` of the 16 tokens `item % J`, J = 1 (retained) or 2
     auto logit_item = [&](uint32_t kbase, int item, int J) {
         const int ks = item / J, j = item % J;
@@ -162,7 +199,7 @@ decode_layer_mma(const __nv_bfloat16* __restrict__ q, const __grid_constant__ db
             m[e] = m_new;
             l[e] *= al[e];
         }
-        unsigned char* const pb = ps + (t & 1) * P_BYTES;
+        unsigned char* const pb = ps + ((t + off) & 1) * P_BYTES;
 #pragma unroll
         for (int j = 0; j < J; ++j) {
             uint32_t hi[2], lo[2];                         // tokens gid and gid + 8 of the 16
@@ -196,7 +233,7 @@ decode_layer_mma(const __nv_bfloat16* __restrict__ q, const __grid_constant__ db
         constexpr int NEXT = decltype(next)::value, J = NEXT == 1 ? 1 : 2, ITEMS = NEXT == 0 ? 0 : 8 * J;
         const uint32_t st = stage_of(t) + frag, kn = stage_of(t + 1) + frag + h * (NEXT == 1 ? HEAD_RET : HEAD_APX);
         if (changed) {
-            const float* f = reinterpret_cast<const float*>(ps + (t & 1) * P_BYTES + 2 * MQ * PS_ROW);
+            const float* f = reinterpret_cast<const float*>(ps + ((t + off) & 1) * P_BYTES + 2 * MQ * PS_ROW);
 #pragma unroll
             for (int mt = 0; mt < 2; ++mt) {
                 const float f0 = f[16 * mt + gid], f1 = f[16 * mt + 8 + gid];
@@ -233,7 +270,7 @@ decode_layer_mma(const __nv_bfloat16* __restrict__ q, const __grid_constant__ db
         } else {
             // key sums over head h (= this warp) for all query heads of the layer: P[32 x 32] K_h[32 x 128]
             const uint32_t kbase = st + h * HEAD_APX;
-            const uint32_t ph = tma::smem_u32(ps + (t & 1) * P_BYTES) + (uint32_t)((r8 + (mat & 1) * 8) * PS_ROW + (mat >> 1) * 16);
+            const uint32_t ph = tma::smem_u32(ps + ((t + off) & 1) * P_BYTES) + (uint32_t)((r8 + (mat & 1) * 8) * PS_ROW + (mat >> 1) * 16);
 #pragma unroll
             for (int kk = 0; kk < 2; ++kk) {
 #pragma unroll
@@ -268,58 +305,77 @@ decode_layer_mma(const __nv_bfloat16* __restrict__ q, const __grid_constant__ db
     using NextApx = std::integral_constant<int, 2>;
 
     __syncthreads();                           // the barriers, P and the factors are initialised
-    prefetch(t_lo);
-    prefetch(t_lo + 1);
-    landed(t_lo);
-    if (t_lo < t_hi && ok) {
+    request(u_first, first_lo, 0);
+    request(u_first, first_lo + 1, 1);
+    for (int ul = u_first; ul <= u_last; ++ul) {
+        const int t_lo = ul == u_first ? first_lo : 0, t_hi = ul == u_last ? last_hi : n_tiles;
+        const size_t u = (size_t)ul * HKV + h;
+        off -= t_lo;
+        if (t_lo < t_hi) {
+            const uint32_t* qrow = reinterpret_cast<const uint32_t*>(q + (u * g + min(gid, g - 1)) * 128);
 #pragma unroll
-        for (int j = 0; j < 2; ++j) sc[j][0] = sc[j][1] = sc[j][2] = sc[j][3] = 0.f;
-        if (t_lo < n_rt) {
+            for (int ks = 0; ks < 8; ++ks) {
+                qa[ks][0] = gid < g ? qrow[ks * 8 + tig] : 0u;
+                qa[ks][1] = gid < g ? qrow[ks * 8 + 4 + tig] : 0u;
+            }
+            landed(t_lo);
+            if (ok) {
 #pragma unroll
-            for (int it = 0; it < 8; ++it) logit_item(stage_of(t_lo) + frag + h * HEAD_RET, it, 1);
-            softmax(Ret{}, t_lo, alpha, bp);
-        } else {
+                for (int j = 0; j < 2; ++j) sc[j][0] = sc[j][1] = sc[j][2] = sc[j][3] = 0.f;
+                if (t_lo < n_rt) {
 #pragma unroll
-            for (int it = 0; it < 16; ++it) logit_item(stage_of(t_lo) + frag + h * HEAD_APX, it, 2);
-            softmax(Apx{}, t_lo, alpha, bp);
-        }
-    }
-    for (int t = t_lo; t < t_hi; ++t) {
-        // P and the factors of tile t are written; everyone is done with tile t - 1, whose stage tile t + 2 takes
-        const int changed = __syncthreads_or((2 * tig < g && alpha[0] != 1.f) || (2 * tig + 1 < g && alpha[1] != 1.f));
-        prefetch(t + 2);
-        landed(t + 1);
-        if (!ok) continue;
-        if (t + 1 == t_hi) { if (t < n_rt) interval(Ret{}, None{}, t, changed); else interval(Apx{}, None{}, t, changed); }
-        else if (t + 1 < n_rt) interval(Ret{}, NextRet{}, t, changed);
-        else if (t < n_rt) interval(Ret{}, NextApx{}, t, changed);
-        else interval(Apx{}, NextApx{}, t, changed);
-    }
-    // ---- records.  Warp h: m, l and sum p v of its own query rows; every warp: its head's key sums for all rows
+                    for (int it = 0; it < 8; ++it) logit_item(stage_of(t_lo) + frag + h * HEAD_RET, it, 1);
+                    softmax(Ret{}, t_lo, alpha, bp);
+                } else {
 #pragma unroll
-    for (int e = 0; e < 2; ++e) {
-#pragma unroll
-        for (int o = 4; o < 32; o <<= 1) l[e] += __shfl_xor_sync(0xffffffffu, l[e], o);
-        if (2 * tig + e < g) {
-            float* rec = partial + ((u * n_splits + split) * g + 2 * tig + e) * REC;
-            if (gid == 0) { rec[0] = m[e] * 0.69314718055994531f; rec[1] = l[e]; }
-#pragma unroll
-            for (int n = 0; n < 8; ++n) { rec[2 + 16 * n + gid] = acc_v[n][e]; rec[2 + 16 * n + 8 + gid] = acc_v[n][2 + e]; }
-        }
-    }
-    const int n_q = HKV * g;
-#pragma unroll
-    for (int mt = 0; mt < 2; ++mt) {
-#pragma unroll
-        for (int half = 0; half < 2; ++half) {
-            const int a = 16 * mt + 8 * half + gid;                 // query head of the layer
-            if (a < n_q) {
-                float* rec = partial + ((((size_t)ul * HKV + a / g) * n_splits + split) * g + a % g) * REC + 2 + 128 + h * 128;
-#pragma unroll
-                for (int n = 0; n < 16; ++n)
-                    *reinterpret_cast<float2*>(rec + n * 8 + 2 * tig) = make_float2(acc_k[mt][n][2 * half], acc_k[mt][n][2 * half + 1]);
+                    for (int it = 0; it < 16; ++it) logit_item(stage_of(t_lo) + frag + h * HEAD_APX, it, 2);
+                    softmax(Apx{}, t_lo, alpha, bp);
+                }
             }
         }
+        for (int t = t_lo; t < t_hi; ++t) {
+            // P and the factors of tile t are written; everyone is done with the tile before it, whose stage is the next to fill
+            const int changed = __syncthreads_or((2 * tig < g && alpha[0] != 1.f) || (2 * tig + 1 < g && alpha[1] != 1.f));
+            request(ul, t + 2, (t + 2 + off) % STAGES);
+            if (t + 1 < t_hi) landed(t + 1);
+            if (!ok) continue;
+            if (t + 1 == t_hi) { if (t < n_rt) interval(Ret{}, None{}, t, changed); else interval(Apx{}, None{}, t, changed); }
+            else if (t + 1 < n_rt) interval(Ret{}, NextRet{}, t, changed);
+            else if (t < n_rt) interval(Ret{}, NextApx{}, t, changed);
+            else interval(Apx{}, NextApx{}, t, changed);
+        }
+        off += t_hi;
+        int slot = b - block_of_cost((long long)ul * pl.weight, pl);
+        if (slot < 0 || slot >= pl.s_max) { atomicCAS(fault, 0, 5); slot = 0; }     // cannot happen; never write out of bounds
+        // ---- records.  Warp h: m, l and sum p v of its own query rows; every warp: its head's key sums for all rows
+#pragma unroll
+        for (int e = 0; e < 2; ++e) {
+#pragma unroll
+            for (int o = 4; o < 32; o <<= 1) l[e] += __shfl_xor_sync(0xffffffffu, l[e], o);
+            if (2 * tig + e < g) {
+                float* rec = partial + ((u * pl.s_max + slot) * g + 2 * tig + e) * REC;
+                if (gid == 0) { rec[0] = m[e] * 0.69314718055994531f; rec[1] = l[e]; }
+#pragma unroll
+                for (int n = 0; n < 8; ++n) { rec[2 + 16 * n + gid] = acc_v[n][e]; rec[2 + 16 * n + 8 + gid] = acc_v[n][2 + e]; }
+            }
+        }
+        const int n_q = HKV * g;
+#pragma unroll
+        for (int mt = 0; mt < 2; ++mt) {
+#pragma unroll
+            for (int half = 0; half < 2; ++half) {
+                const int a = 16 * mt + 8 * half + gid;                 // query head of the layer
+                if (a < n_q) {
+                    float* rec = partial + ((((size_t)ul * HKV + a / g) * pl.s_max + slot) * g + a % g) * REC + 2 + 128 + h * 128;
+#pragma unroll
+                    for (int n = 0; n < 16; ++n)
+                        *reinterpret_cast<float2*>(rec + n * 8 + 2 * tig) = make_float2(acc_k[mt][n][2 * half], acc_k[mt][n][2 * half + 1]);
+                }
+            }
+        }
+        zero_acc();
+        m[0] = m[1] = -INFINITY;
+        l[0] = l[1] = 0.f;
     }
 }
 
@@ -332,10 +388,10 @@ decode_layer_mma(const __nv_bfloat16* __restrict__ q, const __grid_constant__ db
 // 128-column block, the k slots of an MMA step follow that order in both operands), the key sums as bf16
 // hi + lo in shared memory.  What it costs is memory latency (42 MB of records and 64 MB of map from L2 over 256 blocks):
 // hence eight-byte loads with eight splits of two elements in flight, and 16 warps on the map's rows.
-constexpr int MERGE_THREADS = 512;
+constexpr int MERGE_THREADS = 512, MERGE_PAD = 72 * 1024;     // + 46 KB of its own: one block to a multiprocessor, with half of it two
 template <typename TO>
 __global__ void __launch_bounds__(MERGE_THREADS)
-decode_layer_merge_mma(const float* __restrict__ partial, const __nv_bfloat16* __restrict__ W, int L, int g, int n_splits,
+decode_layer_merge_mma(const float* __restrict__ partial, const __nv_bfloat16* __restrict__ W, int L, int g, Plan pl,
                        TO* __restrict__ out) {
     constexpr int KD = HKV * 128;
     __shared__ __align__(16) __nv_bfloat16 akh[8][KD], akl[8][KD];          // 32 KB
@@ -343,12 +399,14 @@ decode_layer_merge_mma(const float* __restrict__ partial, const __nv_bfloat16* _
     const int u = blockIdx.x, tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
     const int h = u % HKV, layer = (u / HKV) % L;
     const int row = lane >> 2, quarter = lane & 3;
-    const float* rec0 = partial + (size_t)u * n_splits * g * REC;
+    const float* rec0 = partial + (size_t)u * pl.s_max * g * REC;
+    const long long c0 = (long long)(u / HKV) * pl.weight;
+    const int n_splits = block_of_cost(c0 + pl.weight - 1, pl) - block_of_cost(c0, pl) + 1;
     for (int i = tid; i < (8 - g) * KD; i += MERGE_THREADS) {            // columns of B beyond the unit's heads
         akh[g + i / KD][i % KD] = __float2bfloat16_rn(0.f);
         akl[g + i / KD][i % KD] = __float2bfloat16_rn(0.f);
     }
-    asm volatile("griddepcontrol.wait;\n" ::: "memory");                 // the split kernel's records
+    asm volatile("griddepcontrol.wait;\n" ::: "memory");                 // the streaming kernel's records
     // factors of the splits: warp a < g takes head a
     if (wid < g) {
         const float mj = lane < n_splits ? rec0[((size_t)lane * g + wid) * REC] : -INFINITY;

@@ -1,6 +1,7 @@
 """Decode with a layer's map where the running maximum moves along the tokens: by little at a time, which leaves the
 softmax's reference behind, and by jumps, which move it; ragged ends of both pools, one pool alone, fewer tiles than
-stages.  Tolerance: 2e-2 absolute, as for the layer-map decode elsewhere."""
+stages; and where a block's share of the tiles begins and ends inside a (sequence, layer) pair.  Tolerance: 2e-2
+absolute, as for the layer-map decode elsewhere."""
 import numpy as np
 import pytest
 import torch
@@ -9,6 +10,16 @@ import paper_2605_23258_b200 as vec
 
 pytestmark = pytest.mark.gpu
 DEV = "cuda"
+
+
+@pytest.mark.parametrize("L,B,g,n_ret,n_apx,jump", [
+    (10, 10, 4, 100, 700, 0.0),                  # fewer pairs than multiprocessors, blocks across their ends
+    (40, 4, 1, 17, 33, 0.0),                     # more pairs than multiprocessors, four tiles each
+    (19, 8, 2, 0, 130, 20.0),
+    (3, 1, 4, 1600, 3300, 0.0),                  # 49 blocks' worth a pair: the limit of records
+])
+def test_decode_layer_pieces(oracle, L, B, g, n_ret, n_apx, jump):
+    _check(oracle, L, B, g, n_ret, n_apx, jump)
 
 
 @pytest.mark.parametrize("g,n_ret,n_apx,jump", [
@@ -20,7 +31,11 @@ DEV = "cuda"
     (4, 17, 33, 0.0),                        # four tiles
 ])
 def test_decode_layer_growth(oracle, g, n_ret, n_apx, jump):
-    Hkv, d, L, B = 8, 128, 2, 2
+    _check(oracle, 2, 2, g, n_ret, n_apx, jump)
+
+
+def _check(oracle, L, B, g, n_ret, n_apx, jump):
+    Hkv, d = 8, 128
     UL, U = L * B, L * B * Hkv
     gen = torch.Generator(device=DEV).manual_seed(n_ret + n_apx)
     q = torch.randn(U, g, d, generator=gen, device=DEV)
@@ -42,7 +57,7 @@ def test_decode_layer_growth(oracle, g, n_ret, n_apx, jump):
     vec.vector_decode_attn_layer(sh, q, cache, W, out, ws)
     torch.cuda.synchronize()
     assert vec.vector_device_fault() == 0
-    for ul in range(UL):
+    for ul in sorted({*range(0, UL, max(1, UL // 5)), UL - 1}):
         sl = slice(ul * Hkv, (ul + 1) * Hkv)
         _, o = oracle.attend_layer(q[sl].reshape(Hkv * g, d).cpu(), rk[sl, :n_ret].cpu(), rv[sl, :n_ret].cpu(), ak[sl, :n_apx].cpu(),
                                    W[ul % L].cpu(), 1.0 / np.sqrt(d))
