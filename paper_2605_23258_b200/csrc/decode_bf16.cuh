@@ -18,7 +18,8 @@
 //   online softmax in fp32 registers, one rescale per 64 keys (exp2, scale folded in)
 //   O += P V  (retained tile)  or  A += P K  (key-only tile: the p-weighted key
 //             sum that the merge step multiplies by W); P enters as bf16 hi in
-//             MMA rows 0-7 and bf16 lo in rows 8-15, one MMA for both parts
+//             MMA rows 0-7 and bf16 lo in rows 8-15, one MMA for both parts; at head_dim 64
+//             a third part keeps all 24 bits of a weight (Cfg::PARTS)
 // A warp keeps one running state (m, l, O or A) per unit and writes it as its
 // partial record when it leaves the unit; a warp that met no tile of a unit the
 // block touches writes an empty record.  The merge kernel combines a unit's
@@ -50,10 +51,18 @@ constexpr int BOX_BYTES = 8192;              // 64 rows x 128 bytes
 constexpr float SLACK = 8.f;
 template <int D, bool ROPE> struct Cfg {
     static constexpr int HALF_BYTES = 64 * 2 * D;                    // 64 rows as D / 64 swizzled boxes
+    // 64 channels: everything to fp32's own precision, as CUDA cores give it.  A softmax weight enters as three bf16 parts, which
+    // keep its 24 bits (two keep sixteen); an MMA cuts its sums off instead of rounding them, so that the sums of
+    // 32 rows start at zero and are added up in fp32; the map is applied to the key sums in fp32.  With up to
+    // four heads the third parts take MMA rows that nobody else uses.  Error of an fp32 output against
+    // fp64, median over the heads of eight sizes of 1 to 64 layers, 8 to 512 units and up to 78642 rows: 1.0e-7 to 1.7e-7 (two parts, sums
+    // in the MMAs: 1.0e-6 to 2.2e-6; CUDA cores: 1.2e-7 to 4.4e-7).  512 units, 431 MB: 82 -> 87 us a step with the appended row.
+    static constexpr bool EXACT = D == 64;
+    static constexpr int PARTS = EXACT ? 3 : 2;
     static constexpr int SLOT_BYTES = 2 * HALF_BYTES;                // retained: K | V; key-only: keys 0-63 | keys 64-127
     // With 64-channel heads a softmax step brings in half the bytes for the same softmax arithmetic: a fourth consumer
     // warp (one to a warp scheduler) makes up for it.
-    // Measured: 512 units, 1639 retained + 3276 key-only rows, 431 MB: 82 us with the appended row = 5.3 TB/s (856 us on
+    // Measured: 512 units, 1639 retained + 3276 key-only rows, 431 MB: 87 us with the appended row = 5.0 TB/s (856 us on
     // CUDA cores).
     // With RoPE decoupling a consumer is a team (decode_rope.cuh): a score warp and some sum warps.
     // Four teams at 64 channels, of two sum warps with as many channel pairs each as the four have at 128.
@@ -191,15 +200,16 @@ __device__ __forceinline__ void produce(const Maps& maps, const Plan& pl, long l
         if (++t == pl.n_tiles) { t = 0; ++u; }
     }
 }
-// The g query heads of a unit as A fragments, rows g .. 7 zero.
+// The g query heads of a unit as A fragments, rows g .. 7 zero; twice: rows 4 .. 7 the same heads as rows 0 .. 3 (g <= 4).
 template <int D>
-__device__ __forceinline__ void load_queries(const __nv_bfloat16* __restrict__ q, int unit, int g, int lane, uint32_t (&qa)[D / 16][2]) {
-    const int gid = lane >> 2, tig = lane & 3;
-    const uint32_t* qrow = reinterpret_cast<const uint32_t*>(q + ((size_t)unit * g + min(gid, g - 1)) * D);
+__device__ __forceinline__ void load_queries(const __nv_bfloat16* __restrict__ q, int unit, int g, int lane, uint32_t (&qa)[D / 16][2],
+                                             bool twice) {
+    const int head = twice ? (lane >> 2) & 3 : lane >> 2, tig = lane & 3;
+    const uint32_t* qrow = reinterpret_cast<const uint32_t*>(q + ((size_t)unit * g + min(head, g - 1)) * D);
 #pragma unroll
     for (int ks = 0; ks < D / 16; ++ks) {
-        qa[ks][0] = gid < g ? qrow[ks * 8 + tig] : 0u;
-        qa[ks][1] = gid < g ? qrow[ks * 8 + 4 + tig] : 0u;
+        qa[ks][0] = head < g ? qrow[ks * 8 + tig] : 0u;
+        qa[ks][1] = head < g ? qrow[ks * 8 + 4 + tig] : 0u;
     }
 }
 // The weights of a softmax step over the 64 keys at kbase (D / 64 swizzled boxes), of which nrows >= 1 are valid: sc (this
@@ -251,19 +261,92 @@ __device__ __forceinline__ float score_step(uint32_t kbase, int nrows, float sca
     m = m_new;
     return alpha;
 }
-// The weights of keys 16 kk .. + 15 as an A fragment: hi in MMA rows 0-7, lo in rows 8-15.
-__device__ __forceinline__ void weights_bf16(const float (&sc)[8][2], int kk, uint32_t (&a)[4]) {
-    const float p00 = sc[2 * kk][0], p01 = sc[2 * kk][1], p10 = sc[2 * kk + 1][0], p11 = sc[2 * kk + 1][1];
-    const __nv_bfloat16 h00 = __float2bfloat16_rn(p00), h01 = __float2bfloat16_rn(p01);
-    const __nv_bfloat16 h10 = __float2bfloat16_rn(p10), h11 = __float2bfloat16_rn(p11);
-    a[0] = pack_bf16(__bfloat162float(h00), __bfloat162float(h01));
-    a[1] = pack_bf16(p00 - __bfloat162float(h00), p01 - __bfloat162float(h01));
-    a[2] = pack_bf16(__bfloat162float(h10), __bfloat162float(h11));
-    a[3] = pack_bf16(p10 - __bfloat162float(h10), p11 - __bfloat162float(h11));
+// The same for 64 channels, on packed pairs: all rows of an accumulator are kept, so that nothing is moved between the MMAs.
+__device__ __forceinline__ float score_step64(uint32_t kbase, int nrows, float scale_log2e, const uint32_t (&qa)[4][2], int lane,
+                                              float& m, float& l, float (&sc)[8][2]) {
+    const int tig = lane & 3, mat = lane >> 3, r8 = lane & 7;
+    const uint32_t row = (uint32_t)(r8 + (mat >> 1) * 8) * 128u, x = (uint32_t)(((mat & 1) ^ r8) << 4);
+    float s[8][4];
+#pragma unroll
+    for (int n = 0; n < 8; ++n) s[n][0] = s[n][1] = s[n][2] = s[n][3] = 0.f;
+#pragma unroll
+    for (int ks = 0; ks < 4; ++ks) {
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            uint32_t b0, b1, b2, b3;
+            ldsm_x4(kbase + j * 16 * 128 + row + ((2 * ks << 4) ^ x), b0, b1, b2, b3);
+            mma_16(s[2 * j], qa[ks][0], 0u, qa[ks][1], 0u, b0, b1);
+            mma_16(s[2 * j + 1], qa[ks][0], 0u, qa[ks][1], 0u, b2, b3);
+        }
+    }
+    const uint64_t c2 = tc::pack2(scale_log2e, scale_log2e);
+    uint64_t v[8];
+    float mx = -INFINITY;
+#pragma unroll
+    for (int n = 0; n < 8; ++n) {
+        v[n] = tc::mul2(tc::pack2(s[n][0], s[n][1]), c2);
+        tc::unpack2(v[n], sc[n][0], sc[n][1]);
+    }
+    if (nrows < KEYS) {
+#pragma unroll
+        for (int n = 0; n < 8; ++n) {
+            const int kc = n * 8 + 2 * tig;
+            if (kc >= nrows) sc[n][0] = -INFINITY;
+            if (kc + 1 >= nrows) sc[n][1] = -INFINITY;
+            v[n] = tc::pack2(sc[n][0], sc[n][1]);
+        }
+    }
+#pragma unroll
+    for (int n = 0; n < 8; ++n) mx = fmaxf(mx, fmaxf(sc[n][0], sc[n][1]));
+    mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 1));
+    mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 2));
+    const float m_new = mx > m + SLACK ? mx : m;      // finite: key 0 of the step is valid for every row
+    const float alpha = tc::ex2(m - m_new);           // 0 on the first step
+    const uint64_t neg = tc::pack2(-m_new, -m_new);
+    uint64_t ls[2] = {tc::pack2(0.f, 0.f), tc::pack2(0.f, 0.f)};
+#pragma unroll
+    for (int n = 0; n < 8; ++n) {
+        float a, b;
+        tc::unpack2(tc::add2(v[n], neg), a, b);
+        sc[n][0] = tc::ex2(a);
+        sc[n][1] = tc::ex2(b);
+        ls[n & 1] = tc::add2(ls[n & 1], tc::pack2(sc[n][0], sc[n][1]));
+    }
+    float l0, l1;
+    tc::unpack2(tc::add2(ls[0], ls[1]), l0, l1);
+    l = fmaf(l, alpha, l0 + l1);
+    m = m_new;
+    return alpha;
 }
-// acc += P x over rows 16 kk .. + 15 of the 64 rows at vbase: D / 8 column tiles of 8 dims.
+// A pair of weights as bf16 parts: what the rounding to the parts before leaves, rounded; three parts leave nothing.
+template <int PARTS>
+__device__ __forceinline__ void split_bf16(float p0, float p1, uint32_t (&part)[3]) {
+#pragma unroll
+    for (int i = 0; i < PARTS; ++i) {
+        part[i] = pack_bf16(p0, p1);
+        if (i + 1 < PARTS)
+            tc::unpack2(tc::fma2(tc::pack2(__uint_as_float(part[i] << 16), __uint_as_float(part[i] & 0xffff0000u)), tc::pack2(-1.f, -1.f),
+                                 tc::pack2(p0, p1)), p0, p1);
+    }
+}
+// The weights of keys 16 kk .. + 15 as an A fragment: first parts in MMA rows 0-7, second parts in rows 8-15.  Third parts:
+// of up to four heads (twice: this thread's head is gid & 3) in rows 4-7, else in a fragment of their own (rows 8-15, third).
+template <int PARTS>
+__device__ __forceinline__ void weights_bf16(const float (&sc)[8][2], int kk, bool twice, int gid, uint32_t (&a)[4], uint32_t (&third)[2]) {
+#pragma unroll
+    for (int x = 0; x < 2; ++x) {
+        uint32_t part[3];
+        split_bf16<PARTS>(sc[2 * kk + x][0], sc[2 * kk + x][1], part);
+        const bool upper = PARTS == 3 && twice && gid >= 4;
+        a[2 * x] = upper ? part[2] : part[0];
+        a[2 * x + 1] = upper ? 0u : part[1];
+        third[x] = PARTS == 3 ? part[2] : 0u;
+    }
+}
+// acc += P x over rows 16 kk .. + 15 of the 64 rows at vbase: D / 8 column tiles of 8 dims.  with_third: P has a third fragment.
 template <int D>
-__device__ __forceinline__ void accumulate_step(uint32_t vbase, int kk, const uint32_t (&a)[4], float (&acc)[D / 8][4], int lane) {
+__device__ __forceinline__ void accumulate_step(uint32_t vbase, int kk, const uint32_t (&a)[4], bool with_third, const uint32_t (&third)[2],
+                                                float (&acc)[D / 8][4], int lane) {
     const int mat = lane >> 3, r8 = lane & 7;             // matrices = (chunk lo|hi) x (rows 0-7|8-15)
     const uint32_t pv_row = (uint32_t)(r8 + (mat & 1) * 8) * 128u, pv_x = (uint32_t)(((mat >> 1) ^ r8) << 4);
 #pragma unroll
@@ -272,18 +355,30 @@ __device__ __forceinline__ void accumulate_step(uint32_t vbase, int kk, const ui
         ldsm_x4_t(vbase + (np >> 2) * BOX_BYTES + kk * 16 * 128 + pv_row + ((((2 * np) & 7) << 4) ^ pv_x), b0, b1, b2, b3);
         mma_16(acc[2 * np], a[0], a[1], a[2], a[3], b0, b1);
         mma_16(acc[2 * np + 1], a[0], a[1], a[2], a[3], b2, b3);
+        if (with_third) {
+            mma_16(acc[2 * np], 0u, third[0], 0u, third[1], b0, b1);
+            mma_16(acc[2 * np + 1], 0u, third[0], 0u, third[1], b2, b3);
+        }
     }
 }
+
+// The key sums of up to eight heads on their way through the map.  128 channels: as bf16 hi + lo (sixteen mantissa bits);
+// 64 channels: fp32.
+template <int D> struct KeySums { __align__(16) __nv_bfloat16 hi[8][D], lo[8][D]; };
+template <> struct KeySums<64> { __align__(16) float v[8][64]; };
+__device__ __forceinline__ void store_key_sum(KeySums<128>& ks, int head, int c, float v) {
+    const __nv_bfloat16 hi = __float2bfloat16_rn(v);
+    ks.hi[head][c] = hi;
+    ks.lo[head][c] = __float2bfloat16_rn(v - __bfloat162float(hi));
+}
+__device__ __forceinline__ void store_key_sum(KeySums<64>& ks, int head, int c, float v) { ks.v[head][c] = v; }
 
 // Rows 16 mt .. + 15 of W times the key sums of n heads: pw[head][row].  One warp, M = 16 output channels, N = the heads
 // (padded to 8), K = D: the A fragments are read straight from the map in global memory, 16 bytes a load -- thread
 // (row r, quarter t) of a warp holds columns 8 (t + 4 jj) .. + 7 of rows r and r + 8, and the k slots of MMA step
-// 2 jj + h stand for columns 8 (t + 4 jj) + 4 h .. + 3, which the B fragments follow; the key sum enters as bf16
-// hi + lo (sixteen mantissa bits), the map's elements are bf16 as stored.
-template <int D>
-__device__ __forceinline__ void map_rows(const __nv_bfloat16* __restrict__ W, int mt, int n, const __nv_bfloat16 (&akh)[8][D],
-                                         const __nv_bfloat16 (&akl)[8][D], float (&pw)[8][D], int lane) {
-    constexpr int PIECES = D / 8;                                    // 16-byte pieces of a row of W
+// 2 jj + h stand for columns 8 (t + 4 jj) + 4 h .. + 3, which the B fragments follow; the map's elements are bf16 as stored.
+__device__ __forceinline__ void map_rows(const __nv_bfloat16* __restrict__ W, int mt, int n, const KeySums<128>& ks, float (&pw)[8][128], int lane) {
+    constexpr int D = 128, PIECES = D / 8;                           // 16-byte pieces of a row of W
     const int row = lane >> 2, quarter = lane & 3;
     const uint4* Wu = reinterpret_cast<const uint4*>(W);
     uint4 A[D / 16];
@@ -297,8 +392,8 @@ __device__ __forceinline__ void map_rows(const __nv_bfloat16* __restrict__ W, in
     for (int jj = 0; jj < D / 32; ++jj) {
         const uint4 r0 = A[2 * jj], r1 = A[2 * jj + 1];
         const int col = 8 * (quarter + 4 * jj);
-        const uint4 bh = *reinterpret_cast<const uint4*>(&akh[row][col]);      // B column = head `row`
-        const uint4 bl = *reinterpret_cast<const uint4*>(&akl[row][col]);
+        const uint4 bh = *reinterpret_cast<const uint4*>(&ks.hi[row][col]);      // B column = head `row`
+        const uint4 bl = *reinterpret_cast<const uint4*>(&ks.lo[row][col]);
         mma_16(d, r0.x, r1.x, r0.y, r1.y, bh.x, bh.y);
         mma_16(d, r0.x, r1.x, r0.y, r1.y, bl.x, bl.y);
         mma_16(d, r0.z, r1.z, r0.w, r1.w, bh.z, bh.w);
@@ -307,6 +402,27 @@ __device__ __forceinline__ void map_rows(const __nv_bfloat16* __restrict__ W, in
     // d[0], d[1]: row `row`, heads 2 quarter and 2 quarter + 1; d[2], d[3]: row `row` + 8
     if (2 * quarter < n) { pw[2 * quarter][16 * mt + row] = d[0]; pw[2 * quarter][16 * mt + row + 8] = d[2]; }
     if (2 * quarter + 1 < n) { pw[2 * quarter + 1][16 * mt + row] = d[1]; pw[2 * quarter + 1][16 * mt + row + 8] = d[3]; }
+}
+// Row c of W times the key sums of one head, 64 channels: a thread's row is 128 bytes, the key sums are the same for a warp.
+__device__ __forceinline__ float map_row(const __nv_bfloat16* __restrict__ W, int c, const KeySums<64>& ks, int head) {
+    const uint4* Wr = reinterpret_cast<const uint4*>(W + (size_t)c * 64);
+    float x[4] = {0.f, 0.f, 0.f, 0.f};
+    uint4 w[8];
+#pragma unroll
+    for (int p = 0; p < 8; ++p) w[p] = Wr[p];
+#pragma unroll
+    for (int p = 0; p < 8; ++p) {
+        const uint32_t e[4] = {w[p].x, w[p].y, w[p].z, w[p].w};
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            const float4 k = *reinterpret_cast<const float4*>(&ks.v[head][8 * p + 4 * h]);
+            x[0] = fmaf(__uint_as_float(e[2 * h] << 16), k.x, x[0]);
+            x[1] = fmaf(__uint_as_float(e[2 * h] & 0xffff0000u), k.y, x[1]);
+            x[2] = fmaf(__uint_as_float(e[2 * h + 1] << 16), k.z, x[2]);
+            x[3] = fmaf(__uint_as_float(e[2 * h + 1] & 0xffff0000u), k.w, x[3]);
+        }
+    }
+    return (x[0] + x[1]) + (x[2] + x[3]);
 }
 
 // The last part of the CLUSTER form: combines the records of a unit, which its cluster's blocks hold in shared
@@ -319,7 +435,7 @@ template <int NT> __device__ __forceinline__ void merge_sync() { asm volatile("b
 constexpr int MAX_CLUSTER = 16;
 template <int D> struct MergeShared {
     __align__(16) float comb[8 * (4 + 2 * D)];                        // this block's sums per head, read by the whole cluster
-    __align__(16) __nv_bfloat16 akh[8][D], akl[8][D];                 // key sums of the heads this block merges, hi and lo
+    KeySums<D> ks;                                                    // key sums of the heads this block merges
     float avs[8][D], pw[8][D];                                        // their value sums; W times the key sums
     float fac[8][MAX_CLUSTER], Ls[8];                                 // factor of every block's sums; sum of the weights
 };
@@ -330,7 +446,7 @@ __device__ __forceinline__ void cluster_merge(const float* recs, unsigned char* 
     constexpr int REC = C::REC, CREC = C::CREC, CW = C::CONSUMER_WARPS, NT = C::THREADS, V4 = 2 * D / 4;
     static_assert(sizeof(MergeShared<D>) <= (C::SLOTS - CW) * C::SLOT_BYTES, "the key sums lie behind it");
     MergeShared<D>& S = *reinterpret_cast<MergeShared<D>*>(room);
-    auto& comb = S.comb; auto& fac = S.fac; auto& Ls = S.Ls; auto& akh = S.akh; auto& akl = S.akl; auto& avs = S.avs; auto& pw = S.pw;
+    auto& comb = S.comb; auto& fac = S.fac; auto& Ls = S.Ls; auto& ks = S.ks; auto& avs = S.avs; auto& pw = S.pw;
     const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
     const int nblk = (int)cl::nctas(), rank = (int)cl::rank();
     merge_sync<NT>();                                                 // the warps' records are written
@@ -356,7 +472,7 @@ __device__ __forceinline__ void cluster_merge(const float* recs, unsigned char* 
         if (c4 == 0) { comb[a * REC] = M; comb[a * REC + 1] = L; }
         *reinterpret_cast<float4*>(comb + a * REC + 4 + 4 * c4) = acc;
     }
-    for (int e = tid; e < 8 * D; e += NT) { akh[e / D][e % D] = __float2bfloat16_rn(0.f); akl[e / D][e % D] = __float2bfloat16_rn(0.f); }
+    for (int e = tid; e < 8 * D; e += NT) store_key_sum(ks, e / D, e % D, 0.f);
     __syncwarp();
     cl::arrive_release();
     cl::wait_acquire();                                               // every block's sums are ready
@@ -395,22 +511,23 @@ __device__ __forceinline__ void cluster_merge(const float* recs, unsigned char* 
         for (int i = 0; i < 4; ++i) {
             const int c = 4 * c4 + i;
             if (c < D) avs[k][c] = v[i];
-            else {
-                const __nv_bfloat16 hi = __float2bfloat16_rn(v[i]);
-                akh[k][c - D] = hi;
-                akl[k][c - D] = __float2bfloat16_rn(v[i] - __bfloat162float(hi));
-            }
+            else store_key_sum(ks, k, c - D, v[i]);
         }
     }
     __syncwarp();
     cl::arrive_release();                                             // this block reads no other block's memory from here on
     merge_sync<NT>();
     if (mine > 0) {
-        for (int mt = wid; mt < D / 16; mt += NT / 32) map_rows<D>(Wu, mt, mine, akh, akl, pw, lane);
-        merge_sync<NT>();
+        if constexpr (D == 128) {
+            for (int mt = wid; mt < D / 16; mt += NT / 32) map_rows(Wu, mt, mine, ks, pw, lane);
+            merge_sync<NT>();
+        }
         for (int e = tid; e < mine * D; e += NT) {
             const int k = e / D, c = e - k * D;
-            const float o = (avs[k][c] + pw[k][c]) / Ls[k];
+            float x;
+            if constexpr (D == 128) x = pw[k][c];
+            else x = map_row(Wu, c, ks, k);
+            const float o = (avs[k][c] + x) / Ls[k];
             const size_t at = (size_t)(rank + k * nblk) * D + c;
             if (out_f32) reinterpret_cast<float*>(out_u)[at] = o;
             else reinterpret_cast<__nv_bfloat16*>(out_u)[at] = __float2bfloat16_rn(o);
@@ -479,8 +596,9 @@ decode_stream_bf16(const __nv_bfloat16* __restrict__ q, const __grid_constant__ 
     }
     // ---------------------------------------------------------------------- consumers
     const int gid = lane >> 2, tig = lane & 3;
+    const bool twice = C::PARTS == 3 && g <= 4;        // MMA rows 4-7 repeat the heads and take the third parts
     uint32_t qa[D / 16][2];
-    float acc[D / 8][4];                  // [dim tile][c0,c1: P_hi rows | c2,c3: P_lo rows]
+    float acc[D / 8][4];                  // [dim tile][c0,c1: rows of first (and third) parts | c2,c3: of second parts]
     float m = -INFINITY, l = 0.f, stash_scale = 1.f;
     bool stashed = false;
 
@@ -489,6 +607,15 @@ decode_stream_bf16(const __nv_bfloat16* __restrict__ q, const __grid_constant__ 
         int slot = b - block_of_tile((long long)unit * pl.n_tiles, pl);
         if (slot < 0 || slot >= pl.s_max) { atomicCAS(fault, 0, 5); slot = 0; }     // cannot happen; never write out of bounds
         return partial + ((((size_t)unit * pl.s_max + slot) * CONSUMER_WARPS + wq) * g + gid) * REC;
+    };
+    auto add_third = [&]() {                 // the whole warp, before store_acc: the third parts' sums to their heads' rows
+        if (twice) {
+#pragma unroll
+            for (int n = 0; n < D / 8; ++n) {
+                acc[n][2] += __shfl_xor_sync(0xffffffffu, acc[n][0], 16);
+                acc[n][3] += __shfl_xor_sync(0xffffffffu, acc[n][1], 16);
+            }
+        }
     };
     auto store_acc = [&](float* dst) {       // dims n*8 + 2 tig + {0,1} of head row gid
 #pragma unroll
@@ -504,6 +631,7 @@ decode_stream_bf16(const __nv_bfloat16* __restrict__ q, const __grid_constant__ 
         float lt = l;
         lt += __shfl_xor_sync(0xffffffffu, lt, 1);
         lt += __shfl_xor_sync(0xffffffffu, lt, 2);
+        add_third();
         if (gid < g) {
             float* rec = record_of(unit);
             if (tig == 0) *reinterpret_cast<float4*>(rec) = make_float4(m * 0.69314718055994531f, lt, stashed ? stash_scale : 1.f, stashed ? 1.f : 0.f);
@@ -521,35 +649,62 @@ decode_stream_bf16(const __nv_bfloat16* __restrict__ q, const __grid_constant__ 
         m = -INFINITY; l = 0.f; stash_scale = 1.f; stashed = false;
     };
     // One softmax step over the 64 keys at kbase, in two parts.  The first leaves the step's weights p in sc (this thread:
-    // head gid, keys 8 n + 2 tig, + 1) and brings m, l and the accumulators to the new running maximum.
-    auto scores64 = [&](uint32_t kbase, int nrows, bool retained, int unit, float (&sc)[8][2]) {
-        const float alpha = score_step<D>(kbase, nrows, scale_log2e, qa, lane, m, l, sc);
+    // head gid, keys 8 n + 2 tig, + 1) and brings m, l and (unless EXACT) the accumulators to the new running maximum.
+    auto scores64 = [&](uint32_t kbase, int nrows, bool retained, int unit, float (&sc)[8][2]) -> float {
+        float alpha;
+        if constexpr (C::EXACT) alpha = score_step64(kbase, nrows, scale_log2e, qa, lane, m, l, sc);
+        else alpha = score_step<D>(kbase, nrows, scale_log2e, qa, lane, m, l, sc);
         if (!retained && !stashed) {           // first key-only keys of this unit for this warp: park sum p v
+            add_third();
             if (gid < g) store_acc(record_of(unit) + 4);
             zero_acc();
             stashed = true;
             stash_scale = 1.f;
         }
         stash_scale *= alpha;
-        if (__any_sync(0xffffffffu, alpha != 1.f)) {
+        if (!C::EXACT && __any_sync(0xffffffffu, alpha != 1.f)) {
 #pragma unroll
             for (int n = 0; n < D / 8; ++n) { acc[n][0] *= alpha; acc[n][1] *= alpha; acc[n][2] *= alpha; acc[n][3] *= alpha; }
         }
+        return alpha;
     };
     // The second part adds p x (the 64 rows at vbase: values, or the keys themselves for a key-only tile).
-    auto accumulate64 = [&](uint32_t vbase, float (&sc)[8][2]) {
+    auto accumulate64 = [&](uint32_t vbase, float (&sc)[8][2], float alpha) {
+        if constexpr (!C::EXACT) {
 #pragma unroll
-        for (int kk = 0; kk < 4; ++kk) {
-            uint32_t a[4];
-            weights_bf16(sc, kk, a);
-            accumulate_step<D>(vbase, kk, a, acc, lane);
+            for (int kk = 0; kk < 4; ++kk) {
+                uint32_t a[4], third[2];
+                weights_bf16<C::PARTS>(sc, kk, twice, gid, a, third);
+                accumulate_step<D>(vbase, kk, a, false, third, acc, lane);
+            }
+        } else {
+#pragma unroll
+            for (int half = 0; half < 2; ++half) {
+                float sum[D / 8][4];                   // of 32 rows, which the accumulators take together
+#pragma unroll
+                for (int n = 0; n < D / 8; ++n) sum[n][0] = sum[n][1] = sum[n][2] = sum[n][3] = 0.f;
+#pragma unroll
+                for (int kk = 2 * half; kk < 2 * half + 2; ++kk) {
+                    uint32_t a[4], third[2];
+                    weights_bf16<C::PARTS>(sc, kk, twice, gid, a, third);
+                    accumulate_step<D>(vbase, kk, a, !twice, third, sum, lane);
+                }
+                const uint64_t f = tc::pack2(alpha, alpha);
+#pragma unroll
+                for (int n = 0; n < D / 8; ++n)
+#pragma unroll
+                    for (int e = 0; e < 4; e += 2) {
+                        const uint64_t o = tc::pack2(acc[n][e], acc[n][e + 1]), x = tc::pack2(sum[n][e], sum[n][e + 1]);
+                        tc::unpack2(half == 0 ? tc::fma2(o, f, x) : tc::add2(o, x), acc[n][e], acc[n][e + 1]);
+                    }
+            }
         }
     };
 
     auto step64 = [&](uint32_t kbase, uint32_t vbase, int nrows, bool retained, int unit) {
         float sc[8][2];
-        scores64(kbase, nrows, retained, unit, sc);
-        accumulate64(vbase, sc);
+        const float alpha = scores64(kbase, nrows, retained, unit, sc);
+        accumulate64(vbase, sc, alpha);
     };
 
     zero_acc();
@@ -563,7 +718,7 @@ decode_stream_bf16(const __nv_bfloat16* __restrict__ q, const __grid_constant__ 
             const int s = i % SLOTS, round = i / SLOTS;
             const int t = (int)(gt_lo + i - (long long)u * pl.n_tiles);
             if (ok) {
-                if (!loaded) { load_queries<D>(q, u, g, lane, qa); loaded = true; }
+                if (!loaded) { load_queries<D>(q, u, g, lane, qa, twice); loaded = true; }
                 ok = tma::mbar_wait_warp(&full_bar[s], round & 1, fault, 2);
             }
             if (!ok) continue;
@@ -589,27 +744,25 @@ decode_stream_bf16(const __nv_bfloat16* __restrict__ q, const __grid_constant__ 
 // Combines the records of a unit, applies the unit's map to the p-weighted key sum and normalises:
 //   o = (sum_j f_j s_j acc_v_j + W sum_j f_j acc_k_j) / sum_j f_j l_j,   f_j = exp(m_j - max m).
 // Every load of a phase is independent of the others, so a phase costs one memory latency.
-// The product W (sum f acc_k) runs on warp-level MMAs (map_rows).
+// The product W (sum f acc_k) runs on warp-level MMAs (map_rows), or, for 64 channels, on CUDA cores (map_row).
 template <typename TO, int D, int MAXT>
 __global__ void __launch_bounds__(MAXT, MAXT == 512 ? 3 : 1)
 decode_merge_bf16(const float* __restrict__ partial, const __nv_bfloat16* __restrict__ W, int LH, int g,
                        Plan pl, int apply_w, int cw, TO* __restrict__ out) {
     constexpr int REC = 4 + 2 * D;
-    __shared__ __align__(16) __nv_bfloat16 akh[8][D], akl[8][D];          // key sums per head, hi and lo halves
-    __shared__ float pw[8][D];                 // W times the key sum
-    __shared__ float fv[8][48], fk[8][48];     // per head, per record: factor for the value part / the key part
+    __shared__ KeySums<D> ks;
+    __shared__ float pw[D == 128 ? 8 : 1][D];  // W times the key sum
+    constexpr int MAX_REC = 12 * Cfg<D, false>::CONSUMER_WARPS, REC_PER_LANE = (MAX_REC + 31) / 32;      // of a unit: twelve blocks' at the most
+    __shared__ float fv[8][MAX_REC], fk[8][MAX_REC];     // per head, per record: factor for the value part / the key part
     __shared__ float Ls[8];
     const int u = blockIdx.x, tid = threadIdx.x, a = tid / D, c = tid % D, lane = tid & 31;
     const int wid = tid >> 5, nwarps = blockDim.x >> 5;
     const __nv_bfloat16* Wu = W + (size_t)(u % LH) * D * D;       // the maps of a layer stay in L2: every sequence of the batch reads them
-    for (int i = tid; i < (8 - g) * D; i += blockDim.x) {         // columns of B beyond the unit's heads
-        akh[g + i / D][i % D] = __float2bfloat16_rn(0.f);
-        akl[g + i / D][i % D] = __float2bfloat16_rn(0.f);
-    }
+    for (int i = tid; i < (8 - g) * D; i += blockDim.x) store_key_sum(ks, g + i / D, i % D, 0.f);      // columns of B beyond the unit's heads
     // the streaming kernel's records from here on
     asm volatile("griddepcontrol.wait;\n" ::: "memory");
     const int first = block_of_tile((long long)u * pl.n_tiles, pl);
-    const int n_rec = (block_of_tile((long long)(u + 1) * pl.n_tiles - 1, pl) - first + 1) * cw;   // <= 48; cw records per block
+    const int n_rec = (block_of_tile((long long)(u + 1) * pl.n_tiles - 1, pl) - first + 1) * cw;   // <= MAX_REC; cw records per block
     const float* base = partial + (size_t)u * pl.s_max * cw * g * REC;
     // The first six records' sums are requested before the headers are looked at, so that the two loads
     // share one memory latency (a unit lies in one or two blocks of the streaming kernel, three records
@@ -624,24 +777,25 @@ decode_merge_bf16(const float* __restrict__ partial, const __nv_bfloat16* __rest
         rk[k] = r[D + c];
     }
     if (c < 32) {
-        // first warp of head a: headers of records lane and lane + 32
-        float mj[2], lj[2], sj[2];
+        // first warp of head a: headers of records lane, lane + 32, ...
+        float mj[REC_PER_LANE], lj[REC_PER_LANE], sj[REC_PER_LANE], M = -INFINITY;
 #pragma unroll
-        for (int k = 0; k < 2; ++k) {
+        for (int k = 0; k < REC_PER_LANE; ++k) {
             const int j = lane + 32 * k;
             mj[k] = -INFINITY; lj[k] = 0.f; sj[k] = 0.f;
             if (j < n_rec) {
                 const float4 h = *reinterpret_cast<const float4*>(base + ((size_t)j * g + a) * REC);
                 mj[k] = h.x; lj[k] = h.y; sj[k] = h.z;
             }
+            M = fmaxf(M, mj[k]);
         }
-        const float M = warp_max(fmaxf(mj[0], mj[1]));
+        M = warp_max(M);
         float Lsum = 0.f;
 #pragma unroll
-        for (int k = 0; k < 2; ++k) {
+        for (int k = 0; k < REC_PER_LANE; ++k) {
             const int j = lane + 32 * k;
             const float f = mj[k] > -INFINITY ? __expf(mj[k] - M) : 0.f;
-            if (j < 48) { fk[a][j] = f; fv[a][j] = f * sj[k]; }
+            if (j < MAX_REC) { fk[a][j] = f; fv[a][j] = f * sj[k]; }
             Lsum += f * lj[k];
         }
         Lsum = warp_sum(Lsum);
@@ -671,15 +825,17 @@ decode_merge_bf16(const float* __restrict__ partial, const __nv_bfloat16* __rest
         store_out(out + ((size_t)u * g + a) * D + c, (av + ak) / Ls[a]);
         return;
     }
-    {
-        const __nv_bfloat16 hi = __float2bfloat16_rn(ak);
-        akh[a][c] = hi;
-        akl[a][c] = __float2bfloat16_rn(ak - __bfloat162float(hi));
+    store_key_sum(ks, a, c, ak);
+    __syncthreads();
+    float x;
+    if constexpr (D == 128) {
+        for (int mt = wid; mt < D / 16; mt += nwarps) map_rows(Wu, mt, g, ks, pw, lane);
+        __syncthreads();
+        x = pw[a][c];
+    } else {
+        x = map_row(Wu, c, ks, a);
     }
-    __syncthreads();
-    for (int mt = wid; mt < D / 16; mt += nwarps) map_rows<D>(Wu, mt, g, akh, akl, pw, lane);
-    __syncthreads();
-    store_out(out + ((size_t)u * g + a) * D + c, (av + pw[a][c]) / Ls[a]);
+    store_out(out + ((size_t)u * g + a) * D + c, (av + x) / Ls[a]);
 }
 
 }  // namespace dbf

@@ -182,7 +182,7 @@ decode_stream_rope(const __nv_bfloat16* __restrict__ q, const __grid_constant__ 
                         if (lane + 32 * k < rows) pos[k] = (uint32_t)__ldg(pr + 32 * k);
                 }
                 if (ok) {
-                    if (!loaded) { load_queries<D>(q, u, g, lane, qa); loaded = true; }
+                    if (!loaded) { load_queries<D>(q, u, g, lane, qa, false); loaded = true; }
                     ok = tma::mbar_wait_warp(&full_bar[s], (i / SLOTS) & 1, fault, 2);
                 }
                 if (!retained && !keys) { keys = true; v_scale[0] = v_scale[1] = 1.f; }       // the value sums are parked at this maximum
