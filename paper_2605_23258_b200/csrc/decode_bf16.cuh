@@ -36,6 +36,7 @@
 #include "cluster.cuh"
 #include "common.cuh"
 #include "internal.h"
+#include "rope.cuh"
 #include "tcgen05.cuh"
 #include "tma.cuh"
 
@@ -67,9 +68,11 @@ template <int D, bool ROPE> struct Cfg {
     // With RoPE decoupling a consumer is a team (decode_rope.cuh): a score warp and some sum warps.
     // Four teams at 64 channels, of two sum warps with as many channel pairs each as the four have at 128.
     static constexpr int CONSUMER_WARPS = D == 128 ? 3 : 4, SUM_WARPS = ROPE ? D / 32 : 0;
-    static constexpr int SLOTS = D == 128 ? 6 : 12;                  // a multiple of CONSUMER_WARPS: a slot always serves the same warp
+    static constexpr int SLOTS = D == 128 ? 6 : ROPE ? 8 : 12;       // a multiple of CONSUMER_WARPS: a slot always serves the same warp
     static constexpr int THREADS = 32 * (CONSUMER_WARPS * (1 + SUM_WARPS) + 1);
-    static constexpr int STEP_BYTES = 2048 + 4 * KEYS + 32;          // RoPE: a step's weights, positions and factors
+    // RoPE: a step buffer: weights [16 keys][first | second parts of 8 keys][head][8 keys], EXACT: third parts alike; positions; factors
+    static constexpr int STEP_THIRD = 2048, STEP_POS = STEP_THIRD + (EXACT ? 1024 : 0), STEP_ALPHA = STEP_POS + 4 * KEYS;
+    static constexpr int STEP_BYTES = STEP_ALPHA + 32;
     static constexpr int P_BYTES = ROPE ? CONSUMER_WARPS * 2 * STEP_BYTES : 0;
     static constexpr int SMEM_BYTES = SLOTS * SLOT_BYTES + P_BYTES + 1024;     // + alignment slack; barriers live in static smem
     static constexpr int REC = 4 + 2 * D;                            // m, l, value-scale, pad, acc_v[D], acc_k[D]
@@ -318,29 +321,18 @@ __device__ __forceinline__ float score_step64(uint32_t kbase, int nrows, float s
     m = m_new;
     return alpha;
 }
-// A pair of weights as bf16 parts: what the rounding to the parts before leaves, rounded; three parts leave nothing.
-template <int PARTS>
-__device__ __forceinline__ void split_bf16(float p0, float p1, uint32_t (&part)[3]) {
-#pragma unroll
-    for (int i = 0; i < PARTS; ++i) {
-        part[i] = pack_bf16(p0, p1);
-        if (i + 1 < PARTS)
-            tc::unpack2(tc::fma2(tc::pack2(__uint_as_float(part[i] << 16), __uint_as_float(part[i] & 0xffff0000u)), tc::pack2(-1.f, -1.f),
-                                 tc::pack2(p0, p1)), p0, p1);
-    }
-}
 // The weights of keys 16 kk .. + 15 as an A fragment: first parts in MMA rows 0-7, second parts in rows 8-15.  Third parts:
 // of up to four heads (twice: this thread's head is gid & 3) in rows 4-7, else in a fragment of their own (rows 8-15, third).
 template <int PARTS>
 __device__ __forceinline__ void weights_bf16(const float (&sc)[8][2], int kk, bool twice, int gid, uint32_t (&a)[4], uint32_t (&third)[2]) {
 #pragma unroll
     for (int x = 0; x < 2; ++x) {
-        uint32_t part[3];
-        split_bf16<PARTS>(sc[2 * kk + x][0], sc[2 * kk + x][1], part);
+        uint32_t part[PARTS];
+        split_bf16(sc[2 * kk + x][0], sc[2 * kk + x][1], part);
         const bool upper = PARTS == 3 && twice && gid >= 4;
-        a[2 * x] = upper ? part[2] : part[0];
+        a[2 * x] = upper ? part[PARTS - 1] : part[0];
         a[2 * x + 1] = upper ? 0u : part[1];
-        third[x] = PARTS == 3 ? part[2] : 0u;
+        third[x] = PARTS == 3 ? part[PARTS - 1] : 0u;
     }
 }
 // acc += P x over rows 16 kk .. + 15 of the 64 rows at vbase: D / 8 column tiles of 8 dims.  with_third: P has a third fragment.

@@ -6,20 +6,22 @@
 // of the tile, so that warps that own whole tiles (decode_bf16.cuh) would be bound by their own instruction chains.  A
 // block therefore has teams, tile i to team i % TEAMS: three of five warps, or, at 64 channels, four of three:
 //   score warp   S = Q K^T and the online softmax, 64 keys a step; it leaves the weights as MMA A fragments (hi and
-//                lo halves; bf16 for values, fp16 for turned keys), the factor the older sums take, and the keys' positions
-//                in one of the team's two step buffers
+//                lo halves; bf16 for values, fp16 for turned keys; at 64 channels three bf16 parts for both), the factor the
+//                older sums take, and the keys' positions in one of the team's two step buffers
 //   sum warps    each owns 16 of the channel pairs (c, c + D/2).  It takes the rows as MMA B fragments straight from
 //                the slot -- both channels of a pair lie in the same thread's fragments -- turns them in registers (fp16,
 //                eleven bits: a turned key is not a bf16 number and eight bits would not keep the key sum within the
-//                tolerance of the output; |k| beyond 65504 saturates) and multiplies: nothing is written back
+//                tolerance of the output; |k| beyond 65504 saturates; at 64 channels three bf16 parts, rope.cuh)
+//                and multiplies: nothing is written back
 // and one producer thread.  What bounds it: HBM once all of this overlaps, and before that the score warps (about 3000
 // cycles per 64 keys, 2300 of them busy) and the sum warps (2500 busy) waiting for one another.  Measured, 128 units of 3000
 // retained + 6000 key-only rows, 393 MB, with the appended row and the merge: 86 us; 104 us with warps that owned whole tiles
 // and twelve helpers that turned keys back in shared memory (a fence and three block barriers per 64 keys).
-// 64 channels, 512 units of 1639 + 3276 rows, in a graph: 112 us; 126 with three teams of five warps, whose score warps
-// took most of the time (72 without rotation).
+// 64 channels, 512 units of 1639 + 3276 rows: 201 us a step with the appended row, bound by the sum warps' instructions (about
+// 1000 for 64 key-only rows; 114 us with fp16 keys, 1139 us on CUDA cores; sum warps of eight pairs 210, five teams 203, loops
+// rolled up 207).  Error of an fp32 output against fp64, median over the heads: 1.8e-7 to 4.1e-7 (fp16: 1.1e-4, CUDA cores: 2.0e-7 to 5.5e-7).
 // The angle is position * theta^(-2c/D), taken as the 32-bit product of the position and the
-// channel's phase (turns per position as a fraction of 2^32), which is the angle modulo one turn.
+// channel's phase (turns per position as a fraction of 2^32), which is the angle modulo one turn; 64 channels: rope.cuh.
 #ifndef VECTOR_DECODE_ROPE_CUH_
 #define VECTOR_DECODE_ROPE_CUH_
 
@@ -27,8 +29,6 @@
 
 namespace vec {
 namespace dbf {
-
-constexpr uint32_t STEP_POS = 2048, STEP_ALPHA = STEP_POS + 4 * KEYS;     // a step buffer: weights [16 keys][hi | lo of 8 keys][head][8 keys], positions, factors
 
 // x and y, the two channels of eight pairs (two keys to a register), turned back by pos[] * phase and left as fp16.
 __device__ __forceinline__ void turn_back(uint32_t& x, uint32_t& y, uint32_t pos0, uint32_t pos1, uint32_t phase) {
@@ -92,6 +92,77 @@ __device__ __forceinline__ void score_step_keys(uint32_t kbase, int nrows, float
         }
 }
 
+// A sum warp's part of a softmax step, 64 channels: rows times weights over 64 rows at base (this lane's place in its column
+// tiles), in three bf16 parts each way.  acc takes the sums of 32 rows at a time, which start at zero (Cfg::EXACT); alpha is the
+// factor of what it held.  st: the step buffer.  Products of parts that lie below 2^-24 of the whole come along where they cost
+// nothing: a fragment holds all parts of the weights.
+__device__ __forceinline__ void sum_step64(uint32_t st, uint32_t base, bool retained, bool with_third, float alpha, const RopePhase (&phase)[2],
+                                           float (&acc)[2][2][4], int lane) {
+    using C = Cfg<64, true>;
+    const int tig = lane & 3;
+#pragma unroll 1
+    for (int half = 0; half < 2; ++half) {
+        float sum[2][2][4];
+#pragma unroll
+        for (int x = 0; x < 2; ++x)
+#pragma unroll
+            for (int p = 0; p < 2; ++p) sum[x][p][0] = sum[x][p][1] = sum[x][p][2] = sum[x][p][3] = 0.f;
+#pragma unroll
+        for (int k2 = 0; k2 < 2; ++k2) {
+            const int kk = 2 * half + k2;
+            uint32_t a[4], third[2] = {0u, 0u}, rx[2][2], ry[2][2];       // B fragments: low and high channels, rows 0-7 | 8-15
+            ldsm_x4(st + kk * 512 + lane * 16, a[0], a[1], a[2], a[3]);
+            if (with_third)
+                asm volatile("ldmatrix.sync.aligned.m8n8.x2.shared.b16 {%0,%1}, [%2];\n"
+                             : "=r"(third[0]), "=r"(third[1]) : "r"(st + C::STEP_THIRD + kk * 256 + (lane & 15) * 16));
+            const uint32_t at = base + kk * 16 * 128;
+            ldsm_x4_t(at, rx[0][0], rx[0][1], rx[1][0], rx[1][1]);
+            ldsm_x4_t(at ^ 64u, ry[0][0], ry[0][1], ry[1][0], ry[1][1]);
+            auto add = [&](float (&s)[4], uint32_t b0, uint32_t b1) { mma_16(s, a[0], a[1], a[2], a[3], b0, b1); };
+            auto add_w3 = [&](float (&s)[4], uint32_t b0, uint32_t b1) { if (with_third) mma_16(s, 0u, third[0], 0u, third[1], b0, b1); };
+            if (retained) {
+#pragma unroll
+                for (int p = 0; p < 2; ++p) {
+                    add(sum[0][p], rx[p][0], rx[p][1]);
+                    add(sum[1][p], ry[p][0], ry[p][1]);
+                    add_w3(sum[0][p], rx[p][0], rx[p][1]);
+                    add_w3(sum[1][p], ry[p][0], ry[p][1]);
+                }
+            } else {
+                uint32_t xp[2][2][3], yp[2][2][3];                        // [column tile][rows 0-7 | 8-15][part]
+#pragma unroll
+                for (int r = 0; r < 2; ++r) {                             // rows 2 tig, + 1 of the eight
+                    uint32_t pos0, pos1;
+                    asm volatile("ld.shared.v2.u32 {%0,%1}, [%2];\n" : "=r"(pos0), "=r"(pos1) : "r"(st + C::STEP_POS + kk * 64 + r * 32 + tig * 8));
+#pragma unroll
+                    for (int p = 0; p < 2; ++p) turn_back_parts(rx[p][r], ry[p][r], (int)pos0, (int)pos1, phase[p], xp[p][r], yp[p][r]);
+                }
+#pragma unroll
+                for (int i = 2; i >= 0; --i)                              // the small parts first
+#pragma unroll
+                    for (int p = 0; p < 2; ++p) {
+                        if (i == 0) {
+                            add_w3(sum[0][p], xp[p][0][0], xp[p][1][0]);
+                            add_w3(sum[1][p], yp[p][0][0], yp[p][1][0]);
+                        }
+                        add(sum[0][p], xp[p][0][i], xp[p][1][i]);
+                        add(sum[1][p], yp[p][0][i], yp[p][1][i]);
+                    }
+            }
+        }
+        const uint64_t f = tc::pack2(alpha, alpha);
+#pragma unroll
+        for (int x = 0; x < 2; ++x)
+#pragma unroll
+            for (int p = 0; p < 2; ++p)
+#pragma unroll
+                for (int e = 0; e < 4; e += 2) {
+                    const uint64_t o = tc::pack2(acc[x][p][e], acc[x][p][e + 1]), s = tc::pack2(sum[x][p][e], sum[x][p][e + 1]);
+                    tc::unpack2(half == 0 ? tc::fma2(o, f, s) : tc::add2(o, s), acc[x][p][e], acc[x][p][e + 1]);
+                }
+    }
+}
+
 // grid, shared memory, partial, CLUSTER: as for decode_stream_bf16.  Warps 0 .. TEAMS - 1 score, the next one is the producer, then
 // come the sum warps, team by team.
 template <int D, bool CLUSTER>
@@ -103,6 +174,8 @@ decode_stream_rope(const __nv_bfloat16* __restrict__ q, const __grid_constant__ 
     using C = Cfg<D, true>;
     constexpr int HALF_BYTES = C::HALF_BYTES, SLOT_BYTES = C::SLOT_BYTES, SLOTS = C::SLOTS, TEAMS = C::CONSUMER_WARPS, SUM_WARPS = C::SUM_WARPS;
     constexpr int REC = C::REC, CREC = C::CREC, PAIRS = 2;                    // column tiles of 8 channel pairs of a sum warp
+    constexpr int STEP_THIRD = C::STEP_THIRD, STEP_POS = C::STEP_POS, STEP_ALPHA = C::STEP_ALPHA;
+    const bool twice = C::EXACT && g <= 4;             // MMA rows 4-7 repeat the heads and take the third parts of the weights
     extern __shared__ unsigned char smem_raw[];
     __shared__ __align__(8) uint64_t full_bar[SLOTS], empty_bar[SLOTS];
     __shared__ __align__(8) uint64_t step_full[TEAMS][2], step_empty[TEAMS][2];
@@ -182,7 +255,7 @@ decode_stream_rope(const __nv_bfloat16* __restrict__ q, const __grid_constant__ 
                         if (lane + 32 * k < rows) pos[k] = (uint32_t)__ldg(pr + 32 * k);
                 }
                 if (ok) {
-                    if (!loaded) { load_queries<D>(q, u, g, lane, qa, false); loaded = true; }
+                    if (!loaded) { load_queries<D>(q, u, g, lane, qa, twice); loaded = true; }
                     ok = tma::mbar_wait_warp(&full_bar[s], (i / SLOTS) & 1, fault, 2);
                 }
                 if (!retained && !keys) { keys = true; v_scale[0] = v_scale[1] = 1.f; }       // the value sums are parked at this maximum
@@ -202,11 +275,18 @@ decode_stream_rope(const __nv_bfloat16* __restrict__ q, const __grid_constant__ 
                     const uint32_t st = steps + k * C::STEP_BYTES;
 #pragma unroll
                     for (int j = 0; j < 4; ++j) {
-                        uint32_t hi[2], lo[2];         // keys gid and gid + 8 of the 16
+                        uint32_t hi[2], lo[2], third[2];         // keys gid and gid + 8 of the 16
 #pragma unroll
                         for (int e = 0; e < 2; ++e) {
                             const float p0 = sc[j][2 * e], p1 = sc[j][2 * e + 1];
-                            if (retained) {
+                            if constexpr (C::EXACT) {
+                                uint32_t part[3];
+                                split_bf16(p0, p1, part);
+                                const bool upper = twice && tig >= 2;
+                                hi[e] = upper ? part[2] : part[0];
+                                lo[e] = upper ? 0u : part[1];
+                                third[e] = part[2];
+                            } else if (retained) {
                                 hi[e] = pack_bf16(p0, p1);
                                 lo[e] = pack_bf16(p0 - __uint_as_float(hi[e] << 16), p1 - __uint_as_float(hi[e] & 0xffff0000u));
                             } else {
@@ -216,6 +296,9 @@ decode_stream_rope(const __nv_bfloat16* __restrict__ q, const __grid_constant__ 
                         }
                         asm volatile("stmatrix.sync.aligned.m8n8.x4.trans.shared.b16 [%0], {%1,%2,%3,%4};\n" ::"r"(st + j * 512 + lane * 16),
                                      "r"(hi[0]), "r"(lo[0]), "r"(hi[1]), "r"(lo[1]) : "memory");
+                        if (C::EXACT && !twice)
+                            asm volatile("stmatrix.sync.aligned.m8n8.x2.trans.shared.b16 [%0], {%1,%2};\n"
+                                         ::"r"(st + STEP_THIRD + j * 256 + (lane & 15) * 16), "r"(third[0]), "r"(third[1]) : "memory");
                     }
                     if (!retained) {
                         asm volatile("st.shared.u32 [%0], %1;\n" ::"r"(st + STEP_POS + lane * 4), "r"(h ? pos[2] : pos[0]) : "memory");
@@ -243,15 +326,26 @@ decode_stream_rope(const __nv_bfloat16* __restrict__ q, const __grid_constant__ 
     // Warp `part` of the team: channel pairs 8 PAIRS part .. + 8 PAIRS - 1, i.e. column tiles PAIRS part + p and D/16 + PAIRS part + p.
     const int part = (wq - TEAMS - 1) % SUM_WARPS;
     const int mat = lane >> 3, r8 = lane & 7;
-    uint32_t phase[PAIRS];                             // of channel pair 8 (PAIRS part + p) + gid, rounded to 32 bits
+    RopePhase phase[PAIRS];                            // of channel pair 8 (PAIRS part + p) + gid; not EXACT: hi alone, the phase rounded to 32 bits
 #pragma unroll
-    for (int p = 0; p < PAIRS; ++p) phase[p] = (uint32_t)((rope.phase[8 * (PAIRS * part + p) + gid] + 0x80000000ull) >> 32);
-    float acc[2][PAIRS][4];                            // [low | high channel of the pair][column tile][hi rows | lo rows]
+    for (int p = 0; p < PAIRS; ++p) phase[p] = rope_phase_words(rope.phase[8 * (PAIRS * part + p) + gid]);
+    float acc[2][PAIRS][4];                            // [low | high channel of the pair][column tile][rows of first (and third) parts | of second parts]
     auto zero_acc = [&]() {
 #pragma unroll
         for (int x = 0; x < 2; ++x)
 #pragma unroll
             for (int p = 0; p < PAIRS; ++p) acc[x][p][0] = acc[x][p][1] = acc[x][p][2] = acc[x][p][3] = 0.f;
+    };
+    auto add_third = [&]() {                           // the whole warp, before store_acc: the third parts' sums to their heads' rows
+        if (twice) {
+#pragma unroll
+            for (int x = 0; x < 2; ++x)
+#pragma unroll
+                for (int p = 0; p < PAIRS; ++p) {
+                    acc[x][p][2] += __shfl_xor_sync(0xffffffffu, acc[x][p][0], 16);
+                    acc[x][p][3] += __shfl_xor_sync(0xffffffffu, acc[x][p][1], 16);
+                }
+        }
     };
     auto store_acc = [&](float* dst) {
 #pragma unroll
@@ -275,6 +369,7 @@ decode_stream_rope(const __nv_bfloat16* __restrict__ q, const __grid_constant__ 
             any = true;
             if (ok) ok = tma::mbar_wait_warp(&full_bar[s], (i / SLOTS) & 1, fault, 2);
             if (!retained && !parked) {                // the unit's first key-only keys: park sum p v
+                add_third();
                 if (gid < g) store_acc(record_of(u, gid) + 4);
                 zero_acc();
                 parked = true;
@@ -289,35 +384,39 @@ decode_stream_rope(const __nv_bfloat16* __restrict__ q, const __grid_constant__ 
                 const uint32_t base = tma::smem_u32(smem + s * SLOT_BYTES) + (retained ? HALF_BYTES : h * HALF_BYTES) + frag;
                 float alpha;
                 asm volatile("ld.shared.f32 %0, [%1];\n" : "=f"(alpha) : "r"(st + STEP_ALPHA + gid * 4));
+                if constexpr (C::EXACT) {
+                    sum_step64(st, base, retained, !twice, alpha, phase, acc, lane);
+                } else {
 #pragma unroll
-                for (int x = 0; x < 2; ++x)
+                    for (int x = 0; x < 2; ++x)
 #pragma unroll
-                    for (int p = 0; p < PAIRS; ++p) { acc[x][p][0] *= alpha; acc[x][p][1] *= alpha; acc[x][p][2] *= alpha; acc[x][p][3] *= alpha; }
+                        for (int p = 0; p < PAIRS; ++p) { acc[x][p][0] *= alpha; acc[x][p][1] *= alpha; acc[x][p][2] *= alpha; acc[x][p][3] *= alpha; }
 #pragma unroll
-                for (int kk = 0; kk < 4; ++kk) {
-                    uint32_t a[4], rx[PAIRS][2], ry[PAIRS][2];            // B fragments: low and high channels, rows 0-7 | 8-15
-                    ldsm_x4(st + kk * 512 + lane * 16, a[0], a[1], a[2], a[3]);
-                    const uint32_t at = base + kk * 16 * 128;
-                    ldsm_x4_t(at, rx[0][0], rx[0][1], rx[1][0], rx[1][1]);
-                    ldsm_x4_t(D == 128 ? at + BOX_BYTES : at ^ 64u, ry[0][0], ry[0][1], ry[1][0], ry[1][1]);
-                    if (retained) {
+                    for (int kk = 0; kk < 4; ++kk) {
+                        uint32_t a[4], rx[PAIRS][2], ry[PAIRS][2];            // B fragments: low and high channels, rows 0-7 | 8-15
+                        ldsm_x4(st + kk * 512 + lane * 16, a[0], a[1], a[2], a[3]);
+                        const uint32_t at = base + kk * 16 * 128;
+                        ldsm_x4_t(at, rx[0][0], rx[0][1], rx[1][0], rx[1][1]);
+                        ldsm_x4_t(D == 128 ? at + BOX_BYTES : at ^ 64u, ry[0][0], ry[0][1], ry[1][0], ry[1][1]);
+                        if (retained) {
 #pragma unroll
-                        for (int p = 0; p < PAIRS; ++p) {
-                            mma_16(acc[0][p], a[0], a[1], a[2], a[3], rx[p][0], rx[p][1]);
-                            mma_16(acc[1][p], a[0], a[1], a[2], a[3], ry[p][0], ry[p][1]);
-                        }
-                    } else {
+                            for (int p = 0; p < PAIRS; ++p) {
+                                mma_16(acc[0][p], a[0], a[1], a[2], a[3], rx[p][0], rx[p][1]);
+                                mma_16(acc[1][p], a[0], a[1], a[2], a[3], ry[p][0], ry[p][1]);
+                            }
+                        } else {
 #pragma unroll
-                        for (int r = 0; r < 2; ++r) {                     // rows 2 tig, + 1 of the eight
-                            uint32_t pos0, pos1;
-                            asm volatile("ld.shared.v2.u32 {%0,%1}, [%2];\n" : "=r"(pos0), "=r"(pos1) : "r"(st + STEP_POS + kk * 64 + r * 32 + tig * 8));
+                            for (int r = 0; r < 2; ++r) {                     // rows 2 tig, + 1 of the eight
+                                uint32_t pos0, pos1;
+                                asm volatile("ld.shared.v2.u32 {%0,%1}, [%2];\n" : "=r"(pos0), "=r"(pos1) : "r"(st + STEP_POS + kk * 64 + r * 32 + tig * 8));
 #pragma unroll
-                            for (int p = 0; p < PAIRS; ++p) turn_back(rx[p][r], ry[p][r], pos0, pos1, phase[p]);
-                        }
+                                for (int p = 0; p < PAIRS; ++p) turn_back(rx[p][r], ry[p][r], pos0, pos1, (uint32_t)phase[p].hi);
+                            }
 #pragma unroll
-                        for (int p = 0; p < PAIRS; ++p) {
-                            mma_16_f16(acc[0][p], a[0], a[1], a[2], a[3], rx[p][0], rx[p][1]);
-                            mma_16_f16(acc[1][p], a[0], a[1], a[2], a[3], ry[p][0], ry[p][1]);
+                            for (int p = 0; p < PAIRS; ++p) {
+                                mma_16_f16(acc[0][p], a[0], a[1], a[2], a[3], rx[p][0], rx[p][1]);
+                                mma_16_f16(acc[1][p], a[0], a[1], a[2], a[3], ry[p][0], ry[p][1]);
+                            }
                         }
                     }
                 }
@@ -327,6 +426,7 @@ decode_stream_rope(const __nv_bfloat16* __restrict__ q, const __grid_constant__ 
             if (ok && lane == 0) tma::mbar_arrive(&empty_bar[s]);
         }
         // the unit's sums; the cluster's merge reads no more of them than the header says
+        add_third();
         if (CLUSTER) {
             // the slot that takes the key sums is the team's, and may hold its last tile
             asm volatile("bar.sync %0, %1;\n" ::"r"(2 + team), "n"(32 * SUM_WARPS) : "memory");

@@ -93,7 +93,7 @@ def test_decode_head64(oracle, rope, g, layers, n_ret, n_apx):
         assert np.max(np.abs(out[u].cpu().double().numpy() - o)) <= 2e-2, u
 
 
-@pytest.mark.parametrize("rope", [False])
+@pytest.mark.parametrize("rope", [False, True])
 @pytest.mark.parametrize("g,units,n_ret,n_apx,sharp", [
     (4, 4, 70, 140, 2.0), (8, 4, 70, 140, 2.0),               # the one-launch form: third parts in spare rows, or in a fragment of their own
     (4, 80, 70, 140, 2.0), (5, 80, 70, 140, 2.0),             # records and merge
@@ -123,3 +123,24 @@ def test_decode_head64_keeps_fp32_precision(oracle, rope, g, units, n_ret, n_apx
         errs.append(np.linalg.norm(out[u].cpu().double().numpy() - o, axis=1) / np.linalg.norm(o, axis=1))
     errs = np.concatenate(errs)
     assert errs.max() <= 1.5e-6 and np.sqrt(np.mean(errs ** 2)) <= 5e-7, (errs.max(), np.sqrt(np.mean(errs ** 2)))
+
+
+def test_decode_head64_rope_keeps_large_keys(oracle):
+    """Keys beyond the fp16 range, and positions of either sign: a turned key keeps bf16's range."""
+    U, g, d, n = 3, 4, 64, 100
+    gen = torch.Generator(device=DEV).manual_seed(3)
+    ak = (torch.randn(U, n, d, generator=gen, device=DEV) * 3e5).to(torch.bfloat16)
+    rk, rv = (torch.zeros(U, 1, d, dtype=torch.bfloat16, device=DEV) for _ in range(2))
+    W = (torch.randn(U, d, d, generator=gen, device=DEV) / 8).to(torch.bfloat16)
+    q = (torch.randn(U, g, d, generator=gen, device=DEV) * 1e-6).to(torch.bfloat16)
+    pos = torch.randint(-131072, 131072, (U, n), generator=gen, device=DEV, dtype=torch.int32)
+    cache = vec.Cache(rk, rv, ak, torch.zeros(U, 1, dtype=torch.int32, device=DEV), pos, 0, n)
+    sh = vec.Shape(1, 1, U * g, U, d, vec.VECTOR_BF16, 16, 7, 0.0, 1, 10000.0)
+    out = torch.full((U, g, d), float("nan"), device=DEV)
+    vec.vector_decode_attn(sh, q, cache, W, out, 0, vec.alloc_workspace(sh, vec.vector_plan_budget(4096, 2048, -1, 16)))
+    torch.cuda.synchronize()
+    for u in range(U):
+        _, o = oracle.attend(q[u].cpu(), rk[u, :0].cpu(), rv[u, :0].cpu(), ak[u].cpu(), W[u].cpu(), 1.0 / np.sqrt(d),
+                             apx_pos=pos[u].cpu().numpy(), rope=True, theta=10000.0)
+        err = np.linalg.norm(out[u].cpu().double().numpy() - o, axis=1) / np.linalg.norm(o, axis=1)
+        assert err.max() <= 3e-6, err
