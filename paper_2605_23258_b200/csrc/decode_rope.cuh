@@ -135,7 +135,7 @@ __device__ __forceinline__ void sum_step64(uint32_t st, uint32_t base, bool reta
                     uint32_t pos0, pos1;
                     asm volatile("ld.shared.v2.u32 {%0,%1}, [%2];\n" : "=r"(pos0), "=r"(pos1) : "r"(st + C::STEP_POS + kk * 64 + r * 32 + tig * 8));
 #pragma unroll
-                    for (int p = 0; p < 2; ++p) turn_back_parts(rx[p][r], ry[p][r], (int)pos0, (int)pos1, phase[p], xp[p][r], yp[p][r]);
+                    for (int p = 0; p < 2; ++p) turn_back_parts(rx[p][r], ry[p][r], rope_angle((int)pos0, phase[p]), rope_angle((int)pos1, phase[p]), xp[p][r], yp[p][r]);
                 }
 #pragma unroll
                 for (int i = 2; i >= 0; --i)                              // the small parts first

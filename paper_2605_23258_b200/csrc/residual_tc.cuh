@@ -17,7 +17,9 @@
 // all stages but one behind the one being issued: 128 KB of row loads stay in flight.
 // With RoPE: the turned key is no longer a bf16 number, so it goes to the tensor cores as a bf16
 // pair hi + lo (two chains over the same W), which keeps it to 2^-17 relative; two stages of
-// K hi | K lo | V (96 KB each).  A loader thread takes its chunks of the keys straight into registers,
+// K hi | K lo | V (96 KB each).  At D = 64 it goes there as three bf16 parts, turned to fp32's own precision (rope.cuh): 64 KB a stage;
+// residuals are then off by 1.1e-7 to 1.4e-7 (2-norm, 64 units of 2000 rows; 2.6e-6 with two parts, 1.6e-7 on CUDA cores), and four
+// sequences of 8 layers of 20011 tokens take 153 us to route (137 and 942).  A loader thread takes its chunks of the keys straight into registers,
 // a pass of the next tile requested as soon as that pass of this tile has been read, turns its eight channel
 // pairs of each of its rows back and writes hi and lo; the values follow with cp.async and a barrier of
 // their own.  With the keys landing in the stage, a tile's loads waited for the epilogue of the tile before last.
@@ -26,6 +28,7 @@
 
 #include "common.cuh"
 #include "internal.h"
+#include "rope.cuh"
 #include "tcgen05.cuh"
 #include "tma.cuh"
 
@@ -75,8 +78,9 @@ template <int D, bool ROPE> struct RCfg {
     static constexpr int OPERAND_BYTES = (D / 64) * BOX_BYTES;     // 128 rows of D bf16 as D / 64 swizzled boxes
     static constexpr int W_BYTES = 2 * D * D;
     static constexpr int STAGES = ROPE ? 2 : D == 128 ? 3 : 5;
-    static constexpr int STAGE_BYTES = (ROPE ? 3 : 2) * OPERAND_BYTES;
-    static constexpr int V_OFFSET = (ROPE ? 2 : 1) * OPERAND_BYTES;
+    static constexpr int PARTS = !ROPE ? 1 : D == 128 ? 2 : 3;     // bf16 parts of a key
+    static constexpr int STAGE_BYTES = (PARTS + 1) * OPERAND_BYTES;
+    static constexpr int V_OFFSET = PARTS * OPERAND_BYTES;
     static constexpr int SMEM_BYTES = STAGES * STAGE_BYTES + W_BYTES + 1024;
     static constexpr int TMEM_COLS = STAGES * D <= 128 ? 128 : STAGES * D <= 256 ? 256 : 512;   // one D-column accumulator per stage
     static constexpr int LOADER_WARPS = 8;
@@ -142,9 +146,15 @@ residual_tc(const __nv_bfloat16* __restrict__ K, const __nv_bfloat16* __restrict
         // the same chunk of the other half: in the second box, or LPR chunks further in the row
         const uint32_t other = D == 128 ? (uint32_t)BOX_BYTES : (uint32_t)(((qc + LPR) ^ (rsub & 7)) << 4) - (uint32_t)((qc ^ (rsub & 7)) << 4);
         constexpr uint32_t PASS_BYTES = RPP * 128;
-        uint2 fr[8];                                                 // phases of this thread's eight channel pairs
+        uint2 fr[8];                                                 // phases of this thread's eight channel pairs; D = 64: as signed words
 #pragma unroll
-        for (int e = 0; e < 8; ++e) fr[e] = reinterpret_cast<const uint2*>(phase_s)[qc * 8 + e];
+        for (int e = 0; e < 8; ++e) {
+            fr[e] = reinterpret_cast<const uint2*>(phase_s)[qc * 8 + e];
+            if constexpr (D == 64) {
+                const RopePhase w = rope_phase_words(phase_s[qc * 8 + e]);
+                fr[e] = make_uint2((uint32_t)w.lo, (uint32_t)w.hi);
+            }
+        }
         int32_t cur[PASSES], nxt[PASSES];
         Cursor at = cursor_at(gt_lo, P.tpu), ahead = at;             // the tile at hand; the tile whose rows are fetched next
         auto fetch_idx = [&](int32_t (&out)[PASSES]) {
@@ -175,11 +185,32 @@ residual_tc(const __nv_bfloat16* __restrict__ K, const __nv_bfloat16* __restrict
         // the next tile's keys (rows listed in next_rows) as soon as they have been read.
         auto turn_back = [&](int i, int s, const int32_t (&pos)[PASSES], const int32_t (&next_rows)[PASSES], const __nv_bfloat16* K_next) {
             const uint32_t hi0 = tma::smem_u32(stage0 + s * R_STAGE_BYTES) + dst_thread, lo0 = hi0 + OPERAND_BYTES;
+            auto store16 = [](uint32_t at, const uint32_t (&v)[4]) {
+                asm volatile("st.shared.v4.u32 [%0], {%1,%2,%3,%4};\n" ::"r"(at), "r"(v[0]), "r"(v[1]), "r"(v[2]), "r"(v[3]) : "memory");
+            };
 #pragma unroll
             for (int p = 0; p < PASSES; ++p) {
                 uint32_t xs[4] = {kx[p].x, kx[p].y, kx[p].z, kx[p].w}, ys[4] = {ky[p].x, ky[p].y, ky[p].z, ky[p].w}, xl[4], yl[4];
                 if (i + 1 < n_my) request(K_next, p, next_rows[p]);
                 const uint32_t tok = pos[p] >= 0 ? (uint32_t)pos[p] : 0u;      // rows past the list are zeros
+                if constexpr (D == 64) {
+                    uint32_t xp[3][4], yp[3][4];
+#pragma unroll
+                    for (int e = 0; e < 4; ++e) {
+                        uint32_t angle[2], xe[3], ye[3];
+#pragma unroll
+                        for (int h = 0; h < 2; ++h) angle[h] = rope_angle((int)tok, RopePhase{(int)fr[2 * e + h].y, (int)fr[2 * e + h].x});
+                        turn_back_parts(xs[e], ys[e], angle[0], angle[1], xe, ye);
+#pragma unroll
+                        for (int i = 0; i < 3; ++i) { xp[i][e] = xe[i]; yp[i][e] = ye[i]; }
+                    }
+#pragma unroll
+                    for (int i = 0; i < 3; ++i) {
+                        store16(hi0 + i * OPERAND_BYTES + p * PASS_BYTES, xp[i]);
+                        store16(hi0 + i * OPERAND_BYTES + other + p * PASS_BYTES, yp[i]);
+                    }
+                    continue;
+                }
 #pragma unroll
                 for (int e = 0; e < 4; ++e) {
                     float x[2], y[2], cs[2], sn[2], xo[2], yo[2];
@@ -200,10 +231,10 @@ residual_tc(const __nv_bfloat16* __restrict__ K, const __nv_bfloat16* __restrict
                     xl[e] = pack2_bf16(xo[0] - __uint_as_float(xs[e] << 16), xo[1] - __uint_as_float(xs[e] & 0xffff0000u));
                     yl[e] = pack2_bf16(yo[0] - __uint_as_float(ys[e] << 16), yo[1] - __uint_as_float(ys[e] & 0xffff0000u));
                 }
-                asm volatile("st.shared.v4.u32 [%0], {%1,%2,%3,%4};\n" ::"r"(hi0 + p * PASS_BYTES), "r"(xs[0]), "r"(xs[1]), "r"(xs[2]), "r"(xs[3]) : "memory");
-                asm volatile("st.shared.v4.u32 [%0], {%1,%2,%3,%4};\n" ::"r"(hi0 + other + p * PASS_BYTES), "r"(ys[0]), "r"(ys[1]), "r"(ys[2]), "r"(ys[3]) : "memory");
-                asm volatile("st.shared.v4.u32 [%0], {%1,%2,%3,%4};\n" ::"r"(lo0 + p * PASS_BYTES), "r"(xl[0]), "r"(xl[1]), "r"(xl[2]), "r"(xl[3]) : "memory");
-                asm volatile("st.shared.v4.u32 [%0], {%1,%2,%3,%4};\n" ::"r"(lo0 + other + p * PASS_BYTES), "r"(yl[0]), "r"(yl[1]), "r"(yl[2]), "r"(yl[3]) : "memory");
+                store16(hi0 + p * PASS_BYTES, xs);
+                store16(hi0 + other + p * PASS_BYTES, ys);
+                store16(lo0 + p * PASS_BYTES, xl);
+                store16(lo0 + other + p * PASS_BYTES, yl);
             }
             fence_async_proxy();
             tma::mbar_arrive(&sy.full[s]);
@@ -307,18 +338,14 @@ residual_tc(const __nv_bfloat16* __restrict__ K, const __nv_bfloat16* __restrict
                 if (i == 0) asm volatile("griddepcontrol.wait;\n" ::: "memory");
                 if (!tma::mbar_wait(&sy.full[s], round & 1, fault, 49)) break;
                 tc::fence_after_sync();
-                const uint32_t hi_addr = tma::smem_u32(stage0 + s * R_STAGE_BYTES), lo_addr = hi_addr + OPERAND_BYTES;
-                const uint32_t d = sy.tmem_base + s * D;
+                const uint32_t k_addr = tma::smem_u32(stage0 + s * R_STAGE_BYTES), d = sy.tmem_base + s * D;
 #pragma unroll
-                for (int ks = 0; ks < D / 16; ++ks) {
-                    const uint32_t o = (ks >> 2) * BOX_BYTES + (ks & 3) * 32;
-                    tc::mma_bf16(d, tc::smem_desc(hi_addr + o), tc::smem_desc(w_addr + o), idesc, ks > 0);
-                }
-                if (ROPE) {
+                for (int x = 0; x < C::PARTS; ++x) {
+                    const uint32_t part = k_addr + (D == 64 ? C::PARTS - 1 - x : x) * OPERAND_BYTES;     // three parts: the smallest first
 #pragma unroll
                     for (int ks = 0; ks < D / 16; ++ks) {
                         const uint32_t o = (ks >> 2) * BOX_BYTES + (ks & 3) * 32;
-                        tc::mma_bf16(d, tc::smem_desc(lo_addr + o), tc::smem_desc(w_addr + o), idesc, 1u);
+                        tc::mma_bf16(d, tc::smem_desc(part + o), tc::smem_desc(w_addr + o), idesc, x > 0 || ks > 0 ? 1u : 0u);
                     }
                 }
                 tc::mma_commit(&sy.done[s]);

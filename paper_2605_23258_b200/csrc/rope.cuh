@@ -18,13 +18,16 @@ __device__ __forceinline__ RopePhase rope_phase_words(unsigned long long phase) 
     return p;
 }
 
-// Sine and cosine of the rotary angles of two positions.  Integer arithmetic takes the angle to the nearest quarter turn and
+// The angle at a position as a 32-bit fraction of a turn.
+__device__ __forceinline__ uint32_t rope_angle(int32_t pos, RopePhase ph) {
+    return (uint32_t)pos * (uint32_t)ph.hi + (uint32_t)__mulhi(pos, ph.lo);
+}
+// Sine and cosine of two such angles.  Integer arithmetic takes an angle to the nearest quarter turn and
 // what remains of it, in [-pi/4, pi/4]; there the Taylor series about zero are good to 2e-9 (sine, five terms) and 2e-10 (cosine,
 // six), and a quarter turn swaps the two or changes their signs.
-__device__ __forceinline__ void rope_cos_sin2(int32_t pos0, int32_t pos1, RopePhase ph, uint64_t& cs2, uint64_t& sn2) {
+__device__ __forceinline__ void rope_cos_sin2(uint32_t angle0, uint32_t angle1, uint64_t& cs2, uint64_t& sn2) {
     // an eighth of a turn more: the upper two bits are the quarter turns, the rest less an eighth what remains
-    const uint32_t u0 = (uint32_t)pos0 * (uint32_t)ph.hi + (uint32_t)__mulhi(pos0, ph.lo) + 0x20000000u;
-    const uint32_t u1 = (uint32_t)pos1 * (uint32_t)ph.hi + (uint32_t)__mulhi(pos1, ph.lo) + 0x20000000u;
+    const uint32_t u0 = angle0 + 0x20000000u, u1 = angle1 + 0x20000000u;
     const float r0 = (float)((int)(u0 & 0x3fffffffu) - 0x20000000), r1 = (float)((int)(u1 & 0x3fffffffu) - 0x20000000);
     const uint64_t z = tc::mul2(tc::pack2(r0, r1), tc::pack2(1.4629180792671596e-9f, 1.4629180792671596e-9f));      // 2 pi / 2^32
     const uint64_t zz = tc::mul2(z, z);
@@ -65,11 +68,10 @@ __device__ __forceinline__ void split_bf16(float p0, float p1, uint32_t (&part)[
     }
 }
 
-// Channels x and y of a pair, two keys (bf16) to a register, turned back by the keys' positions, in three parts each.
-__device__ __forceinline__ void turn_back_parts(uint32_t x, uint32_t y, int32_t pos0, int32_t pos1, RopePhase ph, uint32_t (&xp)[3],
-                                                uint32_t (&yp)[3]) {
+// Two channels x with their partners y (bf16, two to a register), turned back by their angles, in three parts each.
+__device__ __forceinline__ void turn_back_parts(uint32_t x, uint32_t y, uint32_t angle0, uint32_t angle1, uint32_t (&xp)[3], uint32_t (&yp)[3]) {
     uint64_t cs, sn;
-    rope_cos_sin2(pos0, pos1, ph, cs, sn);
+    rope_cos_sin2(angle0, angle1, cs, sn);
     const uint64_t x2 = tc::pack2(__uint_as_float(x << 16), __uint_as_float(x & 0xffff0000u));
     const uint64_t y2 = tc::pack2(__uint_as_float(y << 16), __uint_as_float(y & 0xffff0000u));
     float a, b;

@@ -144,3 +144,33 @@ def test_decode_head64_rope_keeps_large_keys(oracle):
                              apx_pos=pos[u].cpu().numpy(), rope=True, theta=10000.0)
         err = np.linalg.norm(out[u].cpu().double().numpy() - o, axis=1) / np.linalg.norm(o, axis=1)
         assert err.max() <= 3e-6, err
+
+
+@pytest.mark.parametrize("rope", [False, True])
+@pytest.mark.parametrize("units,n_idx", [(3, 129), (200, 700)])
+def test_residual_head64_keeps_fp32_precision(oracle, rope, units, n_idx):
+    """Residuals of values that the map nearly gives: (eps - want) / (2 sqrt(want)) is the error of W k~ along the residual.
+    fp32 leaves a few 2^-24 of the prediction's size, keys kept to 2^-17 about 2^-18.5 of it: at most 2^-22 in the mean square."""
+    d, N = 64, 900
+    gen = torch.Generator(device=DEV).manual_seed(23)
+    K = torch.randn(units, N, d, generator=gen, device=DEV).to(torch.bfloat16)
+    W = (torch.randn(units, d, d, generator=gen, device=DEV) / 8).to(torch.bfloat16)
+    k = K.double()
+    if rope:                                                  # turned back by the token's index
+        angle = torch.arange(N, device=DEV).double()[:, None] * 10000.0 ** (-2.0 * torch.arange(d // 2, device=DEV).double() / d)
+        cs, sn, x, y = torch.cos(angle), torch.sin(angle), k[..., :d // 2], k[..., d // 2:]
+        k = torch.cat([x * cs + y * sn, y * cs - x * sn], dim=-1)
+    pred = torch.bmm(k, W.double().transpose(1, 2))
+    V = (pred + 0.05 * torch.randn(units, N, d, generator=gen, device=DEV)).to(torch.bfloat16)
+    idx = torch.stack([torch.randperm(N, generator=gen, device=DEV)[:n_idx].sort().values for _ in range(units)]).to(torch.int32)
+    sh = vec.Shape(1, 1, units, units, d, vec.VECTOR_BF16, 16, 7, 0.0, int(rope), 10000.0)
+    eps = torch.full((units, n_idx), float("nan"), device=DEV)
+    vec.vector_residual(sh, K, V, W, N, idx, n_idx, eps)
+    torch.cuda.synchronize()
+    assert vec.vector_device_fault() == 0
+    errs = []
+    for u in range(0, units, max(1, units // 8)):
+        want = oracle.residual(K[u].cpu(), V[u].cpu(), W[u].cpu(), idx[u].cpu().numpy(), rope=rope, theta=10000.0)
+        errs.append((eps[u].cpu().double().numpy() - want) / (2 * np.sqrt(want)))
+    rms = float(np.sqrt(np.mean(np.concatenate(errs) ** 2)) / pred.pow(2).mean().sqrt())
+    assert rms <= 2.0 ** -22, rms
