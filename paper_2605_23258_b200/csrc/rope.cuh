@@ -56,15 +56,20 @@ __device__ __forceinline__ void rope_cos_sin2(uint32_t angle0, uint32_t angle1, 
     sn2 = tc::pack2(s0, s1);
 }
 
-// A pair of numbers as bf16 parts: the upper halves of the words, then the same of what they leave; three parts hold all 24 bits.
+// A pair of numbers as bf16 parts, each a part of what the ones before it leave.  Three are the upper halves of the words, cut off:
+// together they hold all 24 bits.  Two are rounded, which halves what they lose and leaves it without a bias.
 template <int PARTS>
 __device__ __forceinline__ void split_bf16(float p0, float p1, uint32_t (&part)[PARTS]) {
 #pragma unroll
     for (int i = 0; i < PARTS; ++i) {
-        part[i] = __byte_perm(__float_as_uint(p0), __float_as_uint(p1), 0x7632);
+        if constexpr (PARTS == 3) {
+            part[i] = __byte_perm(__float_as_uint(p0), __float_as_uint(p1), 0x7632);
+        } else {
+            const __nv_bfloat162 v = __floats2bfloat162_rn(p0, p1);
+            part[i] = *reinterpret_cast<const uint32_t*>(&v);
+        }
         if (i + 1 < PARTS)
-            tc::unpack2(tc::fma2(tc::pack2(__float_as_uint(p0) & 0xffff0000u, __float_as_uint(p1) & 0xffff0000u), tc::pack2(-1.f, -1.f),
-                                 tc::pack2(p0, p1)), p0, p1);
+            tc::unpack2(tc::fma2(tc::pack2(part[i] << 16, part[i] & 0xffff0000u), tc::pack2(-1.f, -1.f), tc::pack2(p0, p1)), p0, p1);
     }
 }
 
