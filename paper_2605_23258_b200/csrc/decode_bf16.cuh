@@ -45,10 +45,11 @@ namespace dbf {
 
 constexpr int KEYS = 64;                     // keys per softmax step (and per TMA box)
 constexpr int BOX_BYTES = 8192;              // 64 rows x 128 bytes
-// The softmax's reference follows the running maximum only when that has moved by more than SLACK (in powers of two): any
-// reference serves, weights up to 2^SLACK cost no precision, and the accumulators are rescaled a few times instead of in every
-// other step (a step of 512 units of 4915 rows, 64 channels: 73.9 -> 72.3 us, with RoPE 131.4 -> 125.8; 128 channels 132.1 ->
-// 131.4 and 170.2 -> 166.8).  tc::ex2 gives zero below 2^-126: next to a weight of at least 2^-SLACK that changes no fp32 sum.
+// 64 channels: the softmax's reference follows the running maximum only when that has moved by more than SLACK (in powers of two):
+// any reference serves weights that keep all 24 bits, and the sums are rescaled a few times instead of in every other step.
+// Weights that keep sixteen bits want the running maximum itself: the largest of them is one then, and exact (with the slack, 131.4
+// against 132.1 us for 512 units of 4915 rows, 128 channels, the outputs were off by up to a quarter more).
+// tc::ex2 gives zero below 2^-126: next to a weight of at least 2^-SLACK that changes no fp32 sum.
 constexpr float SLACK = 8.f;
 template <int D, bool ROPE> struct Cfg {
     static constexpr int HALF_BYTES = 64 * 2 * D;                    // 64 rows as D / 64 swizzled boxes
@@ -251,7 +252,7 @@ __device__ __forceinline__ float score_step(uint32_t kbase, int nrows, float sca
     }
     mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 1));
     mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 2));
-    const float m_new = mx > m + SLACK ? mx : m;      // finite: key 0 of the step is valid for every row
+    const float m_new = fmaxf(m, mx);                 // finite: key 0 of the step is valid for every row
     const float alpha = tc::ex2(m - m_new);           // 0 on the first step
     float ls = 0.f;
 #pragma unroll

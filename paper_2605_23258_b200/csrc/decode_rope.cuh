@@ -78,7 +78,7 @@ __device__ __forceinline__ void score_step_keys(uint32_t kbase, int nrows, float
         for (int e = 0; e < 2; ++e) mx[e] = fmaxf(mx[e], __shfl_xor_sync(0xffffffffu, mx[e], o));
 #pragma unroll
     for (int e = 0; e < 2; ++e) {
-        const float m_new = mx[e] > m[e] + SLACK ? mx[e] : m[e];       // finite: key 0 of the step is valid for every head
+        const float m_new = mx[e] > m[e] + (Cfg<D, true>::EXACT ? SLACK : 0.f) ? mx[e] : m[e];       // finite: key 0 of the step is valid for every head
         alpha[e] = tc::ex2(m[e] - m_new);                              // 0 on the first step
         m[e] = m_new;
         l[e] *= alpha[e];
