@@ -19,7 +19,7 @@
 //   warps 0-7   loaders: gathers of the K rows of a step (cp.async, written in the 128-byte-swizzled operand layout),
 //               published three steps behind the one being issued; thread 0 also issues the W loads (TMA)
 //   warp  8     MMA issuer, TMEM owner (two 256-column accumulators: the epilogue of a pair runs under the next one)
-//   warps 9-12  epilogue: thread = row; its value row comes in 32-byte loads, a head ahead
+//   warps 9-12  epilogue: thread = row; its value row comes in 32-byte loads (16-byte ones where it has to), a head ahead
 // Measured on 16 layers of 4914 listed tokens and 8 heads: 245 us (388 before: one output head at a time, loads waited for in
 // every step, 64-bit divisions in every role), 53 KB a microsecond and multiprocessor: the rate at which L2 delivers.
 #ifndef VECTOR_RESIDUAL_LAYER_TC_CUH_
@@ -70,16 +70,27 @@ __device__ __forceinline__ Cursor cursor_at(long long item, const Params& P) {
     c.t = (int)(tile - (long long)c.ul * P.tpu);
     return c;
 }
-// 32 bytes through the read-only path.
+// 32 bytes through the read-only path: in one load (WIDE, the address a multiple of 32) or in two.
+template <bool WIDE>
 __device__ __forceinline__ void ldg32(const void* p, uint32_t (&r)[64], int at) {
-    asm volatile("ld.global.nc.v8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];\n"
-                 : "=r"(r[at]), "=r"(r[at + 1]), "=r"(r[at + 2]), "=r"(r[at + 3]), "=r"(r[at + 4]), "=r"(r[at + 5]), "=r"(r[at + 6]), "=r"(r[at + 7])
-                 : "l"(p));
+    if constexpr (WIDE) {
+        asm volatile("ld.global.nc.v8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];\n"
+                     : "=r"(r[at]), "=r"(r[at + 1]), "=r"(r[at + 2]), "=r"(r[at + 3]), "=r"(r[at + 4]), "=r"(r[at + 5]), "=r"(r[at + 6]), "=r"(r[at + 7])
+                     : "l"(p));
+    } else {
+#pragma unroll
+        for (int h = 0; h < 8; h += 4)
+            asm volatile("ld.global.nc.v4.b32 {%0,%1,%2,%3}, [%4];\n"
+                         : "=r"(r[at + h]), "=r"(r[at + h + 1]), "=r"(r[at + h + 2]), "=r"(r[at + h + 3])
+                         : "l"((const unsigned char*)p + 4 * h));
+    }
 }
 
 // grid: at most one block per multiprocessor and a range of at least `pairs` items each (so that a tile is cut once at
 // most), THREADS threads, SMEM_BYTES dynamic shared memory.
 // K, V: [UL][Hkv][N][128]; idx: [UL][n_idx]; eps: [UL][n_idx], zero; mapW: (Hkv*128 in, Hkv*128 out, L), box 64 x 128.
+// WIDE: V is a multiple of 32 bytes.  The interface promises 16; rows are 256 bytes apart, so the base decides for all of them.
+template <bool WIDE>
 __global__ void __launch_bounds__(THREADS, 1)
 residual_layer_tc(const __nv_bfloat16* __restrict__ K, const __nv_bfloat16* __restrict__ V,
                   const __grid_constant__ CUtensorMap mapW, const int32_t* __restrict__ idx, const Params P,
@@ -208,7 +219,7 @@ residual_layer_tc(const __nv_bfloat16* __restrict__ K, const __nv_bfloat16* __re
         };
         uint32_t vv[64];                                    // the value row of the head at hand, replaced 64 bytes at a time by the next one's
         auto fetch = [&](const unsigned char* src, int ch) {
-            if (src) { ldg32(src + ch * 64, vv, 16 * ch); ldg32(src + ch * 64 + 32, vv, 16 * ch + 8); }
+            if (src) { ldg32<WIDE>(src + ch * 64, vv, 16 * ch); ldg32<WIDE>(src + ch * 64 + 32, vv, 16 * ch + 8); }
             else {
 #pragma unroll
                 for (int k = 0; k < 16; ++k) vv[16 * ch + k] = 0u;

@@ -392,8 +392,9 @@ static vector_status residual_layer_dispatch(const Dims& dm, int Hkv, int L, con
     if (dm.dtype == VECTOR_BF16 && dm.d == 128) {
         static PerDeviceOnce once;
         if (once.first()) {
-            const cudaError_t e = cudaFuncSetAttribute(rlt::residual_layer_tc, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                       rlt::SMEM_BYTES);
+            cudaError_t e = cudaFuncSetAttribute(rlt::residual_layer_tc<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, rlt::SMEM_BYTES);
+            if (e == cudaSuccess)
+                e = cudaFuncSetAttribute(rlt::residual_layer_tc<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, rlt::SMEM_BYTES);
             if (e != cudaSuccess) { once.undo(); VEC_CUDA_CHECK(e); }
         }
         int* fault = kernel_fault_address();
@@ -411,7 +412,8 @@ static vector_status residual_layer_dispatch(const Dims& dm, int Hkv, int L, con
         // a block gets at least a tile, or exactly half of one where that leaves no more blocks than multiprocessors
         const int blocks = (int)(tiles >= sms ? sms : 2 * tiles <= sms && P.pairs > 1 ? 2 * tiles : tiles);
         if (!eps_zeroed) VEC_CUDA_CHECK(cudaMemsetAsync(eps, 0, (size_t)UL * (size_t)n_idx * sizeof(float), st));
-        VEC_CUDA_CHECK(launch_maybe_dependent(dependent, rlt::residual_layer_tc, dim3(blocks), dim3(rlt::THREADS), rlt::SMEM_BYTES,
+        auto kern = ((uintptr_t)V & 31) == 0 ? rlt::residual_layer_tc<true> : rlt::residual_layer_tc<false>;
+        VEC_CUDA_CHECK(launch_maybe_dependent(dependent, kern, dim3(blocks), dim3(rlt::THREADS), rlt::SMEM_BYTES,
                                               st, (const __nv_bfloat16*)K, (const __nv_bfloat16*)V, mapW, idx, P, eps, fault));
         return VECTOR_OK;
     }

@@ -37,3 +37,24 @@ def test_residual_layer(oracle, layers, Hkv, n_idx):
         dn = np.sqrt((((D + 2) * 2.0 ** -23 * (np.abs(v) + np.abs(k) @ np.abs(w).T)) ** 2).sum(1))
         err = np.abs(eps[0][l].double().cpu().numpy() - want)
         assert np.all(err <= 2 * np.sqrt(want) * dn + dn ** 2 + 2.0 ** -20 * want), (l, float(err.max()))
+
+
+@pytest.mark.parametrize("layers,Hkv,n_idx", [(2, 3, 129), (30, 8, 300)])
+def test_residual_layer_values_at_16_bytes(layers, Hkv, n_idx):
+    """Values that begin at an odd multiple of 16 bytes, which is all that the interface asks for: the same residuals to the bit."""
+    N, d = 400, 128
+    gen = torch.Generator(device=DEV).manual_seed(7)
+    K = torch.randn(layers * Hkv, N, d, generator=gen, device=DEV).to(torch.bfloat16)
+    V = torch.randn(layers * Hkv, N, d, generator=gen, device=DEV).to(torch.bfloat16)
+    W = (torch.randn(layers, Hkv * d, Hkv * d, generator=gen, device=DEV) / np.sqrt(Hkv * d)).to(torch.bfloat16)
+    shifted = torch.empty(V.numel() + 8, dtype=torch.bfloat16, device=DEV)[8:].view(V.shape)
+    shifted.copy_(V)
+    assert V.data_ptr() % 32 == 0 and shifted.data_ptr() % 32 == 16
+    idx = torch.stack([torch.randperm(N, generator=gen, device=DEV)[:n_idx].sort().values for _ in range(layers)]).to(torch.int32)
+    sh = vec.Shape(1, layers, 2 * Hkv, Hkv, d, vec.VECTOR_BF16, 16)
+    eps = [torch.full((layers, n_idx), float("nan"), device=DEV) for _ in range(2)]
+    for e, v in zip(eps, (V, shifted)):
+        vec.vector_residual_layer(sh, K, v, W, N, idx, n_idx, e)
+    torch.cuda.synchronize()
+    assert vec.vector_device_fault() == 0
+    assert torch.equal(eps[0], eps[1])
