@@ -235,7 +235,7 @@ VECTOR_API vector_status vector_compact(const vector_shape* shape, const vector_
 /*
  * Appends a generated token in full: k_new, v_new (device [U][d] of shape->dtype) become row cache->n_ret of ret_k and
  * ret_v, and pos its entry of ret_pos, for every unit.  The caller bumps n_ret afterwards.  VECTOR_ERR_SHAPE if the
- * retained pool is full.
+ * retained pool is full, or if k_new, v_new, ret_k or ret_v is not a multiple of 16 bytes.
  */
 VECTOR_API vector_status vector_append(const vector_shape* shape, const vector_cache* cache, const void* k_new,
                                        const void* v_new, int32_t pos, void* stream);

@@ -140,6 +140,7 @@ extern "C" vector_status vector_append(const vector_shape* shape, const vector_c
     if (rc != VECTOR_OK) return rc;
     if (!cache || !k_new || !v_new || !cache->ret_k || !cache->ret_v || !cache->ret_pos) return VECTOR_ERR_NULL;
     if (cache->n_ret < 0 || cache->n_ret >= cache->cap_ret) return VECTOR_ERR_SHAPE;
+    if (((uintptr_t)k_new | (uintptr_t)v_new | (uintptr_t)cache->ret_k | (uintptr_t)cache->ret_v) & 15) return VECTOR_ERR_SHAPE;
     const int lp = log2_pieces(dm);
     const long long n = (long long)dm.U << (lp + 1);
     VEC_CUDA_CHECK(launch_maybe_dependent(true, append_kernel, dim3((unsigned)((n + 255) / 256)), dim3(256), 0, (cudaStream_t)stream,

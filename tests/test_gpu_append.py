@@ -1,5 +1,5 @@
 """Appending a generated token: the rows, their neighbours and the positions, bit for bit, for every row width; and inputs
-that are assigned rather than copied (another type, broadcast, strided)."""
+that are assigned rather than copied (another type, broadcast, strided, off a 16-byte boundary)."""
 import pytest
 import torch
 
@@ -36,3 +36,26 @@ def test_append_rows(dtype, d, U):
     with pytest.raises(vec.VectorError) as e:
         vec.vector_append(sh, c, steps[0][0], steps[0][1], 0)
     assert e.value.status == -2
+
+
+def _shifted(x):
+    """The same rows, contiguous, one element into their storage."""
+    y = torch.empty(x.numel() + 1, dtype=x.dtype, device=x.device)[1:].view(x.shape)
+    return y.copy_(x)
+
+
+@pytest.mark.parametrize("dtype", [torch.float32, torch.bfloat16])
+def test_append_rows_off_a_16_byte_boundary(dtype):
+    U, d = 3, 64
+    sh = vec.Shape(1, 1, U, U, d, vec.VECTOR_BF16 if dtype == torch.bfloat16 else vec.VECTOR_F32, 16)
+    comp = Compressor(sh, vec.vector_plan_budget(200, 60, 10, 16), extra_rows=3)
+    c, n = comp.cache, comp.cache.n_ret
+    k, v = (torch.randn(U, d, device=DEV).to(dtype) for _ in range(2))
+    for a, b in ((_shifted(k), v), (k, _shifted(v))):
+        assert (a.data_ptr() | b.data_ptr()) % 16 and a.is_contiguous() and b.is_contiguous()
+        comp.append(a, b, 5)
+        assert torch.equal(c.ret_k[:, c.n_ret - 1], k) and torch.equal(c.ret_v[:, c.n_ret - 1], v)
+        with pytest.raises(vec.VectorError) as e:
+            vec.vector_append(sh, c, a, b, 5)
+        assert e.value.status == -2
+    assert c.n_ret == n + 2 and (c.ret_pos[:, n:n + 2] == 5).all()

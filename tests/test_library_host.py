@@ -126,3 +126,15 @@ def test_synthetic_inputs_are_deterministic_and_shaped():
     q = synth.decode_q(wl, 3, "cpu", sq)
     assert q.shape == (8, 4, 128)
     assert torch.equal(q[[2]], synth.decode_q(wl, 3, "cpu", sq, units=[2]))
+
+
+def test_append_to_rows_in_host_memory():
+    """Rows that are assigned rather than copied by a kernel: a cache in host memory."""
+    from paper_2605_23258_b200.pipeline import Compressor
+    sh = vec.Shape(1, 1, 2, 2, 64, vec.VECTOR_F32, 16)
+    comp = Compressor(sh, vec.vector_plan_budget(200, 60, 10, 16), extra_rows=1, device="cpu")
+    c, n = comp.cache, comp.cache.n_ret
+    k, v = torch.randn(2, 64), torch.randn(2, 64)
+    comp.append(k, v, 7)
+    assert c.n_ret == n + 1
+    assert torch.equal(c.ret_k[:, n], k) and torch.equal(c.ret_v[:, n], v) and (c.ret_pos[:, n] == 7).all()
