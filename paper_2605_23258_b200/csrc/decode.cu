@@ -5,8 +5,8 @@
 // both pools once, accumulating p-weighted values and p-weighted keys, and the
 // d x d map is applied once per query head in the merge step.
 //
-// bf16 runs the kernels of decode_bf16.cuh and decode_pertile_tc.cuh; below, for fp32, one
-// launch: a thread block cluster per unit, its blocks a slice each of the logical key range
+// bf16 runs the kernels of decode_bf16.cuh and decode_pertile_tc.cuh; below, for fp32 (and 64-channel bf16 rows off a
+// 16-byte boundary), one launch: a thread block cluster per unit, its blocks a slice each of the logical key range
 // [0, n_ret + n_apx); the blocks' sums are merged over distributed shared memory.
 #include <cmath>
 #include <mutex>
@@ -20,19 +20,22 @@
 
 namespace vec {
 
-template <int EPL> struct RowLoad;
-template <> struct RowLoad<4> {
-    static __device__ __forceinline__ void load(const float* p, int lane, float (&o)[4]) {
-        float4 v = reinterpret_cast<const float4*>(p)[lane];
-        o[0] = v.x; o[1] = v.y; o[2] = v.z; o[3] = v.w;
+// EPL consecutive elements of a row; wide: the rows lie at multiples of 16 bytes (fp32), otherwise, and for bf16, one by one.
+template <int EPL, typename T>
+__device__ __forceinline__ void row_load(const T* __restrict__ p, int lane, bool wide, float (&o)[EPL]) {
+    if (sizeof(T) == 4 && wide) {
+        if constexpr (EPL == 4) {
+            const float4 v = reinterpret_cast<const float4*>(p)[lane];
+            o[0] = v.x; o[1] = v.y; o[2] = v.z; o[3] = v.w;
+        } else {
+            const float2 v = reinterpret_cast<const float2*>(p)[lane];
+            o[0] = v.x; o[1] = v.y;
+        }
+    } else {
+#pragma unroll
+        for (int e = 0; e < EPL; ++e) o[e] = to_f32(p[lane * EPL + e]);
     }
-};
-template <> struct RowLoad<2> {
-    static __device__ __forceinline__ void load(const float* p, int lane, float (&o)[2]) {
-        float2 v = reinterpret_cast<const float2*>(p)[lane];
-        o[0] = v.x; o[1] = v.y;
-    }
-};
+}
 
 // Record of a warp or a block, per head: m, l, pad, acc_v[D], acc_k[D].
 template <int D> struct Rec { static constexpr int floats = 4 + 2 * D; };
@@ -45,11 +48,11 @@ constexpr int F32_WARPS = 8, F32_ROWS = 4, F32_MAX_CLUSTER = 16;
 // (apx_pos): the logit still uses the stored key, only the p-weighted key sum takes the turned one.
 // A lane holds EPL consecutive channels; the partner channel c +- D/2 sits in lane ^ 16.
 // grid (U x cluster size), 256 threads, F32_WARPS * g records of dynamic shared memory.
-template <int D, int G, bool ROPE>
+template <typename T, int D, int G, bool ROPE>
 __global__ void __launch_bounds__(32 * F32_WARPS)
-decode_f32(const float* __restrict__ q, const float* __restrict__ ret_k, const float* __restrict__ ret_v,
-           const float* __restrict__ apx_k, const int32_t* __restrict__ apx_pos, int64_t cap_ret, int64_t cap_apx, int n_ret,
-           int n_apx, int g, int LH, float scale, float theta, const float* __restrict__ W, void* __restrict__ out, int out_bf16) {
+decode_rows(const T* __restrict__ q, const T* __restrict__ ret_k, const T* __restrict__ ret_v, const T* __restrict__ apx_k,
+           const int32_t* __restrict__ apx_pos, int64_t cap_ret, int64_t cap_apx, int n_ret, int n_apx, int g, int LH, float scale,
+           float theta, const T* __restrict__ W, bool wide, void* __restrict__ out, int out_bf16) {
     constexpr int EPL = D / 32, REC = Rec<D>::floats, NT = 32 * F32_WARPS;
     extern __shared__ __align__(16) float recs[];               // [F32_WARPS][g][REC]
     __shared__ __align__(16) float comb[G][REC];                // this block's sums, read by the whole cluster
@@ -73,7 +76,7 @@ decode_f32(const float* __restrict__ q, const float* __restrict__ ret_k, const f
 #pragma unroll
         for (int e = 0; e < EPL; ++e) { av[a][e] = 0.f; ak[a][e] = 0.f; qr[a][e] = 0.f; }
         if (a < g) {
-            RowLoad<EPL>::load(q + ((size_t)u * g + a) * D, lane, qr[a]);
+            row_load(q + ((size_t)u * g + a) * D, lane, wide, qr[a]);
 #pragma unroll
             for (int e = 0; e < EPL; ++e) qr[a][e] *= scale;
         }
@@ -86,8 +89,8 @@ decode_f32(const float* __restrict__ q, const float* __restrict__ ret_k, const f
 #pragma unroll
             for (int e = 0; e < EPL; ++e) { kx[r][e] = 0.f; vx[r][e] = 0.f; }
             if (i < hi) {
-                RowLoad<EPL>::load(i < n_ret ? ret_k + ((size_t)u * cap_ret + i) * D : apx_k + ((size_t)u * cap_apx + (i - n_ret)) * D, lane, kx[r]);
-                if (i < n_ret) RowLoad<EPL>::load(ret_v + ((size_t)u * cap_ret + i) * D, lane, vx[r]);
+                row_load(i < n_ret ? ret_k + ((size_t)u * cap_ret + i) * D : apx_k + ((size_t)u * cap_apx + (i - n_ret)) * D, lane, wide, kx[r]);
+                if (i < n_ret) row_load(ret_v + ((size_t)u * cap_ret + i) * D, lane, wide, vx[r]);
             }
         }
 #pragma unroll
@@ -169,10 +172,10 @@ decode_f32(const float* __restrict__ q, const float* __restrict__ ret_k, const f
     }
     // the map, a row across a warp's lanes, requested before the cluster's barrier
     constexpr int ROWS = D / F32_WARPS;
-    const float* Wu = W + (size_t)(u % LH) * D * D;
+    const T* Wu = W + (size_t)(u % LH) * D * D;
     float wr[ROWS][EPL];
 #pragma unroll
-    for (int r = 0; r < ROWS; ++r) RowLoad<EPL>::load(Wu + (size_t)(r * F32_WARPS + wid) * D, lane, wr[r]);
+    for (int r = 0; r < ROWS; ++r) row_load(Wu + (size_t)(r * F32_WARPS + wid) * D, lane, wide, wr[r]);
     cl::arrive_release();
     cl::wait_acquire();                                         // every block's sums are ready
     const int mine = rank < g ? (g - rank + C - 1) / C : 0;     // this block merges heads rank, rank + C, ...
@@ -209,7 +212,7 @@ decode_f32(const float* __restrict__ q, const float* __restrict__ ret_k, const f
     __syncthreads();
     for (int k = 0; k < mine; ++k) {
         float a[EPL];
-        RowLoad<EPL>::load(aks[k], lane, a);
+        row_load<EPL, float>(aks[k], lane, true, a);
 #pragma unroll
         for (int r = 0; r < ROWS; ++r) {
             float x = 0.f;
@@ -229,16 +232,24 @@ decode_f32(const float* __restrict__ q, const float* __restrict__ ret_k, const f
     cl::wait_acquire();                                         // nobody reads this block's memory any more
 }
 
-template <int D, int G, bool ROPE>
-static vector_status launch_decode_f32(const Dims& dm, const void* q, const vector_cache* ch, const void* W, void* out,
+static bool rows_at_16_bytes(const void* q, const vector_cache* ch, const void* W) {
+    uintptr_t all = (uintptr_t)q | (uintptr_t)W;
+    if (ch->n_ret > 0) all |= (uintptr_t)ch->ret_k | (uintptr_t)ch->ret_v;
+    if (ch->n_apx > 0) all |= (uintptr_t)ch->apx_k;
+    return (all & 15) == 0;
+}
+
+template <typename T, int D, int G, bool ROPE>
+static vector_status launch_decode_rows(const Dims& dm, const void* q, const vector_cache* ch, const void* W, void* out,
                                        int out_dtype, cudaStream_t st) {
-    auto kern = decode_f32<D, G, ROPE>;
+    auto kern = decode_rows<T, D, G, ROPE>;
     static PerDeviceOnce once;
     if (once.first()) {
         cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, F32_WARPS * G * Rec<D>::floats * 4);
         if (e == cudaSuccess) e = cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
         if (e != cudaSuccess) { once.undo(); VEC_CUDA_CHECK(e); }
     }
+    const bool wide = rows_at_16_bytes(q, ch, W);
     // blocks a unit: one pass over the rows of a block's warps at the least, four blocks a multiprocessor at the most
     const int64_t rows = ch->n_ret + ch->n_apx;
     int64_t c = (rows + F32_ROWS * F32_WARPS - 1) / (F32_ROWS * F32_WARPS);
@@ -247,9 +258,9 @@ static vector_status launch_decode_f32(const Dims& dm, const void* q, const vect
     if (c > F32_MAX_CLUSTER) c = F32_MAX_CLUSTER;
     if (c > 8 && c < F32_MAX_CLUSTER) c = 8;                    // beyond the portable size only the largest
     VEC_CUDA_CHECK(launch_maybe_dependent(true, (int)c, kern, dim3((unsigned)(c * dm.U)), dim3(32 * F32_WARPS),
-                                          (size_t)F32_WARPS * dm.g * Rec<D>::floats * 4, st, (const float*)q, (const float*)ch->ret_k,
-                                          (const float*)ch->ret_v, (const float*)ch->apx_k, ch->apx_pos, ch->cap_ret, ch->cap_apx,
-                                          (int)ch->n_ret, (int)ch->n_apx, dm.g, dm.LH, dm.scale, dm.theta, (const float*)W, out,
+                                          (size_t)F32_WARPS * dm.g * Rec<D>::floats * 4, st, (const T*)q, (const T*)ch->ret_k,
+                                          (const T*)ch->ret_v, (const T*)ch->apx_k, ch->apx_pos, ch->cap_ret, ch->cap_apx,
+                                          (int)ch->n_ret, (int)ch->n_apx, dm.g, dm.LH, dm.scale, dm.theta, (const T*)W, wide, out,
                                           out_dtype == VECTOR_BF16 ? 1 : 0));
     return VECTOR_OK;
 }
@@ -395,12 +406,12 @@ static vector_status launch_decode_bf16(const Dims& dm, const void* q, const vec
     return VECTOR_OK;
 }
 
-template <int D, bool ROPE>
+template <typename T, int D, bool ROPE>
 static vector_status launch_decode_g(const Dims& dm, const void* q, const vector_cache* ch, const void* W, void* out, int out_dtype,
                                      cudaStream_t st) {
-    if (dm.g <= 2) return launch_decode_f32<D, 2, ROPE>(dm, q, ch, W, out, out_dtype, st);
-    if (dm.g <= 4) return launch_decode_f32<D, 4, ROPE>(dm, q, ch, W, out, out_dtype, st);
-    return launch_decode_f32<D, 8, ROPE>(dm, q, ch, W, out, out_dtype, st);
+    if (dm.g <= 2) return launch_decode_rows<T, D, 2, ROPE>(dm, q, ch, W, out, out_dtype, st);
+    if (dm.g <= 4) return launch_decode_rows<T, D, 4, ROPE>(dm, q, ch, W, out, out_dtype, st);
+    return launch_decode_rows<T, D, 8, ROPE>(dm, q, ch, W, out, out_dtype, st);
 }
 
 }  // namespace vec
@@ -429,10 +440,14 @@ extern "C" vector_status vector_decode_attn(const vector_shape* shape, const voi
     cudaStream_t st = (cudaStream_t)stream;
     float* partial = (float*)ws;
     if (dm.dtype == VECTOR_F32)
-        return dm.d == 64 ? (dm.rope ? launch_decode_g<64, true>(dm, q, cache, W, out, out_dtype, st)
-                                     : launch_decode_g<64, false>(dm, q, cache, W, out, out_dtype, st))
-                          : (dm.rope ? launch_decode_g<128, true>(dm, q, cache, W, out, out_dtype, st)
-                                     : launch_decode_g<128, false>(dm, q, cache, W, out, out_dtype, st));
+        return dm.d == 64 ? (dm.rope ? launch_decode_g<float, 64, true>(dm, q, cache, W, out, out_dtype, st)
+                                     : launch_decode_g<float, 64, false>(dm, q, cache, W, out, out_dtype, st))
+                          : (dm.rope ? launch_decode_g<float, 128, true>(dm, q, cache, W, out, out_dtype, st)
+                                     : launch_decode_g<float, 128, false>(dm, q, cache, W, out, out_dtype, st));
+    // 64-channel bf16 rows that do not lie at multiples of 16 bytes, which TMA would refuse, run on the CUDA-core kernel
+    if (dm.d == 64 && !rows_at_16_bytes(q, cache, W))
+        return dm.rope ? launch_decode_g<__nv_bfloat16, 64, true>(dm, q, cache, W, out, out_dtype, st)
+                       : launch_decode_g<__nv_bfloat16, 64, false>(dm, q, cache, W, out, out_dtype, st);
     if (dm.d == 64) return launch_decode_bf16<64>(dm, q, cache, W, out, out_dtype, mode, partial, st);
     return launch_decode_bf16<128>(dm, q, cache, W, out, out_dtype, mode, partial, st);
 }

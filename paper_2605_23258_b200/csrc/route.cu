@@ -106,16 +106,16 @@ truncate_kernel(const float* __restrict__ eps, const int32_t* __restrict__ pool_
     truncate_general<NW>(e, n_pool, n_apx, emit, S, L, sel_dyn);
 }
 
-// Step 2 on CUDA cores (fp32).  A warp takes RW listed rows at once, a lane the output channels lane, lane + 32, ...: an
+// Step 2 on CUDA cores (fp32, and 64-channel bf16 rows off a 16-byte boundary).  A warp takes RW listed rows at once, a lane the output channels lane, lane + 32, ...: an
 // element of W^T read from shared memory serves the RW rows, and their loads are under way while W is staged (one row after
 // the other, each from its load to its sum: 30 us for 2 units of 384 rows).  RW = 4 where that leaves a block for
 // every multiprocessor, else 2.  grid (ceil(n_idx / (8 RW)), U), 256 threads; dynamic shared memory: W^T as D * (D+1)
 // floats plus RW key rows per warp.
 // With ROPE the regressor sees the key turned back by its position (the token index): channel c
 // pairs with c + D/2, angle -pos * theta^(-2c/D).
-template <int D, bool ROPE, int RW>
+template <typename T, int D, bool ROPE, int RW>
 __global__ void __launch_bounds__(256)
-residual_generic(const float* __restrict__ K, const float* __restrict__ V, const float* __restrict__ W, int64_t N,
+residual_generic(const T* __restrict__ K, const T* __restrict__ V, const T* __restrict__ W, int64_t N,
                  int LH, const int32_t* __restrict__ idx, int n_idx, float theta, float* __restrict__ eps) {
     constexpr int CPL = D / 32;             // channels per lane
     extern __shared__ __align__(16) float smem[];
@@ -136,15 +136,15 @@ residual_generic(const float* __restrict__ K, const float* __restrict__ V, const
         const bool in = (uint64_t)tok[r] < (uint64_t)N;          // an index outside the unit reads as a row of zeros
 #pragma unroll
         for (int m = 0; m < CPL; ++m) {
-            kr[r][m] = in ? K[((size_t)u * N + tok[r]) * D + lane + 32 * m] : 0.f;
-            vr[r][m] = in ? V[((size_t)u * N + tok[r]) * D + lane + 32 * m] : 0.f;
+            kr[r][m] = in ? to_f32(K[((size_t)u * N + tok[r]) * D + lane + 32 * m]) : 0.f;
+            vr[r][m] = in ? to_f32(V[((size_t)u * N + tok[r]) * D + lane + 32 * m]) : 0.f;
         }
     }
-    const float* Wu = W + (size_t)(u % LH) * D * D;
+    const T* Wu = W + (size_t)(u % LH) * D * D;
 #pragma unroll 16
     for (int e = threadIdx.x; e < D * D; e += 256) {
         const int co = e / D, ci = e % D;
-        Wt[ci * (D + 1) + co] = Wu[e];
+        Wt[ci * (D + 1) + co] = to_f32(Wu[e]);
     }
     float* kw = ks + wid * RW * D;
 #pragma unroll
@@ -198,31 +198,31 @@ residual_generic(const float* __restrict__ K, const float* __restrict__ V, const
     }
 }
 
-template <int D, bool ROPE, int RW>
+template <typename T, int D, bool ROPE, int RW>
 static vector_status launch_residual_rows(const Dims& dm, const void* K, const void* V, const void* W, int64_t N, const int32_t* idx,
                                           int64_t n_idx, float* eps, cudaStream_t st) {
     constexpr int SMEM = (D * (D + 1) + 8 * RW * D) * (int)sizeof(float);
-    auto kern = residual_generic<D, ROPE, RW>;
+    auto kern = residual_generic<T, D, ROPE, RW>;
     static PerDeviceOnce once;
     if (once.first()) {
         const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM);
         if (e != cudaSuccess) { once.undo(); VEC_CUDA_CHECK(e); }
     }
     VEC_CUDA_CHECK(launch_maybe_dependent(true, kern, dim3((unsigned)((n_idx + 8 * RW - 1) / (8 * RW)), dm.U), dim3(256), SMEM, st,
-                                          (const float*)K, (const float*)V, (const float*)W, N, dm.LH, idx, (int)n_idx, dm.theta, eps));
+                                          (const T*)K, (const T*)V, (const T*)W, N, dm.LH, idx, (int)n_idx, dm.theta, eps));
     return VECTOR_OK;
 }
 
-template <int D>
+template <typename T, int D>
 static vector_status launch_residual(const Dims& dm, const void* K, const void* V, const void* W, int64_t N,
                                      const int32_t* idx, int64_t n_idx, float* eps, cudaStream_t st) {
     if (n_idx == 0) return VECTOR_OK;
     const bool many = (n_idx + 31) / 32 * dm.U >= sm_count();
     if (dm.rope)
-        return many ? launch_residual_rows<D, true, 4>(dm, K, V, W, N, idx, n_idx, eps, st)
-                    : launch_residual_rows<D, true, 2>(dm, K, V, W, N, idx, n_idx, eps, st);
-    return many ? launch_residual_rows<D, false, 4>(dm, K, V, W, N, idx, n_idx, eps, st)
-                : launch_residual_rows<D, false, 2>(dm, K, V, W, N, idx, n_idx, eps, st);
+        return many ? launch_residual_rows<T, D, true, 4>(dm, K, V, W, N, idx, n_idx, eps, st)
+                    : launch_residual_rows<T, D, true, 2>(dm, K, V, W, N, idx, n_idx, eps, st);
+    return many ? launch_residual_rows<T, D, false, 4>(dm, K, V, W, N, idx, n_idx, eps, st)
+                : launch_residual_rows<T, D, false, 2>(dm, K, V, W, N, idx, n_idx, eps, st);
 }
 
 // bf16: gather + tcgen05 residual kernel.
@@ -266,11 +266,13 @@ static vector_status launch_residual_tc(const Dims& dm, const void* K, const voi
 static vector_status residual_dispatch(const Dims& dm, const void* K, const void* V, const void* W, int64_t N,
                                        const int32_t* idx, int64_t n_idx, float* eps, cudaStream_t st,
                                        bool dependent = false) {
+    if (dm.dtype == VECTOR_BF16 && dm.d == 64 && (((uintptr_t)K | (uintptr_t)V | (uintptr_t)W) & 15))
+        return launch_residual<__nv_bfloat16, 64>(dm, K, V, W, N, idx, n_idx, eps, st);
     if (dm.dtype == VECTOR_BF16)
         return dm.d == 64 ? launch_residual_tc<64>(dm, K, V, W, N, idx, n_idx, eps, st, dependent)
                           : launch_residual_tc<128>(dm, K, V, W, N, idx, n_idx, eps, st, dependent);
-    return dm.d == 64 ? launch_residual<64>(dm, K, V, W, N, idx, n_idx, eps, st)
-                      : launch_residual<128>(dm, K, V, W, N, idx, n_idx, eps, st);
+    return dm.d == 64 ? launch_residual<float, 64>(dm, K, V, W, N, idx, n_idx, eps, st)
+                      : launch_residual<float, 128>(dm, K, V, W, N, idx, n_idx, eps, st);
 }
 
 // One-time opt-in to the dynamic shared memory of the selection kernels.

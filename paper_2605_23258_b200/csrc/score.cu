@@ -14,18 +14,24 @@
 
 namespace vec {
 
-constexpr int ST = 64;    // tile edge (rows and keys) of the CUDA-core score kernels (fp32)
+constexpr int ST = 64;    // tile edge (rows and keys) of the CUDA-core score kernels
 
 // The CUDA-core passes hold a whole 64 x D tile of each operand in shared memory (rows D + 1 apart) and request the next
 // tile of the one that changes before they work on this one: with 32-channel slices loaded between barriers a pass was a
 // chain of load latencies (13 + 11 us for 2 units of 64 rows and 1024 keys).
 template <int D> struct TileRegs { float4 v[ST * D / 1024]; };
-template <int D>
-__device__ __forceinline__ void tile_request(const float* __restrict__ src, int64_t row0, int64_t n_rows, TileRegs<D>& t) {
+// wide: the rows lie at multiples of 16 bytes (fp32); otherwise, and for bf16, element by element.
+template <typename T, int D>
+__device__ __forceinline__ void tile_request(const T* __restrict__ src, int64_t row0, int64_t n_rows, bool wide, TileRegs<D>& t) {
 #pragma unroll
     for (int e = 0; e < ST * D / 1024; ++e) {
         const int idx = threadIdx.x + 256 * e, r = idx / (D / 4), c4 = idx % (D / 4);
-        t.v[e] = row0 + r < n_rows ? reinterpret_cast<const float4*>(src + (row0 + r) * D)[c4] : make_float4(0.f, 0.f, 0.f, 0.f);
+        t.v[e] = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (row0 + r < n_rows) {
+            const T* p = src + (row0 + r) * D + 4 * c4;
+            if (sizeof(T) == 4 && wide) t.v[e] = *reinterpret_cast<const float4*>(p);
+            else t.v[e] = make_float4(to_f32(p[0]), to_f32(p[1]), to_f32(p[2]), to_f32(p[3]));
+        }
     }
 }
 template <int D>
@@ -61,25 +67,25 @@ __device__ __forceinline__ void tile_qk(const float* Qs, const float* Ks, float 
 template <int D> constexpr int tile_smem() { return 2 * ST * (D + 1) * (int)sizeof(float); }
 
 // grid (n_chunks, row_tiles, U), 256 threads, tile_smem of dynamic shared memory
-template <int D>
+template <typename T, int D>
 __global__ void __launch_bounds__(256)
-score_pass1_generic(const float* __restrict__ Q, const float* __restrict__ K, int64_t N, int R, int w,
-                    float scale, int64_t chunk_len, float2* __restrict__ partial) {
+score_pass1_generic(const T* __restrict__ Q, const T* __restrict__ K, int64_t N, int R, int w,
+                    float scale, int64_t chunk_len, bool wide, float2* __restrict__ partial) {
     extern __shared__ float tiles[];
     float *Qs = tiles, *Ks = tiles + ST * (D + 1);
     asm volatile("griddepcontrol.wait;\n" ::: "memory");        // launched as a programmatic dependent: nothing is touched before
     asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory");
     const int u = blockIdx.z, row0 = blockIdx.y * ST, chunk = blockIdx.x, n_chunks = gridDim.x;
     const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
-    const float* Qu = Q + (size_t)u * R * D;
-    const float* Ku = K + (size_t)u * N * D;
+    const T* Qu = Q + (size_t)u * R * D;
+    const T* Ku = K + (size_t)u * N * D;
     const int64_t k_begin = (int64_t)chunk * chunk_len;
     const int64_t k_end = min(N, k_begin + chunk_len);
     TileRegs<D> next;
-    tile_request<D>(Ku, k_begin, k_end, next);
+    tile_request(Ku, k_begin, k_end, wide, next);
     {
         TileRegs<D> q;
-        tile_request<D>(Qu, row0, R, q);
+        tile_request(Qu, row0, R, wide, q);
         tile_store<D>(q, Qs);
     }
     float m[4], l[4];
@@ -95,7 +101,7 @@ score_pass1_generic(const float* __restrict__ Q, const float* __restrict__ K, in
         __syncthreads();                                  // the tile before this one has been read
         tile_store<D>(next, Ks);
         __syncthreads();
-        if (key0 + ST < k_end) tile_request<D>(Ku, key0 + ST, k_end, next);
+        if (key0 + ST < k_end) tile_request(Ku, key0 + ST, k_end, wide, next);
         float acc[4][4];
         tile_qk<D>(Qs, Ks, acc);
 #pragma unroll
@@ -169,10 +175,11 @@ score_lse_rows(const float2* __restrict__ partial, int R, int n_chunks, float* _
 
 // grid (key_tiles, U), 256 threads, tile_smem of dynamic shared memory.  INLINE_LSE: a block forms the normalisers of its
 // rows itself from the chunk partials (a launch less; every key tile repeats it).
-template <int D, bool INLINE_LSE>
+template <typename T, int D, bool INLINE_LSE>
 __global__ void __launch_bounds__(256)
-score_pass2_generic(const float* __restrict__ Q, const float* __restrict__ K, int64_t N, int R, int w,
-                    float scale, const float2* __restrict__ partial, int n_chunks, const float* __restrict__ lse, float* __restrict__ raw) {
+score_pass2_generic(const T* __restrict__ Q, const T* __restrict__ K, int64_t N, int R, int w,
+                    float scale, const float2* __restrict__ partial, int n_chunks, const float* __restrict__ lse, bool wide,
+                    float* __restrict__ raw) {
     extern __shared__ float tiles[];
     float *Qs = tiles, *Ks = tiles + ST * (D + 1);
     __shared__ float red[16][ST];
@@ -182,12 +189,12 @@ score_pass2_generic(const float* __restrict__ Q, const float* __restrict__ K, in
     const int u = blockIdx.y;
     const int64_t key0 = (int64_t)blockIdx.x * ST;
     const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
-    const float* Qu = Q + (size_t)u * R * D;
+    const T* Qu = Q + (size_t)u * R * D;
     TileRegs<D> next;
     {
         TileRegs<D> k;
-        tile_request<D>(K + (size_t)u * N * D, key0, N, k);
-        tile_request<D>(Qu, 0, R, next);
+        tile_request(K + (size_t)u * N * D, key0, N, wide, k);
+        tile_request(Qu, 0, R, wide, next);
         tile_store<D>(k, Ks);
     }
     float col[4] = {0.f, 0.f, 0.f, 0.f};
@@ -202,7 +209,7 @@ score_pass2_generic(const float* __restrict__ Q, const float* __restrict__ K, in
             lse_s[tid] = lse[(size_t)u * R + row0 + tid];
         }
         __syncthreads();
-        if (row0 + ST < R) tile_request<D>(Qu, row0 + ST, R, next);
+        if (row0 + ST < R) tile_request(Qu, row0 + ST, R, wide, next);
         float acc[4][4];
         tile_qk<D>(Qs, Ks, acc);
 #pragma unroll
@@ -249,32 +256,41 @@ __global__ void score_pool_kernel(const float* __restrict__ raw, int64_t N, int 
     score[gi] = best;
 }
 
-template <int D>
-static vector_status launch_score(const Dims& dm, const float* Q, const float* K, int64_t N, float* scores,
-                                  float* raw, float2* partial, float* lse, cudaStream_t st) {
+// Workspace: chunk partials | lse | raw, where the caller does not take it; fewer chunks where it would not hold theirs.
+template <typename T, int D>
+static vector_status launch_score(const Dims& dm, const void* Q_, const void* K_, int64_t N, float* scores, float* raw_out, char* ws,
+                                  size_t ws_bytes, cudaStream_t st) {
     constexpr int SMEM = tile_smem<D>();
+    const T *Q = (const T*)Q_, *K = (const T*)K_;
+    const bool wide = (((uintptr_t)Q_ | (uintptr_t)K_) & 15) == 0;
     static PerDeviceOnce once;
     if (once.first()) {
-        cudaError_t e = cudaFuncSetAttribute(score_pass1_generic<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM);
-        if (e == cudaSuccess) e = cudaFuncSetAttribute(score_pass2_generic<D, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM);
-        if (e == cudaSuccess) e = cudaFuncSetAttribute(score_pass2_generic<D, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM);
+        cudaError_t e = cudaFuncSetAttribute(score_pass1_generic<T, D>, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM);
+        if (e == cudaSuccess) e = cudaFuncSetAttribute(score_pass2_generic<T, D, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM);
+        if (e == cudaSuccess) e = cudaFuncSetAttribute(score_pass2_generic<T, D, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM);
         if (e != cudaSuccess) { once.undo(); VEC_CUDA_CHECK(e); }
     }
+    const size_t lse_b = align256((size_t)dm.U * dm.R * sizeof(float)), raw_b = raw_out ? 0 : align256((size_t)dm.U * (size_t)N * sizeof(float));
     int n_chunks = score_num_chunks(dm.U, dm.R, N);
+    auto partial_b = [&] { return align256((size_t)dm.U * n_chunks * dm.R * sizeof(float2)); };
+    while (n_chunks > 1 && partial_b() + lse_b + raw_b > ws_bytes) --n_chunks;
+    float2* partial = (float2*)ws;
+    float* lse = (float*)(ws + partial_b());
+    float* raw = raw_out ? raw_out : (float*)(ws + partial_b() + lse_b);
     int64_t chunk_len = (N + n_chunks - 1) / n_chunks;
     chunk_len = (chunk_len + ST - 1) / ST * ST;
     n_chunks = (int)((N + chunk_len - 1) / chunk_len);            // none empty
     const int row_tiles = (dm.R + ST - 1) / ST;
-    VEC_CUDA_CHECK(launch_maybe_dependent(true, score_pass1_generic<D>, dim3(n_chunks, row_tiles, dm.U), dim3(256), SMEM, st, Q, K, N,
-                                          dm.R, dm.w, dm.scale, chunk_len, partial));
+    VEC_CUDA_CHECK(launch_maybe_dependent(true, score_pass1_generic<T, D>, dim3(n_chunks, row_tiles, dm.U), dim3(256), SMEM, st, Q, K, N,
+                                          dm.R, dm.w, dm.scale, chunk_len, wide, partial));
     // the partials of a row tile: no more than the rows' own elements
     const bool inline_lse = n_chunks <= 32;
     if (!inline_lse)
         VEC_CUDA_CHECK(launch_maybe_dependent(true, score_lse_rows, dim3((dm.R + 63) / 64, dm.U), dim3(256), 0, st, partial, dm.R,
                                               n_chunks, lse));
-    VEC_CUDA_CHECK(launch_maybe_dependent(true, inline_lse ? score_pass2_generic<D, true> : score_pass2_generic<D, false>,
+    VEC_CUDA_CHECK(launch_maybe_dependent(true, inline_lse ? score_pass2_generic<T, D, true> : score_pass2_generic<T, D, false>,
                                           dim3((unsigned)((N + ST - 1) / ST), dm.U), dim3(256), SMEM, st, Q, K, N, dm.R, dm.w, dm.scale,
-                                          partial, n_chunks, lse, raw));
+                                          partial, n_chunks, lse, wide, raw));
     int64_t total = (int64_t)dm.U * N;
     VEC_CUDA_CHECK(launch_maybe_dependent(true, score_pool_kernel, dim3((unsigned)((total + 255) / 256)), dim3(256), 0, st, raw, N, dm.w,
                                           dm.pool_kernel / 2, total, scores));
@@ -347,16 +363,13 @@ extern "C" vector_status vector_score(const vector_shape* shape, const void* Q_o
     const bool need_raw = raw_out == nullptr;
     if (!ws || ((uintptr_t)ws & 255) || ws_bytes < score_ws_bytes(dm, N, need_raw)) return VECTOR_ERR_WORKSPACE;
     char* p = (char*)ws;
-    if (score_uses_tc(dm))
-        return dm.d == 64 ? launch_score_tc<64>(dm, Q_obs, K, N, scores, raw_out, p, (cudaStream_t)stream)
-                          : launch_score_tc<128>(dm, Q_obs, K, N, scores, raw_out, p, (cudaStream_t)stream);
-    float2* partial = (float2*)p;
-    p += align256((size_t)dm.U * score_num_chunks(dm.U, dm.R, N) * dm.R * 2 * sizeof(float));
-    float* lse = (float*)p;
-    p += align256((size_t)dm.U * dm.R * sizeof(float));
-    float* raw = need_raw ? (float*)p : raw_out;
     cudaStream_t st = (cudaStream_t)stream;
-    const float *q = (const float*)Q_obs, *k = (const float*)K;
-    return dm.d == 64 ? launch_score<64>(dm, q, k, N, scores, raw, partial, lse, st)
-                      : launch_score<128>(dm, q, k, N, scores, raw, partial, lse, st);
+    // 64-channel bf16 rows that do not lie at multiples of 16 bytes, which TMA would refuse, run on the CUDA-core kernels
+    const bool loose = dm.d == 64 && (((uintptr_t)Q_obs | (uintptr_t)K | (uintptr_t)scores | (uintptr_t)raw_out) & 15);
+    if (score_uses_tc(dm) && !loose)
+        return dm.d == 64 ? launch_score_tc<64>(dm, Q_obs, K, N, scores, raw_out, p, st)
+                          : launch_score_tc<128>(dm, Q_obs, K, N, scores, raw_out, p, st);
+    if (dm.dtype == VECTOR_BF16) return launch_score<__nv_bfloat16, 64>(dm, Q_obs, K, N, scores, raw_out, p, ws_bytes, st);
+    return dm.d == 64 ? launch_score<float, 64>(dm, Q_obs, K, N, scores, raw_out, p, ws_bytes, st)
+                      : launch_score<float, 128>(dm, Q_obs, K, N, scores, raw_out, p, ws_bytes, st);
 }
