@@ -70,7 +70,9 @@ __device__ __forceinline__ void rope_fill_inv_freq(double* inv_freq, int d, floa
 // Kernel launch that may carry the programmatic-dependent attribute: with `dependent` the kernel may
 // be scheduled while the kernel before it in the stream drains (once every block of that one has
 // executed griddepcontrol.launch_dependents, or exited); it must execute griddepcontrol.wait before
-// it touches anything that kernel, or one before it, reads or writes.  cluster > 1: thread block clusters of that size.
+// it touches anything that kernel reads or writes.  Every kernel here lets its dependents start only behind its own wait, so what
+// came before its primary has finished when a dependent starts, along whole chains and across calls: ahead of its wait a
+// kernel may touch what its primary does not.  cluster > 1: thread block clusters of that size.
 template <typename... KArgs, typename... Args>
 inline cudaError_t launch_maybe_dependent(bool dependent, int cluster, void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem,
                                           cudaStream_t st, Args... args) {

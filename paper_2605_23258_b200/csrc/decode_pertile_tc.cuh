@@ -84,6 +84,7 @@ decode_stream_pertile_tc(const __nv_bfloat16* __restrict__ q, const __grid_const
     const int u_last = n_my > 0 ? (int)((gt_hi - 1) / pl.n_tiles) : -1;
 
     // the merge kernel is a programmatic dependent: it reads the records after its own wait
+    asm volatile("griddepcontrol.wait;\n" ::: "memory");         // launched the ordinary way: returns at once
     asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory");
     if (tid == 0) {
 #pragma unroll

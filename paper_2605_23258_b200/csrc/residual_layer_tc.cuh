@@ -103,7 +103,6 @@ residual_layer_tc(const __nv_bfloat16* __restrict__ K, const __nv_bfloat16* __re
     const int n_my = (int)(rtc::range_begin(blockIdx.x + 1, P.n_items, gridDim.x) - it_lo);
     const int H = P.Hkv;
 
-    asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory");
     if (tid == 0) {
 #pragma unroll
         for (int s = 0; s < STAGES; ++s) {
@@ -131,6 +130,7 @@ residual_layer_tc(const __nv_bfloat16* __restrict__ K, const __nv_bfloat16* __re
         bool ok = true;
         if (tid == 0) tma::prefetch_map(&mapW);
         asm volatile("griddepcontrol.wait;\n" ::: "memory");      // idx is complete and visible from here on
+        asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory");
         Cursor at = cursor_at(it_lo, P);
         uint32_t step = 0;
         for (int i = 0; i < n_my && ok; ++i, at.next(P)) {

@@ -114,10 +114,9 @@ residual_tc(const __nv_bfloat16* __restrict__ K, const __nv_bfloat16* __restrict
     const long long gt_hi = range_begin(blockIdx.x + 1, P.n_tiles, gridDim.x);
     const int n_my = (int)(gt_hi - gt_lo);
 
-    // Programmatic launches on both sides (inside vector_route): the kernel after this one may be
-    // scheduled as blocks here finish, and this one may have started before the kernel that writes
-    // idx has drained -- the loaders, the only readers of idx, wait for it below.
-    asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory");
+    // A programmatic dependent of the kernel that writes idx (inside vector_route), whose other blocks may still run: the loaders,
+    // the only readers of idx, wait for it below.  W is loaded ahead of that: the selection does not touch it, and what came
+    // before the selection has finished, since it waits before it lets this kernel start.
     if (tid < 64) phase_s[tid] = rope.phase[tid];
     if (tid == 0) {
 #pragma unroll
@@ -241,6 +240,7 @@ residual_tc(const __nv_bfloat16* __restrict__ K, const __nv_bfloat16* __restrict
         };
         bool ok = true;
         asm volatile("griddepcontrol.wait;\n" ::: "memory");      // idx is complete and visible from here on
+        asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory");
         if (n_my > 0) fetch_idx(cur);
         if constexpr (ROPE) {
             if (n_my > 0) {
@@ -334,7 +334,7 @@ residual_tc(const __nv_bfloat16* __restrict__ K, const __nv_bfloat16* __restrict
                     ++n_units;
                 }
                 // the loaders start only once the kernel that writes idx has drained: do not spend this
-                // thread's bounded polls on that kernel's run time (W, loaded above, is nobody's output)
+                // thread's bounded polls on that kernel's run time (W, loaded above, is not its output)
                 if (i == 0) asm volatile("griddepcontrol.wait;\n" ::: "memory");
                 if (!tma::mbar_wait(&sy.full[s], round & 1, fault, 49)) break;
                 tc::fence_after_sync();

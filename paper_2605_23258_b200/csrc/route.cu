@@ -96,8 +96,8 @@ truncate_kernel(const float* __restrict__ eps, const int32_t* __restrict__ pool_
     } else {
         for (int64_t i = threadIdx.x; i < N; i += 32 * NW) tr[i] = 0;
     }
-    // everything above touches only the tier map; the residuals and the pool list belong to the
-    // kernels before this one (a no-op unless launched as a programmatic dependent)
+    // Everything above touches only the tier map, which the residual kernel, this one's primary, neither reads nor writes, and
+    // nothing before that kernel is still under way: it waits before it lets this one start.  (No wait unless a dependent.)
     asm volatile("griddepcontrol.wait;\n" ::: "memory");
     __syncthreads();
     const int n_ret = n_pool - n_apx;

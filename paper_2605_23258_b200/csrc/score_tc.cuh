@@ -121,7 +121,8 @@ __device__ __forceinline__ void producer_role(const CUtensorMap* mapQ, const CUt
         }
     }
     // The next kernel's blocks may be scheduled from here on, when the last copies are under way: earlier they would
-    // sit beside this block for its whole run.
+    // sit beside this block for its whole run.  (A block with few tiles has not waited yet.)
+    asm volatile("griddepcontrol.wait;\n" ::: "memory");
     asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory");
 }
 
