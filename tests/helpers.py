@@ -63,3 +63,60 @@ def eps_close(got, want, K_rows, V_rows, W):
     tol = 2 * np.sqrt(want) * dn + dn ** 2 + 2.0 ** -21 * want
     err = np.abs(np.asarray(got, np.float64) - want)
     return bool(np.all(err <= tol)), float(np.max(err / tol))
+
+
+def decode_problem(U, g, d, dtype, n_ret, n_apx, seed, sharp=1.0, device="cuda"):
+    """Random pools with two rows to spare, a map per unit and queries.  In both pools the first and last row and the rows on
+    either side of every 64th get a key towards the unit's first query, so that each of them carries a visible share of the output:
+    losing one shows as a thousandth of it or more."""
+    gen = torch.Generator(device=device).manual_seed(seed)
+    q = (torch.randn(U, g, d, generator=gen, device=device) * sharp).to(dtype)
+    unit = q[:, :1].float() / q[:, :1].float().norm(dim=-1, keepdim=True)
+
+    def keys(n):
+        k = torch.randn(U, n + 2, d, generator=gen, device=device)
+        rows = sorted({r for r in (0, n - 1, *range(63, n, 64), *range(64, n, 64)) if 0 <= r < n})
+        if rows:
+            k[:, rows] += 4.0 / sharp * unit
+        return k.to(dtype)
+    rk, ak = keys(n_ret), keys(n_apx)
+    rv = torch.randn(U, n_ret + 2, d, generator=gen, device=device).to(dtype)
+    W = (torch.randn(U, d, d, generator=gen, device=device) / np.sqrt(d)).to(dtype)
+    pos = torch.randint(0, 131072, (U, n_apx + 2), generator=gen, device=device, dtype=torch.int32)
+    ret_pos = torch.zeros(U, n_ret + 2, dtype=torch.int32, device=device)
+    return q, vec.Cache(rk, rv, ak, ret_pos, pos, n_ret, n_apx), W
+
+
+def decode_shape(q, rope):
+    U, g, d = q.shape
+    return vec.Shape(1, 1, U * g, U, d, vec.VECTOR_BF16 if q.dtype == torch.bfloat16 else vec.VECTOR_F32, 16, 7, 0.0, int(rope), 10000.0)
+
+
+def decode_call(q, cache, W, rope, out_dtype=torch.float32, mode=0, times=1):
+    sh = decode_shape(q, rope)
+    out = torch.full(q.shape, float("nan"), dtype=out_dtype, device=q.device)
+    ws = vec.alloc_workspace(sh, vec.vector_plan_budget(16384, 8192, -1, 16))
+    for _ in range(times):
+        vec.vector_decode_attn(sh, q, cache, W, out, mode, ws)
+    torch.cuda.synchronize()
+    assert vec.vector_device_fault() == 0
+    return out
+
+
+def decode_errors(oracle, q, cache, W, out, rope, units):
+    """Per head of the listed units: the 2-norm of what the output is off by, over the output's."""
+    errs = []
+    for u in units:
+        _, o = oracle.attend(q[u].cpu(), cache.ret_k[u, :cache.n_ret].cpu(), cache.ret_v[u, :cache.n_ret].cpu(), cache.apx_k[u, :cache.n_apx].cpu(),
+                             W[u].cpu(), 1.0 / np.sqrt(q.shape[-1]), apx_pos=cache.apx_pos[u, :cache.n_apx].cpu().numpy(), rope=rope, theta=10000.0)
+        errs.append(np.linalg.norm(out[u].cpu().double().numpy() - o, axis=1) / np.linalg.norm(o, axis=1))
+    return np.concatenate(errs)
+
+
+def decode_bound(dtype, d, rope):
+    """What an fp32 output may be off by, per head.  fp32 keys, and 64-channel bf16 heads: a few roundings of exponentials (2^-22) and
+    logits (|s| 2^-24, |s| up to 20), 3e-6.  128-channel bf16 heads: weights and key sums in two bf16 parts, 2^-17 each of a head that
+    one row may carry, 1.5e-5; keys turned back as fp16, 2^-12 each, whose sum may cancel to a third, 8e-4."""
+    if dtype == torch.float32 or d == 64:
+        return 3e-6
+    return 8e-4 if rope else 1.5e-5

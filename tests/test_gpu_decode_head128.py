@@ -10,36 +10,23 @@ import torch
 
 import paper_2605_23258_b200 as vec
 
+from helpers import decode_call, decode_errors, decode_problem
+
 pytestmark = pytest.mark.gpu
 DEV = "cuda"
 
 
 def _decode(rk, rv, ak, W, q):
-    U, g, d = q.shape
-    n_ret, n_apx = rk.shape[1], ak.shape[1]
+    U, n_ret, n_apx = q.shape[0], rk.shape[1], ak.shape[1]
     pos = [torch.zeros(U, n, dtype=torch.int32, device=DEV) for n in (n_ret, n_apx)]
-    sh = vec.Shape(1, 1, U * g, U, d, vec.VECTOR_BF16, 16)
-    out = torch.full((U, g, d), float("nan"), device=DEV)
-    vec.vector_decode_attn(sh, q, vec.Cache(rk, rv, ak, *pos, n_ret, n_apx), W, out, 0, vec.alloc_workspace(sh, vec.vector_plan_budget(16384, 8192, -1, 16)))
-    torch.cuda.synchronize()
-    assert vec.vector_device_fault() == 0
-    return out
+    return decode_call(q, vec.Cache(rk, rv, ak, *pos, n_ret, n_apx), W, False)
 
 
 @pytest.mark.parametrize("g,units,n_ret,n_apx,sharp", [(4, 4, 300, 500, 1.0), (4, 150, 300, 500, 1.0), (8, 100, 64, 700, 2.0), (1, 8, 5000, 9000, 0.2)])
 def test_decode_head128_precision(oracle, g, units, n_ret, n_apx, sharp):
-    d = 128
-    gen = torch.Generator(device=DEV).manual_seed(31)
-    rk, rv = (torch.randn(units, n_ret, d, generator=gen, device=DEV).to(torch.bfloat16) for _ in range(2))
-    ak = torch.randn(units, n_apx, d, generator=gen, device=DEV).to(torch.bfloat16)
-    W = (torch.randn(units, d, d, generator=gen, device=DEV) / np.sqrt(d)).to(torch.bfloat16)
-    q = (torch.randn(units, g, d, generator=gen, device=DEV) * sharp).to(torch.bfloat16)
-    out = _decode(rk, rv, ak, W, q)
-    errs = []
-    for u in range(0, units, max(1, units // 16)):
-        _, o = oracle.attend(q[u].cpu(), rk[u].cpu(), rv[u].cpu(), ak[u].cpu(), W[u].cpu(), 1.0 / np.sqrt(d))
-        errs.append(np.linalg.norm(out[u].cpu().double().numpy() - o, axis=1) / np.linalg.norm(o, axis=1))
-    rms = float(np.sqrt(np.mean(np.concatenate(errs) ** 2)))
+    q, cache, W = decode_problem(units, g, 128, torch.bfloat16, n_ret, n_apx, 31, sharp)
+    errs = decode_errors(oracle, q, cache, W, decode_call(q, cache, W, False), False, range(0, units, max(1, units // 16)))
+    rms = float(np.sqrt(np.mean(errs ** 2)))
     assert rms <= 5e-6, rms
 
 

@@ -1,6 +1,6 @@
 """The fp32 kernels at the sizes where their launches change: normalisers formed inline or by a kernel of their own, ragged
-tiles, clusters of one to sixteen blocks, two or four residual rows a warp.  Tolerances as in the bf16 tests: scores
-1e-3 relative (score_close), residuals within the rounding bound (eps_close), attention 2e-2 absolute."""
+tiles, clusters of one to sixteen blocks, two or four residual rows a warp.  Scores 1e-3 relative (score_close), residuals within
+the rounding bound (eps_close), attention to helpers.decode_bound, 2^-8 more for a bf16 output."""
 import numpy as np
 import pytest
 import torch
@@ -8,7 +8,7 @@ import torch
 import paper_2605_23258_b200 as vec
 from paper_2605_23258_b200 import synth
 
-from helpers import eps_close, oracle_scores, score_close, shape_of
+from helpers import decode_bound, decode_call, decode_errors, decode_problem, eps_close, oracle_scores, score_close, shape_of
 
 pytestmark = pytest.mark.gpu
 DEV = "cuda"
@@ -48,21 +48,9 @@ def test_residual_fp32(oracle, rope, d, U, n_idx):
 @pytest.mark.parametrize("rope", [False, True])
 @pytest.mark.parametrize("d,U,g,n_ret,n_apx", [(64, 1, 1, 1, 0), (64, 2, 8, 0, 31), (128, 3, 2, 33, 32), (128, 1, 5, 700, 900), (64, 300, 4, 40, 70)])
 def test_decode_fp32(oracle, rope, d, U, g, n_ret, n_apx):
-    gen = torch.Generator(device=DEV).manual_seed(U + g)
-    rk, rv = (torch.randn(U, n_ret + 1, d, generator=gen, device=DEV) for _ in range(2))
-    ak = torch.randn(U, n_apx + 1, d, generator=gen, device=DEV)
-    W = torch.randn(U, d, d, generator=gen, device=DEV) / np.sqrt(d)
-    q = torch.randn(U, g, d, generator=gen, device=DEV) * 2
-    pos = torch.randint(0, 131072, (U, n_apx + 1), generator=gen, device=DEV, dtype=torch.int32)
-    cache = vec.Cache(rk, rv, ak, torch.zeros(U, n_ret + 1, dtype=torch.int32, device=DEV), pos, n_ret, n_apx)
-    sh = vec.Shape(1, 1, U * g, U, d, vec.VECTOR_F32, 16, 7, 0.0, int(rope), 10000.0)
-    ws = vec.alloc_workspace(sh, vec.vector_plan_budget(4096, 2048, -1, 16))
-    outs = [torch.full((U, g, d), float("nan"), dtype=dt, device=DEV) for dt in (torch.float32, torch.bfloat16)]
-    for out in outs:
-        vec.vector_decode_attn(sh, q, cache, W, out, 0, ws)
-    torch.cuda.synchronize()
-    for u in range(0, U, max(1, U // 4)):
-        _, o = oracle.attend(q[u].cpu(), rk[u, :n_ret].cpu(), rv[u, :n_ret].cpu(), ak[u, :n_apx].cpu(), W[u].cpu(),
-                             1.0 / np.sqrt(d), apx_pos=pos[u, :n_apx].cpu().numpy(), rope=rope, theta=10000.0)
-        assert np.max(np.abs(outs[0][u].cpu().double().numpy() - o)) <= 2e-2, u
-        assert np.all(np.abs(outs[1][u].cpu().double().numpy() - o) <= 2e-2 + 2.0 ** -8 * np.abs(o)), u
+    q, cache, W = decode_problem(U, g, d, torch.float32, n_ret, n_apx, U + g, sharp=2.0)
+    units = range(0, U, max(1, U // 4))
+    bound = decode_bound(torch.float32, d, rope)
+    for out_dtype, more in ((torch.float32, 0.0), (torch.bfloat16, 2.0 ** -8)):
+        errs = decode_errors(oracle, q, cache, W, decode_call(q, cache, W, rope, out_dtype), rope, units)
+        assert errs.max() <= bound + more, errs.max()

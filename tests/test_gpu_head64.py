@@ -9,7 +9,7 @@ import torch
 import paper_2605_23258_b200 as vec
 from paper_2605_23258_b200 import synth
 
-from helpers import budget_of, calibrated_maps, eps_close, oracle_scores, score_close, shape_of
+from helpers import budget_of, calibrated_maps, decode_call, decode_errors, decode_problem, eps_close, oracle_scores, score_close, shape_of
 
 pytestmark = pytest.mark.gpu
 DEV = "cuda"
@@ -103,25 +103,8 @@ def test_decode_head64_keeps_fp32_precision(oracle, rope, g, units, n_ret, n_apx
     """fp32 output to fp32's own precision, as CUDA cores give it: weights and sums that keep only sixteen bits are off by
     1e-6 and more.  What remains is the exponentials' 2^-22 and the logits' rounding, |s| 2^-24 a few times over with |s| up to
     20: at most about 1e-6 in a head, and less than half of that in the mean square over the heads."""
-    d = 64
-    gen = torch.Generator(device=DEV).manual_seed(17)
-    rk, rv = (torch.randn(units, n_ret + 1, d, generator=gen, device=DEV).to(torch.bfloat16) for _ in range(2))
-    ak = torch.randn(units, n_apx + 1, d, generator=gen, device=DEV).to(torch.bfloat16)
-    W = (torch.randn(units, d, d, generator=gen, device=DEV) / 8).to(torch.bfloat16)
-    q = (torch.randn(units, g, d, generator=gen, device=DEV) * sharp).to(torch.bfloat16)
-    pos = torch.randint(0, 131072, (units, n_apx + 1), generator=gen, device=DEV, dtype=torch.int32)
-    cache = vec.Cache(rk, rv, ak, torch.zeros(units, n_ret + 1, dtype=torch.int32, device=DEV), pos, n_ret, n_apx)
-    sh = vec.Shape(1, 1, units * g, units, d, vec.VECTOR_BF16, 16, 7, 0.0, int(rope), 10000.0)
-    out = torch.full((units, g, d), float("nan"), device=DEV)
-    vec.vector_decode_attn(sh, q, cache, W, out, 0, vec.alloc_workspace(sh, vec.vector_plan_budget(16384, 8192, -1, 16)))
-    torch.cuda.synchronize()
-    assert vec.vector_device_fault() == 0
-    errs = []
-    for u in range(0, units, max(1, units // 16)):
-        _, o = oracle.attend(q[u].cpu(), rk[u, :n_ret].cpu(), rv[u, :n_ret].cpu(), ak[u, :n_apx].cpu(), W[u].cpu(),
-                             1.0 / np.sqrt(d), apx_pos=pos[u, :n_apx].cpu().numpy(), rope=rope, theta=10000.0)
-        errs.append(np.linalg.norm(out[u].cpu().double().numpy() - o, axis=1) / np.linalg.norm(o, axis=1))
-    errs = np.concatenate(errs)
+    q, cache, W = decode_problem(units, g, 64, torch.bfloat16, n_ret, n_apx, 17, sharp)
+    errs = decode_errors(oracle, q, cache, W, decode_call(q, cache, W, rope), rope, range(0, units, max(1, units // 16)))
     assert errs.max() <= 1.5e-6 and np.sqrt(np.mean(errs ** 2)) <= 5e-7, (errs.max(), np.sqrt(np.mean(errs ** 2)))
 
 
