@@ -59,3 +59,11 @@ def test_append_rows_off_a_16_byte_boundary(dtype):
             vec.vector_append(sh, c, a, b, 5)
         assert e.value.status == -2
     assert c.n_ret == n + 2 and (c.ret_pos[:, n:n + 2] == 5).all()
+
+
+def test_calls_go_to_the_current_stream():
+    from paper_2605_23258_b200 import binding
+    side = torch.cuda.Stream()
+    for stream in (torch.cuda.current_stream(), side):
+        with torch.cuda.stream(stream):
+            assert binding._stream(None) == torch.cuda.current_stream().cuda_stream == stream.cuda_stream

@@ -138,3 +138,23 @@ def test_append_to_rows_in_host_memory():
     comp.append(k, v, 7)
     assert c.n_ret == n + 1
     assert torch.equal(c.ret_k[:, n], k) and torch.equal(c.ret_v[:, n], v) and (c.ret_pos[:, n] == 7).all()
+
+
+def test_packed_structs_are_the_c_structs():
+    """The calls pass structs as packed bytes; the ctypes structures beside them spell the fields of the C header out."""
+    sh = vec.Shape(2, 3, 32, 8, 128, vec.VECTOR_BF16, 64, 7, 0.125, 1, 500000.0)
+    assert sh._p() == bytes(sh._c()) and len(sh._p()) == ctypes.sizeof(binding._Shape) == 44
+    b = vec.vector_plan_budget(20011, 4002, -1, 64)
+    assert b._p() == bytes(b._c()) and len(b._p()) == ctypes.sizeof(binding._Budget) == 56
+    t, i = torch.zeros(2, 5, 64), torch.zeros(2, 5, dtype=torch.int32)
+    c = vec.Cache(t, t.clone(), t.clone(), i, i.clone(), 3, 4)
+    want = binding._Cache(c.ret_k.data_ptr(), c.ret_v.data_ptr(), c.apx_k.data_ptr(), c.ret_pos.data_ptr(), c.apx_pos.data_ptr(), 5, 5, 3, 4)
+    assert c._p() == bytes(want) and len(c._p()) == ctypes.sizeof(binding._Cache) == 72
+
+
+def test_struct_fields_follow_the_header():
+    text = re.sub(r"/\*.*?\*/", "", open(os.path.join(ROOT, "include", "vector.h")).read(), flags=re.S)
+    for name, struct in (("vector_shape", binding._Shape), ("vector_budget", binding._Budget), ("vector_cache", binding._Cache)):
+        body = re.search(r"typedef struct \{([^}]*)\} " + name, text).group(1)
+        fields = [f.strip(" *") for line in body.split(";") if line.strip() for f in re.sub(r"^\s*\w+\s*\**", "", line.strip()).split(",")]
+        assert fields == [f for f, _ in struct._fields_]
