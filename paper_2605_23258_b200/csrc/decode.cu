@@ -20,10 +20,10 @@
 
 namespace vec {
 
-// EPL consecutive elements of a row; wide: the rows lie at multiples of 16 bytes (fp32), otherwise, and for bf16, one by one.
-template <int EPL, typename T>
-__device__ __forceinline__ void row_load(const T* __restrict__ p, int lane, bool wide, float (&o)[EPL]) {
-    if (sizeof(T) == 4 && wide) {
+// EPL consecutive elements of a row; WIDE: fp32 rows at multiples of 16 bytes, otherwise one by one.
+template <bool WIDE, int EPL, typename T>
+__device__ __forceinline__ void row_load(const T* __restrict__ p, int lane, float (&o)[EPL]) {
+    if constexpr (WIDE) {
         if constexpr (EPL == 4) {
             const float4 v = reinterpret_cast<const float4*>(p)[lane];
             o[0] = v.x; o[1] = v.y; o[2] = v.z; o[3] = v.w;
@@ -48,11 +48,11 @@ constexpr int F32_WARPS = 8, F32_ROWS = 4, F32_MAX_CLUSTER = 16;
 // (apx_pos): the logit still uses the stored key, only the p-weighted key sum takes the turned one.
 // A lane holds EPL consecutive channels; the partner channel c +- D/2 sits in lane ^ 16.
 // grid (U x cluster size), 256 threads, F32_WARPS * g records of dynamic shared memory.
-template <typename T, int D, int G, bool ROPE>
+template <typename T, int D, int G, bool ROPE, bool WIDE>
 __global__ void __launch_bounds__(32 * F32_WARPS)
 decode_rows(const T* __restrict__ q, const T* __restrict__ ret_k, const T* __restrict__ ret_v, const T* __restrict__ apx_k,
            const int32_t* __restrict__ apx_pos, int64_t cap_ret, int64_t cap_apx, int n_ret, int n_apx, int g, int LH, float scale,
-           float theta, const T* __restrict__ W, bool wide, void* __restrict__ out, int out_bf16) {
+           float theta, const T* __restrict__ W, void* __restrict__ out, int out_bf16) {
     constexpr int EPL = D / 32, REC = Rec<D>::floats, NT = 32 * F32_WARPS;
     extern __shared__ __align__(16) float recs[];               // [F32_WARPS][g][REC]
     __shared__ __align__(16) float comb[G][REC];                // this block's sums, read by the whole cluster
@@ -76,7 +76,7 @@ decode_rows(const T* __restrict__ q, const T* __restrict__ ret_k, const T* __res
 #pragma unroll
         for (int e = 0; e < EPL; ++e) { av[a][e] = 0.f; ak[a][e] = 0.f; qr[a][e] = 0.f; }
         if (a < g) {
-            row_load(q + ((size_t)u * g + a) * D, lane, wide, qr[a]);
+            row_load<WIDE>(q + ((size_t)u * g + a) * D, lane, qr[a]);
 #pragma unroll
             for (int e = 0; e < EPL; ++e) qr[a][e] *= scale;
         }
@@ -89,8 +89,8 @@ decode_rows(const T* __restrict__ q, const T* __restrict__ ret_k, const T* __res
 #pragma unroll
             for (int e = 0; e < EPL; ++e) { kx[r][e] = 0.f; vx[r][e] = 0.f; }
             if (i < hi) {
-                row_load(i < n_ret ? ret_k + ((size_t)u * cap_ret + i) * D : apx_k + ((size_t)u * cap_apx + (i - n_ret)) * D, lane, wide, kx[r]);
-                if (i < n_ret) row_load(ret_v + ((size_t)u * cap_ret + i) * D, lane, wide, vx[r]);
+                row_load<WIDE>(i < n_ret ? ret_k + ((size_t)u * cap_ret + i) * D : apx_k + ((size_t)u * cap_apx + (i - n_ret)) * D, lane, kx[r]);
+                if (i < n_ret) row_load<WIDE>(ret_v + ((size_t)u * cap_ret + i) * D, lane, vx[r]);
             }
         }
 #pragma unroll
@@ -175,7 +175,7 @@ decode_rows(const T* __restrict__ q, const T* __restrict__ ret_k, const T* __res
     const T* Wu = W + (size_t)(u % LH) * D * D;
     float wr[ROWS][EPL];
 #pragma unroll
-    for (int r = 0; r < ROWS; ++r) row_load(Wu + (size_t)(r * F32_WARPS + wid) * D, lane, wide, wr[r]);
+    for (int r = 0; r < ROWS; ++r) row_load<WIDE>(Wu + (size_t)(r * F32_WARPS + wid) * D, lane, wr[r]);
     cl::arrive_release();
     cl::wait_acquire();                                         // every block's sums are ready
     const int mine = rank < g ? (g - rank + C - 1) / C : 0;     // this block merges heads rank, rank + C, ...
@@ -212,7 +212,7 @@ decode_rows(const T* __restrict__ q, const T* __restrict__ ret_k, const T* __res
     __syncthreads();
     for (int k = 0; k < mine; ++k) {
         float a[EPL];
-        row_load<EPL, float>(aks[k], lane, true, a);
+        row_load<true>(aks[k], lane, a);
 #pragma unroll
         for (int r = 0; r < ROWS; ++r) {
             float x = 0.f;
@@ -239,17 +239,16 @@ static bool rows_at_16_bytes(const void* q, const vector_cache* ch, const void* 
     return (all & 15) == 0;
 }
 
-template <typename T, int D, int G, bool ROPE>
+template <typename T, int D, int G, bool ROPE, bool WIDE>
 static vector_status launch_decode_rows(const Dims& dm, const void* q, const vector_cache* ch, const void* W, void* out,
                                        int out_dtype, cudaStream_t st) {
-    auto kern = decode_rows<T, D, G, ROPE>;
+    auto kern = decode_rows<T, D, G, ROPE, WIDE>;
     static PerDeviceOnce once;
     if (once.first()) {
         cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, F32_WARPS * G * Rec<D>::floats * 4);
         if (e == cudaSuccess) e = cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
         if (e != cudaSuccess) { once.undo(); VEC_CUDA_CHECK(e); }
     }
-    const bool wide = rows_at_16_bytes(q, ch, W);
     // blocks a unit: one pass over the rows of a block's warps at the least, four blocks a multiprocessor at the most
     const int64_t rows = ch->n_ret + ch->n_apx;
     int64_t c = (rows + F32_ROWS * F32_WARPS - 1) / (F32_ROWS * F32_WARPS);
@@ -260,7 +259,7 @@ static vector_status launch_decode_rows(const Dims& dm, const void* q, const vec
     VEC_CUDA_CHECK(launch_maybe_dependent(true, (int)c, kern, dim3((unsigned)(c * dm.U)), dim3(32 * F32_WARPS),
                                           (size_t)F32_WARPS * dm.g * Rec<D>::floats * 4, st, (const T*)q, (const T*)ch->ret_k,
                                           (const T*)ch->ret_v, (const T*)ch->apx_k, ch->apx_pos, ch->cap_ret, ch->cap_apx,
-                                          (int)ch->n_ret, (int)ch->n_apx, dm.g, dm.LH, dm.scale, dm.theta, (const T*)W, wide, out,
+                                          (int)ch->n_ret, (int)ch->n_apx, dm.g, dm.LH, dm.scale, dm.theta, (const T*)W, out,
                                           out_dtype == VECTOR_BF16 ? 1 : 0));
     return VECTOR_OK;
 }
@@ -406,12 +405,12 @@ static vector_status launch_decode_bf16(const Dims& dm, const void* q, const vec
     return VECTOR_OK;
 }
 
-template <typename T, int D, bool ROPE>
+template <typename T, int D, bool ROPE, bool WIDE>
 static vector_status launch_decode_g(const Dims& dm, const void* q, const vector_cache* ch, const void* W, void* out, int out_dtype,
                                      cudaStream_t st) {
-    if (dm.g <= 2) return launch_decode_rows<T, D, 2, ROPE>(dm, q, ch, W, out, out_dtype, st);
-    if (dm.g <= 4) return launch_decode_rows<T, D, 4, ROPE>(dm, q, ch, W, out, out_dtype, st);
-    return launch_decode_rows<T, D, 8, ROPE>(dm, q, ch, W, out, out_dtype, st);
+    if (dm.g <= 2) return launch_decode_rows<T, D, 2, ROPE, WIDE>(dm, q, ch, W, out, out_dtype, st);
+    if (dm.g <= 4) return launch_decode_rows<T, D, 4, ROPE, WIDE>(dm, q, ch, W, out, out_dtype, st);
+    return launch_decode_rows<T, D, 8, ROPE, WIDE>(dm, q, ch, W, out, out_dtype, st);
 }
 
 }  // namespace vec
@@ -439,15 +438,18 @@ extern "C" vector_status vector_decode_attn(const vector_shape* shape, const voi
     if (dm.rope && cache->n_apx > 0 && !cache->apx_pos) return VECTOR_ERR_NULL;
     cudaStream_t st = (cudaStream_t)stream;
     float* partial = (float*)ws;
-    if (dm.dtype == VECTOR_F32)
-        return dm.d == 64 ? (dm.rope ? launch_decode_g<float, 64, true>(dm, q, cache, W, out, out_dtype, st)
-                                     : launch_decode_g<float, 64, false>(dm, q, cache, W, out, out_dtype, st))
-                          : (dm.rope ? launch_decode_g<float, 128, true>(dm, q, cache, W, out, out_dtype, st)
-                                     : launch_decode_g<float, 128, false>(dm, q, cache, W, out, out_dtype, st));
-    // 64-channel bf16 rows that do not lie at multiples of 16 bytes, which TMA would refuse, run on the CUDA-core kernel
-    if (dm.d == 64 && !rows_at_16_bytes(q, cache, W))
-        return dm.rope ? launch_decode_g<__nv_bfloat16, 64, true>(dm, q, cache, W, out, out_dtype, st)
-                       : launch_decode_g<__nv_bfloat16, 64, false>(dm, q, cache, W, out, out_dtype, st);
+    // Rows off a 16-byte boundary: element by element, 64-channel bf16 ones, which TMA would refuse, on the CUDA-core kernel too
+    const bool wide = rows_at_16_bytes(q, cache, W);
+    if (dm.dtype == VECTOR_F32) {
+        auto launch = dm.d == 64 ? (dm.rope ? (wide ? launch_decode_g<float, 64, true, true> : launch_decode_g<float, 64, true, false>)
+                                            : (wide ? launch_decode_g<float, 64, false, true> : launch_decode_g<float, 64, false, false>))
+                                 : (dm.rope ? (wide ? launch_decode_g<float, 128, true, true> : launch_decode_g<float, 128, true, false>)
+                                            : (wide ? launch_decode_g<float, 128, false, true> : launch_decode_g<float, 128, false, false>));
+        return launch(dm, q, cache, W, out, out_dtype, st);
+    }
+    if (dm.d == 64 && !wide)
+        return dm.rope ? launch_decode_g<__nv_bfloat16, 64, true, false>(dm, q, cache, W, out, out_dtype, st)
+                       : launch_decode_g<__nv_bfloat16, 64, false, false>(dm, q, cache, W, out, out_dtype, st);
     if (dm.d == 64) return launch_decode_bf16<64>(dm, q, cache, W, out, out_dtype, mode, partial, st);
     return launch_decode_bf16<128>(dm, q, cache, W, out, out_dtype, mode, partial, st);
 }

@@ -20,17 +20,17 @@ constexpr int ST = 64;    // tile edge (rows and keys) of the CUDA-core score ke
 // tile of the one that changes before they work on this one: with 32-channel slices loaded between barriers a pass was a
 // chain of load latencies (13 + 11 us for 2 units of 64 rows and 1024 keys).
 template <int D> struct TileRegs { float4 v[ST * D / 1024]; };
-// wide: the rows lie at multiples of 16 bytes (fp32); otherwise, and for bf16, element by element.
-template <typename T, int D>
-__device__ __forceinline__ void tile_request(const T* __restrict__ src, int64_t row0, int64_t n_rows, bool wide, TileRegs<D>& t) {
+// WIDE: fp32 rows at multiples of 16 bytes; otherwise element by element.
+template <bool WIDE, typename T, int D>
+__device__ __forceinline__ void tile_request(const T* __restrict__ src, int64_t row0, int64_t n_rows, TileRegs<D>& t) {
 #pragma unroll
     for (int e = 0; e < ST * D / 1024; ++e) {
         const int idx = threadIdx.x + 256 * e, r = idx / (D / 4), c4 = idx % (D / 4);
-        t.v[e] = make_float4(0.f, 0.f, 0.f, 0.f);
-        if (row0 + r < n_rows) {
-            const T* p = src + (row0 + r) * D + 4 * c4;
-            if (sizeof(T) == 4 && wide) t.v[e] = *reinterpret_cast<const float4*>(p);
-            else t.v[e] = make_float4(to_f32(p[0]), to_f32(p[1]), to_f32(p[2]), to_f32(p[3]));
+        const T* p = src + (row0 + r) * D + 4 * c4;
+        if constexpr (WIDE) {
+            t.v[e] = row0 + r < n_rows ? *reinterpret_cast<const float4*>(p) : make_float4(0.f, 0.f, 0.f, 0.f);
+        } else {
+            t.v[e] = row0 + r < n_rows ? make_float4(to_f32(p[0]), to_f32(p[1]), to_f32(p[2]), to_f32(p[3])) : make_float4(0.f, 0.f, 0.f, 0.f);
         }
     }
 }
@@ -67,10 +67,10 @@ __device__ __forceinline__ void tile_qk(const float* Qs, const float* Ks, float 
 template <int D> constexpr int tile_smem() { return 2 * ST * (D + 1) * (int)sizeof(float); }
 
 // grid (n_chunks, row_tiles, U), 256 threads, tile_smem of dynamic shared memory
-template <typename T, int D>
+template <typename T, int D, bool WIDE>
 __global__ void __launch_bounds__(256)
 score_pass1_generic(const T* __restrict__ Q, const T* __restrict__ K, int64_t N, int R, int w,
-                    float scale, int64_t chunk_len, bool wide, float2* __restrict__ partial) {
+                    float scale, int64_t chunk_len, float2* __restrict__ partial) {
     extern __shared__ float tiles[];
     float *Qs = tiles, *Ks = tiles + ST * (D + 1);
     asm volatile("griddepcontrol.wait;\n" ::: "memory");        // launched as a programmatic dependent: nothing is touched before
@@ -82,10 +82,10 @@ score_pass1_generic(const T* __restrict__ Q, const T* __restrict__ K, int64_t N,
     const int64_t k_begin = (int64_t)chunk * chunk_len;
     const int64_t k_end = min(N, k_begin + chunk_len);
     TileRegs<D> next;
-    tile_request(Ku, k_begin, k_end, wide, next);
+    tile_request<WIDE>(Ku, k_begin, k_end, next);
     {
         TileRegs<D> q;
-        tile_request(Qu, row0, R, wide, q);
+        tile_request<WIDE>(Qu, row0, R, q);
         tile_store<D>(q, Qs);
     }
     float m[4], l[4];
@@ -101,7 +101,7 @@ score_pass1_generic(const T* __restrict__ Q, const T* __restrict__ K, int64_t N,
         __syncthreads();                                  // the tile before this one has been read
         tile_store<D>(next, Ks);
         __syncthreads();
-        if (key0 + ST < k_end) tile_request(Ku, key0 + ST, k_end, wide, next);
+        if (key0 + ST < k_end) tile_request<WIDE>(Ku, key0 + ST, k_end, next);
         float acc[4][4];
         tile_qk<D>(Qs, Ks, acc);
 #pragma unroll
@@ -175,10 +175,10 @@ score_lse_rows(const float2* __restrict__ partial, int R, int n_chunks, float* _
 
 // grid (key_tiles, U), 256 threads, tile_smem of dynamic shared memory.  INLINE_LSE: a block forms the normalisers of its
 // rows itself from the chunk partials (a launch less; every key tile repeats it).
-template <typename T, int D, bool INLINE_LSE>
+template <typename T, int D, bool INLINE_LSE, bool WIDE>
 __global__ void __launch_bounds__(256)
 score_pass2_generic(const T* __restrict__ Q, const T* __restrict__ K, int64_t N, int R, int w,
-                    float scale, const float2* __restrict__ partial, int n_chunks, const float* __restrict__ lse, bool wide,
+                    float scale, const float2* __restrict__ partial, int n_chunks, const float* __restrict__ lse,
                     float* __restrict__ raw) {
     extern __shared__ float tiles[];
     float *Qs = tiles, *Ks = tiles + ST * (D + 1);
@@ -193,8 +193,8 @@ score_pass2_generic(const T* __restrict__ Q, const T* __restrict__ K, int64_t N,
     TileRegs<D> next;
     {
         TileRegs<D> k;
-        tile_request(K + (size_t)u * N * D, key0, N, wide, k);
-        tile_request(Qu, 0, R, wide, next);
+        tile_request<WIDE>(K + (size_t)u * N * D, key0, N, k);
+        tile_request<WIDE>(Qu, 0, R, next);
         tile_store<D>(k, Ks);
     }
     float col[4] = {0.f, 0.f, 0.f, 0.f};
@@ -209,7 +209,7 @@ score_pass2_generic(const T* __restrict__ Q, const T* __restrict__ K, int64_t N,
             lse_s[tid] = lse[(size_t)u * R + row0 + tid];
         }
         __syncthreads();
-        if (row0 + ST < R) tile_request(Qu, row0 + ST, R, wide, next);
+        if (row0 + ST < R) tile_request<WIDE>(Qu, row0 + ST, R, next);
         float acc[4][4];
         tile_qk<D>(Qs, Ks, acc);
 #pragma unroll
@@ -257,17 +257,16 @@ __global__ void score_pool_kernel(const float* __restrict__ raw, int64_t N, int 
 }
 
 // Workspace: chunk partials | lse | raw, where the caller does not take it; fewer chunks where it would not hold theirs.
-template <typename T, int D>
+template <typename T, int D, bool WIDE>
 static vector_status launch_score(const Dims& dm, const void* Q_, const void* K_, int64_t N, float* scores, float* raw_out, char* ws,
                                   size_t ws_bytes, cudaStream_t st) {
     constexpr int SMEM = tile_smem<D>();
     const T *Q = (const T*)Q_, *K = (const T*)K_;
-    const bool wide = (((uintptr_t)Q_ | (uintptr_t)K_) & 15) == 0;
     static PerDeviceOnce once;
     if (once.first()) {
-        cudaError_t e = cudaFuncSetAttribute(score_pass1_generic<T, D>, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM);
-        if (e == cudaSuccess) e = cudaFuncSetAttribute(score_pass2_generic<T, D, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM);
-        if (e == cudaSuccess) e = cudaFuncSetAttribute(score_pass2_generic<T, D, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM);
+        cudaError_t e = cudaFuncSetAttribute(score_pass1_generic<T, D, WIDE>, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM);
+        if (e == cudaSuccess) e = cudaFuncSetAttribute(score_pass2_generic<T, D, true, WIDE>, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM);
+        if (e == cudaSuccess) e = cudaFuncSetAttribute(score_pass2_generic<T, D, false, WIDE>, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM);
         if (e != cudaSuccess) { once.undo(); VEC_CUDA_CHECK(e); }
     }
     const size_t lse_b = align256((size_t)dm.U * dm.R * sizeof(float)), raw_b = raw_out ? 0 : align256((size_t)dm.U * (size_t)N * sizeof(float));
@@ -281,16 +280,16 @@ static vector_status launch_score(const Dims& dm, const void* Q_, const void* K_
     chunk_len = (chunk_len + ST - 1) / ST * ST;
     n_chunks = (int)((N + chunk_len - 1) / chunk_len);            // none empty
     const int row_tiles = (dm.R + ST - 1) / ST;
-    VEC_CUDA_CHECK(launch_maybe_dependent(true, score_pass1_generic<T, D>, dim3(n_chunks, row_tiles, dm.U), dim3(256), SMEM, st, Q, K, N,
-                                          dm.R, dm.w, dm.scale, chunk_len, wide, partial));
+    VEC_CUDA_CHECK(launch_maybe_dependent(true, score_pass1_generic<T, D, WIDE>, dim3(n_chunks, row_tiles, dm.U), dim3(256), SMEM, st, Q, K, N,
+                                          dm.R, dm.w, dm.scale, chunk_len, partial));
     // the partials of a row tile: no more than the rows' own elements
     const bool inline_lse = n_chunks <= 32;
     if (!inline_lse)
         VEC_CUDA_CHECK(launch_maybe_dependent(true, score_lse_rows, dim3((dm.R + 63) / 64, dm.U), dim3(256), 0, st, partial, dm.R,
                                               n_chunks, lse));
-    VEC_CUDA_CHECK(launch_maybe_dependent(true, inline_lse ? score_pass2_generic<T, D, true> : score_pass2_generic<T, D, false>,
+    VEC_CUDA_CHECK(launch_maybe_dependent(true, inline_lse ? score_pass2_generic<T, D, true, WIDE> : score_pass2_generic<T, D, false, WIDE>,
                                           dim3((unsigned)((N + ST - 1) / ST), dm.U), dim3(256), SMEM, st, Q, K, N, dm.R, dm.w, dm.scale,
-                                          partial, n_chunks, lse, wide, raw));
+                                          partial, n_chunks, lse, raw));
     int64_t total = (int64_t)dm.U * N;
     VEC_CUDA_CHECK(launch_maybe_dependent(true, score_pool_kernel, dim3((unsigned)((total + 255) / 256)), dim3(256), 0, st, raw, N, dm.w,
                                           dm.pool_kernel / 2, total, scores));
@@ -364,12 +363,13 @@ extern "C" vector_status vector_score(const vector_shape* shape, const void* Q_o
     if (!ws || ((uintptr_t)ws & 255) || ws_bytes < score_ws_bytes(dm, N, need_raw)) return VECTOR_ERR_WORKSPACE;
     char* p = (char*)ws;
     cudaStream_t st = (cudaStream_t)stream;
-    // 64-channel bf16 rows that do not lie at multiples of 16 bytes, which TMA would refuse, run on the CUDA-core kernels
-    const bool loose = dm.d == 64 && (((uintptr_t)Q_obs | (uintptr_t)K | (uintptr_t)scores | (uintptr_t)raw_out) & 15);
-    if (score_uses_tc(dm) && !loose)
+    // Rows off a 16-byte boundary: element by element, 64-channel bf16 ones, which TMA would refuse, on the CUDA-core kernels too
+    const bool wide = (((uintptr_t)Q_obs | (uintptr_t)K) & 15) == 0;
+    if (score_uses_tc(dm) && (dm.d == 128 || (wide && (((uintptr_t)scores | (uintptr_t)raw_out) & 15) == 0)))
         return dm.d == 64 ? launch_score_tc<64>(dm, Q_obs, K, N, scores, raw_out, p, st)
                           : launch_score_tc<128>(dm, Q_obs, K, N, scores, raw_out, p, st);
-    if (dm.dtype == VECTOR_BF16) return launch_score<__nv_bfloat16, 64>(dm, Q_obs, K, N, scores, raw_out, p, ws_bytes, st);
-    return dm.d == 64 ? launch_score<float, 64>(dm, Q_obs, K, N, scores, raw_out, p, ws_bytes, st)
-                      : launch_score<float, 128>(dm, Q_obs, K, N, scores, raw_out, p, ws_bytes, st);
+    auto launch = dm.dtype == VECTOR_BF16 ? launch_score<__nv_bfloat16, 64, false>
+                : dm.d == 64 ? (wide ? launch_score<float, 64, true> : launch_score<float, 64, false>)
+                             : (wide ? launch_score<float, 128, true> : launch_score<float, 128, false>);
+    return launch(dm, Q_obs, K, N, scores, raw_out, p, ws_bytes, st);
 }
