@@ -53,18 +53,18 @@ constexpr int BOX_BYTES = 8192;              // 64 rows x 128 bytes
 constexpr float SLACK = 8.f;
 template <int D, bool ROPE> struct Cfg {
     static constexpr int HALF_BYTES = 64 * 2 * D;                    // 64 rows as D / 64 swizzled boxes
-    // 64 channels: everything to fp32's own precision, as CUDA cores give it.  A softmax weight enters as three bf16 parts, which
-    // keep its 24 bits (two keep sixteen); an MMA cuts its sums off instead of rounding them, so that the sums of
-    // 32 rows start at zero and are added up in fp32; the map is applied to the key sums in fp32.  With up to
+    // 64 channels: everything to fp32's own precision, as CUDA cores give it.  A softmax weight and a key sum on its way through the
+    // map enter as three bf16 parts, which keep their 24 bits (two keep sixteen); an MMA cuts its sums off instead of rounding them, so
+    // that the sums of 32 rows and of 32 columns of the map start at zero and are added up in fp32.  With up to
     // four heads the third parts take MMA rows that nobody else uses.  Error of an fp32 output against
-    // fp64, median over the heads of eight sizes of 1 to 64 layers, 8 to 512 units and up to 78642 rows: 1.0e-7 to 1.7e-7 (two parts, sums
-    // in the MMAs: 1.0e-6 to 2.2e-6; CUDA cores: 1.2e-7 to 4.4e-7).  512 units, 431 MB: 82 -> 87 us a step with the appended row.
+    // fp64, median over the heads of ten sizes of 1 to 64 layers, 8 to 512 units and up to 78642 rows: 1.1e-7 to 1.8e-7 (two parts, sums
+    // in the MMAs: 1.0e-6 to 2.2e-6; CUDA cores: 1.2e-7 to 4.4e-7).  512 units, 431 MB: 82 -> 85.5 us a step with the appended row.
     static constexpr bool EXACT = D == 64;
     static constexpr int PARTS = EXACT ? 3 : 2;
     static constexpr int SLOT_BYTES = 2 * HALF_BYTES;                // retained: K | V; key-only: keys 0-63 | keys 64-127
     // With 64-channel heads a softmax step brings in half the bytes for the same softmax arithmetic: a fourth consumer
     // warp (one to a warp scheduler) makes up for it.
-    // Measured: 512 units, 1639 retained + 3276 key-only rows, 431 MB: 87 us with the appended row = 5.0 TB/s (856 us on
+    // Measured: 512 units, 1639 retained + 3276 key-only rows, 431 MB: 85.5 us with the appended row = 5.0 TB/s (856 us on
     // CUDA cores).
     // With RoPE decoupling a consumer is a team (decode_rope.cuh): a score warp and some sum warps.
     // Four teams at 64 channels, of two sum warps with as many channel pairs each as the four have at 128.
@@ -355,23 +355,27 @@ __device__ __forceinline__ void accumulate_step(uint32_t vbase, int kk, const ui
     }
 }
 
-// The key sums of up to eight heads on their way through the map.  128 channels: as bf16 hi + lo (sixteen mantissa bits);
-// 64 channels: fp32.
-template <int D> struct KeySums { __align__(16) __nv_bfloat16 hi[8][D], lo[8][D]; };
-template <> struct KeySums<64> { __align__(16) float v[8][64]; };
-__device__ __forceinline__ void store_key_sum(KeySums<128>& ks, int head, int c, float v) {
-    const __nv_bfloat16 hi = __float2bfloat16_rn(v);
-    ks.hi[head][c] = hi;
-    ks.lo[head][c] = __float2bfloat16_rn(v - __bfloat162float(hi));
+// The key sums of up to eight heads on their way through the map, in bf16 parts: two (sixteen mantissa bits), or three (all 24).
+template <int D> struct KeySums { __align__(16) __nv_bfloat16 part[Cfg<D, false>::PARTS][8][D]; };
+template <int D>
+__device__ __forceinline__ void store_key_sum(KeySums<D>& ks, int head, int c, float v) {
+#pragma unroll
+    for (int i = 0; i < Cfg<D, false>::PARTS; ++i) {
+        const __nv_bfloat16 x = __float2bfloat16_rn(v);
+        ks.part[i][head][c] = x;
+        v -= __bfloat162float(x);
+    }
 }
-__device__ __forceinline__ void store_key_sum(KeySums<64>& ks, int head, int c, float v) { ks.v[head][c] = v; }
 
 // Rows 16 mt .. + 15 of W times the key sums of n heads: pw[head][row].  One warp, M = 16 output channels, N = the heads
 // (padded to 8), K = D: the A fragments are read straight from the map in global memory, 16 bytes a load -- thread
 // (row r, quarter t) of a warp holds columns 8 (t + 4 jj) .. + 7 of rows r and r + 8, and the k slots of MMA step
 // 2 jj + h stand for columns 8 (t + 4 jj) + 4 h .. + 3, which the B fragments follow; the map's elements are bf16 as stored.
-__device__ __forceinline__ void map_rows(const __nv_bfloat16* __restrict__ W, int mt, int n, const KeySums<128>& ks, float (&pw)[8][128], int lane) {
-    constexpr int D = 128, PIECES = D / 8;                           // 16-byte pieces of a row of W
+// Three parts: the MMAs of the first start at zero and are added up in fp32, as the sums before them are (Cfg::EXACT).
+template <int D>
+__device__ __forceinline__ void map_rows(const __nv_bfloat16* __restrict__ W, int mt, int n, const KeySums<D>& ks, float (&pw)[8][D], int lane) {
+    constexpr int PARTS = Cfg<D, false>::PARTS;
+    constexpr int PIECES = D / 8;                                    // 16-byte pieces of a row of W
     const int row = lane >> 2, quarter = lane & 3;
     const uint4* Wu = reinterpret_cast<const uint4*>(W);
     uint4 A[D / 16];
@@ -380,42 +384,37 @@ __device__ __forceinline__ void map_rows(const __nv_bfloat16* __restrict__ W, in
         A[2 * jj + 0] = Wu[(16 * mt + row) * PIECES + quarter + 4 * jj];
         A[2 * jj + 1] = Wu[(16 * mt + row + 8) * PIECES + quarter + 4 * jj];
     }
-    float d[4] = {0.f, 0.f, 0.f, 0.f};
+    float d[4] = {0.f, 0.f, 0.f, 0.f}, small[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll
     for (int jj = 0; jj < D / 32; ++jj) {
         const uint4 r0 = A[2 * jj], r1 = A[2 * jj + 1];
         const int col = 8 * (quarter + 4 * jj);
-        const uint4 bh = *reinterpret_cast<const uint4*>(&ks.hi[row][col]);      // B column = head `row`
-        const uint4 bl = *reinterpret_cast<const uint4*>(&ks.lo[row][col]);
-        mma_16(d, r0.x, r1.x, r0.y, r1.y, bh.x, bh.y);
-        mma_16(d, r0.x, r1.x, r0.y, r1.y, bl.x, bl.y);
-        mma_16(d, r0.z, r1.z, r0.w, r1.w, bh.z, bh.w);
-        mma_16(d, r0.z, r1.z, r0.w, r1.w, bl.z, bl.w);
+        uint4 b[PARTS];
+#pragma unroll
+        for (int i = 0; i < PARTS; ++i) b[i] = *reinterpret_cast<const uint4*>(&ks.part[i][row][col]);      // B column = head `row`
+        if constexpr (PARTS == 3) {
+            float t[2][4] = {{0.f, 0.f, 0.f, 0.f}, {0.f, 0.f, 0.f, 0.f}};
+            mma_16(t[0], r0.x, r1.x, r0.y, r1.y, b[0].x, b[0].y);
+            mma_16(t[1], r0.z, r1.z, r0.w, r1.w, b[0].z, b[0].w);
+#pragma unroll
+            for (int i = 2; i > 0; --i) {
+                mma_16(small, r0.x, r1.x, r0.y, r1.y, b[i].x, b[i].y);
+                mma_16(small, r0.z, r1.z, r0.w, r1.w, b[i].z, b[i].w);
+            }
+#pragma unroll
+            for (int e = 0; e < 4; ++e) d[e] += t[0][e] + t[1][e];
+        } else {
+#pragma unroll
+            for (int i = 0; i < PARTS; ++i) mma_16(d, r0.x, r1.x, r0.y, r1.y, b[i].x, b[i].y);
+#pragma unroll
+            for (int i = 0; i < PARTS; ++i) mma_16(d, r0.z, r1.z, r0.w, r1.w, b[i].z, b[i].w);
+        }
     }
+#pragma unroll
+    for (int e = 0; e < 4; ++e) d[e] += small[e];
     // d[0], d[1]: row `row`, heads 2 quarter and 2 quarter + 1; d[2], d[3]: row `row` + 8
     if (2 * quarter < n) { pw[2 * quarter][16 * mt + row] = d[0]; pw[2 * quarter][16 * mt + row + 8] = d[2]; }
     if (2 * quarter + 1 < n) { pw[2 * quarter + 1][16 * mt + row] = d[1]; pw[2 * quarter + 1][16 * mt + row + 8] = d[3]; }
-}
-// Row c of W times the key sums of one head, 64 channels: a thread's row is 128 bytes, the key sums are the same for a warp.
-__device__ __forceinline__ float map_row(const __nv_bfloat16* __restrict__ W, int c, const KeySums<64>& ks, int head) {
-    const uint4* Wr = reinterpret_cast<const uint4*>(W + (size_t)c * 64);
-    float x[4] = {0.f, 0.f, 0.f, 0.f};
-    uint4 w[8];
-#pragma unroll
-    for (int p = 0; p < 8; ++p) w[p] = Wr[p];
-#pragma unroll
-    for (int p = 0; p < 8; ++p) {
-        const uint32_t e[4] = {w[p].x, w[p].y, w[p].z, w[p].w};
-#pragma unroll
-        for (int h = 0; h < 2; ++h) {
-            const float4 k = *reinterpret_cast<const float4*>(&ks.v[head][8 * p + 4 * h]);
-            x[0] = fmaf(__uint_as_float(e[2 * h] << 16), k.x, x[0]);
-            x[1] = fmaf(__uint_as_float(e[2 * h] & 0xffff0000u), k.y, x[1]);
-            x[2] = fmaf(__uint_as_float(e[2 * h + 1] << 16), k.z, x[2]);
-            x[3] = fmaf(__uint_as_float(e[2 * h + 1] & 0xffff0000u), k.w, x[3]);
-        }
-    }
-    return (x[0] + x[1]) + (x[2] + x[3]);
 }
 
 // The last part of the CLUSTER form: combines the records of a unit, which its cluster's blocks hold in shared
@@ -511,16 +510,11 @@ __device__ __forceinline__ void cluster_merge(const float* recs, unsigned char* 
     cl::arrive_release();                                             // this block reads no other block's memory from here on
     merge_sync<NT>();
     if (mine > 0) {
-        if constexpr (D == 128) {
-            for (int mt = wid; mt < D / 16; mt += NT / 32) map_rows(Wu, mt, mine, ks, pw, lane);
-            merge_sync<NT>();
-        }
+        for (int mt = wid; mt < D / 16; mt += NT / 32) map_rows(Wu, mt, mine, ks, pw, lane);
+        merge_sync<NT>();
         for (int e = tid; e < mine * D; e += NT) {
             const int k = e / D, c = e - k * D;
-            float x;
-            if constexpr (D == 128) x = pw[k][c];
-            else x = map_row(Wu, c, ks, k);
-            const float o = (avs[k][c] + x) / Ls[k];
+            const float o = (avs[k][c] + pw[k][c]) / Ls[k];
             const size_t at = (size_t)(rank + k * nblk) * D + c;
             if (out_f32) reinterpret_cast<float*>(out_u)[at] = o;
             else reinterpret_cast<__nv_bfloat16*>(out_u)[at] = __float2bfloat16_rn(o);
@@ -737,14 +731,14 @@ decode_stream_bf16(const __nv_bfloat16* __restrict__ q, const __grid_constant__ 
 // Combines the records of a unit, applies the unit's map to the p-weighted key sum and normalises:
 //   o = (sum_j f_j s_j acc_v_j + W sum_j f_j acc_k_j) / sum_j f_j l_j,   f_j = exp(m_j - max m).
 // Every load of a phase is independent of the others, so a phase costs one memory latency.
-// The product W (sum f acc_k) runs on warp-level MMAs (map_rows), or, for 64 channels, on CUDA cores (map_row).
+// The product W (sum f acc_k) runs on warp-level MMAs (map_rows).
 template <typename TO, int D, int MAXT>
 __global__ void __launch_bounds__(MAXT, MAXT == 512 ? 3 : 1)
 decode_merge_bf16(const float* __restrict__ partial, const __nv_bfloat16* __restrict__ W, int LH, int g,
                        Plan pl, int apply_w, int cw, TO* __restrict__ out) {
     constexpr int REC = 4 + 2 * D;
     __shared__ KeySums<D> ks;
-    __shared__ float pw[D == 128 ? 8 : 1][D];  // W times the key sum
+    __shared__ float pw[8][D];                 // W times the key sum
     constexpr int MAX_REC = 12 * Cfg<D, false>::CONSUMER_WARPS, REC_PER_LANE = (MAX_REC + 31) / 32;      // of a unit: twelve blocks' at the most
     __shared__ float fv[8][MAX_REC], fk[8][MAX_REC];     // per head, per record: factor for the value part / the key part
     __shared__ float Ls[8];
@@ -820,15 +814,9 @@ decode_merge_bf16(const float* __restrict__ partial, const __nv_bfloat16* __rest
     }
     store_key_sum(ks, a, c, ak);
     __syncthreads();
-    float x;
-    if constexpr (D == 128) {
-        for (int mt = wid; mt < D / 16; mt += nwarps) map_rows(Wu, mt, g, ks, pw, lane);
-        __syncthreads();
-        x = pw[a][c];
-    } else {
-        x = map_row(Wu, c, ks, a);
-    }
-    store_out(out + ((size_t)u * g + a) * D + c, (av + x) / Ls[a]);
+    for (int mt = wid; mt < D / 16; mt += nwarps) map_rows(Wu, mt, g, ks, pw, lane);
+    __syncthreads();
+    store_out(out + ((size_t)u * g + a) * D + c, (av + pw[a][c]) / Ls[a]);
 }
 
 }  // namespace dbf

@@ -17,7 +17,7 @@
 // cycles per 64 keys, 2300 of them busy) and the sum warps (2500 busy) waiting for one another.  Measured, 128 units of 3000
 // retained + 6000 key-only rows, 393 MB, with the appended row and the merge: 86 us; 104 us with warps that owned whole tiles
 // and twelve helpers that turned keys back in shared memory (a fence and three block barriers per 64 keys).
-// 64 channels, 512 units of 1639 + 3276 rows: 201 us a step with the appended row, bound by the sum warps' instructions (about
+// 64 channels, 512 units of 1639 + 3276 rows: 197 us a step with the appended row, bound by the sum warps' instructions (about
 // 1000 for 64 key-only rows; 114 us with fp16 keys, 1139 us on CUDA cores; sum warps of eight pairs 210, five teams 203, loops
 // rolled up 207).  Error of an fp32 output against fp64, median over the heads: 1.8e-7 to 4.1e-7 (fp16: 1.1e-4, CUDA cores: 2.0e-7 to 5.5e-7).
 // The angle is position * theta^(-2c/D), taken as the 32-bit product of the position and the
