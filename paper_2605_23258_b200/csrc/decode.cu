@@ -282,16 +282,16 @@ int* kernel_fault_address() {
 // Blocks per unit of the one-launch (cluster) form, 0 = stream and merge.  A cluster lies within one GPC and every
 // block fills its multiprocessor, so the largest size is taken at which all U clusters are resident at once.  That may
 // use fewer multiprocessors than the streaming form (48 units would need clusters of three that fit), whose second
-// kernel and records in global memory cost as much as some tiles of a block: twice as many of 64 channels, which are half
+// kernel and records in global memory cost as much as some tiles of a block: more of 64 channels, which are half
 // the size, and fewer with RoPE, whose tiles take longer.  The form with the fewer tiles a block, that cost included, runs.
-// Measured, four query heads, us per step in a graph, cluster against stream: 128 channels, 8 units of 2457 rows 9.2 / 12.4,
-// of 19660 rows 21.9 / 25.2; 48 units of 1200 rows 13.4 / 15.7, 2457 rows 18.3 / 18.7, 4800 rows 27.9 / 25.7, with RoPE 15.2 /
-// 18.0, 23.2 / 22.6, 38.6 / 33.5; 64 channels, 48 units of 4800 rows 16.1 / 18.8, with RoPE of 2457 rows 17.4 / 18.3, 4800 rows
-// 28.0 / 25.8.
+// Measured, four query heads, us per step in a graph, cluster against stream: 128 channels, 8 units of 2457 rows 9.4 / 12.5,
+// of 19660 rows 22.5 / 25.4; 48 units of 1200 rows 13.5 / 16.1, 2457 rows 18.5 / 19.5, 4800 rows 26.6 / 24.8, with RoPE 15.6 /
+// 19.1, 23.7 / 23.8, 37.7 / 32.8; 64 channels, 48 units of 4800 rows 18.1 / 20.1, 7200 rows 23.3 / 23.4, with RoPE 1200 rows 16.9 /
+// 21.2, 2457 rows 27.7 / 27.1, 4800 rows 45.2 / 38.2.
 template <int D, bool ROPE>
 static int decode_cluster_size(const dbf::Plan& pl, int U) {
     using C = dbf::Cfg<D, ROPE>;
-    constexpr int MAXC = dbf::MAX_CLUSTER, EXTRA_TILES = (ROPE ? 6 : 9) * 128 / D;
+    constexpr int MAXC = dbf::MAX_CLUSTER, EXTRA_TILES = D == 128 ? (ROPE ? 6 : 9) : ROPE ? 2 : 13;
     static int resident[PerDeviceOnce::kMax][MAXC + 1] = {};      // clusters of each size the device holds at once
     static std::mutex mu;
     int dev = -1;
