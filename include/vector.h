@@ -28,9 +28,11 @@
  *    row-major, one d x d map per (layer, KV head): index l * n_kv_heads + h.
  *  - Supported: head_dim 64 or 128; dtype fp32 or bf16; n_q_heads % n_kv_heads == 0,
  *    g <= 8; window * g <= 1024; pool_kernel odd, 1..15; at most 65535 units per call;
- *    every device pointer 16-byte aligned.  The tensor-core kernels (tcgen05 score passes and residual,
- *    TMA-fed decode) serve bf16; fp32, and head_dim 64 with one map per layer, run on CUDA-core kernels of
- *    the same interface, written for parity rather than speed.
+ *    every device pointer 16-byte aligned (vector_score, vector_residual and vector_decode_attn also take fp32
+ *    rows, and bf16 rows of 64 channels, at any element).  The tensor-core kernels (tcgen05 score passes and
+ *    residual, TMA-fed decode) serve bf16; fp32 runs on CUDA-core kernels of the same interface, written for
+ *    parity rather than speed, and so do with one map per layer head_dim 64 and, in decode, every bf16 shape but
+ *    head_dim 128 with 8 KV heads and at most 32 query heads per layer.
  */
 #ifndef VECTOR_H_
 #define VECTOR_H_
@@ -250,6 +252,9 @@ VECTOR_API vector_status vector_append(const vector_shape* shape, const vector_c
  *                       three times slower than mode 0, which gives the same sum by linearity
  * With shape->rope_enabled, k~_i is the stored key turned back by cache->apx_pos (required then);
  * the logit always uses the stored key.
+ * Arithmetic: logits and sums in fp32.  fp32, and bf16 with head_dim 64: everything else too.  bf16 with
+ * head_dim 128: the p_i and sum_A p_i k~_i are carried to sixteen bits, and a k~_i turned back to eleven (fp16:
+ * |k~| beyond 65504 saturates).
  * q: device [U][g][d] of shape->dtype; out: device [U][g][d] of out_dtype.
  */
 VECTOR_API vector_status vector_decode_attn(const vector_shape* shape, const void* q, const vector_cache* cache,
