@@ -8,23 +8,29 @@
 // with N = 256 per h'; the epilogue subtracts the value rows of the two heads, squares and adds along
 // its TMEM lane.
 //
-// What bounds it is what a tile fetches: the keys once per pair of output heads and the whole map, 3.25 MB for
-// 17.7 us of tensor work at Hkv = 8, mostly from L2.  So the loads are kept in flight across steps (half a head's
-// channels, 48 KB, in one of four stages), the products take two output heads at a time (a third fewer bytes than
-// head by head), and the value rows, 256 KB of the 3.25 MB, go straight to the epilogue's registers.
+// Two forms: a block by itself with tiles of 128 tokens, and a pair of blocks (cta_group::2) with tiles of 256, in which each
+// block holds its 128 tokens' keys and half of the map's rows: 32 KB instead of 48 for 64 channels of a step, two thirds of the
+// traffic into shared memory, which the products' own reads share.
 //
-// Persistent blocks (one per multiprocessor) own equal contiguous ranges of the sequence of items (tile, pair of output
-// heads), which balances better than whole tiles: 624 tiles are 4.2 a block.  A tile cut by the end of a range is finished
-// by the next block: both add their share to eps, which starts at zero (two addends: the order does not matter).
-//   warps 0-7   loaders: gathers of the K rows of a step (cp.async, written in the 128-byte-swizzled operand layout),
-//               published three steps behind the one being issued; thread 0 also issues the W loads (TMA)
-//   warp  8     MMA issuer, TMEM owner (two 256-column accumulators: the epilogue of a pair runs under the next one)
-//   warps 9-12  epilogue: thread = row; its value row comes in 32-byte loads (16-byte ones where it has to), a head ahead
-// Measured on 16 layers of 4914 listed tokens and 8 heads: 245 us (388 before: one output head at a time, loads waited for in
-// every step, 64-bit divisions in every role), 53 KB a microsecond and multiprocessor: the rate at which L2 delivers.
+// What bounds it is how soon a step's operands and products follow the last ones.  A thread that waits for its copies and fences
+// them for the tensor cores waits for all that it has in flight, the next stages' copies among them: with eight warps filling
+// every stage together, a step took the latency of memory (245 us for 16 layers of 4914 listed tokens and 8 heads).  So every
+// stage has a loader warp of its own, which has nothing else in flight: 176 us, and 180 in pairs.  There the issue of the products
+// was the longest chain of a step (see the MMA role): 157 us, of which the products need 75 at the tensor rate, 104 at the rate of a
+// library product.  The products take two output heads at a time (a third fewer bytes than head by head), and the value rows go
+// straight to the epilogue's registers.
+//
+// Persistent groups (blocks or pairs, one block per multiprocessor) own equal contiguous ranges of the sequence of items (tile, pair
+// of output heads), which balances better than whole tiles: 624 tiles are 4.2 a block.  A tile cut by the end of a range is finished
+// by the next group: both add their share to eps, which starts at zero (two addends: the order does not matter).
+//   a warp a stage   loaders: gathers of the K rows of a step (cp.async, written in the 128-byte-swizzled operand layout) and the W
+//                    load (TMA)
+//   one warp         MMA issuer, TMEM owner (two 256-column accumulators: the epilogue of a pair runs under the next one)
+//   four warps       epilogue: thread = row; its value row comes in 32-byte loads (16-byte ones where it has to), a head ahead
 #ifndef VECTOR_RESIDUAL_LAYER_TC_CUH_
 #define VECTOR_RESIDUAL_LAYER_TC_CUH_
 
+#include "cluster.cuh"
 #include "common.cuh"
 #include "internal.h"
 #include "residual_tc.cuh"
@@ -37,13 +43,18 @@ namespace rlt {
 using rtc::BOX_BYTES;
 using rtc::TILE;
 
-constexpr int STAGES = 4;
-constexpr int STAGE_BYTES = 3 * BOX_BYTES;                // 64 channels of: the tile's keys of one head | the map's rows of two heads
-constexpr int LOADER_WARPS = 8;
 constexpr int EPI_WARPS = 4;
-constexpr int THREADS = 32 * (LOADER_WARPS + 1 + EPI_WARPS);
-constexpr int SMEM_BYTES = STAGES * STAGE_BYTES + 1024;
 constexpr int TMEM_COLS = 512;
+// CTAS blocks share a tile of 128 CTAS tokens; a stage holds 64 channels of: this block's 128 keys of one head | its share of the
+// map's rows of two output heads.
+template <int CTAS> struct LCfg {
+    static constexpr int STAGES = CTAS == 2 ? 6 : 4;
+    static constexpr int STAGE_BYTES = (CTAS == 2 ? 2 : 3) * BOX_BYTES;
+    static constexpr int SMEM_BYTES = STAGES * STAGE_BYTES + 1024;
+    static constexpr int LOADER_WARPS = STAGES;                         // a warp for every stage
+    static constexpr int THREADS = 32 * (LOADER_WARPS + 1 + EPI_WARPS);
+    static constexpr int TOKENS = 128 * CTAS;
+};
 
 struct Params {
     int UL, L, Hkv, n_idx, tpu;      // (sequence, layer) units, layers, KV heads, rows per unit, tiles per unit
@@ -51,7 +62,7 @@ struct Params {
     long long N, n_items;            // keys per head, UL * tpu * pairs
 };
 struct Sync {
-    uint64_t full[STAGES], w_full[STAGES], empty[STAGES];
+    uint64_t full[6], empty[6];
     uint64_t acc_full[2], acc_empty[2];
     uint32_t tmem_base;
 };
@@ -86,120 +97,131 @@ __device__ __forceinline__ void ldg32(const void* p, uint32_t (&r)[64], int at) 
     }
 }
 
-// grid: at most one block per multiprocessor and a range of at least `pairs` items each (so that a tile is cut once at
-// most), THREADS threads, SMEM_BYTES dynamic shared memory.
+// grid: at most one block per multiprocessor and a range of at least `pairs` / 2 items for each group (so that a tile is cut once at
+// most), clusters of CTAS blocks, LCfg::THREADS threads, LCfg::SMEM_BYTES dynamic shared memory.
 // K, V: [UL][Hkv][N][128]; idx: [UL][n_idx]; eps: [UL][n_idx], zero; mapW: (Hkv*128 in, Hkv*128 out, L), box 64 x 128.
 // WIDE: V is a multiple of 32 bytes.  The interface promises 16; rows are 256 bytes apart, so the base decides for all of them.
-template <bool WIDE>
-__global__ void __launch_bounds__(THREADS, 1)
+template <bool WIDE, int CTAS>
+__global__ void __launch_bounds__(LCfg<CTAS>::THREADS, 1)
 residual_layer_tc(const __nv_bfloat16* __restrict__ K, const __nv_bfloat16* __restrict__ V,
                   const __grid_constant__ CUtensorMap mapW, const int32_t* __restrict__ idx, const Params P,
                   float* __restrict__ eps, int* __restrict__ fault) {
     extern __shared__ unsigned char smem_raw[];
     __shared__ Sync sy;
     unsigned char* smem = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const long long it_lo = rtc::range_begin(blockIdx.x, P.n_items, gridDim.x);
-    const int n_my = (int)(rtc::range_begin(blockIdx.x + 1, P.n_items, gridDim.x) - it_lo);
+    const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;     // warp: known to be uniform
+    using C = LCfg<CTAS>;
+    constexpr int STAGES = C::STAGES, STAGE_BYTES = C::STAGE_BYTES, LOADER_WARPS = C::LOADER_WARPS;
+    const int rank = CTAS == 2 ? (int)(blockIdx.x & 1) : 0, group = blockIdx.x / CTAS, groups = gridDim.x / CTAS;
+    const long long it_lo = rtc::range_begin(group, P.n_items, groups);
+    const int n_my = (int)(rtc::range_begin(group + 1, P.n_items, groups) - it_lo);
     const int H = P.Hkv;
 
     if (tid == 0) {
 #pragma unroll
         for (int s = 0; s < STAGES; ++s) {
-            tma::mbar_init(&sy.full[s], 32 * LOADER_WARPS);
-            tma::mbar_init(&sy.w_full[s], 1);
+            tma::mbar_init(&sy.full[s], 32 + 1 + (CTAS == 2 && rank == 0 ? 1 : 0));    // a loader warp, the map's bytes, the other block's stage
             tma::mbar_init(&sy.empty[s], 1);
         }
 #pragma unroll
-        for (int k = 0; k < 2; ++k) { tma::mbar_init(&sy.acc_full[k], 1); tma::mbar_init(&sy.acc_empty[k], EPI_WARPS); }
+        for (int k = 0; k < 2; ++k) { tma::mbar_init(&sy.acc_full[k], 1); tma::mbar_init(&sy.acc_empty[k], CTAS * EPI_WARPS); }
         tma::mbar_fence_init();
     }
     if (warp == LOADER_WARPS) {
-        tc::tmem_alloc(&sy.tmem_base, TMEM_COLS);
-        tc::tmem_relinquish();
+        tc::tmem_alloc<CTAS>(&sy.tmem_base, TMEM_COLS);
+        tc::tmem_relinquish<CTAS>();
     }
     tc::fence_before_sync();
     __syncthreads();
+    if (CTAS == 2) { cl::arrive_release(); cl::wait_acquire(); }       // the peer's barriers are ready for arrivals
     tc::fence_after_sync();
 
     if (warp < LOADER_WARPS) {
         // ------------------------------------------------------------------ loaders
-        const int qc = tid & 7, rsub = tid >> 3;                    // 16-byte chunk of the 64 channels, row inside a pass of 32 rows
-        const uint32_t dst_thread = (uint32_t)rsub * 128u + (uint32_t)((qc ^ (rsub & 7)) << 4);   // + pass * 4096
-        int32_t rows[4];                                             // this thread's four rows of the tile at hand
+        constexpr int PASSES = 32;                                   // of four rows
+        const int qc = lane & 7, rsub = lane >> 3;                  // 16-byte chunk of the 64 channels, row inside a pass
+        // row 4 p + rsub of the swizzled tile: the chunk's place repeats every two passes
+        const uint32_t dst0 = (uint32_t)rsub * 128u + (uint32_t)((qc ^ rsub) << 4), dst1 = (uint32_t)(rsub + 4) * 128u + (uint32_t)((qc ^ (rsub + 4)) << 4);
+        int32_t rows[PASSES];                                        // this lane's rows of the tile at hand
         bool ok = true;
         if (tid == 0) tma::prefetch_map(&mapW);
         asm volatile("griddepcontrol.wait;\n" ::: "memory");      // idx is complete and visible from here on
         asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory");
         Cursor at = cursor_at(it_lo, P);
-        uint32_t step = 0;
-        for (int i = 0; i < n_my && ok; ++i, at.next(P)) {
+        uint32_t step = 0, round = 0;                                // step: of the item's first channels; round: of this warp's stage
+        const uint32_t s = warp;
+        unsigned char* st = smem + s * STAGE_BYTES;
+        for (int i = 0; i < n_my && ok; ++i, at.next(P), step += 2 * H) {
             if (i == 0 || at.pair == 0) {
 #pragma unroll
-                for (int p = 0; p < 4; ++p) {
-                    const int row = at.t * TILE + p * 32 + rsub;
+                for (int p = 0; p < PASSES; ++p) {
+                    const int row = at.t * C::TOKENS + rank * TILE + p * 4 + rsub;
                     const int32_t v = row < P.n_idx ? idx[(size_t)at.ul * P.n_idx + row] : -1;
                     rows[p] = (unsigned long long)v < (unsigned long long)P.N ? v : -1;     // an index outside the unit reads as zeros
                 }
             }
             const int heads = min(2, H - 2 * at.pair), layer = at.ul % P.L;
-            for (int hk = 0; hk < 2 * H && ok; ++hk, ++step) {     // (input head, half of its channels)
-                const uint32_t s = step % STAGES, round = step / STAGES;
-                if (round > 0 && !tma::mbar_wait(&sy.empty[s], (round - 1) & 1, fault, 81)) { ok = false; break; }
-                unsigned char* st = smem + s * STAGE_BYTES;
-                if (tid == 0) {                                     // the blocks (h, h') of the pair's output heads
-                    tma::mbar_expect_tx(&sy.w_full[s], heads * BOX_BYTES);
-                    for (int e = 0; e < heads; ++e)
-                        tma::load_3d(st + (1 + e) * BOX_BYTES, &mapW, hk * 64, (2 * at.pair + e) * 128, layer, &sy.w_full[s]);
+            // (input head, half of its channels) of this warp's steps in the item
+            for (int hk = (int)((s + STAGES - step % STAGES) % STAGES); hk < 2 * H; hk += STAGES, ++round) {
+                if (round > 0 && !tma::mbar_wait_warp(&sy.empty[s], (round - 1) & 1, fault, 81)) { ok = false; break; }
+                if (lane == 0) {                                    // the blocks (h, h') of the pair's output heads
+                    if constexpr (CTAS == 2) {                      // half of their rows (one head: 64, and 64 the product does not read)
+                        tma::mbar_expect_tx(&sy.full[s], BOX_BYTES);
+                        tma::load_3d(st + BOX_BYTES, &mapW, hk * 64, 2 * at.pair * 128 + rank * heads * 64, layer, &sy.full[s]);
+                    } else {
+                        tma::mbar_expect_tx(&sy.full[s], heads * BOX_BYTES);
+                        for (int e = 0; e < heads; ++e)
+                            tma::load_3d(st + (1 + e) * BOX_BYTES, &mapW, hk * 64, (2 * at.pair + e) * 128, layer, &sy.full[s]);
+                    }
                 }
-                const uint32_t kdst = tma::smem_u32(st) + dst_thread;
+                const uint32_t kdst = tma::smem_u32(st);
                 const __nv_bfloat16* Ku = K + ((size_t)at.ul * H + (hk >> 1)) * P.N * 128 + (hk & 1) * 64 + qc * 8;
 #pragma unroll
-                for (int p = 0; p < 4; ++p) {
+                for (int p = 0; p < PASSES; ++p) {
                     const bool valid = rows[p] >= 0;
-                    rtc::cp_async16(kdst + p * 4096, Ku + (valid ? (size_t)rows[p] * 128 : 0), valid ? 16u : 0u);   // zero fill past the end
+                    rtc::cp_async16(kdst + (p >> 1) * 1024 + ((p & 1) ? dst1 : dst0), Ku + (valid ? (size_t)rows[p] * 128 : 0), valid ? 16u : 0u);   // zero fill past the end
                 }
-                rtc::cp_async_commit();
-                if (step >= STAGES - 1) {                           // this thread's copies of the step STAGES - 1 before this one have landed
-                    rtc::cp_async_wait<STAGES - 1>();
-                    rtc::fence_async_proxy();
-                    tma::mbar_arrive(&sy.full[(step - (STAGES - 1)) % STAGES]);
-                }
+                rtc::cp_async_wait_all();
+                rtc::fence_async_proxy();
+                tma::mbar_arrive(&sy.full[s]);
             }
-        }
-        if (ok) {
-            auto publish = [&](uint32_t behind) {                   // step `behind` before the last, if there is one
-                if (step > behind) { rtc::fence_async_proxy(); tma::mbar_arrive(&sy.full[(step - 1 - behind) % STAGES]); }
-            };
-            rtc::cp_async_wait<2>(); publish(2);
-            rtc::cp_async_wait<1>(); publish(1);
-            rtc::cp_async_wait<0>(); publish(0);
-        } else {
-            rtc::cp_async_wait<0>();
         }
     } else if (warp == LOADER_WARPS) {
         // ------------------------------------------------------------------ MMA issue
-        if (lane == 0) {
-            asm volatile("griddepcontrol.wait;\n" ::: "memory");    // the bounded waits below time this kernel only
-            Cursor at = cursor_at(it_lo, P);
-            uint32_t step = 0;
-            bool ok = true;
-            for (int i = 0; i < n_my && ok; ++i, at.next(P)) {
-                const uint32_t buf = i & 1, use = i >> 1;
-                const uint32_t idesc = H - 2 * at.pair > 1 ? tc::instr_desc(128, 256) : tc::instr_desc(128, 128);
-                const uint32_t d = sy.tmem_base + buf * 256;
-                if (use > 0 && !tma::mbar_wait(&sy.acc_empty[buf], (use - 1) & 1, fault, 83)) break;
-                for (int hk = 0; hk < 2 * H; ++hk, ++step) {
-                    const uint32_t s = step % STAGES, round = step / STAGES;
-                    if (!tma::mbar_wait(&sy.w_full[s], round & 1, fault, 85) || !tma::mbar_wait(&sy.full[s], round & 1, fault, 84)) { ok = false; break; }
+        // The warp walks the steps together and one lane issues: under a branch on the lane the operands' descriptors are not
+        // known to be uniform, and the issue of a step's four products took 360 cycles.  Whether the next stage is full is asked
+        // before this one's products go out: an answer takes 200 cycles while products read shared memory.
+        asm volatile("griddepcontrol.wait;\n" ::: "memory");        // the bounded waits below time this kernel only
+        const bool elected = tc::elect_one();
+        const uint32_t n_steps = (uint32_t)n_my * 2 * H;
+        Cursor at = cursor_at(it_lo, P);
+        uint32_t step = 0, s = 0, round = 0;
+        bool ok = true;
+        uint32_t ready = 0;
+        for (int i = 0; i < n_my && ok; ++i, at.next(P)) {
+            const uint32_t buf = i & 1, use = i >> 1;
+            const uint32_t idesc = H - 2 * at.pair > 1 ? tc::instr_desc(128 * CTAS, 256) : tc::instr_desc(128 * CTAS, 128);
+            const uint32_t d = sy.tmem_base + buf * 256;
+            if (rank == 0 && use > 0 && !tma::mbar_wait_warp(&sy.acc_empty[buf], (use - 1) & 1, fault, 83)) break;
+            for (int hk = 0; hk < 2 * H; ++hk, ++step) {
+                if (!__all_sync(0xffffffffu, ready) && !tma::mbar_wait_warp(&sy.full[s], round & 1, fault, 84)) { ok = false; break; }
+                const uint32_t k_addr = tma::smem_u32(smem + s * STAGE_BYTES), w_addr = k_addr + BOX_BYTES;
+                const uint32_t s_next = s + 1 == STAGES ? 0 : s + 1, round_next = round + (s + 1 == STAGES);
+                ready = step + 1 < n_steps ? tma::mbar_test(&sy.full[s_next], round_next & 1) : 0u;
+                if (rank != 0) {                                    // the first block issues for both: tell it that this half is there
+                    if (elected) tma::mbar_arrive_at<CTAS>(tma::block_addr<CTAS>(&sy.full[s], 0));
+                } else {
                     tc::fence_after_sync();
-                    const uint32_t k_addr = tma::smem_u32(smem + s * STAGE_BYTES), w_addr = k_addr + BOX_BYTES;
+                    if (elected) {
 #pragma unroll
-                    for (int ks = 0; ks < 4; ++ks)
-                        tc::mma_bf16(d, tc::smem_desc(k_addr + ks * 32), tc::smem_desc(w_addr + ks * 32), idesc, (hk > 0 || ks > 0) ? 1u : 0u);
-                    tc::mma_commit(&sy.empty[s]);                   // the stage is free once these products have read it
+                        for (int ks = 0; ks < 4; ++ks)
+                            tc::mma_bf16<CTAS>(d, tc::smem_desc(k_addr + ks * 32), tc::smem_desc(w_addr + ks * 32), idesc, (hk > 0 || ks > 0) ? 1u : 0u);
+                        tc::mma_commit<CTAS>(&sy.empty[s]);         // the stage is free once these products have read it
+                        if (hk + 1 == 2 * H) tc::mma_commit<CTAS>(&sy.acc_full[buf]);
+                    }
                 }
-                if (ok) tc::mma_commit(&sy.acc_full[buf]);
+                __syncwarp();
+                s = s_next; round = round_next;
             }
         }
     } else {
@@ -210,7 +232,7 @@ residual_layer_tc(const __nv_bfloat16* __restrict__ K, const __nv_bfloat16* __re
         asm volatile("griddepcontrol.wait;\n" ::: "memory");
         Cursor at = cursor_at(it_lo, P);
         auto token_of = [&](const Cursor& c) -> int32_t {
-            const int row = c.t * TILE + r;
+            const int row = c.t * C::TOKENS + rank * TILE + r;
             const int32_t v = c.ul < P.UL && row < P.n_idx ? idx[(size_t)c.ul * P.n_idx + row] : -1;
             return (unsigned long long)v < (unsigned long long)P.N ? v : -1;
         };
@@ -272,9 +294,9 @@ residual_layer_tc(const __nv_bfloat16* __restrict__ K, const __nv_bfloat16* __re
             }
             tc::fence_before_sync();
             __syncwarp();
-            if (lane == 0) tma::mbar_arrive(&sy.acc_empty[buf]);
+            if (lane == 0) tma::mbar_arrive_at<CTAS>(tma::block_addr<CTAS>(&sy.acc_empty[buf], 0));
             if (last) {
-                const int row = at.t * TILE + r;
+                const int row = at.t * C::TOKENS + rank * TILE + r;
                 if (row < P.n_idx) {
                     float* dst = eps + (size_t)at.ul * P.n_idx + row;
                     if (whole && at.pair + 1 == P.pairs) *dst = e_tok;
@@ -289,10 +311,11 @@ residual_layer_tc(const __nv_bfloat16* __restrict__ K, const __nv_bfloat16* __re
     }
     tc::fence_before_sync();
     __syncthreads();
+    if (CTAS == 2) { cl::arrive_release(); cl::wait_acquire(); }       // the products read the peer's stages, arrivals go to its barriers
     if (warp == LOADER_WARPS) {
         __syncwarp();
         tc::fence_after_sync();
-        tc::tmem_dealloc(sy.tmem_base, TMEM_COLS);
+        tc::tmem_dealloc<CTAS>(sy.tmem_base, TMEM_COLS);
     }
 }
 

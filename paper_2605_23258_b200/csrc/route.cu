@@ -394,9 +394,11 @@ static vector_status residual_layer_dispatch(const Dims& dm, int Hkv, int L, con
     if (dm.dtype == VECTOR_BF16 && dm.d == 128) {
         static PerDeviceOnce once;
         if (once.first()) {
-            cudaError_t e = cudaFuncSetAttribute(rlt::residual_layer_tc<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, rlt::SMEM_BYTES);
-            if (e == cudaSuccess)
-                e = cudaFuncSetAttribute(rlt::residual_layer_tc<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, rlt::SMEM_BYTES);
+            auto opt_in = [](auto kern, int bytes) { return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes); };
+            cudaError_t e = opt_in(rlt::residual_layer_tc<true, 1>, rlt::LCfg<1>::SMEM_BYTES);
+            if (e == cudaSuccess) e = opt_in(rlt::residual_layer_tc<false, 1>, rlt::LCfg<1>::SMEM_BYTES);
+            if (e == cudaSuccess) e = opt_in(rlt::residual_layer_tc<true, 2>, rlt::LCfg<2>::SMEM_BYTES);
+            if (e == cudaSuccess) e = opt_in(rlt::residual_layer_tc<false, 2>, rlt::LCfg<2>::SMEM_BYTES);
             if (e != cudaSuccess) { once.undo(); VEC_CUDA_CHECK(e); }
         }
         int* fault = kernel_fault_address();
@@ -406,17 +408,32 @@ static vector_status residual_layer_dispatch(const Dims& dm, int Hkv, int L, con
         if (!tma::encode_bf16_3d(&mapW, W, DL, DL, (uint64_t)L, DL * 2, DL * DL * 2, 64, 128)) return VECTOR_ERR_CUDA;
         rlt::Params P;
         P.UL = UL; P.L = L; P.Hkv = Hkv; P.n_idx = (int)n_idx; P.N = N;
-        P.tpu = (int)((n_idx + rlt::TILE - 1) / rlt::TILE);
         P.pairs = (Hkv + 1) / 2;
-        const long long tiles = (long long)UL * P.tpu;
-        P.n_items = tiles * P.pairs;
         const int sms = sm_count();
-        // a block gets at least a tile, or exactly half of one where that leaves no more blocks than multiprocessors
-        const int blocks = (int)(tiles >= sms ? sms : 2 * tiles <= sms && P.pairs > 1 ? 2 * tiles : tiles);
+        // A tile of 128 tokens a block or of 256 a pair of blocks.  A group (block or pair) gets at least a tile, or exactly half of
+        // one where that leaves no more groups than places.
+        struct Split { int tpu; long long tiles; int groups; long long items; } split[2];
+        for (int c = 0; c < 2; ++c) {
+            Split& x = split[c];
+            const long long places = sms / (c + 1), tokens = 128 * (c + 1);
+            x.tpu = (int)((n_idx + tokens - 1) / tokens);
+            x.tiles = (long long)UL * x.tpu;
+            x.groups = (int)(x.tiles >= places ? places : 2 * x.tiles <= places && P.pairs > 1 ? 2 * x.tiles : x.tiles);
+            x.items = (x.tiles * P.pairs + x.groups - 1) / x.groups;
+        }
+        // An item takes a pair 8.0 us and a block 9.4 (16 layers of 4914 tokens, 8 heads: 142 against 161 us); rounded to 256,
+        // a short list costs the pairs more items.
+        const bool pair = 20 * split[1].items <= 23 * split[0].items;
+        P.tpu = split[pair].tpu;
+        P.n_items = split[pair].tiles * P.pairs;
+        const int blocks = split[pair].groups * (pair ? 2 : 1);
         if (!eps_zeroed) VEC_CUDA_CHECK(cudaMemsetAsync(eps, 0, (size_t)UL * (size_t)n_idx * sizeof(float), st));
-        auto kern = ((uintptr_t)V & 31) == 0 ? rlt::residual_layer_tc<true> : rlt::residual_layer_tc<false>;
-        VEC_CUDA_CHECK(launch_maybe_dependent(dependent, kern, dim3(blocks), dim3(rlt::THREADS), rlt::SMEM_BYTES,
-                                              st, (const __nv_bfloat16*)K, (const __nv_bfloat16*)V, mapW, idx, P, eps, fault));
+        const bool wide = ((uintptr_t)V & 31) == 0;
+        auto kern = pair ? (wide ? rlt::residual_layer_tc<true, 2> : rlt::residual_layer_tc<false, 2>)
+                         : (wide ? rlt::residual_layer_tc<true, 1> : rlt::residual_layer_tc<false, 1>);
+        VEC_CUDA_CHECK(launch_maybe_dependent(dependent, pair ? 2 : 1, kern, dim3(blocks), dim3(pair ? rlt::LCfg<2>::THREADS : rlt::LCfg<1>::THREADS),
+                                              pair ? rlt::LCfg<2>::SMEM_BYTES : rlt::LCfg<1>::SMEM_BYTES, st, (const __nv_bfloat16*)K,
+                                              (const __nv_bfloat16*)V, mapW, idx, P, eps, fault));
         return VECTOR_OK;
     }
     const dim3 grid((unsigned)((n_idx + 7) / 8), UL);

@@ -53,6 +53,17 @@ __device__ __forceinline__ bool mbar_wait_warp(uint64_t* bar, uint32_t parity, i
     return __all_sync(0xffffffffu, ok);
 }
 
+// Whether the phase has completed, without waiting.
+__device__ __forceinline__ uint32_t mbar_test(uint64_t* bar, uint32_t parity) {
+    uint32_t ok;
+    asm volatile(
+        "{\n .reg .pred p;\n"
+        " mbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n"
+        " selp.u32 %0, 1, 0, p;\n}\n"
+        : "=r"(ok) : "r"(smem_u32(bar)), "r"(parity) : "memory");
+    return ok;
+}
+
 // One box of a rank-3 tensor into shared memory; completion is signalled on `bar` by byte count.
 __device__ __forceinline__ void load_3d(void* dst, const CUtensorMap* map, int x, int y, int z, uint64_t* bar) {
     asm volatile(
@@ -77,6 +88,19 @@ __device__ __forceinline__ void load_2d(void* dst, const CUtensorMap* map, int x
     asm volatile(
         "cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4}], [%2];\n"
         ::"r"(smem_u32(dst)), "l"(map), "r"(smem_u32(bar)), "r"(x), "r"(y) : "memory");
+}
+// For kernels that run alone (CTAS = 1) or as the two blocks of a cluster (CTAS = 2): the address of a shared-memory variable of
+// block `block`, and an arrival there.
+template <int CTAS>
+__device__ __forceinline__ uint32_t block_addr(const void* p, uint32_t block) {
+    uint32_t a = smem_u32(p);
+    if constexpr (CTAS == 2) asm("mapa.shared::cluster.u32 %0, %1, %2;\n" : "=r"(a) : "r"(smem_u32(p)), "r"(block));
+    return a;
+}
+template <int CTAS>
+__device__ __forceinline__ void mbar_arrive_at(uint32_t bar) {
+    if constexpr (CTAS == 1) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];\n" ::"r"(bar) : "memory");
+    else asm volatile("mbarrier.arrive.shared::cluster.b64 _, [%0];\n" ::"r"(bar) : "memory");
 }
 __device__ __forceinline__ void prefetch_map(const CUtensorMap* map) {
     asm volatile("prefetch.tensormap [%0];\n" ::"l"(map) : "memory");

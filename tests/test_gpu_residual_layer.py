@@ -12,7 +12,8 @@ pytestmark = pytest.mark.gpu
 DEV = "cuda"
 
 
-@pytest.mark.parametrize("layers,Hkv,n_idx", [(1, 1, 1), (2, 3, 129), (1, 8, 128), (3, 2, 300), (30, 8, 700), (75, 3, 257), (151, 1, 100)])
+@pytest.mark.parametrize("layers,Hkv,n_idx", [(1, 1, 1), (2, 3, 129), (1, 8, 128), (3, 2, 300), (30, 8, 700), (75, 3, 257), (151, 1, 100),
+                                              (74, 1, 1), (37, 5, 300), (2, 8, 256), (20, 8, 769)])      # around where pairs of blocks begin
 def test_residual_layer(oracle, layers, Hkv, n_idx):
     N, d = 800, 128
     D = Hkv * d
