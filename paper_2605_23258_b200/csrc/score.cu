@@ -300,7 +300,7 @@ static vector_status launch_score(const Dims& dm, const void* Q_, const void* K_
 template <int D>
 static vector_status launch_score_tc(const Dims& dm, const void* Q, const void* K, int64_t N, float* scores,
                                      float* raw_out, char* ws, cudaStream_t st) {
-    constexpr int SMEM = stc::Cfg<D>::SMEM_BYTES;
+    constexpr int SMEM = stc::Cfg<D>::SMEM_BYTES, SMEM_POOLED = SMEM + 2 * stc::POOLED_KEYS * 4;
     const ScoreTcPlan pl = score_tc_plan(dm.U, dm.R, N);
     float2* partial = (float2*)ws;
     ws += align256((size_t)dm.U * 2 * pl.n_chunks * dm.R * 2 * sizeof(float));
@@ -309,11 +309,15 @@ static vector_status launch_score_tc(const Dims& dm, const void* Q, const void* 
     float* raw_part = (float*)ws;
     static PerDeviceOnce once;
     if (once.first()) {
-        cudaError_t e = cudaFuncSetAttribute(stc::score_pass1_tc<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM);
-        if (e == cudaSuccess)
-            e = cudaFuncSetAttribute(stc::score_pass2_tc<D, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM);
-        if (e == cudaSuccess)
-            e = cudaFuncSetAttribute(stc::score_pass2_tc<D, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM);
+        auto opt_in = [](auto kern, int bytes) { return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes); };
+        cudaError_t e = opt_in(stc::score_pass1_tc<D, 1>, SMEM);
+        if (e == cudaSuccess) e = opt_in(stc::score_pass1_tc<D, 2>, SMEM);
+        if (e == cudaSuccess) e = opt_in(stc::score_pass2_tc<D, true, 1, true>, SMEM_POOLED);
+        if (e == cudaSuccess) e = opt_in(stc::score_pass2_tc<D, true, 2, true>, SMEM_POOLED);
+        if (e == cudaSuccess) e = opt_in(stc::score_pass2_tc<D, true, 1, false>, SMEM);
+        if (e == cudaSuccess) e = opt_in(stc::score_pass2_tc<D, true, 2, false>, SMEM);
+        if (e == cudaSuccess) e = opt_in(stc::score_pass2_tc<D, false, 1, false>, SMEM);
+        if (e == cudaSuccess) e = opt_in(stc::score_pass2_tc<D, false, 2, false>, SMEM);
         if (e != cudaSuccess) { once.undo(); VEC_CUDA_CHECK(e); }
     }
     int* fault = kernel_fault_address();
@@ -324,25 +328,46 @@ static vector_status launch_score_tc(const Dims& dm, const void* Q, const void* 
         return VECTOR_ERR_CUDA;
     stc::Params P;
     P.U = dm.U; P.R = dm.R; P.RG = pl.RG; P.w = dm.w; P.N = N;
-    P.nt = pl.nt; P.tpc = pl.tpc; P.n_chunks = pl.n_chunks; P.n_items = pl.n_items;
+    P.tpc = pl.tpc; P.step = pl.tpc * stc::KT; P.lead = 0; P.n_chunks = P.lse_chunks = pl.n_chunks; P.n_items = pl.n_items;
     P.c = dm.scale * 1.4426950408889634f;
     const int sms = sm_count();
     const int blocks = pl.n_items < sms ? pl.n_items : sms;
-    stc::score_pass1_tc<D><<<blocks, stc::THREADS, SMEM, st>>>(mapQ, mapK, P, partial, fault);
+    const bool one = dm.R <= 128;
+    auto pass1 = one ? stc::score_pass1_tc<D, 1> : stc::score_pass1_tc<D, 2>;
+    pass1<<<blocks, stc::THREADS, SMEM, st>>>(mapQ, mapK, P, partial, fault);
     VEC_LAUNCH_CHECK();
     // A block has one or two items: the passes are short, so the second forms the normalisers itself and each kernel after
     // the first is a programmatic dependent of the one before it.  Long passes are launched the ordinary way: as a
     // dependent, pass 2 has its blocks placed as multiprocessors fall free and no longer side by side, where the row
     // groups of a key chunk share what they fetch (640 units of 1024 rows, 131072 keys: 53.7 ms against 52.9).
     const bool few = pl.n_items <= 2 * blocks;
+    if (few && pl.RG == 1) {
+        // Pooling in the second pass: its chunks overlap, so they have a tile more where their number would go up.
+        const int r = dm.pool_kernel / 2;
+        stc::Params P2 = P;
+        P2.lead = r;
+        for (P2.tpc = pl.tpc; P2.tpc <= pl.tpc + 1 && P2.tpc * stc::KT <= stc::POOLED_KEYS; ++P2.tpc) {
+            P2.step = P2.tpc * stc::KT - 2 * r;
+            P2.n_chunks = (int)((N + P2.step - 1) / P2.step);
+            const long long items = (long long)dm.U * P2.n_chunks;
+            if (items > (long long)sms * ((pl.n_items + blocks - 1) / blocks)) continue;       // no more rounds than without
+            P2.n_items = (int)items;
+            auto pass2 = one ? stc::score_pass2_tc<D, true, 1, true> : stc::score_pass2_tc<D, true, 2, true>;
+            VEC_CUDA_CHECK(launch_maybe_dependent(true, pass2, dim3(items < sms ? (unsigned)items : sms), dim3(stc::THREADS), SMEM_POOLED, st, mapQ,
+                                                  mapK, P2, partial, lse2, raw_part, raw_out, scores, fault));
+            return VECTOR_OK;
+        }
+    }
+    auto pass2 = one ? (few ? stc::score_pass2_tc<D, true, 1, false> : stc::score_pass2_tc<D, false, 1, false>)
+                     : (few ? stc::score_pass2_tc<D, true, 2, false> : stc::score_pass2_tc<D, false, 2, false>);
     if (!few)
         VEC_CUDA_CHECK(launch_maybe_dependent(false, stc::score_lse2_rows, dim3((dm.R + 127) / 128, dm.U), dim3(256), 0, st, partial, dm.R,
                                               pl.n_chunks, lse2));
-    VEC_CUDA_CHECK(launch_maybe_dependent(few, few ? stc::score_pass2_tc<D, true> : stc::score_pass2_tc<D, false>, dim3(blocks),
-                                          dim3(stc::THREADS), SMEM, st, mapQ, mapK, P, partial, lse2, raw_part, fault));
+    VEC_CUDA_CHECK(launch_maybe_dependent(few, pass2, dim3(blocks), dim3(stc::THREADS), SMEM, st, mapQ, mapK, P, partial, lse2, raw_part,
+                                          raw_out, scores, fault));
     const dim3 gp((unsigned)((N + stc::POOL_TILE - 1) / stc::POOL_TILE), dm.U);
     VEC_CUDA_CHECK(launch_maybe_dependent(few, (N & 3) == 0 ? stc::score_pool_parts_v4 : stc::score_pool_parts, gp, dim3(256), 0, st,
-                                          raw_part, 2 * pl.RG, N, dm.w, dm.pool_kernel / 2, raw_out, scores));
+                                          raw_part, (dm.R + 127) / 128, N, dm.w, dm.pool_kernel / 2, raw_out, scores));
     return VECTOR_OK;
 }
 

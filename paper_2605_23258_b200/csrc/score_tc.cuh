@@ -21,8 +21,10 @@
 //              refilled the other keeps the exponential unit busy; each thread owns one TMEM lane
 //   warp  16   producer: TMA loads of the Q row group (once per item) and of the
 //              K tiles into a ring of 4 or 8 stages (128-byte swizzle, zero fill past the end)
-//   warp  17   MMA issuer (one thread) and owner of the TMEM allocation
+//   warp  17   MMA issuer and owner of the TMEM allocation
 // All hand-offs are mbarriers; every wait is bounded and records a fault code.
+// Units of at most 128 rows (NB = 1) give every warpgroup whole tiles: 280 units of 96 rows over 78299 keys 2.60 -> 1.88 ms with
+// their pooling.  Few units are pooled by the second pass itself: 8 units of 256 rows over 8192 keys 27.4 -> 23.3 us.
 // Measured at 64 channels, 128 units of 4 heads x 64 rows over 15013 keys: 0.298 ms (6.32 ms on CUDA cores).
 #ifndef VECTOR_SCORE_TC_CUH_
 #define VECTOR_SCORE_TC_CUH_
@@ -55,20 +57,22 @@ constexpr int TMEM_COLS = 512;
 struct Params {
     int U, R, RG, w;            // units, rows per unit, row groups per unit, window
     long long N;                // keys per unit
-    int nt, tpc, n_chunks;      // key tiles per unit, tiles per chunk, chunks per unit
+    int tpc, n_chunks;          // key tiles per chunk, chunks per unit
+    int step, lead;             // chunk c begins at key c * step - lead
     int n_items;                // U * n_chunks * RG
+    int lse_chunks;             // second pass: chunks of the first one
     float c;                    // logit scale * log2(e)
 };
 
-struct Item { int u, chunk, rg, t0, t1; };
+struct Item { int u, chunk, rg, key0, tiles; };      // key0 may be negative: keys before the first read as zeros
 __device__ __forceinline__ Item decode_item(int it, const Params& P) {
     Item i;
     i.rg = it % P.RG;
     const int uc = it / P.RG;
     i.chunk = uc % P.n_chunks;
     i.u = uc / P.n_chunks;
-    i.t0 = i.chunk * P.tpc;
-    i.t1 = min(P.nt, i.t0 + P.tpc);
+    i.key0 = i.chunk * P.step - P.lead;
+    i.tiles = min((int)((P.N - i.key0 + KT - 1) / KT), P.tpc);
     return i;
 }
 
@@ -83,6 +87,9 @@ struct Sync {
 // Producer and MMA roles are the same in both passes up to which operand is A and the tile shape.
 //   PASS 1: per key tile two MMAs  D[buf = 2 (tile & 1) + rb] (128 x 128) = Q[rb] K^T
 //   PASS 2: per key tile one MMA   D[buf = tile & 1]         (128 x 256) = K Q^T
+// NB = 1 is for units of at most 128 rows, which have no second block of 128 rows in a row group: a tile has one accumulator of
+// 128 columns (pass 2: of the rows rounded up to 16) and goes to one of four warpgroups, where both groups' second warpgroups
+// would idle and half the products be padding.
 template <int D>
 __device__ __forceinline__ void producer_role(const CUtensorMap* mapQ, const CUtensorMap* mapK, const Params& P,
                                               Sync& sy, unsigned char* Qs, unsigned char* Ks, int* fault) {
@@ -107,16 +114,16 @@ __device__ __forceinline__ void producer_role(const CUtensorMap* mapQ, const CUt
         if (icount == NQ) asm volatile("griddepcontrol.wait;\n" ::: "memory");      // as in the MMA role
         // With one row group held, its successor has to wait for the item's last product: the next keys go first
         // (they waited behind it: 4 to 5 thousand cycles an item, of 22 thousand at 15 tiles of 64 channels).
-        const int q_at = min(im.t0 + STAGES, im.t1) - 1;
+        const int q_at = min(STAGES, im.tiles) - 1;
         if (NQ > 1 && !load_q(im)) return;
-        for (int t = im.t0; t < im.t1; ++t, ++kcount) {
+        for (int t = 0; t < im.tiles; ++t, ++kcount) {
             const uint32_t s = kcount % STAGES, round = kcount / STAGES;
             if (kcount == STAGES) asm volatile("griddepcontrol.wait;\n" ::: "memory");
             if (round > 0 && !tma::mbar_wait(&sy.k_empty[s], (round - 1) & 1, fault, 12)) return;
             tma::mbar_expect_tx(&sy.k_full[s], K_STAGE_BYTES);
 #pragma unroll
             for (int kh = 0; kh < HALVES; ++kh)
-                tma::load_3d(Ks + s * K_STAGE_BYTES + kh * BOX_BYTES, mapK, kh * 64, t * KT, im.u, &sy.k_full[s]);
+                tma::load_3d(Ks + s * K_STAGE_BYTES + kh * BOX_BYTES, mapK, kh * 64, im.key0 + t * KT, im.u, &sy.k_full[s]);
             if (NQ == 1 && t == q_at && !load_q(im)) return;
         }
     }
@@ -126,53 +133,55 @@ __device__ __forceinline__ void producer_role(const CUtensorMap* mapQ, const CUt
     asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory");
 }
 
-template <int PASS, int D>
+// First pass: the warp walks the tiles together and one lane issues.  Under a branch on the lane the operands' descriptors are not
+// known to be uniform, which costs some 75 cycles a product (27.2 -> 26.1 ms for 640 units of 1024 rows and 131072 keys).  Whether
+// the next keys are there is asked before this tile's products go out.  The second pass is called by one lane: with its products
+// in quicker succession the softmax warps, which read the rows' normalisers from the same shared memory, fall behind (23.8 -> 25.5 ms).
+template <int PASS, int D, int NB>
 __device__ __forceinline__ void mma_role(const Params& P, Sync& sy, unsigned char* Qs, unsigned char* Ks, int* fault) {
     constexpr int STAGES = Cfg<D>::STAGES, K_STAGE_BYTES = Cfg<D>::K_STAGE_BYTES, K_STEPS = D / 16, NQ = Cfg<D>::NQ;
     const uint32_t k_addr = tma::smem_u32(Ks);
     const uint32_t tmem = sy.tmem_base;
-    uint32_t kcount = 0, icount = 0;
+    constexpr bool WARP = PASS == 1;
+    const bool elected = WARP ? elect_one() : true;
+    auto wait = [&](uint64_t* bar, uint32_t parity, int code) { return WARP ? tma::mbar_wait_warp(bar, parity, fault, code) : tma::mbar_wait(bar, parity, fault, code); };
+    auto together = [&]() { if (WARP) __syncwarp(); };
+    uint32_t kcount = 0, icount = 0, k_ready = 0;
     // the softmax warps of the second pass start once the first has drained: do not spend bounded polls on its run time
     asm volatile("griddepcontrol.wait;\n" ::: "memory");
     for (int it = blockIdx.x; it < P.n_items; it += gridDim.x, ++icount) {
         const Item im = decode_item(it, P);
         const uint32_t qb = icount % NQ, q_addr = tma::smem_u32(Qs) + qb * Cfg<D>::Q_BYTES;
-        if (!tma::mbar_wait(&sy.q_full[qb], (icount / NQ) & 1, fault, 21)) return;
+        if (!wait(&sy.q_full[qb], (icount / NQ) & 1, 21)) return;
         fence_after_sync();
-        for (int t = im.t0; t < im.t1; ++t, ++kcount) {
+        for (int t = 0; t < im.tiles; ++t, ++kcount) {
             const uint32_t s = kcount % STAGES, round = kcount / STAGES;
-            if (!tma::mbar_wait(&sy.k_full[s], round & 1, fault, 22)) return;
+            if (!(WARP && __all_sync(0xffffffffu, k_ready)) && !wait(&sy.k_full[s], round & 1, 22)) return;
+            if (WARP) k_ready = t + 1 < im.tiles ? tma::mbar_test(&sy.k_full[(kcount + 1) % STAGES], ((kcount + 1) / STAGES) & 1) : 0u;
             fence_after_sync();
             const uint32_t ks_addr = k_addr + s * K_STAGE_BYTES;
-            if (PASS == 1) {
 #pragma unroll
-                for (int rb = 0; rb < 2; ++rb) {
-                    const uint32_t buf = (kcount & 1) * 2 + rb, use = kcount >> 1;
-                    if (use > 0 && !tma::mbar_wait(&sy.acc_empty[buf], (use - 1) & 1, fault, 23)) return;
-                    fence_after_sync();
+            for (int rb = 0; rb < (PASS == 1 ? NB : 1); ++rb) {
+                const uint32_t buf = NB == 1 ? kcount & 3 : PASS == 1 ? (kcount & 1) * 2 + rb : kcount & 1, use = NB == 1 ? kcount >> 2 : kcount >> 1;
+                if (use > 0 && !wait(&sy.acc_empty[buf], (use - 1) & 1, 22 + PASS)) return;
+                fence_after_sync();
+                if (elected) {
 #pragma unroll
                     for (int ks = 0; ks < K_STEPS; ++ks) {
                         const uint32_t kh = ks >> 2, ko = (ks & 3) * 32;
-                        mma_bf16(tmem + buf * 128, smem_desc(q_addr + kh * 2 * BOX_BYTES + rb * BOX_BYTES + ko),
-                                 smem_desc(ks_addr + kh * BOX_BYTES + ko), instr_desc(128, 128), ks > 0);
+                        const uint64_t kd = smem_desc(ks_addr + kh * BOX_BYTES + ko);
+                        const uint64_t qd = smem_desc(q_addr + kh * 2 * BOX_BYTES + rb * BOX_BYTES + ko);
+                        if (PASS == 1) mma_bf16(tmem + buf * 128, qd, kd, instr_desc(128, 128), ks > 0);
+                        else mma_bf16(tmem + buf * 128 * NB, kd, qd, NB == 1 ? instr_desc(128, (P.R + 15) & ~15) : instr_desc(128, 256), ks > 0);
                     }
                     mma_commit(&sy.acc_full[buf]);
+                    if (PASS == 2 || rb + 1 == NB) mma_commit(&sy.k_empty[s]);      // the stage is free once these products have read it
                 }
-            } else {
-                const uint32_t buf = kcount & 1, use = kcount >> 1;
-                if (use > 0 && !tma::mbar_wait(&sy.acc_empty[buf], (use - 1) & 1, fault, 24)) return;
-                fence_after_sync();
-#pragma unroll
-                for (int ks = 0; ks < K_STEPS; ++ks) {
-                    const uint32_t kh = ks >> 2, ko = (ks & 3) * 32;
-                    mma_bf16(tmem + buf * 256, smem_desc(ks_addr + kh * BOX_BYTES + ko),
-                             smem_desc(q_addr + kh * 2 * BOX_BYTES + ko), instr_desc(128, 256), ks > 0);
-                }
-                mma_commit(&sy.acc_full[buf]);
+                together();
             }
-            mma_commit(&sy.k_empty[s]);       // the stage is free once these MMAs have read it
         }
-        mma_commit(&sy.q_empty[qb]);
+        if (elected) mma_commit(&sy.q_empty[qb]);
+        together();
     }
 }
 
@@ -352,23 +361,26 @@ __device__ __forceinline__ void softmax_tile_pass1(uint32_t taddr, float c, long
 // Masked tiles: row j of the window (j0 = window index of the tile's first row, advancing cyclically
 // with period w) sees this key only if key - (N - w) <= j.
 // 16 columns at a time: the rows' lse, 16 registers, are then on their way before the accumulator's load is waited for.
-template <bool MASKED>
-__device__ __forceinline__ float softmax_tile_pass2(uint32_t taddr, float c, const float* nl_w, long long key_rel,
+// PIECES: 16-row pieces of the tile, 0: `pieces` of them.
+template <bool MASKED, int PIECES>
+__device__ __forceinline__ float softmax_tile_pass2(uint32_t taddr, float c, const float* nl_w, int pieces, long long key_rel,
                                                     int j0, int w, uint64_t& empty_bar, int lane) {
     uint32_t ra[16], rb[16];
     tmem_ld16(taddr, ra);
     uint64_t acc = pack2(0.f, 0.f);
     float sm = 0.f;
     int j = j0;
+    const int n_ch = PIECES ? PIECES : pieces;
 #pragma unroll
     for (int ch = 0; ch < 8; ++ch) {
+        if (!PIECES && ch >= n_ch) break;
         uint32_t (&cur)[16] = (ch & 1) ? rb : ra;
         uint32_t (&nxt)[16] = (ch & 1) ? ra : rb;
         float4 n[4];
 #pragma unroll
         for (int i = 0; i < 4; ++i) n[i] = reinterpret_cast<const float4*>(nl_w + ch * 16)[i];
         tmem_ld_wait16(cur);
-        if (ch < 7) {
+        if (ch + 1 < n_ch) {
             tmem_ld16(taddr + (ch + 1) * 16, nxt);
         } else {
             fence_before_sync();
@@ -395,48 +407,62 @@ __device__ __forceinline__ float softmax_tile_pass2(uint32_t taddr, float c, con
 // ---- pass 1 -----------------------------------------------------------------
 // partial[((u * n_chunks + chunk) * 2 + group) * R + row] = (reference, sum of exp2 against it) of the
 // row over the visible keys of the chunk's even (group 0) or odd (group 1) tiles, in units of log2 (logit * scale * log2 e).  grid: one block per SM.
-template <int D>
+// NB = 1: warpgroup v takes the tiles 4 i + v; those of one parity are added up in shared memory at the end of an item.
+template <int D, int NB>
 __global__ void __launch_bounds__(THREADS, 1)
 score_pass1_tc(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__ CUtensorMap mapK, const Params P,
                float2* __restrict__ partial, int* __restrict__ fault) {
     extern __shared__ unsigned char smem_raw[];
     __shared__ Sync sy;
+    __shared__ float2 upper[NB == 1 ? 4 : 1][128];                  // NB = 1: what the last two warpgroups found, two items in turn
     unsigned char* smem = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
     unsigned char* Qs = smem;
     unsigned char* Ks = smem + Cfg<D>::NQ * Cfg<D>::Q_BYTES;
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0), lane = threadIdx.x & 31;
     block_setup(sy, 4);
 
     if (warp == SOFTMAX_WARPS) {
         if (lane == 0) producer_role<D>(&mapQ, &mapK, P, sy, Qs, Ks, fault);
     } else if (warp == SOFTMAX_WARPS + 1) {
-        if (lane == 0) mma_role<1, D>(P, sy, Qs, Ks, fault);
+        mma_role<1, D, NB>(P, sy, Qs, Ks, fault);
     } else {
-        const int grp = warp >> 3, wg = (warp >> 2) & 1, quarter = warp & 3;
+        // NB = 2: tiles of parity grp, row block wg.  NB = 1: tiles tgrp mod 4; grp is their parity.
+        const int tgrp = warp >> 2, grp = NB == 2 ? warp >> 3 : tgrp & 1, wg = NB == 2 ? (warp >> 2) & 1 : 0, quarter = warp & 3;
         const uint32_t lane_addr = sy.tmem_base + ((uint32_t)(quarter * 32) << 16);
         const long long vis0 = P.N - P.w;               // keys below this index are visible to every row
-        uint32_t tcount = 0;
+        uint32_t tcount = 0, icount = 0;
         bool ok = true;
-        for (int it = blockIdx.x; it < P.n_items && ok; it += gridDim.x) {
+        for (int it = blockIdx.x; it < P.n_items && (NB == 1 || ok); it += gridDim.x, ++icount) {
             const Item im = decode_item(it, P);
             const int row = im.rg * RG_ROWS + wg * 128 + quarter * 32 + lane;
             const bool wg_active = im.rg * RG_ROWS + wg * 128 < P.R;
             const long long last_visible = vis0 + (row % P.w);
             float m = -INFINITY, l = 0.f;
-            for (int t = im.t0; t < im.t1; ++t, ++tcount) {
-                if ((int)(tcount & 1) != grp) continue;
-                const uint32_t buf = (tcount & 1) * 2 + wg, use = tcount >> 1;
-                if (!tma::mbar_wait_warp(&sy.acc_full[buf], use & 1, fault, 31)) { ok = false; break; }
+            for (int t = 0; t < im.tiles; ++t, ++tcount) {
+                if (NB == 2 ? (int)(tcount & 1) != grp : (int)(tcount & 3) != tgrp) continue;
+                const uint32_t buf = NB == 2 ? (tcount & 1) * 2 + wg : tcount & 3, use = NB == 2 ? tcount >> 1 : tcount >> 2;
+                if (!ok || !tma::mbar_wait_warp(&sy.acc_full[buf], use & 1, fault, 31)) { ok = false; break; }
                 fence_after_sync();
                 if (wg_active) {
                     const uint32_t taddr = lane_addr + buf * 128;
-                    const long long key0 = (long long)t * KT;
+                    const long long key0 = im.key0 + t * KT;
                     if (key0 + KT <= vis0) softmax_tile_pass1<false>(taddr, P.c, 0, 0, m, l, sy.acc_empty[buf], lane);
                     else softmax_tile_pass1<true>(taddr, P.c, key0, last_visible, m, l, sy.acc_empty[buf], lane);
                 } else {
                     __syncwarp();
                     if (lane == 0) tma::mbar_arrive(&sy.acc_empty[buf]);
                 }
+            }
+            if (NB == 1) {
+                float2 (&up)[128] = upper[NB == 1 ? 2 * (icount & 1) + grp : 0];
+                if (tgrp >= 2) up[quarter * 32 + lane] = make_float2(m, l);
+                // one barrier an item: whoever writes this half again, two items on, has seen every warp past this item
+                asm volatile("bar.sync 1, %0;\n" ::"n"(32 * SOFTMAX_WARPS) : "memory");
+                if (tgrp >= 2) continue;
+                const float2 o = up[quarter * 32 + lane];
+                const float M = fmaxf(m, o.x);
+                if (M > -INFINITY) l = l * ex2(m - M) + o.y * ex2(o.x - M);
+                m = M;
             }
             if (ok && row < P.R)
                 partial[(((size_t)im.u * P.n_chunks + im.chunk) * 2 + grp) * P.R + row] = make_float2(m, l);
@@ -483,17 +509,22 @@ score_lse2_rows(const float2* __restrict__ partial, int R, int n_chunks, float* 
     if ((threadIdx.x & 1) == 0) lse2[(size_t)u * R + row] = l;
 }
 
-// raw_part[(u * 2 RG + 2 rg + h) * N + key] = sum over rows [rg*256 + h*128, +128) of the softmax
-// probability of `key`; the parts are added up by the pooling kernel.  grid: one block per SM.
+// raw_part[(u * parts + 2 rg + h) * N + key] = sum over rows [rg*256 + h*128, +128) of the softmax
+// probability of `key`, parts = ceil(R / 128); the parts are added up by the pooling kernel.  grid: one block per SM.
 // INLINE_LSE, for blocks with few items: the rows' normalisers are formed from the chunk partials at the start of each
 // item, two threads a row, which saves a launch (one layer, 8 heads, 256 rows, 8192 keys: 26.5 us against 36.0 with a
 // kernel of its own, one block a unit).  With many items the stall at each item's start adds up, and score_lse2_rows
 // leaves them in lse2 beforehand.
-template <int D, bool INLINE_LSE>
+// POOLED, where blocks have few items and a unit one row group: a chunk's sums stay in shared memory, behind the K ring, and the
+// block pools them itself: a launch less, and the sums make no trip through memory.  Its chunks overlap by the pooling radius
+// r = P.lead on both sides.
+constexpr int POOLED_KEYS = 3072;                    // sums of a chunk, for every 128 rows, in 24 KB
+template <int D, bool INLINE_LSE, int NB, bool POOLED>
 __global__ void __launch_bounds__(THREADS, 1)
 score_pass2_tc(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__ CUtensorMap mapK, const Params P,
                const float2* __restrict__ partial, const float* __restrict__ lse2, float* __restrict__ raw_part,
-               int* __restrict__ fault) {
+               float* __restrict__ raw_out, float* __restrict__ score, int* __restrict__ fault) {
+    static_assert(INLINE_LSE || !POOLED, "only where blocks have few items");
     extern __shared__ unsigned char smem_raw[];
     __shared__ Sync sy;
     // -lse2 of the item's rows: INLINE_LSE, 256 rows, two items in turn; else a copy of its 128 rows for every warp
@@ -501,15 +532,16 @@ score_pass2_tc(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__
     unsigned char* smem = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
     unsigned char* Qs = smem;
     unsigned char* Ks = smem + Cfg<D>::NQ * Cfg<D>::Q_BYTES;
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    block_setup(sy, 8);
+    const int warp = __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0), lane = threadIdx.x & 31;
+    block_setup(sy, 4 * NB);
 
     if (warp == SOFTMAX_WARPS) {
         if (lane == 0) producer_role<D>(&mapQ, &mapK, P, sy, Qs, Ks, fault);
     } else if (warp == SOFTMAX_WARPS + 1) {
-        if (lane == 0) mma_role<2, D>(P, sy, Qs, Ks, fault);
+        if (lane == 0) mma_role<2, D, NB>(P, sy, Qs, Ks, fault);
     } else {
-        const int grp = warp >> 3, wg = (warp >> 2) & 1, quarter = warp & 3;
+        const int grp = NB == 2 ? warp >> 3 : warp >> 2, wg = NB == 2 ? (warp >> 2) & 1 : 0, quarter = warp & 3;      // as in pass 1
+        const int parts = (P.R + 127) / 128, pieces = (P.R + 15) / 16;
         const uint32_t lane_addr = sy.tmem_base + ((uint32_t)(quarter * 32) << 16);
         const int key_in_tile = quarter * 32 + lane;
         const long long vis0 = P.N - P.w;
@@ -524,11 +556,11 @@ score_pass2_tc(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__
             if constexpr (INLINE_LSE) {
                 float* nl_item = neg_lse[2 * (icount & 1)];
                 const int r = threadIdx.x >> 1, row = im.rg * RG_ROWS + r;
-                const float lse = row < P.R ? row_lse2(partial + (size_t)im.u * 2 * P.n_chunks * P.R + row, P.R, P.n_chunks) : INFINITY;
+                const float lse = row < P.R ? row_lse2(partial + (size_t)im.u * 2 * P.lse_chunks * P.R + row, P.R, P.lse_chunks) : INFINITY;
                 if ((threadIdx.x & 1) == 0) nl_item[r] = -lse;           // -inf: padding rows add 0
                 // one barrier an item: whoever writes this half again, two items on, has seen every warp past this item
                 asm volatile("bar.sync 1, %0;\n" ::"n"(32 * SOFTMAX_WARPS) : "memory");
-                if (!ok) continue;
+                if (!ok && !POOLED) continue;                          // POOLED: there are more barriers to meet
                 nl_w = nl_item + wg * 128;
             } else {
                 nl_w = neg_lse[warp];
@@ -540,25 +572,45 @@ score_pass2_tc(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__
                 }
                 __syncwarp();
             }
-            float* out = raw_part + ((size_t)im.u * 2 * P.RG + 2 * im.rg + wg) * P.N;
-            for (int t = im.t0; t < im.t1; ++t, ++tcount) {
-                if ((int)(tcount & 1) != grp) continue;
-                const uint32_t buf = tcount & 1, use = tcount >> 1;
-                if (!tma::mbar_wait_warp(&sy.acc_full[buf], use & 1, fault, 32)) { ok = false; break; }
+            float* out = POOLED ? reinterpret_cast<float*>(Ks + Cfg<D>::STAGES * Cfg<D>::K_STAGE_BYTES) + wg * POOLED_KEYS - im.key0
+                                : raw_part + ((size_t)im.u * parts + 2 * im.rg + wg) * P.N;
+            for (int t = 0; t < im.tiles; ++t, ++tcount) {
+                if ((int)(tcount & (NB == 2 ? 1 : 3)) != grp) continue;
+                const uint32_t buf = NB == 2 ? tcount & 1 : tcount & 3, use = NB == 2 ? tcount >> 1 : tcount >> 2;
+                if (!ok || !tma::mbar_wait_warp(&sy.acc_full[buf], use & 1, fault, 32)) { ok = false; break; }
                 fence_after_sync();
-                const long long key = (long long)t * KT + key_in_tile;
-                float colsum = 0.f;
-                if (wg_active) {
-                    const uint32_t taddr = lane_addr + buf * 256 + wg * 128;
-                    if ((long long)t * KT + KT <= vis0)
-                        colsum = softmax_tile_pass2<false>(taddr, P.c, nl_w, 0, 0, 0, sy.acc_empty[buf], lane);
-                    else
-                        colsum = softmax_tile_pass2<true>(taddr, P.c, nl_w, key - vis0, row_base % P.w, P.w, sy.acc_empty[buf], lane);
-                } else {
+                const long long key = im.key0 + t * KT + key_in_tile;
+                if (!wg_active) {
                     __syncwarp();
                     if (lane == 0) tma::mbar_arrive(&sy.acc_empty[buf]);
+                    continue;
                 }
-                if (key < P.N) out[key] = colsum;           // zero for a row block past the last row
+                constexpr int PIECES = NB == 2 ? 8 : 0;
+                const uint32_t taddr = lane_addr + (buf * NB + wg) * 128;
+                float colsum;
+                if (im.key0 + t * KT + KT <= vis0)
+                    colsum = softmax_tile_pass2<false, PIECES>(taddr, P.c, nl_w, pieces, 0, 0, 0, sy.acc_empty[buf], lane);
+                else
+                    colsum = softmax_tile_pass2<true, PIECES>(taddr, P.c, nl_w, pieces, key - vis0, row_base % P.w, P.w, sy.acc_empty[buf], lane);
+                if (POOLED || key < P.N) out[key] = colsum;
+            }
+            if constexpr (POOLED) {
+                float* const sums = reinterpret_cast<float*>(Ks + Cfg<D>::STAGES * Cfg<D>::K_STAGE_BYTES);
+                const int r = P.lead, prefix = (int)vis0 - im.key0, n = (int)min((long long)P.step, P.N - (im.key0 + r));     // keys of this chunk, behind its first r sums
+                asm volatile("bar.sync 2, %0;\n" ::"n"(32 * SOFTMAX_WARPS) : "memory");
+                for (int j = threadIdx.x; j < im.tiles * KT; j += 32 * SOFTMAX_WARPS) {
+                    const float v = parts == 2 ? sums[j] + sums[POOLED_KEYS + j] : sums[j];
+                    if (raw_out && ok && j >= r && j < r + n) raw_out[(size_t)im.u * P.N + im.key0 + j] = v;
+                    sums[j] = im.key0 + j >= 0 && j < prefix ? v : -INFINITY;      // pooling looks at the prefix only
+                }
+                asm volatile("bar.sync 2, %0;\n" ::"n"(32 * SOFTMAX_WARPS) : "memory");
+                for (int j = threadIdx.x; j < n; j += 32 * SOFTMAX_WARPS) {
+                    const int last = min(j + 2 * r, im.tiles * KT - 1);
+                    float best = sums[j];
+                    for (int k = j + 1; k <= last; ++k) best = fmaxf(best, sums[k]);
+                    if (ok) score[(size_t)im.u * P.N + im.key0 + r + j] = r + j < prefix ? best : INFINITY;
+                }
+                // a warp writes sums of the next item when every warp has read these: behind that item's first barrier
             }
         }
     }
@@ -577,16 +629,25 @@ score_pool_parts(const float* __restrict__ raw_part, int parts, long long N, int
     const long long i0 = (long long)blockIdx.x * POOL_TILE;
     const float* base = raw_part + (size_t)u * parts * N;
     const long long P = N - w;
-    for (int e = threadIdx.x; e < POOL_TILE + 2 * r; e += 256) {
-        const long long i = i0 - r + e;
-        float v = -INFINITY;
-        if (i >= 0 && i < N) {
-            v = 0.f;
-            for (int p = 0; p < parts; ++p) v += base[(size_t)p * N + i];
-            if (raw_out && e >= r && e < POOL_TILE + r) raw_out[(size_t)u * N + i] = v;
-            if (i >= P) v = -INFINITY;           // pooling looks at the prefix only
+    constexpr int PT = (POOL_TILE + 16 + 255) / 256;            // sums a thread forms, their loads in flight together
+    float v[PT];
+#pragma unroll
+    for (int k = 0; k < PT; ++k) v[k] = 0.f;
+#pragma unroll 2
+    for (int p = 0; p < parts; ++p)
+#pragma unroll
+        for (int k = 0; k < PT; ++k) {
+            const int e = threadIdx.x + 256 * k;
+            const long long i = i0 - r + e;
+            if (e < POOL_TILE + 2 * r && i >= 0 && i < N) v[k] += base[(size_t)p * N + i];
         }
-        rs[e] = v;
+#pragma unroll
+    for (int k = 0; k < PT; ++k) {
+        const int e = threadIdx.x + 256 * k;
+        const long long i = i0 - r + e;
+        if (e >= POOL_TILE + 2 * r) continue;
+        if (raw_out && e >= r && e < POOL_TILE + r && i < N) raw_out[(size_t)u * N + i] = v[k];
+        rs[e] = i >= 0 && i < P ? v[k] : -INFINITY;             // pooling looks at the prefix only
     }
     __syncthreads();
     for (int e = threadIdx.x; e < POOL_TILE; e += 256) {
