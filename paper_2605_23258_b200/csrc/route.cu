@@ -15,12 +15,12 @@ namespace vec {
 
 using sel::Layout;
 
-// Blocks of 32 warps (one resident per multiprocessor, masks and list in up to 200 KB) for inputs beyond a
-// quarter of a million elements, of 16 warps (two resident) for medium ones and of 8 warps (four resident)
-// for short ones, where what a block costs is its fixed sequence of barriers rather than its passes.
-constexpr int SEL_SHORT = 8192, SEL_MANY = 32768, SEL_LONG = 262144;
-constexpr size_t SEL_SMEM_LONG = 200 * 1024, SEL_SMEM_MID = 92 * 1024, SEL_SMEM_SHORT = 36 * 1024;
-#define VEC_SEL_BOUNDS(NW) __launch_bounds__(32 * NW, NW == 32 ? 1 : NW == 16 ? 2 : 4)
+// Inputs of up to 32768 elements are held in registers, by 16 warps up to half of that.  Longer ones: blocks of 32 warps (one
+// resident per multiprocessor, masks and list in up to 200 KB) beyond a quarter of a million elements, of 16 warps (two resident)
+// below.
+constexpr int SEL_REGS16 = 16384, SEL_REGS = 32768, SEL_LONG = 262144;
+constexpr size_t SEL_SMEM_LONG = 200 * 1024, SEL_SMEM_MID = 92 * 1024;
+#define VEC_SEL_BOUNDS(NW) __launch_bounds__(32 * NW, NW == 32 ? 1 : 2)
 
 // The general selection (select_emit) as functions of their own: the kernels run the lean path inline and
 // come here only when it gives up, so its registers are not theirs to carry.
@@ -104,6 +104,59 @@ truncate_kernel(const float* __restrict__ eps, const int32_t* __restrict__ pool_
     const TruncateOut emit = {pool_idx + (size_t)u * n_pool, tr, ret_idx + (size_t)u * n_ret, apx_idx + (size_t)u * n_apx, N};
     if (L.keyed && n_apx > 0 && sel::select_lean<true, NW, false>(e, n_pool, n_apx, S, L, sel_dyn, emit)) return;
     truncate_general<NW>(e, n_pool, n_apx, emit, S, L, sel_dyn);
+}
+
+// Steps 1 and 3 with the input in registers.  grid (U), 32 NW threads.
+struct PoolRegsOut {
+    int32_t* out;
+    __device__ __forceinline__ void put(int i, int pos) const { out[pos] = i; }
+};
+template <int E> struct TruncateRegsOut {
+    TruncateOut to;
+    const int32_t (&token)[E];
+    __device__ __forceinline__ void put(int j, int p, bool is_apx, int pos) const { to.put(p, token[j], is_apx, pos); }
+};
+template <int NW, int E>
+__global__ void VEC_SEL_BOUNDS(NW)
+pool_select_regs(const float* __restrict__ scores, int64_t N, int n_pool, int32_t* __restrict__ pool_idx, float* __restrict__ zero) {
+    __shared__ __align__(16) sel::RegScratch<NW> S;
+    sel::regs_clear(S);
+    // as in pool_select_kernel
+    asm volatile("griddepcontrol.wait;\n" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory");
+    const int u = blockIdx.x;
+    if (n_pool <= 0) return;
+    if (zero)
+        for (int i = threadIdx.x; i < n_pool; i += 32 * NW) zero[(size_t)u * n_pool + i] = 0.f;
+    __syncthreads();
+    sel::select_regs<false, NW, E, true>(scores + (size_t)u * N, (int)N, n_pool, S, PoolRegsOut{pool_idx + (size_t)u * n_pool});
+}
+
+template <int NW, int E>
+__global__ void VEC_SEL_BOUNDS(NW)
+truncate_regs(const float* __restrict__ eps, const int32_t* __restrict__ pool_idx, int64_t N, int n_pool, int n_apx,
+              uint8_t* __restrict__ tier, int32_t* __restrict__ ret_idx, int32_t* __restrict__ apx_idx) {
+    __shared__ __align__(16) sel::RegScratch<NW> S;
+    const int u = blockIdx.x;
+    uint8_t* tr = tier + (size_t)u * N;
+    const int32_t* pool = pool_idx + (size_t)u * n_pool;
+    if ((N & 15) == 0 && ((uintptr_t)tier & 15) == 0) {
+        for (int64_t i = threadIdx.x; i < N / 16; i += 32 * NW) reinterpret_cast<uint4*>(tr)[i] = make_uint4(0, 0, 0, 0);
+    } else {
+        for (int64_t i = threadIdx.x; i < N; i += 32 * NW) tr[i] = 0;
+    }
+    sel::regs_clear(S);
+    // Everything above touches only the tier map, which the residual kernel, this one's primary, neither reads nor writes, and
+    // nothing before that kernel is still under way: it waits before it lets this one start.  (No wait unless a dependent.)  The
+    // list of the pool was written before that kernel.
+    int32_t token[E];
+    const int groups = sel::regs_groups<NW>(n_pool), p0 = (threadIdx.x >> 5) * groups * 32 + (threadIdx.x & 31);
+#pragma unroll
+    for (int j = 0; j < E; ++j) token[j] = j < groups && p0 + 32 * j < n_pool ? pool[p0 + 32 * j] : 0;
+    asm volatile("griddepcontrol.wait;\n" ::: "memory");
+    __syncthreads();
+    const TruncateOut to = {pool, tr, ret_idx + (size_t)u * (n_pool - n_apx), apx_idx + (size_t)u * n_apx, N};
+    sel::select_regs<true, NW, E, false>(eps + (size_t)u * n_pool, n_pool, n_apx, S, TruncateRegsOut<E>{to, token});
 }
 
 // Step 2 on CUDA cores (fp32, and 64-channel bf16 rows off a 16-byte boundary).  A warp takes RW listed rows at once, a lane the output channels lane, lane + 32, ...: an
@@ -281,24 +334,19 @@ static vector_status select_kernels_setup() {
     if (!once.first()) return VECTOR_OK;
     cudaError_t e = cudaFuncSetAttribute(pool_select_kernel<32>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SEL_SMEM_LONG);
     if (e == cudaSuccess) e = cudaFuncSetAttribute(pool_select_kernel<16>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SEL_SMEM_MID);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(pool_select_kernel<8>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SEL_SMEM_SHORT);
     if (e == cudaSuccess) e = cudaFuncSetAttribute(truncate_kernel<32>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SEL_SMEM_LONG);
     if (e == cudaSuccess) e = cudaFuncSetAttribute(truncate_kernel<16>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SEL_SMEM_MID);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(truncate_kernel<8>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SEL_SMEM_SHORT);
     if (e != cudaSuccess) { once.undo(); VEC_CUDA_CHECK(e); }
     return VECTOR_OK;
 }
 
-// Block size, shared-memory budget and smallest useful list of U selections over n elements each.  Short
-// inputs take the small blocks; so do medium ones when there are units enough to fill the small blocks'
-// slots twice over (the phases after the two passes are latency, which more resident blocks hide).
+// Block size and shared-memory layout of selections over n > SEL_REGS elements each.
 struct SelPlan { int nw; Layout L; };
-static SelPlan plan_selection(int64_t n, int U) {
+static SelPlan plan_selection(int64_t n) {
     SelPlan p;
-    const bool small = n < SEL_SHORT || (n < SEL_MANY && U >= 2 * 4 * sm_count());
-    const size_t budget = small ? SEL_SMEM_SHORT : n < SEL_LONG ? SEL_SMEM_MID : SEL_SMEM_LONG;
-    const int min_cand = small ? 1024 : 2048;
-    p.nw = small ? 8 : n < SEL_LONG ? 16 : 32;
+    const size_t budget = n < SEL_LONG ? SEL_SMEM_MID : SEL_SMEM_LONG;
+    const int min_cand = 2048;
+    p.nw = n < SEL_LONG ? 16 : 32;
     p.L = sel::plan_layout(n, false, budget, min_cand, p.nw);
     if (!p.L.keyed) p.L = sel::plan_layout(n, true, budget, min_cand, p.nw);       // the general path stages the images
     return p;
@@ -309,13 +357,19 @@ static vector_status launch_pool_select(const Dims& dm, const vector_budget* bud
     vector_status rc = select_kernels_setup();
     if (rc != VECTOR_OK) return rc;
     const int64_t n = budget->n_tokens;
-    const SelPlan p = plan_selection(n, dm.U);
+    if (n <= SEL_REGS) {
+        auto kern = n <= 2048 ? pool_select_regs<16, 4> : n <= 4096 ? pool_select_regs<16, 8> : n <= 8192 ? pool_select_regs<16, 16>
+                  : n <= SEL_REGS16 ? pool_select_regs<16, 32> : pool_select_regs<32, 32>;
+        VEC_CUDA_CHECK(launch_maybe_dependent(true, kern, dim3(dm.U), dim3(n <= SEL_REGS16 ? 512 : 1024), 0, st, scores, n,
+                                              (int)budget->n_pool, pool, zero));
+        return VECTOR_OK;
+    }
+    const SelPlan p = plan_selection(n);
     const Layout L = p.L;
 #define VEC_POOL(NW)                                                                                                     \
     VEC_CUDA_CHECK(launch_maybe_dependent(true, pool_select_kernel<NW>, dim3(dm.U), dim3(32 * NW), L.bytes(), st, scores, n, \
                                           (int)budget->n_pool, pool, zero, L))
-    if (p.nw == 8) VEC_POOL(8);
-    else if (p.nw == 16) VEC_POOL(16);
+    if (p.nw == 16) VEC_POOL(16);
     else VEC_POOL(32);
 #undef VEC_POOL
     return VECTOR_OK;
@@ -326,15 +380,22 @@ static vector_status launch_truncate(const Dims& dm, const vector_budget* budget
                                      bool dependent = false) {
     vector_status rc = select_kernels_setup();
     if (rc != VECTOR_OK) return rc;
-    const SelPlan p = plan_selection(budget->n_pool, dm.U);
-    const Layout L = p.L;
     // dependent: may start (and clear the tier map) while the kernel before it in the stream drains
+    const int64_t n = budget->n_pool;
+    if (n <= SEL_REGS) {
+        auto kern = n <= 2048 ? truncate_regs<16, 4> : n <= 4096 ? truncate_regs<16, 8> : n <= 8192 ? truncate_regs<16, 16>
+                  : n <= SEL_REGS16 ? truncate_regs<32, 16> : truncate_regs<32, 32>;
+        VEC_CUDA_CHECK(launch_maybe_dependent(dependent, kern, dim3(dm.U), dim3(n <= 8192 ? 512 : 1024), 0, st, eps, pool,
+                                              (int64_t)budget->n_tokens, (int)n, (int)budget->n_apx, tier, ret_idx, apx_idx));
+        return VECTOR_OK;
+    }
+    const SelPlan p = plan_selection(n);
+    const Layout L = p.L;
 #define VEC_TRUNC(NW)                                                                                                   \
     VEC_CUDA_CHECK(launch_maybe_dependent(dependent, truncate_kernel<NW>, dim3(dm.U), dim3(32 * NW), L.bytes(), st, eps, \
                                           pool, (int64_t)budget->n_tokens, (int)budget->n_pool, (int)budget->n_apx, tier, \
                                           ret_idx, apx_idx, L))
-    if (p.nw == 8) VEC_TRUNC(8);
-    else if (p.nw == 16) VEC_TRUNC(16);
+    if (p.nw == 16) VEC_TRUNC(16);
     else VEC_TRUNC(32);
 #undef VEC_TRUNC
     return VECTOR_OK;

@@ -2,7 +2,8 @@
 // building block of Step 1 (the n_pool largest scores) and Step 3 (the n_apx smallest
 // residuals) of the routing (paper Section 3.2).  One thread block per unit.
 //
-// The k-th key is found on an order-preserving 32-bit image of the fp32 value.  Two paths:
+// The k-th key is found on an order-preserving 32-bit image of the fp32 value.  Inputs of up to 32768 elements stay in
+// registers (select_regs, at the end of this file).  Longer ones have two paths:
 //
 // select_lean (the one that normally runs): a histogram of the leading 11 bits over the whole input;
 //   one more pass that writes, per 32 elements, a bit mask of the elements whose leading bits beat the
@@ -659,6 +660,109 @@ __device__ __forceinline__ bool select_lean(const float* __restrict__ vals, int 
         }
     }
     return true;
+}
+
+// ---- short and medium inputs ----------------------------------------------------------------------
+// The whole input in registers: E images a thread, one read of memory, every later pass without one.  Warp w owns
+// `groups` runs of 32 consecutive elements, register j of its lanes the run w * groups + j, so that a ballot over a register
+// is the mask of 32 consecutive elements and ranks in index order are sums of counts.  The k-th key comes from three
+// histograms (11, 11 and 10 bits; the later ones count the elements that share the digits before), whatever the values: many
+// equal ones, none to choose.  What bounds it is a chain of some ten block barriers.
+template <int NW> struct RegScratch {
+    int hist[3][SEL_BINS];
+    int bc[3][2];                 // (digit, rank inside it) of the three digits
+    int part[32];
+    int gt[NW], tie[NW];
+};
+template <int NW>
+__device__ __forceinline__ void regs_clear(RegScratch<NW>& S) {
+    int4* h = reinterpret_cast<int4*>(&S.hist[0][0]);
+#pragma unroll
+    for (int b = threadIdx.x; b < 3 * SEL_BINS / 4; b += 32 * NW) h[b] = make_int4(0, 0, 0, 0);
+}
+template <int NW> __host__ __device__ constexpr int regs_groups(int n) { return ((n + 31) / 32 + NW - 1) / NW; }
+
+// S.hist is zero and visible; k = 0 chooses nothing.  CHOSEN_ONLY: sink.put(i, pos) for every chosen element i; otherwise
+// sink.put(j, i, chosen, pos) for every element, element i being this lane's register j and pos its rank among the chosen or
+// among the others.
+template <bool SMALLEST, int NW, int E, bool CHOSEN_ONLY, typename Sink>
+__device__ __forceinline__ void select_regs(const float* __restrict__ vals, int n, int k, RegScratch<NW>& S, Sink sink) {
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    const unsigned lt = (1u << lane) - 1u;
+    const int groups = regs_groups<NW>(n);                   // <= E
+    const int i0 = wid * groups * 32 + lane;
+    const int mine = i0 < n ? min(groups, (n - i0 + 31) / 32) : 0;      // registers of this lane that hold an element
+    uint32_t key[E];
+#pragma unroll
+    for (int j = 0; j < E; ++j) {
+        // (volatile: a read-only load could be moved ahead of the caller's wait for the kernel that writes vals)
+        key[j] = 0u;
+        if (j < mine) asm volatile("ld.global.b32 %0, [%1];\n" : "=r"(key[j]) : "l"(vals + i0 + 32 * j) : "memory");
+    }
+#pragma unroll
+    for (int j = 0; j < E; ++j) {
+        key[j] = image_of_bits<SMALLEST>(key[j]);
+        if (j < mine) atomicAdd(&S.hist[0][key[j] >> 21], 1);
+    }
+    __syncthreads();
+    uint32_t kth = 0xffffffffu;                              // k = 0: nothing is larger, and no ties are taken
+    int take_ties = 0;
+    if (k > 0) {                                             // block-uniform
+        pick_bin<NW>(S.hist[0], k, S.bc[0], S.part);
+        __syncthreads();
+        const uint32_t d0 = (uint32_t)S.bc[0][0];
+#pragma unroll
+        for (int j = 0; j < E; ++j)
+            if (j < mine && key[j] >> 21 == d0) atomicAdd(&S.hist[1][(key[j] >> 10) & 2047], 1);
+        __syncthreads();
+        pick_bin<NW>(S.hist[1], S.bc[0][1], S.bc[1], S.part);
+        __syncthreads();
+        const uint32_t d1 = (d0 << 11) | (uint32_t)S.bc[1][0];
+#pragma unroll
+        for (int j = 0; j < E; ++j)
+            if (j < mine && key[j] >> 10 == d1) atomicAdd(&S.hist[2][key[j] & 1023], 1);
+        __syncthreads();
+        pick_bin<NW>(S.hist[2], S.bc[1][1], S.bc[2], S.part);
+        __syncthreads();
+        kth = (d1 << 10) | (uint32_t)S.bc[2][0];
+        take_ties = S.bc[2][1];                              // all strictly better elements are chosen; `take_ties` ties complete k
+    }
+    // ---- ranks: better elements and ties of every warp's piece; ties go to the lowest indices
+    int better = 0, ties = 0;
+#pragma unroll
+    for (int j = 0; j < E; ++j) {
+        better += j < mine && key[j] > kth;
+        ties += j < mine && key[j] == kth;
+    }
+    better = __reduce_add_sync(FULL, better);
+    ties = __reduce_add_sync(FULL, ties);
+    if (lane == 0) { S.gt[wid] = better; S.tie[wid] = ties; }
+    __syncthreads();
+    int pos, ties_left;
+    {
+        const int t = lane < NW ? S.tie[lane] : 0;
+        const int before = lane_scan_incl(t, lane) - t;
+        const int quota = max(0, min(t, take_ties - before));
+        const int c = (lane < NW ? S.gt[lane] : 0) + quota;
+        const int first = lane_scan_incl(c, lane) - c;
+        pos = __shfl_sync(FULL, first, wid);
+        ties_left = __shfl_sync(FULL, quota, wid);
+    }
+    // ---- handing out in index order
+#pragma unroll
+    for (int j = 0; j < E; ++j) {
+        if (j >= groups) break;
+        const bool in = j < mine;
+        const unsigned tb = __ballot_sync(FULL, in && key[j] == kth);
+        const int take = min(ties_left, __popc(tb));
+        const bool chosen = in && (key[j] > kth || (key[j] == kth && __popc(tb & lt) < take));
+        const unsigned cb = __ballot_sync(FULL, chosen);
+        const int i = i0 + 32 * j, before = pos + __popc(cb & lt);
+        if constexpr (CHOSEN_ONLY) { if (chosen) sink.put(i, before); }
+        else { if (in) sink.put(j, i, chosen, chosen ? before : i - before); }
+        pos += __popc(cb);
+        ties_left -= take;
+    }
 }
 
 // Shared-memory plan of one selection over n elements within `budget_bytes`: a candidate list of
