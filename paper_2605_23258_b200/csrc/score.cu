@@ -27,23 +27,25 @@ __device__ __forceinline__ void tile_request(const T* __restrict__ src, int64_t 
     for (int e = 0; e < ST * D / 1024; ++e) {
         const int idx = threadIdx.x + 256 * e, r = idx / (D / 4), c4 = idx % (D / 4);
         const T* p = src + (row0 + r) * D + 4 * c4;
+        const bool in = (uint64_t)(row0 + r) < (uint64_t)n_rows;            // rows before the first and behind the last read as zeros
         if constexpr (WIDE) {
-            t.v[e] = row0 + r < n_rows ? *reinterpret_cast<const float4*>(p) : make_float4(0.f, 0.f, 0.f, 0.f);
+            t.v[e] = in ? *reinterpret_cast<const float4*>(p) : make_float4(0.f, 0.f, 0.f, 0.f);
         } else {
-            t.v[e] = row0 + r < n_rows ? make_float4(to_f32(p[0]), to_f32(p[1]), to_f32(p[2]), to_f32(p[3])) : make_float4(0.f, 0.f, 0.f, 0.f);
+            t.v[e] = in ? make_float4(to_f32(p[0]), to_f32(p[1]), to_f32(p[2]), to_f32(p[3])) : make_float4(0.f, 0.f, 0.f, 0.f);
         }
     }
 }
+// Rows of the tiles in shared memory are PITCH<D> floats apart: 16-byte accesses, whose rows begin four banks apart.
+template <int D> constexpr int PITCH = D + 4;
 template <int D>
 __device__ __forceinline__ void tile_store(const TileRegs<D>& t, float* dst) {
 #pragma unroll
     for (int e = 0; e < ST * D / 1024; ++e) {
         const int idx = threadIdx.x + 256 * e, r = idx / (D / 4), c = idx % (D / 4) * 4;
-        float* p = dst + r * (D + 1) + c;
-        p[0] = t.v[e].x; p[1] = t.v[e].y; p[2] = t.v[e].z; p[3] = t.v[e].w;
+        *reinterpret_cast<float4*>(dst + r * PITCH<D> + c) = t.v[e];
     }
 }
-// acc[i][j] = sum_c Qs[ty + 16 i][c] * Ks[tx + 16 j][c]
+// acc[i][j] = sum_c Qs[ty + 16 i][c] * Ks[tx + 16 j][c].  Reads of shared memory are what bounds it: four channels a load.
 template <int D>
 __device__ __forceinline__ void tile_qk(const float* Qs, const float* Ks, float acc[4][4]) {
     const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
@@ -51,28 +53,33 @@ __device__ __forceinline__ void tile_qk(const float* Qs, const float* Ks, float 
     for (int i = 0; i < 4; ++i)
 #pragma unroll
         for (int j = 0; j < 4; ++j) acc[i][j] = 0.f;
-#pragma unroll 16
-    for (int kk = 0; kk < D; ++kk) {
-        float a[4], b[4];
+#pragma unroll 4
+    for (int kk = 0; kk < D; kk += 4) {
+        float4 a[4], b[4];
 #pragma unroll
-        for (int i = 0; i < 4; ++i) a[i] = Qs[(ty + 16 * i) * (D + 1) + kk];
+        for (int i = 0; i < 4; ++i) a[i] = *reinterpret_cast<const float4*>(Qs + (ty + 16 * i) * PITCH<D> + kk);
 #pragma unroll
-        for (int j = 0; j < 4; ++j) b[j] = Ks[(tx + 16 * j) * (D + 1) + kk];
+        for (int j = 0; j < 4; ++j) b[j] = *reinterpret_cast<const float4*>(Ks + (tx + 16 * j) * PITCH<D> + kk);
 #pragma unroll
         for (int i = 0; i < 4; ++i)
 #pragma unroll
-            for (int j = 0; j < 4; ++j) acc[i][j] = fmaf(a[i], b[j], acc[i][j]);
+            for (int j = 0; j < 4; ++j) {
+                acc[i][j] = fmaf(a[i].x, b[j].x, acc[i][j]);
+                acc[i][j] = fmaf(a[i].y, b[j].y, acc[i][j]);
+                acc[i][j] = fmaf(a[i].z, b[j].z, acc[i][j]);
+                acc[i][j] = fmaf(a[i].w, b[j].w, acc[i][j]);
+            }
     }
 }
-template <int D> constexpr int tile_smem() { return 2 * ST * (D + 1) * (int)sizeof(float); }
+template <int D> constexpr int tile_smem() { return 2 * ST * PITCH<D> * (int)sizeof(float); }
 
 // grid (n_chunks, row_tiles, U), 256 threads, tile_smem of dynamic shared memory
 template <typename T, int D, bool WIDE>
 __global__ void __launch_bounds__(256)
 score_pass1_generic(const T* __restrict__ Q, const T* __restrict__ K, int64_t N, int R, int w,
                     float scale, int64_t chunk_len, float2* __restrict__ partial) {
-    extern __shared__ float tiles[];
-    float *Qs = tiles, *Ks = tiles + ST * (D + 1);
+    extern __shared__ __align__(16) float tiles[];
+    float *Qs = tiles, *Ks = tiles + ST * PITCH<D>;
     asm volatile("griddepcontrol.wait;\n" ::: "memory");        // launched as a programmatic dependent: nothing is touched before
     asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory");
     const int u = blockIdx.z, row0 = blockIdx.y * ST, chunk = blockIdx.x, n_chunks = gridDim.x;
@@ -174,20 +181,21 @@ score_lse_rows(const float2* __restrict__ partial, int R, int n_chunks, float* _
 }
 
 // grid (key_tiles, U), 256 threads, tile_smem of dynamic shared memory.  INLINE_LSE: a block forms the normalisers of its
-// rows itself from the chunk partials (a launch less; every key tile repeats it).
-template <typename T, int D, bool INLINE_LSE, bool WIDE>
+// rows itself from the chunk partials (a launch less; every key tile repeats it).  POOLED: the block pools its sums itself (another
+// launch less); its tiles overlap by the pooling radius on both sides, raw may be null.
+template <typename T, int D, bool INLINE_LSE, bool WIDE, bool POOLED>
 __global__ void __launch_bounds__(256)
 score_pass2_generic(const T* __restrict__ Q, const T* __restrict__ K, int64_t N, int R, int w,
                     float scale, const float2* __restrict__ partial, int n_chunks, const float* __restrict__ lse,
-                    float* __restrict__ raw) {
-    extern __shared__ float tiles[];
-    float *Qs = tiles, *Ks = tiles + ST * (D + 1);
+                    float* __restrict__ raw, int r, float* __restrict__ score) {
+    extern __shared__ __align__(16) float tiles[];
+    float *Qs = tiles, *Ks = tiles + ST * PITCH<D>;
     __shared__ float red[16][ST];
     __shared__ float lse_s[ST];
     asm volatile("griddepcontrol.wait;\n" ::: "memory");
     asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory");
     const int u = blockIdx.y;
-    const int64_t key0 = (int64_t)blockIdx.x * ST;
+    const int64_t key0 = POOLED ? (int64_t)blockIdx.x * (ST - 2 * r) - r : (int64_t)blockIdx.x * ST;       // POOLED: -r at first
     const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
     const T* Qu = Q + (size_t)u * R * D;
     TileRegs<D> next;
@@ -234,7 +242,22 @@ score_pass2_generic(const T* __restrict__ Q, const T* __restrict__ K, int64_t N,
 #pragma unroll
         for (int t = 0; t < 16; ++t) s += red[t][tid];
         int64_t key = key0 + tid;
-        if (key < N) raw[(size_t)u * N + key] = s;
+        if constexpr (!POOLED) {
+            if (key < N) raw[(size_t)u * N + key] = s;
+        } else {
+            const bool own = tid >= r && tid < ST - r && key < N;
+            if (raw && own) raw[(size_t)u * N + key] = s;
+            lse_s[tid] = key >= 0 && key < N - w ? s : -INFINITY;            // pooling looks at the prefix only
+        }
+    }
+    if constexpr (POOLED) {
+        __syncthreads();
+        const int64_t key = key0 + tid;
+        if (tid >= r && tid < ST - r && key < N) {
+            float best = -INFINITY;
+            for (int k = tid - r; k <= tid + r; ++k) best = fmaxf(best, lse_s[k]);
+            score[(size_t)u * N + key] = key < N - w ? best : INFINITY;
+        }
     }
 }
 
@@ -265,8 +288,9 @@ static vector_status launch_score(const Dims& dm, const void* Q_, const void* K_
     static PerDeviceOnce once;
     if (once.first()) {
         cudaError_t e = cudaFuncSetAttribute(score_pass1_generic<T, D, WIDE>, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM);
-        if (e == cudaSuccess) e = cudaFuncSetAttribute(score_pass2_generic<T, D, true, WIDE>, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM);
-        if (e == cudaSuccess) e = cudaFuncSetAttribute(score_pass2_generic<T, D, false, WIDE>, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM);
+        if (e == cudaSuccess) e = cudaFuncSetAttribute(score_pass2_generic<T, D, true, WIDE, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM);
+        if (e == cudaSuccess) e = cudaFuncSetAttribute(score_pass2_generic<T, D, true, WIDE, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM);
+        if (e == cudaSuccess) e = cudaFuncSetAttribute(score_pass2_generic<T, D, false, WIDE, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM);
         if (e != cudaSuccess) { once.undo(); VEC_CUDA_CHECK(e); }
     }
     const size_t lse_b = align256((size_t)dm.U * dm.R * sizeof(float)), raw_b = raw_out ? 0 : align256((size_t)dm.U * (size_t)N * sizeof(float));
@@ -287,9 +311,17 @@ static vector_status launch_score(const Dims& dm, const void* Q_, const void* K_
     if (!inline_lse)
         VEC_CUDA_CHECK(launch_maybe_dependent(true, score_lse_rows, dim3((dm.R + 63) / 64, dm.U), dim3(256), 0, st, partial, dm.R,
                                               n_chunks, lse));
-    VEC_CUDA_CHECK(launch_maybe_dependent(true, inline_lse ? score_pass2_generic<T, D, true, WIDE> : score_pass2_generic<T, D, false, WIDE>,
+    // The launch that pooling costs counts where the second pass is short: no more blocks than multiprocessors, overlaps included.
+    const int r = dm.pool_kernel / 2;
+    const int64_t tiles_pooled = (N + ST - 2 * r - 1) / (ST - 2 * r);
+    if (inline_lse && tiles_pooled * dm.U <= sm_count()) {
+        VEC_CUDA_CHECK(launch_maybe_dependent(true, score_pass2_generic<T, D, true, WIDE, true>, dim3((unsigned)tiles_pooled, dm.U), dim3(256), SMEM, st,
+                                              Q, K, N, dm.R, dm.w, dm.scale, partial, n_chunks, lse, raw_out, r, scores));
+        return VECTOR_OK;
+    }
+    VEC_CUDA_CHECK(launch_maybe_dependent(true, inline_lse ? score_pass2_generic<T, D, true, WIDE, false> : score_pass2_generic<T, D, false, WIDE, false>,
                                           dim3((unsigned)((N + ST - 1) / ST), dm.U), dim3(256), SMEM, st, Q, K, N, dm.R, dm.w, dm.scale,
-                                          partial, n_chunks, lse, raw));
+                                          partial, n_chunks, lse, raw, r, scores));
     int64_t total = (int64_t)dm.U * N;
     VEC_CUDA_CHECK(launch_maybe_dependent(true, score_pool_kernel, dim3((unsigned)((total + 255) / 256)), dim3(256), 0, st, raw, N, dm.w,
                                           dm.pool_kernel / 2, total, scores));
