@@ -237,8 +237,10 @@ static vector_status launch_layer_mma(const Dims& dm, int L, const void* q, cons
     static PerDeviceOnce once;
     if (once.first()) {
         cudaError_t e = cudaFuncSetAttribute(dlm::decode_layer_mma, cudaFuncAttributeMaxDynamicSharedMemorySize, dlm::SMEM_BYTES);
-        if (e == cudaSuccess) e = cudaFuncSetAttribute(dlm::decode_layer_merge_mma<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, dlm::MERGE_PAD);
-        if (e == cudaSuccess) e = cudaFuncSetAttribute(dlm::decode_layer_merge_mma<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, dlm::MERGE_PAD);
+        if (e == cudaSuccess) e = cudaFuncSetAttribute(dlm::decode_layer_merge_mma<float, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, dlm::MERGE_PAD);
+        if (e == cudaSuccess) e = cudaFuncSetAttribute(dlm::decode_layer_merge_mma<T, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, dlm::MERGE_PAD);
+        if (e == cudaSuccess) e = cudaFuncSetAttribute(dlm::decode_layer_merge_mma<float, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, dlm::MERGE_PAD);
+        if (e == cudaSuccess) e = cudaFuncSetAttribute(dlm::decode_layer_merge_mma<T, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, dlm::MERGE_PAD);
         if (e != cudaSuccess) { once.undo(); VEC_CUDA_CHECK(e); }
     }
     const int UL = dm.U / dlm::HKV;
@@ -261,13 +263,17 @@ static vector_status launch_layer_mma(const Dims& dm, int L, const void* q, cons
     // The merge's blocks start while the streaming kernel's last ones run, three to each multiprocessor that is free by then:
     // shared memory that nobody uses keeps them to one or two when that is enough for all of them.  Measured so and with three to
     // a multiprocessor, us a step in a graph: 32 pairs of 600 rows 38 / 43, of 7200 rows 133 / 140; 16 of 4900 rows 62 / 76.
-    const size_t pad = dm.U <= sm_count() ? dlm::MERGE_PAD : dm.U <= 2 * sm_count() ? dlm::MERGE_PAD / 2 : 0;
+    // With more units than that, a block takes as many sequences as have room in the product's columns: it fetches 256 KB of the map
+    // once for all of them.  70 pairs of 349 rows 56 -> 46 us; 32 pairs of 7200 rows, two units a multiprocessor, 136.3 and 137.1.
+    const int batch = UL / L, seqs = dm.U > 2 * sm_count() ? (8 / dm.g < batch ? 8 / dm.g : batch) : 1;
+    const int blocks = L * dlm::HKV * ((batch + seqs - 1) / seqs);
+    const size_t pad = blocks <= sm_count() ? dlm::MERGE_PAD : blocks <= 2 * sm_count() ? dlm::MERGE_PAD / 2 : 0;
     if (out_dtype == VECTOR_F32)
-        VEC_CUDA_CHECK(launch_maybe_dependent(true, dlm::decode_layer_merge_mma<float>, dim3(dm.U), dim3(dlm::MERGE_THREADS), pad, st, partial,
-                                              (const T*)W, L, dm.g, pl, (float*)out));
+        VEC_CUDA_CHECK(launch_maybe_dependent(true, seqs > 1 ? dlm::decode_layer_merge_mma<float, true> : dlm::decode_layer_merge_mma<float, false>,
+                                              dim3(blocks), dim3(dlm::MERGE_THREADS), pad, st, partial, (const T*)W, L, dm.g, batch, seqs, pl, (float*)out));
     else
-        VEC_CUDA_CHECK(launch_maybe_dependent(true, dlm::decode_layer_merge_mma<T>, dim3(dm.U), dim3(dlm::MERGE_THREADS), pad, st, partial,
-                                              (const T*)W, L, dm.g, pl, (T*)out));
+        VEC_CUDA_CHECK(launch_maybe_dependent(true, seqs > 1 ? dlm::decode_layer_merge_mma<T, true> : dlm::decode_layer_merge_mma<T, false>,
+                                              dim3(blocks), dim3(dlm::MERGE_THREADS), pad, st, partial, (const T*)W, L, dm.g, batch, seqs, pl, (T*)out));
     return VECTOR_OK;
 }
 

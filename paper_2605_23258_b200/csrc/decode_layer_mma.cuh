@@ -381,47 +381,57 @@ decode_layer_mma(const __nv_bfloat16* __restrict__ q, const __grid_constant__ db
 // Merge for the same shapes: combines the splits' records of a unit, applies row block h of the layer's map
 // to the merged key sums of all heads and normalises,
 //   o_a = (sum_s f_s acc_v_s + W[h rows] sum_s f_s acc_k_s) / sum_s f_s l_s,   f_s = exp(m_s - max m).
-// grid (U), 512 threads.  The product runs on warp-level MMAs: M = the head's 128 output channels (warps w and w + 8:
-// rows 16 w .., each half of the input heads), N = the unit's g query heads (padded to 8), K = 8 x 128; A fragments straight
+// SHARED: a block takes `seqs` sequences of one (layer, head), whose query heads are the product's columns: the map's rows, 256 KB
+// a block, are what most of a merge fetches from L2 where units are many and their records few.
+// grid (layers * HKV * ceil(batch / seqs)), seqs * g <= 8; without SHARED seqs = 1; 512 threads.  The product runs on warp-level MMAs: M = the head's 128 output channels (warps w and w + 8:
+// rows 16 w .., each half of the input heads), N = the sequences' query heads (padded to 8), K = 8 x 128; A fragments straight
 // from the map (16-byte loads: thread (row r, quarter t) holds columns 8 (t + 4 jj) .. + 7 of rows r and r + 8 of a
 // 128-column block, the k slots of an MMA step follow that order in both operands), the key sums as bf16
 // hi + lo in shared memory.  What it costs is memory latency (42 MB of records and 64 MB of map from L2 over 256 blocks):
 // hence eight-byte loads with eight splits of two elements in flight, and 16 warps on the map's rows.
 constexpr int MERGE_THREADS = 512, MERGE_PAD = 72 * 1024;     // + 46 KB of its own: one block to a multiprocessor, with half of it two
-template <typename TO>
+template <typename TO, bool SHARED>
 __global__ void __launch_bounds__(MERGE_THREADS)
-decode_layer_merge_mma(const float* __restrict__ partial, const __nv_bfloat16* __restrict__ W, int L, int g, Plan pl,
+decode_layer_merge_mma(const float* __restrict__ partial, const __nv_bfloat16* __restrict__ W, int L, int g, int batch, int seqs, Plan pl,
                        TO* __restrict__ out) {
     constexpr int KD = HKV * 128;
     __shared__ __align__(16) __nv_bfloat16 akh[8][KD], akl[8][KD];          // 32 KB
     __shared__ float accv[8][128], pw[2][8][128], fs[8][32], Ls[8];
-    const int u = blockIdx.x, tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
-    const int h = u % HKV, layer = (u / HKV) % L;
+    __shared__ int splits[8];                            // records of a sequence
+    const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+    const int h = blockIdx.x % HKV, layer = (blockIdx.x / HKV) % L, b0 = blockIdx.x / (HKV * L) * seqs;
+    const int n_heads = SHARED ? min(seqs, batch - b0) * g : g;          // columns in use: sequence b0 + a / g, query head a % g
     const int row = lane >> 2, quarter = lane & 3;
-    const float* rec0 = partial + (size_t)u * pl.s_max * g * REC;
-    const long long c0 = (long long)(u / HKV) * pl.weight;
-    const int n_splits = block_of_cost(c0 + pl.weight - 1, pl) - block_of_cost(c0, pl) + 1;
-    for (int i = tid; i < (8 - g) * KD; i += MERGE_THREADS) {            // columns of B beyond the unit's heads
-        akh[g + i / KD][i % KD] = __float2bfloat16_rn(0.f);
-        akl[g + i / KD][i % KD] = __float2bfloat16_rn(0.f);
+    auto pair_of = [&](int a) { return (b0 + (SHARED ? a / g : 0)) * L + layer; };
+    auto records_of = [&](int a) { return partial + (((size_t)pair_of(a) * HKV + h) * pl.s_max * g + (SHARED ? a % g : a)) * REC; };      // g * REC apart
+    auto splits_of = [&](int a) {
+        const long long c0 = (long long)pair_of(a) * pl.weight;
+        return block_of_cost(c0 + pl.weight - 1, pl) - block_of_cost(c0, pl) + 1;
+    };
+    const int splits0 = SHARED ? 0 : splits_of(0);
+    for (int i = tid; i < (8 - n_heads) * KD; i += MERGE_THREADS) {      // columns of B beyond them
+        akh[n_heads + i / KD][i % KD] = __float2bfloat16_rn(0.f);
+        akl[n_heads + i / KD][i % KD] = __float2bfloat16_rn(0.f);
     }
     asm volatile("griddepcontrol.wait;\n" ::: "memory");                 // the streaming kernel's records
-    // factors of the splits: warp a < g takes head a
-    if (wid < g) {
-        const float mj = lane < n_splits ? rec0[((size_t)lane * g + wid) * REC] : -INFINITY;
-        const float lj = lane < n_splits ? rec0[((size_t)lane * g + wid) * REC + 1] : 0.f;
+    // factors of the splits: warp a < n_heads takes column a
+    if (wid < n_heads) {
+        const int n_splits = SHARED ? splits_of(wid) : splits0;
+        const float* rec = records_of(wid) + (size_t)lane * g * REC;
+        const float mj = lane < n_splits ? rec[0] : -INFINITY;
+        const float lj = lane < n_splits ? rec[1] : 0.f;
         const float M = warp_max(mj);
         const float f = mj > -INFINITY ? __expf(mj - M) : 0.f;
         fs[wid][lane] = f;
         const float Lsum = warp_sum(f * lj);
-        if (lane == 0) Ls[wid] = Lsum;
+        if (lane == 0) { Ls[wid] = Lsum; if (SHARED) splits[wid] = n_splits; }
     }
     __syncthreads();
     // merged sums: a thread has two neighbouring elements of a record's 128 + 1024 values
     constexpr int PAIRS = (128 + KD) / 2;
-    for (int i = tid; i < g * PAIRS; i += MERGE_THREADS) {
-        const int a = i / PAIRS, e = (i - a * PAIRS) * 2;
-        const float* src = rec0 + (size_t)a * REC + 2 + e;
+    for (int i = tid; i < n_heads * PAIRS; i += MERGE_THREADS) {
+        const int a = i / PAIRS, e = (i - a * PAIRS) * 2, n_splits = SHARED ? splits[a] : splits0;
+        const float* src = records_of(a) + 2 + e;
         float v0 = 0.f, v1 = 0.f;
         for (int s0 = 0; s0 < n_splits; s0 += 8) {
             float2 x[8];
@@ -469,13 +479,13 @@ decode_layer_merge_mma(const float* __restrict__ partial, const __nv_bfloat16* _
             }
         }
         // d[0], d[1]: row `row`, heads 2 quarter and 2 quarter + 1; d[2], d[3]: row `row` + 8
-        if (2 * quarter < g) { pw[half][2 * quarter][r0] = d[0]; pw[half][2 * quarter][r0 + 8] = d[2]; }
-        if (2 * quarter + 1 < g) { pw[half][2 * quarter + 1][r0] = d[1]; pw[half][2 * quarter + 1][r0 + 8] = d[3]; }
+        if (2 * quarter < n_heads) { pw[half][2 * quarter][r0] = d[0]; pw[half][2 * quarter][r0 + 8] = d[2]; }
+        if (2 * quarter + 1 < n_heads) { pw[half][2 * quarter + 1][r0] = d[1]; pw[half][2 * quarter + 1][r0 + 8] = d[3]; }
     }
     __syncthreads();
-    for (int i = tid; i < g * 128; i += MERGE_THREADS) {
+    for (int i = tid; i < n_heads * 128; i += MERGE_THREADS) {
         const int a = i >> 7, c = i & 127;
-        store_out(out + ((size_t)u * g + a) * 128 + c, (accv[a][c] + (pw[0][a][c] + pw[1][a][c])) / Ls[a]);
+        store_out(out + (((size_t)pair_of(a) * HKV + h) * g + (SHARED ? a % g : a)) * 128 + c, (accv[a][c] + (pw[0][a][c] + pw[1][a][c])) / Ls[a]);
     }
 }
 
