@@ -667,9 +667,7 @@ __device__ __forceinline__ bool select_lean(const float* __restrict__ vals, int 
 // `groups` runs of 32 consecutive elements, register j of its lanes the run w * groups + j, so that a ballot over a register
 // is the mask of 32 consecutive elements and ranks in index order are sums of counts.  The k-th key comes from three
 // histograms (11, 11 and 10 bits; the later ones count the elements that share the digits before), whatever the values: many
-// equal ones, none to choose.  What bounds it is a chain of some ten block barriers and
-// the walk over the registers between them: of 20 000 cycles for 16384 elements by 16 warps 1 400 to load, 4 000 to the first
-// digit, 5 400 to the last, 1 700 to count, 7 700 to hand out with two ballots a register (one, but for a warp whose ties are divided).
+// equal ones, none to choose.  What bounds it is a chain of some ten block barriers.
 template <int NW> struct RegScratch {
     int hist[3][SEL_BINS];
     int bc[3][2];                 // (digit, rank inside it) of the three digits
@@ -741,7 +739,6 @@ __device__ __forceinline__ void select_regs(const float* __restrict__ vals, int 
     if (lane == 0) { S.gt[wid] = better; S.tie[wid] = ties; }
     __syncthreads();
     int pos, ties_left;
-    bool split;                                              // some of this warp's ties are chosen and some are not
     {
         const int t = lane < NW ? S.tie[lane] : 0;
         const int before = lane_scan_incl(t, lane) - t;
@@ -750,21 +747,15 @@ __device__ __forceinline__ void select_regs(const float* __restrict__ vals, int 
         const int first = lane_scan_incl(c, lane) - c;
         pos = __shfl_sync(FULL, first, wid);
         ties_left = __shfl_sync(FULL, quota, wid);
-        split = ties_left > 0 && ties_left < __shfl_sync(FULL, t, wid);
     }
     // ---- handing out in index order
-    const bool with_ties = ties_left > 0;
 #pragma unroll
     for (int j = 0; j < E; ++j) {
         if (j >= groups) break;
         const bool in = j < mine;
-        bool chosen = in && (key[j] > kth || (with_ties && key[j] == kth));
-        int take = 0;
-        if (split) {                                         // warp-uniform, rare: the lowest indices only
-            const unsigned tb = __ballot_sync(FULL, in && key[j] == kth);
-            take = min(ties_left, __popc(tb));
-            chosen = in && (key[j] > kth || (key[j] == kth && __popc(tb & lt) < take));
-        }
+        const unsigned tb = __ballot_sync(FULL, in && key[j] == kth);
+        const int take = min(ties_left, __popc(tb));
+        const bool chosen = in && (key[j] > kth || (key[j] == kth && __popc(tb & lt) < take));
         const unsigned cb = __ballot_sync(FULL, chosen);
         const int i = i0 + 32 * j, before = pos + __popc(cb & lt);
         if constexpr (CHOSEN_ONLY) { if (chosen) sink.put(i, before); }
