@@ -14,7 +14,9 @@
 //   one warp    MMA issuer, TMEM owner; also TMA-loads the unit's W when the range enters a new unit
 //   4 warps     epilogue: thread = row
 // Without RoPE: stages of K | V (three of 64 KB at D = 128, five of 32 KB at D = 64), tiles published
-// all stages but one behind the one being issued: 128 KB of row loads stay in flight.
+// one behind the one being issued: the fence that comes before waits for the newer tiles' copies too, so that a tile held back
+// longer waits for more of them.  256 lists of 9829 of 32768 tokens, routed, us: one behind 261 at D = 128 and 189 at D = 64, all
+// stages but one 267 and 200.
 // With RoPE: the turned key is no longer a bf16 number, so it goes to the tensor cores as a bf16
 // pair hi + lo (two chains over the same W), which keeps it to 2^-17 relative; two stages of
 // K hi | K lo | V (96 KB each).  At D = 64 it goes there as three bf16 parts, turned to fp32's own precision (rope.cuh): 64 KB a stage;
@@ -293,24 +295,16 @@ residual_tc(const __nv_bfloat16* __restrict__ K, const __nv_bfloat16* __restrict
                     cp_async16(vdst + other + p * PASS_BYTES, Vu + ro + D / 2, nb);
                 }
                 cp_async_commit();
-                if (i >= STAGES - 1) {                   // this thread's copies of the tile STAGES - 1 before this one have landed
-                    cp_async_wait<STAGES - 1>();
+                if (i >= 1) {                            // this thread's copies of the tile before this one have landed
+                    cp_async_wait<1>();
                     fence_async_proxy();
-                    tma::mbar_arrive(&sy.full[(i - (STAGES - 1)) % STAGES]);
+                    tma::mbar_arrive(&sy.full[(i - 1) % STAGES]);
                 }
 #pragma unroll
                 for (int p = 0; p < PASSES; ++p) cur[p] = nxt[p];
             }
-            if (ok) {
-                auto publish = [&](int behind) {             // tile n_my - 1 - behind, if there is one
-                    if (n_my > behind) { fence_async_proxy(); tma::mbar_arrive(&sy.full[(n_my - 1 - behind) % STAGES]); }
-                };
-                if constexpr (STAGES == 5) { cp_async_wait<3>(); publish(3); cp_async_wait<2>(); publish(2); }
-                cp_async_wait<1>(); publish(1);
-                cp_async_wait<0>(); publish(0);
-            } else {
-                cp_async_wait<0>();
-            }
+            cp_async_wait<0>();
+            if (ok && n_my > 0) { fence_async_proxy(); tma::mbar_arrive(&sy.full[(n_my - 1) % STAGES]); }
         }
     } else if (warp == R_LOADER_WARPS) {
         // ------------------------------------------------------------------ W loads and MMA issue
