@@ -15,7 +15,9 @@ namespace vec {
 
 using sel::Layout;
 
-// Inputs of up to 32768 elements are held in registers, by 16 warps up to half of that.  Longer ones: blocks of 32 warps (one
+// Inputs of up to 32768 elements are held in registers, by 16 warps up to half of that (32 registers a thread are what 64 of them
+// leave room for).  Step 1 with two passes over memory and in registers, us: 16 lists of 3968 elements 14.3 / 5.5, of 16384
+// 15.3 / 13.6, 128 of 3804 10.5 / 6.1, 256 of 20011 28.0 / 27.7, of 32768 36.9 / 37.5.  Longer ones: blocks of 32 warps (one
 // resident per multiprocessor, masks and list in up to 200 KB) beyond a quarter of a million elements, of 16 warps (two resident)
 // below.
 constexpr int SEL_REGS16 = 16384, SEL_REGS = 32768, SEL_LONG = 262144;

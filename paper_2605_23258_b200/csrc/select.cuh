@@ -667,7 +667,10 @@ __device__ __forceinline__ bool select_lean(const float* __restrict__ vals, int 
 // `groups` runs of 32 consecutive elements, register j of its lanes the run w * groups + j, so that a ballot over a register
 // is the mask of 32 consecutive elements and ranks in index order are sums of counts.  The k-th key comes from three
 // histograms (11, 11 and 10 bits; the later ones count the elements that share the digits before), whatever the values: many
-// equal ones, none to choose.  What bounds it is a chain of some ten block barriers.
+// equal ones, none to choose.  What bounds it is a chain of some ten block barriers and
+// the walk over the registers between them: of 20 000 cycles for 16384 elements by 16 warps 1 400 to load, 4 000 to the first
+// digit, 5 400 to the last, 1 700 to count, 7 700 to hand out.  (One ballot a register in place of two, where a warp's ties are not
+// divided: 13.5 -> 15.3 us.)
 template <int NW> struct RegScratch {
     int hist[3][SEL_BINS];
     int bc[3][2];                 // (digit, rank inside it) of the three digits
