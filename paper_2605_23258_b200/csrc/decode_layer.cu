@@ -237,10 +237,10 @@ static vector_status launch_layer_mma(const Dims& dm, int L, const void* q, cons
     static PerDeviceOnce once;
     if (once.first()) {
         cudaError_t e = cudaFuncSetAttribute(dlm::decode_layer_mma, cudaFuncAttributeMaxDynamicSharedMemorySize, dlm::SMEM_BYTES);
-        if (e == cudaSuccess) e = cudaFuncSetAttribute(dlm::decode_layer_merge_mma<float, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, dlm::MERGE_PAD);
-        if (e == cudaSuccess) e = cudaFuncSetAttribute(dlm::decode_layer_merge_mma<T, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, dlm::MERGE_PAD);
-        if (e == cudaSuccess) e = cudaFuncSetAttribute(dlm::decode_layer_merge_mma<float, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, dlm::MERGE_PAD);
-        if (e == cudaSuccess) e = cudaFuncSetAttribute(dlm::decode_layer_merge_mma<T, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, dlm::MERGE_PAD);
+        if (e == cudaSuccess) e = cudaFuncSetAttribute(dlm::decode_layer_merge_mma<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, dlm::MERGE_PAD);
+        if (e == cudaSuccess) e = cudaFuncSetAttribute(dlm::decode_layer_merge_mma<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, dlm::MERGE_PAD);
+        if (e == cudaSuccess) e = cudaFuncSetAttribute(dlm::decode_layer_merge_shared<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, dlm::MERGE_PAD);
+        if (e == cudaSuccess) e = cudaFuncSetAttribute(dlm::decode_layer_merge_shared<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, dlm::MERGE_PAD);
         if (e != cudaSuccess) { once.undo(); VEC_CUDA_CHECK(e); }
     }
     const int UL = dm.U / dlm::HKV;
@@ -268,12 +268,12 @@ static vector_status launch_layer_mma(const Dims& dm, int L, const void* q, cons
     const int batch = UL / L, seqs = dm.U > 2 * sm_count() ? (8 / dm.g < batch ? 8 / dm.g : batch) : 1;
     const int blocks = L * dlm::HKV * ((batch + seqs - 1) / seqs);
     const size_t pad = blocks <= sm_count() ? dlm::MERGE_PAD : blocks <= 2 * sm_count() ? dlm::MERGE_PAD / 2 : 0;
-    if (out_dtype == VECTOR_F32)
-        VEC_CUDA_CHECK(launch_maybe_dependent(true, seqs > 1 ? dlm::decode_layer_merge_mma<float, true> : dlm::decode_layer_merge_mma<float, false>,
-                                              dim3(blocks), dim3(dlm::MERGE_THREADS), pad, st, partial, (const T*)W, L, dm.g, batch, seqs, pl, (float*)out));
-    else
-        VEC_CUDA_CHECK(launch_maybe_dependent(true, seqs > 1 ? dlm::decode_layer_merge_mma<T, true> : dlm::decode_layer_merge_mma<T, false>,
-                                              dim3(blocks), dim3(dlm::MERGE_THREADS), pad, st, partial, (const T*)W, L, dm.g, batch, seqs, pl, (T*)out));
+    auto merge = [&](auto* o, auto one, auto shared) {
+        if (seqs == 1) return launch_maybe_dependent(true, one, dim3(blocks), dim3(dlm::MERGE_THREADS), pad, st, partial, (const T*)W, L, dm.g, pl, o);
+        return launch_maybe_dependent(true, shared, dim3(blocks), dim3(dlm::MERGE_THREADS), pad, st, partial, (const T*)W, L, dm.g, batch, seqs, pl, o);
+    };
+    if (out_dtype == VECTOR_F32) VEC_CUDA_CHECK(merge((float*)out, dlm::decode_layer_merge_mma<float>, dlm::decode_layer_merge_shared<float>));
+    else VEC_CUDA_CHECK(merge((T*)out, dlm::decode_layer_merge_mma<T>, dlm::decode_layer_merge_shared<T>));
     return VECTOR_OK;
 }
 

@@ -381,18 +381,111 @@ decode_layer_mma(const __nv_bfloat16* __restrict__ q, const __grid_constant__ db
 // Merge for the same shapes: combines the splits' records of a unit, applies row block h of the layer's map
 // to the merged key sums of all heads and normalises,
 //   o_a = (sum_s f_s acc_v_s + W[h rows] sum_s f_s acc_k_s) / sum_s f_s l_s,   f_s = exp(m_s - max m).
-// SHARED: a block takes `seqs` sequences of one (layer, head), whose query heads are the product's columns: the map's rows, 256 KB
-// a block, are what most of a merge fetches from L2 where units are many and their records few.
-// grid (layers * HKV * ceil(batch / seqs)), seqs * g <= 8; without SHARED seqs = 1; 512 threads.  The product runs on warp-level MMAs: M = the head's 128 output channels (warps w and w + 8:
-// rows 16 w .., each half of the input heads), N = the sequences' query heads (padded to 8), K = 8 x 128; A fragments straight
+// grid (U), 512 threads.  The product runs on warp-level MMAs: M = the head's 128 output channels (warps w and w + 8:
+// rows 16 w .., each half of the input heads), N = the unit's g query heads (padded to 8), K = 8 x 128; A fragments straight
 // from the map (16-byte loads: thread (row r, quarter t) holds columns 8 (t + 4 jj) .. + 7 of rows r and r + 8 of a
 // 128-column block, the k slots of an MMA step follow that order in both operands), the key sums as bf16
 // hi + lo in shared memory.  What it costs is memory latency (42 MB of records and 64 MB of map from L2 over 256 blocks):
 // hence eight-byte loads with eight splits of two elements in flight, and 16 warps on the map's rows.
 constexpr int MERGE_THREADS = 512, MERGE_PAD = 72 * 1024;     // + 46 KB of its own: one block to a multiprocessor, with half of it two
-template <typename TO, bool SHARED>
+template <typename TO>
 __global__ void __launch_bounds__(MERGE_THREADS)
-decode_layer_merge_mma(const float* __restrict__ partial, const __nv_bfloat16* __restrict__ W, int L, int g, int batch, int seqs, Plan pl,
+decode_layer_merge_mma(const float* __restrict__ partial, const __nv_bfloat16* __restrict__ W, int L, int g, Plan pl,
+                       TO* __restrict__ out) {
+    constexpr int KD = HKV * 128;
+    __shared__ __align__(16) __nv_bfloat16 akh[8][KD], akl[8][KD];          // 32 KB
+    __shared__ float accv[8][128], pw[2][8][128], fs[8][32], Ls[8];
+    const int u = blockIdx.x, tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+    const int h = u % HKV, layer = (u / HKV) % L;
+    const int row = lane >> 2, quarter = lane & 3;
+    const float* rec0 = partial + (size_t)u * pl.s_max * g * REC;
+    const long long c0 = (long long)(u / HKV) * pl.weight;
+    const int n_splits = block_of_cost(c0 + pl.weight - 1, pl) - block_of_cost(c0, pl) + 1;
+    for (int i = tid; i < (8 - g) * KD; i += MERGE_THREADS) {            // columns of B beyond the unit's heads
+        akh[g + i / KD][i % KD] = __float2bfloat16_rn(0.f);
+        akl[g + i / KD][i % KD] = __float2bfloat16_rn(0.f);
+    }
+    asm volatile("griddepcontrol.wait;\n" ::: "memory");                 // the streaming kernel's records
+    // factors of the splits: warp a < g takes head a
+    if (wid < g) {
+        const float mj = lane < n_splits ? rec0[((size_t)lane * g + wid) * REC] : -INFINITY;
+        const float lj = lane < n_splits ? rec0[((size_t)lane * g + wid) * REC + 1] : 0.f;
+        const float M = warp_max(mj);
+        const float f = mj > -INFINITY ? __expf(mj - M) : 0.f;
+        fs[wid][lane] = f;
+        const float Lsum = warp_sum(f * lj);
+        if (lane == 0) Ls[wid] = Lsum;
+    }
+    __syncthreads();
+    // merged sums: a thread has two neighbouring elements of a record's 128 + 1024 values
+    constexpr int PAIRS = (128 + KD) / 2;
+    for (int i = tid; i < g * PAIRS; i += MERGE_THREADS) {
+        const int a = i / PAIRS, e = (i - a * PAIRS) * 2;
+        const float* src = rec0 + (size_t)a * REC + 2 + e;
+        float v0 = 0.f, v1 = 0.f;
+        for (int s0 = 0; s0 < n_splits; s0 += 8) {
+            float2 x[8];
+#pragma unroll
+            for (int k = 0; k < 8; ++k) x[k] = *reinterpret_cast<const float2*>(src + (size_t)min(s0 + k, n_splits - 1) * g * REC);   // always a valid record
+#pragma unroll
+            for (int k = 0; k < 8; ++k) {
+                const float f = s0 + k < n_splits ? fs[a][s0 + k] : 0.f;
+                v0 = fmaf(f, x[k].x, v0);
+                v1 = fmaf(f, x[k].y, v1);
+            }
+        }
+        if (e < 128) { accv[a][e] = v0; accv[a][e + 1] = v1; }
+        else {
+            const uint32_t hi = dbf::pack_bf16(v0, v1);
+            *reinterpret_cast<uint32_t*>(&akh[a][e - 128]) = hi;
+            *reinterpret_cast<uint32_t*>(&akl[a][e - 128]) = dbf::pack_bf16(v0 - __uint_as_float(hi << 16), v1 - __uint_as_float(hi & 0xffff0000u));
+        }
+    }
+    __syncthreads();
+    // rows 16 (wid % 8) .. of the head's block of the map times the key sums of four input heads
+    {
+        const int half = wid >> 3, r0 = 16 * (wid & 7) + row;
+        const uint4* Wr0 = reinterpret_cast<const uint4*>(W + ((size_t)layer * KD + (size_t)h * 128 + r0) * KD);
+        const uint4* Wr1 = Wr0 + 8 * (KD / 8);                 // row + 8
+        float d[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll 2
+        for (int kc = half * (HKV / 2); kc < (half + 1) * (HKV / 2); ++kc) {                     // 128 columns a time: 16 pieces of 16 bytes per row
+            uint4 A[8];
+#pragma unroll
+            for (int jj = 0; jj < 4; ++jj) {
+                A[2 * jj + 0] = Wr0[kc * 16 + quarter + 4 * jj];
+                A[2 * jj + 1] = Wr1[kc * 16 + quarter + 4 * jj];
+            }
+#pragma unroll
+            for (int jj = 0; jj < 4; ++jj) {
+                const uint4 a0 = A[2 * jj], a1 = A[2 * jj + 1];
+                const int col = kc * 128 + 8 * (quarter + 4 * jj);
+                const uint4 bh = *reinterpret_cast<const uint4*>(&akh[row][col]);      // B column = head `row`
+                const uint4 bl = *reinterpret_cast<const uint4*>(&akl[row][col]);
+                dbf::mma_16(d, a0.x, a1.x, a0.y, a1.y, bh.x, bh.y);
+                dbf::mma_16(d, a0.x, a1.x, a0.y, a1.y, bl.x, bl.y);
+                dbf::mma_16(d, a0.z, a1.z, a0.w, a1.w, bh.z, bh.w);
+                dbf::mma_16(d, a0.z, a1.z, a0.w, a1.w, bl.z, bl.w);
+            }
+        }
+        // d[0], d[1]: row `row`, heads 2 quarter and 2 quarter + 1; d[2], d[3]: row `row` + 8
+        if (2 * quarter < g) { pw[half][2 * quarter][r0] = d[0]; pw[half][2 * quarter][r0 + 8] = d[2]; }
+        if (2 * quarter + 1 < g) { pw[half][2 * quarter + 1][r0] = d[1]; pw[half][2 * quarter + 1][r0 + 8] = d[3]; }
+    }
+    __syncthreads();
+    for (int i = tid; i < g * 128; i += MERGE_THREADS) {
+        const int a = i >> 7, c = i & 127;
+        store_out(out + ((size_t)u * g + a) * 128 + c, (accv[a][c] + (pw[0][a][c] + pw[1][a][c])) / Ls[a]);
+    }
+}
+
+// The same for many units: a block takes `seqs` sequences of one (layer, head), whose query heads are the product's columns.  The
+// map's rows, 256 KB a block, are what most of a merge fetches from L2 where units are many and their records few.  A kernel of its
+// own: as a variant of the other one it cost that one 1 to 7 % (six pairs of 2215 rows, 25.5 us a step).
+// grid (layers * HKV * ceil(batch / seqs)), 512 threads, seqs * g <= 8.
+template <typename TO>
+__global__ void __launch_bounds__(MERGE_THREADS)
+decode_layer_merge_shared(const float* __restrict__ partial, const __nv_bfloat16* __restrict__ W, int L, int g, int batch, int seqs, Plan pl,
                        TO* __restrict__ out) {
     constexpr int KD = HKV * 128;
     __shared__ __align__(16) __nv_bfloat16 akh[8][KD], akl[8][KD];          // 32 KB
@@ -400,15 +493,14 @@ decode_layer_merge_mma(const float* __restrict__ partial, const __nv_bfloat16* _
     __shared__ int splits[8];                            // records of a sequence
     const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
     const int h = blockIdx.x % HKV, layer = (blockIdx.x / HKV) % L, b0 = blockIdx.x / (HKV * L) * seqs;
-    const int n_heads = SHARED ? min(seqs, batch - b0) * g : g;          // columns in use: sequence b0 + a / g, query head a % g
+    const int n_heads = min(seqs, batch - b0) * g;       // columns in use: sequence b0 + a / g, query head a % g
     const int row = lane >> 2, quarter = lane & 3;
-    auto pair_of = [&](int a) { return (b0 + (SHARED ? a / g : 0)) * L + layer; };
-    auto records_of = [&](int a) { return partial + (((size_t)pair_of(a) * HKV + h) * pl.s_max * g + (SHARED ? a % g : a)) * REC; };      // g * REC apart
+    auto pair_of = [&](int a) { return (b0 + a / g) * L + layer; };
+    auto records_of = [&](int a) { return partial + (((size_t)pair_of(a) * HKV + h) * pl.s_max * g + a % g) * REC; };      // g * REC apart
     auto splits_of = [&](int a) {
         const long long c0 = (long long)pair_of(a) * pl.weight;
         return block_of_cost(c0 + pl.weight - 1, pl) - block_of_cost(c0, pl) + 1;
     };
-    const int splits0 = SHARED ? 0 : splits_of(0);
     for (int i = tid; i < (8 - n_heads) * KD; i += MERGE_THREADS) {      // columns of B beyond them
         akh[n_heads + i / KD][i % KD] = __float2bfloat16_rn(0.f);
         akl[n_heads + i / KD][i % KD] = __float2bfloat16_rn(0.f);
@@ -416,7 +508,7 @@ decode_layer_merge_mma(const float* __restrict__ partial, const __nv_bfloat16* _
     asm volatile("griddepcontrol.wait;\n" ::: "memory");                 // the streaming kernel's records
     // factors of the splits: warp a < n_heads takes column a
     if (wid < n_heads) {
-        const int n_splits = SHARED ? splits_of(wid) : splits0;
+        const int n_splits = splits_of(wid);
         const float* rec = records_of(wid) + (size_t)lane * g * REC;
         const float mj = lane < n_splits ? rec[0] : -INFINITY;
         const float lj = lane < n_splits ? rec[1] : 0.f;
@@ -424,13 +516,13 @@ decode_layer_merge_mma(const float* __restrict__ partial, const __nv_bfloat16* _
         const float f = mj > -INFINITY ? __expf(mj - M) : 0.f;
         fs[wid][lane] = f;
         const float Lsum = warp_sum(f * lj);
-        if (lane == 0) { Ls[wid] = Lsum; if (SHARED) splits[wid] = n_splits; }
+        if (lane == 0) { Ls[wid] = Lsum; splits[wid] = n_splits; }
     }
     __syncthreads();
     // merged sums: a thread has two neighbouring elements of a record's 128 + 1024 values
     constexpr int PAIRS = (128 + KD) / 2;
     for (int i = tid; i < n_heads * PAIRS; i += MERGE_THREADS) {
-        const int a = i / PAIRS, e = (i - a * PAIRS) * 2, n_splits = SHARED ? splits[a] : splits0;
+        const int a = i / PAIRS, e = (i - a * PAIRS) * 2, n_splits = splits[a];
         const float* src = records_of(a) + 2 + e;
         float v0 = 0.f, v1 = 0.f;
         for (int s0 = 0; s0 < n_splits; s0 += 8) {
@@ -485,7 +577,7 @@ decode_layer_merge_mma(const float* __restrict__ partial, const __nv_bfloat16* _
     __syncthreads();
     for (int i = tid; i < n_heads * 128; i += MERGE_THREADS) {
         const int a = i >> 7, c = i & 127;
-        store_out(out + (((size_t)pair_of(a) * HKV + h) * g + (SHARED ? a % g : a)) * 128 + c, (accv[a][c] + (pw[0][a][c] + pw[1][a][c])) / Ls[a]);
+        store_out(out + (((size_t)pair_of(a) * HKV + h) * g + a % g) * 128 + c, (accv[a][c] + (pw[0][a][c] + pw[1][a][c])) / Ls[a]);
     }
 }
 
