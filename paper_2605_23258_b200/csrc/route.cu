@@ -15,14 +15,11 @@ namespace vec {
 
 using sel::Layout;
 
-// Inputs of up to 32768 elements are held in registers, by 16 warps up to half of that (32 registers a thread are what 64 of them
-// leave room for).  Step 1 with two passes over memory and in registers, us: 16 lists of 3968 elements 14.3 / 5.5, of 16384
-// 15.3 / 13.6, 128 of 3804 10.5 / 6.1, 256 of 20011 28.0 / 27.7, of 32768 36.9 / 37.5.  Longer ones: blocks of 32 warps (one
-// resident per multiprocessor, masks and list in up to 200 KB) beyond a quarter of a million elements, of 16 warps (two resident)
-// below.
+// Forms of a selection: the input in registers (select_regs), or two passes over it in memory (select.cuh) by blocks of 8 warps (four
+// resident per multiprocessor), of 16 (two) or of 32 (one, with masks and list in up to 200 KB) warps.
 constexpr int SEL_REGS16 = 16384, SEL_REGS = 32768, SEL_LONG = 262144;
-constexpr size_t SEL_SMEM_LONG = 200 * 1024, SEL_SMEM_MID = 92 * 1024;
-#define VEC_SEL_BOUNDS(NW) __launch_bounds__(32 * NW, NW == 32 ? 1 : 2)
+constexpr size_t SEL_SMEM_LONG = 200 * 1024, SEL_SMEM_MID = 92 * 1024, SEL_SMEM_SHORT = 36 * 1024;
+#define VEC_SEL_BOUNDS(NW) __launch_bounds__(32 * NW, NW == 32 ? 1 : NW == 16 ? 2 : 4)
 
 // The general selection (select_emit) as functions of their own: the kernels run the lean path inline and
 // come here only when it gives up, so its registers are not theirs to carry.
@@ -336,22 +333,42 @@ static vector_status select_kernels_setup() {
     if (!once.first()) return VECTOR_OK;
     cudaError_t e = cudaFuncSetAttribute(pool_select_kernel<32>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SEL_SMEM_LONG);
     if (e == cudaSuccess) e = cudaFuncSetAttribute(pool_select_kernel<16>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SEL_SMEM_MID);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(pool_select_kernel<8>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SEL_SMEM_SHORT);
     if (e == cudaSuccess) e = cudaFuncSetAttribute(truncate_kernel<32>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SEL_SMEM_LONG);
     if (e == cudaSuccess) e = cudaFuncSetAttribute(truncate_kernel<16>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SEL_SMEM_MID);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(truncate_kernel<8>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SEL_SMEM_SHORT);
     if (e != cudaSuccess) { once.undo(); VEC_CUDA_CHECK(e); }
     return VECTOR_OK;
 }
 
-// Block size and shared-memory layout of selections over n > SEL_REGS elements each.
-struct SelPlan { int nw; Layout L; };
-static SelPlan plan_selection(int64_t n) {
-    SelPlan p;
-    const size_t budget = n < SEL_LONG ? SEL_SMEM_MID : SEL_SMEM_LONG;
-    const int min_cand = 2048;
-    p.nw = n < SEL_LONG ? 16 : 32;
-    p.L = sel::plan_layout(n, false, budget, min_cand, p.nw);
-    if (!p.L.keyed) p.L = sel::plan_layout(n, true, budget, min_cand, p.nw);       // the general path stages the images
-    return p;
+// Warps of a block that passes over memory, 0: the input in registers.  U lists of n elements.  Up to 8192 elements registers win by
+// up to twice, beyond that only where every list has a multiprocessor to itself (one block fills its register file); many lists are
+// served best by the small blocks, whose phases of latency overlap, until their share of shared memory gets short.  us, registers /
+// 8 warps / 16 warps.  Step 1: 2368 lists of 3000 elements 41 / 41 / 66; 444 of 6500 14.4 / 14.5 / 18.8, 592 of 6500 17.0 / 14.8 /
+// 21.2; 148 of 12000 10.6 / 13.6 / 10.9, 296 of 12000 15.0 / 15.8 / 14.1, 592 of 12000 27.7 / 21.3 / 26.3, 1184 of 14000 57 / 70 / 62,
+// 148 of 20011 13.8 / 23.8 / 16.4, 296 of 20011 26.5 / 32.4 / 21.7, 1184 of 20011 109 / 109 / 99.  Step 3: 2368 lists of 8192 108 /
+// 111 / 135; 148 of 12000 12.8 / 21.9 / 16.1, 296 of 12000 24.5 / 25.9 / 22.4, 592 of 12000 49 / 41 / 45, 1184 of 16384 126 / 107 /
+// 113; 148 of 20011 in 64 registers a thread, which do not hold image and token, 41.9 / 35.0 / 25.3; 888 of 20011 - / 125 / 118, 1184
+// of 20011 - / 149 / 155, of 26000 - / 179 / 177.
+static int selection_warps(int64_t n, int U, bool step3) {
+    const int sms = sm_count();
+    if (n <= (step3 ? 8192 : 4096)) return 0;
+    if (n <= 8192) return U <= 3 * sms ? 0 : 8;
+    if (n <= SEL_REGS16) {
+        if (U <= sms) return 0;
+        if (U <= 2 * sms) return 16;
+        if (step3 || n <= 12288) return 8;
+        return U <= 4 * sms ? 16 : 0;
+    }
+    if (!step3 && n <= SEL_REGS && U <= sms) return 0;
+    if (step3 && n <= 24576 && U >= 8 * sms) return 8;
+    return n < SEL_LONG ? 16 : 32;
+}
+static Layout selection_layout(int64_t n, int nw) {
+    const size_t budget = nw == 8 ? SEL_SMEM_SHORT : nw == 16 ? SEL_SMEM_MID : SEL_SMEM_LONG;
+    const int min_cand = nw == 8 ? 1024 : 2048;
+    const Layout L = sel::plan_layout(n, false, budget, min_cand, nw);
+    return L.keyed ? L : sel::plan_layout(n, true, budget, min_cand, nw);       // the general path stages the images
 }
 
 static vector_status launch_pool_select(const Dims& dm, const vector_budget* budget, const float* scores, int32_t* pool,
@@ -359,21 +376,17 @@ static vector_status launch_pool_select(const Dims& dm, const vector_budget* bud
     vector_status rc = select_kernels_setup();
     if (rc != VECTOR_OK) return rc;
     const int64_t n = budget->n_tokens;
-    if (n <= SEL_REGS) {
+    const int nw = selection_warps(n, dm.U, false);
+    if (nw == 0) {
         auto kern = n <= 2048 ? pool_select_regs<16, 4> : n <= 4096 ? pool_select_regs<16, 8> : n <= 8192 ? pool_select_regs<16, 16>
                   : n <= SEL_REGS16 ? pool_select_regs<16, 32> : pool_select_regs<32, 32>;
         VEC_CUDA_CHECK(launch_maybe_dependent(true, kern, dim3(dm.U), dim3(n <= SEL_REGS16 ? 512 : 1024), 0, st, scores, n,
                                               (int)budget->n_pool, pool, zero));
         return VECTOR_OK;
     }
-    const SelPlan p = plan_selection(n);
-    const Layout L = p.L;
-#define VEC_POOL(NW)                                                                                                     \
-    VEC_CUDA_CHECK(launch_maybe_dependent(true, pool_select_kernel<NW>, dim3(dm.U), dim3(32 * NW), L.bytes(), st, scores, n, \
-                                          (int)budget->n_pool, pool, zero, L))
-    if (p.nw == 16) VEC_POOL(16);
-    else VEC_POOL(32);
-#undef VEC_POOL
+    const Layout L = selection_layout(n, nw);
+    auto kern = nw == 8 ? pool_select_kernel<8> : nw == 16 ? pool_select_kernel<16> : pool_select_kernel<32>;
+    VEC_CUDA_CHECK(launch_maybe_dependent(true, kern, dim3(dm.U), dim3(32 * nw), L.bytes(), st, scores, n, (int)budget->n_pool, pool, zero, L));
     return VECTOR_OK;
 }
 
@@ -384,22 +397,18 @@ static vector_status launch_truncate(const Dims& dm, const vector_budget* budget
     if (rc != VECTOR_OK) return rc;
     // dependent: may start (and clear the tier map) while the kernel before it in the stream drains
     const int64_t n = budget->n_pool;
-    if (n <= SEL_REGS) {
+    const int nw = selection_warps(n, dm.U, true);
+    if (nw == 0) {
         auto kern = n <= 2048 ? truncate_regs<16, 4> : n <= 4096 ? truncate_regs<16, 8> : n <= 8192 ? truncate_regs<16, 16>
-                  : n <= SEL_REGS16 ? truncate_regs<32, 16> : truncate_regs<32, 32>;
+                  : truncate_regs<32, 16>;
         VEC_CUDA_CHECK(launch_maybe_dependent(dependent, kern, dim3(dm.U), dim3(n <= 8192 ? 512 : 1024), 0, st, eps, pool,
                                               (int64_t)budget->n_tokens, (int)n, (int)budget->n_apx, tier, ret_idx, apx_idx));
         return VECTOR_OK;
     }
-    const SelPlan p = plan_selection(n);
-    const Layout L = p.L;
-#define VEC_TRUNC(NW)                                                                                                   \
-    VEC_CUDA_CHECK(launch_maybe_dependent(dependent, truncate_kernel<NW>, dim3(dm.U), dim3(32 * NW), L.bytes(), st, eps, \
-                                          pool, (int64_t)budget->n_tokens, (int)budget->n_pool, (int)budget->n_apx, tier, \
-                                          ret_idx, apx_idx, L))
-    if (p.nw == 16) VEC_TRUNC(16);
-    else VEC_TRUNC(32);
-#undef VEC_TRUNC
+    const Layout L = selection_layout(n, nw);
+    auto kern = nw == 8 ? truncate_kernel<8> : nw == 16 ? truncate_kernel<16> : truncate_kernel<32>;
+    VEC_CUDA_CHECK(launch_maybe_dependent(dependent, kern, dim3(dm.U), dim3(32 * nw), L.bytes(), st, eps, pool, (int64_t)budget->n_tokens,
+                                          (int)n, (int)budget->n_apx, tier, ret_idx, apx_idx, L));
     return VECTOR_OK;
 }
 

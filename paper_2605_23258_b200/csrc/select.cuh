@@ -2,8 +2,8 @@
 // building block of Step 1 (the n_pool largest scores) and Step 3 (the n_apx smallest
 // residuals) of the routing (paper Section 3.2).  One thread block per unit.
 //
-// The k-th key is found on an order-preserving 32-bit image of the fp32 value.  Inputs of up to 32768 elements stay in
-// registers (select_regs, at the end of this file).  Longer ones have two paths:
+// The k-th key is found on an order-preserving 32-bit image of the fp32 value.  Short inputs, and medium ones where lists are few,
+// stay in registers (select_regs, at the end of this file; the rule is in route.cu).  The others have two paths:
 //
 // select_lean (the one that normally runs): a histogram of the leading 11 bits over the whole input;
 //   one more pass that writes, per 32 elements, a bit mask of the elements whose leading bits beat the

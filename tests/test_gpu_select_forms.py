@@ -1,0 +1,68 @@
+"""Selections where the form changes with the number of lists as well as their length: exact in every list (indices and tiers are whole
+numbers), against a stable sort.  And Step 3 just past the lengths that registers hold: 22 % more elements took 2.6 times as long
+when their images and tokens were kept in registers that were not there; passing over memory it is 1.4 times."""
+import pytest
+import torch
+
+import paper_2605_23258_b200 as vec
+
+pytestmark = pytest.mark.gpu
+DEV = "cuda"
+
+
+def _lists(share, n, ties):
+    U = int(share * torch.cuda.get_device_properties(0).multi_processor_count) + 1
+    gen = torch.Generator(device=DEV).manual_seed(n)
+    v = torch.rand(U, n, generator=gen, device=DEV) ** 4
+    if ties:
+        v = torch.round(v * 64) / 64
+    return U, v
+
+
+@pytest.mark.parametrize("ties", [False, True])
+@pytest.mark.parametrize("share,n", [(0.9, 16384), (0.9, 16385), (0.9, 32768), (1, 8192), (1, 8193), (1, 16385), (2, 12288), (2, 12289), (3, 4096), (3, 4097),
+                                     (3, 8192), (3, 16384), (4, 12289), (4, 16384), (8, 4097), (8, 8193), (8, 16385), (8, 24576), (8, 24577)])
+def test_forms(share, n, ties):
+    U, v = _lists(share, n, ties)
+    sh = vec.Shape(1, 1, U, U, 64, vec.VECTOR_F32, 1)
+    k = n // 3 * 2
+    out = torch.empty(U, k, dtype=torch.int32, device=DEV)
+    vec.vector_pool_select(sh, vec.Budget(n, k, 0, k, 0, k, n - k), v, out)
+    want = torch.sort(v, dim=1, descending=True, stable=True).indices[:, :k].sort(dim=1).values
+    assert torch.equal(out.long(), want)
+    N = n + 37
+    pool = (torch.arange(n, device=DEV) + (torch.arange(n, device=DEV) >= n // 2) * 37).to(torch.int32).repeat(U, 1).contiguous()
+    tier = torch.empty(U, N, dtype=torch.uint8, device=DEV)
+    ret, apx = (torch.empty(U, m, dtype=torch.int32, device=DEV) for m in (n - k, k))
+    vec.vector_truncate(sh, vec.Budget(N, n - k // 2, k // 2, n, k, n - k, N - n), v, pool, tier, ret, apx)
+    order = torch.sort(v, dim=1, stable=True).indices
+    places = (order[:, k:].sort(dim=1).values, order[:, :k].sort(dim=1).values)
+    want_tier = torch.zeros_like(tier)
+    for got, at, t in ((ret, places[0], 2), (apx, places[1], 1)):
+        tokens = torch.gather(pool.long(), 1, at)
+        assert torch.equal(got.long(), tokens)
+        want_tier.scatter_(1, tokens, t)
+    assert torch.equal(tier, want_tier)
+
+
+def test_step3_past_the_registers():
+    us = []
+    for n in (16384, 20011):
+        U, v = _lists(8, n, False)
+        sh = vec.Shape(1, 1, U, U, 64, vec.VECTOR_F32, 1)
+        k = n // 4 * 2
+        pool = torch.arange(n, dtype=torch.int32, device=DEV).repeat(U, 1).contiguous()
+        tier = torch.empty(U, n, dtype=torch.uint8, device=DEV)
+        ret, apx = (torch.empty(U, m, dtype=torch.int32, device=DEV) for m in (n - k, k))
+        b = vec.Budget(n, n - k // 2, k // 2, n, k, n - k, 0)
+        times = []
+        for _ in range(12):
+            a, e = (torch.cuda.Event(enable_timing=True) for _ in range(2))
+            a.record()
+            for _ in range(5):
+                vec.vector_truncate(sh, b, v, pool, tier, ret, apx)
+            e.record()
+            torch.cuda.synchronize()
+            times.append(a.elapsed_time(e))
+        us.append(min(times))
+    assert us[1] < 2 * us[0], us
