@@ -493,9 +493,12 @@ static vector_status residual_layer_dispatch(const Dims& dm, int Hkv, int L, con
             x.groups = (int)(x.tiles >= places ? places : 2 * x.tiles <= places && P.pairs > 1 ? 2 * x.tiles : x.tiles);
             x.items = (x.tiles * P.pairs + x.groups - 1) / x.groups;
         }
-        // An item takes a pair 8.0 us and a block 9.4 (16 layers of 4914 tokens, 8 heads: 142 against 161 us); rounded to 256,
-        // a short list costs the pairs more items.
-        const bool pair = 20 * split[1].items <= 23 * split[0].items;
+        // us: a pair of blocks takes Hkv items + 2, the 2 for a cluster's start and a stage's first fill by one warp, a block by itself 1.175
+        // Hkv items; rounded to 256, a short list costs the pairs more items.  A call of pairs / blocks: 16 layers of 5000 tokens, 8 heads 150 /
+        // 169, 4 heads 51 / 55, 3 heads 41 / 46; one layer of 300 tokens, 4 heads 14.0 / 12.6, 3 heads 13.1 / 11.9, one head 10.5 / 8.5; 37
+        // layers of 700 tokens, 3 heads 18.0 / 17.8.  One and two heads leave the second block's half of the map short: 16 layers of 5000
+        // tokens, one head 16.7 / 15.1, two heads 27.4 / 26.3.
+        const bool pair = Hkv > 2 && 40 * Hkv * split[1].items + 80 <= 47 * Hkv * split[0].items;
         P.tpu = split[pair].tpu;
         P.n_items = split[pair].tiles * P.pairs;
         const int blocks = split[pair].groups * (pair ? 2 : 1);
