@@ -16,7 +16,7 @@ namespace vec {
 
 constexpr int ST = 64;    // tile edge (rows and keys) of the CUDA-core score kernels
 
-// The CUDA-core passes hold a whole 64 x D tile of each operand in shared memory (rows D + 1 apart) and request the next
+// The CUDA-core passes hold a whole 64 x D tile of each operand in shared memory (rows PITCH<D> apart) and request the next
 // tile of the one that changes before they work on this one: with 32-channel slices loaded between barriers a pass was a
 // chain of load latencies (13 + 11 us for 2 units of 64 rows and 1024 keys).
 template <int D> struct TileRegs { float4 v[ST * D / 1024]; };
@@ -45,15 +45,16 @@ __device__ __forceinline__ void tile_store(const TileRegs<D>& t, float* dst) {
         *reinterpret_cast<float4*>(dst + r * PITCH<D> + c) = t.v[e];
     }
 }
-// acc[i][j] = sum_c Qs[ty + 16 i][c] * Ks[tx + 16 j][c].  Reads of shared memory are what bounds it: four channels a load.
-template <int D>
+// acc[i][j] = sum_c Qs[ty + 16 i][c] * Ks[tx + 16 j][c].  Reads of shared memory are what bounds it: four channels a load, UNROLL loads
+// of each row under way.
+template <int D, int UNROLL>
 __device__ __forceinline__ void tile_qk(const float* Qs, const float* Ks, float acc[4][4]) {
     const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
 #pragma unroll
     for (int i = 0; i < 4; ++i)
 #pragma unroll
         for (int j = 0; j < 4; ++j) acc[i][j] = 0.f;
-#pragma unroll 4
+#pragma unroll (UNROLL)
     for (int kk = 0; kk < D; kk += 4) {
         float4 a[4], b[4];
 #pragma unroll
@@ -71,11 +72,16 @@ __device__ __forceinline__ void tile_qk(const float* Qs, const float* Ks, float 
             }
     }
 }
+// Blocks that outnumber four a multiprocessor (MANY, 64 channels): three resident at 80 registers instead of two at 114 to 127, which
+// unroll the channels.  us, MANY / not: 148 units of 32 rows and 300 keys 35 / 39, 32 of 2000 keys 48 / 52; few blocks, 8 units of 2000 keys
+// 21 / 16, one unit of 256 rows and 32768 keys 111 / 91.  At 128 channels two blocks are resident either way.
+template <bool MANY> constexpr int MIN_BLOCKS = MANY ? 3 : 2;
+template <int D> static bool many_blocks(int64_t blocks) { return D == 64 && blocks > 4 * (int64_t)sm_count(); }
 template <int D> constexpr int tile_smem() { return 2 * ST * PITCH<D> * (int)sizeof(float); }
 
 // grid (n_chunks, row_tiles, U), 256 threads, tile_smem of dynamic shared memory
-template <typename T, int D, bool WIDE>
-__global__ void __launch_bounds__(256)
+template <typename T, int D, bool WIDE, bool MANY>
+__global__ void __launch_bounds__(256, MIN_BLOCKS<MANY>)
 score_pass1_generic(const T* __restrict__ Q, const T* __restrict__ K, int64_t N, int R, int w,
                     float scale, int64_t chunk_len, float2* __restrict__ partial) {
     extern __shared__ __align__(16) float tiles[];
@@ -110,7 +116,7 @@ score_pass1_generic(const T* __restrict__ Q, const T* __restrict__ K, int64_t N,
         __syncthreads();
         if (key0 + ST < k_end) tile_request<WIDE>(Ku, key0 + ST, k_end, next);
         float acc[4][4];
-        tile_qk<D>(Qs, Ks, acc);
+        tile_qk<D, MANY ? 1 : 4>(Qs, Ks, acc);
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
             float s[4], mx = m[i];
@@ -183,8 +189,8 @@ score_lse_rows(const float2* __restrict__ partial, int R, int n_chunks, float* _
 // grid (key_tiles, U), 256 threads, tile_smem of dynamic shared memory.  INLINE_LSE: a block forms the normalisers of its
 // rows itself from the chunk partials (a launch less; every key tile repeats it).  POOLED: the block pools its sums itself (another
 // launch less); its tiles overlap by the pooling radius on both sides, raw may be null.
-template <typename T, int D, bool INLINE_LSE, bool WIDE, bool POOLED>
-__global__ void __launch_bounds__(256)
+template <typename T, int D, bool INLINE_LSE, bool WIDE, bool POOLED, bool MANY>
+__global__ void __launch_bounds__(256, MIN_BLOCKS<MANY>)
 score_pass2_generic(const T* __restrict__ Q, const T* __restrict__ K, int64_t N, int R, int w,
                     float scale, const float2* __restrict__ partial, int n_chunks, const float* __restrict__ lse,
                     float* __restrict__ raw, int r, float* __restrict__ score) {
@@ -219,7 +225,7 @@ score_pass2_generic(const T* __restrict__ Q, const T* __restrict__ K, int64_t N,
         __syncthreads();
         if (row0 + ST < R) tile_request<WIDE>(Qu, row0 + ST, R, next);
         float acc[4][4];
-        tile_qk<D>(Qs, Ks, acc);
+        tile_qk<D, MANY ? 1 : 4>(Qs, Ks, acc);
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
             int row = row0 + ty + 16 * i;
@@ -285,12 +291,17 @@ static vector_status launch_score(const Dims& dm, const void* Q_, const void* K_
                                   size_t ws_bytes, cudaStream_t st) {
     constexpr int SMEM = tile_smem<D>();
     const T *Q = (const T*)Q_, *K = (const T*)K_;
+    constexpr bool M = D == 64;              // the kernels for many blocks, where there are such
     static PerDeviceOnce once;
     if (once.first()) {
-        cudaError_t e = cudaFuncSetAttribute(score_pass1_generic<T, D, WIDE>, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM);
-        if (e == cudaSuccess) e = cudaFuncSetAttribute(score_pass2_generic<T, D, true, WIDE, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM);
-        if (e == cudaSuccess) e = cudaFuncSetAttribute(score_pass2_generic<T, D, true, WIDE, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM);
-        if (e == cudaSuccess) e = cudaFuncSetAttribute(score_pass2_generic<T, D, false, WIDE, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM);
+        auto opt_in = [](auto kern) { return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM); };
+        cudaError_t e = opt_in(score_pass1_generic<T, D, WIDE, false>);
+        if (e == cudaSuccess) e = opt_in(score_pass1_generic<T, D, WIDE, M>);
+        if (e == cudaSuccess) e = opt_in(score_pass2_generic<T, D, true, WIDE, true, false>);
+        if (e == cudaSuccess) e = opt_in(score_pass2_generic<T, D, true, WIDE, false, false>);
+        if (e == cudaSuccess) e = opt_in(score_pass2_generic<T, D, true, WIDE, false, M>);
+        if (e == cudaSuccess) e = opt_in(score_pass2_generic<T, D, false, WIDE, false, false>);
+        if (e == cudaSuccess) e = opt_in(score_pass2_generic<T, D, false, WIDE, false, M>);
         if (e != cudaSuccess) { once.undo(); VEC_CUDA_CHECK(e); }
     }
     const size_t lse_b = align256((size_t)dm.U * dm.R * sizeof(float)), raw_b = raw_out ? 0 : align256((size_t)dm.U * (size_t)N * sizeof(float));
@@ -304,8 +315,9 @@ static vector_status launch_score(const Dims& dm, const void* Q_, const void* K_
     chunk_len = (chunk_len + ST - 1) / ST * ST;
     n_chunks = (int)((N + chunk_len - 1) / chunk_len);            // none empty
     const int row_tiles = (dm.R + ST - 1) / ST;
-    VEC_CUDA_CHECK(launch_maybe_dependent(true, score_pass1_generic<T, D, WIDE>, dim3(n_chunks, row_tiles, dm.U), dim3(256), SMEM, st, Q, K, N,
-                                          dm.R, dm.w, dm.scale, chunk_len, partial));
+    auto pass1 = many_blocks<D>((int64_t)n_chunks * row_tiles * dm.U) ? score_pass1_generic<T, D, WIDE, M> : score_pass1_generic<T, D, WIDE, false>;
+    VEC_CUDA_CHECK(launch_maybe_dependent(true, pass1, dim3(n_chunks, row_tiles, dm.U), dim3(256), SMEM, st, Q, K, N, dm.R, dm.w, dm.scale,
+                                          chunk_len, partial));
     // the partials of a row tile: no more than the rows' own elements
     const bool inline_lse = n_chunks <= 32;
     if (!inline_lse)
@@ -315,12 +327,15 @@ static vector_status launch_score(const Dims& dm, const void* Q_, const void* K_
     const int r = dm.pool_kernel / 2;
     const int64_t tiles_pooled = (N + ST - 2 * r - 1) / (ST - 2 * r);
     if (inline_lse && tiles_pooled * dm.U <= sm_count()) {
-        VEC_CUDA_CHECK(launch_maybe_dependent(true, score_pass2_generic<T, D, true, WIDE, true>, dim3((unsigned)tiles_pooled, dm.U), dim3(256), SMEM, st,
+        VEC_CUDA_CHECK(launch_maybe_dependent(true, score_pass2_generic<T, D, true, WIDE, true, false>, dim3((unsigned)tiles_pooled, dm.U), dim3(256), SMEM, st,
                                               Q, K, N, dm.R, dm.w, dm.scale, partial, n_chunks, lse, raw_out, r, scores));
         return VECTOR_OK;
     }
-    VEC_CUDA_CHECK(launch_maybe_dependent(true, inline_lse ? score_pass2_generic<T, D, true, WIDE, false> : score_pass2_generic<T, D, false, WIDE, false>,
-                                          dim3((unsigned)((N + ST - 1) / ST), dm.U), dim3(256), SMEM, st, Q, K, N, dm.R, dm.w, dm.scale,
+    const int64_t tiles = (N + ST - 1) / ST;
+    auto pass2 = many_blocks<D>(tiles * dm.U)
+                     ? (inline_lse ? score_pass2_generic<T, D, true, WIDE, false, M> : score_pass2_generic<T, D, false, WIDE, false, M>)
+                     : (inline_lse ? score_pass2_generic<T, D, true, WIDE, false, false> : score_pass2_generic<T, D, false, WIDE, false, false>);
+    VEC_CUDA_CHECK(launch_maybe_dependent(true, pass2, dim3((unsigned)tiles, dm.U), dim3(256), SMEM, st, Q, K, N, dm.R, dm.w, dm.scale,
                                           partial, n_chunks, lse, raw, r, scores));
     int64_t total = (int64_t)dm.U * N;
     VEC_CUDA_CHECK(launch_maybe_dependent(true, score_pool_kernel, dim3((unsigned)((total + 255) / 256)), dim3(256), 0, st, raw, N, dm.w,

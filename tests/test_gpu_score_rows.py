@@ -32,3 +32,27 @@ def test_score(oracle, units, d, g, w, N, pool):
         for got, want in ((raw[u], raw_o), (scores[u], sc_o)):
             ok, worst = score_close(got.cpu().numpy()[None], want[None], g * w)
             assert ok, (u, worst)
+
+
+@pytest.mark.parametrize("units,d,g,w,N,pool", [
+    (1, 64, 1, 16, 65, 1), (2, 64, 2, 3, 64 - 14 + 1, 15), (2, 128, 1, 2, 2 * (64 - 14) + 1, 15), (1, 128, 3, 1, 1, 15), (1, 64, 1, 5, 6, 15),
+    (2, 128, 4, 32, 2 * (64 - 6) + 1, 7), (1, 128, 2, 50, 58, 7), (1, 64, 5, 20, 20, 15), (1, 64, 2, 40, 2047, 1),
+    (150, 64, 1, 32, 300, 7), (130, 64, 5, 16, 300, 15), (40, 64, 1, 70, 1100, 1), (2, 64, 8, 100, 4000, 5), (150, 128, 1, 32, 290, 7)])
+def test_score_fp32(oracle, units, d, g, w, N, pool):
+    """fp32 on CUDA cores: lengths that end one key into a tile, windows narrower than the pooling radius, pools of one key; so few tiles
+    that the second pass pools them, and more blocks than four a multiprocessor.  Raw sums asked for or not."""
+    gen = torch.Generator(device=DEV).manual_seed(d + g + w + N)
+    K = torch.randn(units, N, d, generator=gen, device=DEV)
+    Q = torch.randn(units, g, w, d, generator=gen, device=DEV) * 2
+    sh = vec.Shape(1, units, g, 1, d, vec.VECTOR_F32, w, pool)
+    ws = vec.alloc_workspace(sh, vec.vector_plan_budget(N, N, 0, w))
+    scores, raw, again = (torch.full((units, N), float("nan"), device=DEV) for _ in range(3))
+    vec.vector_score(sh, Q, K, N, scores, raw, ws)
+    vec.vector_score(sh, Q, K, N, again, None, ws)
+    torch.cuda.synchronize()
+    assert torch.equal(scores, again)
+    for u in sorted({0, units // 2, units - 1}):
+        raw_o, sc_o = oracle.score(Q[u].cpu(), K[u].cpu(), d ** -0.5, pool)
+        for got, want in ((raw[u], raw_o), (scores[u], sc_o)):
+            ok, worst = score_close(got.cpu().numpy()[None], want[None], g * w)
+            assert ok, (u, worst)
