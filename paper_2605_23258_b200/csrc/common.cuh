@@ -72,7 +72,9 @@ __device__ __forceinline__ void rope_fill_inv_freq(double* inv_freq, int d, floa
 // executed griddepcontrol.launch_dependents, or exited); it must execute griddepcontrol.wait before
 // it touches anything that kernel reads or writes.  Every kernel here lets its dependents start only behind its own wait, so what
 // came before its primary has finished when a dependent starts, along whole chains and across calls: ahead of its wait a
-// kernel may touch what its primary does not.  cluster > 1: thread block clusters of that size.
+// kernel may touch what its primary does not.  What it reads behind the wait reaches it through pointers that are not both const and
+// __restrict__, and not through __ldg or ld.global.nc: the compiler takes those for data that nobody writes while the kernel runs, and
+// may read it ahead of the wait.  cluster > 1: thread block clusters of that size.
 template <typename... KArgs, typename... Args>
 inline cudaError_t launch_maybe_dependent(bool dependent, int cluster, void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem,
                                           cudaStream_t st, Args... args) {

@@ -16,8 +16,8 @@ constexpr int COMPACT_PASSES = 4;
 // idx_div = 1: one pair of index lists per unit; idx_div = Hkv: one pair per (sequence, layer), shared
 // by the layer's KV heads (routing with one map per layer).
 __global__ void __launch_bounds__(COMPACT_THREADS)
-compact_kernel(const uint4* __restrict__ K, const uint4* __restrict__ V, int64_t N, int lp,
-               const int32_t* __restrict__ ret_idx, const int32_t* __restrict__ apx_idx, int n_ret, int n_apx,
+compact_kernel(const uint4* K, const uint4* V, int64_t N, int lp,
+               const int32_t* ret_idx, const int32_t* apx_idx, int n_ret, int n_apx,
                uint4* __restrict__ ret_k, uint4* __restrict__ ret_v, uint4* __restrict__ apx_k,
                int32_t* __restrict__ ret_pos, int32_t* __restrict__ apx_pos, int64_t cap_ret, int64_t cap_apx,
                int chunks, int idx_div) {
@@ -68,7 +68,7 @@ compact_kernel(const uint4* __restrict__ K, const uint4* __restrict__ V, int64_t
 // What an append costs is its launch (three tensor assignments took 21 us of host time for 8 units of 128 channels), so
 // the kernel is a programmatic dependent of what precedes it and lets its own dependent (the decode step) start early.
 __global__ void __launch_bounds__(256)
-append_kernel(const uint4* __restrict__ k_new, const uint4* __restrict__ v_new, int lp, long long n, int64_t row, int64_t cap_ret,
+append_kernel(const uint4* k_new, const uint4* v_new, int lp, long long n, int64_t row, int64_t cap_ret,
               int32_t pos, uint4* __restrict__ ret_k, uint4* __restrict__ ret_v, int32_t* __restrict__ ret_pos) {
     asm volatile("griddepcontrol.wait;\n" ::: "memory");
     asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory");

@@ -22,7 +22,7 @@ namespace vec {
 
 // EPL consecutive elements of a row; WIDE: fp32 rows at multiples of 16 bytes, otherwise one by one.
 template <bool WIDE, int EPL, typename T>
-__device__ __forceinline__ void row_load(const T* __restrict__ p, int lane, float (&o)[EPL]) {
+__device__ __forceinline__ void row_load(const T* p, int lane, float (&o)[EPL]) {
     if constexpr (WIDE) {
         if constexpr (EPL == 4) {
             const float4 v = reinterpret_cast<const float4*>(p)[lane];
@@ -50,9 +50,9 @@ constexpr int F32_WARPS = 8, F32_ROWS = 4, F32_MAX_CLUSTER = 16;
 // grid (U x cluster size), 256 threads, F32_WARPS * g records of dynamic shared memory.
 template <typename T, int D, int G, bool ROPE, bool WIDE>
 __global__ void __launch_bounds__(32 * F32_WARPS)
-decode_rows(const T* __restrict__ q, const T* __restrict__ ret_k, const T* __restrict__ ret_v, const T* __restrict__ apx_k,
-           const int32_t* __restrict__ apx_pos, int64_t cap_ret, int64_t cap_apx, int n_ret, int n_apx, int g, int LH, float scale,
-           float theta, const T* __restrict__ W, void* __restrict__ out, int out_bf16) {
+decode_rows(const T* q, const T* ret_k, const T* ret_v, const T* apx_k,
+           const int32_t* apx_pos, int64_t cap_ret, int64_t cap_apx, int n_ret, int n_apx, int g, int LH, float scale,
+           float theta, const T* W, void* __restrict__ out, int out_bf16) {
     constexpr int EPL = D / 32, REC = Rec<D>::floats, NT = 32 * F32_WARPS;
     extern __shared__ __align__(16) float recs[];               // [F32_WARPS][g][REC]
     __shared__ __align__(16) float comb[G][REC];                // this block's sums, read by the whole cluster

@@ -206,7 +206,7 @@ __device__ __forceinline__ void produce(const Maps& maps, const Plan& pl, long l
 }
 // The g query heads of a unit as A fragments, rows g .. 7 zero; twice: rows 4 .. 7 the same heads as rows 0 .. 3 (g <= 4).
 template <int D>
-__device__ __forceinline__ void load_queries(const __nv_bfloat16* __restrict__ q, int unit, int g, int lane, uint32_t (&qa)[D / 16][2],
+__device__ __forceinline__ void load_queries(const __nv_bfloat16* q, int unit, int g, int lane, uint32_t (&qa)[D / 16][2],
                                              bool twice) {
     const int head = twice ? (lane >> 2) & 3 : lane >> 2, tig = lane & 3;
     const uint32_t* qrow = reinterpret_cast<const uint32_t*>(q + ((size_t)unit * g + min(head, g - 1)) * D);
@@ -373,7 +373,7 @@ __device__ __forceinline__ void store_key_sum(KeySums<D>& ks, int head, int c, f
 // 2 jj + h stand for columns 8 (t + 4 jj) + 4 h .. + 3, which the B fragments follow; the map's elements are bf16 as stored.
 // Three parts: the MMAs of the first start at zero and are added up in fp32, as the sums before them are (Cfg::EXACT).
 template <int D>
-__device__ __forceinline__ void map_rows(const __nv_bfloat16* __restrict__ W, int mt, int n, const KeySums<D>& ks, float (&pw)[8][D], int lane) {
+__device__ __forceinline__ void map_rows(const __nv_bfloat16* W, int mt, int n, const KeySums<D>& ks, float (&pw)[8][D], int lane) {
     constexpr int PARTS = Cfg<D, false>::PARTS;
     constexpr int PIECES = D / 8;                                    // 16-byte pieces of a row of W
     const int row = lane >> 2, quarter = lane & 3;
@@ -432,7 +432,7 @@ template <int D> struct MergeShared {
     float fac[8][MAX_CLUSTER], Ls[8];                                 // factor of every block's sums; sum of the weights
 };
 template <int D, bool ROPE>
-__device__ __forceinline__ void cluster_merge(const float* recs, unsigned char* room, const __nv_bfloat16* __restrict__ Wu, int g,
+__device__ __forceinline__ void cluster_merge(const float* recs, unsigned char* room, const __nv_bfloat16* Wu, int g,
                                               void* __restrict__ out_u, bool out_f32) {
     using C = Cfg<D, ROPE>;
     constexpr int REC = C::REC, CREC = C::CREC, CW = C::CONSUMER_WARPS, NT = C::THREADS, V4 = 2 * D / 4;
@@ -530,9 +530,9 @@ __device__ __forceinline__ void cluster_merge(const float* recs, unsigned char* 
 // CLUSTER writes out itself and does not use partial.
 template <int D, bool CLUSTER>
 __global__ void __launch_bounds__(Cfg<D, false>::THREADS, 1)
-decode_stream_bf16(const __nv_bfloat16* __restrict__ q, const __grid_constant__ Maps maps, Plan pl, int n_ret,
+decode_stream_bf16(const __nv_bfloat16* q, const __grid_constant__ Maps maps, Plan pl, int n_ret,
                         int n_apx, int g, int LH, float scale_log2e, float* __restrict__ partial,
-                        int* __restrict__ fault, const __nv_bfloat16* __restrict__ W, void* __restrict__ out, int out_f32) {
+                        int* __restrict__ fault, const __nv_bfloat16* W, void* __restrict__ out, int out_f32) {
     using C = Cfg<D, false>;
     constexpr int HALF_BYTES = C::HALF_BYTES, SLOT_BYTES = C::SLOT_BYTES, SLOTS = C::SLOTS;
     constexpr int CONSUMER_WARPS = C::CONSUMER_WARPS, REC = C::REC, CREC = C::CREC;
@@ -734,7 +734,7 @@ decode_stream_bf16(const __nv_bfloat16* __restrict__ q, const __grid_constant__ 
 // The product W (sum f acc_k) runs on warp-level MMAs (map_rows).
 template <typename TO, int D, int MAXT>
 __global__ void __launch_bounds__(MAXT, MAXT == 512 ? 3 : 1)
-decode_merge_bf16(const float* __restrict__ partial, const __nv_bfloat16* __restrict__ W, int LH, int g,
+decode_merge_bf16(const float* partial, const __nv_bfloat16* W, int LH, int g,
                        Plan pl, int apply_w, int cw, TO* __restrict__ out) {
     constexpr int REC = 4 + 2 * D;
     __shared__ KeySums<D> ks;

@@ -88,7 +88,7 @@ __host__ __device__ inline int block_of_cost(long long x, const Plan& p) { retur
 // grid (plan.B), THREADS threads, SMEM_BYTES dynamic shared memory.  partial: [U][s_max][g][REC]; slot of (pair, block b) =
 // b - block_of_cost(first cost of the pair).
 __global__ void __launch_bounds__(THREADS, 1)
-decode_layer_mma(const __nv_bfloat16* __restrict__ q, const __grid_constant__ dbf::Maps maps, Plan pl, int n_ret, int n_apx, int g,
+decode_layer_mma(const __nv_bfloat16* q, const __grid_constant__ dbf::Maps maps, Plan pl, int n_ret, int n_apx, int g,
                  float scale_log2e, float* __restrict__ partial, int* __restrict__ fault) {
     __shared__ __align__(8) uint64_t full_bar[STAGES];
     if (threadIdx.x == 0) {
@@ -390,7 +390,7 @@ decode_layer_mma(const __nv_bfloat16* __restrict__ q, const __grid_constant__ db
 constexpr int MERGE_THREADS = 512, MERGE_PAD = 72 * 1024;     // + 46 KB of its own: one block to a multiprocessor, with half of it two
 template <typename TO>
 __global__ void __launch_bounds__(MERGE_THREADS)
-decode_layer_merge_mma(const float* __restrict__ partial, const __nv_bfloat16* __restrict__ W, int L, int g, Plan pl,
+decode_layer_merge_mma(const float* partial, const __nv_bfloat16* W, int L, int g, Plan pl,
                        TO* __restrict__ out) {
     constexpr int KD = HKV * 128;
     __shared__ __align__(16) __nv_bfloat16 akh[8][KD], akl[8][KD];          // 32 KB
@@ -485,7 +485,7 @@ decode_layer_merge_mma(const float* __restrict__ partial, const __nv_bfloat16* _
 // grid (layers * HKV * ceil(batch / seqs)), 512 threads, seqs * g <= 8.
 template <typename TO>
 __global__ void __launch_bounds__(MERGE_THREADS)
-decode_layer_merge_shared(const float* __restrict__ partial, const __nv_bfloat16* __restrict__ W, int L, int g, int batch, int seqs, Plan pl,
+decode_layer_merge_shared(const float* partial, const __nv_bfloat16* W, int L, int g, int batch, int seqs, Plan pl,
                        TO* __restrict__ out) {
     constexpr int KD = HKV * 128;
     __shared__ __align__(16) __nv_bfloat16 akh[8][KD], akl[8][KD];          // 32 KB

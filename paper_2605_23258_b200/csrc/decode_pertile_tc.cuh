@@ -70,7 +70,7 @@ struct Sync {
 // grid (plan.B), THREADS threads, SMEM_BYTES dynamic shared memory.
 // partial: [U][s_max][CONSUMERS][g][REC]; slot of (unit u, block b) = b - block_of_tile(first tile of u).
 __global__ void __launch_bounds__(THREADS, 1)
-decode_stream_pertile_tc(const __nv_bfloat16* __restrict__ q, const __grid_constant__ Maps maps, Plan pl, int n_ret, int n_apx,
+decode_stream_pertile_tc(const __nv_bfloat16* q, const __grid_constant__ Maps maps, Plan pl, int n_ret, int n_apx,
                          int g, int LH, float scale_log2e, float* __restrict__ partial, int* __restrict__ fault) {
     extern __shared__ unsigned char smem_raw[];
     __shared__ Sync sy;

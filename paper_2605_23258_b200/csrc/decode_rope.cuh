@@ -167,10 +167,10 @@ __device__ __forceinline__ void sum_step64(uint32_t st, uint32_t base, bool reta
 // come the sum warps, team by team.
 template <int D, bool CLUSTER>
 __global__ void __launch_bounds__(Cfg<D, true>::THREADS, 1)
-decode_stream_rope(const __nv_bfloat16* __restrict__ q, const __grid_constant__ Maps maps, Plan pl, int n_ret, int n_apx, int g,
+decode_stream_rope(const __nv_bfloat16* q, const __grid_constant__ Maps maps, Plan pl, int n_ret, int n_apx, int g,
                    int LH, float scale_log2e, float* __restrict__ partial, int* __restrict__ fault,
-                   const int32_t* __restrict__ apx_pos, long long cap_apx, const __grid_constant__ RopePhases rope,
-                   const __nv_bfloat16* __restrict__ W, void* __restrict__ out, int out_f32) {
+                   const int32_t* apx_pos, long long cap_apx, const __grid_constant__ RopePhases rope,
+                   const __nv_bfloat16* W, void* __restrict__ out, int out_f32) {
     using C = Cfg<D, true>;
     constexpr int HALF_BYTES = C::HALF_BYTES, SLOT_BYTES = C::SLOT_BYTES, SLOTS = C::SLOTS, TEAMS = C::CONSUMER_WARPS, SUM_WARPS = C::SUM_WARPS;
     constexpr int REC = C::REC, CREC = C::CREC, PAIRS = 2;                    // column tiles of 8 channel pairs of a sum warp
@@ -252,7 +252,7 @@ decode_stream_rope(const __nv_bfloat16* __restrict__ q, const __grid_constant__ 
                     const int32_t* pr = apx_pos + (size_t)u * cap_apx + r0 + lane;
 #pragma unroll
                     for (int k = 0; k < 4; ++k)
-                        if (lane + 32 * k < rows) pos[k] = (uint32_t)__ldg(pr + 32 * k);
+                        if (lane + 32 * k < rows) pos[k] = (uint32_t)pr[32 * k];
                 }
                 if (ok) {
                     if (!loaded) { load_queries<D>(q, u, g, lane, qa, twice); loaded = true; }

@@ -81,17 +81,17 @@ __device__ __forceinline__ Cursor cursor_at(long long item, const Params& P) {
     c.t = (int)(tile - (long long)c.ul * P.tpu);
     return c;
 }
-// 32 bytes through the read-only path: in one load (WIDE, the address a multiple of 32) or in two.
+// 32 bytes: in one load (WIDE, the address a multiple of 32) or in two.
 template <bool WIDE>
 __device__ __forceinline__ void ldg32(const void* p, uint32_t (&r)[64], int at) {
     if constexpr (WIDE) {
-        asm volatile("ld.global.nc.v8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];\n"
+        asm volatile("ld.global.v8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];\n"
                      : "=r"(r[at]), "=r"(r[at + 1]), "=r"(r[at + 2]), "=r"(r[at + 3]), "=r"(r[at + 4]), "=r"(r[at + 5]), "=r"(r[at + 6]), "=r"(r[at + 7])
                      : "l"(p));
     } else {
 #pragma unroll
         for (int h = 0; h < 8; h += 4)
-            asm volatile("ld.global.nc.v4.b32 {%0,%1,%2,%3}, [%4];\n"
+            asm volatile("ld.global.v4.b32 {%0,%1,%2,%3}, [%4];\n"
                          : "=r"(r[at + h]), "=r"(r[at + h + 1]), "=r"(r[at + h + 2]), "=r"(r[at + h + 3])
                          : "l"((const unsigned char*)p + 4 * h));
     }
@@ -103,8 +103,8 @@ __device__ __forceinline__ void ldg32(const void* p, uint32_t (&r)[64], int at) 
 // WIDE: V is a multiple of 32 bytes.  The interface promises 16; rows are 256 bytes apart, so the base decides for all of them.
 template <bool WIDE, int CTAS>
 __global__ void __launch_bounds__(LCfg<CTAS>::THREADS, 1)
-residual_layer_tc(const __nv_bfloat16* __restrict__ K, const __nv_bfloat16* __restrict__ V,
-                  const __grid_constant__ CUtensorMap mapW, const int32_t* __restrict__ idx, const Params P,
+residual_layer_tc(const __nv_bfloat16* K, const __nv_bfloat16* V,
+                  const __grid_constant__ CUtensorMap mapW, const int32_t* idx, const Params P,
                   float* __restrict__ eps, int* __restrict__ fault) {
     extern __shared__ unsigned char smem_raw[];
     __shared__ Sync sy;

@@ -98,8 +98,8 @@ struct RSync {
 // grid: min(multiprocessors, n_tiles) blocks, RCfg::THREADS threads, RCfg::SMEM_BYTES dynamic shared memory.
 template <int D, bool ROPE>
 __global__ void __launch_bounds__(RCfg<D, ROPE>::THREADS, 1)
-residual_tc(const __nv_bfloat16* __restrict__ K, const __nv_bfloat16* __restrict__ V,
-                 const __grid_constant__ CUtensorMap mapW, const int32_t* __restrict__ idx, const Params P,
+residual_tc(const __nv_bfloat16* K, const __nv_bfloat16* V,
+                 const __grid_constant__ CUtensorMap mapW, const int32_t* idx, const Params P,
                  const __grid_constant__ RopePhases rope, float* __restrict__ eps, int* __restrict__ fault) {
     extern __shared__ unsigned char smem_raw[];
     __shared__ RSync sy;
@@ -178,8 +178,8 @@ residual_tc(const __nv_bfloat16* __restrict__ K, const __nv_bfloat16* __restrict
             kx[p] = ky[p] = make_uint4(0u, 0u, 0u, 0u);                  // zero past the end of the list
             if (row >= 0) {
                 const __nv_bfloat16* kr = Ku + (size_t)row * D;
-                kx[p] = __ldg(reinterpret_cast<const uint4*>(kr));
-                ky[p] = __ldg(reinterpret_cast<const uint4*>(kr + D / 2));
+                kx[p] = *reinterpret_cast<const uint4*>(kr);
+                ky[p] = *reinterpret_cast<const uint4*>(kr + D / 2);
             }
         };
         // Turns the pairs of tile i (rows listed in pos), writes them to stage s and publishes it; a pass's registers take

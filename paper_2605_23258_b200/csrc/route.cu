@@ -24,7 +24,7 @@ constexpr size_t SEL_SMEM_LONG = 200 * 1024, SEL_SMEM_MID = 92 * 1024, SEL_SMEM_
 // The general selection (select_emit) as functions of their own: the kernels run the lean path inline and
 // come here only when it gives up, so its registers are not theirs to carry.
 template <int NW>
-__device__ __noinline__ void pool_select_general(const float* __restrict__ s, int n, int n_pool, int32_t* __restrict__ out,
+__device__ __noinline__ void pool_select_general(const float* s, int n, int n_pool, int32_t* __restrict__ out,
                                                  sel::Scratch& S, const Layout& L, uint32_t* dyn) {
     sel::select_emit<false, NW, true>(s, n, n_pool, true, S, L, dyn, [&](int i, bool chosen, int pos) { if (chosen) out[pos] = i; });
 }
@@ -50,7 +50,7 @@ struct TruncateOut {
 };
 
 template <int NW>
-__device__ __noinline__ void truncate_general(const float* __restrict__ e, int n_pool, int n_apx, const TruncateOut& emit,
+__device__ __noinline__ void truncate_general(const float* e, int n_pool, int n_apx, const TruncateOut& emit,
                                               sel::Scratch& S, const Layout& L, uint32_t* dyn) {
     sel::select_emit<true, NW, false>(e, n_pool, n_apx, n_apx > 0, S, L, dyn, emit);
 }
@@ -59,7 +59,7 @@ __device__ __noinline__ void truncate_general(const float* __restrict__ e, int n
 // for a residual kernel that adds its results up.
 template <int NW>
 __global__ void VEC_SEL_BOUNDS(NW)
-pool_select_kernel(const float* __restrict__ scores, int64_t N, int n_pool, int32_t* __restrict__ pool_idx, float* __restrict__ zero,
+pool_select_kernel(const float* scores, int64_t N, int n_pool, int32_t* __restrict__ pool_idx, float* __restrict__ zero,
                    const Layout L) {
     __shared__ sel::Scratch S;
     extern __shared__ __align__(16) uint32_t sel_dyn[];
@@ -82,7 +82,7 @@ pool_select_kernel(const float* __restrict__ scores, int64_t N, int n_pool, int3
 // staged there when the lean path cannot run and they fit).
 template <int NW>
 __global__ void VEC_SEL_BOUNDS(NW)
-truncate_kernel(const float* __restrict__ eps, const int32_t* __restrict__ pool_idx, int64_t N, int n_pool,
+truncate_kernel(const float* eps, const int32_t* pool_idx, int64_t N, int n_pool,
                 int n_apx, uint8_t* __restrict__ tier, int32_t* __restrict__ ret_idx,
                 int32_t* __restrict__ apx_idx, const Layout L) {
     __shared__ sel::Scratch S;
@@ -117,7 +117,7 @@ template <int E> struct TruncateRegsOut {
 };
 template <int NW, int E>
 __global__ void VEC_SEL_BOUNDS(NW)
-pool_select_regs(const float* __restrict__ scores, int64_t N, int n_pool, int32_t* __restrict__ pool_idx, float* __restrict__ zero) {
+pool_select_regs(const float* scores, int64_t N, int n_pool, int32_t* __restrict__ pool_idx, float* __restrict__ zero) {
     __shared__ __align__(16) sel::RegScratch<NW> S;
     sel::regs_clear(S);
     // as in pool_select_kernel
@@ -133,7 +133,7 @@ pool_select_regs(const float* __restrict__ scores, int64_t N, int n_pool, int32_
 
 template <int NW, int E>
 __global__ void VEC_SEL_BOUNDS(NW)
-truncate_regs(const float* __restrict__ eps, const int32_t* __restrict__ pool_idx, int64_t N, int n_pool, int n_apx,
+truncate_regs(const float* eps, const int32_t* pool_idx, int64_t N, int n_pool, int n_apx,
               uint8_t* __restrict__ tier, int32_t* __restrict__ ret_idx, int32_t* __restrict__ apx_idx) {
     __shared__ __align__(16) sel::RegScratch<NW> S;
     const int u = blockIdx.x;
@@ -167,8 +167,8 @@ truncate_regs(const float* __restrict__ eps, const int32_t* __restrict__ pool_id
 // pairs with c + D/2, angle -pos * theta^(-2c/D).
 template <typename T, int D, bool ROPE, int RW>
 __global__ void __launch_bounds__(256)
-residual_generic(const T* __restrict__ K, const T* __restrict__ V, const T* __restrict__ W, int64_t N,
-                 int LH, const int32_t* __restrict__ idx, int n_idx, float theta, float* __restrict__ eps) {
+residual_generic(const T* K, const T* V, const T* W, int64_t N,
+                 int LH, const int32_t* idx, int n_idx, float theta, float* __restrict__ eps) {
     constexpr int CPL = D / 32;             // channels per lane
     extern __shared__ __align__(16) float smem[];
     __shared__ double inv_freq[ROPE ? D / 2 : 1];

@@ -22,7 +22,7 @@ constexpr int ST = 64;    // tile edge (rows and keys) of the CUDA-core score ke
 template <int D> struct TileRegs { float4 v[ST * D / 1024]; };
 // WIDE: fp32 rows at multiples of 16 bytes; otherwise element by element.
 template <bool WIDE, typename T, int D>
-__device__ __forceinline__ void tile_request(const T* __restrict__ src, int64_t row0, int64_t n_rows, TileRegs<D>& t) {
+__device__ __forceinline__ void tile_request(const T* src, int64_t row0, int64_t n_rows, TileRegs<D>& t) {
 #pragma unroll
     for (int e = 0; e < ST * D / 1024; ++e) {
         const int idx = threadIdx.x + 256 * e, r = idx / (D / 4), c4 = idx % (D / 4);
@@ -82,7 +82,7 @@ template <int D> constexpr int tile_smem() { return 2 * ST * PITCH<D> * (int)siz
 // grid (n_chunks, row_tiles, U), 256 threads, tile_smem of dynamic shared memory
 template <typename T, int D, bool WIDE, bool MANY>
 __global__ void __launch_bounds__(256, MIN_BLOCKS<MANY>)
-score_pass1_generic(const T* __restrict__ Q, const T* __restrict__ K, int64_t N, int R, int w,
+score_pass1_generic(const T* Q, const T* K, int64_t N, int R, int w,
                     float scale, int64_t chunk_len, float2* __restrict__ partial) {
     extern __shared__ __align__(16) float tiles[];
     float *Qs = tiles, *Ks = tiles + ST * PITCH<D>;
@@ -150,7 +150,7 @@ score_pass1_generic(const T* __restrict__ Q, const T* __restrict__ K, int64_t N,
 }
 
 // lse of a row from its chunk partials, `stride` apart, four lanes (of one aligned group) together.
-__device__ __forceinline__ float row_lse(const float2* __restrict__ p, int stride, int n_chunks) {
+__device__ __forceinline__ float row_lse(const float2* p, int stride, int n_chunks) {
     const int part = threadIdx.x & 3;
     float M = -INFINITY, L = 0.f;
     for (int c0 = part; c0 < n_chunks; c0 += 16) {
@@ -178,7 +178,7 @@ __device__ __forceinline__ float row_lse(const float2* __restrict__ p, int strid
 }
 // lse[u][row].  grid (ceil(R / 64), U), 256 threads
 __global__ void __launch_bounds__(256)
-score_lse_rows(const float2* __restrict__ partial, int R, int n_chunks, float* __restrict__ lse) {
+score_lse_rows(const float2* partial, int R, int n_chunks, float* __restrict__ lse) {
     asm volatile("griddepcontrol.wait;\n" ::: "memory");
     asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory");
     const int row = blockIdx.x * 64 + (threadIdx.x >> 2);
@@ -191,8 +191,8 @@ score_lse_rows(const float2* __restrict__ partial, int R, int n_chunks, float* _
 // launch less); its tiles overlap by the pooling radius on both sides, raw may be null.
 template <typename T, int D, bool INLINE_LSE, bool WIDE, bool POOLED, bool MANY>
 __global__ void __launch_bounds__(256, MIN_BLOCKS<MANY>)
-score_pass2_generic(const T* __restrict__ Q, const T* __restrict__ K, int64_t N, int R, int w,
-                    float scale, const float2* __restrict__ partial, int n_chunks, const float* __restrict__ lse,
+score_pass2_generic(const T* Q, const T* K, int64_t N, int R, int w,
+                    float scale, const float2* partial, int n_chunks, const float* lse,
                     float* __restrict__ raw, int r, float* __restrict__ score) {
     extern __shared__ __align__(16) float tiles[];
     float *Qs = tiles, *Ks = tiles + ST * PITCH<D>;
@@ -268,7 +268,7 @@ score_pass2_generic(const T* __restrict__ Q, const T* __restrict__ K, int64_t N,
 }
 
 // score[i] = max_{|j-i| <= r, 0 <= j < N-w} raw[j] for i < N-w ; +inf for the window tokens
-__global__ void score_pool_kernel(const float* __restrict__ raw, int64_t N, int w, int r, int64_t total,
+__global__ void score_pool_kernel(const float* raw, int64_t N, int w, int r, int64_t total,
                                   float* __restrict__ score) {
     asm volatile("griddepcontrol.wait;\n" ::: "memory");
     asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory");

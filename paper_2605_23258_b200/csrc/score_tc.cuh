@@ -474,7 +474,7 @@ score_pass1_tc(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__
 // ---- pass 2 -----------------------------------------------------------------
 // log2 of a row's sum of exp2(logit2) from its 2 n_chunks (reference, sum) partials, `stride` apart: the even lane of a
 // pair takes the even tiles' partials, the odd lane the odd tiles', eight loads in flight each.
-__device__ __forceinline__ float row_lse2(const float2* __restrict__ p, int stride, int n_chunks) {
+__device__ __forceinline__ float row_lse2(const float2* p, int stride, int n_chunks) {
     const size_t step = 2 * (size_t)stride;
     p += (size_t)(threadIdx.x & 1) * stride;
     float M = -INFINITY, L = 0.f;
@@ -500,7 +500,7 @@ __device__ __forceinline__ float row_lse2(const float2* __restrict__ p, int stri
 
 // lse2[u][row] = log2 sum over all visible keys of exp2(logit2).  grid (ceil(R / 128), U), 256 threads.
 __global__ void __launch_bounds__(256)
-score_lse2_rows(const float2* __restrict__ partial, int R, int n_chunks, float* __restrict__ lse2) {
+score_lse2_rows(const float2* partial, int R, int n_chunks, float* __restrict__ lse2) {
     asm volatile("griddepcontrol.wait;\n" ::: "memory");
     asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory");
     const int u = blockIdx.y, row = blockIdx.x * 128 + (threadIdx.x >> 1);
@@ -522,7 +522,7 @@ constexpr int POOLED_KEYS = 3072;                    // sums of a chunk, for eve
 template <int D, bool INLINE_LSE, int NB, bool POOLED>
 __global__ void __launch_bounds__(THREADS, 1)
 score_pass2_tc(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__ CUtensorMap mapK, const Params P,
-               const float2* __restrict__ partial, const float* __restrict__ lse2, float* __restrict__ raw_part,
+               const float2* partial, const float* lse2, float* __restrict__ raw_part,
                float* __restrict__ raw_out, float* __restrict__ score, int* __restrict__ fault) {
     static_assert(INLINE_LSE || !POOLED, "only where blocks have few items");
     extern __shared__ unsigned char smem_raw[];
@@ -621,7 +621,7 @@ score_pass2_tc(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__
 // prefix i < N - w; +inf for the window tokens.  grid (ceil(N / 1024), U), 256 threads.
 constexpr int POOL_TILE = 1024;
 __global__ void __launch_bounds__(256)
-score_pool_parts(const float* __restrict__ raw_part, int parts, long long N, int w, int r, float* __restrict__ raw_out,
+score_pool_parts(const float* raw_part, int parts, long long N, int w, int r, float* __restrict__ raw_out,
                  float* __restrict__ score) {
     __shared__ float rs[POOL_TILE + 16];
     asm volatile("griddepcontrol.wait;\n" ::: "memory");        // the second pass's sums
@@ -664,7 +664,7 @@ score_pool_parts(const float* __restrict__ raw_part, int parts, long long N, int
 
 // The same for N a multiple of 4: 16-byte loads and stores, four keys per thread.
 __global__ void __launch_bounds__(256)
-score_pool_parts_v4(const float* __restrict__ raw_part, int parts, long long N, int w, int r, float* __restrict__ raw_out,
+score_pool_parts_v4(const float* raw_part, int parts, long long N, int w, int r, float* __restrict__ raw_out,
                     float* __restrict__ score) {
     __shared__ __align__(16) float rs[POOL_TILE + 16];          // keys i0 - 8 .. i0 + POOL_TILE + 8
     asm volatile("griddepcontrol.wait;\n" ::: "memory");        // the second pass's sums

@@ -112,7 +112,7 @@ __device__ __forceinline__ void pick_bin(const int* hist, int remaining, int* bc
 // matches prefix under mask.  Eight independent loads in flight per thread: the pass is bound by
 // memory latency otherwise.
 template <bool SMALLEST>
-__device__ __forceinline__ void hist_pass_all(const float* __restrict__ vals, int n, int shift, uint32_t digit_mask,
+__device__ __forceinline__ void hist_pass_all(const float* vals, int n, int shift, uint32_t digit_mask,
                                               uint32_t prefix, uint32_t mask, int* hist, uint32_t* stage_out) {
     for (int base = 0; base < n; base += 8 * blockDim.x) {
         float v[8];
@@ -141,7 +141,7 @@ __device__ __forceinline__ int ordered_chunk(int n, int nw) { return (((n + nw -
 // are not chosen, and groups of 32 without a chosen one are passed over.  All threads of the block
 // (32 NW of them) call it; dyn is the block's dynamic shared memory laid out as L describes.
 template <bool SMALLEST, int NW, bool CHOSEN_ONLY, typename Emit>
-__device__ __forceinline__ void select_emit(const float* __restrict__ vals, int n, int k, bool any, Scratch& S, const Layout L,
+__device__ __forceinline__ void select_emit(const float* vals, int n, int k, bool any, Scratch& S, const Layout L,
                                             uint32_t* dyn, Emit emit) {
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     const unsigned lt = (1u << lane) - 1u;
@@ -370,20 +370,20 @@ __device__ __forceinline__ uint32_t image_of_bits(uint32_t u) {
 // Histogram of the leading 11 bits of every element: 16-byte loads, DEPTH of them in flight per thread all the
 // time (a slot's next load is issued as soon as its value has been taken).
 template <bool SMALLEST, int DEPTH>
-__device__ __forceinline__ void hist_pass_lean(const float* __restrict__ vals, int n, int* hist) {
+__device__ __forceinline__ void hist_pass_lean(const float* vals, int n, int* hist) {
     const int nt = blockDim.x;
     if ((reinterpret_cast<uintptr_t>(vals) & 15) == 0) {
         const uint4* p = reinterpret_cast<const uint4*>(vals);
         const int n4 = n >> 2;
         uint4 nx[DEPTH];
 #pragma unroll
-        for (int j = 0; j < DEPTH; ++j) if ((int)threadIdx.x + j * nt < n4) nx[j] = __ldg(p + threadIdx.x + j * nt);
+        for (int j = 0; j < DEPTH; ++j) if ((int)threadIdx.x + j * nt < n4) nx[j] = p[threadIdx.x + j * nt];
         for (int base = threadIdx.x; base < n4; base += DEPTH * nt) {
 #pragma unroll
             for (int j = 0; j < DEPTH; ++j) {
                 if (base + j * nt < n4) {
                     const uint4 x = nx[j];
-                    if (base + (DEPTH + j) * nt < n4) nx[j] = __ldg(p + base + (DEPTH + j) * nt);     // the slot's next load
+                    if (base + (DEPTH + j) * nt < n4) nx[j] = p[base + (DEPTH + j) * nt];     // the slot's next load
                     atomicAdd(&hist[image_of_bits<SMALLEST>(x.x) >> 21], 1);
                     atomicAdd(&hist[image_of_bits<SMALLEST>(x.y) >> 21], 1);
                     atomicAdd(&hist[image_of_bits<SMALLEST>(x.z) >> 21], 1);
@@ -418,7 +418,7 @@ constexpr int SMALL_MAX = 256;
 __host__ __device__ constexpr int lean_loads_per_lane(int nw) { return nw == 32 ? 4 : 2; }
 
 template <bool SMALLEST, int NW, bool CHOSEN_ONLY, typename Sink>
-__device__ __forceinline__ bool select_lean(const float* __restrict__ vals, int n, int k, Scratch& S, const Layout L,
+__device__ __forceinline__ bool select_lean(const float* vals, int n, int k, Scratch& S, const Layout L,
                                             uint32_t* dyn, Sink sink) {
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     constexpr int NT = 32 * NW;
@@ -457,7 +457,7 @@ __device__ __forceinline__ bool select_lean(const float* __restrict__ vals, int 
         auto issue = [&](int base) {
             if (vec_ok && base + CH <= w1) {
 #pragma unroll
-                for (int q = 0; q < TPL; ++q) r[q] = __ldg(reinterpret_cast<const uint4*>(vals + base + 128 * q + 4 * lane));
+                for (int q = 0; q < TPL; ++q) r[q] = *reinterpret_cast<const uint4*>(vals + base + 128 * q + 4 * lane);
             } else {
 #pragma unroll
                 for (int q = 0; q < TPL; ++q) {
@@ -689,7 +689,7 @@ template <int NW> __host__ __device__ constexpr int regs_groups(int n) { return 
 // sink.put(j, i, chosen, pos) for every element, element i being this lane's register j and pos its rank among the chosen or
 // among the others.
 template <bool SMALLEST, int NW, int E, bool CHOSEN_ONLY, typename Sink>
-__device__ __forceinline__ void select_regs(const float* __restrict__ vals, int n, int k, RegScratch<NW>& S, Sink sink) {
+__device__ __forceinline__ void select_regs(const float* vals, int n, int k, RegScratch<NW>& S, Sink sink) {
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     const unsigned lt = (1u << lane) - 1u;
     const int groups = regs_groups<NW>(n);                   // <= E
@@ -697,11 +697,7 @@ __device__ __forceinline__ void select_regs(const float* __restrict__ vals, int 
     const int mine = i0 < n ? min(groups, (n - i0 + 31) / 32) : 0;      // registers of this lane that hold an element
     uint32_t key[E];
 #pragma unroll
-    for (int j = 0; j < E; ++j) {
-        // (volatile: a read-only load could be moved ahead of the caller's wait for the kernel that writes vals)
-        key[j] = 0u;
-        if (j < mine) asm volatile("ld.global.b32 %0, [%1];\n" : "=r"(key[j]) : "l"(vals + i0 + 32 * j) : "memory");
-    }
+    for (int j = 0; j < E; ++j) key[j] = j < mine ? __float_as_uint(vals[i0 + 32 * j]) : 0u;
 #pragma unroll
     for (int j = 0; j < E; ++j) {
         key[j] = image_of_bits<SMALLEST>(key[j]);

@@ -1,6 +1,7 @@
 """The order that programmatic dependent launches rest on, read from the sources: a kernel lets its dependents start
 (griddepcontrol.launch_dependents) only directly behind its own griddepcontrol.wait.  Then all that came before a kernel's primary
-has finished when it starts, whatever chain the calls form."""
+has finished when it starts, whatever chain the calls form.  And what a kernel reads behind its wait is no read-only data to the
+compiler, which could read that ahead of the wait."""
 import glob
 import os
 import re
@@ -17,3 +18,27 @@ def test_dependents_start_behind_the_wait():
                 found += 1
                 assert re.match(r'\s*asm volatile\("griddepcontrol\.wait', lines[i - 1]), f"{os.path.basename(path)}: {line.strip()}"
     assert found >= 15
+
+
+def _chain_files():
+    """The sources that wait for a primary, and the headers that they include."""
+    text = {os.path.basename(p): open(p).read() for p in glob.glob(os.path.join(CSRC, "*.cu")) + glob.glob(os.path.join(CSRC, "*.cuh"))}
+    files = {f for f in text if 'asm volatile("griddepcontrol.wait' in text[f]}
+    while True:
+        more = {h for f in files for h in re.findall(r'#include "(\w+\.cuh)"', text[f])} - files
+        if not more:
+            return {f: re.sub(r"//[^\n]*", "", text[f]) for f in files}
+        files |= more
+
+
+def test_nothing_read_behind_the_wait_is_read_only():
+    files = _chain_files()
+    assert len(files) >= 12 and "select.cuh" in files
+    for name, text in files.items():
+        assert not re.search(r"__ldg\b|\.nc\.", text), name
+        starts = [m.start() for m in re.finditer(r"__global__|__device__", text)] + [len(text)]
+        for lo, hi in zip(starts, starts[1:]):
+            function = text[lo:hi]
+            if re.search(r"const [\w:]+\s*\* __restrict__", function):        # only a kernel that is launched the ordinary way
+                assert function.startswith("__global__") and "griddepcontrol" not in function and "_role<" not in function, \
+                    (name, function[:120])
