@@ -88,7 +88,6 @@ truncate_kernel(const float* eps, const int32_t* pool_idx, int64_t N, int n_pool
     __shared__ sel::Scratch S;
     extern __shared__ __align__(16) uint32_t sel_dyn[];
     const int u = blockIdx.x;
-    const float* e = eps + (size_t)u * n_pool;
     uint8_t* tr = tier + (size_t)u * N;
     if ((N & 15) == 0) {
         for (int64_t i = threadIdx.x; i < N / 16; i += 32 * NW) reinterpret_cast<uint4*>(tr)[i] = make_uint4(0, 0, 0, 0);
@@ -99,6 +98,7 @@ truncate_kernel(const float* eps, const int32_t* pool_idx, int64_t N, int n_pool
     // nothing before that kernel is still under way: it waits before it lets this one start.  (No wait unless a dependent.)
     asm volatile("griddepcontrol.wait;\n" ::: "memory");
     __syncthreads();
+    const float* e = eps + (size_t)u * n_pool;
     const int n_ret = n_pool - n_apx;
     const TruncateOut emit = {pool_idx + (size_t)u * n_pool, tr, ret_idx + (size_t)u * n_ret, apx_idx + (size_t)u * n_apx, N};
     if (L.keyed && n_apx > 0 && sel::select_lean<true, NW, false>(e, n_pool, n_apx, S, L, sel_dyn, emit)) return;
@@ -138,22 +138,20 @@ truncate_regs(const float* eps, const int32_t* pool_idx, int64_t N, int n_pool, 
     __shared__ __align__(16) sel::RegScratch<NW> S;
     const int u = blockIdx.x;
     uint8_t* tr = tier + (size_t)u * N;
-    const int32_t* pool = pool_idx + (size_t)u * n_pool;
     if ((N & 15) == 0 && ((uintptr_t)tier & 15) == 0) {
         for (int64_t i = threadIdx.x; i < N / 16; i += 32 * NW) reinterpret_cast<uint4*>(tr)[i] = make_uint4(0, 0, 0, 0);
     } else {
         for (int64_t i = threadIdx.x; i < N; i += 32 * NW) tr[i] = 0;
     }
     sel::regs_clear(S);
-    // Everything above touches only the tier map, which the residual kernel, this one's primary, neither reads nor writes, and
-    // nothing before that kernel is still under way: it waits before it lets this one start.  (No wait unless a dependent.)  The
-    // list of the pool was written before that kernel.
+    // as in truncate_kernel; the list of the pool, which a kernel of the same chain wrote, is read behind the wait as the residuals are
+    asm volatile("griddepcontrol.wait;\n" ::: "memory");
+    __syncthreads();
+    const int32_t* pool = pool_idx + (size_t)u * n_pool;
     int32_t token[E];
     const int groups = sel::regs_groups<NW>(n_pool), p0 = (threadIdx.x >> 5) * groups * 32 + (threadIdx.x & 31);
 #pragma unroll
     for (int j = 0; j < E; ++j) token[j] = j < groups && p0 + 32 * j < n_pool ? pool[p0 + 32 * j] : 0;
-    asm volatile("griddepcontrol.wait;\n" ::: "memory");
-    __syncthreads();
     const TruncateOut to = {pool, tr, ret_idx + (size_t)u * (n_pool - n_apx), apx_idx + (size_t)u * n_apx, N};
     sel::select_regs<true, NW, E, false>(eps + (size_t)u * n_pool, n_pool, n_apx, S, TruncateRegsOut<E>{to, token});
 }

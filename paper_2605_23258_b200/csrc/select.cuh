@@ -697,7 +697,11 @@ __device__ __forceinline__ void select_regs(const float* vals, int n, int k, Reg
     const int mine = i0 < n ? min(groups, (n - i0 + 31) / 32) : 0;      // registers of this lane that hold an element
     uint32_t key[E];
 #pragma unroll
-    for (int j = 0; j < E; ++j) key[j] = j < mine ? __float_as_uint(vals[i0 + 32 * j]) : 0u;
+    for (int j = 0; j < E; ++j) {
+        // volatile, so that all are under way before the first is counted: 12.7 -> 11.7 us for 148 lists of 16384
+        key[j] = 0u;
+        if (j < mine) asm volatile("ld.global.b32 %0, [%1];\n" : "=r"(key[j]) : "l"(vals + i0 + 32 * j) : "memory");
+    }
 #pragma unroll
     for (int j = 0; j < E; ++j) {
         key[j] = image_of_bits<SMALLEST>(key[j]);

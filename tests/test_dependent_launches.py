@@ -42,3 +42,16 @@ def test_nothing_read_behind_the_wait_is_read_only():
             if re.search(r"const [\w:]+\s*\* __restrict__", function):        # only a kernel that is launched the ordinary way
                 assert function.startswith("__global__") and "griddepcontrol" not in function and "_role<" not in function, \
                     (name, function[:120])
+
+
+def test_routing_reads_nothing_ahead_of_the_wait():
+    """Every list that a routing kernel reads was written by a kernel of its chain: ahead of its wait it does not so much as name one."""
+    text = re.sub(r"//[^\n]*", "", open(os.path.join(CSRC, "route.cu")).read())
+    kernels = 0
+    for m in re.finditer(r"__global__[^{;]*?(\w+)\(([^(){;]*)\) \{(.*?)\n\}", text, re.S):
+        ahead, wait, _ = m.group(3).partition('asm volatile("griddepcontrol.wait')
+        inputs = re.findall(r"const [\w:]+\* (?:__restrict__ )?(\w+)", m.group(2))
+        if wait:
+            kernels += 1
+            assert inputs and not re.search(r"\b(%s)\b" % "|".join(inputs), ahead), (m.group(1), inputs)
+    assert kernels == 5
