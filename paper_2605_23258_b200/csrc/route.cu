@@ -345,7 +345,7 @@ static vector_status select_kernels_setup() {
 // 8 warps / 16 warps.  Step 1: 2368 lists of 3000 elements 41 / 41 / 66; 444 of 6500 14.4 / 14.5 / 18.8, 592 of 6500 17.0 / 14.8 /
 // 21.2; 148 of 12000 10.6 / 13.6 / 10.9, 296 of 12000 15.0 / 15.8 / 14.1, 592 of 12000 27.7 / 21.3 / 26.3, 1184 of 14000 57 / 70 / 62,
 // 148 of 20011 13.8 / 23.8 / 16.4, 296 of 20011 26.5 / 32.4 / 21.7, 1184 of 20011 109 / 109 / 99.  Step 3: 2368 lists of 8192 108 /
-// 111 / 135; 148 of 12000 12.8 / 21.9 / 16.1, 296 of 12000 24.5 / 25.9 / 22.4, 592 of 12000 49 / 41 / 45, 1184 of 16384 126 / 107 /
+// 111 / 135; 148 of 12000 12.8 / 21.9 / 16.1, 296 of 12000 24.5 / 25.9 / 22.4, 592 of 12000 49 / 41 / 45, 640 of 16384 77 / 76 / 73, 1184 of 16384 126 / 107 /
 // 113; 148 of 20011 in 64 registers a thread, which do not hold image and token, 41.9 / 35.0 / 25.3; 888 of 20011 - / 125 / 118, 1184
 // of 20011 - / 149 / 155, of 26000 - / 179 / 177.
 static int selection_warps(int64_t n, int U, bool step3) {
@@ -355,8 +355,8 @@ static int selection_warps(int64_t n, int U, bool step3) {
     if (n <= SEL_REGS16) {
         if (U <= sms) return 0;
         if (U <= 2 * sms) return 16;
-        if (step3 || n <= 12288) return 8;
-        return U <= 4 * sms ? 16 : 0;
+        if (step3) return U <= 4 * sms || U >= 8 * sms ? 8 : 16;          // a second round of small blocks that is nearly empty
+        return n <= 12288 ? 8 : U <= 4 * sms ? 16 : 0;
     }
     if (!step3 && n <= SEL_REGS && U <= sms) return 0;
     if (step3 && n <= 24576 && U >= 8 * sms) return 8;

@@ -21,7 +21,7 @@ def _lists(share, n, ties):
 
 @pytest.mark.parametrize("ties", [False, True])
 @pytest.mark.parametrize("share,n", [(0.9, 16384), (0.9, 16385), (0.9, 32768), (1, 8192), (1, 8193), (1, 16385), (2, 12288), (2, 12289), (3, 4096), (3, 4097),
-                                     (3, 8192), (3, 16384), (4, 12289), (4, 16384), (8, 4097), (8, 8193), (8, 16385), (8, 24576), (8, 24577)])
+                                     (3, 8192), (3, 16384), (4, 12289), (4, 16384), (4.5, 8193), (8, 4097), (8, 8193), (8, 16385), (8, 24576), (8, 24577)])
 def test_forms(share, n, ties):
     U, v = _lists(share, n, ties)
     sh = vec.Shape(1, 1, U, U, 64, vec.VECTOR_F32, 1)
