@@ -78,6 +78,16 @@ pool_select_kernel(const float* scores, int64_t N, int n_pool, int32_t* __restri
     pool_select_general<NW>(s, n, n_pool, out, S, L, sel_dyn);
 }
 
+// n bytes set to zero by a block, 16 at a time where they lie so.
+template <int NW>
+__device__ __forceinline__ void clear_bytes(uint8_t* p, int64_t n) {
+    if (((n | (int64_t)(uintptr_t)p) & 15) == 0) {
+        for (int64_t i = threadIdx.x; i < n / 16; i += 32 * NW) reinterpret_cast<uint4*>(p)[i] = make_uint4(0, 0, 0, 0);
+    } else {
+        for (int64_t i = threadIdx.x; i < n; i += 32 * NW) p[i] = 0;
+    }
+}
+
 // Step 3.  grid (U), 32 NW threads, L.bytes() of dynamic shared memory (the residuals' images are
 // staged there when the lean path cannot run and they fit).
 template <int NW>
@@ -89,11 +99,7 @@ truncate_kernel(const float* eps, const int32_t* pool_idx, int64_t N, int n_pool
     extern __shared__ __align__(16) uint32_t sel_dyn[];
     const int u = blockIdx.x;
     uint8_t* tr = tier + (size_t)u * N;
-    if ((N & 15) == 0) {
-        for (int64_t i = threadIdx.x; i < N / 16; i += 32 * NW) reinterpret_cast<uint4*>(tr)[i] = make_uint4(0, 0, 0, 0);
-    } else {
-        for (int64_t i = threadIdx.x; i < N; i += 32 * NW) tr[i] = 0;
-    }
+    clear_bytes<NW>(tr, N);
     // Everything above touches only the tier map, which the residual kernel, this one's primary, neither reads nor writes, and
     // nothing before that kernel is still under way: it waits before it lets this one start.  (No wait unless a dependent.)
     asm volatile("griddepcontrol.wait;\n" ::: "memory");
@@ -138,11 +144,7 @@ truncate_regs(const float* eps, const int32_t* pool_idx, int64_t N, int n_pool, 
     __shared__ __align__(16) sel::RegScratch<NW> S;
     const int u = blockIdx.x;
     uint8_t* tr = tier + (size_t)u * N;
-    if ((N & 15) == 0 && ((uintptr_t)tier & 15) == 0) {
-        for (int64_t i = threadIdx.x; i < N / 16; i += 32 * NW) reinterpret_cast<uint4*>(tr)[i] = make_uint4(0, 0, 0, 0);
-    } else {
-        for (int64_t i = threadIdx.x; i < N; i += 32 * NW) tr[i] = 0;
-    }
+    clear_bytes<NW>(tr, N);
     sel::regs_clear(S);
     // as in truncate_kernel; the list of the pool, which a kernel of the same chain wrote, is read behind the wait as the residuals are
     asm volatile("griddepcontrol.wait;\n" ::: "memory");

@@ -77,3 +77,21 @@ def test_decode(dtype, d, rope, U, g, n_ret, n_apx):
     vec.vector_decode_attn(sh, q, vec.Cache(rk, rv, ak, ret_pos, pos, n_ret, n_apx), W, want, 0, ws)
     vec.vector_decode_attn(sh, _shifted(q), vec.Cache(_shifted(rk), _shifted(rv), _shifted(ak), ret_pos, pos, n_ret, n_apx), _shifted(W), got, 0, ws)
     _same(got, want, dtype == torch.float32)
+
+
+@pytest.mark.parametrize("n", [500, 9000, 17000])
+def test_tier_map(n):
+    """A tier map one byte into its storage, in every form of Step 3 (three lists of 9000 are held in registers, 400 are not)."""
+    for U in (3, 400):
+        gen = torch.Generator(device=DEV).manual_seed(n)
+        eps = torch.rand(U, n, generator=gen, device=DEV)
+        N, k = (n + 31) // 16 * 16, n // 4 * 2
+        pool = torch.arange(N - n, N, dtype=torch.int32, device=DEV).repeat(U, 1).contiguous()
+        sh = vec.Shape(1, 1, U, U, 64, vec.VECTOR_F32, 1)
+        ret, apx = (torch.empty(U, m, dtype=torch.int32, device=DEV) for m in (n - k, k))
+        tiers = torch.full((U, N), 9, dtype=torch.uint8, device=DEV), torch.full((U * N + 1,), 9, dtype=torch.uint8, device=DEV)
+        for t in (tiers[0], tiers[1][1:].view(U, N)):
+            vec.vector_truncate(sh, vec.Budget(N, n - k // 2, k // 2, n, k, n - k, N - n), eps, pool, t, ret, apx)
+        torch.cuda.synchronize()
+        assert torch.equal(tiers[0], tiers[1][1:].view(U, N)) and tiers[1][0] == 9
+        assert torch.equal(tiers[0].sum(1), torch.full((U,), 2 * (n - k) + k, device=DEV))
