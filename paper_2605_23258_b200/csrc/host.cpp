@@ -139,9 +139,12 @@ ScoreTcPlan score_tc_plan(int U, int R, int64_t N) {
 size_t score_ws_bytes(const Dims& D, int64_t N, bool need_raw) {
     if (score_uses_tc(D)) {
         const ScoreTcPlan p = score_tc_plan(D.U, D.R, N);
+        // a row of key sums for every 128 rows; calls of 64 channels whose rows lie off a 16-byte boundary run on CUDA cores with this
+        // workspace and take what a second row leaves for more chunks
+        const int sums = D.d == 64 ? 2 * p.RG : (D.R + 127) / 128;
         return align256((size_t)D.U * 2 * p.n_chunks * D.R * 2 * sizeof(float)) + // (reference, sum) partials, two per chunk
                align256((size_t)D.U * D.R * sizeof(float)) +                        // lse
-               align256((size_t)D.U * 2 * p.RG * (size_t)N * sizeof(float));        // per-row-block key sums
+               align256((size_t)D.U * sums * (size_t)N * sizeof(float));
     }
     size_t b = 0;
     b += align256((size_t)D.U * score_num_chunks(D.U, D.R, N) * D.R * 2 * sizeof(float));  // (max, sum) partials

@@ -56,3 +56,21 @@ def test_score_fp32(oracle, units, d, g, w, N, pool):
         for got, want in ((raw[u], raw_o), (scores[u], sc_o)):
             ok, worst = score_close(got.cpu().numpy()[None], want[None], g * w)
             assert ok, (u, worst)
+
+
+@pytest.mark.parametrize("d,rows", [(128, 96), (128, 300), (64, 96)])
+def test_workspace_is_enough(d, rows):
+    """With little to select, the scores' sums are what the workspace is sized by: nothing is written behind it."""
+    U, N = 200, 20000
+    gen = torch.Generator(device=DEV).manual_seed(rows)
+    K = torch.randn(U, N, d, generator=gen, device=DEV).to(torch.bfloat16)
+    Q = torch.randn(U, 1, rows, d, generator=gen, device=DEV).to(torch.bfloat16)
+    sh = vec.Shape(1, U, 1, 1, d, vec.VECTOR_BF16, rows)
+    need = vec.vector_workspace_bytes(sh, vec.vector_plan_budget(N, 512, -1, rows))
+    room = torch.full((need + 65536,), 7, dtype=torch.uint8, device=DEV)
+    got, want = (torch.full((U, N), float("nan"), device=DEV) for _ in range(2))
+    vec.vector_score(sh, Q, K, N, got, None, room[:need])
+    vec.vector_score(sh, Q, K, N, want, None, torch.empty(2 * need, dtype=torch.uint8, device=DEV))
+    torch.cuda.synchronize()
+    assert vec.vector_device_fault() == 0
+    assert torch.equal(got, want) and bool((room[need:] == 7).all())

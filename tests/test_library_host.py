@@ -158,3 +158,12 @@ def test_struct_fields_follow_the_header():
         body = re.search(r"typedef struct \{([^}]*)\} " + name, text).group(1)
         fields = [f.strip(" *") for line in body.split(";") if line.strip() for f in re.sub(r"^\s*\w+\s*\**", "", line.strip()).split(",")]
         assert fields == [f for f, _ in struct._fields_]
+
+
+def test_workspace_of_scores_of_few_rows():
+    """Units of up to 128 rows have one row of key sums: nearly all of the workspace where keys are many, with little to select."""
+    for rows, sums in ((96, 1), (128, 1), (129, 2), (256, 2), (300, 3)):
+        N, U = 131072, 64
+        sh = vec.Shape(1, 8, 8, 8, 128, vec.VECTOR_BF16, rows)
+        need = vec.vector_workspace_bytes(sh, vec.vector_plan_budget(N, 1024, -1, rows))
+        assert sums * U * N * 4 <= need < (sums + 0.5) * U * N * 4, (rows, need)
