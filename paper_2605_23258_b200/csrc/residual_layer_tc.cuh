@@ -202,12 +202,14 @@ residual_layer_tc(const __nv_bfloat16* K, const __nv_bfloat16* V,
             const uint32_t buf = i & 1, use = i >> 1;
             const uint32_t idesc = H - 2 * at.pair > 1 ? tc::instr_desc(128 * CTAS, 256) : tc::instr_desc(128 * CTAS, 128);
             const uint32_t d = sy.tmem_base + buf * 256;
-            if (rank == 0 && use > 0 && !tma::mbar_wait_warp(&sy.acc_empty[buf], (use - 1) & 1, fault, 83)) break;
+            if (rank == 0 && use > 0 && !tma::mbar_wait_warp<CTAS>(&sy.acc_empty[buf], (use - 1) & 1, fault, 83)) break;
+            tma::acquire_pair<CTAS>();
             for (int hk = 0; hk < 2 * H; ++hk, ++step) {
-                if (!__all_sync(0xffffffffu, ready) && !tma::mbar_wait_warp(&sy.full[s], round & 1, fault, 84)) { ok = false; break; }
+                if (!__all_sync(0xffffffffu, ready) && !tma::mbar_wait_warp<CTAS>(&sy.full[s], round & 1, fault, 84)) { ok = false; break; }
                 const uint32_t k_addr = tma::smem_u32(smem + s * STAGE_BYTES), w_addr = k_addr + BOX_BYTES;
                 const uint32_t s_next = s + 1 == STAGES ? 0 : s + 1, round_next = round + (s + 1 == STAGES);
-                ready = step + 1 < n_steps ? tma::mbar_test(&sy.full[s_next], round_next & 1) : 0u;
+                ready = step + 1 < n_steps ? tma::mbar_test<CTAS>(&sy.full[s_next], round_next & 1) : 0u;
+                tma::acquire_pair<CTAS>();                          // this block's loaders and, in the first block, the other's warp
                 if (rank != 0) {                                    // the first block issues for both: tell it that this half is there
                     if (elected) tma::mbar_arrive_at<CTAS>(tma::block_addr<CTAS>(&sy.full[s], 0));
                 } else {

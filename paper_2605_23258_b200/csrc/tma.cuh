@@ -27,19 +27,29 @@ __device__ __forceinline__ void mbar_expect_tx(uint64_t* bar, uint32_t bytes) {
 __device__ __forceinline__ void mbar_arrive(uint64_t* bar) {
     asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];\n" ::"r"(smem_u32(bar)) : "memory");
 }
+// CTAS = 2, here and below: the phase has arrivals of the other block of a pair (mbar_arrive_at); acquire_pair() behind the wait.
+template <int CTAS = 1>
 __device__ __forceinline__ bool mbar_try_wait(uint64_t* bar, uint32_t parity) {
     uint32_t ok;
-    asm volatile(
-        "{\n .reg .pred p;\n"
-        " mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n"
-        " selp.u32 %0, 1, 0, p;\n}\n"
-        : "=r"(ok) : "r"(smem_u32(bar)), "r"(parity) : "memory");
+    if constexpr (CTAS == 1)
+        asm volatile(
+            "{\n .reg .pred p;\n"
+            " mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n"
+            " selp.u32 %0, 1, 0, p;\n}\n"
+            : "=r"(ok) : "r"(smem_u32(bar)), "r"(parity) : "memory");
+    else
+        asm volatile(
+            "{\n .reg .pred p;\n"
+            " mbarrier.try_wait.parity.relaxed.cluster.shared::cta.b64 p, [%1], %2;\n"
+            " selp.u32 %0, 1, 0, p;\n}\n"
+            : "=r"(ok) : "r"(smem_u32(bar)), "r"(parity) : "memory");
     return ok != 0;
 }
 // Bounded wait; returns false (after recording `code` in *fault) if the phase never completed.
+template <int CTAS = 1>
 __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, int* fault, int code) {
     for (uint32_t i = 0; i < kSpinLimit; ++i)
-        if (mbar_try_wait(bar, parity)) return true;
+        if (mbar_try_wait<CTAS>(bar, parity)) return true;
     atomicCAS(fault, 0, code);
     return false;
 }
@@ -47,20 +57,29 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, int* f
 // The same wait for a whole warp: every lane polls, and the warp leaves the wait converged (the
 // warp-wide .aligned instructions that follow such a wait -- ldmatrix, mma, tcgen05.ld -- require
 // it).  All lanes get the same answer.
+template <int CTAS = 1>
 __device__ __forceinline__ bool mbar_wait_warp(uint64_t* bar, uint32_t parity, int* fault, int code) {
-    const bool ok = mbar_wait(bar, parity, fault, code);
+    const bool ok = mbar_wait<CTAS>(bar, parity, fault, code);
     __syncwarp();
     return __all_sync(0xffffffffu, ok);
 }
 
 // Whether the phase has completed, without waiting.
+template <int CTAS = 1>
 __device__ __forceinline__ uint32_t mbar_test(uint64_t* bar, uint32_t parity) {
     uint32_t ok;
-    asm volatile(
-        "{\n .reg .pred p;\n"
-        " mbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n"
-        " selp.u32 %0, 1, 0, p;\n}\n"
-        : "=r"(ok) : "r"(smem_u32(bar)), "r"(parity) : "memory");
+    if constexpr (CTAS == 1)
+        asm volatile(
+            "{\n .reg .pred p;\n"
+            " mbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n"
+            " selp.u32 %0, 1, 0, p;\n}\n"
+            : "=r"(ok) : "r"(smem_u32(bar)), "r"(parity) : "memory");
+    else
+        asm volatile(
+            "{\n .reg .pred p;\n"
+            " mbarrier.test_wait.parity.relaxed.cluster.shared::cta.b64 p, [%1], %2;\n"
+            " selp.u32 %0, 1, 0, p;\n}\n"
+            : "=r"(ok) : "r"(smem_u32(bar)), "r"(parity) : "memory");
     return ok;
 }
 
@@ -97,10 +116,23 @@ __device__ __forceinline__ uint32_t block_addr(const void* p, uint32_t block) {
     if constexpr (CTAS == 2) asm("mapa.shared::cluster.u32 %0, %1, %2;\n" : "=r"(a) : "r"(smem_u32(p)), "r"(block));
     return a;
 }
+// From block to block: an arrival there (mbar_arrive_at) releases, and acquire_pair() behind the wait for it acquires, at the scope of
+// the cluster, what lies in shared memory -- the keys that a block's loaders wrote and fenced for the tensor cores, which products
+// issued by the other block read there.  The order is made by fences that are restricted to shared memory, with the arrival and the polls
+// relaxed: an arrival that releases and polls that acquire at that scope order all memory, at the cost of all that the multiprocessor has in
+// flight and of its L1 (a route of 16 layers, 8 heads: 341 us; so 196, as without any order).
 template <int CTAS>
 __device__ __forceinline__ void mbar_arrive_at(uint32_t bar) {
-    if constexpr (CTAS == 1) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];\n" ::"r"(bar) : "memory");
-    else asm volatile("mbarrier.arrive.shared::cluster.b64 _, [%0];\n" ::"r"(bar) : "memory");
+    if constexpr (CTAS == 1) {
+        asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];\n" ::"r"(bar) : "memory");
+    } else {
+        asm volatile("fence.release.sync_restrict::shared::cta.cluster;\n" ::: "memory");
+        asm volatile("mbarrier.arrive.relaxed.cluster.shared::cluster.b64 _, [%0];\n" ::"r"(bar) : "memory");
+    }
+}
+template <int CTAS>
+__device__ __forceinline__ void acquire_pair() {
+    if constexpr (CTAS == 2) asm volatile("fence.acquire.sync_restrict::shared::cluster.cluster;\n" ::: "memory");
 }
 __device__ __forceinline__ void prefetch_map(const CUtensorMap* map) {
     asm volatile("prefetch.tensormap [%0];\n" ::"l"(map) : "memory");
