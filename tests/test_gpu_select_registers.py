@@ -45,3 +45,27 @@ def test_selections(oracle, n, kind):
             # the lists lie back to back
             assert np.array_equal(ret.flatten()[u * (n - k):(u + 1) * (n - k)].cpu().numpy(), r), (k, u)
             assert np.array_equal(apx.flatten()[u * k:(u + 1) * k].cpu().numpy(), a), (k, u)
+
+
+@pytest.mark.parametrize("n,lists", [(100, 3), (2500, 3), (9000, 3), (9000, 400), (20000, 3), (40000, 3)])
+def test_order_of_special_values(n, lists):
+    """-0 is below +0, a NaN without its sign bit is above +inf and one with it below -inf, in every form of both steps; ties, NaNs of
+    the same bits among them, go to the lowest index.  Against a stable sort of the 32-bit images."""
+    gen = torch.Generator(device=DEV).manual_seed(n)
+    v = torch.randn(lists, n, generator=gen, device=DEV)
+    kinds = torch.randint(0, 12, (lists, n), generator=gen, device=DEV)
+    for k, bits in enumerate((0, -2 ** 31, 0x7f800000, -0x800000, 0x7fc00000, -0x400000, 0x7fc00001, 1)):
+        v = torch.where(kinds == k, torch.full_like(kinds, bits).to(torch.int32).view(torch.float32), v)
+    image = v.view(torch.int32)
+    image = torch.where(image < 0, image ^ 0x7fffffff, image)
+    sh = vec.Shape(1, 1, lists, lists, 64, vec.VECTOR_F32, 1)
+    for k in (n // 16 * 2, n // 4 * 2, n // 2 * 2 - 2):
+        out = torch.empty(lists, k, dtype=torch.int32, device=DEV)
+        vec.vector_pool_select(sh, vec.Budget(n, k, 0, k, 0, k, n - k), v, out)
+        assert torch.equal(out.long(), torch.sort(image, dim=1, descending=True, stable=True).indices[:, :k].sort(dim=1).values), k
+        pool = torch.arange(n, dtype=torch.int32, device=DEV).repeat(lists, 1).contiguous()
+        tier = torch.empty(lists, n, dtype=torch.uint8, device=DEV)
+        ret, apx = (torch.empty(lists, m, dtype=torch.int32, device=DEV) for m in (n - k, k))
+        vec.vector_truncate(sh, vec.Budget(n, n - k // 2, k // 2, n, k, n - k, 0), v, pool, tier, ret, apx)
+        order = torch.sort(image, dim=1, stable=True).indices
+        assert torch.equal(apx.long(), order[:, :k].sort(dim=1).values) and torch.equal(ret.long(), order[:, k:].sort(dim=1).values), k
