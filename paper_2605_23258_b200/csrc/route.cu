@@ -88,8 +88,7 @@ __device__ __forceinline__ void clear_bytes(uint8_t* p, int64_t n) {
     }
 }
 
-// Step 3.  grid (U), 32 NW threads, L.bytes() of dynamic shared memory (the residuals' images are
-// staged there when the lean path cannot run and they fit).
+// Step 3.  grid (U), 32 NW threads, L.bytes() of dynamic shared memory.
 template <int NW>
 __global__ void VEC_SEL_BOUNDS(NW)
 truncate_kernel(const float* eps, const int32_t* pool_idx, int64_t N, int n_pool,
@@ -367,8 +366,7 @@ static int selection_warps(int64_t n, int U, bool step3) {
 static Layout selection_layout(int64_t n, int nw) {
     const size_t budget = nw == 8 ? SEL_SMEM_SHORT : nw == 16 ? SEL_SMEM_MID : SEL_SMEM_LONG;
     const int min_cand = nw == 8 ? 1024 : 2048;
-    const Layout L = sel::plan_layout(n, false, budget, min_cand, nw);
-    return L.keyed ? L : sel::plan_layout(n, true, budget, min_cand, nw);       // the general path stages the images
+    return sel::plan_layout(n, budget, min_cand, nw);
 }
 
 static vector_status launch_pool_select(const Dims& dm, const vector_budget* budget, const float* scores, int32_t* pool,

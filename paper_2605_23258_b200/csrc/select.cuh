@@ -15,8 +15,7 @@
 // select_emit (the general one) runs: a most-significant-digit radix select with digits of 11, 11 and
 //   10 bits whose passes fall back to re-reading the input when the list or the masks do not fit.
 //
-// The masks, the candidate list, the warps' transposition tiles and (general path, residuals) the
-// images kept by pass 1 live in dynamic shared memory sized to the input.
+// The masks, the candidate list and the warps' transposition tiles live in dynamic shared memory sized to the input.
 #ifndef VECTOR_SELECT_CUH_
 #define VECTOR_SELECT_CUH_
 
@@ -46,17 +45,16 @@ struct __align__(16) Scratch {
     uint32_t small[256];          // offsets of the candidates that share the k-th key's leading bits (lean path)
     OrderedScratch os;
 };
-// Dynamic shared memory of one selection: cand[cand_cap] | sel_mask[groups] | tie_mask[groups] | stage[stage_words]
-// or, for the lean path, ... | tie_mask[groups] | tiles[tile_words].
+// Dynamic shared memory of one selection: cand[cand_cap] | sel_mask[groups] | tie_mask[groups] and, for the lean path,
+// tiles[tile_words].
 // With `keyed` the list is read as cand_cap / 2 indices followed by their cand_cap / 2 images (the lean path).
 struct Layout {
     int cand_cap;                 // candidates the list holds (words)
     int groups;                   // mask words (one per 32 elements), 0 = masks not kept
-    int stage_words;              // images kept by pass 1 (0 or n)
     int keyed;                    // 1: the lean path may run (masks kept, cand_cap a multiple of 8)
     int tile_words;               // the lean path's per-warp transposition tiles, behind the masks
     __host__ __device__ size_t bytes() const {
-        return ((size_t)cand_cap + 2 * (size_t)groups + (size_t)stage_words + (size_t)tile_words) * 4;
+        return ((size_t)cand_cap + 2 * (size_t)groups + (size_t)tile_words) * 4;
     }
 };
 
@@ -113,7 +111,7 @@ __device__ __forceinline__ void pick_bin(const int* hist, int remaining, int* bc
 // memory latency otherwise.
 template <bool SMALLEST>
 __device__ __forceinline__ void hist_pass_all(const float* vals, int n, int shift, uint32_t digit_mask,
-                                              uint32_t prefix, uint32_t mask, int* hist, uint32_t* stage_out) {
+                                              uint32_t prefix, uint32_t mask, int* hist) {
     for (int base = 0; base < n; base += 8 * blockDim.x) {
         float v[8];
 #pragma unroll
@@ -125,7 +123,6 @@ __device__ __forceinline__ void hist_pass_all(const float* vals, int n, int shif
         for (int j = 0; j < 8; ++j) {
             const int i = base + j * blockDim.x + threadIdx.x;
             const uint32_t key = select_image<SMALLEST>(v[j]);
-            if (stage_out && i < n) stage_out[i] = key;          // keep the image for the later passes
             hist_add(hist, (key >> shift) & digit_mask, i < n && (key & mask) == prefix);
         }
     }
@@ -148,7 +145,6 @@ __device__ __forceinline__ void select_emit(const float* vals, int n, int k, boo
     int32_t* cand = reinterpret_cast<int32_t*>(dyn);
     uint32_t* sel_mask = dyn + L.cand_cap;
     uint32_t* tie_mask = sel_mask + L.groups;
-    uint32_t* stage = L.stage_words ? tie_mask + L.groups : nullptr;
     const bool masked = L.groups > 0;
     const int per_w = ordered_chunk(n, NW);
     const int w0 = min(n, wid * per_w), w1 = min(n, w0 + per_w);
@@ -162,7 +158,7 @@ __device__ __forceinline__ void select_emit(const float* vals, int n, int k, boo
         for (int b = threadIdx.x; b < SEL_BINS; b += blockDim.x) S.hist[b] = 0;
         if (threadIdx.x == 0) { S.n_cand = 0; S.overflow = 0; }
         __syncthreads();
-        hist_pass_all<SMALLEST>(vals, n, 21, 2047u, 0u, 0u, S.hist, stage);
+        hist_pass_all<SMALLEST>(vals, n, 21, 2047u, 0u, 0u, S.hist);
         __syncthreads();
         pick_bin<NW>(S.hist, k, S.bc, S.part);
         __syncthreads();
@@ -177,7 +173,7 @@ __device__ __forceinline__ void select_emit(const float* vals, int n, int k, boo
 #pragma unroll
             for (int j = 0; j < 4; ++j) {
                 const int i = base + 32 * j + lane;
-                kv[j] = i >= w1 ? 0u : stage ? stage[i] : select_image<SMALLEST>(vals[i]);
+                kv[j] = i >= w1 ? 0u : select_image<SMALLEST>(vals[i]);
             }
 #pragma unroll
             for (int j = 0; j < 4; ++j) {
@@ -211,11 +207,11 @@ __device__ __forceinline__ void select_emit(const float* vals, int n, int k, boo
         __syncthreads();
         if (listed) {
             for (int j = threadIdx.x; j < n_cand; j += blockDim.x) {
-                const uint32_t key = stage ? stage[cand[j]] : select_image<SMALLEST>(vals[cand[j]]);
+                const uint32_t key = select_image<SMALLEST>(vals[cand[j]]);
                 hist_add(S.hist, key & 1023, (key & mask) == prefix);
             }
         } else {
-            hist_pass_all<SMALLEST>(vals, n, 0, 1023u, prefix, mask, S.hist, nullptr);
+            hist_pass_all<SMALLEST>(vals, n, 0, 1023u, prefix, mask, S.hist);
         }
         __syncthreads();
         pick_bin<NW>(S.hist, remaining, S.bc, S.part);
@@ -229,7 +225,7 @@ __device__ __forceinline__ void select_emit(const float* vals, int n, int k, boo
         if (masked && listed) {
             for (int j = threadIdx.x; j < n_cand; j += blockDim.x) {
                 const int i = cand[j];
-                const uint32_t key = stage ? stage[i] : select_image<SMALLEST>(vals[i]);
+                const uint32_t key = select_image<SMALLEST>(vals[i]);
                 if (key > kth) atomicOr(&sel_mask[i >> 5], 1u << (i & 31));
                 else if (key == kth) atomicOr(&tie_mask[i >> 5], 1u << (i & 31));
             }
@@ -239,7 +235,7 @@ __device__ __forceinline__ void select_emit(const float* vals, int n, int k, boo
 #pragma unroll
                 for (int j = 0; j < 4; ++j) {
                     const int i = base + 32 * j + lane;
-                    kv[j] = i >= w1 ? 0u : stage ? stage[i] : select_image<SMALLEST>(vals[i]);
+                    kv[j] = i >= w1 ? 0u : select_image<SMALLEST>(vals[i]);
                 }
 #pragma unroll
                 for (int j = 0; j < 4; ++j) {
@@ -266,7 +262,7 @@ __device__ __forceinline__ void select_emit(const float* vals, int n, int k, boo
 #pragma unroll
             for (int j = 0; j < 4; ++j) {
                 const int i = base + 32 * j + lane;
-                kv[j] = i >= w1 ? 0u : stage ? stage[i] : select_image<SMALLEST>(vals[i]);
+                kv[j] = i >= w1 ? 0u : select_image<SMALLEST>(vals[i]);
             }
 #pragma unroll
             for (int j = 0; j < 4; ++j) {
@@ -308,7 +304,7 @@ __device__ __forceinline__ void select_emit(const float* vals, int n, int k, boo
         for (int base = w0; base < w1; base += 32) {
             const int i = base + lane;
             const bool in = i < w1;
-            const uint32_t key = in ? (stage ? stage[i] : select_image<SMALLEST>(vals[i])) : 0u;
+            const uint32_t key = in ? select_image<SMALLEST>(vals[i]) : 0u;
             const bool tie = any && in && key == kth;
             const unsigned tb = __ballot_sync(FULL, tie);
             const bool chosen = any && in && (key > kth || (tie && __popc(tb & lt) < ties_left));
@@ -768,34 +764,26 @@ __device__ __forceinline__ void select_regs(const float* vals, int n, int k, Reg
     }
 }
 
-// Shared-memory plan of one selection over n elements within `budget_bytes`: a candidate list of
-// at least `min_cand` entries, the masks when they fit, the staged images when asked for and they
-// fit, and whatever is left goes to a longer candidate list (up to 16384 entries: a quarter binade
-// rarely holds more).
-inline Layout plan_layout(int64_t n, bool want_stage, size_t budget_bytes, int min_cand, int nw) {
-    Layout L;
-    L.groups = 0; L.stage_words = 0; L.keyed = 0; L.tile_words = 0;
-    size_t used = (size_t)min_cand * 4;
+// Shared-memory plan of one selection over n elements in memory within `budget_bytes`, by blocks of nw warps: the masks, the lean path's
+// tiles and, in what they leave, its list of up to 32768 candidates (a quarter binade rarely holds more).  Where the masks leave no room
+// for that (over half a million elements in 200 KB), the general path's: a candidate list of `min_cand` to 16384 entries, and the masks
+// when they fit.
+inline Layout plan_layout(int64_t n, size_t budget_bytes, int min_cand, int nw) {
+    Layout L = {};
+    const size_t words = budget_bytes / 4;
     const size_t groups = ((size_t)((n + 31) / 32) + 3) & ~size_t(3);       // whole 16-byte groups: what follows stays aligned
-    if (used + 2 * groups * 4 <= budget_bytes) { L.groups = (int)groups; used += 2 * groups * 4; }
-    if (want_stage && used + (size_t)n * 4 <= budget_bytes) { L.stage_words = (int)n; used += (size_t)n * 4; }
-    size_t cap = (budget_bytes - used) / 4 + (size_t)min_cand;
-    const size_t want = (size_t)(n < 16384 ? n : 16384);
-    if (cap > want) cap = want;
-    if (cap < (size_t)min_cand) cap = (size_t)min_cand;
-    L.cand_cap = (int)cap;
-    L.keyed = 0;
-    if (L.groups > 0 && L.stage_words == 0) {
-        // the lean path: indices and images side by side, twice the words when they fit
-        const size_t tiles = (size_t)nw * lean_loads_per_lane(nw) * 128;
-        const size_t fixed = 2 * groups + tiles;
-        if (budget_bytes / 4 > fixed) {
-            // words: index and image of every candidate, in shares of whole 4-entry groups for up to 32 warps
-            size_t keyed = (2 * (size_t)(n < 32768 ? n : 32768) + 255) & ~size_t(255);
-            const size_t room = (budget_bytes / 4 - fixed) & ~size_t(255);
-            if (keyed > room) keyed = room;
-            if (keyed >= 512) { L.cand_cap = (int)keyed; L.keyed = 1; L.tile_words = (int)tiles; }
-        }
+    if (2 * groups + (size_t)min_cand <= words) L.groups = (int)groups;
+    const size_t tiles = (size_t)nw * lean_loads_per_lane(nw) * 128;
+    if (L.groups > 0 && words >= 2 * groups + tiles + 512) {
+        // words: index and image of every candidate, in shares of whole 4-entry groups for up to 32 warps
+        const size_t most = (2 * (size_t)(n < 32768 ? n : 32768) + 255) & ~size_t(255);
+        const size_t room = (words - 2 * groups - tiles) & ~size_t(255);
+        L.cand_cap = (int)(most < room ? most : room);
+        L.keyed = 1;
+        L.tile_words = (int)tiles;
+    } else {
+        const size_t room = words - 2 * (size_t)L.groups;
+        L.cand_cap = (int)(room < 16384 ? room : 16384);
     }
     return L;
 }
