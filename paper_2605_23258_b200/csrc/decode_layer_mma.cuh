@@ -378,6 +378,49 @@ decode_layer_mma(const __nv_bfloat16* q, const __grid_constant__ dbf::Maps maps,
     }
 }
 
+// Two neighbouring elements of a column's records, which begin at src and lie g * REC apart, under the factors f of its splits.
+__device__ __forceinline__ void merge_two(const float* src, int n_splits, int g, const float (&fs)[32], float& v0, float& v1) {
+    v0 = v1 = 0.f;
+    for (int s0 = 0; s0 < n_splits; s0 += 8) {
+        float2 x[8];
+#pragma unroll
+        for (int k = 0; k < 8; ++k) x[k] = *reinterpret_cast<const float2*>(src + (size_t)min(s0 + k, n_splits - 1) * g * REC);   // always a valid record
+#pragma unroll
+        for (int k = 0; k < 8; ++k) {
+            const float f = s0 + k < n_splits ? fs[s0 + k] : 0.f;
+            v0 = fmaf(f, x[k].x, v0);
+            v1 = fmaf(f, x[k].y, v1);
+        }
+    }
+}
+// d += rows Wr and Wr + 8 of the map (this thread's columns of them) times the key sums of four input heads, the first or the last four.
+__device__ __forceinline__ void map_rows_times_keys(const __nv_bfloat16* Wr, const __nv_bfloat16 (&akh)[8][HKV * 128],
+                                                    const __nv_bfloat16 (&akl)[8][HKV * 128], int half, int row, int quarter, float (&d)[4]) {
+    constexpr int KD = HKV * 128;
+    const uint4* Wr0 = reinterpret_cast<const uint4*>(Wr);
+    const uint4* Wr1 = Wr0 + 8 * (KD / 8);                 // row + 8
+#pragma unroll 2
+    for (int kc = half * (HKV / 2); kc < (half + 1) * (HKV / 2); ++kc) {                     // 128 columns a time: 16 pieces of 16 bytes per row
+        uint4 A[8];
+#pragma unroll
+        for (int jj = 0; jj < 4; ++jj) {
+            A[2 * jj + 0] = Wr0[kc * 16 + quarter + 4 * jj];
+            A[2 * jj + 1] = Wr1[kc * 16 + quarter + 4 * jj];
+        }
+#pragma unroll
+        for (int jj = 0; jj < 4; ++jj) {
+            const uint4 a0 = A[2 * jj], a1 = A[2 * jj + 1];
+            const int col = kc * 128 + 8 * (quarter + 4 * jj);
+            const uint4 bh = *reinterpret_cast<const uint4*>(&akh[row][col]);      // B column = head `row`
+            const uint4 bl = *reinterpret_cast<const uint4*>(&akl[row][col]);
+            dbf::mma_16(d, a0.x, a1.x, a0.y, a1.y, bh.x, bh.y);
+            dbf::mma_16(d, a0.x, a1.x, a0.y, a1.y, bl.x, bl.y);
+            dbf::mma_16(d, a0.z, a1.z, a0.w, a1.w, bh.z, bh.w);
+            dbf::mma_16(d, a0.z, a1.z, a0.w, a1.w, bl.z, bl.w);
+        }
+    }
+}
+
 // Merge for the same shapes: combines the splits' records of a unit, applies row block h of the layer's map
 // to the merged key sums of all heads and normalises,
 //   o_a = (sum_s f_s acc_v_s + W[h rows] sum_s f_s acc_k_s) / sum_s f_s l_s,   f_s = exp(m_s - max m).
@@ -422,18 +465,8 @@ decode_layer_merge_mma(const float* partial, const __nv_bfloat16* W, int L, int 
     for (int i = tid; i < g * PAIRS; i += MERGE_THREADS) {
         const int a = i / PAIRS, e = (i - a * PAIRS) * 2;
         const float* src = rec0 + (size_t)a * REC + 2 + e;
-        float v0 = 0.f, v1 = 0.f;
-        for (int s0 = 0; s0 < n_splits; s0 += 8) {
-            float2 x[8];
-#pragma unroll
-            for (int k = 0; k < 8; ++k) x[k] = *reinterpret_cast<const float2*>(src + (size_t)min(s0 + k, n_splits - 1) * g * REC);   // always a valid record
-#pragma unroll
-            for (int k = 0; k < 8; ++k) {
-                const float f = s0 + k < n_splits ? fs[a][s0 + k] : 0.f;
-                v0 = fmaf(f, x[k].x, v0);
-                v1 = fmaf(f, x[k].y, v1);
-            }
-        }
+        float v0, v1;
+        merge_two(src, n_splits, g, fs[a], v0, v1);
         if (e < 128) { accv[a][e] = v0; accv[a][e + 1] = v1; }
         else {
             const uint32_t hi = dbf::pack_bf16(v0, v1);
@@ -445,29 +478,8 @@ decode_layer_merge_mma(const float* partial, const __nv_bfloat16* W, int L, int 
     // rows 16 (wid % 8) .. of the head's block of the map times the key sums of four input heads
     {
         const int half = wid >> 3, r0 = 16 * (wid & 7) + row;
-        const uint4* Wr0 = reinterpret_cast<const uint4*>(W + ((size_t)layer * KD + (size_t)h * 128 + r0) * KD);
-        const uint4* Wr1 = Wr0 + 8 * (KD / 8);                 // row + 8
         float d[4] = {0.f, 0.f, 0.f, 0.f};
-#pragma unroll 2
-        for (int kc = half * (HKV / 2); kc < (half + 1) * (HKV / 2); ++kc) {                     // 128 columns a time: 16 pieces of 16 bytes per row
-            uint4 A[8];
-#pragma unroll
-            for (int jj = 0; jj < 4; ++jj) {
-                A[2 * jj + 0] = Wr0[kc * 16 + quarter + 4 * jj];
-                A[2 * jj + 1] = Wr1[kc * 16 + quarter + 4 * jj];
-            }
-#pragma unroll
-            for (int jj = 0; jj < 4; ++jj) {
-                const uint4 a0 = A[2 * jj], a1 = A[2 * jj + 1];
-                const int col = kc * 128 + 8 * (quarter + 4 * jj);
-                const uint4 bh = *reinterpret_cast<const uint4*>(&akh[row][col]);      // B column = head `row`
-                const uint4 bl = *reinterpret_cast<const uint4*>(&akl[row][col]);
-                dbf::mma_16(d, a0.x, a1.x, a0.y, a1.y, bh.x, bh.y);
-                dbf::mma_16(d, a0.x, a1.x, a0.y, a1.y, bl.x, bl.y);
-                dbf::mma_16(d, a0.z, a1.z, a0.w, a1.w, bh.z, bh.w);
-                dbf::mma_16(d, a0.z, a1.z, a0.w, a1.w, bl.z, bl.w);
-            }
-        }
+        map_rows_times_keys(W + ((size_t)layer * KD + (size_t)h * 128 + r0) * KD, akh, akl, half, row, quarter, d);
         // d[0], d[1]: row `row`, heads 2 quarter and 2 quarter + 1; d[2], d[3]: row `row` + 8
         if (2 * quarter < g) { pw[half][2 * quarter][r0] = d[0]; pw[half][2 * quarter][r0 + 8] = d[2]; }
         if (2 * quarter + 1 < g) { pw[half][2 * quarter + 1][r0] = d[1]; pw[half][2 * quarter + 1][r0 + 8] = d[3]; }
@@ -481,7 +493,7 @@ decode_layer_merge_mma(const float* partial, const __nv_bfloat16* W, int L, int 
 
 // The same for many units: a block takes `seqs` sequences of one (layer, head), whose query heads are the product's columns.  The
 // map's rows, 256 KB a block, are what most of a merge fetches from L2 where units are many and their records few.  A kernel of its
-// own: as a variant of the other one it cost that one 1 to 7 % (six pairs of 2215 rows, 25.5 us a step).
+// own: as two instances of one body the other one lost 1 to 5 % (a pair of 2215 rows 34.3 -> 36.1 us a step, 40 of 349 rows 52.6 -> 55.4).
 // grid (layers * HKV * ceil(batch / seqs)), 512 threads, seqs * g <= 8.
 template <typename TO>
 __global__ void __launch_bounds__(MERGE_THREADS)
@@ -524,18 +536,8 @@ decode_layer_merge_shared(const float* partial, const __nv_bfloat16* W, int L, i
     for (int i = tid; i < n_heads * PAIRS; i += MERGE_THREADS) {
         const int a = i / PAIRS, e = (i - a * PAIRS) * 2, n_splits = splits[a];
         const float* src = records_of(a) + 2 + e;
-        float v0 = 0.f, v1 = 0.f;
-        for (int s0 = 0; s0 < n_splits; s0 += 8) {
-            float2 x[8];
-#pragma unroll
-            for (int k = 0; k < 8; ++k) x[k] = *reinterpret_cast<const float2*>(src + (size_t)min(s0 + k, n_splits - 1) * g * REC);   // always a valid record
-#pragma unroll
-            for (int k = 0; k < 8; ++k) {
-                const float f = s0 + k < n_splits ? fs[a][s0 + k] : 0.f;
-                v0 = fmaf(f, x[k].x, v0);
-                v1 = fmaf(f, x[k].y, v1);
-            }
-        }
+        float v0, v1;
+        merge_two(src, n_splits, g, fs[a], v0, v1);
         if (e < 128) { accv[a][e] = v0; accv[a][e + 1] = v1; }
         else {
             const uint32_t hi = dbf::pack_bf16(v0, v1);
@@ -547,29 +549,8 @@ decode_layer_merge_shared(const float* partial, const __nv_bfloat16* W, int L, i
     // rows 16 (wid % 8) .. of the head's block of the map times the key sums of four input heads
     {
         const int half = wid >> 3, r0 = 16 * (wid & 7) + row;
-        const uint4* Wr0 = reinterpret_cast<const uint4*>(W + ((size_t)layer * KD + (size_t)h * 128 + r0) * KD);
-        const uint4* Wr1 = Wr0 + 8 * (KD / 8);                 // row + 8
         float d[4] = {0.f, 0.f, 0.f, 0.f};
-#pragma unroll 2
-        for (int kc = half * (HKV / 2); kc < (half + 1) * (HKV / 2); ++kc) {                     // 128 columns a time: 16 pieces of 16 bytes per row
-            uint4 A[8];
-#pragma unroll
-            for (int jj = 0; jj < 4; ++jj) {
-                A[2 * jj + 0] = Wr0[kc * 16 + quarter + 4 * jj];
-                A[2 * jj + 1] = Wr1[kc * 16 + quarter + 4 * jj];
-            }
-#pragma unroll
-            for (int jj = 0; jj < 4; ++jj) {
-                const uint4 a0 = A[2 * jj], a1 = A[2 * jj + 1];
-                const int col = kc * 128 + 8 * (quarter + 4 * jj);
-                const uint4 bh = *reinterpret_cast<const uint4*>(&akh[row][col]);      // B column = head `row`
-                const uint4 bl = *reinterpret_cast<const uint4*>(&akl[row][col]);
-                dbf::mma_16(d, a0.x, a1.x, a0.y, a1.y, bh.x, bh.y);
-                dbf::mma_16(d, a0.x, a1.x, a0.y, a1.y, bl.x, bl.y);
-                dbf::mma_16(d, a0.z, a1.z, a0.w, a1.w, bh.z, bh.w);
-                dbf::mma_16(d, a0.z, a1.z, a0.w, a1.w, bl.z, bl.w);
-            }
-        }
+        map_rows_times_keys(W + ((size_t)layer * KD + (size_t)h * 128 + r0) * KD, akh, akl, half, row, quarter, d);
         // d[0], d[1]: row `row`, heads 2 quarter and 2 quarter + 1; d[2], d[3]: row `row` + 8
         if (2 * quarter < n_heads) { pw[half][2 * quarter][r0] = d[0]; pw[half][2 * quarter][r0 + 8] = d[2]; }
         if (2 * quarter + 1 < n_heads) { pw[half][2 * quarter + 1][r0] = d[1]; pw[half][2 * quarter + 1][r0 + 8] = d[3]; }
