@@ -16,7 +16,7 @@
 // them for the tensor cores waits for all that it has in flight, the next stages' copies among them: with eight warps filling
 // every stage together, a step took the latency of memory (245 us for 16 layers of 4914 listed tokens and 8 heads).  So every
 // stage has a loader warp of its own, which has nothing else in flight: 176 us, and 180 in pairs.  There the issue of the products
-// was the longest chain of a step (see the MMA role): 157 us, of which the products need 75 at the tensor rate, 104 at the rate of a
+// was the longest chain of a step (see the MMA role): 157 us (in a graph by itself 143, by single blocks 161), of which the products need 75 at the tensor rate, 104 at the rate of a
 // library product.  The products take two output heads at a time (a third fewer bytes than head by head), and the value rows go
 // straight to the epilogue's registers.
 //

@@ -2,6 +2,8 @@
 each is cut in two, and so many that blocks' ranges end inside tiles.  Bound: fp32 accumulation of exact products over
 Hkv d inputs in any order, |eps - want| <= 2 sqrt(want) |delta| + |delta|^2 + 2^-20 want, delta_c = (D + 2) 2^-23
 (|v_c| + sum |W||k|)."""
+import re
+
 import numpy as np
 import pytest
 import torch
@@ -61,30 +63,27 @@ def test_residual_layer_values_at_16_bytes(layers, Hkv, n_idx):
     assert torch.equal(eps[0], eps[1])
 
 
-def test_few_heads_cost_no_pairs():
-    """One layer of one head is the same products as one unit with a map of its own.  In pairs of blocks, which pay for more heads
-    only, the call took 2.2 to 2.35 times as long; a block by itself takes 1.8 to 1.9 times."""
-    N, d, n_idx = 600, 128, 300
-    gen = torch.Generator(device=DEV).manual_seed(3)
-    K, V = (torch.randn(1, N, d, generator=gen, device=DEV).to(torch.bfloat16) for _ in range(2))
-    W = (torch.randn(1, d, d, generator=gen, device=DEV) / np.sqrt(d)).to(torch.bfloat16)
-    idx = torch.randperm(N, generator=gen, device=DEV)[:n_idx].sort().values.to(torch.int32)[None].contiguous()
-    sh = vec.Shape(1, 1, 1, 1, d, vec.VECTOR_BF16, 16)
-    eps = torch.empty(1, n_idx, device=DEV)
-    graphs, us = [], [[], []]
-    for call in (vec.vector_residual, vec.vector_residual_layer):
-        call(sh, K, V, W, N, idx, n_idx, eps)
+def _blocks_a_tile(layers, Hkv, n_idx):
+    """Blocks that share a tile in the kernel that this call launches, by its name in a profile."""
+    N, d = 2 * n_idx, 128
+    K = torch.zeros(layers * Hkv, N, d, dtype=torch.bfloat16, device=DEV)
+    W = torch.zeros(layers, Hkv * d, Hkv * d, dtype=torch.bfloat16, device=DEV)
+    idx = torch.arange(n_idx, dtype=torch.int32, device=DEV).repeat(layers, 1).contiguous()
+    eps = torch.empty(layers, n_idx, device=DEV)
+    sh = vec.Shape(1, layers, Hkv, Hkv, d, vec.VECTOR_BF16, 16)
+    vec.vector_residual_layer(sh, K, K, W, N, idx, n_idx, eps)
+    with torch.profiler.profile(activities=[torch.profiler.ProfilerActivity.CUDA]) as prof:
+        vec.vector_residual_layer(sh, K, K, W, N, idx, n_idx, eps)
         torch.cuda.synchronize()
-        graphs.append(torch.cuda.CUDAGraph())
-        with torch.cuda.graph(graphs[-1]):
-            for _ in range(40):
-                call(sh, K, V, W, N, idx, n_idx, eps)
-    for _ in range(20):
-        for g, t in zip(graphs, us):
-            a, e = (torch.cuda.Event(enable_timing=True) for _ in range(2))
-            a.record()
-            g.replay()
-            e.record()
-            torch.cuda.synchronize()
-            t.append(a.elapsed_time(e))
-    assert min(us[1]) < 2.05 * min(us[0]), [min(t) for t in us]
+    names = [e.name for e in prof.events() if "residual_layer_tc" in e.name]
+    if not names:
+        pytest.skip("no kernel names from the profiler")
+    return int(re.search(r"residual_layer_tc<.*?(\d)\)?>", names[0]).group(1))
+
+
+def test_few_heads_and_short_lists_take_single_blocks():
+    """Pairs of blocks cost 2 us before their first item: one head of 300 tokens takes 10.5 us so and 8.5 by blocks by themselves."""
+    for shape in ((1, 1, 300), (16, 1, 5000), (16, 2, 5000), (1, 3, 300), (1, 4, 300)):
+        assert _blocks_a_tile(*shape) == 1, shape
+    for shape in ((16, 8, 5000), (1, 8, 1500), (37, 5, 1500)):
+        assert _blocks_a_tile(*shape) == 2, shape
