@@ -340,33 +340,38 @@ static vector_status select_kernels_setup() {
     return VECTOR_OK;
 }
 
-// Warps of a block that passes over memory, 0: the input in registers.  U lists of n elements.  Up to 8192 elements registers win by
-// up to twice, beyond that only where every list has a multiprocessor to itself (one block fills its register file); many lists are
-// served best by the small blocks, whose phases of latency overlap, until their share of shared memory gets short.  us, registers /
-// 8 warps / 16 warps.  Step 1: 2368 lists of 3000 elements 41 / 41 / 66; 444 of 6500 14.4 / 14.5 / 18.8, 592 of 6500 17.0 / 14.8 /
-// 21.2; 148 of 12000 10.6 / 13.6 / 10.9, 296 of 12000 15.0 / 15.8 / 14.1, 592 of 12000 27.7 / 21.3 / 26.3, 1184 of 14000 57 / 70 / 62,
-// 148 of 20011 13.8 / 23.8 / 16.4, 296 of 20011 26.5 / 32.4 / 21.7, 1184 of 20011 109 / 109 / 99.  Step 3: 2368 lists of 8192 108 /
-// 111 / 135; 148 of 12000 12.8 / 21.9 / 16.1, 296 of 12000 24.5 / 25.9 / 22.4, 592 of 12000 49 / 41 / 45, 640 of 16384 77 / 76 / 73, 1184 of 16384 126 / 107 /
-// 113; 148 of 20011 in 64 registers a thread, which do not hold image and token, 41.9 / 35.0 / 25.3; 888 of 20011 - / 125 / 118, 1184
-// of 20011 - / 149 / 155, of 26000 - / 179 / 177.
-static int selection_warps(int64_t n, int U, bool step3) {
-    const int sms = sm_count();
-    if (n <= (step3 ? 8192 : 4096)) return 0;
-    if (n <= 8192) return U <= 3 * sms ? 0 : 8;
-    if (n <= SEL_REGS16) {
-        if (U <= sms) return 0;
-        if (U <= 2 * sms) return 16;
-        if (step3) return U <= 4 * sms || U >= 8 * sms ? 8 : 16;          // a second round of small blocks that is nearly empty
-        return n <= 12288 ? 8 : U <= 4 * sms ? 16 : 0;
-    }
-    if (!step3 && n <= SEL_REGS && U <= sms) return 0;
-    if (step3 && n <= 24576 && U >= 8 * sms) return 8;
-    return n < SEL_LONG ? 16 : 32;
-}
 static Layout selection_layout(int64_t n, int nw) {
     const size_t budget = nw == 8 ? SEL_SMEM_SHORT : nw == 16 ? SEL_SMEM_MID : SEL_SMEM_LONG;
-    const int min_cand = nw == 8 ? 1024 : 2048;
-    return sel::plan_layout(n, budget, min_cand, nw);
+    return sel::plan_layout(n, budget, nw == 8 ? 1024 : 2048, nw);
+}
+// Warps of a block that passes over memory, 0: the input in registers.  Registers win for every count of short lists and, up to their
+// length, where a list has a multiprocessor to itself.  Many longer lists are served best by the small blocks, whose phases of latency
+// overlap; their second round (4 to 8 lists a multiprocessor) is nearly empty.
+// Step 1 writes its list out in one sweep where it fits the candidates' place in shared memory, by scattered stores where it does
+// not, which decides between the forms.  us, scores from HBM, registers / 8 / 16 warps, `*`: the list does not fit.  148 lists of 12000
+// 10.6 / 13.6 / 10.9, of 20011 14.4 / 26.8 / 19.2; 256 of 14000 16.5 / 19.8 / 15.8, of 20011 27.8 / 29.8 / 23.3; 444 of 6500 14.4 / 14.5 / 18.8, 592 of
+// 8192 19.5 / 17.1 / 23.7; 592 of 14000, 0.3 of them listed, 30.6 / 26.1 / 30.6, half of them 30.6 / 40.4* / 31.8; 592 of 26000, 0.15 listed, 62.9 /
+// 43.5 / 48.2, 0.3 listed 62.2 / 54.3* / 48.9, 0.8 listed 63.1 / 97.3* / 94.3*; 640 of 32767, 0.15 listed, 86 / 85 / 79; 1184 of 16384, 0.3 listed,
+// 63 / 56 / -, half of them 64 / 84* / -.
+static int pool_select_warps(int64_t n, int U, int64_t n_pool) {
+    const int sms = sm_count();
+    auto list_fits = [&](int nw) { return n_pool <= selection_layout(n, nw).cand_cap; };
+    if (n <= 4096 || (n <= SEL_REGS && U <= sms)) return 0;
+    if (n <= 8192) return U <= 3 * sms || !list_fits(8) ? 0 : 8;
+    if (n <= SEL_REGS) {
+        if (U > 2 * sms && list_fits(8) && (n <= 20480 || U <= 4 * sms || U >= 8 * sms)) return 8;
+        return (n <= SEL_REGS16 ? U <= 2 * sms : list_fits(16)) ? 16 : 0;
+    }
+    return n < SEL_LONG ? 16 : 32;
+}
+// Step 3, us as above: 148 lists of 12000 12.8 / 21.9 / 16.1, 296 of 12000 24.5 / 25.9 / 22.4, 592 of 12000 49 / 41 / 45, 640 of 16384 77 / 76 / 73, 1184
+// of 16384 126 / 107 / 113; 2368 of 5000 84 / 82 / 111, of 8192 108 / 111 / 135; 148 of 20011 in 64 registers a thread, which do not hold image
+// and token, 41.9 / 35.0 / 25.3; 888 of 20011 - / 125 / 118, 1184 of 20011 - / 149 / 155, of 26000 - / 179 / 177.
+static int truncate_warps(int64_t n, int U) {
+    const int sms = sm_count();
+    if (n <= 8192 || (n <= SEL_REGS16 && U <= sms)) return 0;
+    if (n <= SEL_REGS16 ? U > 2 * sms && (U <= 4 * sms || U >= 8 * sms) : n <= 24576 && U >= 8 * sms) return 8;
+    return n < SEL_LONG ? 16 : 32;
 }
 
 static vector_status launch_pool_select(const Dims& dm, const vector_budget* budget, const float* scores, int32_t* pool,
@@ -374,7 +379,7 @@ static vector_status launch_pool_select(const Dims& dm, const vector_budget* bud
     vector_status rc = select_kernels_setup();
     if (rc != VECTOR_OK) return rc;
     const int64_t n = budget->n_tokens;
-    const int nw = selection_warps(n, dm.U, false);
+    const int nw = pool_select_warps(n, dm.U, budget->n_pool);
     if (nw == 0) {
         auto kern = n <= 2048 ? pool_select_regs<16, 4> : n <= 4096 ? pool_select_regs<16, 8> : n <= 8192 ? pool_select_regs<16, 16>
                   : n <= SEL_REGS16 ? pool_select_regs<16, 32> : pool_select_regs<32, 32>;
@@ -395,7 +400,7 @@ static vector_status launch_truncate(const Dims& dm, const vector_budget* budget
     if (rc != VECTOR_OK) return rc;
     // dependent: may start (and clear the tier map) while the kernel before it in the stream drains
     const int64_t n = budget->n_pool;
-    const int nw = selection_warps(n, dm.U, true);
+    const int nw = truncate_warps(n, dm.U);
     if (nw == 0) {
         auto kern = n <= 2048 ? truncate_regs<16, 4> : n <= 4096 ? truncate_regs<16, 8> : n <= 8192 ? truncate_regs<16, 16>
                   : truncate_regs<32, 16>;

@@ -1,4 +1,4 @@
-"""Selections where the form changes with the number of lists as well as their length: exact in every list (indices and tiers are whole
+"""Selections where the form changes with the number of lists, their length and what is taken of them: exact in every list (indices and tiers are whole
 numbers), against a stable sort.  And Step 3 just past the lengths that registers hold: 22 % more elements took 2.6 times as long
 when their images and tokens were kept in registers that were not there; passing over memory it is 1.4 times."""
 import pytest
@@ -21,11 +21,13 @@ def _lists(share, n, ties):
 
 @pytest.mark.parametrize("ties", [False, True])
 @pytest.mark.parametrize("share,n", [(0.9, 16384), (0.9, 16385), (0.9, 32768), (1, 8192), (1, 8193), (1, 16385), (2, 12288), (2, 12289), (3, 4096), (3, 4097),
-                                     (3, 8192), (3, 16384), (4, 12289), (4, 16384), (4.5, 8193), (8, 4097), (8, 8193), (8, 16385), (8, 24576), (8, 24577)])
-def test_forms(share, n, ties):
+                                     (3, 8192), (3, 16384), (4, 12289), (4, 16384), (4.5, 8193), (4.5, 20481), (8, 4097), (8, 8193), (8, 16385), (8, 24576),
+                                     (8, 24577), (3, 32768)])
+@pytest.mark.parametrize("taken", [0.1, 2 / 3, 0.95])
+def test_forms(share, n, ties, taken):
     U, v = _lists(share, n, ties)
     sh = vec.Shape(1, 1, U, U, 64, vec.VECTOR_F32, 1)
-    k = n // 3 * 2
+    k = int(n * taken) // 2 * 2
     out = torch.empty(U, k, dtype=torch.int32, device=DEV)
     vec.vector_pool_select(sh, vec.Budget(n, k, 0, k, 0, k, n - k), v, out)
     want = torch.sort(v, dim=1, descending=True, stable=True).indices[:, :k].sort(dim=1).values
