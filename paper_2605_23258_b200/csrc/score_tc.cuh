@@ -25,7 +25,7 @@
 // All hand-offs are mbarriers; every wait is bounded and records a fault code.
 // Units of at most 128 rows (NB = 1) give every warpgroup whole tiles: 280 units of 96 rows over 78299 keys 2.60 -> 1.88 ms with
 // their pooling.  Few units are pooled by the second pass itself: 8 units of 256 rows over 8192 keys 27.4 -> 23.3 us.
-// Measured at 64 channels, 128 units of 4 heads x 64 rows over 15013 keys: 0.298 ms (6.32 ms on CUDA cores).
+// Measured at 64 channels, 128 units of 4 heads x 64 rows over 15013 keys: 0.282 ms (6.32 ms on CUDA cores).
 #ifndef VECTOR_SCORE_TC_CUH_
 #define VECTOR_SCORE_TC_CUH_
 
@@ -213,40 +213,31 @@ __device__ __forceinline__ void block_teardown(Sync& sy) {
     }
 }
 
-// sum_i exp2(v[i] * c + n[i]) over 32 (pass 1) or 16 (pass 2) accumulator columns; n is either one value for all
-// columns (pass 1: minus the row's reference) or a table in shared memory (pass 2: minus the rows' lse).
-// Written in three stages (all FMAs, all exponentials, a tree of adds) so that the MUFU
-// operations issue back to back and nothing waits on the result of the one just before it.
-template <int C>
-__device__ __forceinline__ void sum_tree(const float (&e)[C], uint64_t& acc) {
-    uint64_t p[C / 2];
-#pragma unroll
-    for (int i = 0; i < C / 2; ++i) p[i] = pack2(e[2 * i], e[2 * i + 1]);
-#pragma unroll
-    for (int w = C / 4; w >= 1; w >>= 1)
-#pragma unroll
-        for (int i = 0; i < w; ++i) p[i] = add2(p[i], p[i + w]);
-    acc = add2(acc, p[0]);
-}
 // The exponential unit (16 results per clock per SM) is what bounds both passes, so POLY16 of every
 // 16 exponentials are evaluated on the FMA pipe instead: 2^x = 2^n p(f) with n = round(x),
 // f = x - n in [-1/2, 1/2] and p the degree-4 minimax polynomial of 2^f (relative error 2.7e-6);
-// n is added to the exponent field.  x is clamped to [-126, 128]: results below 2^-126 do not
-// matter to a sum whose largest term is of order one, and at the upper end (UPPER: the first pass, whose
-// reference lags; in the second no logit exceeds its row's normaliser by more than rounding) the exponent field must
-// not wrap -- 2^128 comes out as about 3.4e38 (or a NaN), which the overflow test of the first pass
-// (sum above 2^64, or not finite) catches, whereas a wrapped exponent would pass as a tiny term.
+// n is added to the exponent field.  x is clamped from below to -126: smaller results do not
+// matter to a sum whose largest term is of order one.  UPPER (the first pass, whose reference lags; in the second no logit exceeds
+// its row's normaliser by more than rounding): n is clamped from above to 128, as an integer while the polynomial is under way,
+// and multiplied in as 2^n: from 128 on that is infinite, which the overflow test of the first pass (sum above 2^64, or not
+// finite) catches, whereas a wrapped exponent would pass as a tiny term; an infinite x ends as a NaN, which it catches too.
 #ifndef VECTOR_SCORE_POLY16
 #define VECTOR_SCORE_POLY16 4
 #endif
 constexpr int POLY16 = VECTOR_SCORE_POLY16;
+// p * 2^n for t = 1.5 * 2^23 + n: one multiply-add on the bits.
+__device__ __forceinline__ float scaled(float p, float t) {
+    uint32_t r;
+    asm("mad.lo.u32 %0, %1, 8388608, %2;\n" : "=r"(r) : "r"(__float_as_uint(t)), "r"(__float_as_uint(p)));
+    return __uint_as_float(r);
+}
 template <bool UPPER>
-__device__ __forceinline__ void exp2_poly_pair(float x0, float x1, float& e0, float& e1) {
-    const float magic = 12582912.f;                    // 1.5 * 2^23: adding it leaves round(x) in the low mantissa bits
-    x0 = fmaxf(x0, -126.f);
-    x1 = fmaxf(x1, -126.f);
-    if (UPPER) { x0 = fminf(x0, 128.f); x1 = fminf(x1, 128.f); }
-    const uint64_t x2 = pack2(x0, x1);
+__device__ __forceinline__ uint64_t exp2_poly_pair(uint64_t x2) {
+    constexpr int BIAS = UPPER ? 127 : 0;
+    const float magic = 12582912.f + BIAS;             // 1.5 * 2^23: adding it leaves round(x) + BIAS in the low mantissa bits
+    float x0, x1, t0, t1;
+    unpack2(x2, x0, x1);
+    x2 = pack2(fmaxf(x0, -126.f), fmaxf(x1, -126.f));
     const uint64_t t2 = add2(x2, pack2(magic, magic));
     const uint64_t n2 = add2(t2, pack2(-magic, -magic));
     const uint64_t f2 = fma2(n2, pack2(-1.f, -1.f), x2);
@@ -255,43 +246,68 @@ __device__ __forceinline__ void exp2_poly_pair(float x0, float x1, float& e0, fl
     p2 = fma2(p2, f2, pack2(0.240247443318367f, 0.240247443318367f));
     p2 = fma2(p2, f2, pack2(0.6931217908859253f, 0.6931217908859253f));
     p2 = fma2(p2, f2, pack2(0.9999992847442627f, 0.9999992847442627f));
-    float p0, p1, t0, t1;
-    unpack2(p2, p0, p1);
     unpack2(t2, t0, t1);
-    e0 = __uint_as_float(__float_as_uint(p0) + (__float_as_uint(t0) << 23));
-    e1 = __uint_as_float(__float_as_uint(p1) + (__float_as_uint(t1) << 23));
-}
-// e[i] = 2^x[i] for C exponents: the first POLY16 of every 16 by polynomial, the rest by MUFU.
-template <bool UPPER, int C>
-__device__ __forceinline__ void exp2_all(const float (&x)[C], float (&e)[C]) {
-#pragma unroll
-    for (int i = 0; i < C; i += 2) {
-        if ((i & 15) < POLY16) exp2_poly_pair<UPPER>(x[i], x[i + 1], e[i], e[i + 1]);
-        else { e[i] = ex2(x[i]); e[i + 1] = ex2(x[i + 1]); }
+    if constexpr (UPPER) {
+        const int top = 0x4B400000 + 127 + 128;
+        return mul2(p2, pack2((uint32_t)min(__float_as_int(t0), top) << 23, (uint32_t)min(__float_as_int(t1), top) << 23));
+    } else {
+        float p0, p1;
+        unpack2(p2, p0, p1);
+        return pack2(scaled(p0, t0), scaled(p1, t1));
     }
 }
+// The exponentials of a pair of exponents, the `pair`-th of a run: POLY16 of every 16 are evaluated by polynomial, spread out among
+// the others.
+template <bool UPPER>
+__device__ __forceinline__ uint64_t exp2_pair(uint64_t x2, int pair) {
+    if (pair * (POLY16 / 2) % 8 < POLY16 / 2) return exp2_poly_pair<UPPER>(x2);
+    float x0, x1;
+    unpack2(x2, x0, x1);
+    x0 = ex2(x0);
+    x1 = ex2(x1);
+    return pack2(x0, x1);
+}
+// sum_i exp2(v[i] * c + n[i]) over 32 (pass 1) or 16 (pass 2) accumulator columns; n is either one value for all
+// columns (pass 1: minus the row's reference) or a table in shared memory (pass 2: minus the rows' lse).
+// 32 columns are written as two halves whose stages overlap -- the second half's exponents are formed between the first half's
+// exponentials -- so that a warp keeps the FMA pipe and the exponential unit busy together; with all FMAs, then all exponentials, then
+// all adds one after the other the four warps of a scheduler found themselves in the same stage (pass 1 alone, without its products:
+// 1.82 -> 1.65 ms for 64 units of 1024 rows and 131072 keys; 640 units, both passes, at the 1000 W cap: 50.7 -> 49.9 ms).
 __device__ __forceinline__ float exp2_sum32(const uint32_t (&v)[32], float c, float n) {
     const uint64_t c2 = pack2(c, c), n2 = pack2(n, n);
-    float x[32], e[32];
+    uint64_t x[16], acc[4];
 #pragma unroll
-    for (int i = 0; i < 32; i += 2) unpack2(fma2(pack2(v[i], v[i + 1]), c2, n2), x[i], x[i + 1]);
-    exp2_all<true>(x, e);
-    uint64_t acc = pack2(0.f, 0.f);
-    sum_tree(e, acc);
+    for (int i = 0; i < 8; ++i) x[i] = fma2(pack2(v[2 * i], v[2 * i + 1]), c2, n2);
+#pragma unroll
+    for (int h = 0; h < 16; h += 8) {
+        uint64_t e[8];
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+            e[i] = exp2_pair<true>(x[h + i], i);
+            if (h == 0) x[8 + i] = fma2(pack2(v[16 + 2 * i], v[17 + 2 * i]), c2, n2);
+        }
+#pragma unroll
+        for (int i = 0; i < 8; ++i) acc[i & 3] = h == 0 && i < 4 ? e[i] : add2(acc[i & 3], e[i]);
+    }
     float s0, s1;
-    unpack2(acc, s0, s1);
+    unpack2(add2(add2(acc[0], acc[1]), add2(acc[2], acc[3])), s0, s1);
     return s0 + s1;
 }
 __device__ __forceinline__ void exp2_acc16(const uint32_t (&v)[16], float c, const float4 (&n)[4], uint64_t& acc) {
     const uint64_t c2 = pack2(c, c);
-    float x[16], e[16];
+    uint64_t x[8];
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
-        unpack2(fma2(pack2(v[4 * i], v[4 * i + 1]), c2, pack2(n[i].x, n[i].y)), x[4 * i], x[4 * i + 1]);
-        unpack2(fma2(pack2(v[4 * i + 2], v[4 * i + 3]), c2, pack2(n[i].z, n[i].w)), x[4 * i + 2], x[4 * i + 3]);
+        x[2 * i] = fma2(pack2(v[4 * i], v[4 * i + 1]), c2, pack2(n[i].x, n[i].y));
+        x[2 * i + 1] = fma2(pack2(v[4 * i + 2], v[4 * i + 3]), c2, pack2(n[i].z, n[i].w));
     }
-    exp2_all<false>(x, e);
-    sum_tree(e, acc);
+#pragma unroll
+    for (int i = 0; i < 8; ++i) x[i] = exp2_pair<false>(x[i], i);
+#pragma unroll
+    for (int w = 4; w >= 1; w >>= 1)
+#pragma unroll
+        for (int i = 0; i < w; ++i) x[i] = add2(x[i], x[i + w]);
+    acc = add2(acc, x[0]);
 }
 __device__ __forceinline__ float max32(const uint32_t (&v)[32]) {
     float a = max3(__uint_as_float(v[0]), __uint_as_float(v[1]), __uint_as_float(v[2]));
