@@ -395,12 +395,11 @@ static vector_status launch_decode_bf16(const Dims& dm, const void* q, const vec
     const int apply_w = mode == 1 ? 0 : 1;
     const int cw = mode == 1 ? dpt::CONSUMERS : dm.rope ? Rope::CONSUMER_WARPS : Plain::CONSUMER_WARPS;   // records a block leaves per unit
     const T* Wp = (const T*)W;
-    // blocks of D g threads; up to 512 threads leave the merge 40 registers a thread with three blocks resident
-#define VEC_MERGE(TO, MAXT)                                                                                                  \
-    VEC_CUDA_CHECK(launch_maybe_dependent(true, dbf::decode_merge_bf16<TO, D, MAXT>, dim3(dm.U), dim3(D * dm.g), 0, st, rec, \
-                                          Wp, dm.LH, dm.g, pl, apply_w, cw, (TO*)out))
-    if (out_dtype == VECTOR_F32) { if (D * dm.g <= 512) VEC_MERGE(float, 512); else VEC_MERGE(float, 1024); }
-    else { if (D * dm.g <= 512) VEC_MERGE(T, 512); else VEC_MERGE(T, 1024); }
+#define VEC_MERGE(TO, HEADS)                                                                                                     \
+    VEC_CUDA_CHECK(launch_maybe_dependent(true, dbf::decode_merge_bf16<TO, D, HEADS>, dim3(dbf::MergeCfg<D, HEADS>::blocks(dm.U, sm_count())), \
+                                          dim3(dbf::MergeCfg<D, HEADS>::THREADS), 0, st, rec, Wp, dm.LH, dm.U, dm.g, pl, apply_w, cw, (TO*)out))
+    if (out_dtype == VECTOR_F32) { if (dm.g <= 2) VEC_MERGE(float, 2); else if (dm.g <= 4) VEC_MERGE(float, 4); else VEC_MERGE(float, 8); }
+    else { if (dm.g <= 2) VEC_MERGE(T, 2); else if (dm.g <= 4) VEC_MERGE(T, 4); else VEC_MERGE(T, 8); }
 #undef VEC_MERGE
     return VECTOR_OK;
 }

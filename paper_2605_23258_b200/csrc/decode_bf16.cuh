@@ -92,6 +92,7 @@ struct Plan {
     long long T;               // tiles of all units
     int B;                     // blocks
     int s_max;                 // record slots per unit
+    bool narrow;               // products of T and B fit 32 bits
 };
 __host__ __device__ inline Plan make_plan(int U, long long n_ret, long long n_apx, int max_blocks) {
     Plan p;
@@ -104,11 +105,16 @@ __host__ __device__ inline Plan make_plan(int U, long long n_ret, long long n_ap
     if (b > 11LL * U) b = 11LL * U;              // at most 12 record slots per unit (merge kernel limit)
     p.B = (int)(b < 1 ? 1 : b);
     p.s_max = (p.B + U - 1) / U + 1;
+    p.narrow = p.T * p.B < (1LL << 32);
     return p;
 }
-// Block b owns the tiles [b T / B, (b+1) T / B).
+// Block b owns the tiles [b T / B, (b+1) T / B).  A division of 64 bits takes some hundred instructions, which every thread of the
+// merge went through twice a unit.
 __host__ __device__ inline long long tile_begin(int b, const Plan& p) { return (long long)b * p.T / p.B; }
-__host__ __device__ inline int block_of_tile(long long x, const Plan& p) { return (int)(((x + 1) * p.B - 1) / p.T); }
+__host__ __device__ inline int block_of_tile(long long x, const Plan& p) {
+    if (p.narrow) return (int)((((unsigned)x + 1) * (unsigned)p.B - 1) / (unsigned)p.T);
+    return (int)(((x + 1) * p.B - 1) / p.T);
+}
 
 __device__ __forceinline__ void ldsm_x4(uint32_t addr, uint32_t& r0, uint32_t& r1, uint32_t& r2, uint32_t& r3) {
     asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4];\n"
@@ -367,24 +373,29 @@ __device__ __forceinline__ void store_key_sum(KeySums<D>& ks, int head, int c, f
     }
 }
 
-// Rows 16 mt .. + 15 of W times the key sums of n heads: pw[head][row].  One warp, M = 16 output channels, N = the heads
+// Rows 16 mt .. + 15 of W times the key sums of the heads.  One warp, M = 16 output channels, N = the heads
 // (padded to 8), K = D: the A fragments are read straight from the map in global memory, 16 bytes a load -- thread
 // (row r, quarter t) of a warp holds columns 8 (t + 4 jj) .. + 7 of rows r and r + 8, and the k slots of MMA step
 // 2 jj + h stand for columns 8 (t + 4 jj) + 4 h .. + 3, which the B fragments follow; the map's elements are bf16 as stored.
 // Three parts: the MMAs of the first start at zero and are added up in fp32, as the sums before them are (Cfg::EXACT).
+// d[0], d[1]: row lane / 4 of the 16, heads 2 (lane % 4) and + 1; d[2], d[3]: row lane / 4 + 8.
 template <int D>
-__device__ __forceinline__ void map_rows(const __nv_bfloat16* W, int mt, int n, const KeySums<D>& ks, float (&pw)[8][D], int lane) {
-    constexpr int PARTS = Cfg<D, false>::PARTS;
+__device__ __forceinline__ void map_fragments(const __nv_bfloat16* W, int mt, uint4 (&A)[D / 16], int lane) {
     constexpr int PIECES = D / 8;                                    // 16-byte pieces of a row of W
     const int row = lane >> 2, quarter = lane & 3;
     const uint4* Wu = reinterpret_cast<const uint4*>(W);
-    uint4 A[D / 16];
 #pragma unroll
     for (int jj = 0; jj < D / 32; ++jj) {
         A[2 * jj + 0] = Wu[(16 * mt + row) * PIECES + quarter + 4 * jj];
         A[2 * jj + 1] = Wu[(16 * mt + row + 8) * PIECES + quarter + 4 * jj];
     }
-    float d[4] = {0.f, 0.f, 0.f, 0.f}, small[4] = {0.f, 0.f, 0.f, 0.f};
+}
+template <int D>
+__device__ __forceinline__ void map_product(const uint4 (&A)[D / 16], const KeySums<D>& ks, float (&d)[4], int lane) {
+    constexpr int PARTS = Cfg<D, false>::PARTS;
+    const int row = lane >> 2, quarter = lane & 3;
+    float small[4] = {0.f, 0.f, 0.f, 0.f};
+    d[0] = d[1] = d[2] = d[3] = 0.f;
 #pragma unroll
     for (int jj = 0; jj < D / 32; ++jj) {
         const uint4 r0 = A[2 * jj], r1 = A[2 * jj + 1];
@@ -412,7 +423,15 @@ __device__ __forceinline__ void map_rows(const __nv_bfloat16* W, int mt, int n, 
     }
 #pragma unroll
     for (int e = 0; e < 4; ++e) d[e] += small[e];
-    // d[0], d[1]: row `row`, heads 2 quarter and 2 quarter + 1; d[2], d[3]: row `row` + 8
+}
+// The same, of n heads, into pw[head][row].
+template <int D>
+__device__ __forceinline__ void map_rows(const __nv_bfloat16* W, int mt, int n, const KeySums<D>& ks, float (&pw)[8][D], int lane) {
+    const int row = lane >> 2, quarter = lane & 3;
+    uint4 A[D / 16];
+    float d[4];
+    map_fragments<D>(W, mt, A, lane);
+    map_product<D>(A, ks, d, lane);
     if (2 * quarter < n) { pw[2 * quarter][16 * mt + row] = d[0]; pw[2 * quarter][16 * mt + row + 8] = d[2]; }
     if (2 * quarter + 1 < n) { pw[2 * quarter + 1][16 * mt + row] = d[1]; pw[2 * quarter + 1][16 * mt + row + 8] = d[3]; }
 }
@@ -727,96 +746,135 @@ decode_stream_bf16(const __nv_bfloat16* q, const __grid_constant__ Maps maps, Pl
     merge_unit();
 }
 
-// Merge: grid (U), D g threads -- thread (a, c) owns output dim c of head a.
-// Combines the records of a unit, applies the unit's map to the p-weighted key sum and normalises:
+// Merge: combines the records of a unit, applies the unit's map to the p-weighted key sum and normalises:
 //   o = (sum_j f_j s_j acc_v_j + W sum_j f_j acc_k_j) / sum_j f_j l_j,   f_j = exp(m_j - max m).
-// Every load of a phase is independent of the others, so a phase costs one memory latency.
-// The product W (sum f acc_k) runs on warp-level MMAs (map_rows).
-template <typename TO, int D, int MAXT>
-__global__ void __launch_bounds__(MAXT, MAXT == 512 ? 3 : 1)
-decode_merge_bf16(const float* partial, const __nv_bfloat16* W, int LH, int g,
+// A thread owns four channels of a head's value or key sum; its warp reads that head's headers, a record a lane, and hands the factors
+// round by shuffles, so that sums and headers share one memory latency and no barrier lies between them.  The map's fragments (MMAs,
+// map_fragments) are requested ahead of the wait for the streaming kernel, which does not touch the map: they come in while that
+// kernel drains.  What bounds it is that chain, one trip to L2 and a product a unit.
+// Up to four heads: as many blocks as are resident at once, each with an equal range of the units, ordered by map, so that the
+// sequences that share one find it in their block's registers; the next unit's records are requested before this one's product.
+// Up to eight heads: a block a unit, since registers for the next unit would cost the second resident block.
+// Blocks and records in flight as measured, us of a whole step in a graph: 2048 units of four heads of 128 channels 272 with two blocks
+// and six records, 275 with three and four, 278 with four and three; of one head 142 with three and three, 145 with four; 64 channels and
+// two heads 90.5 with blocks of 64 threads, 93 with 128.  Against a thread a channel, the factors through shared memory and the map
+// behind them: 2048 units of four heads 279 -> 272, 96 units of two heads 32.4 -> 29.4, 1536 units of eight heads and 1324 rows
+// 144 -> 128, with RoPE and 661 rows 121 -> 105.
+template <int D, int HEADS> struct MergeCfg {
+    static constexpr int THREADS = D == 64 && HEADS == 2 ? 64 : HEADS == 8 ? 4 * D : 2 * D;      // a head's sums take D / 2
+    static constexpr int RESIDENT = D == 128 ? (HEADS == 2 ? 3 : 2) : HEADS == 2 ? 8 : 4;
+    static constexpr int AHEAD = HEADS == 4 ? 6 : D == 128 && HEADS == 2 ? 3 : 4;      // records whose sums are requested together
+    static constexpr bool RANGE = HEADS <= 4;
+    static constexpr int MAP_WARPS = THREADS / 32 < D / 16 ? THREADS / 32 : D / 16, ROWS = D / 16 / MAP_WARPS;      // warps with rows of the map, blocks of 16 rows each
+    static constexpr int blocks(int U, int sms) { return RANGE && U > RESIDENT * sms ? RESIDENT * sms : U; }
+};
+template <typename TO, int D, int HEADS>
+__global__ void __launch_bounds__(MergeCfg<D, HEADS>::THREADS, MergeCfg<D, HEADS>::RESIDENT)
+decode_merge_bf16(const float* partial, const __nv_bfloat16* W, int LH, int U, int g,
                        Plan pl, int apply_w, int cw, TO* __restrict__ out) {
-    constexpr int REC = 4 + 2 * D;
-    __shared__ KeySums<D> ks;
-    __shared__ float pw[8][D];                 // W times the key sum
+    using C = MergeCfg<D, HEADS>;
+    constexpr int REC = 4 + 2 * D, NT = C::THREADS;
     constexpr int MAX_REC = 12 * Cfg<D, false>::CONSUMER_WARPS, REC_PER_LANE = (MAX_REC + 31) / 32;      // of a unit: twelve blocks' at the most
-    __shared__ float fv[8][MAX_REC], fk[8][MAX_REC];     // per head, per record: factor for the value part / the key part
-    __shared__ float Ls[8];
-    const int u = blockIdx.x, tid = threadIdx.x, a = tid / D, c = tid % D, lane = tid & 31;
-    const int wid = tid >> 5, nwarps = blockDim.x >> 5;
-    const __nv_bfloat16* Wu = W + (size_t)(u % LH) * D * D;       // the maps of a layer stay in L2: every sequence of the batch reads them
-    for (int i = tid; i < (8 - g) * D; i += blockDim.x) store_key_sum(ks, g + i / D, i % D, 0.f);      // columns of B beyond the unit's heads
+    constexpr int BUFS = C::RANGE ? 2 : 1;                  // of two units in turn
+    __shared__ KeySums<D> ks[BUFS];
+    __shared__ __align__(16) float sums[BUFS][HEADS][2 * D];      // value sums; without the map the key sums too
+    __shared__ float Ls[BUFS][HEADS];
+    const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+    const int a = tid / (D / 2), c4 = tid % (D / 2);        // a head's value sums, then its key sums, four channels a thread
+    const bool mine = a < g, value = c4 < D / 4, mapping = apply_w && wid < C::MAP_WARPS;      // mine, mapping: whole warps
+    const int batch = U / LH;
+    const int i_lo = C::RANGE ? (int)((long long)blockIdx.x * U / gridDim.x) : (int)blockIdx.x;
+    const int i_hi = C::RANGE ? (int)((long long)(blockIdx.x + 1) * U / gridDim.x) : i_lo + 1;
+    uint4 A[C::ROWS][D / 16];
+    auto map_of = [&](int i) {
+#pragma unroll
+        for (int r = 0; r < C::ROWS; ++r) map_fragments<D>(W + (size_t)(i / batch) * D * D, wid + r * C::MAP_WARPS, A[r], lane);
+    };
+    if (mapping) map_of(i_lo);
+    for (int i = tid; i < BUFS * (8 - g) * D; i += NT) store_key_sum(ks[i % BUFS], g + i / BUFS / D, i / BUFS % D, 0.f);      // columns of B beyond the unit's heads
     // the streaming kernel's records from here on
     asm volatile("griddepcontrol.wait;\n" ::: "memory");
-    const int first = block_of_tile((long long)u * pl.n_tiles, pl);
-    const int n_rec = (block_of_tile((long long)(u + 1) * pl.n_tiles - 1, pl) - first + 1) * cw;   // <= MAX_REC; cw records per block
-    const float* base = partial + (size_t)u * pl.s_max * cw * g * REC;
-    // The first six records' sums are requested before the headers are looked at, so that the two loads
-    // share one memory latency (a unit lies in one or two blocks of the streaming kernel, three records
-    // each, unless it is very long).
-    constexpr int NPRE = 6;
-    float rv[NPRE], rk[NPRE];
+
+    constexpr int NPRE = C::AHEAD;                          // a unit lies in one or two blocks of the streaming kernel, three or four records each, unless it is very long
+    const size_t step = (size_t)g * REC;                    // from record to record
+    int n_rec;
+    const float* base;
+    float4 v[NPRE], hd[REC_PER_LANE];                       // sums; headers of records lane, lane + 32
+    auto sums_from = [&](int j0) {
 #pragma unroll
-    for (int k = 0; k < NPRE; ++k) {
-        const int j = min(k, n_rec - 1);
-        const float* r = base + ((size_t)j * g + a) * REC + 4;
-        rv[k] = r[c];
-        rk[k] = r[D + c];
-    }
-    if (c < 32) {
-        // first warp of head a: headers of records lane, lane + 32, ...
-        float mj[REC_PER_LANE], lj[REC_PER_LANE], sj[REC_PER_LANE], M = -INFINITY;
+        for (int k = 0; k < NPRE; ++k) v[k] = *reinterpret_cast<const float4*>(base + min(j0 + k, n_rec - 1) * step + 4 + 4 * c4);
+    };
+    auto request = [&](int i) {
+        const int u = i % batch * LH + i / batch;
+        const int first = block_of_tile((long long)u * pl.n_tiles, pl);
+        n_rec = (block_of_tile((long long)(u + 1) * pl.n_tiles - 1, pl) - first + 1) * cw;       // <= MAX_REC; cw records per block
+        base = partial + ((size_t)u * pl.s_max * cw * g + a) * REC;
+        sums_from(0);
 #pragma unroll
-        for (int k = 0; k < REC_PER_LANE; ++k) {
-            const int j = lane + 32 * k;
-            mj[k] = -INFINITY; lj[k] = 0.f; sj[k] = 0.f;
-            if (j < n_rec) {
-                const float4 h = *reinterpret_cast<const float4*>(base + ((size_t)j * g + a) * REC);
-                mj[k] = h.x; lj[k] = h.y; sj[k] = h.z;
+        for (int k = 0; k < REC_PER_LANE; ++k)
+            hd[k] = lane + 32 * k < n_rec ? *reinterpret_cast<const float4*>(base + (lane + 32 * k) * step) : make_float4(-INFINITY, 0.f, 0.f, 0.f);
+    };
+    if (mine) request(i_lo);
+    for (int i = i_lo; i < i_hi; ++i) {
+        const int buf = C::RANGE ? i & 1 : 0, u = i % batch * LH + i / batch;
+        if (mine) {
+            float M = hd[0].x;
+#pragma unroll
+            for (int k = 1; k < REC_PER_LANE; ++k) M = fmaxf(M, hd[k].x);
+            M = warp_max(M);
+            float Lsum = 0.f, fk[REC_PER_LANE], fv[REC_PER_LANE];                                // factors of the key and of the value sums
+#pragma unroll
+            for (int k = 0; k < REC_PER_LANE; ++k) {
+                fk[k] = hd[k].x > -INFINITY ? __expf(hd[k].x - M) : 0.f;
+                fv[k] = fk[k] * hd[k].z;
+                Lsum += fk[k] * hd[k].y;
             }
-            M = fmaxf(M, mj[k]);
-        }
-        M = warp_max(M);
-        float Lsum = 0.f;
+            Lsum = warp_sum(Lsum);
+            float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
+            for (int j0 = 0; j0 < n_rec; j0 += NPRE) {
+                if (j0 > 0) sums_from(j0);
 #pragma unroll
-        for (int k = 0; k < REC_PER_LANE; ++k) {
-            const int j = lane + 32 * k;
-            const float f = mj[k] > -INFINITY ? __expf(mj[k] - M) : 0.f;
-            if (j < MAX_REC) { fk[a][j] = f; fv[a][j] = f * sj[k]; }
-            Lsum += f * lj[k];
-        }
-        Lsum = warp_sum(Lsum);
-        if (lane == 0) Ls[a] = Lsum;
-    }
-    __syncthreads();
-    float av = 0.f, ak = 0.f;
-    for (int j0 = 0; j0 < n_rec; j0 += NPRE) {
-        if (j0 > 0) {
-#pragma unroll
-            for (int k = 0; k < NPRE; ++k) {
-                const int j = min(j0 + k, n_rec - 1);
-                const float* r = base + ((size_t)j * g + a) * REC + 4;
-                rv[k] = r[c];
-                rk[k] = r[D + c];
+                for (int k = 0; k < NPRE; ++k) {
+                    const int j = j0 + k;
+                    if (j >= n_rec) break;
+                    float f0 = fk[0], f1 = fv[0];
+                    if (REC_PER_LANE > 1 && j >= 32) { f0 = fk[REC_PER_LANE - 1]; f1 = fv[REC_PER_LANE - 1]; }
+                    f0 = __shfl_sync(0xffffffffu, f0, j & 31);
+                    f1 = __shfl_sync(0xffffffffu, f1, j & 31);
+                    const float f = value ? f1 : f0;
+                    acc.x = fmaf(f, v[k].x, acc.x); acc.y = fmaf(f, v[k].y, acc.y); acc.z = fmaf(f, v[k].z, acc.z); acc.w = fmaf(f, v[k].w, acc.w);
+                }
+            }
+            if (C::RANGE && i + 1 < i_hi) request(i + 1);
+            if (c4 == 0) Ls[buf][a] = Lsum;
+            if (value || !apply_w) {                        // per-tile form: the second part of a record is already sum p (W k)
+                *reinterpret_cast<float4*>(&sums[buf][a][4 * c4]) = acc;
+            } else {
+                const int c = 4 * c4 - D;
+                store_key_sum(ks[buf], a, c, acc.x); store_key_sum(ks[buf], a, c + 1, acc.y);
+                store_key_sum(ks[buf], a, c + 2, acc.z); store_key_sum(ks[buf], a, c + 3, acc.w);
             }
         }
+        // one barrier a unit: whoever writes this half again, two units on, has seen every warp past this unit
+        __syncthreads();
+        TO* const o = out + (size_t)u * g * D;
+        if (mapping) {
+            const int head = 2 * (lane & 3);
+            float d[C::ROWS][4];
 #pragma unroll
-        for (int k = 0; k < NPRE; ++k) {
-            if (j0 + k < n_rec) {
-                av = fmaf(fv[a][j0 + k], rv[k], av);
-                ak = fmaf(fk[a][j0 + k], rk[k], ak);
-            }
+            for (int r = 0; r < C::ROWS; ++r) map_product<D>(A[r], ks[buf], d[r], lane);
+            if (C::RANGE && i + 1 < i_hi && (i + 1) % batch == 0) map_of(i + 1);
+#pragma unroll
+            for (int r = 0; r < C::ROWS; ++r)
+#pragma unroll
+                for (int e = 0; e < 4; ++e) {
+                    const int h = head + (e & 1), c = 16 * (wid + r * C::MAP_WARPS) + (lane >> 2) + 8 * (e >> 1);
+                    if (h < g) store_out(o + h * D + c, (sums[buf][h][c] + d[r][e]) / Ls[buf][h]);
+                }
+        } else if (!apply_w) {
+            for (int e = tid; e < g * D; e += NT) store_out(o + e, (sums[buf][e / D][e % D] + sums[buf][e / D][D + e % D]) / Ls[buf][e / D]);
         }
     }
-    if (!apply_w) {           // per-tile form: the second part of a record is already sum p (W k)
-        store_out(out + ((size_t)u * g + a) * D + c, (av + ak) / Ls[a]);
-        return;
-    }
-    store_key_sum(ks, a, c, ak);
-    __syncthreads();
-    for (int mt = wid; mt < D / 16; mt += nwarps) map_rows(Wu, mt, g, ks, pw, lane);
-    __syncthreads();
-    store_out(out + ((size_t)u * g + a) * D + c, (av + pw[a][c]) / Ls[a]);
 }
 
 }  // namespace dbf
