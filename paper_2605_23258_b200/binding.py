@@ -1,4 +1,4 @@
-"""ctypes binding of libvector: argument marshalling only.
+"""Binding of libvector: argument marshalling only.
 
 Every function has the name and the argument order of its C entry point
 (``include/vector.h``).  Tensors are ``torch`` tensors used as typed device (or,
@@ -6,6 +6,9 @@ for calibration, host) buffers; the binding checks dtype, device and
 contiguity, passes raw pointers, and raises :class:`VectorError` on a non-zero
 status.  There is no fallback: if the shared library is missing the import of
 any entry point fails loudly.
+
+The calls of a serving loop try the extension module first (``csrc/marshal.cpp``), which marshals plain tensors and structs without a
+Python object for every pointer and answers None, having done nothing, where an argument is anything else; ctypes then takes the call.
 """
 from __future__ import annotations
 
@@ -20,6 +23,7 @@ VECTOR_F32, VECTOR_BF16 = 0, 1
 _HERE = os.path.dirname(os.path.abspath(__file__))
 _LIB_PATH = os.path.join(_HERE, "libvector.so")
 _lib = None
+_marshal_module = None
 
 
 class VectorError(RuntimeError):
@@ -192,6 +196,17 @@ def load_library() -> ctypes.CDLL:
     return lib
 
 
+def _marshal():
+    """The extension module, bound to the loaded library; raises if it has not been built."""
+    global _marshal_module
+    if _marshal_module is None:
+        lib = load_library()
+        from . import _marshal as module
+        module.bind(lib._handle, Shape, Budget, Cache)
+        _marshal_module = module
+    return _marshal_module
+
+
 def _check(rc: int, where: str):
     if rc != 0:
         raise VectorError(rc, where)
@@ -295,6 +310,11 @@ def alloc_cache(shape: Shape, budget: Budget, extra_rows: int = 0, device="cuda"
 
 
 def vector_score(shape: Shape, Q_obs, K, N: int, scores, raw_out=None, ws=None, stream=None):
+    rc = (_marshal_module or _marshal()).score(shape, Q_obs, K, N, scores, raw_out, ws, stream)
+    if rc is not None:
+        if rc:
+            _check(rc, "vector_score")
+        return
     wp, wn = _ws(ws)
     rc = load_library().vector_score(shape._p(), _dev(Q_obs, shape.torch_dtype, "Q_obs"),
                                      _dev(K, shape.torch_dtype, "K"), N, _dev(scores, torch.float32, "scores"),
@@ -336,6 +356,11 @@ def vector_truncate(shape: Shape, budget: Budget, eps, pool_idx, tier, ret_idx, 
 
 def vector_route(shape: Shape, budget: Budget, scores, K, V, W, tier, ret_idx, apx_idx, eps_out=None,
                  pool_idx_out=None, ws=None, stream=None):
+    rc = (_marshal_module or _marshal()).route(shape, budget, scores, K, V, W, tier, ret_idx, apx_idx, eps_out, pool_idx_out, ws, stream)
+    if rc is not None:
+        if rc:
+            _check(rc, "vector_route")
+        return
     wp, wn = _ws(ws)
     rc = load_library().vector_route(shape._p(), budget._p(),
                                      _dev(scores, torch.float32, "scores"), _dev(K, shape.torch_dtype, "K"),
@@ -380,6 +405,11 @@ def vector_sync_check(stream=None):
 
 
 def vector_compact(shape: Shape, budget: Budget, K, V, ret_idx, apx_idx, cache: Cache, stream=None):
+    rc = (_marshal_module or _marshal()).compact(shape, budget, K, V, ret_idx, apx_idx, cache, stream)
+    if rc is not None:
+        if rc:
+            _check(rc, "vector_compact")
+        return
     c = cache._p()
     rc = load_library().vector_compact(shape._p(), budget._p(),
                                        _dev(K, shape.torch_dtype, "K"), _dev(V, shape.torch_dtype, "V"),
@@ -390,13 +420,32 @@ def vector_compact(shape: Shape, budget: Budget, K, V, ret_idx, apx_idx, cache: 
 
 def vector_append(shape: Shape, cache: Cache, k_new, v_new, pos: int, stream=None):
     """k_new, v_new [U][d] become row cache.n_ret of the retained pool; the caller bumps cache.n_ret."""
+    rc = (_marshal_module or _marshal()).append(shape, cache, k_new, v_new, pos, stream)
+    if rc is not None:
+        if rc:
+            _check(rc, "vector_append")
+        return
     c = cache._p()
     rc = load_library().vector_append(shape._p(), c, _dev(k_new, shape.torch_dtype, "k_new"),
                                       _dev(v_new, shape.torch_dtype, "v_new"), pos, _stream(stream))
     _check(rc, "vector_append")
 
 
+def append_rows(shape: Shape, cache: Cache, k_new, v_new, pos) -> bool:
+    """vector_append where one kernel can copy the rows: plain rows of the shape's size and type on the current device, and room for one
+    more.  False, having done nothing, anywhere else."""
+    rc = (_marshal_module or _marshal()).append_rows(shape, cache, k_new, v_new, pos)
+    if rc:
+        _check(rc, "vector_append")
+    return rc is not None
+
+
 def vector_decode_attn(shape: Shape, q, cache: Cache, W, out, mode: int = 0, ws=None, stream=None):
+    rc = (_marshal_module or _marshal()).decode_attn(shape, q, cache, W, out, mode, ws, stream)
+    if rc is not None:
+        if rc:
+            _check(rc, "vector_decode_attn")
+        return
     wp, wn = _ws(ws)
     c = cache._p()
     if out.dtype not in (torch.float32, torch.bfloat16):
@@ -429,6 +478,11 @@ def vector_residual_layer(shape: Shape, K, V, W_layer, N: int, idx, n_idx: int, 
 
 def vector_route_layer(shape: Shape, budget: Budget, layer_scores, K, V, W_layer, tier, ret_idx, apx_idx,
                        eps_out=None, pool_idx_out=None, ws=None, stream=None):
+    rc = (_marshal_module or _marshal()).route_layer(shape, budget, layer_scores, K, V, W_layer, tier, ret_idx, apx_idx, eps_out, pool_idx_out, ws, stream)
+    if rc is not None:
+        if rc:
+            _check(rc, "vector_route_layer")
+        return
     wp, wn = _ws(ws)
     rc = load_library().vector_route_layer(shape._p(), budget._p(),
                                            _dev(layer_scores, torch.float32, "layer_scores"),
@@ -441,6 +495,11 @@ def vector_route_layer(shape: Shape, budget: Budget, layer_scores, K, V, W_layer
 
 
 def vector_compact_layer(shape: Shape, budget: Budget, K, V, ret_idx, apx_idx, cache: Cache, stream=None):
+    rc = (_marshal_module or _marshal()).compact_layer(shape, budget, K, V, ret_idx, apx_idx, cache, stream)
+    if rc is not None:
+        if rc:
+            _check(rc, "vector_compact_layer")
+        return
     c = cache._p()
     rc = load_library().vector_compact_layer(shape._p(), budget._p(),
                                              _dev(K, shape.torch_dtype, "K"), _dev(V, shape.torch_dtype, "V"),
@@ -450,6 +509,11 @@ def vector_compact_layer(shape: Shape, budget: Budget, K, V, ret_idx, apx_idx, c
 
 
 def vector_decode_attn_layer(shape: Shape, q, cache: Cache, W_layer, out, ws=None, stream=None):
+    rc = (_marshal_module or _marshal()).decode_attn_layer(shape, q, cache, W_layer, out, ws, stream)
+    if rc is not None:
+        if rc:
+            _check(rc, "vector_decode_attn_layer")
+        return
     wp, wn = _ws(ws)
     c = cache._p()
     if out.dtype not in (torch.float32, torch.bfloat16):
@@ -478,6 +542,11 @@ def vector_decode_attn_static(shape: Shape, q, cache: Cache, W, out, mode: int =
     that need more raise VectorError (workspace).  Calls on one device share that array,
     so calls that overlap on the GPU race; make the first call per device at start-up.
     """
+    rc = (_marshal_module or _marshal()).decode_attn_static(shape, q, cache, W, out, mode, stream)
+    if rc is not None:
+        if rc:
+            _check(rc, "vector_decode_attn_static")
+        return
     c = cache._p()
     if out.dtype not in (torch.float32, torch.bfloat16):
         raise ValueError("out must be fp32 or bf16")

@@ -1,4 +1,4 @@
-"""Builds libvector.so (the C-ABI CUDA library) in-tree with nvcc for sm_100a."""
+"""Builds libvector.so (the C-ABI CUDA library) in-tree with nvcc for sm_100a, and the extension module that marshals arguments."""
 from __future__ import annotations
 
 import os
@@ -9,6 +9,7 @@ HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(HERE, "csrc")
 INCLUDE = os.path.join(os.path.dirname(HERE), "include")
 LIB = os.path.join(HERE, "libvector.so")
+MARSHAL = os.path.join(HERE, "_marshal.so")
 
 SOURCES = ["host.cpp", "score.cu", "keydiff.cu", "route.cu", "compact.cu", "decode.cu", "decode_layer.cu", "diagnostics.cu"]
 NVCC_FLAGS = ["-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
@@ -23,18 +24,35 @@ def _nvcc() -> str:
     raise RuntimeError("nvcc not found")
 
 
+def _older(target: str, deps) -> bool:
+    return not os.path.exists(target) or any(os.path.getmtime(d) > os.path.getmtime(target) for d in [*deps, os.path.join(INCLUDE, "vector.h"), __file__])
+
+
 def _stale() -> bool:
-    if not os.path.exists(LIB):
-        return True
-    t = os.path.getmtime(LIB)
-    deps = [os.path.join(CSRC, f) for f in os.listdir(CSRC)] + [os.path.join(INCLUDE, "vector.h"), __file__]
-    return any(os.path.getmtime(d) > t for d in deps)
+    return _older(LIB, [os.path.join(CSRC, f) for f in os.listdir(CSRC) if f != "marshal.cpp"])
+
+
+def build_marshal(force: bool = False) -> str:
+    """The extension module behind the binding (csrc/marshal.cpp): plain C++ against the headers of Python and torch."""
+    src = os.path.join(CSRC, "marshal.cpp")
+    if not force and not _older(MARSHAL, [src]):
+        return MARSHAL
+    import sysconfig
+    from torch.utils.cpp_extension import include_paths, library_paths
+    cuda = os.path.dirname(os.path.dirname(os.path.realpath(_nvcc())))
+    incs = [INCLUDE, *include_paths(), sysconfig.get_paths()["include"], os.path.join(cuda, "include")]
+    tmp = MARSHAL + f".tmp{os.getpid()}"
+    subprocess.check_call([os.environ.get("CXX", "g++"), "-O2", "-std=c++17", "-fPIC", "-shared", "-fvisibility=hidden", *(f"-I{i}" for i in incs), src,
+                           *(f"-L{p}" for p in library_paths()), "-ltorch_python", "-ltorch_cpu", "-lc10", "-lc10_cuda", "-o", tmp])
+    os.replace(tmp, MARSHAL)
+    return MARSHAL
 
 
 def build(force: bool = False, verbose: bool = False) -> str:
     """Compile every translation unit to an object and link the shared library.  Extra nvcc flags can be
     given in the environment variable VECTOR_NVCC_FLAGS (e.g. -DVECTOR_SCORE_POLY16=6 for the sweep of the
     share of softmax exponentials evaluated on the FMA pipe)."""
+    build_marshal(force)
     if not force and not _stale():
         return LIB
     objdir = os.path.join(HERE, "_build")
