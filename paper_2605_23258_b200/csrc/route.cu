@@ -374,6 +374,13 @@ static int truncate_warps(int64_t n, int U) {
     return n < SEL_LONG ? 16 : 32;
 }
 
+// With the input in registers, 32 warps a block instead of 16: half the elements a thread, where a list has a multiprocessor to itself
+// (two blocks of 16 warps share one, which 32 would take for themselves) and is long enough that counting and handing out outweigh the
+// barriers.  us in a graph, 16 / 32 warps, Step 1 and Step 3: 8 lists of 2048 3.8 / 3.7 and 4.5 / 4.6, of 3000 4.5 / 4.2 and 6.0 / 5.6, of
+// 8192 6.9 / 6.2 and 9.3 / 8.4, of 16384 11.2 / 9.3 (Step 3 had 32 there already); 148 of 8192 7.2 / 6.4 and 9.6 / 8.8; 200 of 3000
+// 5.9 / 6.4 and 8.1 / 10.3, of 8192 9.5 / 11.8 and 14.3 / 15.9.
+static bool regs_wide(int64_t n, int U) { return n > 2048 && U <= sm_count(); }
+
 static vector_status launch_pool_select(const Dims& dm, const vector_budget* budget, const float* scores, int32_t* pool,
                                         cudaStream_t st, float* zero = nullptr) {
     vector_status rc = select_kernels_setup();
@@ -381,9 +388,12 @@ static vector_status launch_pool_select(const Dims& dm, const vector_budget* bud
     const int64_t n = budget->n_tokens;
     const int nw = pool_select_warps(n, dm.U, budget->n_pool);
     if (nw == 0) {
-        auto kern = n <= 2048 ? pool_select_regs<16, 4> : n <= 4096 ? pool_select_regs<16, 8> : n <= 8192 ? pool_select_regs<16, 16>
-                  : n <= SEL_REGS16 ? pool_select_regs<16, 32> : pool_select_regs<32, 32>;
-        VEC_CUDA_CHECK(launch_maybe_dependent(true, kern, dim3(dm.U), dim3(n <= SEL_REGS16 ? 512 : 1024), 0, st, scores, n,
+        const bool wide = regs_wide(n, dm.U) || n > SEL_REGS16;
+        auto kern = wide ? (n <= 4096 ? pool_select_regs<32, 4> : n <= 8192 ? pool_select_regs<32, 8> : n <= SEL_REGS16 ? pool_select_regs<32, 16>
+                                                                                                                  : pool_select_regs<32, 32>)
+                         : n <= 2048 ? pool_select_regs<16, 4> : n <= 4096 ? pool_select_regs<16, 8> : n <= 8192 ? pool_select_regs<16, 16>
+                                                                                                                 : pool_select_regs<16, 32>;
+        VEC_CUDA_CHECK(launch_maybe_dependent(true, kern, dim3(dm.U), dim3(wide ? 1024 : 512), 0, st, scores, n,
                                               (int)budget->n_pool, pool, zero));
         return VECTOR_OK;
     }
@@ -402,9 +412,10 @@ static vector_status launch_truncate(const Dims& dm, const vector_budget* budget
     const int64_t n = budget->n_pool;
     const int nw = truncate_warps(n, dm.U);
     if (nw == 0) {
-        auto kern = n <= 2048 ? truncate_regs<16, 4> : n <= 4096 ? truncate_regs<16, 8> : n <= 8192 ? truncate_regs<16, 16>
-                  : truncate_regs<32, 16>;
-        VEC_CUDA_CHECK(launch_maybe_dependent(dependent, kern, dim3(dm.U), dim3(n <= 8192 ? 512 : 1024), 0, st, eps, pool,
+        const bool wide = regs_wide(n, dm.U) || n > 8192;
+        auto kern = wide ? (n <= 4096 ? truncate_regs<32, 4> : n <= 8192 ? truncate_regs<32, 8> : truncate_regs<32, 16>)
+                         : n <= 2048 ? truncate_regs<16, 4> : n <= 4096 ? truncate_regs<16, 8> : truncate_regs<16, 16>;
+        VEC_CUDA_CHECK(launch_maybe_dependent(dependent, kern, dim3(dm.U), dim3(wide ? 1024 : 512), 0, st, eps, pool,
                                               (int64_t)budget->n_tokens, (int)n, (int)budget->n_apx, tier, ret_idx, apx_idx));
         return VECTOR_OK;
     }

@@ -47,6 +47,13 @@ def test_forms(share, n, ties, taken):
     assert torch.equal(tier, want_tier)
 
 
+@pytest.mark.parametrize("ties", [False, True])
+@pytest.mark.parametrize("share,n", [(0.9935, 2048), (0.9935, 2049), (0.9935, 4096), (0.9935, 4097), (0.9935, 8191), (1, 2049), (1, 4097), (0.01, 8192)])
+def test_forms_in_registers_by_lists(share, n, ties):
+    """As many lists as multiprocessors, and one more: blocks of 32 and of 16 warps."""
+    test_forms(share, n, ties, 2 / 3)
+
+
 def test_step3_past_the_registers():
     us = []
     for n in (16384, 20011):
