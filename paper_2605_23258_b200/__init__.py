@@ -1,7 +1,7 @@
 """B200-native VECTOR hot path: thin Python binding over the C-ABI CUDA library.
 
 The package holds the CUDA sources (``csrc/``), the in-tree build of
-``libvector.so`` and a ctypes binding whose functions carry the same names as
+``libvector.so`` and a binding whose functions carry the same names as
 the C entry points.  PyTorch is used only for device memory and streams.
 """
 from .binding import (  # noqa: F401
