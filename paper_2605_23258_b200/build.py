@@ -37,9 +37,10 @@ def build_marshal(force: bool = False) -> str:
     src = os.path.join(CSRC, "marshal.cpp")
     if not force and not _older(MARSHAL, [src]):
         return MARSHAL
+    import shutil
     import sysconfig
     from torch.utils.cpp_extension import include_paths, library_paths
-    cuda = os.path.dirname(os.path.dirname(os.path.realpath(_nvcc())))
+    cuda = os.path.dirname(os.path.dirname(os.path.realpath(shutil.which(_nvcc()) or _nvcc())))
     incs = [INCLUDE, *include_paths(), sysconfig.get_paths()["include"], os.path.join(cuda, "include")]
     tmp = MARSHAL + f".tmp{os.getpid()}"
     subprocess.check_call([os.environ.get("CXX", "g++"), "-O2", "-std=c++17", "-fPIC", "-shared", "-fvisibility=hidden", *(f"-I{i}" for i in incs), src,
