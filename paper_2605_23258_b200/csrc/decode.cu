@@ -10,6 +10,7 @@
 // [0, n_ret + n_apx); the blocks' sums are merged over distributed shared memory.
 #include <cmath>
 #include <mutex>
+#include <type_traits>
 
 #include "cluster.cuh"
 #include "common.cuh"
@@ -395,13 +396,43 @@ static vector_status launch_decode_bf16(const Dims& dm, const void* q, const vec
     const int apply_w = mode == 1 ? 0 : 1;
     const int cw = mode == 1 ? dpt::CONSUMERS : dm.rope ? Rope::CONSUMER_WARPS : Plain::CONSUMER_WARPS;   // records a block leaves per unit
     const T* Wp = (const T*)W;
-#define VEC_MERGE(TO, HEADS)                                                                                                     \
-    VEC_CUDA_CHECK(launch_maybe_dependent(true, dbf::decode_merge_bf16<TO, D, HEADS>, dim3(dbf::MergeCfg<D, HEADS>::blocks(dm.U, sm_count())), \
-                                          dim3(dbf::MergeCfg<D, HEADS>::THREADS), 0, st, rec, Wp, dm.LH, dm.U, dm.g, pl, apply_w, cw, (TO*)out))
-    if (out_dtype == VECTOR_F32) { if (dm.g <= 2) VEC_MERGE(float, 2); else if (dm.g <= 4) VEC_MERGE(float, 4); else VEC_MERGE(float, 8); }
-    else { if (dm.g <= 2) VEC_MERGE(T, 2); else if (dm.g <= 4) VEC_MERGE(T, 4); else VEC_MERGE(T, 8); }
+    // The form by units a multiprocessor (`full`, rounded up).  A block a unit with everything requested ahead is the fastest while all units' blocks are
+    // resident at once; registers decide how many are.  us of a whole step in a graph, one sequence, 96 / 600 / 1800 rows a unit:
+    //   128 channels, two heads, 592 units: four blocks of 128 threads 17.2 / 31.5 / 65.4, ranges by three of 256 threads 21.3 / 35.5 / 69.2, a thread
+    //   a channel 19.3 / 35.5 / 69.7; 740 units, five blocks: 20.3 / 39.5 / 81.1 (22.8 / 41.9 / 83.6, 20.9 / 41.5 / 83.9); 900 units, a thread a channel
+    //   25.3 / 48.2 / 96.9, ranges 28.8 / 50.5 / 99.1; 4096 units of one head and 96 / 600 rows 84.6 / 183 and 100 / 197.
+    //   Three heads: 440 units, three blocks 14.6 / 26.7 / 49.1 (ranges by two 16.7 / 28.7 / 51.0, a thread a channel 16.2 / 29.1 / 51.9); 900 units,
+    //   a thread a channel 27.2 / 49.8 / 99.2, ranges 29.1 / 50.9 / 100.2.
+    //   Four heads: 440 units, three blocks 14.9 / 27.0 / 49.9 (ranges by two 16.8 / 29.3 / 51.6); 900 units, ranges 29.0 / 52.0 / 101.6, a thread a channel
+    //   30.3 / 53.4 / 103.3.  Ranges go on paying where sequences share maps: 2048 units of eight sequences 0.95 to 0.98 of a thread a channel.
+    //   64 channels: 740 units of four heads, a block a unit with seven resident 14.9 / 26.8 / 49.3, ranges by four 17.0 / 29.1 / 50.5; 1280 units of
+    //   two heads, a block a unit 20.5 / 41.7 / 80.1, ranges 23.4 / 44.5 / 83.1.
+    // More than four heads take a block a unit at any number of units.
+    const int full = (dm.U + sm_count() - 1) / sm_count();
+    auto merge = [&](auto* o) -> vector_status {
+        using TO = std::remove_pointer_t<decltype(o)>;
+        auto launch = [&](auto kern, int blocks, int threads) -> vector_status {
+            VEC_CUDA_CHECK(launch_maybe_dependent(true, kern, dim3(blocks), dim3(threads), 0, st, rec, Wp, dm.LH, dm.U, dm.g, pl, apply_w, cw, o));
+            return VECTOR_OK;
+        };
+#define VEC_MERGE(HEADS, RES) \
+    return launch(dbf::decode_merge_bf16<TO, D, HEADS, RES>, dbf::MergeCfg<D, HEADS, RES>::blocks(dm.U, sm_count()), dbf::MergeCfg<D, HEADS, RES>::THREADS)
+        if constexpr (D == 128) {
+            if (dm.g <= 2 && full <= 4) VEC_MERGE(2, 4);
+            if (dm.g <= 2 && full <= 5) VEC_MERGE(2, 5);
+            if (dm.g <= 3 && full > 3) return launch(dbf::decode_merge_channels<TO, D>, dm.U, D * dm.g);
+            if (dm.g <= 4 && full == 3) VEC_MERGE(4, 3);
+            if (dm.g <= 4) VEC_MERGE(4, 2);
+            VEC_MERGE(8, 2);
+        } else {
+            if (dm.g <= 2) VEC_MERGE(2, 8);
+            if (dm.g <= 4 && full > 4) VEC_MERGE(4, 7);
+            if (dm.g <= 4) VEC_MERGE(4, 4);
+            VEC_MERGE(8, 4);
+        }
 #undef VEC_MERGE
-    return VECTOR_OK;
+    };
+    return out_dtype == VECTOR_F32 ? merge((float*)out) : merge((T*)out);
 }
 
 template <typename T, int D, bool ROPE, bool WIDE>

@@ -751,28 +751,24 @@ decode_stream_bf16(const __nv_bfloat16* q, const __grid_constant__ Maps maps, Pl
 // A thread owns four channels of a head's value or key sum; its warp reads that head's headers, a record a lane, and hands the factors
 // round by shuffles, so that sums and headers share one memory latency and no barrier lies between them.  The map's fragments (MMAs,
 // map_fragments) are requested ahead of the wait for the streaming kernel, which does not touch the map: they come in while that
-// kernel drains.  What bounds it is that chain, one trip to L2 and a product a unit.
-// Up to four heads: as many blocks as are resident at once, each with an equal range of the units, ordered by map, so that the
+// kernel drains.  What bounds it is that chain, one trip to L2 and a product a unit, as long as every unit has its block on the chip at
+// once (RESIDENT a multiprocessor); beyond, the units in flight.  Which form takes how many units: launch_decode_bf16.
+// RANGE: as many blocks as are resident at once, each with an equal range of the units, ordered by map, so that the
 // sequences that share one find it in their block's registers; the next unit's records are requested before this one's product.
-// Up to eight heads: a block a unit, since registers for the next unit would cost the second resident block.
-// Blocks and records in flight as measured, us of a whole step in a graph: 2048 units of four heads of 128 channels 272 with two blocks
-// and six records, 275 with three and four, 278 with four and three; of one head 142 with three and three, 145 with four; 64 channels and
-// two heads 90.5 with blocks of 64 threads, 93 with 128.  Against a thread a channel, the factors through shared memory and the map
-// behind them: 2048 units of four heads 279 -> 272, 96 units of two heads 32.4 -> 29.4, 1536 units of eight heads and 1324 rows
-// 144 -> 128, with RoPE and 661 rows 121 -> 105.
-template <int D, int HEADS> struct MergeCfg {
-    static constexpr int THREADS = D == 64 && HEADS == 2 ? 64 : HEADS == 8 ? 4 * D : 2 * D;      // a head's sums take D / 2
-    static constexpr int RESIDENT = D == 128 ? (HEADS == 2 ? 3 : 2) : HEADS == 2 ? 8 : 4;
-    static constexpr int AHEAD = HEADS == 4 ? 6 : D == 128 && HEADS == 2 ? 3 : 4;      // records whose sums are requested together
-    static constexpr bool RANGE = HEADS <= 4;
+// Otherwise a block a unit.  Spilled, bytes a thread: 52 with five resident blocks of two heads, 12 with three of four, 48 with two of eight
+// (12 at 64 channels).
+template <int D, int HEADS, int RES> struct MergeCfg {
+    static constexpr int THREADS = HEADS * D / 2, RESIDENT = RES;      // a head's sums take D / 2
+    static constexpr bool RANGE = HEADS == 4 && RES == (D == 128 ? 2 : 4);
+    static constexpr int AHEAD = RANGE ? 6 : D == 128 && HEADS <= 4 ? 3 : 4;      // records whose sums are requested together
     static constexpr int MAP_WARPS = THREADS / 32 < D / 16 ? THREADS / 32 : D / 16, ROWS = D / 16 / MAP_WARPS;      // warps with rows of the map, blocks of 16 rows each
     static constexpr int blocks(int U, int sms) { return RANGE && U > RESIDENT * sms ? RESIDENT * sms : U; }
 };
-template <typename TO, int D, int HEADS>
-__global__ void __launch_bounds__(MergeCfg<D, HEADS>::THREADS, MergeCfg<D, HEADS>::RESIDENT)
+template <typename TO, int D, int HEADS, int RES>
+__global__ void __launch_bounds__(MergeCfg<D, HEADS, RES>::THREADS, RES)
 decode_merge_bf16(const float* partial, const __nv_bfloat16* W, int LH, int U, int g,
                        Plan pl, int apply_w, int cw, TO* __restrict__ out) {
-    using C = MergeCfg<D, HEADS>;
+    using C = MergeCfg<D, HEADS, RES>;
     constexpr int REC = 4 + 2 * D, NT = C::THREADS;
     constexpr int MAX_REC = 12 * Cfg<D, false>::CONSUMER_WARPS, REC_PER_LANE = (MAX_REC + 31) / 32;      // of a unit: twelve blocks' at the most
     constexpr int BUFS = C::RANGE ? 2 : 1;                  // of two units in turn
@@ -875,6 +871,87 @@ decode_merge_bf16(const float* partial, const __nv_bfloat16* W, int LH, int U, i
             for (int e = tid; e < g * D; e += NT) store_out(o + e, (sums[buf][e / D][e % D] + sums[buf][e / D][D + e % D]) / Ls[buf][e / D]);
         }
     }
+}
+
+// The same for up to three heads in many units of 128 channels, where units in flight are what counts: a thread a channel, D g of them
+// and 40 registers each (8 to 12 bytes spilled), the factors through shared memory and the map read behind them.
+template <typename TO, int D>
+__global__ void __launch_bounds__(3 * D, 4)
+decode_merge_channels(const float* partial, const __nv_bfloat16* W, int LH, int U, int g,
+                      Plan pl, int apply_w, int cw, TO* __restrict__ out) {
+    constexpr int REC = 4 + 2 * D;
+    constexpr int MAX_REC = 12 * Cfg<D, false>::CONSUMER_WARPS, REC_PER_LANE = (MAX_REC + 31) / 32;
+    __shared__ KeySums<D> ks;
+    __shared__ float pw[8][D];                 // W times the key sum
+    __shared__ float fv[3][MAX_REC], fk[3][MAX_REC];     // per head, per record: factor for the value part / the key part
+    __shared__ float Ls[3];
+    const int u = blockIdx.x, tid = threadIdx.x, a = tid / D, c = tid % D, lane = tid & 31;
+    const int wid = tid >> 5, nwarps = blockDim.x >> 5;
+    const __nv_bfloat16* Wu = W + (size_t)(u % LH) * D * D;
+    for (int i = tid; i < (8 - g) * D; i += blockDim.x) store_key_sum(ks, g + i / D, i % D, 0.f);      // columns of B beyond the unit's heads
+    // the streaming kernel's records from here on
+    asm volatile("griddepcontrol.wait;\n" ::: "memory");
+    const int first = block_of_tile((long long)u * pl.n_tiles, pl);
+    const int n_rec = (block_of_tile((long long)(u + 1) * pl.n_tiles - 1, pl) - first + 1) * cw;
+    const float* base = partial + (size_t)u * pl.s_max * cw * g * REC;
+    constexpr int NPRE = 6;                              // records whose sums are requested together, the first ones before the headers
+    float rv[NPRE], rk[NPRE];
+    auto sums_from = [&](int j0) {
+#pragma unroll
+        for (int k = 0; k < NPRE; ++k) {
+            const int j = min(j0 + k, n_rec - 1);
+            const float* r = base + ((size_t)j * g + a) * REC + 4;
+            rv[k] = r[c];
+            rk[k] = r[D + c];
+        }
+    };
+    sums_from(0);
+    if (c < 32) {
+        // first warp of head a: headers of records lane, lane + 32, ...
+        float mj[REC_PER_LANE], lj[REC_PER_LANE], sj[REC_PER_LANE], M = -INFINITY;
+#pragma unroll
+        for (int k = 0; k < REC_PER_LANE; ++k) {
+            const int j = lane + 32 * k;
+            mj[k] = -INFINITY; lj[k] = 0.f; sj[k] = 0.f;
+            if (j < n_rec) {
+                const float4 h = *reinterpret_cast<const float4*>(base + ((size_t)j * g + a) * REC);
+                mj[k] = h.x; lj[k] = h.y; sj[k] = h.z;
+            }
+            M = fmaxf(M, mj[k]);
+        }
+        M = warp_max(M);
+        float Lsum = 0.f;
+#pragma unroll
+        for (int k = 0; k < REC_PER_LANE; ++k) {
+            const int j = lane + 32 * k;
+            const float f = mj[k] > -INFINITY ? __expf(mj[k] - M) : 0.f;
+            if (j < MAX_REC) { fk[a][j] = f; fv[a][j] = f * sj[k]; }
+            Lsum += f * lj[k];
+        }
+        Lsum = warp_sum(Lsum);
+        if (lane == 0) Ls[a] = Lsum;
+    }
+    __syncthreads();
+    float av = 0.f, ak = 0.f;
+    for (int j0 = 0; j0 < n_rec; j0 += NPRE) {
+        if (j0 > 0) sums_from(j0);
+#pragma unroll
+        for (int k = 0; k < NPRE; ++k) {
+            if (j0 + k < n_rec) {
+                av = fmaf(fv[a][j0 + k], rv[k], av);
+                ak = fmaf(fk[a][j0 + k], rk[k], ak);
+            }
+        }
+    }
+    if (!apply_w) {           // per-tile form: the second part of a record is already sum p (W k)
+        store_out(out + ((size_t)u * g + a) * D + c, (av + ak) / Ls[a]);
+        return;
+    }
+    store_key_sum(ks, a, c, ak);
+    __syncthreads();
+    for (int mt = wid; mt < D / 16; mt += nwarps) map_rows(Wu, mt, g, ks, pw, lane);
+    __syncthreads();
+    store_out(out + ((size_t)u * g + a) * D + c, (av + pw[a][c]) / Ls[a]);
 }
 
 }  // namespace dbf
