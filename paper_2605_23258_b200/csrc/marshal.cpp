@@ -1,8 +1,9 @@
 // Argument marshalling of the calls that a serving loop makes, as a CPython module: what binding.py does with ctypes, without a Python
-// object for every pointer.  A call here answers the plain case -- tensors of exactly torch's own classes, structs and counts of exactly
-// their own types, the current stream -- and returns None for everything else (other types, a wrong dtype, device or layout, a given
-// stream), before anything has been launched: binding.py then takes its own path, which raises what it
-// raised before.
+// object for every pointer.  A call here answers the plain case -- tensors of exactly torch's own classes, structs of exactly the binding's
+// own classes, numbers that struct.pack and ctypes would take, the current stream -- and returns None for everything else (other classes, a wrong
+// dtype, device or layout, a tensor missing, a given stream), before anything has been launched: binding.py then takes its own path,
+// which raises what it raised before.  What is refused is refused without an exception, at the first argument that is not plain: the struct's
+// class, which comes first, costs a subclass 0.1 us.
 // A step of one layer (append and attention, 10.5 us on the device) took 14.2 us of host time, 6.3 of them in the library.
 #include <Python.h>
 
@@ -11,6 +12,8 @@
 #include <c10/cuda/CUDAStream.h>
 #include <dlfcn.h>
 #include <torch/csrc/autograd/python_variable.h>
+
+#include <cmath>
 
 #include "vector.h"
 
@@ -30,125 +33,144 @@ const char* const spelled[NAMES] = {"batch", "n_layers", "n_q_heads", "n_kv_head
                                     "n_evict", "ret_k", "ret_v", "apx_k", "ret_pos", "apx_pos"};
 PyObject* name[NAMES];
 
-// The plain case does not hold: the caller's own path decides.
-struct Otherwise {};
-
-struct Ref {                                            // an owned reference
+struct Ref {                                            // an owned reference, or none
     PyObject* o;
-    explicit Ref(PyObject* p) : o(p) { if (!p) { PyErr_Clear(); throw Otherwise(); } }
-    ~Ref() { Py_DECREF(o); }
+    explicit Ref(PyObject* p) : o(p) {}
+    ~Ref() { Py_XDECREF(o); }
     Ref(const Ref&) = delete;
 };
-Ref attr(PyObject* o, Name n) { return Ref(PyObject_GetAttr(o, name[n])); }
-
-int64_t integer(PyObject* o) {
-    if (!PyLong_CheckExact(o)) throw Otherwise();
-    int over = 0;
-    const long long v = PyLong_AsLongLongAndOverflow(o, &over);
-    if (over) throw Otherwise();
-    return v;
-}
-int32_t integer32(PyObject* o) {
-    const int64_t v = integer(o);
-    if (v != (int32_t)v) throw Otherwise();
-    return (int32_t)v;
-}
-float number(PyObject* o) {
-    if (!PyFloat_CheckExact(o)) throw Otherwise();
-    const double v = PyFloat_AS_DOUBLE(o);
-    if (!(v >= -3.4e38 && v <= 3.4e38)) throw Otherwise();
-    return (float)v;
-}
-const at::Tensor& tensor(PyObject* o) {
-    if (!THPVariable_CheckExact(o)) throw Otherwise();
-    return THPVariable_Unpack(o);
-}
-
-vector_shape shape_of(PyObject* o) {
-    if (Py_TYPE(o) != shape_type) throw Otherwise();
-    vector_shape s;
-    s.batch = integer32(attr(o, BATCH).o);
-    s.n_layers = integer32(attr(o, N_LAYERS).o);
-    s.n_q_heads = integer32(attr(o, N_Q_HEADS).o);
-    s.n_kv_heads = integer32(attr(o, N_KV_HEADS).o);
-    s.head_dim = integer32(attr(o, HEAD_DIM).o);
-    s.dtype = integer32(attr(o, DTYPE).o);
-    s.window = integer32(attr(o, WINDOW).o);
-    s.pool_kernel = integer32(attr(o, POOL_KERNEL).o);
-    s.sm_scale = number(attr(o, SM_SCALE).o);
-    s.rope_enabled = integer32(attr(o, ROPE_ENABLED).o);
-    s.rope_theta = number(attr(o, ROPE_THETA).o);
-    return s;
-}
-vector_budget budget_of(PyObject* o) {
-    if (Py_TYPE(o) != budget_type) throw Otherwise();
-    vector_budget b;
-    b.n_tokens = integer(attr(o, N_TOKENS).o);
-    b.n_budget_pairs = integer(attr(o, N_BUDGET_PAIRS).o);
-    b.n_a = integer(attr(o, N_A).o);
-    b.n_pool = integer(attr(o, N_POOL).o);
-    b.n_apx = integer(attr(o, N_APX).o);
-    b.n_ret = integer(attr(o, N_RET).o);
-    b.n_evict = integer(attr(o, N_EVICT).o);
-    return b;
-}
-vector_cache cache_of(PyObject* o) {
-    if (Py_TYPE(o) != cache_type) throw Otherwise();
-    const Ref rk = attr(o, RET_K), rv = attr(o, RET_V), ak = attr(o, APX_K), rp = attr(o, RET_POS), ap = attr(o, APX_POS);
-    const at::Tensor &trk = tensor(rk.o), &tak = tensor(ak.o);
-    if (trk.dim() < 2 || tak.dim() < 2) throw Otherwise();
-    vector_cache c;
-    c.ret_k = trk.data_ptr();
-    c.ret_v = tensor(rv.o).data_ptr();
-    c.apx_k = tak.data_ptr();
-    c.ret_pos = (decltype(c.ret_pos))tensor(rp.o).data_ptr();
-    c.apx_pos = (decltype(c.apx_pos))tensor(ap.o).data_ptr();
-    c.cap_ret = trk.size(1);
-    c.cap_apx = tak.size(1);
-    c.n_ret = integer(attr(o, N_RET).o);
-    c.n_apx = integer(attr(o, N_APX).o);
-    return c;
-}
+struct Workspace { void* p = nullptr; size_t n = 0; };
+struct Out { void* p = nullptr; int32_t type = 0; };
 at::ScalarType type_of(const vector_shape& s) { return s.dtype == VECTOR_BF16 ? at::kBFloat16 : at::kFloat; }
-void* device(PyObject* o, at::ScalarType type) {
-    if (o == Py_None) return nullptr;
-    const at::Tensor& t = tensor(o);
-    if (!t.is_cuda() || !t.is_contiguous() || t.scalar_type() != type) throw Otherwise();
-    return t.data_ptr();
-}
-struct Workspace { void* p; size_t n; };
-Workspace workspace(PyObject* o) {
-    Workspace w = {device(o, at::kByte), 0};
-    if (o != Py_None) w.n = (size_t)tensor(o).numel();
-    return w;
-}
-struct Out { void* p; int32_t type; };
-Out output(PyObject* o) {
-    const at::ScalarType type = tensor(o).scalar_type();
-    if (type != at::kFloat && type != at::kBFloat16) throw Otherwise();
-    return {device(o, type), type == at::kBFloat16 ? VECTOR_BF16 : VECTOR_F32};
-}
-void* stream_of(PyObject* o) {
-    if (o != Py_None) throw Otherwise();
-    return c10::cuda::getCurrentCUDAStream().stream();
-}
 
-// What `call` returns as a Python integer; None where the plain case does not hold.  The library runs without the interpreter's lock,
-// as it does under ctypes.
+// Reads a call's arguments.  `plain` turns false at the first one that is not: what is read from then on is nothing and means nothing.
+struct Reader {
+    bool plain = true;
+    bool need(bool holds) { return plain = plain && holds; }
+    PyObject* attr(PyObject* o, Name n) {               // new, or null
+        PyObject* v = plain ? PyObject_GetAttr(o, name[n]) : nullptr;
+        need(v);
+        return v;
+    }
+    int64_t integer(PyObject* o) {                      // an argument: ctypes takes an int
+        if (!need(o && PyLong_Check(o))) return 0;
+        int over = 0;
+        const long long v = PyLong_AsLongLongAndOverflow(o, &over);
+        need(!over);
+        return v;
+    }
+    int32_t integer32(PyObject* o) {
+        const int64_t v = integer(o);
+        need(v == (int32_t)v);
+        return (int32_t)v;
+    }
+    int64_t field(PyObject* o, Name n) {                // a struct's field: struct.pack takes whatever is an index
+        const Ref v(attr(o, n));
+        if (!plain || PyLong_Check(v.o)) return integer(v.o);
+        if (!need(PyIndex_Check(v.o))) return 0;
+        const Ref i(PyNumber_Index(v.o));
+        return need(i.o) ? integer(i.o) : 0;
+    }
+    int32_t field32(PyObject* o, Name n) {
+        const int64_t v = field(o, n);
+        need(v == (int32_t)v);
+        return (int32_t)v;
+    }
+    float number(PyObject* o, Name n) {                 // whatever is a float, an integer too
+        const Ref v(attr(o, n));
+        if (!plain) return 0.f;
+        const double x = PyFloat_AsDouble(v.o);
+        need(!PyErr_Occurred() && std::isfinite((float)x));
+        return (float)x;
+    }
+    const at::Tensor* tensor(PyObject* o) { return need(o && THPVariable_CheckExact(o)) ? &THPVariable_Unpack(o) : nullptr; }
+    void* device(PyObject* o, at::ScalarType type) {
+        const at::Tensor* t = tensor(o);
+        return t && need(t->is_cuda() && t->is_contiguous() && t->scalar_type() == type) ? t->data_ptr() : nullptr;
+    }
+    void* optional(PyObject* o, at::ScalarType type) { return o == Py_None ? nullptr : device(o, type); }
+    Workspace workspace(PyObject* o) {
+        Workspace w;
+        w.p = optional(o, at::kByte);
+        if (plain && o != Py_None) w.n = (size_t)tensor(o)->numel();
+        return w;
+    }
+    Out output(PyObject* o) {
+        Out out;
+        const at::Tensor* t = tensor(o);
+        if (!t || !need(t->scalar_type() == at::kFloat || t->scalar_type() == at::kBFloat16)) return out;
+        out.type = t->scalar_type() == at::kBFloat16 ? VECTOR_BF16 : VECTOR_F32;
+        out.p = device(o, t->scalar_type());
+        return out;
+    }
+    void* stream(PyObject* o) { return need(o == Py_None) ? c10::cuda::getCurrentCUDAStream().stream() : nullptr; }
+    vector_shape shape(PyObject* o) {
+        vector_shape s = {};
+        if (!need(Py_TYPE(o) == shape_type)) return s;
+        s.batch = field32(o, BATCH);
+        s.n_layers = field32(o, N_LAYERS);
+        s.n_q_heads = field32(o, N_Q_HEADS);
+        s.n_kv_heads = field32(o, N_KV_HEADS);
+        s.head_dim = field32(o, HEAD_DIM);
+        s.dtype = field32(o, DTYPE);
+        s.window = field32(o, WINDOW);
+        s.pool_kernel = field32(o, POOL_KERNEL);
+        s.sm_scale = number(o, SM_SCALE);
+        s.rope_enabled = field32(o, ROPE_ENABLED);
+        s.rope_theta = number(o, ROPE_THETA);
+        return s;
+    }
+    vector_budget budget(PyObject* o) {
+        vector_budget b = {};
+        if (!need(Py_TYPE(o) == budget_type)) return b;
+        b.n_tokens = field(o, N_TOKENS);
+        b.n_budget_pairs = field(o, N_BUDGET_PAIRS);
+        b.n_a = field(o, N_A);
+        b.n_pool = field(o, N_POOL);
+        b.n_apx = field(o, N_APX);
+        b.n_ret = field(o, N_RET);
+        b.n_evict = field(o, N_EVICT);
+        return b;
+    }
+    vector_cache cache(PyObject* o) {
+        vector_cache c = {};
+        if (!need(Py_TYPE(o) == cache_type)) return c;
+        const Ref rk(attr(o, RET_K)), rv(attr(o, RET_V)), ak(attr(o, APX_K)), rp(attr(o, RET_POS)), ap(attr(o, APX_POS));
+        const at::Tensor *trk = tensor(rk.o), *trv = tensor(rv.o), *tak = tensor(ak.o), *trp = tensor(rp.o), *tap = tensor(ap.o);
+        if (!plain || !need(trk->dim() >= 2 && tak->dim() >= 2)) return c;
+        c.ret_k = trk->data_ptr();
+        c.ret_v = trv->data_ptr();
+        c.apx_k = tak->data_ptr();
+        c.ret_pos = (decltype(c.ret_pos))trp->data_ptr();
+        c.apx_pos = (decltype(c.apx_pos))tap->data_ptr();
+        c.cap_ret = trk->size(1);
+        c.cap_apx = tak->size(1);
+        c.n_ret = field(o, N_RET);
+        c.n_apx = field(o, N_APX);
+        return c;
+    }
+};
+
+// What `call` returns as a Python integer; None where the plain case does not hold.
 template <typename F>
 PyObject* plain(Py_ssize_t given, Py_ssize_t wanted, F call) {
     if (given != wanted) { PyErr_SetString(PyExc_TypeError, "wrong number of arguments"); return nullptr; }
+    Reader r;
+    long rc = 0;
     try {
-        return PyLong_FromLong(call());
-    } catch (const Otherwise&) {
+        rc = call(r);
     } catch (const std::exception&) {                   // torch's refusals: a tensor without storage, say
+        r.plain = false;
     }
+    if (r.plain) return PyLong_FromLong(rc);
     PyErr_Clear();
     Py_RETURN_NONE;
 }
+// The library runs without the interpreter's lock, as it does under ctypes; nothing runs where the plain case does not hold.
 template <typename F>
-long unlocked(F f) {
-    long rc;
+long run(const Reader& r, F f) {
+    long rc = 0;
+    if (!r.plain) return rc;
     Py_BEGIN_ALLOW_THREADS
     rc = (long)f();
     Py_END_ALLOW_THREADS
@@ -157,115 +179,114 @@ long unlocked(F f) {
 
 #define METHOD(name) PyObject* name(PyObject*, PyObject* const* a, Py_ssize_t n)
 METHOD(score) {                                         // shape, Q_obs, K, N, scores, raw_out, ws, stream
-    return plain(n, 8, [&] {
-        const vector_shape s = shape_of(a[0]);
-        void *q = device(a[1], type_of(s)), *k = device(a[2], type_of(s));
-        const int64_t N = integer(a[3]);
-        float *out = (float*)device(a[4], at::kFloat), *raw = (float*)device(a[5], at::kFloat);
-        const Workspace w = workspace(a[6]);
-        void* st = stream_of(a[7]);
-        return unlocked([&] { return p_vector_score(&s, q, k, N, out, raw, w.p, w.n, st); });
+    return plain(n, 8, [&](Reader& r) {
+        const vector_shape s = r.shape(a[0]);
+        void *q = r.device(a[1], type_of(s)), *k = r.device(a[2], type_of(s));
+        const int64_t N = r.integer(a[3]);
+        float *out = (float*)r.device(a[4], at::kFloat), *raw = (float*)r.optional(a[5], at::kFloat);
+        const Workspace w = r.workspace(a[6]);
+        void* st = r.stream(a[7]);
+        return run(r, [&] { return p_vector_score(&s, q, k, N, out, raw, w.p, w.n, st); });
     });
 }
 template <typename Fn>
-long route_with(Fn fn, PyObject* const* a) {            // shape, budget, scores, K, V, W, tier, ret_idx, apx_idx, eps_out, pool_idx_out, ws, stream
-    const vector_shape s = shape_of(a[0]);
-    const vector_budget b = budget_of(a[1]);
+long route_with(Fn fn, Reader& r, PyObject* const* a) { // shape, budget, scores, K, V, W, tier, ret_idx, apx_idx, eps_out, pool_idx_out, ws, stream
+    const vector_shape s = r.shape(a[0]);
+    const vector_budget b = r.budget(a[1]);
     const at::ScalarType type = type_of(s);
-    const float* scores = (const float*)device(a[2], at::kFloat);
-    void *k = device(a[3], type), *v = device(a[4], type), *w = device(a[5], type);
-    uint8_t* tier = (uint8_t*)device(a[6], at::kByte);
-    int32_t *ret = (int32_t*)device(a[7], at::kInt), *apx = (int32_t*)device(a[8], at::kInt);
-    float* eps = (float*)device(a[9], at::kFloat);
-    int32_t* pool = (int32_t*)device(a[10], at::kInt);
-    const Workspace ws = workspace(a[11]);
-    void* st = stream_of(a[12]);
-    return unlocked([&] { return fn(&s, &b, scores, k, v, w, tier, ret, apx, eps, pool, ws.p, ws.n, st); });
+    const float* scores = (const float*)r.device(a[2], at::kFloat);
+    void *k = r.device(a[3], type), *v = r.device(a[4], type), *w = r.device(a[5], type);
+    uint8_t* tier = (uint8_t*)r.device(a[6], at::kByte);
+    int32_t *ret = (int32_t*)r.device(a[7], at::kInt), *apx = (int32_t*)r.device(a[8], at::kInt);
+    float* eps = (float*)r.optional(a[9], at::kFloat);
+    int32_t* pool = (int32_t*)r.optional(a[10], at::kInt);
+    const Workspace ws = r.workspace(a[11]);
+    void* st = r.stream(a[12]);
+    return run(r, [&] { return fn(&s, &b, scores, k, v, w, tier, ret, apx, eps, pool, ws.p, ws.n, st); });
 }
-METHOD(route) { return plain(n, 13, [&] { return route_with(p_vector_route, a); }); }
-METHOD(route_layer) { return plain(n, 13, [&] { return route_with(p_vector_route_layer, a); }); }
+METHOD(route) { return plain(n, 13, [&](Reader& r) { return route_with(p_vector_route, r, a); }); }
+METHOD(route_layer) { return plain(n, 13, [&](Reader& r) { return route_with(p_vector_route_layer, r, a); }); }
 template <typename Fn>
-long compact_with(Fn fn, PyObject* const* a) {          // shape, budget, K, V, ret_idx, apx_idx, cache, stream
-    const vector_shape s = shape_of(a[0]);
-    const vector_budget b = budget_of(a[1]);
-    void *k = device(a[2], type_of(s)), *v = device(a[3], type_of(s));
-    const int32_t *ret = (const int32_t*)device(a[4], at::kInt), *apx = (const int32_t*)device(a[5], at::kInt);
-    const vector_cache c = cache_of(a[6]);
-    void* st = stream_of(a[7]);
-    return unlocked([&] { return fn(&s, &b, k, v, ret, apx, &c, st); });
+long compact_with(Fn fn, Reader& r, PyObject* const* a) {      // shape, budget, K, V, ret_idx, apx_idx, cache, stream
+    const vector_shape s = r.shape(a[0]);
+    const vector_budget b = r.budget(a[1]);
+    void *k = r.device(a[2], type_of(s)), *v = r.device(a[3], type_of(s));
+    const int32_t *ret = (const int32_t*)r.device(a[4], at::kInt), *apx = (const int32_t*)r.device(a[5], at::kInt);
+    const vector_cache c = r.cache(a[6]);
+    void* st = r.stream(a[7]);
+    return run(r, [&] { return fn(&s, &b, k, v, ret, apx, &c, st); });
 }
-METHOD(compact) { return plain(n, 8, [&] { return compact_with(p_vector_compact, a); }); }
-METHOD(compact_layer) { return plain(n, 8, [&] { return compact_with(p_vector_compact_layer, a); }); }
+METHOD(compact) { return plain(n, 8, [&](Reader& r) { return compact_with(p_vector_compact, r, a); }); }
+METHOD(compact_layer) { return plain(n, 8, [&](Reader& r) { return compact_with(p_vector_compact_layer, r, a); }); }
 METHOD(decode_attn) {                                   // shape, q, cache, W, out, mode, ws, stream
-    return plain(n, 8, [&] {
-        const vector_shape s = shape_of(a[0]);
-        void* q = device(a[1], type_of(s));
-        const vector_cache c = cache_of(a[2]);
-        void* W = device(a[3], type_of(s));
-        const Out out = output(a[4]);
-        const int32_t mode = integer32(a[5]);
-        const Workspace w = workspace(a[6]);
-        void* st = stream_of(a[7]);
-        return unlocked([&] { return p_vector_decode_attn(&s, q, &c, W, out.p, out.type, mode, w.p, w.n, st); });
+    return plain(n, 8, [&](Reader& r) {
+        const vector_shape s = r.shape(a[0]);
+        void* q = r.device(a[1], type_of(s));
+        const vector_cache c = r.cache(a[2]);
+        void* W = r.device(a[3], type_of(s));
+        const Out out = r.output(a[4]);
+        const int32_t mode = r.integer32(a[5]);
+        const Workspace w = r.workspace(a[6]);
+        void* st = r.stream(a[7]);
+        return run(r, [&] { return p_vector_decode_attn(&s, q, &c, W, out.p, out.type, mode, w.p, w.n, st); });
     });
 }
 METHOD(decode_attn_layer) {                             // shape, q, cache, W_layer, out, ws, stream
-    return plain(n, 7, [&] {
-        const vector_shape s = shape_of(a[0]);
-        void* q = device(a[1], type_of(s));
-        const vector_cache c = cache_of(a[2]);
-        void* W = device(a[3], type_of(s));
-        const Out out = output(a[4]);
-        const Workspace w = workspace(a[5]);
-        void* st = stream_of(a[6]);
-        return unlocked([&] { return p_vector_decode_attn_layer(&s, q, &c, W, out.p, out.type, w.p, w.n, st); });
+    return plain(n, 7, [&](Reader& r) {
+        const vector_shape s = r.shape(a[0]);
+        void* q = r.device(a[1], type_of(s));
+        const vector_cache c = r.cache(a[2]);
+        void* W = r.device(a[3], type_of(s));
+        const Out out = r.output(a[4]);
+        const Workspace w = r.workspace(a[5]);
+        void* st = r.stream(a[6]);
+        return run(r, [&] { return p_vector_decode_attn_layer(&s, q, &c, W, out.p, out.type, w.p, w.n, st); });
     });
 }
 METHOD(decode_attn_static) {                            // shape, q, cache, W, out, mode, stream
-    return plain(n, 7, [&] {
-        const vector_shape s = shape_of(a[0]);
-        void* q = device(a[1], type_of(s));
-        const vector_cache c = cache_of(a[2]);
-        void* W = device(a[3], type_of(s));
-        const Out out = output(a[4]);
-        const int32_t mode = integer32(a[5]);
-        void* st = stream_of(a[6]);
-        return unlocked([&] { return p_vector_decode_attn_static(&s, q, &c, W, out.p, out.type, mode, st); });
+    return plain(n, 7, [&](Reader& r) {
+        const vector_shape s = r.shape(a[0]);
+        void* q = r.device(a[1], type_of(s));
+        const vector_cache c = r.cache(a[2]);
+        void* W = r.device(a[3], type_of(s));
+        const Out out = r.output(a[4]);
+        const int32_t mode = r.integer32(a[5]);
+        void* st = r.stream(a[6]);
+        return run(r, [&] { return p_vector_decode_attn_static(&s, q, &c, W, out.p, out.type, mode, st); });
     });
 }
 METHOD(append) {                                        // shape, cache, k_new, v_new, pos, stream
-    return plain(n, 6, [&] {
-        const vector_shape s = shape_of(a[0]);
-        const vector_cache c = cache_of(a[1]);
-        void *k = device(a[2], type_of(s)), *v = device(a[3], type_of(s));
-        const int32_t pos = integer32(a[4]);
-        void* st = stream_of(a[5]);
-        return unlocked([&] { return p_vector_append(&s, &c, k, v, pos, st); });
+    return plain(n, 6, [&](Reader& r) {
+        const vector_shape s = r.shape(a[0]);
+        const vector_cache c = r.cache(a[1]);
+        void *k = r.device(a[2], type_of(s)), *v = r.device(a[3], type_of(s));
+        const int32_t pos = r.integer32(a[4]);
+        void* st = r.stream(a[5]);
+        return run(r, [&] { return p_vector_append(&s, &c, k, v, pos, st); });
     });
 }
 // Compressor.append's own conditions on top: plain rows of the shape's size on the current device, room for one more, and not what the
 // entry point refuses (rows off a 16-byte boundary): those rows are assigned.
 METHOD(append_rows) {                                   // shape, cache, k_new, v_new, pos
-    return plain(n, 5, [&] {
-        const vector_shape s = shape_of(a[0]);
-        const vector_cache c = cache_of(a[1]);
-        if ((PyObject*)Py_TYPE(a[2]) != THPVariableClass || (PyObject*)Py_TYPE(a[3]) != THPVariableClass) throw Otherwise();
-        const Ref rk = attr(a[1], RET_K), rv = attr(a[1], RET_V), rp = attr(a[1], RET_POS);
-        const at::Tensor &trk = tensor(rk.o), &trv = tensor(rv.o), &tk = tensor(a[2]), &tv = tensor(a[3]);
-        if (trk.dim() != 3 || tk.dim() != 2 || tv.dim() != 2) throw Otherwise();
-        const int64_t U = trk.size(0), cap = trk.size(1), d = trk.size(2);
-        const bool rows = tk.size(0) == U && tk.size(1) == d && tv.size(0) == U && tv.size(1) == d && d == s.head_dim &&
+    return plain(n, 5, [&](Reader& r) {
+        const vector_shape s = r.shape(a[0]);
+        const vector_cache c = r.cache(a[1]);
+        r.need((PyObject*)Py_TYPE(a[2]) == THPVariableClass && (PyObject*)Py_TYPE(a[3]) == THPVariableClass);
+        const Ref rk(r.attr(a[1], RET_K)), rv(r.attr(a[1], RET_V)), rp(r.attr(a[1], RET_POS));
+        const at::Tensor *trk = r.tensor(rk.o), *trv = r.tensor(rv.o), *trp = r.tensor(rp.o), *tk = r.tensor(a[2]), *tv = r.tensor(a[3]);
+        if (!r.plain || !r.need(trk->dim() == 3 && tk->dim() == 2 && tv->dim() == 2)) return 0L;
+        const int64_t U = trk->size(0), cap = trk->size(1), d = trk->size(2);
+        const bool rows = tk->size(0) == U && tk->size(1) == d && tv->size(0) == U && tv->size(1) == d && d == s.head_dim &&
                           U == (int64_t)s.batch * s.n_layers * s.n_kv_heads;
         const int dev = c10::cuda::current_device();
-        const bool here = tk.get_device() == dev && tv.get_device() == dev && trk.get_device() == dev && trv.get_device() == dev;
-        if (!rows || !here || c.n_ret >= cap || trv.nbytes() != trk.nbytes() || !trk.is_contiguous() || !trv.is_contiguous() ||
-            tensor(rp.o).numel() != U * cap || tk.requires_grad() || tv.requires_grad())
-            throw Otherwise();
-        void *k = device(a[2], type_of(s)), *v = device(a[3], type_of(s));
-        const int32_t pos = integer32(a[4]);
-        void* st = stream_of(Py_None);
-        const long rc = unlocked([&] { return p_vector_append(&s, &c, k, v, pos, st); });
-        if (rc == VECTOR_ERR_SHAPE) throw Otherwise();
+        const bool here = tk->get_device() == dev && tv->get_device() == dev && trk->get_device() == dev && trv->get_device() == dev;
+        r.need(rows && here && c.n_ret < cap && trv->nbytes() == trk->nbytes() && trk->is_contiguous() && trv->is_contiguous() &&
+               trp->numel() == U * cap && !tk->requires_grad() && !tv->requires_grad());
+        void *k = r.device(a[2], type_of(s)), *v = r.device(a[3], type_of(s));
+        const int32_t pos = r.integer32(a[4]);
+        void* st = r.stream(Py_None);
+        const long rc = run(r, [&] { return p_vector_append(&s, &c, k, v, pos, st); });
+        r.need(rc != VECTOR_ERR_SHAPE);
         return rc;
     });
 }
