@@ -230,6 +230,11 @@ def _stream(stream) -> int:
     return stream.cuda_stream if hasattr(stream, "cuda_stream") else int(stream)
 
 
+def _handle(stream):
+    """The same for the extension module, which asks for the current stream itself."""
+    return None if stream is None else _stream(stream)
+
+
 def _ws(ws: torch.Tensor | None):
     if ws is None:
         return None, 0
@@ -310,7 +315,7 @@ def alloc_cache(shape: Shape, budget: Budget, extra_rows: int = 0, device="cuda"
 
 
 def vector_score(shape: Shape, Q_obs, K, N: int, scores, raw_out=None, ws=None, stream=None):
-    rc = (_marshal_module or _marshal()).score(shape, Q_obs, K, N, scores, raw_out, ws, stream)
+    rc = (_marshal_module or _marshal()).score(shape, Q_obs, K, N, scores, raw_out, ws, _handle(stream))
     if rc is not None:
         if rc:
             _check(rc, "vector_score")
@@ -356,7 +361,7 @@ def vector_truncate(shape: Shape, budget: Budget, eps, pool_idx, tier, ret_idx, 
 
 def vector_route(shape: Shape, budget: Budget, scores, K, V, W, tier, ret_idx, apx_idx, eps_out=None,
                  pool_idx_out=None, ws=None, stream=None):
-    rc = (_marshal_module or _marshal()).route(shape, budget, scores, K, V, W, tier, ret_idx, apx_idx, eps_out, pool_idx_out, ws, stream)
+    rc = (_marshal_module or _marshal()).route(shape, budget, scores, K, V, W, tier, ret_idx, apx_idx, eps_out, pool_idx_out, ws, _handle(stream))
     if rc is not None:
         if rc:
             _check(rc, "vector_route")
@@ -405,7 +410,7 @@ def vector_sync_check(stream=None):
 
 
 def vector_compact(shape: Shape, budget: Budget, K, V, ret_idx, apx_idx, cache: Cache, stream=None):
-    rc = (_marshal_module or _marshal()).compact(shape, budget, K, V, ret_idx, apx_idx, cache, stream)
+    rc = (_marshal_module or _marshal()).compact(shape, budget, K, V, ret_idx, apx_idx, cache, _handle(stream))
     if rc is not None:
         if rc:
             _check(rc, "vector_compact")
@@ -420,7 +425,7 @@ def vector_compact(shape: Shape, budget: Budget, K, V, ret_idx, apx_idx, cache: 
 
 def vector_append(shape: Shape, cache: Cache, k_new, v_new, pos: int, stream=None):
     """k_new, v_new [U][d] become row cache.n_ret of the retained pool; the caller bumps cache.n_ret."""
-    rc = (_marshal_module or _marshal()).append(shape, cache, k_new, v_new, pos, stream)
+    rc = (_marshal_module or _marshal()).append(shape, cache, k_new, v_new, pos, _handle(stream))
     if rc is not None:
         if rc:
             _check(rc, "vector_append")
@@ -441,7 +446,7 @@ def append_rows(shape: Shape, cache: Cache, k_new, v_new, pos) -> bool:
 
 
 def vector_decode_attn(shape: Shape, q, cache: Cache, W, out, mode: int = 0, ws=None, stream=None):
-    rc = (_marshal_module or _marshal()).decode_attn(shape, q, cache, W, out, mode, ws, stream)
+    rc = (_marshal_module or _marshal()).decode_attn(shape, q, cache, W, out, mode, ws, _handle(stream))
     if rc is not None:
         if rc:
             _check(rc, "vector_decode_attn")
@@ -478,7 +483,7 @@ def vector_residual_layer(shape: Shape, K, V, W_layer, N: int, idx, n_idx: int, 
 
 def vector_route_layer(shape: Shape, budget: Budget, layer_scores, K, V, W_layer, tier, ret_idx, apx_idx,
                        eps_out=None, pool_idx_out=None, ws=None, stream=None):
-    rc = (_marshal_module or _marshal()).route_layer(shape, budget, layer_scores, K, V, W_layer, tier, ret_idx, apx_idx, eps_out, pool_idx_out, ws, stream)
+    rc = (_marshal_module or _marshal()).route_layer(shape, budget, layer_scores, K, V, W_layer, tier, ret_idx, apx_idx, eps_out, pool_idx_out, ws, _handle(stream))
     if rc is not None:
         if rc:
             _check(rc, "vector_route_layer")
@@ -495,7 +500,7 @@ def vector_route_layer(shape: Shape, budget: Budget, layer_scores, K, V, W_layer
 
 
 def vector_compact_layer(shape: Shape, budget: Budget, K, V, ret_idx, apx_idx, cache: Cache, stream=None):
-    rc = (_marshal_module or _marshal()).compact_layer(shape, budget, K, V, ret_idx, apx_idx, cache, stream)
+    rc = (_marshal_module or _marshal()).compact_layer(shape, budget, K, V, ret_idx, apx_idx, cache, _handle(stream))
     if rc is not None:
         if rc:
             _check(rc, "vector_compact_layer")
@@ -509,7 +514,7 @@ def vector_compact_layer(shape: Shape, budget: Budget, K, V, ret_idx, apx_idx, c
 
 
 def vector_decode_attn_layer(shape: Shape, q, cache: Cache, W_layer, out, ws=None, stream=None):
-    rc = (_marshal_module or _marshal()).decode_attn_layer(shape, q, cache, W_layer, out, ws, stream)
+    rc = (_marshal_module or _marshal()).decode_attn_layer(shape, q, cache, W_layer, out, ws, _handle(stream))
     if rc is not None:
         if rc:
             _check(rc, "vector_decode_attn_layer")
@@ -542,7 +547,7 @@ def vector_decode_attn_static(shape: Shape, q, cache: Cache, W, out, mode: int =
     that need more raise VectorError (workspace).  Calls on one device share that array,
     so calls that overlap on the GPU race; make the first call per device at start-up.
     """
-    rc = (_marshal_module or _marshal()).decode_attn_static(shape, q, cache, W, out, mode, stream)
+    rc = (_marshal_module or _marshal()).decode_attn_static(shape, q, cache, W, out, mode, _handle(stream))
     if rc is not None:
         if rc:
             _check(rc, "vector_decode_attn_static")

@@ -1,7 +1,7 @@
 // Argument marshalling of the calls that a serving loop makes, as a CPython module: what binding.py does with ctypes, without a Python
 // object for every pointer.  A call here answers the plain case -- tensors of exactly torch's own classes, structs of exactly the binding's
-// own classes, numbers that struct.pack and ctypes would take, the current stream -- and returns None for everything else (other classes, a wrong
-// dtype, device or layout, a tensor missing, a given stream), before anything has been launched: binding.py then takes its own path,
+// own classes, numbers that struct.pack and ctypes would take, the current stream or a stream's handle -- and returns None for everything else
+// (other classes, a wrong dtype, device or layout, a tensor missing), before anything has been launched: binding.py then takes its own path,
 // which raises what it raised before.  What is refused is refused without an exception, at the first argument that is not plain: the struct's
 // class, which comes first, costs a subclass 0.1 us.
 // A step of one layer (append and attention, 10.5 us on the device) took 14.2 us of host time, 6.3 of them in the library.
@@ -103,7 +103,14 @@ struct Reader {
         out.p = device(o, t->scalar_type());
         return out;
     }
-    void* stream(PyObject* o) { return need(o == Py_None) ? c10::cuda::getCurrentCUDAStream().stream() : nullptr; }
+    void* stream(PyObject* o) {                         // None, the current one, or a handle
+        if (!plain) return nullptr;
+        if (o == Py_None) return c10::cuda::getCurrentCUDAStream().stream();
+        if (!need(PyLong_CheckExact(o))) return nullptr;
+        void* p = PyLong_AsVoidPtr(o);
+        need(!PyErr_Occurred());
+        return p;
+    }
     vector_shape shape(PyObject* o) {
         vector_shape s = {};
         if (!need(Py_TYPE(o) == shape_type)) return s;

@@ -60,3 +60,54 @@ def test_numbers_that_are_refused():
         with pytest.raises(Exception) as e:
             vec.vector_workspace_bytes(vec.Shape(**{**sh, **bad}), budget)
         assert type(e.value).__module__ in ("struct", "builtins")
+
+
+class _Handle:
+    def __init__(self, stream):
+        self.cuda_stream = stream.cuda_stream
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("form", ["object", "handle", "wrapped", "default"])
+def test_a_given_stream(monkeypatch, form):
+    """Every call of a loop on a given stream, without ctypes, against ctypes on the same stream; the stream that it says is the one that
+    runs it: work queued there ahead of the call is seen by it."""
+    sh = vec.Shape(1, 1, 4, 2, D, vec.VECTOR_BF16, 16)
+    got = []
+    for plain in (True, False):
+        side = torch.cuda.default_stream() if form == "default" else torch.cuda.Stream()
+        st = {"object": side, "handle": side.cuda_stream, "wrapped": _Handle(side), "default": 0}[form]
+        c, q, W, k, v = _problem(sh)
+        b, ws = c.budget, c.ws
+        K, Q = torch.randn(2, N, D, generator=torch.Generator().manual_seed(1)).cuda().bfloat16(), q.repeat_interleave(16, 1).view(2, 2, 16, D).contiguous()
+        out, out2 = (torch.zeros(2, 2, D, device="cuda") for _ in range(2))
+        k2, big = torch.zeros_like(k), torch.zeros(64 << 20, device="cuda")
+        torch.cuda.synchronize()
+        with monkeypatch.context() as m:
+            if plain:
+                _no_ctypes(m)
+            else:
+                m.setattr(B, "_marshal_module", _Nothing())
+            with torch.cuda.stream(side):
+                for _ in range(20):
+                    big.add_(1)
+                k2.copy_(k)
+            vec.vector_score(sh, Q, K, N, c.scores, None, ws, st)
+            vec.vector_route(sh, b, c.scores, K, K, W, c.tier, c.ret_idx, c.apx_idx, None, None, ws, st)
+            c.cache.n_ret = b.n_ret
+            vec.vector_compact(sh, b, K, K, c.ret_idx, c.apx_idx, c.cache, st)
+            vec.vector_append(sh, c.cache, k2, v, N, st)
+            c.cache.n_ret += 1
+            vec.vector_decode_attn(sh, q, c.cache, W, out, 0, ws, st)
+            vec.vector_decode_attn_static(sh, q, c.cache, W, out2, 0, st)
+        torch.cuda.synchronize()
+        assert torch.equal(c.cache.ret_k[:, c.cache.n_ret - 1], k)
+        got.append((c.scores, c.tier, c.ret_idx, c.apx_idx, c.cache.ret_k[:, :c.cache.n_ret], c.cache.ret_v[:, :c.cache.n_ret], out, out2))
+    assert all(torch.equal(a, b) for a, b in zip(*got))
+
+
+class _Nothing:
+    """Leaves every call to ctypes."""
+
+    def __getattr__(self, name):
+        return lambda *args: None
