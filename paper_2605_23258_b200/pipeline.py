@@ -65,14 +65,30 @@ class Compressor:
 
     def append(self, k_new, v_new, pos: int):
         """Keeps a generated token in full: writes its row behind the retained pool."""
-        c = self.cache
+        c, sh = self.cache, self.shape
         # One kernel copies plain rows on the current device; the rest of what can be assigned to the rows is assigned: other types,
         # strided rows, rows off a 16-byte boundary.
-        if B.append_rows(self.shape, c, k_new, v_new, pos):
+        if B.append_rows(sh, c, k_new, v_new, pos):
             c.n_ret += 1
             return
-        if c.n_ret >= c.ret_k.shape[1]:
+        rk, rv = c.ret_k, c.ret_v
+        U, cap, d = rk.shape
+        if c.n_ret >= cap:
             raise ValueError("retained pool is full")
+        # A shape or a cache of a class that packs in its own way: the entry point itself says what it refuses.
+        if (type(pos) is int and -2**31 <= pos < 2**31 and type(k_new) is type(v_new) is torch.Tensor
+                and k_new.shape == v_new.shape == (U, d) and U == sh.units and d == sh.head_dim
+                and k_new.get_device() == v_new.get_device() == rv.get_device() == rk.get_device() >= 0 and rk.get_device() == torch.cuda.current_device()
+                and k_new.dtype == v_new.dtype == sh.torch_dtype and k_new.is_contiguous() and v_new.is_contiguous()
+                and rv.nbytes == rk.nbytes and rk.is_contiguous() and rv.is_contiguous() and c.ret_pos.numel() == U * cap
+                and not (k_new.requires_grad or v_new.requires_grad)):
+            try:
+                B.vector_append(sh, c, k_new, v_new, pos)
+                c.n_ret += 1
+                return
+            except B.VectorError as e:
+                if e.status != -2:
+                    raise
         c.ret_k[:, c.n_ret] = k_new
         c.ret_v[:, c.n_ret] = v_new
         c.ret_pos[:, c.n_ret] = pos

@@ -111,3 +111,57 @@ class _Nothing:
 
     def __getattr__(self, name):
         return lambda *args: None
+
+
+class _Shape(vec.Shape):
+    """A program's own shape."""
+
+
+class _Cache(vec.Cache):
+    """A program's own cache."""
+
+
+class _Packs(vec.Shape):
+    """One that packs in its own way: the module may not read it."""
+
+    def _p(self):
+        return vec.Shape(1, 1, 4, 2, D, vec.VECTOR_BF16, 16)._p()
+
+
+class _Typed(vec.Shape):
+    torch_dtype = torch.bfloat16
+
+
+class _PacksCache(vec.Cache):
+    def _p(self):
+        return vec.Cache._p(self)
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("shape,cache", [(_Shape, vec.Cache), (vec.Shape, _Cache), (_Shape, _Cache), (_Packs, vec.Cache), (_Typed, vec.Cache), (vec.Shape, _PacksCache)])
+def test_appending_with_classes_of_the_program(shape, cache):
+    """One kernel, as for the binding's own classes; rows that it refuses are assigned."""
+    c, q, W, k, v = _problem(vec.Shape(1, 1, 4, 2, D, vec.VECTOR_BF16, 16))
+    c.shape, o = shape(1, 1, 4, 2, D, vec.VECTOR_BF16, 16), c.cache
+    c.cache = cache(o.ret_k, o.ret_v, o.apx_k, o.ret_pos, o.apx_pos, o.n_ret, o.n_apx)
+    n, before = c.cache.n_ret, vec.vector_kernel_launches()
+    c.append(k, v, N)
+    assert vec.vector_kernel_launches() == before + 1 and c.cache.n_ret == n + 1
+    shifted = torch.empty(2 * D + 1, dtype=torch.bfloat16, device="cuda")[1:].view(2, D).copy_(k)
+    for i, (a, b) in enumerate(((k.double(), v), (shifted, v), (k, v[:1]))):
+        c.append(a, b, N + 1 + i)
+    assert vec.vector_kernel_launches() == before + 1 and c.cache.n_ret == n + 4
+    assert all(torch.equal(c.cache.ret_k[:, n + i], k) for i in range(4)) and torch.equal(c.cache.ret_v[:, n + 1], v)
+    assert torch.equal(c.cache.ret_pos[:, n:n + 4], torch.arange(N, N + 4, device="cuda", dtype=torch.int32).expand(2, 4))
+    with pytest.raises(ValueError):
+        c.append(k, v, N)
+
+
+@pytest.mark.gpu
+def test_which_classes_the_module_reads():
+    c, q, W, k, v = _problem(vec.Shape(1, 1, 4, 2, D, vec.VECTOR_BF16, 16))
+    o, out = c.cache, torch.empty(2, 2, D, device="cuda")
+    for shape, cache, read in ((vec.Shape, vec.Cache, True), (_Shape, _Cache, True), (_Packs, vec.Cache, False), (_Typed, vec.Cache, False), (vec.Shape, _PacksCache, False)):
+        rc = B._marshal().decode_attn(shape(1, 1, 4, 2, D, vec.VECTOR_BF16, 16), q, cache(o.ret_k, o.ret_v, o.apx_k, o.ret_pos, o.apx_pos, o.n_ret, o.n_apx),
+                                      W, out, 0, c.ws, None)
+        assert rc == 0 if read else rc is None
