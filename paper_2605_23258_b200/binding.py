@@ -8,13 +8,15 @@ status.  There is no fallback: if the shared library is missing the import of
 any entry point fails loudly.
 
 The calls of a serving loop try the extension module first (``csrc/marshal.cpp``), which marshals plain tensors and structs without a
-Python object for every pointer and answers None, having done nothing, where an argument is anything else; ctypes then takes the call.
+Python object for every pointer and answers None, having done nothing, where an argument is anything else; ctypes then takes the call,
+and all calls where the module has not been built.
 """
 from __future__ import annotations
 
 import ctypes
 import os
 import struct
+import warnings
 from dataclasses import dataclass
 
 import torch
@@ -196,13 +198,25 @@ def load_library() -> ctypes.CDLL:
     return lib
 
 
+class _CtypesOnly:
+    """Stands in for the extension module where there is none: leaves every call to ctypes."""
+
+    def __getattr__(self, name):
+        return lambda *args: None
+
+
 def _marshal():
-    """The extension module, bound to the loaded library; raises if it has not been built."""
+    """The extension module, bound to the loaded library; where it has not been built, or cannot be loaded, a warning and its stand-in."""
     global _marshal_module
     if _marshal_module is None:
         lib = load_library()
-        from . import _marshal as module
-        module.bind(lib._handle, Shape, Budget, Cache)
+        try:
+            from . import _marshal as module
+            module.bind(lib._handle, Shape, Budget, Cache)
+        except ImportError as e:
+            warnings.warn(f"the extension module beside {_LIB_PATH} cannot be used ({e}): every call goes through ctypes, at some microseconds more; "
+                          "build it with `python -m paper_2605_23258_b200.build`", RuntimeWarning, stacklevel=3)
+            module = _CtypesOnly()
         _marshal_module = module
     return _marshal_module
 

@@ -4,6 +4,7 @@ from __future__ import annotations
 import os
 import subprocess
 import sys
+import warnings
 
 HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(HERE, "csrc")
@@ -52,10 +53,19 @@ def build_marshal(force: bool = False) -> str:
 def build(force: bool = False, verbose: bool = False) -> str:
     """Compile every translation unit to an object and link the shared library.  Extra nvcc flags can be
     given in the environment variable VECTOR_NVCC_FLAGS (e.g. -DVECTOR_SCORE_POLY16=6 for the sweep of the
-    share of softmax exponentials evaluated on the FMA pipe)."""
-    build_marshal(force)
-    if not force and not _stale():
-        return LIB
+    share of softmax exponentials evaluated on the FMA pipe).  The library comes first and needs nvcc only; where the extension module
+    cannot be compiled, that is a warning."""
+    if force or _stale():
+        _build_library(verbose)
+    try:
+        build_marshal(force)
+    except Exception as e:
+        warnings.warn(f"the extension module that marshals arguments was not built ({e!r}): it needs a C++ compiler, Python's headers and a CUDA build of "
+                      "torch; without it every call goes through ctypes", RuntimeWarning)
+    return LIB
+
+
+def _build_library(verbose: bool) -> None:
     objdir = os.path.join(HERE, "_build")
     os.makedirs(objdir, exist_ok=True)
     nvcc = _nvcc()
@@ -77,7 +87,6 @@ def build(force: bool = False, verbose: bool = False) -> str:
     tmp = LIB + f".tmp{os.getpid()}"
     subprocess.check_call([nvcc, "-shared", "-o", tmp, *objs, "-gencode", "arch=compute_100a,code=sm_100a"])
     os.replace(tmp, LIB)
-    return LIB
 
 
 if __name__ == "__main__":
