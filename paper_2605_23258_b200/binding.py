@@ -14,8 +14,11 @@ and all calls where the module has not been built.
 from __future__ import annotations
 
 import ctypes
+import importlib.machinery
+import importlib.util
 import os
 import struct
+import sysconfig
 import warnings
 from dataclasses import dataclass
 
@@ -198,6 +201,12 @@ def load_library() -> ctypes.CDLL:
     return lib
 
 
+def marshal_path() -> str:
+    """The extension module's file.  Its code has the layouts of torch's and Python's objects compiled in, so the name carries both versions:
+    another torch or Python looks for another file."""
+    return os.path.join(_HERE, f"_marshal-torch{torch.__version__}{sysconfig.get_config_var('EXT_SUFFIX')}")
+
+
 class _CtypesOnly:
     """Stands in for the extension module where there is none: leaves every call to ctypes."""
 
@@ -210,11 +219,14 @@ def _marshal():
     global _marshal_module
     if _marshal_module is None:
         lib = load_library()
+        path = marshal_path()
         try:
-            from . import _marshal as module
+            loader = importlib.machinery.ExtensionFileLoader(f"{__package__}._marshal", path)
+            module = importlib.util.module_from_spec(importlib.util.spec_from_file_location(loader.name, path, loader=loader))
+            loader.exec_module(module)
             module.bind(lib._handle, Shape, Budget, Cache)
         except ImportError as e:
-            warnings.warn(f"the extension module beside {_LIB_PATH} cannot be used ({e}): every call goes through ctypes, at some microseconds more; "
+            warnings.warn(f"the extension module {path} cannot be used ({e}): every call goes through ctypes, at some microseconds more; "
                           "build it with `python -m paper_2605_23258_b200.build`", RuntimeWarning, stacklevel=3)
             module = _CtypesOnly()
         _marshal_module = module

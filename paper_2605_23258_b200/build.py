@@ -6,11 +6,12 @@ import subprocess
 import sys
 import warnings
 
+from .binding import marshal_path
+
 HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(HERE, "csrc")
 INCLUDE = os.path.join(os.path.dirname(HERE), "include")
 LIB = os.path.join(HERE, "libvector.so")
-MARSHAL = os.path.join(HERE, "_marshal.so")
 
 SOURCES = ["host.cpp", "score.cu", "keydiff.cu", "route.cu", "compact.cu", "decode.cu", "decode_layer.cu", "diagnostics.cu"]
 NVCC_FLAGS = ["-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
@@ -35,19 +36,21 @@ def _stale() -> bool:
 
 def build_marshal(force: bool = False) -> str:
     """The extension module behind the binding (csrc/marshal.cpp): plain C++ against the headers of Python and torch."""
-    src = os.path.join(CSRC, "marshal.cpp")
-    if not force and not _older(MARSHAL, [src]):
-        return MARSHAL
+    src, target = os.path.join(CSRC, "marshal.cpp"), marshal_path()
+    if not force and not _older(target, [src]):
+        return target
     import shutil
     import sysconfig
+    import torch
     from torch.utils.cpp_extension import include_paths, library_paths
     cuda = os.path.dirname(os.path.dirname(os.path.realpath(shutil.which(_nvcc()) or _nvcc())))
     incs = [INCLUDE, *include_paths(), sysconfig.get_paths()["include"], os.path.join(cuda, "include")]
-    tmp = MARSHAL + f".tmp{os.getpid()}"
-    subprocess.check_call([os.environ.get("CXX", "g++"), "-O2", "-std=c++17", "-fPIC", "-shared", "-fvisibility=hidden", *(f"-I{i}" for i in incs), src,
+    tmp = target + f".tmp{os.getpid()}"
+    subprocess.check_call([os.environ.get("CXX", "g++"), "-O2", "-std=c++17", "-fPIC", "-shared", "-fvisibility=hidden",
+                           f"-D_GLIBCXX_USE_CXX11_ABI={int(torch.compiled_with_cxx11_abi())}", *(f"-I{i}" for i in incs), src,
                            *(f"-L{p}" for p in library_paths()), "-ltorch_python", "-ltorch_cpu", "-lc10", "-lc10_cuda", "-o", tmp])
-    os.replace(tmp, MARSHAL)
-    return MARSHAL
+    os.replace(tmp, target)
+    return target
 
 
 def build(force: bool = False, verbose: bool = False) -> str:
