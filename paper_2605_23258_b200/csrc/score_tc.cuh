@@ -228,6 +228,7 @@ __device__ __forceinline__ void block_teardown(Sync& sy) {
 #define VECTOR_SCORE_POLY16 4
 #endif
 constexpr int POLY16 = VECTOR_SCORE_POLY16;
+static_assert(POLY16 >= 0 && POLY16 <= 16 && POLY16 % 2 == 0, "VECTOR_SCORE_POLY16: exponentials go by pairs, an even number of 16");
 // p * 2^n for t = 1.5 * 2^23 + n: one multiply-add on the bits.
 __device__ __forceinline__ float scaled(float p, float t) {
     uint32_t r;
