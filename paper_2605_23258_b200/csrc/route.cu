@@ -388,6 +388,7 @@ static vector_status launch_pool_select(const Dims& dm, const vector_budget* bud
     const int64_t n = budget->n_tokens;
     const int nw = pool_select_warps(n, dm.U, budget->n_pool);
     if (nw == 0) {
+        // Beyond 8192 elements lists that share multiprocessors come here, too, where they do not fit the blocks' shared memory.
         const bool wide = regs_wide(n, dm.U) || n > SEL_REGS16;
         auto kern = wide ? (n <= 4096 ? pool_select_regs<32, 4> : n <= 8192 ? pool_select_regs<32, 8> : n <= SEL_REGS16 ? pool_select_regs<32, 16>
                                                                                                                   : pool_select_regs<32, 32>)
@@ -412,7 +413,7 @@ static vector_status launch_truncate(const Dims& dm, const vector_budget* budget
     const int64_t n = budget->n_pool;
     const int nw = truncate_warps(n, dm.U);
     if (nw == 0) {
-        const bool wide = regs_wide(n, dm.U) || n > 8192;
+        const bool wide = regs_wide(n, dm.U);           // beyond 8192 elements Step 3 takes registers for at most one list a multiprocessor only
         auto kern = wide ? (n <= 4096 ? truncate_regs<32, 4> : n <= 8192 ? truncate_regs<32, 8> : truncate_regs<32, 16>)
                          : n <= 2048 ? truncate_regs<16, 4> : n <= 4096 ? truncate_regs<16, 8> : truncate_regs<16, 16>;
         VEC_CUDA_CHECK(launch_maybe_dependent(dependent, kern, dim3(dm.U), dim3(wide ? 1024 : 512), 0, st, eps, pool,
