@@ -16,9 +16,10 @@
 // them for the tensor cores waits for all that it has in flight, the next stages' copies among them: with eight warps filling
 // every stage together, a step took the latency of memory (245 us for 16 layers of 4914 listed tokens and 8 heads).  So every
 // stage has a loader warp of its own, which has nothing else in flight: 176 us, and 180 in pairs.  There the issue of the products
-// was the longest chain of a step (see the MMA role): 157 us (in a graph by itself 143, by single blocks 161), of which the products
-// need 75 at the tensor rate, 104 at the rate of a library product.  The products take two output heads at a time (a third fewer bytes
-// than head by head), and the value rows go straight to the epilogue's registers.
+// was the longest chain of a step (see the MMA role): 154 us from start to end, 143 of them behind the selection that it waits for (by
+// single blocks 161), of which the products need 75 at the tensor rate, 104 at the rate of a library product.  That is at 1965 MHz: a loop
+// of these calls settles at 1340 MHz under the 1000 W cap, 173 us behind the selection.  The products take two output heads at a time (a
+// third fewer bytes than head by head), and the value rows go straight to the epilogue's registers.
 //
 // Persistent groups (blocks or pairs, one block per multiprocessor) own equal contiguous ranges of the sequence of items (tile, pair
 // of output heads), which balances better than whole tiles: 624 tiles are 4.2 a block.  A tile cut by the end of a range is finished

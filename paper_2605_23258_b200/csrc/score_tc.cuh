@@ -216,8 +216,9 @@ __device__ __forceinline__ void block_teardown(Sync& sy) {
     }
 }
 
-// The exponential unit (16 results per clock per SM) is what bounds both passes, so POLY16 of every
-// 16 exponentials are evaluated on the FMA pipe instead: 2^x = 2^n p(f) with n = round(x),
+// The exponential unit (16 results per clock per SM) is the busiest of both passes, 0.75 and 0.78 with POLY16 of every 16 exponentials
+// evaluated on the FMA pipe instead (0.51 and 0.54; issue slots 0.55, tensor pipe 0.50); what bounds a long call is the 1000 W cap, where
+// four and six of 16 take the same time.  2^x = 2^n p(f) with n = round(x),
 // f = x - n in [-1/2, 1/2] and p the degree-4 minimax polynomial of 2^f (relative error 2.7e-6);
 // n is added to the exponent field.  x is clamped from below to -126: smaller results do not
 // matter to a sum whose largest term is of order one.  UPPER (the first pass, whose reference lags; in the second no logit exceeds
