@@ -1,6 +1,10 @@
 """The forms of the decode merge, on either side of each line of the rule between them, with RoPE records too and with units of so many
 records that a lane reads two headers.  Sampled units against the oracle."""
+import json
+import os
 import re
+import subprocess
+import sys
 
 import pytest
 import torch
@@ -43,21 +47,32 @@ def test_two_headers_a_lane(oracle, U, g, d, n_ret, n_apx, rope):
     _checked(oracle, U, g, d, n_ret, n_apx, rope)
 
 
-def _merge_kernel(d, g, U):
-    q, cache, W = decode_problem(U, g, d, torch.bfloat16, 64, 64, 5)
-    decode_call(q, cache, W, False)
-    with torch.profiler.profile(activities=[torch.profiler.ProfilerActivity.CUDA]) as prof:
-        decode_call(q, cache, W, False)
-    names = [e.name for e in prof.events() if "decode_merge" in e.name]
+def _merge_kernels(shapes):
+    """The merge that each (d, g, U) takes, by its name in a profile: of a process of its own, since a process does not profile again and again."""
+    program = """if True:
+        import json, sys
+        import torch
+        from helpers import decode_call, decode_problem
+        names = []
+        with torch.profiler.profile(activities=[torch.profiler.ProfilerActivity.CUDA]) as prof:
+            for d, g, U in json.loads(sys.argv[1]):
+                decode_call(*decode_problem(U, g, d, torch.bfloat16, 64, 64, 5), False)
+        print(json.dumps([e.name for e in sorted(prof.events(), key=lambda e: e.time_range.start) if "decode_merge" in e.name]))
+    """
+    here = os.path.dirname(os.path.abspath(__file__))
+    env = dict(os.environ, PYTHONPATH=os.pathsep.join([os.path.dirname(here), here, os.environ.get("PYTHONPATH", "")]))
+    done = subprocess.run([sys.executable, "-c", program, json.dumps(shapes)], stdout=subprocess.PIPE, text=True, check=True, timeout=300, env=env)
+    names = json.loads(done.stdout.splitlines()[-1])
     if not names:
         pytest.skip("no kernel names from the profiler")
-    return names[0]
+    assert len(names) == len(shapes)
+    return names
 
 
 def test_many_units_keep_enough_in_flight():
     """Three blocks of 256 threads a multiprocessor took 28.6 us for 900 units of two heads and 96 rows, a thread a channel 25.3; two for
     384 units of four heads 16.3, three 14.7."""
-    for g in (1, 2, 3):
-        assert "decode_merge_channels" in _merge_kernel(128, g, 6 * SMS + 12), g
-    for d, g, full, resident in ((128, 2, 3, 4), (128, 2, 5, 5), (128, 4, 2, 2), (128, 4, 3, 3), (64, 4, 5, 7)):
-        assert re.search(r"decode_merge_bf16<.*?(\d+)\)?>", _merge_kernel(d, g, full * SMS)).group(1) == str(resident), (d, g, full)
+    resident = {(128, 2, 3): 4, (128, 2, 5): 5, (128, 4, 2): 2, (128, 4, 3): 3, (64, 4, 5): 7}      # by units a multiprocessor
+    names = _merge_kernels([(128, g, 6 * SMS + 12) for g in (1, 2, 3)] + [(d, g, full * SMS) for d, g, full in resident])
+    assert all("decode_merge_channels" in name for name in names[:3]), names[:3]
+    assert [re.search(r"decode_merge_bf16<.*?(\d+)\)?>", name).group(1) for name in names[3:]] == [str(r) for r in resident.values()]
